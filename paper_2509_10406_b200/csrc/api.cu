@@ -17,6 +17,14 @@ int clear_status(void* ws, cudaStream_t st) {
   return cudaMemsetAsync(ws, 0, kStatusWords * sizeof(int32_t), st) == cudaSuccess ? MUSE_OK : MUSE_ERR_CUDA;
 }
 
+size_t cluster_ws_bytes(const Dims& d, bool q, bool k) {
+  size_t n = kStatusWords * sizeof(int32_t);
+  if (q) n += lloyd_ws_bytes(d, d.B * d.Hq, d.Cq);
+  if (k) n += lloyd_ws_bytes(d, d.B * d.Hkv, d.Ck);
+  const size_t draws = kStatusWords * sizeof(int32_t) + (((size_t)d.B * (d.Hq > d.Hkv ? d.Hq : d.Hkv) * d.N * sizeof(float) + 255) & ~size_t(255));
+  return n > draws ? n : draws;                            // (muse_kmeanspp_init shares this size)
+}
+
 // A deliberately unreachable wait: nothing ever arrives at the barrier, so the bounded wait runs out
 // after `limit_clocks` and the kernel reports through the status word like any production kernel.
 __global__ void k_selftest_wait(int* status, unsigned limit_clocks) {
@@ -67,7 +75,18 @@ int resolve(const muse_params_t* p, Dims* d) {
 
 }  // namespace
 
-namespace muse { bool path_forced(unsigned bit) { return (g_forced_paths & bit) != 0; } }
+namespace muse {
+bool path_forced(unsigned bit) { return (g_forced_paths & bit) != 0; }
+
+int sm_count() {
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) {
+    cudaGetLastError();
+    return 148;
+  }
+  return n;
+}
+}  // namespace muse
 
 #ifdef MUSE_DEBUG
 namespace muse {
@@ -137,8 +156,7 @@ int muse_workspace_bytes(const muse_params_t* p, size_t out[6]) {
   int rc = resolve(p, &d);
   if (rc != MUSE_OK) return rc;
   if (out == nullptr) return MUSE_ERR_INVALID_ARG;
-  size_t cq = lloyd_ws_bytes(d, d.B * d.Hq, d.Cq, 0), ck = lloyd_ws_bytes(d, d.B * d.Hkv, d.Ck, 1);
-  out[0] = cq > ck ? cq : ck;
+  out[0] = cluster_ws_bytes(d, true, true);                // both sides run side by side
   out[1] = summarize_ws_bytes(d, p->dtype);
   out[2] = attn_fwd_ws_bytes(d, p->dtype);
   out[3] = attn_bwd_ws_bytes(d, p->dtype);
@@ -189,24 +207,30 @@ int muse_cluster(const muse_params_t* p, const void* Q, const void* K, const int
   if (rc != MUSE_OK) return rc;
   if (ws == nullptr || !aligned16(ws)) return MUSE_ERR_INVALID_ARG;
   if (Q == nullptr && K == nullptr) return MUSE_ERR_INVALID_ARG;
-  size_t need[6];
-  muse_workspace_bytes(p, need);
-  if (ws_bytes < need[0]) return MUSE_ERR_WORKSPACE;
-  if (clear_status(ws, stream) != MUSE_OK) return MUSE_ERR_CUDA;
+  if (ws_bytes < cluster_ws_bytes(d, Q != nullptr, K != nullptr)) return MUSE_ERR_WORKSPACE;
+  LloydSide sides[2] = {};
+  int n = 0;
   if (Q != nullptr) {
     if (assign_q == nullptr || qbar == nullptr || !aligned16(Q) || !aligned16(qbar)) return MUSE_ERR_INVALID_ARG;
     if (p->init_mode == MUSE_INIT_INDICES && init_q == nullptr) return MUSE_ERR_INVALID_ARG;
-    rc = lloyd(d, p->dtype, Q, d.B * d.Hq, d.Cq, 0, init_q, p->init_mode, p->seed, p->kmeans_iters, assign_q, qbar, ws, stream);
-    if (rc != MUSE_OK) return rc;
+    sides[n].X = Q; sides[n].problems = d.B * d.Hq; sides[n].C = d.Cq; sides[n].kind = 0;
+    sides[n].init_idx = init_q; sides[n].assign = assign_q; sides[n].centres = qbar;
+    ++n;
   }
   if (K != nullptr) {
     if (assign_k == nullptr || kcent == nullptr || !aligned16(K) || !aligned16(kcent)) return MUSE_ERR_INVALID_ARG;
     if (p->init_mode == MUSE_INIT_INDICES && init_k == nullptr) return MUSE_ERR_INVALID_ARG;
-    rc = lloyd(d, p->dtype, K, d.B * d.Hkv, d.Ck, 1, init_k, p->init_mode, p->seed, p->kmeans_iters, assign_k, kcent, ws, stream);
-    if (rc != MUSE_OK) return rc;
+    sides[n].X = K; sides[n].problems = d.B * d.Hkv; sides[n].C = d.Ck; sides[n].kind = 1;
+    sides[n].init_idx = init_k; sides[n].assign = assign_k; sides[n].centres = kcent;
+    ++n;
   }
+  Arena ar(ws);
+  int* status = ar.take<int32_t>(kStatusWords);
+  for (int k = 0; k < n; ++k) lloyd_side_ws(d, ar, sides[k]);
+  if (clear_status(ws, stream) != MUSE_OK) return MUSE_ERR_CUDA;
+  rc = lloyd(d, p->dtype, sides, n, p->init_mode, p->seed, p->kmeans_iters, status, stream);
   prof_mark(nullptr, stream);
-  return MUSE_OK;
+  return rc;
 }
 
 static size_t up256(size_t x) { return (x + 255) & ~size_t(255); }

@@ -672,7 +672,7 @@ int summ_bwd_tc(const Dims& d, const void* Kp, const void* Vp, const int32_t* of
                 void* qsplit, int per_block, int* status, cudaStream_t st);
 
 struct BwdWs {
-  int32_t *status, *off_q, *perm_q, *sort_scratch, *ret_scratch;
+  int32_t *status, *off_q, *perm_q, *ret_scratch;
   __nv_bfloat16* qsplit;
   float *delta, *dQacc, *dq_part, *dK_orig, *dV_orig, *dK_perm, *dV_perm, *dkappa, *dnu, *dS;
   float *dkappa_b, *dnu_b, *dS_b;           // gradients of the per-block summaries (two-level retrieval), fp32
@@ -685,7 +685,6 @@ static BwdWs bwd_ws(const Dims& d, Arena& ar) {
   w.status = ar.take<int32_t>(64);          // ws[0]: non-zero if a bounded device-side wait gave up
   w.off_q = ar.take<int32_t>(pq * (d.S * d.Cq + 1));
   w.perm_q = ar.take<int32_t>(pq * d.N);
-  w.sort_scratch = ar.take<int32_t>(pq * sort_ws_elems(d.N, d.Cq * d.S));
   w.ret_scratch = ar.take<int32_t>(pq * ret_index_elems(d));
   w.delta = ar.take<float>(pq * d.N);
   w.dQacc = ar.take<float>(pq * d.N * d.D);
@@ -753,7 +752,8 @@ static int attn_bwd_t(const Dims& d, int dtype, const T* Q, const T* K, const T*
   }
   int use_ret = 0;
   if (d.SB > 0) {
-    int rc = bucket_sort(0, assign_q, pq, d.N, d.Cq, d.S, d.Bs, 0, w.off_q, w.perm_q, w.sort_scratch, st);
+    const SortSide side = {assign_q, w.off_q, w.perm_q, pq, d.Cq, 0};
+    int rc = bucket_sort(&side, 1, d.N, d.S, d.Bs, st);
     if (rc != MUSE_OK) return rc;
     RetIndex ri = {};
     if (d.m > 0) {

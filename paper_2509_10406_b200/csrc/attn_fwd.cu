@@ -7,7 +7,6 @@
 
 namespace muse {
 
-int launch_scan(int32_t* cnt, int problems, int nkeys, int nchunks, int32_t* off, cudaStream_t st);
 int local_fwd_tc(const Dims& d, const void* Q, const void* K, const void* V, float* o_loc, float* lse_loc, int* status,
                  cudaStream_t st);
 bool far_fwd_tc_supported(const Dims& d, int dtype);
@@ -82,6 +81,30 @@ __global__ void k_ret_fill(Dims d, const int32_t* __restrict__ sel, const int32_
   }
 }
 
+// Exclusive scan of a head's counts; off[key] = start of the key's run.
+__global__ void __launch_bounds__(1024)
+k_ret_scan(int32_t* __restrict__ cnt, int nkeys, int32_t* __restrict__ off) {
+  __shared__ int32_t wsum[32];
+  const int prob = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  int32_t* c = cnt + (size_t)prob * nkeys;
+  int32_t* o = off + (size_t)prob * (nkeys + 1);
+  int carry = 0;
+  for (int e0 = 0; e0 < nkeys; e0 += 1024) {
+    const int e = e0 + tid, v = e < nkeys ? c[e] : 0;
+    int inc = v;
+#pragma unroll
+    for (int s = 1; s < 32; s <<= 1) { const int x = __shfl_up_sync(0xffffffffu, inc, s); if (lane >= s) inc += x; }
+    if (lane == 31) wsum[warp] = inc;
+    __syncthreads();
+    int base = carry, all = 0;
+    for (int w = 0; w < 32; ++w) { const int x = wsum[w]; if (w < warp) base += x; all += x; }
+    if (e < nkeys) { c[e] = base + inc - v; o[e] = base + inc - v; }
+    carry += all;
+    __syncthreads();
+  }
+  if (tid == 0) o[nkeys] = carry;
+}
+
 size_t ret_index_elems(const Dims& d) {
   // cursor [SB*Ck] + goff [SB*Ck+1] + pairs [N*m*max(k2,1)], each rounded up to 64 ints
   auto up = [](size_t x) { return (x + 63) & ~size_t(63); };
@@ -103,8 +126,9 @@ int build_ret_index(const Dims& d, const int32_t* sel, const int32_t* bsel, int3
   prof_mark("k_ret_count", st);
   k_ret_count<<<grid, 256, 0, st>>>(d, sel, bsel, out->cursor);
   MUSE_LAUNCH_OK();
-  int rc = launch_scan(out->cursor, pq, nkeys, 1, out->goff, st);
-  if (rc != MUSE_OK) return rc;
+  prof_mark("k_ret_scan", st);
+  k_ret_scan<<<pq, 1024, 0, st>>>(out->cursor, nkeys, out->goff);
+  MUSE_LAUNCH_OK();
   prof_mark("k_ret_fill", st);
   k_ret_fill<<<grid, 256, 0, st>>>(d, sel, bsel, out->cursor, out->pairs);
   MUSE_LAUNCH_OK();
@@ -548,7 +572,7 @@ __global__ void k_merge(Dims dm, const float* __restrict__ o_far, const float* _
 // ---------------------------------------------------------------------------------------------
 template <class T> constexpr bool kTensorT() { return sizeof(T) == 2; }
 
-struct FwdWs { int32_t *status, *off_q, *perm_q, *sort_scratch, *ret_scratch, *sel_tmp, *bsel_tmp; float *o_far, *lse_far, *o_loc, *lse_loc, *o_part, *l_part, *o_near, *lse_near, *csub; };
+struct FwdWs { int32_t *status, *off_q, *perm_q, *ret_scratch, *sel_tmp, *bsel_tmp; float *o_far, *lse_far, *o_loc, *lse_loc, *o_part, *l_part, *o_near, *lse_near, *csub; };
 
 static FwdWs fwd_ws(const Dims& d, Arena& ar) {
   FwdWs w;
@@ -556,7 +580,6 @@ static FwdWs fwd_ws(const Dims& d, Arena& ar) {
   w.status = ar.take<int32_t>(64);          // ws[0]: non-zero if a bounded device-side wait gave up
   w.off_q = ar.take<int32_t>(pq * (d.S * d.Cq + 1));
   w.perm_q = ar.take<int32_t>(pq * d.N);
-  w.sort_scratch = ar.take<int32_t>(pq * sort_ws_elems(d.N, d.Cq * d.S));
   w.ret_scratch = ar.take<int32_t>(pq * ret_index_elems(d));
   w.sel_tmp = ar.take<int32_t>(pq * d.N * (d.m > 0 ? d.m : 1));
   w.o_far = ar.take<float>(pq * d.N * d.D);
@@ -607,7 +630,8 @@ static int attn_fwd_t(const Dims& d, const T* Q, const T* K, const T* V, const i
   k_far_defaults<<<dim3(cdiv(d.N, 256), pq), 256, 0, st>>>(d, w.lse_far, sel);
   MUSE_LAUNCH_OK();
   if (d.SB > 0) {
-    int rc = bucket_sort(0, assign_q, pq, d.N, d.Cq, d.S, d.Bs, 0, w.off_q, w.perm_q, w.sort_scratch, st);
+    const SortSide side = {assign_q, w.off_q, w.perm_q, pq, d.Cq, 0};
+    int rc = bucket_sort(&side, 1, d.N, d.S, d.Bs, st);
     if (rc != MUSE_OK) return rc;
     if (far_fwd_tc_supported(d, dtype) && !path_forced(kForceFarSimt)) {
       rc = far_fwd_tc(d, summ_ptrs(L, base), Q, w.off_q, w.perm_q, sel_in, sel, w.o_far, w.lse_far, w.status, st);

@@ -5,6 +5,7 @@
 #include <stdint.h>
 #include <stddef.h>
 #include <math.h>
+#include <utility>
 #include "../../include/muse.h"
 
 namespace muse {
@@ -88,6 +89,12 @@ template <int EPL> __device__ __forceinline__ void stv(__nv_bfloat16* p, const f
   else { __nv_bfloat162 b = __floats2bfloat162_rn(x[0], x[1]); *reinterpret_cast<uint32_t*>(p) = *reinterpret_cast<uint32_t*>(&b); }
 }
 
+// One step of a running arg-min, as two selects: left to itself the compiler turns the comparison into a branch, and a
+// sweep over a row of distances then costs a divergence per element.  A NaN never compares below the minimum.
+__device__ __forceinline__ void argmin_step(float v, int i, float& best, int& bidx) {
+  asm("{\n.reg .pred p;\nsetp.lt.f32 p, %2, %0;\nselp.f32 %0, %2, %0, p;\nselp.b32 %1, %3, %1, p;\n}\n" : "+f"(best), "+r"(bidx) : "f"(v), "r"(i));
+}
+
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -98,6 +105,42 @@ __device__ __forceinline__ float warp_max(float v) {
   for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
   return v;
 }
+
+// ---- launches -------------------------------------------------------------------------------
+// Programmatic dependent launch: a kernel started with launch_pdl may begin while its predecessor on the stream still
+// runs; it must call pdl_wait() before its first access to global memory (that wait covers the whole predecessor,
+// which in turn waited for its own).  pdl_trigger() lets the successor begin.  A stage here is a chain of short
+// kernels, and this takes the launch latency and the block set-up (barriers, tensor memory) out of the chain.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <class... KA, class... A>
+inline int launch_pdl_cluster(void (*kernel)(KA...), dim3 grid, int threads, size_t smem, int cluster, cudaStream_t st, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cluster; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  if (smem > 48 * 1024 && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+    cudaGetLastError();
+    return MUSE_ERR_CUDA;
+  }
+  if (cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...) != cudaSuccess) { cudaGetLastError(); return MUSE_ERR_CUDA; }
+  return MUSE_OK;
+}
+template <class... KA, class... A>
+inline int launch_pdl(void (*kernel)(KA...), dim3 grid, int threads, size_t smem, cudaStream_t st, A&&... args) {
+  return launch_pdl_cluster(kernel, grid, threads, smem, 1, st, std::forward<A>(args)...);
+}
+#define MUSE_RC(expr) do { int rc_ = (expr); if (rc_ != MUSE_OK) return rc_; } while (0)
+int sm_count();                            // multiprocessors of the current device (api.cu)
 
 // per-kernel timing hook (no-op unless muse_profile(1) was called); name = nullptr ends a call
 void prof_mark(const char* name, cudaStream_t st);
@@ -142,16 +185,26 @@ enum ForcePath : unsigned {
 bool path_forced(unsigned bit);
 
 // ---- stage launchers (each enqueues on `st`, returns MUSE_OK or MUSE_ERR_CUDA) ---------------
-// clustering side: kind 0 = queries (key = block*C + cluster), kind 1 = keys (key = cluster*S + block)
-size_t sort_ws_elems(int N, int nkeys);   // int32 scratch elements per problem for bucket_sort
-int bucket_sort(int dtype_unused, const int32_t* assign, int problems, int N, int C, int S, int Bs,
-                int kind, int32_t* off, int32_t* perm, int32_t* scratch, cudaStream_t st);
+// Stable counting sort of every problem's tokens (bucket_sort.cu), up to two sides in one launch.
+// kind 0 (queries): segments (block, cluster) contiguous, off [C*S+1] by block * C + cluster;
+// kind 1 (keys): a cluster's blocks are one contiguous run, off [C*S+1] by cluster * S + block.
+struct SortSide { const int32_t* assign; int32_t* off; int32_t* perm; int problems, C, kind; };
+int bucket_sort(const SortSide* sides, int nsides, int N, int S, int Bs, cudaStream_t st);
 
-int lloyd(const Dims& d, int dtype, const void* X, int problems, int C, int kind,
-          const int32_t* init_idx, int init_mode, uint64_t seed, int T,
-          int32_t* assign, float* centres, void* ws, cudaStream_t st, float* dist_out = nullptr);   // dist_out: [problems, N, C]
-                                                                                               // |c|^2 - 2 x.c of the final assignment (optional)
-size_t lloyd_ws_bytes(const Dims& d, int problems, int C, int kind);
+// Lloyd iterations of one or both sides at once (kind 0 queries, 1 keys); the scratch pointers are carved from a
+// workspace by lloyd_side_ws.  cnorm is padded per problem to whole tiles of kAsgTile centres (infinity in the padding).
+constexpr int kAsgTile = 128;
+struct LloydSide {
+  const void* X; int problems, C, kind;
+  const int32_t* init_idx;
+  int32_t* assign; float* centres;
+  float* dist;                             // [problems, N, C] |c|^2 - 2 x.c of the final assignment (optional)
+  float* cnorm; int32_t* off; int32_t* perm; void* chi; void* clo;
+};
+void lloyd_side_ws(const Dims& d, Arena& ar, LloydSide& s);
+int lloyd(const Dims& d, int dtype, LloydSide* sides, int nsides, int init_mode, uint64_t seed, int T, int* status, cudaStream_t st);
+size_t lloyd_ws_bytes(const Dims& d, int problems, int C);      // scratch of one side (without the status words)
+int assign_tc(const LloydSide* sides, int nsides, int N, int D, int* status, cudaStream_t st);
 
 // the paper's own clustering: one streaming pass (state = totals, counts; n_batches < 0: to the end) and the
 // per-block assignment under a bucket-size cap (factor <= 0: plain nearest centroid)

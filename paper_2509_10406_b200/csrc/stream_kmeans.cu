@@ -580,15 +580,22 @@ k_cap_overflow(int N, int C, int S, int Bs, int cap, const float* __restrict__ d
   }
 }
 
+struct BalancedWs { int32_t *status, *rank; float* dist; };
+
+static BalancedWs balanced_ws(const Dims& d, Arena& ar, LloydSide& s) {
+  BalancedWs w;
+  w.status = ar.take<int32_t>(kStatusWords);
+  lloyd_side_ws(d, ar, s);
+  w.rank = ar.take<int32_t>((size_t)s.problems * d.N);
+  w.dist = ar.take<float>((size_t)s.problems * d.N * s.C);       // |c|^2 - 2 x.c of every (vector, centroid), written by step 1
+  return w;
+}
+
 size_t balanced_ws_bytes(const Dims& d, int problems, int C) {
   Arena ar(nullptr);
-  ar.take<char>(lloyd_ws_bytes(d, problems, C, 0));
-  ar.take<float>((size_t)problems * C);
-  ar.take<int32_t>((size_t)problems * (C * d.S + 1));
-  ar.take<int32_t>((size_t)problems * d.N);
-  ar.take<int32_t>((size_t)problems * sort_ws_elems(d.N, C * d.S));
-  ar.take<int32_t>((size_t)problems * d.N);
-  ar.take<float>((size_t)problems * d.N * C);
+  LloydSide s = {};
+  s.problems = problems; s.C = C;
+  balanced_ws(d, ar, s);
   return ar.used;
 }
 
@@ -597,18 +604,17 @@ int balanced_assign(const Dims& d, int dtype, const void* X, int problems, int C
   const int cap = factor > 0.f ? (int)ceil((double)factor * d.Bs / C) : d.Bs;
   const bool binds = cap < d.Bs;               // otherwise the cap cannot bind: plain nearest centroid
   Arena ar(ws);
-  ar.take<char>(lloyd_ws_bytes(d, problems, C, 0));
-  ar.take<float>((size_t)problems * C);
-  int32_t* off = ar.take<int32_t>((size_t)problems * (C * d.S + 1));
-  int32_t* perm = ar.take<int32_t>((size_t)problems * d.N);
-  int32_t* scratch = ar.take<int32_t>((size_t)problems * sort_ws_elems(d.N, C * d.S));
-  int32_t* rank = ar.take<int32_t>((size_t)problems * d.N);
-  float* dist = ar.take<float>((size_t)problems * d.N * C);      // |c|^2 - 2 x.c of every (vector, centroid), written by step 1
+  LloydSide s = {};
+  s.X = X; s.problems = problems; s.C = C; s.kind = kind; s.assign = assign; s.centres = const_cast<float*>(centres);
+  const BalancedWs w = balanced_ws(d, ar, s);
+  if (binds) s.dist = w.dist;
   // step 1a: nearest centroid of every vector (the Lloyd path's final assignment against given centres)
-  int rc = lloyd(d, dtype, X, problems, C, kind, nullptr, MUSE_INIT_CENTRES, 0, 0, assign, const_cast<float*>(centres), ws, st,
-                 binds ? dist : nullptr);
+  int rc = lloyd(d, dtype, &s, 1, MUSE_INIT_CENTRES, 0, 0, w.status, st);
   if (rc != MUSE_OK || !binds) return rc;
-  rc = bucket_sort(0, assign, problems, d.N, C, d.S, d.Bs, 0, off, perm, scratch, st);      // key = block * C + cluster
+  int32_t *off = s.off, *perm = s.perm, *rank = w.rank;
+  float* dist = w.dist;
+  const SortSide side = {assign, off, perm, problems, C, 0};                                // key = block * C + cluster
+  rc = bucket_sort(&side, 1, d.N, d.S, d.Bs, st);
   if (rc != MUSE_OK) return rc;
   prof_mark("k_bucket_rank", st);
   k_bucket_rank<<<dim3(cdiv(d.N, 256), problems), 256, 0, st>>>(assign, off, perm, d.N, C, d.S, d.Bs, rank);

@@ -237,9 +237,9 @@ static int summarize_t(const Dims& d, int dtype, const T* K, const T* V, const i
   Arena ar(ws);
   int32_t* status = ar.take<int32_t>(kStatusWords);      // cleared by the entry point
   if (status_in != nullptr) status = status_in;
-  int32_t* sort_scratch = ar.take<int32_t>(sort_ws_elems(d.N, d.Ck * d.S) * (size_t)pk);
   int rc = MUSE_OK;
-  if (assign_k != nullptr) rc = bucket_sort(0, assign_k, pk, d.N, d.Ck, d.S, d.Bs, 1, off_k, perm_k, sort_scratch, st);
+  const SortSide side = {assign_k, off_k, perm_k, pk, d.Ck, 1};
+  if (assign_k != nullptr) rc = bucket_sort(&side, 1, d.N, d.S, d.Bs, st);
   if (rc != MUSE_OK) return rc;
   SummLayout L = summ_layout(d, dtype);
   char* base = (char*)summaries;
@@ -282,7 +282,6 @@ static int summarize_planes(const Dims& d, int dtype, const T* Kp, const T* Vp, 
 size_t summarize_ws_bytes(const Dims& d, int dtype) {
   Arena ar(nullptr);
   ar.take<int32_t>(kStatusWords);
-  ar.take<int32_t>((size_t)d.B * d.Hkv * sort_ws_elems(d.N, d.Ck * d.S));
   ar.take<__nv_bfloat16>(2 * (size_t)d.B * d.Hq * d.Cq * d.D);
   return ar.used;
 }

@@ -133,6 +133,21 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
+// Warp-wide forms: the whole warp runs the issuing loop and one elected lane (always the same for a full warp) executes
+// the instruction.  With warp-uniform control flow the descriptors stay in uniform registers; issued from inside an
+// `if (lane == 0)` each MMA costs a chain of moves from vector to uniform registers instead.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+  return p != 0;
+}
+__device__ __forceinline__ void mma_bf16_ss_warp(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+  if (elect_one()) mma_bf16_ss(d_tmem, adesc, bdesc, idesc, accumulate);
+}
+__device__ __forceinline__ void mma_commit_warp(uint64_t* bar) { if (elect_one()) mma_commit(bar); }
+// warp index that the compiler knows to be the same for the whole warp
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
+
 // ---- TMEM -> registers: 32 lanes x 32 columns; lane i of warp w reads TMEM lane 32*(w%4)+i -----------
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
   uint32_t r[32];
