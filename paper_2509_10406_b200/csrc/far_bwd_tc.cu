@@ -65,8 +65,8 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
   __shared__ int32_t rows[NP * NR];
   __shared__ __align__(16) float Ls[NP * NR], ds[NP * NR], qb[D], part[2][TJ], dsid[2][TJ];
   const int i = blockIdx.x, pl = blockIdx.y, pq = blockIdx.z;
-  const int blk = dm.causal ? pl + 1 : 0, Ck = dm.Ck, NJ = Ck / TJ, MW = Ck >> 5, m = dm.m;
-  const int tid = threadIdx.x, warp = tid >> 5, wg = tid >> 7, L = tid & 127;
+  const int blk = dm.causal ? pl + 1 : 0, Ck = dm.Ck, NJ = (Ck + TJ - 1) / TJ, m = dm.m;
+  const int tid = threadIdx.x, warp = tc::warp_index(), wg = tid >> 7, L = tid & 127;
 #ifdef MUSE_PHASE_CLOCKS
   const long long t_in_ = clock64();
   long long t_loop_ = 0, t_end_ = 0;
@@ -89,7 +89,8 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
   }
   unsigned char* sm = sm_raw + ((1024u - (tc::smem_u32(sm_raw) & 1023u)) & 1023u);
   uint32_t* smask = reinterpret_cast<uint32_t*>(sm + oMask);
-  const size_t ent0 = (((size_t)pq * dm.SB + pl) * dm.Cq + i) * Ck;
+  const int seg = (pq * dm.SB + pl) * dm.Cq + i;
+  const size_t ent0 = (size_t)seg * Ck;
   const bf16* Qp = Q + (size_t)pq * dm.N * D;
   const bf16* dOp = dO + (size_t)pq * dm.N * D;
   const int32_t* pm = perm_q + (size_t)pq * dm.N;
@@ -109,24 +110,22 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
                  aPt = tc::smem_u32(sm + oPt), aGt = tc::smem_u32(sm + oGt);
 
   auto issue_kappa = [&](int jt_) {                       // issuer: the two kappa tiles of cluster tile jt_
-    tc::mbar_expect_tx(&bar_full, 2 * kTile);
-    const int row = (int)(ent0 + (size_t)jt_ * TJ);
-    for (int g = 0; g < G; ++g) {
-      tc::tma_load_2d(sm + oHi + g * TJ * 128, &tm_khi, 64 * g, row, &bar_full);
-      tc::tma_load_2d(sm + oLo + g * TJ * 128, &tm_klo, 64 * g, row, &bar_full);
+    tc::mbar_expect_tx_warp(&bar_full, 2 * kTile);
+    for (int g = 0; g < G; ++g) {                         // (rows past Ck are zeros)
+      tc::tma_load_3d_warp(sm + oHi + g * TJ * 128, &tm_khi, 64 * g, jt_ * TJ, seg, &bar_full);
+      tc::tma_load_3d_warp(sm + oLo + g * TJ * 128, &tm_klo, 64 * g, jt_ * TJ, seg, &bar_full);
     }
   };
   auto issue_nu = [&](int jt_) {                          // issuer: its nu tile
-    tc::mbar_expect_tx(&bar_nu, kTile);
-    const int row = (int)(ent0 + (size_t)jt_ * TJ);
-    for (int g = 0; g < G; ++g) tc::tma_load_2d(sm + oNu + g * TJ * 128, &tm_nu, 64 * g, row, &bar_nu);
+    tc::mbar_expect_tx_warp(&bar_nu, kTile);
+    for (int g = 0; g < G; ++g) tc::tma_load_3d_warp(sm + oNu + g * TJ * 128, &tm_nu, 64 * g, jt_ * TJ, seg, &bar_nu);
   };
   for (int s0 = p0; s0 < p1 && ok; s0 += NP * NR) {        // sweep: up to 64 rows
     const int ns = min(NP * NR, p1 - s0), np = (ns + NR - 1) / NR;
     __syncthreads();
     // the operand tiles are free (every product of the previous sweep has completed): the first cluster
     // tile travels while the rows are gathered
-    if (tid == ISSUER) { issue_kappa(0); issue_nu(0); }
+    if (warp == ISSUER / 32) { issue_kappa(0); issue_nu(0); }
     if (tid < NP * NR) {
       int t = tid < ns && MUSE_IN_RANGE(s0 + tid, dm.N) ? pm[s0 + tid] : -1;
       if (t >= 0 && !MUSE_IN_RANGE(t, dm.N)) t = -1;
@@ -134,7 +133,7 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
       Ls[tid] = t >= 0 ? LSE[(size_t)pq * dm.N + t] * kLog2e : 0.f;
       ds[tid] = t >= 0 ? delta[(size_t)pq * dm.N + t] : 0.f;
     }
-    for (int e = tid; e < 2 * Ck; e += THREADS) smask[e] = 0u;
+    for (int e = tid; e < 2 * NJ * TJ; e += THREADS) smask[e] = 0u;
     __syncthreads();
     for (int e = tid; e < NP * NR * CPR; e += THREADS) {
       const int r = e / CPR, ck = e % CPR, kb = ck >> 3, c = ck & 7, p = r / NR, rr = r % NR;
@@ -166,10 +165,10 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
       Lc[4 * k] = a.x; Lc[4 * k + 1] = a.y; Lc[4 * k + 2] = a.z; Lc[4 * k + 3] = a.w;
       dc[4 * k] = b.x; dc[4 * k + 1] = b.y; dc[4 * k + 2] = b.z; dc[4 * k + 3] = b.w;
     }
-    float bnext = beta[ent0 + L];
+    float bnext = L < Ck ? beta[ent0 + L] : -INFINITY;
     const bool later_sweep = s0 > p0;                       // gradients of earlier sweeps are already stored: add to them
     if (later_sweep) {
-      if (tid == ISSUER) tc::tma_store_wait_all();
+      if (warp == ISSUER / 32) tc::tma_store_wait_all_warp();
       __syncthreads();
     }
 #ifdef MUSE_PHASE_CLOCKS
@@ -183,12 +182,12 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
       const float bj = bnext;                               // loaded one tile ahead
       const bool alive = bj != -INFINITY;                   // an empty cluster has beta = mu = -inf
       const float sig2 = dm.sigma * kLog2e, bj2 = alive ? bj * kLog2e : 0.f;
-      if (jt + 1 < NJ) bnext = beta[ent0 + j + TJ];
+      if (jt + 1 < NJ) bnext = j + TJ < Ck ? beta[ent0 + j + TJ] : -INFINITY;
       float gsum = 0.f, gt2 = 0.f, pdp = 0.f;
-      const float mu1 = 1.f + mu[ent0 + j];                               // 1 + accumulated log-mass of cluster j
+      const float mu1 = j < Ck ? 1.f + mu[ent0 + j] : 0.f;                              // 1 + accumulated log-mass of cluster j
       for (int p = 0; p < np && ok; ++p) {
         const uint32_t aQ = tc::smem_u32(sm + oQ + p * kRows), aDO = tc::smem_u32(sm + oDO + p * kRows);
-        if (tid == ISSUER) {
+        if (warp == ISSUER / 32) {
           if (p == 0) {
             if (!tc::mbar_wait(&bar_full, ph_full)) ok = false;
             if (!tc::mbar_wait(&bar_nu, ph_full)) ok = false;
@@ -197,20 +196,20 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
           const uint32_t idesc = tc::idesc_bf16(TJ, NR, 0, 0);
 #pragma unroll
           for (int ks = 0; ks < D / 16; ++ks)
-            tc::mma_bf16_ss(tbase + cS, tc::smem_desc_sw128(aHi + (ks / 4) * TJ * 128 + (ks % 4) * 32, 16, 1024),
+            tc::mma_bf16_ss_warp(tbase + cS, tc::smem_desc_sw128(aHi + (ks / 4) * TJ * 128 + (ks % 4) * 32, 16, 1024),
                             tc::smem_desc_sw128(aQ + (ks / 4) * NR * 128 + (ks % 4) * 32, 16, 1024), idesc, ks > 0);
 #pragma unroll
           for (int ks = 0; ks < D / 16; ++ks)
-            tc::mma_bf16_ss(tbase + cS, tc::smem_desc_sw128(aLo + (ks / 4) * TJ * 128 + (ks % 4) * 32, 16, 1024),
+            tc::mma_bf16_ss_warp(tbase + cS, tc::smem_desc_sw128(aLo + (ks / 4) * TJ * 128 + (ks % 4) * 32, 16, 1024),
                             tc::smem_desc_sw128(aQ + (ks / 4) * NR * 128 + (ks % 4) * 32, 16, 1024), idesc, 1);
 #pragma unroll
           for (int ks = 0; ks < D / 16; ++ks)
-            tc::mma_bf16_ss(tbase + cDP, tc::smem_desc_sw128(aNu + (ks / 4) * TJ * 128 + (ks % 4) * 32, 16, 1024),
+            tc::mma_bf16_ss_warp(tbase + cDP, tc::smem_desc_sw128(aNu + (ks / 4) * TJ * 128 + (ks % 4) * 32, 16, 1024),
                             tc::smem_desc_sw128(aDO + (ks / 4) * NR * 128 + (ks % 4) * 32, 16, 1024), idesc, ks > 0);
-          tc::mma_commit(&bar1);
+          tc::mma_commit_warp(&bar1);
           if (p == 0) {
-            tc::tma_store_wait_read();        // the previous tile's stores have read the staging tiles, which the
-            tc::mbar_arrive(&bar_st);         // compute warps write again (P / G tiles first)
+            tc::tma_store_wait_read_warp();        // the previous tile's stores have read the staging tiles, which the
+            if (tc::elect_one()) tc::mbar_arrive(&bar_st);         // compute warps write again (P / G tiles first)
           }
           if (!tc::mbar_wait(&bar1, ph1)) ok = false;
           if (p + 1 == np && jt + 1 < NJ && ok) issue_nu(jt + 1);     // the nu tile is only read by the products above
@@ -269,7 +268,7 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
         tc::fence_async_smem();
         tc::fence_before_sync();
         __syncthreads();
-        if (tid == ISSUER) {
+        if (warp == ISSUER / 32) {
           tc::fence_after_sync();
           const uint32_t id_row = tc::idesc_bf16(TJ, D, 0, 1);      // A K-major (P / G), B = query rows, MN-major
           // A = kappa tile MN-major, B = G MN-major.  M = 128 output dims even when D = 64: the second 64-dim group of the
@@ -277,22 +276,22 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
           const uint32_t id_dq = tc::idesc_bf16(128, NR, 1, 1);
 #pragma unroll
           for (int ks = 0; ks < NR / 16; ++ks)
-            tc::mma_bf16_ss(tbase + cDNU, tc::smem_desc_sw128(aPt + ks * 32, 16, 1024),
+            tc::mma_bf16_ss_warp(tbase + cDNU, tc::smem_desc_sw128(aPt + ks * 32, 16, 1024),
                             tc::smem_desc_sw128(aDO + ks * 16 * 128, NR * 128, 1024), id_row, !(p == 0 && ks == 0));
 #pragma unroll
           for (int ks = 0; ks < NR / 16; ++ks)
-            tc::mma_bf16_ss(tbase + cDKA, tc::smem_desc_sw128(aGt + ks * 32, 16, 1024),
+            tc::mma_bf16_ss_warp(tbase + cDKA, tc::smem_desc_sw128(aGt + ks * 32, 16, 1024),
                             tc::smem_desc_sw128(aQ + ks * 16 * 128, NR * 128, 1024), id_row, !(p == 0 && ks == 0));
-          tc::mma_commit(&bar2);              // the read-out of dnu / dkappa can start while the dq products still run
+          tc::mma_commit_warp(&bar2);              // the read-out of dnu / dkappa can start while the dq products still run
 #pragma unroll
           for (int ks = 0; ks < TJ / 16; ++ks)
-            tc::mma_bf16_ss(tbase + cDQ + p * NR, tc::smem_desc_sw128(aHi + ks * 16 * 128, TJ * 128, 1024),
+            tc::mma_bf16_ss_warp(tbase + cDQ + p * NR, tc::smem_desc_sw128(aHi + ks * 16 * 128, TJ * 128, 1024),
                             tc::smem_desc_sw128(aGt + ks * 16 * 128, TJ * 128, 1024), id_dq, !(jt == 0 && ks == 0));
 #pragma unroll
           for (int ks = 0; ks < TJ / 16; ++ks)
-            tc::mma_bf16_ss(tbase + cDQ + p * NR, tc::smem_desc_sw128(aLo + ks * 16 * 128, TJ * 128, 1024),
+            tc::mma_bf16_ss_warp(tbase + cDQ + p * NR, tc::smem_desc_sw128(aLo + ks * 16 * 128, TJ * 128, 1024),
                             tc::smem_desc_sw128(aGt + ks * 16 * 128, TJ * 128, 1024), id_dq, 1);
-          tc::mma_commit(&bar3);
+          tc::mma_commit_warp(&bar3);
           // every MMA on the operand tiles has completed: the next cluster tile may overwrite them
           if (!tc::mbar_wait(&bar3, ph3)) ok = false;
           if (p + 1 == np && jt + 1 < NJ && ok) issue_kappa(jt + 1);
@@ -368,24 +367,23 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
 #ifdef MUSE_PHASE_CLOCKS
       if (rec_) status[36 + 3 * wg] = (int)(clock64() - k3_);
 #endif
-      if (tid == ISSUER && ok) {
-        const int c1 = grad_by_key_cluster ? i : 0;
-        const int c2 = grad_by_key_cluster ? (pq * dm.SB + pl) * Ck + jt * TJ : (int)(ent0 + (size_t)jt * TJ);
+      if (warp == ISSUER / 32 && ok) {
+        const int c1 = grad_by_key_cluster ? i : 0, c2 = jt * TJ, c3 = grad_by_key_cluster ? pq * dm.SB + pl : seg;
         if (!later_sweep) {
           for (int g = 0; g < G; ++g) {
-            tc::tma_store_3d(&tm_gnu, sm + oStN + g * TJ * 128, 64 * g, c1, c2);
-            tc::tma_store_3d(&tm_gka, sm + oStK + g * TJ * 128, 64 * g, c1, c2);
+            tc::tma_store_4d_warp(&tm_gnu, sm + oStN + g * TJ * 128, 64 * g, c1, c2, c3);
+            tc::tma_store_4d_warp(&tm_gka, sm + oStK + g * TJ * 128, 64 * g, c1, c2, c3);
           }
         } else {                              // a further sweep of a long segment adds to the stored rows
           for (int g = 0; g < G; ++g) {
-            tc::tma_reduce_add_3d(&tm_gnu, sm + oStN + g * TJ * 128, 64 * g, c1, c2);
-            tc::tma_reduce_add_3d(&tm_gka, sm + oStK + g * TJ * 128, 64 * g, c1, c2);
+            tc::tma_reduce_add_4d_warp(&tm_gnu, sm + oStN + g * TJ * 128, 64 * g, c1, c2, c3);
+            tc::tma_reduce_add_4d_warp(&tm_gka, sm + oStK + g * TJ * 128, 64 * g, c1, c2, c3);
           }
         }
-        tc::tma_store_commit();
+        tc::tma_store_commit_warp();
       }
       tc::fence_before_sync();
-      if (wg == 0 && ok) dS[gent] = (later_sweep ? dS[gent] : 0.f) + dsid[0][L] + dsid[1][L];
+      if (wg == 0 && ok && j < Ck) dS[gent] = (later_sweep ? dS[gent] : 0.f) + dsid[0][L] + dsid[1][L];
 #ifdef MUSE_PHASE_CLOCKS
       k4_ = clock64();
       pc[0] += k1_ - k0_; pc[1] += k2_ - k1_; pc[2] += k3_ - k2_; pc[3] += k4_ - k3_; pc[4] += 1; pc[5] = np;
@@ -416,7 +414,7 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
   }
   tc::fence_before_sync();
   __syncthreads();
-  if (tid == ISSUER) tc::tma_store_wait_read();             // the staging tiles must outlive the stores' reads only
+  if (warp == ISSUER / 32) tc::tma_store_wait_read_warp();             // the staging tiles must outlive the stores' reads only
   if (warp == 0) tc::tmem_dealloc(tbase, 512);
   if (!ok && tid == 0) report_status(status, 4);
 #ifdef MUSE_PHASE_CLOCKS
@@ -428,29 +426,27 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
 
 bool far_bwd_tc_supported(const Dims& d, int dtype) {
   // (the far-set mask, 8 bytes per key cluster, shares the CTA's shared memory with 200 KB of tiles)
-  return dtype == MUSE_BF16 && (d.D == 64 || d.D == 128) && d.Ck % fb::TJ == 0 && d.Ck <= 2048;
+  return dtype == MUSE_BF16 && (d.D == 64 || d.D == 128) && d.Ck <= 2048;
 }
 
 int far_bwd_tc(const Dims& d, const SummPtrs& sp, const void* Q, const void* dO, const float* qbar, const float* LSE,
                const float* delta, const int32_t* off_q, const int32_t* perm_q, const int32_t* sel, float* dQacc,
                void* dkappa, void* dnu, float* dS, int grad_by_key_cluster, int* status, cudaStream_t st) {
-  const uint64_t ent = (uint64_t)d.B * d.Hq * d.SB * d.Cq * d.Ck;
+  const uint64_t Dd = (uint64_t)d.D, Cq = (uint64_t)d.Cq, Ck = (uint64_t)d.Ck, planes = (uint64_t)d.B * d.Hq * d.SB;
+  if (planes * Cq * Ck >= (1ull << 31)) return MUSE_ERR_UNSUPPORTED;
+  const uint64_t dims[3] = {Dd, Ck, planes * Cq}, str[2] = {Dd * 2, Ck * Dd * 2};       // summaries [segments][Ck][D]
+  const uint32_t box3[3] = {64, (uint32_t)fb::TJ, 1}, box4[4] = {64, 1, (uint32_t)fb::TJ, 1};
   CUtensorMap khi, klo, nu;
-  const uint64_t Dd = (uint64_t)d.D;
-  int rc = make_tmap_bf16_rows(&khi, sp.khi, ent, d.D, fb::TJ);
-  if (rc == MUSE_OK) rc = make_tmap_bf16_rows(&klo, sp.klo, ent, d.D, fb::TJ);
-  if (rc == MUSE_OK) rc = make_tmap_bf16_rows(&nu, sp.nu, ent, d.D, fb::TJ);
-  // gradient tensors for the tiled stores: (d, i, plane * Ck + j) when grouped by key cluster, else (d, 1, entry)
+  MUSE_RC(make_tmap_bf16_nd(&khi, sp.khi, 3, dims, str, box3));
+  MUSE_RC(make_tmap_bf16_nd(&klo, sp.klo, 3, dims, str, box3));
+  MUSE_RC(make_tmap_bf16_nd(&nu, sp.nu, 3, dims, str, box3));
+  // gradient tensors for the tiled stores: (d, i, j, plane) when grouped by key cluster, else (d, 1, j, segment)
   CUtensorMap gka, gnu;
-  const uint64_t rows_j = (uint64_t)d.B * d.Hq * d.SB * d.Ck;
-  const uint64_t dims_a[3] = {Dd, (uint64_t)d.Cq, rows_j}, str_a[2] = {Dd * 2, (uint64_t)d.Cq * Dd * 2};
-  const uint64_t dims_b[3] = {Dd, 1, ent}, str_b[2] = {Dd * 2, Dd * 2};
-  const uint32_t box[3] = {64, 1, (uint32_t)fb::TJ};
-  if (rc == MUSE_OK) rc = make_tmap_bf16_nd(&gka, dkappa, 3, grad_by_key_cluster ? dims_a : dims_b, grad_by_key_cluster ? str_a : str_b, box);
-  if (rc == MUSE_OK) rc = make_tmap_bf16_nd(&gnu, dnu, 3, grad_by_key_cluster ? dims_a : dims_b, grad_by_key_cluster ? str_a : str_b, box);
-  if (rc != MUSE_OK) return rc;
-  if (ent >= (1ull << 31)) return MUSE_ERR_UNSUPPORTED;      // 32-bit tile coordinates
-  const size_t mask_bytes = (size_t)fb::NP * fb::NR * (d.Ck / 32) * 4;
+  const uint64_t dims_a[4] = {Dd, Cq, Ck, planes}, str_a[3] = {Dd * 2, Cq * Dd * 2, Ck * Cq * Dd * 2};
+  const uint64_t dims_b[4] = {Dd, 1, Ck, planes * Cq}, str_b[3] = {Dd * 2, Dd * 2, Ck * Dd * 2};
+  MUSE_RC(make_tmap_bf16_nd(&gka, dkappa, 4, grad_by_key_cluster ? dims_a : dims_b, grad_by_key_cluster ? str_a : str_b, box4));
+  MUSE_RC(make_tmap_bf16_nd(&gnu, dnu, 4, grad_by_key_cluster ? dims_a : dims_b, grad_by_key_cluster ? str_a : str_b, box4));
+  const size_t mask_bytes = (size_t)cdiv(d.Ck, fb::TJ) * fb::TJ * 8;
   prof_mark("k_far_bwd_tc", st);
   if (d.D == 128) {
     const size_t smem = (size_t)fb::Lay<128>::oMask + mask_bytes + 1024;

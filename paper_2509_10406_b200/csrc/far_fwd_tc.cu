@@ -1,4 +1,5 @@
-// Far-field forward on the tensor cores (bf16 mode, D = 64 or 128, Ck a multiple of 128, Ck <= 2048).
+// Far-field forward on the tensor cores (bf16 mode, D = 64 or 128, Ck <= 2048).  Clusters come in tiles of 128; the
+// tensor maps end at Ck, so the rows of the last tile past it are zeros, and their beta is taken as -infinity.
 // One CTA per (query cluster i, plane, head) segment; its queries (32 on average at the headline
 // sizes, up to 64 per pass) share the Ck accumulated summaries of (i, plane).  The summaries sit
 // on the MMA M side (128 clusters per tile, one TMEM lane each) and the queries on the N side
@@ -18,7 +19,7 @@
 namespace muse {
 
 typedef __nv_bfloat16 bf16;
-int make_tmap_bf16_rows(void* out_map, const void* base, uint64_t rows, uint32_t cols, uint32_t box_rows);
+int make_tmap_bf16_nd(void* out_map, const void* base, int rank, const uint64_t* dims, const uint64_t* strides_bytes, const uint32_t* box);
 
 constexpr int kFJ = 128;                            // clusters per tile
 // Queries per pass FR and per selection step FQ (one warp each) are template parameters: 64 / 16 up to 1024
@@ -239,8 +240,8 @@ k_far_fwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
   __shared__ float rinv[FR];
   __shared__ int32_t selq[kMaxM];
   const int i = blockIdx.x, pl = blockIdx.y, pq = blockIdx.z;
-  const int blk = dm.causal ? pl + 1 : 0, Ck = dm.Ck, NJ = Ck / kFJ, m = dm.m;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int blk = dm.causal ? pl + 1 : 0, Ck = dm.Ck, NJ = (Ck + kFJ - 1) / kFJ, CkP = NJ * kFJ, m = dm.m;   // CkP: clusters rounded up to whole tiles
+  const int tid = threadIdx.x, warp = tc::warp_index(), lane = tid & 31;
   const int32_t* oq = off_q + (size_t)pq * (dm.S * dm.Cq + 1) + (size_t)blk * dm.Cq + i;
   const int p0 = oq[0], p1 = oq[1];
   if (p0 >= p1) return;
@@ -250,7 +251,8 @@ k_far_fwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
   unsigned char* Pm = sm;
   float* sc = reinterpret_cast<float*>(sm + p_bytes);
   unsigned char* Qs = sm + p_bytes + sc_bytes;
-  const size_t ent0 = (((size_t)pq * dm.SB + pl) * dm.Cq + i) * Ck;
+  const int seg = (pq * dm.SB + pl) * dm.Cq + i;
+  const size_t ent0 = (size_t)seg * Ck;
   const float* mup = mu + ent0;
   const float* bep = beta + ent0;
   const bf16* Qp = Q + (size_t)pq * dm.N * D;
@@ -287,12 +289,12 @@ k_far_fwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
   const uint32_t tbase = tbase_s;
   uint32_t cntA = 0, cntD = 0, done_ph = 0;   // tiles of the earlier passes (same in every thread); phase of `done`
   bool ok = true;
-  // TMA producers: lane 0 of warps 0, 2, 3, 4.  One thread sustains only about 30 bytes per clock
+  // TMA producers: warps 0, 2, 3, 4 (an elected lane each).  One thread sustains only about 30 bytes per clock
   // (every bulk-tensor instruction holds it for some 270 clocks per 16 KB box, every wait after one
   // for some 500), several threads add up.  Producer p serves the tiles whose running index is
   // p modulo the producer count, and that count divides the ring depth, so a ring stage always
   // belongs to one producer and its waits on the stage's barrier never fall a phase behind.
-  const int prod = lane != 0 ? -1 : warp == 0 ? 0 : (warp >= 2 && warp <= 4) ? warp - 1 : -1;
+  const int prod = warp == 0 ? 0 : (warp >= 2 && warp <= 4) ? warp - 1 : -1;
   const int WA = nsA % 4 == 0 ? 4 : nsA % 3 == 0 ? 3 : nsA % 2 == 0 ? 2 : 1;
   const int WD = nsD % 4 == 0 ? 4 : nsD % 2 == 0 ? 2 : 1;
   const int lq = warp & 3, tg = warp >> 2;            // TMEM lane quarter of this warp, tile group
@@ -315,10 +317,9 @@ k_far_fwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
     auto produce_a = [&](int t) {
       const int s = sa;
       if (!tc::mbar_wait(&bars.emptyA[s], pha ^ 1)) { ok = false; return; }
-      tc::mbar_expect_tx(&bars.fullA[s], kTileBytes);
+      tc::mbar_expect_tx_warp(&bars.fullA[s], kTileBytes);
       const void* map = (t & 1) ? (const void*)&tm_klo : (const void*)&tm_khi;
-      const int row = (int)(ent0 + (size_t)(t >> 1) * kFJ);
-      for (int g = 0; g < G; ++g) tc::tma_load_2d(sm + s * kTileBytes + g * kFJ * 128, map, 64 * g, row, &bars.fullA[s]);
+      for (int g = 0; g < G; ++g) tc::tma_load_3d_warp(sm + s * kTileBytes + g * kFJ * 128, map, 64 * g, (t >> 1) * kFJ, seg, &bars.fullA[s]);
     };
     const int TA = 2 * NJ, TA0 = min(nsA, TA);
     if (prod >= 0 && prod < WA)
@@ -341,9 +342,9 @@ k_far_fwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
           if (wa == prod) produce_a(t);
       // bring the nu tiles of this segment into L2 while the selection runs
       for (int t = prod; t < NJ; t += 4) {
-        for (int g = 0; g < G; ++g) tc::tma_prefetch_2d(&tm_nu, 64 * g, (int)(ent0 + (size_t)t * kFJ));
+        for (int g = 0; g < G; ++g) tc::tma_prefetch_3d_warp(&tm_nu, 64 * g, t * kFJ, seg);
       }
-    } else if (tid == 32) {
+    } else if (warp == 1) {
       tc::fence_after_sync();
       const uint32_t idesc = tc::idesc_bf16(kFJ, FR, 0, 0);
       const uint64_t dq0 = tc::smem_desc_sw128(tc::smem_u32(Qs), 16, 1024), da0 = tc::smem_desc_sw128(tc::smem_u32(sm), 16, 1024);
@@ -364,18 +365,18 @@ k_far_fwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
 
 #pragma unroll
         for (int ks = 0; ks < D / 16; ++ks)
-          tc::mma_bf16_ss(dcol, tc::desc_step(da, (ks / 4) * kFJ * 128 + (ks % 4) * 32),
+          tc::mma_bf16_ss_warp(dcol, tc::desc_step(da, (ks / 4) * kFJ * 128 + (ks % 4) * 32),
                           tc::desc_step(dq0, (ks / 4) * FR * 128 + (ks % 4) * 32), idesc, (u & 1) || ks > 0);
-        tc::mma_commit(&bars.emptyA[s]);
+        tc::mma_commit_warp(&bars.emptyA[s]);
         if (++s == nsA) { s = 0; ph ^= 1; }
       }
-      if (ok) tc::mma_commit(&bars.done);
+      if (ok) tc::mma_commit_warp(&bars.done);
     }
     float bq[KT];                                       // beta of this thread's clusters, loaded ahead of the TMEM reads
 #pragma unroll
-    for (int k = 0; k < KT; ++k) { const int jt = tg + NTG * k; bq[k] = jt < NJ ? bep[jt * kFJ + (tid & 127)] : 0.f; }
+    for (int k = 0; k < KT; ++k) { const int j = (tg + NTG * k) * kFJ + (tid & 127); bq[k] = j < Ck ? bep[j] : -INFINITY; }
     // only the consumer polls the mbarrier; everyone else sleeps at the hardware barrier
-    if (tid == 32) {
+    if (warp == 1) {
       if (!tc::mbar_wait(&bars.done, done_ph)) ok = false;
       tc::fence_before_sync();
     }
@@ -401,7 +402,7 @@ k_far_fwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
         const int j = jt * kFJ + (tid & 127);
         const float b = bq[k];
 #pragma unroll
-        for (int r = 0; r < FQ; ++r) sc[r * Ck + j] = b == -INFINITY ? -INFINITY : fmaf(v[r], dm.sigma, b);
+        for (int r = 0; r < FQ; ++r) sc[r * CkP + j] = b == -INFINITY ? -INFINITY : fmaf(v[r], dm.sigma, b);
       }
       __syncthreads();
 #ifdef MUSE_PHASE_CLOCKS
@@ -409,7 +410,7 @@ k_far_fwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
 #endif
       // ---- C: selection + softmax of the far set; P (bf16) as a K-major operand [64][Ck]
       const int r = qs * FQ + warp;                    // one query per warp
-      float* s = sc + warp * Ck;
+      float* s = sc + warp * CkP;
       float sum = 0.f, mx = -INFINITY;
       if (r < n) {
         const int t = rows[r];
@@ -425,17 +426,17 @@ k_far_fwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
 #ifdef MUSE_PHASE_CLOCKS
           if (warp == 0 && blockIdx.x == 200 && blockIdx.y == 5 && blockIdx.z == 1 && r0 == p0 && qs == 0) dbg = status + 56;
 #endif
-          select_top_m<NKMAX>(s, Ck, m, so, lane, Pm + r * 128, FR * 128, Ck >= 512, dbg);
+          select_top_m<NKMAX>(s, CkP, m, so, lane, Pm + r * 128, FR * 128, CkP >= 512, dbg);
         }
         __syncwarp();
 #ifdef MUSE_PHASE_CLOCKS
         cb2 = clock64();
 #endif
-        for (int j = lane; j < Ck; j += 32) mx = fmaxf(mx, s[j]);
+        for (int j = lane; j < CkP; j += 32) mx = fmaxf(mx, s[j]);
         mx = warp_max(mx);
       }
       // probabilities, 8 consecutive clusters (one 16-byte chunk) per lane and step
-      for (int q = lane; q < Ck / 8; q += 32) {
+      for (int q = lane; q < CkP / 8; q += 32) {
         const float4 s0 = *reinterpret_cast<const float4*>(s + q * 8), s1 = *reinterpret_cast<const float4*>(s + q * 8 + 4);
         const float sv[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
         uint32_t w[4];
@@ -477,11 +478,10 @@ k_far_fwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
         if (++w == WD) w = 0;
         if (w_ != prod) continue;
         if (!tc::mbar_wait(&bars.emptyD[s_], ph_ ^ 1)) { ok = false; break; }
-        tc::mbar_expect_tx(&bars.fullD[s_], kTileBytes);
-        const int row = (int)(ent0 + (size_t)t * kFJ);
-        for (int g = 0; g < G; ++g) tc::tma_load_2d(ring + s_ * kTileBytes + g * kFJ * 128, &tm_nu, 64 * g, row, &bars.fullD[s_]);
+        tc::mbar_expect_tx_warp(&bars.fullD[s_], kTileBytes);
+        for (int g = 0; g < G; ++g) tc::tma_load_3d_warp(ring + s_ * kTileBytes + g * kFJ * 128, &tm_nu, 64 * g, t * kFJ, seg, &bars.fullD[s_]);
       }
-    } else if (tid == 32 && ok) {
+    } else if (warp == 1 && ok) {
       tc::fence_after_sync();
       // M = 128 output dims even when D = 64: the second 64-dim group of the MN-major operand then reads whatever
       // follows the tile in shared memory, and output lanes 64..127 hold numbers that nobody reads
@@ -502,14 +502,14 @@ k_far_fwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
         const uint64_t da = tc::desc_step(dn0, (uint32_t)s * kTileBytes), dp = tc::desc_step(dp0, (uint32_t)(2 * u) * (FR * 128));
 #pragma unroll
         for (int ks = 0; ks < kFJ / 16; ++ks)
-          tc::mma_bf16_ss(tbase, tc::desc_step(da, ks * 16 * 128), tc::desc_step(dp, (ks / 4) * (FR * 128) + (ks % 4) * 32), idesc,
+          tc::mma_bf16_ss_warp(tbase, tc::desc_step(da, ks * 16 * 128), tc::desc_step(dp, (ks / 4) * (FR * 128) + (ks % 4) * 32), idesc,
                           u > 0 || ks > 0);
-        tc::mma_commit(&bars.emptyD[s]);
+        tc::mma_commit_warp(&bars.emptyD[s]);
         if (++s == nsD) { s = 0; ph ^= 1; }
       }
-      if (ok) tc::mma_commit(&bars.done);
+      if (ok) tc::mma_commit_warp(&bars.done);
     }
-    if (tid == 32) {
+    if (warp == 1) {
       if (!tc::mbar_wait(&bars.done, done_ph)) ok = false;
       tc::fence_before_sync();
     }
@@ -545,22 +545,25 @@ k_far_fwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
 }
 
 bool far_fwd_tc_supported(const Dims& d, int dtype) {
-  return dtype == MUSE_BF16 && (d.D == 64 || d.D == 128) && d.Ck % kFJ == 0 && d.Ck <= 2048 && d.Ck >= kFJ;
+  return dtype == MUSE_BF16 && (d.D == 64 || d.D == 128) && d.Ck <= 2048;
 }
 
 int far_fwd_tc(const Dims& d, const SummPtrs& sp, const void* Q, const int32_t* off_q, const int32_t* perm_q,
                const int32_t* sel_in, int32_t* sel_out, float* o_far, float* lse_far, int* status, cudaStream_t st) {
-  const uint64_t ent = (uint64_t)d.B * d.Hq * d.SB * d.Cq * d.Ck;
+  // [segments][Ck][D]
+  const uint64_t dims[3] = {(uint64_t)d.D, (uint64_t)d.Ck, (uint64_t)d.B * d.Hq * d.SB * d.Cq};
+  const uint64_t strides[2] = {(uint64_t)d.D * 2, (uint64_t)d.Ck * d.D * 2};
+  const uint32_t box[3] = {64, kFJ, 1};
   CUtensorMap khi, klo, nu;
-  int rc = make_tmap_bf16_rows(&khi, sp.khi, ent, d.D, kFJ);
-  if (rc == MUSE_OK) rc = make_tmap_bf16_rows(&klo, sp.klo, ent, d.D, kFJ);
-  if (rc == MUSE_OK) rc = make_tmap_bf16_rows(&nu, sp.nu, ent, d.D, kFJ);
-  if (rc != MUSE_OK) return rc;
+  MUSE_RC(make_tmap_bf16_nd(&khi, sp.khi, 3, dims, strides, box));
+  MUSE_RC(make_tmap_bf16_nd(&klo, sp.klo, 3, dims, strides, box));
+  MUSE_RC(make_tmap_bf16_nd(&nu, sp.nu, 3, dims, strides, box));
+  const int CkP = cdiv(d.Ck, kFJ) * kFJ;
   const bool wide = d.Ck > 1024;                                         // 32 queries per pass, 8 per selection step
   const int FR = wide ? 32 : 64, FQ = wide ? 8 : 16;
   const int tile_bytes = kFJ * d.D * 2;
-  const int p_bytes = FR * d.Ck * 2;                                     // P: bf16 [FR][Ck]
-  int sc_bytes = FQ * d.Ck * 4;                                          // FQ score rows, later the nu ring
+  const int p_bytes = FR * CkP * 2;                                    // P: bf16 [FR][Ck]
+  int sc_bytes = FQ * CkP * 4;                                         // FQ score rows, later the nu ring
   if (sc_bytes < 2 * tile_bytes) sc_bytes = 2 * tile_bytes;
   int nsA = (p_bytes + sc_bytes) / tile_bytes, nsD = sc_bytes / tile_bytes;
   nsA = nsA > kMaxStA ? kMaxStA : nsA;
@@ -570,7 +573,7 @@ int far_fwd_tc(const Dims& d, const SummPtrs& sp, const void* Q, const int32_t* 
   prof_mark("k_far_fwd_tc", st);
   // TMEM columns: all FR x Ck scores of a pass (the output of phase D reuses them), a power of two >= 32
   int tcols = 32;
-  while (tcols < FR * (d.Ck / kFJ)) tcols *= 2;
+  while (tcols < FR * (CkP / kFJ)) tcols *= 2;
 #define MUSE_FAR_FWD_LAUNCH(FR_, FQ_, D_, NK_, MB_)                                                                              \
   do {                                                                                                                         \
     MUSE_CUDA_OK(cudaFuncSetAttribute(k_far_fwd_tc<FR_, FQ_, D_, NK_, MB_>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \

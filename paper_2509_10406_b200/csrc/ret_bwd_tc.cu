@@ -67,7 +67,7 @@ k_ret_bwd_pairs_tc(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__
   __shared__ uint32_t tbase_s;
   __shared__ int32_t ok_s[kOkCache];
   __shared__ int32_t tok_s[2][kPairs];                      // tokens of the tile each half is gathering
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = tc::warp_index(), lane = tid & 31;
   // With spatial block selection (k2 > 0) the CTA owns one BUCKET (cluster j, block bb): its pairs are the (query, slot,
   // chosen block) triples that chose the block, and every one of them sees the whole bucket (as in the forward kernel).
   const bool bucket = dm.k2 > 0;
@@ -288,7 +288,7 @@ k_ret_bwd_pairs_tc(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__
       const uint32_t ka = tc::smem_u32(sm + oK), va = tc::smem_u32(sm + oV);
       const uint32_t np0 = np;
       for (int tile = tile0; tile < ntiles; tile += tstep, ++np) {
-        if (lane == 0) {
+        {
           const uint32_t ph = np & 1;
           RBCLK(0)
           wait(&B.q_full, ph);                               // the tile's Q and dO rows are in shared memory
@@ -298,10 +298,10 @@ k_ret_bwd_pairs_tc(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__
           RBCLK(2)
           const uint32_t id1 = tc::idesc_bf16(kPairs, kKeys, 0, 0);
 #pragma unroll
-          for (int ks = 0; ks < D / 16; ++ks) tc::mma_bf16_ss(tbase + cS, desc_k<kPairs>(qa, ks), desc_k<kKeys>(ka, ks), id1, ks > 0);
+          for (int ks = 0; ks < D / 16; ++ks) tc::mma_bf16_ss_warp(tbase + cS, desc_k<kPairs>(qa, ks), desc_k<kKeys>(ka, ks), id1, ks > 0);
 #pragma unroll
-          for (int ks = 0; ks < D / 16; ++ks) tc::mma_bf16_ss(tbase + cDP, desc_k<kPairs>(da, ks), desc_k<kKeys>(va, ks), id1, ks > 0);
-          tc::mma_commit(&B.s_done);
+          for (int ks = 0; ks < D / 16; ++ks) tc::mma_bf16_ss_warp(tbase + cDP, desc_k<kPairs>(da, ks), desc_k<kKeys>(va, ks), id1, ks > 0);
+          tc::mma_commit_warp(&B.s_done);
           RBCLK(3)
           wait(&B.pg_ready, ph);                             // P and G are in shared memory, S and dP consumed
           tc::fence_after_sync();
@@ -313,15 +313,15 @@ k_ret_bwd_pairs_tc(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__
           const bool acc = np > np0;                                     // the accumulators start at zero in every sweep
 #pragma unroll
           for (int ks = 0; ks < kKeys / 16; ++ks)
-            tc::mma_bf16_ss(tbase + cDQ, tc::smem_desc_sw128(ga + ks * 32, 16, 1024), desc_mn<kKeys>(ka, ks), id_dq, ks > 0);
+            tc::mma_bf16_ss_warp(tbase + cDQ, tc::smem_desc_sw128(ga + ks * 32, 16, 1024), desc_mn<kKeys>(ka, ks), id_dq, ks > 0);
 #pragma unroll
           for (int ks = 0; ks < kPairs / 16; ++ks)
-            tc::mma_bf16_ss(tbase + cDV, desc_mn<kPairs>(da, ks), tc::smem_desc_sw128(pa + ks * 16 * 128, kPairs * 128, 1024), id_t, acc || ks > 0);
+            tc::mma_bf16_ss_warp(tbase + cDV, desc_mn<kPairs>(da, ks), tc::smem_desc_sw128(pa + ks * 16 * 128, kPairs * 128, 1024), id_t, acc || ks > 0);
 #pragma unroll
           for (int ks = 0; ks < kPairs / 16; ++ks)
-            tc::mma_bf16_ss(tbase + cDK, desc_mn<kPairs>(qa, ks), tc::smem_desc_sw128(ga + ks * 16 * 128, kPairs * 128, 1024), id_t, acc || ks > 0);
-          tc::mma_commit(&B.m2_done);
-          tc::mma_commit(&B.q_empty);                        // ... and the Q / dO tiles refilled
+            tc::mma_bf16_ss_warp(tbase + cDK, desc_mn<kPairs>(qa, ks), tc::smem_desc_sw128(ga + ks * 16 * 128, kPairs * 128, 1024), id_t, acc || ks > 0);
+          tc::mma_commit_warp(&B.m2_done);
+          tc::mma_commit_warp(&B.q_empty);                        // ... and the Q / dO tiles refilled
           RBCLK(5)
 #ifdef MUSE_PHASE_CLOCKS
           pc[7] += 1;
@@ -329,7 +329,7 @@ k_ret_bwd_pairs_tc(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__
         }
         __syncwarp();
       }
-      if (lane == 0 && np > np0) {                           // all products done before the key tiles are replaced or the CTA ends
+      if (np > np0) {                           // all products done before the key tiles are replaced or the CTA ends
         wait(&B.m2_done, (np - 1) & 1);
         tc::fence_after_sync();
       }

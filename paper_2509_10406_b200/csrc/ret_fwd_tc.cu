@@ -44,20 +44,6 @@ __device__ __forceinline__ void cp_async16(void* smem_dst, const void* src, bool
   const int n = valid ? 16 : 0;                            // 0 source bytes: the 16 bytes are zero-filled
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(tc::smem_u32(smem_dst)), "l"(src), "r"(n) : "memory");
 }
-// D[tmem] (+)= A[tmem] * B[smem]: A is a 128-row bf16 matrix in tensor memory, two K-elements per 32-bit column
-__device__ __forceinline__ void mma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n"
-      ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
-}
-// registers -> TMEM, 32 lanes x 16 columns; complete when the call returns
-__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&v)[16]) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
-      :: "r"(taddr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]), "r"(v[9]),
-         "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]) : "memory");
-  asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-}
 }  // namespace rf
 
 template <int D>
@@ -73,7 +59,7 @@ k_ret_fwd_pairs_tc(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__
   __shared__ uint32_t tbase_s;
   __shared__ int32_t ok_s[kOkCache];
   __shared__ int32_t tok_s[kPairs];                        // tokens of the tile being gathered
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = tc::warp_index(), lane = tid & 31;
   // Without spatial block selection the CTA owns a key cluster and its pairs of every plane (a query sees the cluster's
   // keys of the earlier blocks).  With it (k2 > 0) the CTA owns one BUCKET (cluster, block bb): its pairs are the
   // (query, slot, chosen block) triples that chose this block, and every one of them sees the whole bucket.
@@ -225,7 +211,8 @@ k_ret_fwd_pairs_tc(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__
               pk2[i / 2] = *reinterpret_cast<uint32_t*>(&b2);
             }
             // P over the logits already consumed: keys [32 g, 32 g + 32) -> columns [16 g, 16 g + 16)
-            tmem_st16(tl + SM::cS + 16 * g, pk2);
+            tc::tmem_st16_issue(tl + SM::cS + 16 * g, pk2);
+            tc::tmem_st_wait();
           }
           tc::fence_before_sync();
           tc::mbar_arrive(&bars.p_ready);
@@ -303,29 +290,29 @@ k_ret_fwd_pairs_tc(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__
         last = last_n;
         if (nk16 == 0) continue;
         const uint32_t ph = nproc & 1;
-        if (lane == 0) {
+        {
           wait(&bars.q_full, ph);                            // the tile's Q rows are in shared memory
           if (nproc > 0) wait(&bars.o_done, ph ^ 1);         // the previous product has read P: the logits may be overwritten
           tc::fence_after_sync();
           const uint32_t idesc = tc::idesc_bf16(kPairs, nk16, 0, 0);
 #pragma unroll
           for (int ks = 0; ks < D / 16; ++ks)
-            tc::mma_bf16_ss(tbase + SM::cS, tc::smem_desc_sw128(qa + (ks / 4) * kPairs * 128 + (ks % 4) * 32, 16, 1024),
+            tc::mma_bf16_ss_warp(tbase + SM::cS, tc::smem_desc_sw128(qa + (ks / 4) * kPairs * 128 + (ks % 4) * 32, 16, 1024),
                             tc::smem_desc_sw128(ka + (ks / 4) * kKeys * 128 + (ks % 4) * 32, 16, 1024), idesc, ks > 0);
-          tc::mma_commit(&bars.s_done);
-          tc::mma_commit(&bars.q_empty);                     // ... and the Q buffer refilled, once these products are done
+          tc::mma_commit_warp(&bars.s_done);
+          tc::mma_commit_warp(&bars.q_empty);                     // ... and the Q buffer refilled, once these products are done
           wait(&bars.p_ready, ph);                           // P is in tensor memory
           if (nproc > 0) wait(&bars.o_free, ph ^ 1);         // the previous output has been read out
           tc::fence_after_sync();
           const uint32_t idesc2 = tc::idesc_bf16(kPairs, D, 0, 1);
           for (int ks = 0; ks < nk16 / 16; ++ks)
-            mma_bf16_ts(tbase + SM::cO, tbase + SM::cS + 8 * ks, tc::smem_desc_sw128(va + ks * 16 * 128, kKeys * 128, 1024), idesc2, ks > 0);
-          tc::mma_commit(&bars.o_done);
+            tc::mma_bf16_ts_warp(tbase + SM::cO, tbase + SM::cS + 8 * ks, tc::smem_desc_sw128(va + ks * 16 * 128, kKeys * 128, 1024), idesc2, ks > 0);
+          tc::mma_commit_warp(&bars.o_done);
         }
         __syncwarp();
         ++nproc;
       }
-      if (lane == 0 && nproc > 0) {                          // all products done before the tiles are replaced or the CTA ends
+      if (nproc > 0) {                          // all products done before the tiles are replaced or the CTA ends
         wait(&bars.o_done, (nproc - 1) & 1);
         tc::fence_after_sync();
       }

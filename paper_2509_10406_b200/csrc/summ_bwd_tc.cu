@@ -1,5 +1,5 @@
 // Key-side pass of the backward through the accumulated summaries, on the tensor cores
-// (bf16 mode, D = 64 or 128, Cq a multiple of 8).  One CTA per (key cluster j, head).  For every
+// (bf16 mode, D = 64 or 128).  One CTA per (key cluster j, head).  For every
 // plane pl the summary (i, j, pl) was built from the keys u of cluster j in blocks <= pl, with
 // weights w_iu = exp(sigma qbar_i.k_u - mu_ij(pl)) <= 1.  Given the far-field gradients
 // (dkappa, dnu, dS) of that plane:
@@ -57,7 +57,7 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
   __shared__ uint32_t tbase_s;
   const int j = blockIdx.x, pq = blockIdx.y;
   const int b_ = pq / dm.Hq, h = pq % dm.Hq, pk = b_ * dm.Hkv + dm.hm.g[h];
-  const int tid = threadIdx.x, warp = tid >> 5, wg = tid >> 7, L = tid & 127;
+  const int tid = threadIdx.x, warp = tc::warp_index(), wg = tid >> 7, L = tid & 127;
   const bool cw = warp < 8;                               // compute warp (the ninth warp only issues)
   const int32_t* ok_ = off_k + (size_t)pk * (dm.Ck * dm.S + 1) + (size_t)j * dm.S;
   const int32_t* oq = off_q + (size_t)pq * (dm.S * dm.Cq + 1);
@@ -89,12 +89,12 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
 #endif
   for (int c0 = kbeg; c0 < kvis && ok; c0 += NU) {        // 64 keys of the cluster at a time (usually one chunk)
     __syncthreads();
-    if (tid == ISSUER) {
-      tc::mbar_expect_tx(&bar_kv, 2 * kKeys);
+    if (warp == ISSUER / 32) {
+      tc::mbar_expect_tx_warp(&bar_kv, 2 * kKeys);
       const int row = (int)((size_t)pk * dm.N + c0);
       for (int g = 0; g < G; ++g) {
-        tc::tma_load_2d(sm + oK + g * NU * 128, &tm_K, 64 * g, row, &bar_kv);
-        tc::tma_load_2d(sm + oV + g * NU * 128, &tm_V, 64 * g, row, &bar_kv);
+        tc::tma_load_2d_warp(sm + oK + g * NU * 128, &tm_K, 64 * g, row, &bar_kv);
+        tc::tma_load_2d_warp(sm + oV + g * NU * 128, &tm_V, 64 * g, row, &bar_kv);
       }
     }
     int pl0 = 0;                                          // planes [pl0, pl_end) see this chunk (bucket ends grow with the plane)
@@ -109,24 +109,23 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
       const bool in_range = cw && i < dm.Cq;
       const int ic = in_range ? i : 0;
       auto issue_grad = [&](int pl, int buf) {            // thread 0: both gradient tiles of (plane, j, i0..i0+127)
-        tc::mbar_expect_tx(&bar_g[buf], 2 * kTile);
-        const int row = (int)((((size_t)pq * dm.SB + pl) * dm.Ck + j) * dm.Cq + i0);
+        tc::mbar_expect_tx_warp(&bar_g[buf], 2 * kTile);
+        const int row = (pq * dm.SB + pl) * dm.Ck + j;    // (rows i >= Cq are zeros)
         unsigned char* dka = sm + (buf ? oQlo : oDka0);
         unsigned char* dnu = sm + (buf ? oDnu1 : oDnu0);
         for (int g = 0; g < G; ++g) {
-          tc::tma_load_2d(dka + g * TI * 128, &tm_dka, 64 * g, row, &bar_g[buf]);
-          tc::tma_load_2d(dnu + g * TI * 128, &tm_dnu, 64 * g, row, &bar_g[buf]);
+          tc::tma_load_3d_warp(dka + g * TI * 128, &tm_dka, 64 * g, i0, row, &bar_g[buf]);
+          tc::tma_load_3d_warp(dnu + g * TI * 128, &tm_dnu, 64 * g, i0, row, &bar_g[buf]);
         }
       };
       PCLK(7)
       __syncthreads();                                    // every MMA that read the centroid tiles has completed (bar2 waited)
-      if (tid == ISSUER) {
+      if (warp == ISSUER / 32) {
         // sigma * qbar tile as bf16 hi + lo operands (split once per layer), and the first gradient tiles
-        tc::mbar_expect_tx(&bar_q, 2 * kTile);
-        const int r = pq * dm.Cq + i0;
+        tc::mbar_expect_tx_warp(&bar_q, 2 * kTile);
         for (int g = 0; g < G; ++g) {
-          tc::tma_load_2d(sm + oQhi + g * TI * 128, &tm_qhi, 64 * g, r, &bar_q);
-          tc::tma_load_2d(sm + oQlo + g * TI * 128, &tm_qlo, 64 * g, r, &bar_q);
+          tc::tma_load_3d_warp(sm + oQhi + g * TI * 128, &tm_qhi, 64 * g, i0, pq, &bar_q);
+          tc::tma_load_3d_warp(sm + oQlo + g * TI * 128, &tm_qlo, 64 * g, i0, pq, &bar_q);
         }
         if (pl0 < pl_end) issue_grad(pl0, 0);
       }
@@ -138,19 +137,19 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
         if (in_range && (per_block || oq[(size_t)blk * dm.Cq + i + 1] > oq[(size_t)blk * dm.Cq + i])) livemask |= 1u << pl;
       }
       // tilt logits l_iu = sigma qbar_i . k_u, the same for every plane: once per centroid tile
-      if (tid == ISSUER) {
+      if (warp == ISSUER / 32) {
         if (!tc::mbar_wait(&bar_q, ph_q)) ok = false;
         tc::fence_after_sync();
         const uint32_t idesc = tc::idesc_bf16(TI, NU, 0, 0);
 #pragma unroll
         for (int ks = 0; ks < D / 16; ++ks)
-          tc::mma_bf16_ss(tbase + cL, tc::smem_desc_sw128(aQhi + (ks / 4) * TI * 128 + (ks % 4) * 32, 16, 1024),
+          tc::mma_bf16_ss_warp(tbase + cL, tc::smem_desc_sw128(aQhi + (ks / 4) * TI * 128 + (ks % 4) * 32, 16, 1024),
                           tc::smem_desc_sw128(aK + (ks / 4) * NU * 128 + (ks % 4) * 32, 16, 1024), idesc, ks > 0);
 #pragma unroll
         for (int ks = 0; ks < D / 16; ++ks)
-          tc::mma_bf16_ss(tbase + cL, tc::smem_desc_sw128(aQlo + (ks / 4) * TI * 128 + (ks % 4) * 32, 16, 1024),
+          tc::mma_bf16_ss_warp(tbase + cL, tc::smem_desc_sw128(aQlo + (ks / 4) * TI * 128 + (ks % 4) * 32, 16, 1024),
                           tc::smem_desc_sw128(aK + (ks / 4) * NU * 128 + (ks % 4) * 32, 16, 1024), idesc, 1);
-        tc::mma_commit(&bar_l);
+        tc::mma_commit_warp(&bar_l);
       }
       ph_q ^= 1;
       __syncwarp();
@@ -182,19 +181,19 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
         // tiles go to the tensor cores as they land.  The D-contractions of this plane do not depend on the
         // previous plane's i-contractions: they are issued first, and only the W / Wc tiles and the other
         // gradient buffer wait for those.
-        if (tid == ISSUER) {
+        if (warp == ISSUER / 32) {
           if (!tc::mbar_wait(&bar_g[buf], ph_g[buf])) ok = false;
           tc::fence_after_sync();
           const uint32_t idesc = tc::idesc_bf16(TI, NU, 0, 0);
 #pragma unroll
           for (int ks = 0; ks < D / 16; ++ks)
-            tc::mma_bf16_ss(tbase + cX1, tc::smem_desc_sw128(aDka + (ks / 4) * TI * 128 + (ks % 4) * 32, 16, 1024),
+            tc::mma_bf16_ss_warp(tbase + cX1, tc::smem_desc_sw128(aDka + (ks / 4) * TI * 128 + (ks % 4) * 32, 16, 1024),
                             tc::smem_desc_sw128(aK + (ks / 4) * NU * 128 + (ks % 4) * 32, 16, 1024), idesc, ks > 0);
 #pragma unroll
           for (int ks = 0; ks < D / 16; ++ks)
-            tc::mma_bf16_ss(tbase + cX2, tc::smem_desc_sw128(aDnu + (ks / 4) * TI * 128 + (ks % 4) * 32, 16, 1024),
+            tc::mma_bf16_ss_warp(tbase + cX2, tc::smem_desc_sw128(aDnu + (ks / 4) * TI * 128 + (ks % 4) * 32, 16, 1024),
                             tc::smem_desc_sw128(aV + (ks / 4) * NU * 128 + (ks % 4) * 32, 16, 1024), idesc, ks > 0);
-          tc::mma_commit(&bar1);
+          tc::mma_commit_warp(&bar1);
           if (k > 0 && !tc::mbar_wait(&bar2, ph2)) ok = false;      // the previous plane's MMAs are done with the other buffer
           if (pl + 1 < pl_end && ok) issue_grad(pl + 1, buf ^ 1);
         }
@@ -228,26 +227,26 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
         tc::fence_async_smem();
         tc::fence_before_sync();
         __syncthreads();
-        if (tid == ISSUER) {
+        if (warp == ISSUER / 32) {
           tc::fence_after_sync();
           // A [i][d] and B [i][u]: both contract over rows.  M = 128 output dims even when D = 64: the second 64-dim group
           // of the A operand is then the tile that follows in shared memory, and output lanes 64..127 hold numbers that nobody reads
           const uint32_t idesc = tc::idesc_bf16(128, NU, 1, 1);
 #pragma unroll
           for (int ks = 0; ks < TI / 16; ++ks)
-            tc::mma_bf16_ss(tbase + cDK, tc::smem_desc_sw128(aDka + ks * 16 * 128, TI * 128, 1024),
+            tc::mma_bf16_ss_warp(tbase + cDK, tc::smem_desc_sw128(aDka + ks * 16 * 128, TI * 128, 1024),
                             tc::smem_desc_sw128(aW + ks * 16 * 128, TI * 128, 1024), idesc, started || ks > 0);
           if (dm.agg_grad) {
 #pragma unroll
             for (int ks = 0; ks < TI / 16; ++ks)
-              tc::mma_bf16_ss(tbase + cDK, tc::smem_desc_sw128(aQhi + ks * 16 * 128, TI * 128, 1024),
+              tc::mma_bf16_ss_warp(tbase + cDK, tc::smem_desc_sw128(aQhi + ks * 16 * 128, TI * 128, 1024),
                               tc::smem_desc_sw128(aWc + ks * 16 * 128, TI * 128, 1024), idesc, 1);
           }
 #pragma unroll
           for (int ks = 0; ks < TI / 16; ++ks)
-            tc::mma_bf16_ss(tbase + cDV, tc::smem_desc_sw128(aDnu + ks * 16 * 128, TI * 128, 1024),
+            tc::mma_bf16_ss_warp(tbase + cDV, tc::smem_desc_sw128(aDnu + ks * 16 * 128, TI * 128, 1024),
                             tc::smem_desc_sw128(aW + ks * 16 * 128, TI * 128, 1024), idesc, started || ks > 0);
-          tc::mma_commit(&bar2);
+          tc::mma_commit_warp(&bar2);
         }
         started = true;
         __syncwarp();
@@ -292,10 +291,11 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
 }
 
 bool summ_bwd_tc_supported(const Dims& d, int dtype) {
-  return dtype == MUSE_BF16 && (d.D == 64 || d.D == 128) && d.Cq % 8 == 0;
+  return dtype == MUSE_BF16 && (d.D == 64 || d.D == 128);
 }
 
 int make_tmap_bf16_rows(void* out_map, const void* base, uint64_t rows, uint32_t cols, uint32_t box_rows);
+int make_tmap_bf16_nd(void* out_map, const void* base, int rank, const uint64_t* dims, const uint64_t* strides_bytes, const uint32_t* box);
 
 int summ_bwd_tc(const Dims& d, const void* Kp, const void* Vp, const int32_t* off_k, const int32_t* off_q, const float* qbar,
                 const float* mu, const void* dkappa, const void* dnu, const float* dS, float* dK_perm, float* dV_perm,
@@ -305,14 +305,15 @@ int summ_bwd_tc(const Dims& d, const void* Kp, const void* Vp, const int32_t* of
   bf16* qlo = qhi + (size_t)d.B * d.Hq * d.Cq * d.D;
   int rcq = split_qbar(d, qbar, qhi, qlo, st);
   if (rcq != MUSE_OK) return rcq;
-  CUtensorMap tqh, tql;
-  rcq = make_tmap_bf16_rows(&tqh, qhi, (uint64_t)d.B * d.Hq * d.Cq, d.D, sb::TI);
-  if (rcq == MUSE_OK) rcq = make_tmap_bf16_rows(&tql, qlo, (uint64_t)d.B * d.Hq * d.Cq, d.D, sb::TI);
-  if (rcq != MUSE_OK) return rcq;
-  CUtensorMap tdka, tdnu, tK, tV;
-  const uint64_t grows = (uint64_t)d.B * d.Hq * d.SB * d.Ck * d.Cq;       // gradient entries, [plane][j][i]
-  int rc = make_tmap_bf16_rows(&tdka, dkappa, grows, d.D, sb::TI);
-  if (rc == MUSE_OK) rc = make_tmap_bf16_rows(&tdnu, dnu, grows, d.D, sb::TI);
+  const uint64_t Dd = (uint64_t)d.D, Cq = (uint64_t)d.Cq;
+  const uint64_t str[2] = {Dd * 2, Cq * Dd * 2};
+  const uint64_t dims_q[3] = {Dd, Cq, (uint64_t)d.B * d.Hq}, dims_g[3] = {Dd, Cq, (uint64_t)d.B * d.Hq * d.SB * d.Ck};   // gradients [plane][j][i]
+  const uint32_t box[3] = {64, (uint32_t)sb::TI, 1};
+  CUtensorMap tqh, tql, tdka, tdnu, tK, tV;
+  int rc = make_tmap_bf16_nd(&tqh, qhi, 3, dims_q, str, box);
+  if (rc == MUSE_OK) rc = make_tmap_bf16_nd(&tql, qlo, 3, dims_q, str, box);
+  if (rc == MUSE_OK) rc = make_tmap_bf16_nd(&tdka, dkappa, 3, dims_g, str, box);
+  if (rc == MUSE_OK) rc = make_tmap_bf16_nd(&tdnu, dnu, 3, dims_g, str, box);
   if (rc == MUSE_OK) rc = make_tmap_bf16_rows(&tK, Kp, (uint64_t)d.B * d.Hkv * d.N, d.D, sb::NU);
   if (rc == MUSE_OK) rc = make_tmap_bf16_rows(&tV, Vp, (uint64_t)d.B * d.Hkv * d.N, d.D, sb::NU);
   if (rc != MUSE_OK) return rc;

@@ -67,7 +67,7 @@ k_summarize_tc(Dims dm, const __grid_constant__ CUtensorMap tm_K, const __grid_c
   __shared__ uint32_t tbase_s;
   const int j = blockIdx.x, i0 = blockIdx.y * TI, pq = blockIdx.z;
   const int b_ = pq / dm.Hq, h = pq % dm.Hq, pk = b_ * dm.Hkv + dm.hm.g[h];
-  const int tid = threadIdx.x, warp = tid >> 5, wg = tid >> 7, row = tid & 127, i = i0 + row;
+  const int tid = threadIdx.x, warp = tc::warp_index(), wg = tid >> 7, row = tid & 127, i = i0 + row;
   unsigned char* sm = sm_raw + ((1024u - (tc::smem_u32(sm_raw) & 1023u)) & 1023u);
   const int32_t* off = off_k + (size_t)pk * (dm.Ck * dm.S + 1) + (size_t)j * dm.S;
   if (warp == 0) tc::tmem_alloc(&tbase_s, 512);
@@ -76,12 +76,12 @@ k_summarize_tc(Dims dm, const __grid_constant__ CUtensorMap tm_K, const __grid_c
   __syncthreads();
   tc::fence_after_sync();
   // sigma * qbar tile as bf16 hi and lo operands, split once per layer and loaded here by TMA
-  if (tid == 0) {
-    tc::mbar_expect_tx(&bar_q, 2 * kTile);
+  if (warp == 0) {
+    tc::mbar_expect_tx_warp(&bar_q, 2 * kTile);
     const int r = pq * dm.Cq + i0;
     for (int g = 0; g < G; ++g) {
-      tc::tma_load_2d(sm + oQhi + g * TI * 128, &tm_qhi, 64 * g, r, &bar_q);
-      tc::tma_load_2d(sm + oQlo + g * TI * 128, &tm_qlo, 64 * g, r, &bar_q);
+      tc::tma_load_2d_warp(sm + oQhi + g * TI * 128, &tm_qhi, 64 * g, r, &bar_q);
+      tc::tma_load_2d_warp(sm + oQlo + g * TI * 128, &tm_qlo, 64 * g, r, &bar_q);
     }
   }
   const uint32_t tbase = tbase_s, tlane = tbase + ((uint32_t)((warp & 3) * 32) << 16);
@@ -107,12 +107,12 @@ k_summarize_tc(Dims dm, const __grid_constant__ CUtensorMap tm_K, const __grid_c
   // A bucket usually holds far fewer than 64 keys: only the 16-key groups in use are loaded and contracted.
   auto issue_kv = [&](int c0, int nk) {
     const int ng_ = (nk + 15) >> 4;
-    tc::mbar_expect_tx(&bar_kv, ng_ * 2 * G * (16 * 128));
+    tc::mbar_expect_tx_warp(&bar_kv, ng_ * 2 * G * (16 * 128));
     const int r = (int)((size_t)pk * dm.N + c0);
     for (int g = 0; g < ng_; ++g)
       for (int cg = 0; cg < G; ++cg) {
-        tc::tma_load_2d(sm + oK + cg * NU * 128 + g * 16 * 128, &tm_K, 64 * cg, r + 16 * g, &bar_kv);
-        tc::tma_load_2d(sm + oV + cg * NU * 128 + g * 16 * 128, &tm_V, 64 * cg, r + 16 * g, &bar_kv);
+        tc::tma_load_2d_warp(sm + oK + cg * NU * 128 + g * 16 * 128, &tm_K, 64 * cg, r + 16 * g, &bar_kv);
+        tc::tma_load_2d_warp(sm + oV + cg * NU * 128 + g * 16 * 128, &tm_V, 64 * cg, r + 16 * g, &bar_kv);
       }
   };
   auto issue_after = [&](int c_end) {                  // the chunk that starts at key c_end, if any
@@ -120,7 +120,7 @@ k_summarize_tc(Dims dm, const __grid_constant__ CUtensorMap tm_K, const __grid_c
     while (npl < dm.SB && off[npl + 1] <= c_end) ++npl;
     if (npl < dm.SB) issue_kv(c_end, min(NU, off[npl + 1] - c_end));
   };
-  if (tid == 32) issue_after(off[0]);
+  if (warp == 1) issue_after(off[0]);
   for (int pl = 0; pl < dm.SB && ok; ++pl) {
     const int p0 = off[pl], p1 = off[pl + 1];
     (void)MUSE_IN_RANGE(p1, dm.N + 1); (void)MUSE_IN_RANGE(p0, p1 + 1);     // (the tiles come through tensor maps, which clip)
@@ -134,20 +134,20 @@ k_summarize_tc(Dims dm, const __grid_constant__ CUtensorMap tm_K, const __grid_c
       PCLK(0)
       __syncthreads();
       const int ng = (nk + 15) >> 4;
-      if (tid == 0) {
+      if (warp == 0) {
         if (!q_ready) { if (!tc::mbar_wait(&bar_q, 0)) ok = false; q_ready = true; }
         if (!tc::mbar_wait(&bar_kv, ph_kv)) ok = false;
         tc::fence_after_sync();
         const uint32_t idesc = tc::idesc_bf16(TI, 16 * ng, 0, 0);
 #pragma unroll
         for (int ks = 0; ks < D / 16; ++ks)
-          tc::mma_bf16_ss(tbase + cL, tc::smem_desc_sw128(aQhi + (ks / 4) * TI * 128 + (ks % 4) * 32, 16, 1024),
+          tc::mma_bf16_ss_warp(tbase + cL, tc::smem_desc_sw128(aQhi + (ks / 4) * TI * 128 + (ks % 4) * 32, 16, 1024),
                           tc::smem_desc_sw128(aK + (ks / 4) * NU * 128 + (ks % 4) * 32, 16, 1024), idesc, ks > 0);
 #pragma unroll
         for (int ks = 0; ks < D / 16; ++ks)
-          tc::mma_bf16_ss(tbase + cL, tc::smem_desc_sw128(aQlo + (ks / 4) * TI * 128 + (ks % 4) * 32, 16, 1024),
+          tc::mma_bf16_ss_warp(tbase + cL, tc::smem_desc_sw128(aQlo + (ks / 4) * TI * 128 + (ks % 4) * 32, 16, 1024),
                           tc::smem_desc_sw128(aK + (ks / 4) * NU * 128 + (ks % 4) * 32, 16, 1024), idesc, 1);
-        tc::mma_commit(&bar1);
+        tc::mma_commit_warp(&bar1);
       }
       ph_kv ^= 1;
       __syncwarp();
@@ -189,24 +189,24 @@ k_summarize_tc(Dims dm, const __grid_constant__ CUtensorMap tm_K, const __grid_c
       tc::fence_before_sync();
       __syncthreads();
       PCLK(2)
-      if (tid == 0) {
+      if (warp == 0) {
         tc::fence_after_sync();
         const uint32_t idesc = tc::idesc_bf16(TI, D, 0, 1);          // A = W (K-major over keys), B = key rows (MN-major)
         for (int ks = 0; ks < ng; ++ks) {
-          tc::mma_bf16_ss(tbase + cUk, tc::smem_desc_sw128(aWhi + ks * 32, 16, 1024), tc::smem_desc_sw128(aK + ks * 16 * 128, NU * 128, 1024), idesc, ks > 0);
-          tc::mma_bf16_ss(tbase + cUv, tc::smem_desc_sw128(aWhi + ks * 32, 16, 1024), tc::smem_desc_sw128(aV + ks * 16 * 128, NU * 128, 1024), idesc, ks > 0);
+          tc::mma_bf16_ss_warp(tbase + cUk, tc::smem_desc_sw128(aWhi + ks * 32, 16, 1024), tc::smem_desc_sw128(aK + ks * 16 * 128, NU * 128, 1024), idesc, ks > 0);
+          tc::mma_bf16_ss_warp(tbase + cUv, tc::smem_desc_sw128(aWhi + ks * 32, 16, 1024), tc::smem_desc_sw128(aV + ks * 16 * 128, NU * 128, 1024), idesc, ks > 0);
         }
         for (int ks = 0; ks < ng; ++ks) {
-          tc::mma_bf16_ss(tbase + cUk, tc::smem_desc_sw128(aWlo + ks * 32, 16, 1024), tc::smem_desc_sw128(aK + ks * 16 * 128, NU * 128, 1024), idesc, 1);
-          tc::mma_bf16_ss(tbase + cUv, tc::smem_desc_sw128(aWlo + ks * 32, 16, 1024), tc::smem_desc_sw128(aV + ks * 16 * 128, NU * 128, 1024), idesc, 1);
+          tc::mma_bf16_ss_warp(tbase + cUk, tc::smem_desc_sw128(aWlo + ks * 32, 16, 1024), tc::smem_desc_sw128(aK + ks * 16 * 128, NU * 128, 1024), idesc, 1);
+          tc::mma_bf16_ss_warp(tbase + cUv, tc::smem_desc_sw128(aWlo + ks * 32, 16, 1024), tc::smem_desc_sw128(aV + ks * 16 * 128, NU * 128, 1024), idesc, 1);
         }
-        tc::mma_commit(&bar2);
+        tc::mma_commit_warp(&bar2);
       }
       __syncwarp();
       if (!tc::mbar_wait(&bar2, ph2)) ok = false;
       ph2 ^= 1;
       tc::fence_after_sync();
-      if (tid == 32 && ok) issue_after(c0 + nk);         // key / value tiles are free again (not thread 0: it issues the MMAs)
+      if (warp == 1 && ok) issue_after(c0 + nk);         // key / value tiles are free again (not thread 0: it issues the MMAs)
       PCLK(3)
 #pragma unroll
       for (int d0 = 0; d0 < D; d0 += 32) {              // acc[0..D/2): kappa dims (D/2) wg.., acc[D/2..D): nu dims (D/2) wg..
@@ -233,7 +233,7 @@ k_summarize_tc(Dims dm, const __grid_constant__ CUtensorMap tm_K, const __grid_c
     }
     // kappa hi / lo (warpgroup 0) and nu (warpgroup 1) as swizzled [128 rows][2 x 128 B] tiles; they leave
     // by TMA (rows of consecutive query clusters are Ck entries apart in memory) while the next plane is computed
-    if (tid == 0) tc::tma_store_wait_read();                           // the previous plane's stores have read the tiles
+    if (warp == 0) tc::tma_store_wait_read_warp();                           // the previous plane's stores have read the tiles
     __syncthreads();
     // this warpgroup's half of the row (dims [HD wg, HD wg + HD)) in 16-byte chunks of 8 dims: chunk c of column group gq
 #pragma unroll
@@ -255,21 +255,21 @@ k_summarize_tc(Dims dm, const __grid_constant__ CUtensorMap tm_K, const __grid_c
     }
     tc::fence_async_smem();
     __syncthreads();
-    if (tid == 0 && ok) {
+    if (warp == 0 && ok) {
       const int P = pq * dm.SB + pl;
       for (int g = 0; g < G; ++g) {
-        tc::tma_store_4d(&tm_okhi, sm + oStage + g * TI * 128, 64 * g, j, i0, P);
-        tc::tma_store_4d(&tm_oklo, sm + oStage + kTile + g * TI * 128, 64 * g, j, i0, P);
-        tc::tma_store_4d(&tm_onu, sm + oStage + 2 * kTile + g * TI * 128, 64 * g, j, i0, P);
+        tc::tma_store_4d_warp(&tm_okhi, sm + oStage + g * TI * 128, 64 * g, j, i0, P);
+        tc::tma_store_4d_warp(&tm_oklo, sm + oStage + kTile + g * TI * 128, 64 * g, j, i0, P);
+        tc::tma_store_4d_warp(&tm_onu, sm + oStage + 2 * kTile + g * TI * 128, 64 * g, j, i0, P);
       }
-      tc::tma_store_commit();
+      tc::tma_store_commit_warp();
     }
     PCLK(5)
   }
 #ifdef MUSE_PHASE_CLOCKS
   if (tid == 0 && blockIdx.x == 5 && blockIdx.y == 0 && blockIdx.z == 0) for (int k = 0; k < 8; ++k) status[56 + k] = (int)pc[k];
 #endif
-  if (tid == 0) tc::tma_store_wait_all();
+  if (warp == 0) tc::tma_store_wait_all_warp();
   tc::fence_before_sync();
   __syncthreads();
   if (warp == 0) tc::tmem_dealloc(tbase, 512);

@@ -1,0 +1,49 @@
+"""GPU: the tensor-core far-field and key-side kernels at cluster counts that no tile divides, and both sides of the
+streaming clustering in one call against each side alone."""
+import numpy as np
+import pytest
+import torch
+
+from tests.gpu_util import to_np
+from tests.test_gpu_backward import _backward_parity
+from tests.test_gpu_cluster import CASES
+from tests.test_gpu_forward import TC_BWD_KERNELS, TC_FWD_KERNELS, _forward_parity
+
+pytestmark = pytest.mark.gpu
+
+RAGGED = [("d64", 5, 1, 1, 3), ("d64", 130, 127, 5, 4), ("d128", 9, 129, 8, 3), ("d128", 37, 300, 16, 4), ("d128", 3, 1100, 8, 3)]
+
+
+@pytest.mark.parametrize("base,Cq,Ck,m,S", RAGGED)
+def test_forward_at_ragged_cluster_counts(base, Cq, Ck, m, S):
+    w = CASES[base].with_(Hq=2, Hkv=1, N=510 * S, S=S, Cq=Cq, Ck=Ck, m=m, components=64)
+    _forward_parity(w, 128.0, expect_kernels=TC_FWD_KERNELS)
+
+
+@pytest.mark.parametrize("base,Cq,Ck,m,S", RAGGED)
+def test_backward_at_ragged_cluster_counts(base, Cq, Ck, m, S):
+    w = CASES[base].with_(Hq=2, Hkv=1, N=510 * S, S=S, Cq=Cq, Ck=Ck, m=m, components=64)
+    _backward_parity(w, 128.0, expect_kernels=TC_BWD_KERNELS)
+
+
+@pytest.mark.parametrize("Hq,Hkv,D,Cq,Ck,cap", [(2, 1, 64, 20, 600, 1.25), (4, 4, 128, 130, 40, 1.5), (1, 1, 64, 64, 33, 4.0)])
+def test_streaming_both_sides_at_once_equals_each_side_alone(Hq, Hkv, D, Cq, Ck, cap):
+    from paper_2509_10406_b200 import binding as mb
+    N, S = 4000, 4
+    g = torch.Generator(device="cuda").manual_seed(Cq)
+    Q, K = (torch.randn(1, h, N, D, generator=g, device="cuda").bfloat16() for h in (Hq, Hkv))
+    p = mb.make_params(B=1, Hq=Hq, Hkv=Hkv, N=N, D=D, Cq=Cq, Ck=Ck, m=0, n_blocks=S, seed=11)
+    e = lambda *s, dt=torch.float32: torch.empty(*s, dtype=dt, device="cuda")  # noqa: E731
+    ws = e(mb.muse_stream_workspace_bytes(p), dt=torch.uint8)
+    both = [e(1, Hq, N, dt=torch.int32), e(1, Hkv, N, dt=torch.int32), e(1, Hq, Cq, D), e(1, Hkv, Ck, D)]
+    mb.muse_cluster_streaming(p, Q, K, *both, ws, cap_factor=cap)
+    torch.cuda.synchronize()
+    assert mb.muse_status(ws) == 0
+    for side, X, H, C, assign, cen in ((0, Q, Hq, Cq, both[0], both[2]), (1, K, Hkv, Ck, both[1], both[3])):
+        tot, cnt, c1, a1 = e(1, H, C, D), e(1, H, C), e(1, H, C, D), e(1, H, N, dt=torch.int32)
+        mb.muse_stream_kmeans(p, X, side, tot, cnt, c1, ws)
+        mb.muse_balanced_assign(p, X, side, c1, a1, ws, cap_factor=cap)
+        torch.cuda.synchronize()
+        assert np.array_equal(to_np(c1), to_np(cen)) and np.array_equal(to_np(a1), to_np(assign))
+        size = np.bincount(to_np(a1)[0, 0, :N // S], minlength=C)
+        assert size.sum() == N // S and size.max() <= max(1, int(np.ceil(cap * (N // S) / C)))
