@@ -235,15 +235,29 @@ int muse_cluster(const muse_params_t* p, const void* Q, const void* K, const int
 
 static size_t up256(size_t x) { return (x + 255) & ~size_t(255); }
 
+// muse_cluster_streaming: the balanced assignment's scratch for both sides, then each side's streaming state
+struct StreamWs { float *totals[2], *counts[2]; size_t total; };
+static StreamWs stream_ws(const Dims& d, void* ws) {
+  const int problems[2] = {d.B * d.Hq, d.B * d.Hkv}, C[2] = {d.Cq, d.Ck};
+  StreamWs w;
+  size_t at = up256(balanced_ws_bytes(d, problems, C, 2));
+  for (int k = 0; k < 2; ++k) {
+    const size_t rows = (size_t)problems[k] * C[k];
+    w.totals[k] = reinterpret_cast<float*>((char*)ws + at);
+    at += up256(rows * d.D * sizeof(float));
+    w.counts[k] = reinterpret_cast<float*>((char*)ws + at);
+    at += up256(rows * sizeof(float));
+  }
+  w.total = at;
+  return w;
+}
+
 int muse_stream_workspace_bytes(const muse_params_t* p, size_t* bytes) {
   Dims d;
   int rc = resolve(p, &d);
   if (rc != MUSE_OK) return rc;
   if (bytes == nullptr) return MUSE_ERR_INVALID_ARG;
-  const size_t pq = (size_t)d.B * d.Hq, pk = (size_t)d.B * d.Hkv;
-  const size_t bal = std::max(balanced_ws_bytes(d, (int)pq, d.Cq), balanced_ws_bytes(d, (int)pk, d.Ck));
-  const size_t tot = std::max(pq * d.Cq, pk * d.Ck);
-  *bytes = up256(bal) + up256(tot * d.D * sizeof(float)) + up256(tot * sizeof(float));
+  *bytes = stream_ws(d, nullptr).total;
   return MUSE_OK;
 }
 
@@ -276,8 +290,8 @@ int muse_stream_kmeans(const muse_params_t* p, const void* X, int side, float be
   if (!(beta > 0.f) || beta > 1.f) return MUSE_ERR_INVALID_ARG;
   if (ws_bytes < 256) return MUSE_ERR_WORKSPACE;
   if (clear_status(ws, stream) != MUSE_OK) return MUSE_ERR_CUDA;
-  rc = stream_kmeans(d, p->dtype, X, side == 0 ? d.B * d.Hq : d.B * d.Hkv, side == 0 ? d.Cq : d.Ck, side, p->seed, beta,
-                     first_batch, n_batches, totals, counts, centres, assign_stream, (int32_t*)ws, stream);
+  const StreamSide s = {X, totals, counts, centres, assign_stream, side == 0 ? d.B * d.Hq : d.B * d.Hkv, side == 0 ? d.Cq : d.Ck, side};
+  rc = stream_kmeans(d, p->dtype, &s, 1, p->seed, beta, first_batch, n_batches, (int32_t*)ws, stream);
   prof_mark(nullptr, stream);
   return rc;
 }
@@ -290,9 +304,10 @@ int muse_balanced_assign(const muse_params_t* p, const void* X, int side, const 
   if (!X || !centres || !assign || !ws || (side != 0 && side != 1)) return MUSE_ERR_INVALID_ARG;
   if (!aligned16(X) || !aligned16(centres) || !aligned16(ws)) return MUSE_ERR_INVALID_ARG;
   const int problems = side == 0 ? d.B * d.Hq : d.B * d.Hkv, C = side == 0 ? d.Cq : d.Ck;
-  if (ws_bytes < balanced_ws_bytes(d, problems, C)) return MUSE_ERR_WORKSPACE;
+  if (ws_bytes < balanced_ws_bytes(d, &problems, &C, 1)) return MUSE_ERR_WORKSPACE;
   if (clear_status(ws, stream) != MUSE_OK) return MUSE_ERR_CUDA;
-  rc = balanced_assign(d, p->dtype, X, problems, C, side, centres, cap_factor, assign, ws, stream);
+  const BalancedSide s = {X, centres, assign, problems, C, side};
+  rc = balanced_assign(d, p->dtype, &s, 1, cap_factor, ws, stream);
   prof_mark(nullptr, stream);
   return rc;
 }
@@ -308,26 +323,25 @@ int muse_cluster_streaming(const muse_params_t* p, const void* Q, const void* K,
   size_t need = 0;
   muse_stream_workspace_bytes(p, &need);
   if (ws_bytes < need) return MUSE_ERR_WORKSPACE;
-  if (clear_status(ws, stream) != MUSE_OK) return MUSE_ERR_CUDA;
-  const size_t pq = (size_t)d.B * d.Hq, pk = (size_t)d.B * d.Hkv;
-  const size_t bal = up256(std::max(balanced_ws_bytes(d, (int)pq, d.Cq), balanced_ws_bytes(d, (int)pk, d.Ck)));
-  const size_t tot = std::max(pq * d.Cq, pk * d.Ck);
-  float* totals = reinterpret_cast<float*>((char*)ws + bal);
-  float* counts = reinterpret_cast<float*>((char*)ws + bal + up256(tot * d.D * sizeof(float)));
+  const StreamWs w = stream_ws(d, ws);
+  StreamSide ss[2];
+  BalancedSide bs[2];
+  int n = 0;
   for (int side = 0; side < 2; ++side) {
     const void* X = side == 0 ? Q : K;
     if (X == nullptr) continue;
     int32_t* assign = side == 0 ? assign_q : assign_k;
     float* cen = side == 0 ? qbar : kcent;
     if (assign == nullptr || cen == nullptr || !aligned16(X) || !aligned16(cen)) return MUSE_ERR_INVALID_ARG;
-    const int problems = side == 0 ? (int)pq : (int)pk, C = side == 0 ? d.Cq : d.Ck;
-    rc = stream_kmeans(d, p->dtype, X, problems, C, side, p->seed, beta, 0, -1, totals, counts, cen, nullptr, (int32_t*)ws, stream);
-    if (rc != MUSE_OK) return rc;
-    rc = balanced_assign(d, p->dtype, X, problems, C, side, cen, cap_factor, assign, ws, stream);
-    if (rc != MUSE_OK) return rc;
+    const int problems = d.B * (side == 0 ? d.Hq : d.Hkv), C = side == 0 ? d.Cq : d.Ck;
+    ss[n] = StreamSide{X, w.totals[side], w.counts[side], cen, nullptr, problems, C, side};
+    bs[n++] = BalancedSide{X, cen, assign, problems, C, side};
   }
+  if (clear_status(ws, stream) != MUSE_OK) return MUSE_ERR_CUDA;
+  rc = stream_kmeans(d, p->dtype, ss, n, p->seed, beta, 0, -1, (int32_t*)ws, stream);
+  if (rc == MUSE_OK) rc = balanced_assign(d, p->dtype, bs, n, cap_factor, ws, stream);
   prof_mark(nullptr, stream);
-  return MUSE_OK;
+  return rc;
 }
 
 int muse_summarize(const muse_params_t* p, const void* K, const void* V, const int32_t* assign_k,

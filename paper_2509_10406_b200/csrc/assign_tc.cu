@@ -36,7 +36,7 @@ constexpr int kRows = 128, kCols = kAsgTile, kThreads = (8 + kXProd + kCProd + 1
 
 struct Bars { uint64_t xfull[kXStages], xempty[kXStages], full[kMaxPieces], empty[kMaxPieces], tfull[2][2], tempty[2][2]; };
 
-struct Side { const float* cnorm; int32_t* assign; float* dist; int problems, C, NT, upp; };   // upp = units per problem
+struct Side { const float* cnorm; int32_t* assign; float* dist; const int32_t* flags; int problems, C, NT, upp; };   // upp = units per problem
 struct Args { Side s[2]; int N, ns; };
 
 // Walks the units whose cost interval starts inside this CTA's share of the total cost (a unit costs NT).
@@ -68,7 +68,16 @@ struct Walk {
   }
 };
 
-template <int D, int R, bool DIST>     // R: point tiles per unit; DIST: also write the matrix |c|^2 - 2 x.c (the balanced assignment's second step reads it)
+// DIST: the units without a flagged point tile are passed over by every role
+template <int R> __device__ __forceinline__ bool flagged(const Args& g, const Walk& w) {
+  const Side& sd = g.s[w.side];
+  const int tiles = (g.N + kRows - 1) / kRows;
+  int f = 0;
+  for (int r = 0; r < R; ++r) if (w.u * R + r < tiles) f |= sd.flags[(size_t)w.prob * tiles + w.u * R + r];
+  return f != 0;
+}
+
+template <int D, int R, bool DIST>     // R: point tiles per unit; DIST: write |c|^2 - 2 x.c of the flagged tiles instead of the assignments
 __global__ void __launch_bounds__(kThreads, 1)
 k_assign_tc(const __grid_constant__ CUtensorMap tx0, const __grid_constant__ CUtensorMap th0, const __grid_constant__ CUtensorMap tl0,
             const __grid_constant__ CUtensorMap tx1, const __grid_constant__ CUtensorMap th1, const __grid_constant__ CUtensorMap tl1,
@@ -100,7 +109,8 @@ k_assign_tc(const __grid_constant__ CUtensorMap tx0, const __grid_constant__ CUt
   if (warp >= 8 && warp < 8 + kXProd) {
     if ((tid & 31) == 0) {                                 // ---- points: this thread takes every kXProd-th tile
       int turn = warp - 8;
-      for (int s = 0, ph = 0; w.more() && ok; w.next(g))
+      for (int s = 0, ph = 0; w.more() && ok; w.next(g)) {
+        if (DIST && !flagged<R>(g, w)) continue;
         for (int r = 0; r < R; ++r) {
           if (turn == 0) {
             if (!tc::mbar_wait(&bars.xempty[s], ph ^ 1)) { ok = false; break; }
@@ -113,6 +123,7 @@ k_assign_tc(const __grid_constant__ CUtensorMap tx0, const __grid_constant__ CUt
           turn = turn == 0 ? kXProd - 1 : turn - 1;
           if (++s == kXStages) { s = 0; ph ^= 1; }
         }
+      }
     }
   } else if (warp >= 8 + kXProd && warp < 8 + kXProd + kCProd) {
     if ((tid & 31) == 0) {                                 // ---- centre pieces: this thread takes every kCProd-th piece
@@ -120,7 +131,8 @@ k_assign_tc(const __grid_constant__ CUtensorMap tx0, const __grid_constant__ CUt
       bool fresh = true;
       for (int s = 0, ph = 0; w.more() && ok; fresh = w.next(g)) {
         const Side& sd = g.s[w.side];
-        if (sd.NT * PPT <= ns && !fresh) continue;         // resident
+        if (DIST && !flagged<R>(g, w)) continue;
+        if (!DIST && sd.NT * PPT <= ns && !fresh) continue;         // resident
         for (int t = 0; t < sd.NT && ok; ++t)
 #pragma unroll
           for (int p = 0; p < PPT; ++p) {
@@ -142,8 +154,9 @@ k_assign_tc(const __grid_constant__ CUtensorMap tx0, const __grid_constant__ CUt
     int s = 0, ph = 0, x = 0, xph = 0, b = 0, bph = 0;
     int s0 = 0;                                            // first ring slot of a resident problem
     while (w.more() && ok) {
+      if (DIST && !flagged<R>(g, w)) { w.next(g); continue; }
       const int NT = g.s[w.side].NT;
-      const bool res = NT * PPT <= ns;
+      const bool res = !DIST && NT * PPT <= ns;            // (with units passed over, a problem's first and last are not known)
       uint64_t dx[R];
       int xs[R];
 #pragma unroll
@@ -194,6 +207,7 @@ k_assign_tc(const __grid_constant__ CUtensorMap tx0, const __grid_constant__ CUt
     const int row = tid & 127, r = warp >> 2;
     const uint32_t tlane = tbase + ((uint32_t)((warp & 3) * 32) << 16) + r * 2 * kCols;
     for (int b = 0, bph = 0; w.more() && ok; w.next(g)) {
+      if (DIST && !flagged<R>(g, w)) continue;
       const Side& sd = g.s[w.side];
       const int C = sd.C, at = (w.u * R + r) * kRows + row;
       const float* cn = sd.cnorm + (size_t)w.prob * sd.NT * kCols;
@@ -221,9 +235,9 @@ k_assign_tc(const __grid_constant__ CUtensorMap tx0, const __grid_constant__ CUt
             v[k + 2] = fmaf(-2.f, v[k + 2], n4.z); v[k + 3] = fmaf(-2.f, v[k + 3], n4.w);
 #pragma unroll
             for (int e = 0; e < 4; ++e)
-              argmin_step(v[k + e], c0 + k + e, best[e], bidx[e]);      // ascending index: ties keep the lower
+              if (!DIST) argmin_step(v[k + e], c0 + k + e, best[e], bidx[e]);      // ascending index: ties keep the lower
           }
-          if (DIST && at < N) {                            // optional output: the whole matrix |c|^2 - 2 x.c
+          if (DIST && at < N) {
             float* dr = sd.dist + ((size_t)w.prob * N + at) * C + c0;
             if (c0 + 32 <= C && (C & 3) == 0) {
 #pragma unroll
@@ -237,10 +251,9 @@ k_assign_tc(const __grid_constant__ CUtensorMap tx0, const __grid_constant__ CUt
         b ^= 1; bph ^= b == 0;
       }
 #pragma unroll
-      for (int e = 1; e < 4; ++e)
-        if (best[e] < best[0] || (best[e] == best[0] && bidx[e] < bidx[0])) { best[0] = best[e]; bidx[0] = bidx[e]; }
+      for (int e = 1; e < 4; ++e) argmin_tie_step(best[e], bidx[e], best[0], bidx[0]);
       // a row of NaN or infinities never compares below the running minimum: it goes to cluster 0
-      if (ok && at < N) sd.assign[(size_t)w.prob * N + at] = (unsigned)bidx[0] < (unsigned)C ? bidx[0] : 0;
+      if (!DIST && ok && at < N) sd.assign[(size_t)w.prob * N + at] = (unsigned)bidx[0] < (unsigned)C ? bidx[0] : 0;
     }
   }
   if (!ok) report_status(status, MUSE_STATUS_ASSIGN_TIMEOUT);
@@ -251,10 +264,10 @@ k_assign_tc(const __grid_constant__ CUtensorMap tx0, const __grid_constant__ CUt
 
 }  // namespace at
 
-int assign_tc(const LloydSide* sides, int nsides, int N, int D, int* status, cudaStream_t st) {
+int assign_tc(const LloydSide* sides, int nsides, int N, int D, int distances, int* status, cudaStream_t st) {
   at::Args g = {};
   CUtensorMap m[6];
-  bool dist = false;
+  const bool dist = distances != 0;
   const int sms = sm_count();
   long long tiles = 0;
   for (int k = 0; k < nsides; ++k) tiles += (long long)sides[k].problems * cdiv(N, at::kRows);
@@ -267,9 +280,8 @@ int assign_tc(const LloydSide* sides, int nsides, int N, int D, int* status, cud
     MUSE_RC(make_tmap_bf16_rows(&m[3 * k], s.X, (uint64_t)s.problems * N, (uint32_t)D, at::kRows));
     MUSE_RC(make_tmap_bf16_rows(&m[3 * k + 1], s.chi, (uint64_t)s.problems * s.C, (uint32_t)D, at::kCols));
     MUSE_RC(make_tmap_bf16_rows(&m[3 * k + 2], s.clo, (uint64_t)s.problems * s.C, (uint32_t)D, at::kCols));
-    g.s[k] = at::Side{s.cnorm, s.assign, s.dist, k < nsides ? s.problems : 0, s.C, cdiv(s.C, at::kCols), cdiv(N, at::kRows * R)};
+    g.s[k] = at::Side{s.cnorm, s.assign, s.dist, s.flags, k < nsides ? s.problems : 0, s.C, cdiv(s.C, at::kCols), cdiv(N, at::kRows * R)};
     units += (long long)g.s[k].problems * g.s[k].upp;
-    dist = dist || (k < nsides && s.dist != nullptr);
   }
   const int grid = units < sms ? (int)units : sms;
   const size_t smem = (size_t)at::kXStages * at::kRows * D * 2 + (size_t)g.ns * at::kPiece + 1024;

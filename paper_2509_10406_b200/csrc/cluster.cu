@@ -70,7 +70,7 @@ constexpr int kAsgThreads = 256;
 
 template <int D, int RPT, int CPT>
 __global__ void __launch_bounds__(kAsgThreads)
-k_assign(const __grid_constant__ LloydSides g, int write_dist) {
+k_assign(const __grid_constant__ LloydSides g, int distances) {
   constexpr int LD = D + 4, ROWS = 16 * RPT, COLS = 16 * CPT;
   extern __shared__ float smf[];
   float* Xs = smf;                       // [ROWS][LD]
@@ -88,7 +88,8 @@ k_assign(const __grid_constant__ LloydSides g, int write_dist) {
   const float* Xp = (const float*)sd.X + (size_t)prob * N * D;
   const float* Cp = sd.centres + (size_t)prob * C * D;
   const float* cnp = sd.cnorm + cnorm_index(prob, 0, C);
-  float* dist_out = write_dist ? sd.dist : nullptr;
+  if (distances && sd.flags[(size_t)prob * cdiv(N, kAsgTile) + row0 / kAsgTile] == 0) return;
+  float* dist_out = distances ? sd.dist : nullptr;
   for (int e = tid; e < ROWS * (D / 4); e += kAsgThreads) {
     int r = e / (D / 4), q = e % (D / 4);
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -157,19 +158,19 @@ k_assign(const __grid_constant__ LloydSides g, int write_dist) {
 }
 
 template <int D, int RPT, int CPT>
-static int assign_f32_v(const LloydSides& g, int nprob, int write_dist, cudaStream_t st) {
+static int assign_f32_v(const LloydSides& g, int nprob, int distances, cudaStream_t st) {
   const size_t smem = (size_t)((16 * RPT + 16 * CPT) * (D + 4) + 16 * CPT) * sizeof(float);
-  return launch_pdl(k_assign<D, RPT, CPT>, dim3(cdiv(g.N, 16 * RPT), nprob), kAsgThreads, smem, st, g, write_dist);
+  return launch_pdl(k_assign<D, RPT, CPT>, dim3(cdiv(g.N, 16 * RPT), nprob), kAsgThreads, smem, st, g, distances);
 }
 
 template <int D>
-static int assign_f32(const LloydSides& g, int nsides, int write_dist, cudaStream_t st) {
+static int assign_f32(const LloydSides& g, int nsides, int distances, cudaStream_t st) {
   int nprob = 0, C = 0;
   for (int k = 0; k < nsides; ++k) { nprob += g.s[k].problems; C = C > g.s[k].C ? C : g.s[k].C; }
   prof_mark("k_assign", st);
-  if ((long long)nprob * cdiv(g.N, 128) >= 2 * sm_count()) return assign_f32_v<D, 8, 4>(g, nprob, write_dist, st);   // two rounds of full tiles
-  if (C > 16) return assign_f32_v<D, 2, 4>(g, nprob, write_dist, st);
-  return assign_f32_v<D, 2, 1>(g, nprob, write_dist, st);
+  if ((long long)nprob * cdiv(g.N, 128) >= 2 * sm_count()) return assign_f32_v<D, 8, 4>(g, nprob, distances, st);   // two rounds of full tiles
+  if (C > 16) return assign_f32_v<D, 2, 4>(g, nprob, distances, st);
+  return assign_f32_v<D, 2, 1>(g, nprob, distances, st);
 }
 
 // Centre update: mean of the members, summed with a fixed reduction tree (slot s of the CTA adds members
@@ -289,11 +290,9 @@ static int lloyd_t(LloydSides& g, const Dims& d, int nsides, int init_mode, uint
   for (int it = 0; it <= T_iters; ++it) {
     const bool last = it == T_iters;
     if (sizeof(T) == 2) {                      // bf16 inputs: distances on the tensor cores
-      LloydSide s[2] = {g.s[0], g.s[1]};
-      if (!last) s[0].dist = s[1].dist = nullptr;
-      MUSE_RC(assign_tc(s, nsides, d.N, D, status, st));
+      MUSE_RC(assign_tc(g.s, nsides, d.N, D, 0, status, st));
     } else {
-      MUSE_RC(assign_f32<D>(g, nsides, last, st));
+      MUSE_RC(assign_f32<D>(g, nsides, 0, st));
     }
     if (last) break;
     MUSE_RC(bucket_sort(sort, nsides, d.N, d.S, d.Bs, st));
@@ -301,6 +300,14 @@ static int lloyd_t(LloydSides& g, const Dims& d, int nsides, int init_mode, uint
     MUSE_RC(launch_pdl(k_update<T, D>, dim3((unsigned)centres), kUpdThreads, 0, st, g));
   }
   return MUSE_OK;
+}
+
+int assign_distances(const Dims& d, int dtype, const LloydSide& side, int* status, cudaStream_t st) {
+  if (dtype == MUSE_BF16) return assign_tc(&side, 1, d.N, d.D, 1, status, st);
+  LloydSides g = {};
+  g.s[0] = side;
+  g.N = d.N; g.S = d.S;
+  return d.D == 64 ? assign_f32<64>(g, 1, 1, st) : assign_f32<128>(g, 1, 1, st);
 }
 
 void lloyd_side_ws(const Dims& d, Arena& ar, LloydSide& s) {

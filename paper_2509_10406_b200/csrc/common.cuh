@@ -89,10 +89,14 @@ template <int EPL> __device__ __forceinline__ void stv(__nv_bfloat16* p, const f
   else { __nv_bfloat162 b = __floats2bfloat162_rn(x[0], x[1]); *reinterpret_cast<uint32_t*>(p) = *reinterpret_cast<uint32_t*>(&b); }
 }
 
-// One step of a running arg-min, as two selects: left to itself the compiler turns the comparison into a branch, and a
-// sweep over a row of distances then costs a divergence per element.  A NaN never compares below the minimum.
+// One step of a running arg-min as two selects (left to itself the compiler makes a branch of the comparison).  A NaN
+// never compares below the minimum.  The second form is for candidates in any order: the lower index on a tie.
 __device__ __forceinline__ void argmin_step(float v, int i, float& best, int& bidx) {
   asm("{\n.reg .pred p;\nsetp.lt.f32 p, %2, %0;\nselp.f32 %0, %2, %0, p;\nselp.b32 %1, %3, %1, p;\n}\n" : "+f"(best), "+r"(bidx) : "f"(v), "r"(i));
+}
+__device__ __forceinline__ void argmin_tie_step(float v, int i, float& best, int& bidx) {
+  asm("{\n.reg .pred p, q, r;\nsetp.lt.f32 p, %2, %0;\nsetp.eq.f32 q, %2, %0;\nsetp.lt.and.s32 r, %3, %1, q;\nor.pred p, p, r;\n"
+      "selp.f32 %0, %2, %0, p;\nselp.b32 %1, %3, %1, p;\n}\n" : "+f"(best), "+r"(bidx) : "f"(v), "r"(i));
 }
 
 __device__ __forceinline__ float warp_sum(float v) {
@@ -198,24 +202,26 @@ struct LloydSide {
   const void* X; int problems, C, kind;
   const int32_t* init_idx;
   int32_t* assign; float* centres;
-  float* dist;                             // [problems, N, C] |c|^2 - 2 x.c of the final assignment (optional)
+  float* dist;                             // assign_distances: [problems, N, C] |c|^2 - 2 x.c ...
+  const int32_t* flags;                    // ... of the 128-vector tiles flagged here [problems, ceil(N / 128)]
   float* cnorm; int32_t* off; int32_t* perm; void* chi; void* clo;
 };
 void lloyd_side_ws(const Dims& d, Arena& ar, LloydSide& s);
 int lloyd(const Dims& d, int dtype, LloydSide* sides, int nsides, int init_mode, uint64_t seed, int T, int* status, cudaStream_t st);
 size_t lloyd_ws_bytes(const Dims& d, int problems, int C);      // scratch of one side (without the status words)
-int assign_tc(const LloydSide* sides, int nsides, int N, int D, int* status, cudaStream_t st);
+int assign_tc(const LloydSide* sides, int nsides, int N, int D, int distances, int* status, cudaStream_t st);
+int assign_distances(const Dims& d, int dtype, const LloydSide& side, int* status, cudaStream_t st);   // after lloyd on the same centres
 
 // the paper's own clustering: one streaming pass (state = totals, counts; n_batches < 0: to the end) and the
 // per-block assignment under a bucket-size cap (factor <= 0: plain nearest centroid)
 int kmeanspp(int dtype, const void* X, int problems, int N, int D, int C, int kind, uint64_t seed, float* mind2,
              int32_t* idx_out, int* status, cudaStream_t st);
-int stream_kmeans(const Dims& d, int dtype, const void* X, int problems, int C, int kind, uint64_t seed, float beta,
-                  int first_batch, int n_batches, float* totals, float* counts, float* centres, int32_t* assign_stream,
+struct StreamSide { const void* X; float *totals, *counts, *centres; int32_t* assign_stream; int problems, C, kind; };
+int stream_kmeans(const Dims& d, int dtype, const StreamSide* sides, int n, uint64_t seed, float beta, int first_batch, int n_batches,
                   int32_t* status, cudaStream_t st);
-int balanced_assign(const Dims& d, int dtype, const void* X, int problems, int C, int kind, const float* centres, float factor,
-                    int32_t* assign, void* ws, cudaStream_t st);
-size_t balanced_ws_bytes(const Dims& d, int problems, int C);
+struct BalancedSide { const void* X; const float* centres; int32_t* assign; int problems, C, kind; };
+int balanced_assign(const Dims& d, int dtype, const BalancedSide* sides, int n, float factor, void* ws, cudaStream_t st);
+size_t balanced_ws_bytes(const Dims& d, const int* problems, const int* C, int n);
 
 // assign_k == nullptr: the keys are already bucketed (off_k, perm_k are inputs) and `status` names the
 // caller's status words; counts / ksum / vsum (untilted per-bucket statistics) may be nullptr
