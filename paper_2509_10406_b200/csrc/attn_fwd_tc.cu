@@ -165,193 +165,6 @@ __device__ __forceinline__ void tc_teardown(TcCtx& c, int tid, int* status) {
   if (!c.ok && tid == 0) report_status(status, 1);
 }
 
-// ---- local (block-diagonal) attention ------------------------------------------------------------
-// 256 threads: thread (row, warpgroup w) owns key columns [32 w, 32 w + 32) of every 64-key tile and
-// output dims [D/2 w, D/2 w + D/2) of its row; the two halves of a row share the running maximum
-// through shared memory.  Software pipeline over the key tiles t (K and V tiles arrive by TMA):
-//   S(t+1) = Q K_{t+1}^T is issued as soon as S(t) has landed (two S buffers in TMEM, two K tiles in
-//   shared memory), so it runs while the threads do the softmax of tile t; O(t) = P(t) V_t is
-//   awaited at the start of iteration t + 1, which frees P and V for tile t + 1; O accumulates in TMEM.
-constexpr int kLfThreads = 256;
-
-template <int D> struct LfSmem {
-  static constexpr int q = 0, k = q + kTcM * D * 2, v = k + 2 * kTcN * D * 2, p = v + kTcN * D * 2, total = p + kTcM * kTcN * 2 + 1024;
-};
-
-template <int D>
-__global__ void __launch_bounds__(kLfThreads, 2)
-k_local_fwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
-               const bf16* __restrict__ Q, float* __restrict__ o_loc, float* __restrict__ lse_loc, int* __restrict__ status) {
-  extern __shared__ __align__(1024) unsigned char sm_raw[];
-  __shared__ uint64_t barS[2], barK[2], barV, barPV;
-  __shared__ uint32_t tbase_s;
-  __shared__ float mx_s[2][kTcM];
-  constexpr int HD = D / 2, kKB = kTcN * D * 2;
-  constexpr uint32_t cO = 2 * kTcN;                        // TMEM: S0 | S1 | O
-  const int tid = threadIdx.x, warp = tid >> 5, row = tid & 127, wg = tid >> 7;
-  unsigned char* sm = sm_raw + ((1024u - (tc::smem_u32(sm_raw) & 1023u)) & 1023u);
-  unsigned char *Qs = sm + LfSmem<D>::q, *Ks = sm + LfSmem<D>::k, *Vs = sm + LfSmem<D>::v, *Ps = sm + LfSmem<D>::p;
-  if (warp == 0) tc::tmem_alloc(&tbase_s, 256);
-  if (tid == 0) {
-    tc::mbar_init(&barS[0], 1); tc::mbar_init(&barS[1], 1); tc::mbar_init(&barK[0], 1); tc::mbar_init(&barK[1], 1);
-    tc::mbar_init(&barV, 1); tc::mbar_init(&barPV, 1); tc::mbar_init_fence();
-  }
-  const int tpb = cdiv(dm.Bs, kTcM);
-  // heaviest tiles (latest in a block) first
-  const int lin = blockIdx.x, qt = tpb - 1 - lin / dm.S, blk = lin % dm.S, pq = blockIdx.y;
-  const int b_ = pq / dm.Hq, h = pq % dm.Hq, pk = b_ * dm.Hkv + dm.hm.g[h];
-  const int bstart = blk * dm.Bs, bend = bstart + dm.Bs;
-  const int q0 = bstart + qt * kTcM, nq = min(kTcM, bend - q0);
-  const bf16* Qb = Q + (size_t)pq * dm.N * D;
-  const int k_lo = bstart, k_hi = q0 + nq;                  // causal: keys up to the tile's last row
-  const int T = (k_hi - k_lo + kTcN - 1) / kTcN;
-  const int krow0 = pk * dm.N + k_lo;                       // row of the first key in the [B*Hkv*N][D] tensors
-  for (int e = tid; e < kTcM * (D / 8); e += kLfThreads) {
-    const int r = e / (D / 8), ck = e % (D / 8);
-    uint4 v = make_uint4(0u, 0u, 0u, 0u);
-    if (r < nq) v = reinterpret_cast<const uint4*>(Qb + (size_t)(q0 + r) * D)[ck];
-    *reinterpret_cast<uint4*>(Qs + (ck >> 3) * kTcM * 128 + tc::sw128_off(r, ck & 7)) = v;
-  }
-  tc::fence_async_smem();
-  tc::fence_before_sync();
-  __syncthreads();
-  tc::fence_after_sync();
-  const uint32_t tbase = tbase_s, tl = tbase + ((uint32_t)((warp & 3) * 32) << 16);
-  const uint32_t qa = tc::smem_u32(Qs), ka = tc::smem_u32(Ks), va = tc::smem_u32(Vs), pa = tc::smem_u32(Ps);
-  bool ok = true;
-  // Thread 0 issues the MMAs, thread 32 the tile loads: a bulk-tensor instruction holds its thread for some
-  // 270 clocks per 16 KB box, and every row of the tile waits for thread 0 at the next barrier.
-  // Rows past the block's visible keys are loaded too (they are masked).
-  auto load_k = [&](int t) {
-    tc::mbar_expect_tx(&barK[t & 1], kKB);
-    for (int g = 0; g < D / 64; ++g) tc::tma_load_2d(Ks + (t & 1) * kKB + g * kTcN * 128, &tm_k, 64 * g, krow0 + t * kTcN, &barK[t & 1]);
-  };
-  auto load_v = [&](int t) {
-    tc::mbar_expect_tx(&barV, kKB);
-    for (int g = 0; g < D / 64; ++g) tc::tma_load_2d(Vs + g * kTcN * 128, &tm_v, 64 * g, krow0 + t * kTcN, &barV);
-  };
-  auto issue_s = [&](int t) {                               // S(t) = Q K_t^T into S buffer t & 1
-    if (!tc::mbar_wait(&barK[t & 1], (t >> 1) & 1)) ok = false;
-    tc::fence_after_sync();
-    const uint32_t idesc = tc::idesc_bf16(kTcM, kTcN, 0, 0);
-    const uint32_t kat = ka + (t & 1) * kKB;
-#pragma unroll
-    for (int ks = 0; ks < D / 16; ++ks)
-      tc::mma_bf16_ss(tbase + (t & 1) * kTcN, tc::smem_desc_sw128(qa + (ks / 4) * kTcM * 128 + (ks % 4) * 32, 16, 1024),
-                      tc::smem_desc_sw128(kat + (ks / 4) * kTcN * 128 + (ks % 4) * 32, 16, 1024), idesc, ks > 0);
-    tc::mma_commit(&barS[t & 1]);
-  };
-  if (tid == 32) {
-    load_k(0);
-    if (T > 1) load_k(1);
-  }
-  if (tid == 0) issue_s(0);
-  const float scale2 = dm.sigma * 1.4426950408889634f;
-  const int my_limit = q0 + row;                            // last visible key of this row
-  // The output accumulates in TMEM over all key tiles.  m2 is the exponent base in use for this row (log2
-  // units): it follows the running maximum lazily, only when that has grown by more than kLazy (probabilities
-  // then stay below 2^kLazy), and only then is the accumulator rescaled, for every row of the tile at once.
-  constexpr float kLazy = 8.f;
-  float m2 = -INFINITY, l = 0.f;                            // l: this warpgroup's share of the row sum
-  for (int t = 0; t < T && ok; ++t) {
-    const int c0 = k_lo + t * kTcN, nk = min(kTcN, k_hi - c0);
-    if (!tc::mbar_wait(&barS[t & 1], (t >> 1) & 1)) { ok = false; break; }
-    tc::fence_after_sync();
-    if (tid == 0 && t + 1 < T) issue_s(t + 1);              // runs during this tile's softmax
-    __syncwarp();
-    if (t > 0) {                                            // O(t-1) has landed: P and V are free (thread 0 has seen it too)
-      if (!tc::mbar_wait(&barPV, (t - 1) & 1)) ok = false;
-      tc::fence_after_sync();
-    }
-    if (tid == 32) {
-      load_v(t);
-      if (t + 2 < T) load_k(t + 2);                         // over K_t, which S(t) has consumed
-    }
-    float s[32];
-    tc::tmem_ld32(tl + (t & 1) * kTcN + 32 * wg, s);
-    const int vis = min(nk, my_limit - c0 + 1) - 32 * wg;  // visible columns among this thread's 32
-    float mx = -INFINITY;
-#pragma unroll
-    for (int i = 0; i < 32; ++i) { s[i] = i < vis ? s[i] * scale2 : -INFINITY; mx = fmaxf(mx, s[i]); }
-    mx_s[wg][row] = mx;
-    // (the first tile gives every row a finite maximum: it holds the block's first key)
-    const int grow = __syncthreads_or(t > 0 && mx > m2 + kLazy);
-    const float mt = fmaxf(mx_s[0][row], mx_s[1][row]);
-    if (t == 0) {
-      m2 = mt;
-    } else if (grow) {
-      const float mn = mt > m2 + kLazy ? mt : m2;           // rows that did not grow keep their base (factor 1)
-      const float resc = tc::fast_exp2(m2 - mn);
-#pragma unroll
-      for (int d0 = 0; d0 < HD; d0 += 32) {
-        float v[32];
-        tc::tmem_ld32(tl + cO + wg * HD + d0, v);
-#pragma unroll
-        for (int i = 0; i < 32; ++i) v[i] *= resc;
-        tc::tmem_st32(tl + cO + wg * HD + d0, v);
-      }
-      l *= resc;
-      m2 = mn;
-    }
-    const float base = m2 == -INFINITY ? 0.f : m2;
-    float rs = 0.f;
-#pragma unroll
-    for (int ch = 0; ch < 4; ++ch) {
-      uint32_t pk[4];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        __nv_bfloat162 b = __floats2bfloat162_rn(tc::fast_exp2(s[8 * ch + 2 * e] - base), tc::fast_exp2(s[8 * ch + 2 * e + 1] - base));
-        rs += __low2float(b) + __high2float(b);             // the rounded values, as the P V product sees them
-        pk[e] = *reinterpret_cast<uint32_t*>(&b);
-      }
-      *reinterpret_cast<uint4*>(Ps + tc::sw128_off(row, 4 * wg + ch)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-    }
-    l += rs;
-    tc::fence_async_smem();
-    tc::fence_before_sync();
-    __syncthreads();
-    if (tid == 0) {
-      if (!tc::mbar_wait(&barV, t & 1)) ok = false;
-      tc::fence_after_sync();
-      const uint32_t idesc = tc::idesc_bf16(kTcM, D, 0, 1);
-#pragma unroll
-      for (int ks = 0; ks < kTcN / 16; ++ks)
-        tc::mma_bf16_ss(tbase + cO, tc::smem_desc_sw128(pa + ks * 32, 16, 1024),
-                        tc::smem_desc_sw128(va + ks * 16 * 128, kTcN * 128, 1024), idesc, t > 0 || ks > 0);
-      tc::mma_commit(&barPV);
-    }
-    __syncwarp();
-  }
-  if (ok && T > 0) {
-    if (!tc::mbar_wait(&barPV, (T - 1) & 1)) ok = false;
-    tc::fence_after_sync();
-  }
-  // the two halves of the row sum meet
-  __syncthreads();
-  mx_s[wg][row] = l;
-  __syncthreads();
-  const float lt = mx_s[0][row] + mx_s[1][row];
-  if (ok && T > 0) {
-    const size_t t = (size_t)pq * dm.N + q0 + row;
-    const float inv = 1.f / lt;
-    float4* dst = reinterpret_cast<float4*>(o_loc + t * D + wg * HD);
-#pragma unroll
-    for (int d0 = 0; d0 < HD; d0 += 32) {
-      float v[32];
-      tc::tmem_ld32(tl + cO + wg * HD + d0, v);
-      if (row < nq) {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) dst[d0 / 4 + i] = make_float4(v[4 * i] * inv, v[4 * i + 1] * inv, v[4 * i + 2] * inv, v[4 * i + 3] * inv);
-      }
-    }
-    if (wg == 0 && row < nq) lse_loc[t] = (m2 + log2f(lt)) * 0.6931471805599453f;
-  }
-  tc::fence_before_sync();
-  __syncthreads();
-  if (warp == 0) tc::tmem_dealloc(tbase, 256);
-  if (!ok && tid == 0) report_status(status, 1);
-}
-
 // ---- exact retrieval ---------------------------------------------------------------------------------
 // A popular cluster is retrieved by thousands of queries of a block: its 128-pair tiles are
 // spread over kRetFwdSplit CTAs.
@@ -411,28 +224,6 @@ k_ret_fwd_tc(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ Kp, c
     }
   }
   tc_teardown<D>(c, tid, status);
-}
-
-int make_tmap_bf16_rows(void* out_map, const void* base, uint64_t rows, uint32_t cols, uint32_t box_rows);
-
-int local_fwd_tc(const Dims& d, const void* Q, const void* K, const void* V, float* o_loc, float* lse_loc, int* status,
-                 cudaStream_t st) {
-  const int pq = d.B * d.Hq;
-  CUtensorMap tk, tv;
-  int rc = make_tmap_bf16_rows(&tk, K, (uint64_t)d.B * d.Hkv * d.N, (uint32_t)d.D, kTcN);
-  if (rc == MUSE_OK) rc = make_tmap_bf16_rows(&tv, V, (uint64_t)d.B * d.Hkv * d.N, (uint32_t)d.D, kTcN);
-  if (rc != MUSE_OK) return rc;
-  dim3 grid(d.S * cdiv(d.Bs, kTcM), pq);
-  prof_mark("k_local_fwd_tc", st);
-  if (d.D == 128) {
-    MUSE_CUDA_OK(cudaFuncSetAttribute(k_local_fwd_tc<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, LfSmem<128>::total));
-    k_local_fwd_tc<128><<<grid, kLfThreads, LfSmem<128>::total, st>>>(d, tk, tv, (const bf16*)Q, o_loc, lse_loc, status);
-  } else {
-    MUSE_CUDA_OK(cudaFuncSetAttribute(k_local_fwd_tc<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, LfSmem<64>::total));
-    k_local_fwd_tc<64><<<grid, kLfThreads, LfSmem<64>::total, st>>>(d, tk, tv, (const bf16*)Q, o_loc, lse_loc, status);
-  }
-  MUSE_LAUNCH_OK();
-  return MUSE_OK;
 }
 
 int ret_fwd_pairs_tc(const Dims& d, const void* Q, const void* Kp, const void* Vp, const int32_t* off_k, const int32_t* goff,
