@@ -16,7 +16,6 @@
 namespace muse {
 
 typedef __nv_bfloat16 bf16;
-int make_tmap_bf16_rows(void* out_map, const void* base, uint64_t rows, uint32_t cols, uint32_t box_rows);
 constexpr int kBM = 128, kBN = 64;
 constexpr float kLog2e = 1.4426950408889634f;
 
@@ -196,51 +195,6 @@ __device__ __forceinline__ bool dq_rows_tc(BwdCtx& c, const bf16* __restrict__ K
     tc::fence_after_sync();
   }
   return !first;          // false: no key tile was processed, the accumulator holds nothing
-}
-
-// Reads this thread's accumulator row (D columns starting at column `col`), scales it by `f`
-// and, if `write`, stores it.  The TMEM load is warp-collective, so EVERY thread of the CTA
-// must call this; only the global store is predicated.
-template <int D>
-__device__ __forceinline__ void read_acc_row(const BwdCtx& c, uint32_t col, float f, float* __restrict__ dst, bool write, int tid) {
-  const uint32_t t = c.tbase + ((uint32_t)(((tid >> 5) & 3) * 32) << 16) + col;
-#pragma unroll
-  for (int d0 = 0; d0 < D; d0 += 32) {
-    float v[32];
-    tc::tmem_ld32(t + d0, v);
-    if (write) {
-#pragma unroll
-      for (int i = 0; i < 32; i += 4)
-        *reinterpret_cast<float4*>(dst + d0 + i) = make_float4(v[i] * f, v[i + 1] * f, v[i + 2] * f, v[i + 3] * f);
-    }
-  }
-}
-
-template <int D>
-__global__ void __launch_bounds__(kRowsThreads)
-k_local_bwd_dq_tc(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ K, const bf16* __restrict__ V,
-                  const bf16* __restrict__ dO, const float* __restrict__ LSE, const float* __restrict__ delta,
-                  float* __restrict__ dQacc, int* __restrict__ status) {
-  extern __shared__ __align__(1024) unsigned char sm_raw[];
-  __shared__ uint64_t bar[2];
-  __shared__ uint32_t tbase_s;
-  const int tid = threadIdx.x, row = tid & 127, wg = tid >> 7;
-  BwdCtx c;
-  bwd_setup(c, sm_raw, bar, &tbase_s, RowsSmem<D>::cols, tid);
-  const int tpb = cdiv(dm.Bs, kBM);
-  const int lin = blockIdx.x, qt = tpb - 1 - lin / dm.S, blk = lin % dm.S, pq = blockIdx.y;
-  const int b_ = pq / dm.Hq, h = pq % dm.Hq, pk = b_ * dm.Hkv + dm.hm.g[h];
-  const int bstart = blk * dm.Bs, bend = bstart + dm.Bs;
-  const int q0 = bstart + qt * kBM, nq = min(kBM, bend - q0);
-  const bf16* Qb = Q + (size_t)pq * dm.N * D; const bf16* dOb = dO + (size_t)pq * dm.N * D;
-  const bf16* Kb = K + (size_t)pk * dm.N * D; const bf16* Vb = V + (size_t)pk * dm.N * D;
-  fill_tile<D, kBM, kRowsThreads>(c.sm + RowsSmem<D>::q, nq, [&](int r) { return Qb + (size_t)(q0 + r) * D; }, tid);
-  fill_tile<D, kBM, kRowsThreads>(c.sm + RowsSmem<D>::dO, nq, [&](int r) { return dOb + (size_t)(q0 + r) * D; }, tid);
-  const size_t t = (size_t)pq * dm.N + q0 + row;
-  const float L2 = row < nq ? LSE[t] * kLog2e : 0.f, dl = row < nq ? delta[t] : 0.f;
-  dq_rows_tc<D>(c, Kb, Vb, bstart, q0 + nq, [&](int r) { return q0 + r; }, dm.sigma * kLog2e, L2, dl, tid);
-  if (c.ok) read_acc_row<D / 2>(c, 2 * kBN + wg * (D / 2), dm.sigma, dQacc + t * D + wg * (D / 2), row < nq, tid);   // each warpgroup half a row
-  bwd_teardown(c, RowsSmem<D>::cols, tid, status);
 }
 
 constexpr int kRetSplitRows = 4;      // CTAs sharing the 128-pair tiles of one (cluster, plane) group
@@ -428,211 +382,6 @@ __device__ __forceinline__ void dkdv_step_tc(BwdCtx& c, const float* __restrict_
 
 constexpr int kKeysThreads = 256;       // keys-on-M kernels: two warpgroups share the 64 query columns
 
-// Local (block-diagonal) dK, dV: one CTA = 128 keys of a block against the query tiles (64 rows) that see
-// them.  Software pipeline over the query tiles t, all operand tiles by TMA:
-//   MMA1(t+1) (S^T = K Q^T, dP^T = V dO^T into the second accumulator buffer) is issued as soon as
-//   MMA1(t) has landed, so it runs while the threads turn S^T(t), dP^T(t) into P^T, G^T;
-//   MMA2(t) (dV += P^T dO, dK += G^T Q) runs during the next iteration; Q / dO tiles sit in a ring of
-//   three, refilled as soon as the MMAs that read a slot have completed.
-template <int D> struct LdkSmem {
-  static constexpr int k = 0, v = k + kBM * D * 2, qd = v + kBM * D * 2, tile = 2 * kBN * D * 2,       // ring slot = Q tile | dO tile
-                       pt = qd + 3 * tile, gt = pt + kBM * kBN * 2, total = gt + kBM * kBN * 2 + 1024;
-  static constexpr uint32_t cDV = 256, cDK = 256 + D, cols = 512;   // S^T / dP^T buffers at 0 / 64 and 128 / 192
-};
-
-// Warps 0-7 do the arithmetic; lane 0 of a ninth warp issues every TMA load and MMA, so that issuing never
-// delays a warp that the others wait for at the barriers.
-constexpr int kLdkThreads = kKeysThreads + 32, kLdkIssuer = kKeysThreads;
-
-template <int D>
-__global__ void __launch_bounds__(kLdkThreads, 1)
-k_local_bwd_dkdv_tc(Dims dm, const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_do,
-                    const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
-                    const float* __restrict__ LSE, const float* __restrict__ delta,
-                    float* __restrict__ dK_orig, float* __restrict__ dV_orig, int* __restrict__ status) {
-  typedef LdkSmem<D> SM;
-  extern __shared__ __align__(1024) unsigned char sm_raw[];
-  __shared__ uint64_t barKV, barQ[3], bar1[2], bar2;
-  __shared__ uint32_t tbase_s;
-  __shared__ __align__(16) float Ls[3][kBN], ds[3][kBN];
-  const int tid = threadIdx.x, warp = tid >> 5, row = tid & 127, wg = tid >> 7;
-  unsigned char* sm = sm_raw + ((1024u - (tc::smem_u32(sm_raw) & 1023u)) & 1023u);
-  if (warp == 0) tc::tmem_alloc(&tbase_s, SM::cols);
-  if (tid == 0) {
-    tc::mbar_init(&barKV, 1); tc::mbar_init(&bar2, 1);
-    for (int k = 0; k < 3; ++k) tc::mbar_init(&barQ[k], 1);
-    tc::mbar_init(&bar1[0], 1); tc::mbar_init(&bar1[1], 1);
-    tc::mbar_init_fence();
-  }
-  const int lin = blockIdx.x, kt = lin / dm.S, blk = lin % dm.S, pq = blockIdx.y;   // early key tiles (most work) first
-  const int b_ = pq / dm.Hq, h = pq % dm.Hq, pk = b_ * dm.Hkv + dm.hm.g[h];
-  const int bstart = blk * dm.Bs, bend = bstart + dm.Bs;
-  const int k0 = bstart + kt * kBM, nk = min(kBM, bend - k0);
-  const int T = (bend - k0 + kBN - 1) / kBN;                // query tiles that see these keys
-  const int u = k0 + row;
-  // threads 0..63: L (log2 units) and delta of query tile t; loaded into registers one tile before they are
-  // stored, so that no warp waits for global memory in front of a barrier
-  // (nothing may depend on the loaded values before store_scalars: a dependent instruction placed earlier
-  // would make these warps wait for global memory)
-  float Lnext = 0.f, dnext = 0.f;
-  auto fetch_scalars = [&](int t) {
-    if (tid < kBN && t < T) {
-      const int q = min(k0 + t * kBN + tid, bend - 1);
-      Lnext = LSE[(size_t)pq * dm.N + q];
-      dnext = delta[(size_t)pq * dm.N + q];
-    }
-  };
-  auto store_scalars = [&](int t) {
-    if (tid < kBN && t < T) {
-      const bool in = k0 + t * kBN + tid < bend;
-      Ls[t % 3][tid] = in ? Lnext * kLog2e : 0.f; ds[t % 3][tid] = in ? dnext : 0.f;
-    }
-  };
-  fetch_scalars(0); store_scalars(0); fetch_scalars(1); store_scalars(1); fetch_scalars(2); store_scalars(2);
-  fetch_scalars(3);
-  tc::fence_before_sync();
-  __syncthreads();
-  tc::fence_after_sync();
-  const uint32_t tbase = tbase_s, tl = tbase + ((uint32_t)((warp & 3) * 32) << 16);
-  const uint32_t ka = tc::smem_u32(sm + SM::k), va = tc::smem_u32(sm + SM::v), pa = tc::smem_u32(sm + SM::pt), ga = tc::smem_u32(sm + SM::gt);
-  bool ok = true;
-  // thread 0 only
-  auto load_qd = [&](int t) {
-    unsigned char* slot = sm + SM::qd + (t % 3) * SM::tile;
-    tc::mbar_expect_tx(&barQ[t % 3], SM::tile);
-    const int r = pq * dm.N + k0 + t * kBN;
-    for (int g = 0; g < D / 64; ++g) {
-      tc::tma_load_2d(slot + g * kBN * 128, &tm_q, 64 * g, r, &barQ[t % 3]);
-      tc::tma_load_2d(slot + kBN * D * 2 + g * kBN * 128, &tm_do, 64 * g, r, &barQ[t % 3]);
-    }
-  };
-  // one descriptor per operand buffer, stepped per MMA (K-major views; the MN-major views of the ring differ in lbo)
-  const uint64_t dk0 = tc::smem_desc_sw128(ka, 16, 1024), dv0 = tc::smem_desc_sw128(va, 16, 1024),
-                 dq0 = tc::smem_desc_sw128(tc::smem_u32(sm + SM::qd), 16, 1024),
-                 dqm0 = tc::smem_desc_sw128(tc::smem_u32(sm + SM::qd), kBN * 128, 1024),
-                 dp0 = tc::smem_desc_sw128(pa, 16, 1024), dg0 = tc::smem_desc_sw128(ga, 16, 1024);
-  auto issue1 = [&](int t) {                                // S^T(t) = K Q_t^T, dP^T(t) = V dO_t^T into accumulator buffer t & 1
-    if (!tc::mbar_wait(&barQ[t % 3], (t / 3) & 1)) ok = false;
-    tc::fence_after_sync();
-    const uint32_t slot = (uint32_t)(t % 3) * SM::tile;
-    const uint32_t idesc = tc::idesc_bf16(kBM, kBN, 0, 0), cb = tbase + (t & 1) * 2 * kBN;
-    const uint64_t qd = tc::desc_step(dq0, slot), dd = tc::desc_step(dq0, slot + kBN * D * 2);
-#pragma unroll
-    for (int ks = 0; ks < D / 16; ++ks)
-      tc::mma_bf16_ss(cb, tc::desc_step(dk0, (ks / 4) * kBM * 128 + (ks % 4) * 32), tc::desc_step(qd, (ks / 4) * kBN * 128 + (ks % 4) * 32), idesc, ks > 0);
-#pragma unroll
-    for (int ks = 0; ks < D / 16; ++ks)
-      tc::mma_bf16_ss(cb + kBN, tc::desc_step(dv0, (ks / 4) * kBM * 128 + (ks % 4) * 32), tc::desc_step(dd, (ks / 4) * kBN * 128 + (ks % 4) * 32), idesc, ks > 0);
-    tc::mma_commit(&bar1[t & 1]);
-  };
-  if (tid == kLdkIssuer) {
-    tc::mbar_expect_tx(&barKV, 2 * kBM * D * 2);
-    for (int g = 0; g < D / 64; ++g) {
-      tc::tma_load_2d(sm + SM::k + g * kBM * 128, &tm_k, 64 * g, pk * dm.N + k0, &barKV);
-      tc::tma_load_2d(sm + SM::v + g * kBM * 128, &tm_v, 64 * g, pk * dm.N + k0, &barKV);
-    }
-    load_qd(0);
-    if (T > 1) load_qd(1);
-    if (T > 2) load_qd(2);
-    if (!tc::mbar_wait(&barKV, 0)) ok = false;
-    issue1(0);
-  }
-  const float scale2 = dm.sigma * kLog2e;
-  // Two loops over the query tiles, one per role, that meet at one CTA-wide barrier per tile (P^T / G^T
-  // written).  Each role's instructions are contiguous: no warp jumps over the other role's code.  Every warp
-  // runs all T tiles whatever happens (after a wait ran out the remaining waits are skipped).
-  if (warp == 8) {
-    for (int t = 0; t < T; ++t) {
-      if (tid == kLdkIssuer) {
-        if (t + 1 < T) issue1(t + 1);                       // its accumulator buffer was read before the last barrier
-        if (t > 0) {                                        // MMA2(t - 1) has completed: its ring slot is free
-          if (ok && !tc::mbar_wait(&bar2, (t - 1) & 1)) ok = false;
-          if (t + 2 < T) load_qd(t + 2);
-        }
-      }
-      tc::fence_before_sync();
-      __syncthreads();
-      if (tid == kLdkIssuer) {
-        tc::fence_after_sync();
-        const uint32_t slot = (uint32_t)(t % 3) * SM::tile;
-        const uint32_t idesc = tc::idesc_bf16(kBM, D, 0, 1);
-        const uint64_t qm = tc::desc_step(dqm0, slot), dm_ = tc::desc_step(dqm0, slot + kBN * D * 2);
-        const uint32_t acc = t > 0;
-#pragma unroll
-        for (int ks = 0; ks < kBN / 16; ++ks)
-          tc::mma_bf16_ss(tbase + SM::cDV, tc::desc_step(dp0, ks * 32), tc::desc_step(dm_, ks * 16 * 128), idesc, ks > 0 ? 1u : acc);
-#pragma unroll
-        for (int ks = 0; ks < kBN / 16; ++ks)
-          tc::mma_bf16_ss(tbase + SM::cDK, tc::desc_step(dg0, ks * 32), tc::desc_step(qm, ks * 16 * 128), idesc, ks > 0 ? 1u : acc);
-        tc::mma_commit(&bar2);
-      }
-      __syncwarp();
-    }
-  } else {
-    for (int t = 0; t < T; ++t) {
-      const int q0 = k0 + t * kBN, nq = min(kBN, bend - q0);
-      if (ok && !tc::mbar_wait(&bar1[t & 1], (t >> 1) & 1)) ok = false;
-      tc::fence_after_sync();
-      float p[32], g[32];
-      {
-        float s[32], dp[32];
-        tc::tmem_ld32(tl + (t & 1) * 2 * kBN + 32 * wg, s);
-        tc::tmem_ld32(tl + (t & 1) * 2 * kBN + kBN + 32 * wg, dp);
-        const float* Lt = Ls[t % 3] + 32 * wg;
-        const float* dt = ds[t % 3] + 32 * wg;
-        // bit c of `vis`: query column 32 wg + c exists and sees this thread's key (causal, key inside the tile)
-        const int lo = max(0, u - q0 - 32 * wg), hi = row < nk ? min(32, nq - 32 * wg) : 0;
-        const uint32_t vis = hi > lo ? ((hi >= 32 ? 0xffffffffu : (1u << hi) - 1u) & (lo >= 32 ? 0u : 0xffffffffu << lo)) : 0u;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          const float4 a = *reinterpret_cast<const float4*>(Lt + 4 * k), b = *reinterpret_cast<const float4*>(dt + 4 * k);
-          const float Lc[4] = {a.x, a.y, a.z, a.w}, dc[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const float ev = tc::fast_exp2(fmaf(s[4 * k + e], scale2, -Lc[e]));
-            const float pv = (vis >> (4 * k + e)) & 1u ? ev : 0.f;
-            p[4 * k + e] = pv;
-            g[4 * k + e] = pv * (dp[4 * k + e] - dc[e]);
-          }
-        }
-      }
-      if (t > 0) {                                          // MMA2(t - 1) has completed: P^T / G^T are free
-        if (ok && !tc::mbar_wait(&bar2, (t - 1) & 1)) ok = false;
-        tc::fence_after_sync();
-        store_scalars(t + 2);                               // fetched during the previous tile
-        fetch_scalars(t + 3);
-      }
-      store_row32(sm + SM::pt, row, wg, p);
-      store_row32(sm + SM::gt, row, wg, g);
-      tc::fence_async_smem();
-      tc::fence_before_sync();
-      __syncthreads();
-    }
-  }
-  ok = __syncthreads_and(ok);
-  if (ok && T > 0) { if (!tc::mbar_wait(&bar2, (T - 1) & 1)) ok = false; }
-  tc::fence_after_sync();
-  if (warp < 8) {                                           // warpgroup 0 writes dV, warpgroup 1 writes dK (all their threads run the TMEM loads)
-    const size_t at = ((size_t)pq * dm.N + k0 + row) * D;
-    float* dst = (wg == 0 ? dV_orig : dK_orig) + at;
-    const float f = wg == 0 ? 1.f : dm.sigma;
-#pragma unroll
-    for (int d0 = 0; d0 < D; d0 += 32) {
-      float v[32];
-      tc::tmem_ld32(tl + (wg == 0 ? SM::cDV : SM::cDK) + d0, v);
-      if (ok && row < nk) {
-#pragma unroll
-        for (int i = 0; i < 32; i += 4)
-          *reinterpret_cast<float4*>(dst + d0 + i) = make_float4(v[i] * f, v[i + 1] * f, v[i + 2] * f, v[i + 3] * f);
-      }
-    }
-  }
-  tc::fence_before_sync();
-  __syncthreads();
-  if (warp == 0) tc::tmem_dealloc(tbase, SM::cols);
-  if (!ok && tid == 0) report_status(status, 2);
-}
-
 // One CTA per (key cluster j, plane, split, head): 128-key tiles of the run the plane sees, fed with
 // every kRetSplit-th tile of 64 retrieving pairs.  Popular clusters are retrieved by thousands of
 // queries, so the pair tiles are spread over kRetSplit CTAs and over the planes; each CTA adds
@@ -748,24 +497,6 @@ k_ret_bwd_dkdv_tc(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ 
     }                                                                                                             \
     MUSE_LAUNCH_OK();                                                                                             \
   } while (0)
-
-int local_bwd_tc(const Dims& d, const void* Q, const void* K, const void* V, const void* dO, const float* LSE,
-                 const float* delta, float* dQacc, float* dK_orig, float* dV_orig, int* status, cudaStream_t st) {
-  const int pq = d.B * d.Hq;
-  dim3 grid(d.S * cdiv(d.Bs, kBM), pq);
-  CUtensorMap tq, tdo, tk, tv;
-  int rc = make_tmap_bf16_rows(&tq, Q, (uint64_t)pq * d.N, (uint32_t)d.D, kBN);
-  if (rc == MUSE_OK) rc = make_tmap_bf16_rows(&tdo, dO, (uint64_t)pq * d.N, (uint32_t)d.D, kBN);
-  if (rc == MUSE_OK) rc = make_tmap_bf16_rows(&tk, K, (uint64_t)d.B * d.Hkv * d.N, (uint32_t)d.D, kBM);
-  if (rc == MUSE_OK) rc = make_tmap_bf16_rows(&tv, V, (uint64_t)d.B * d.Hkv * d.N, (uint32_t)d.D, kBM);
-  if (rc != MUSE_OK) return rc;
-  prof_mark("k_local_bwd_dkdv_tc", st);
-  MUSE_TC_LAUNCH(k_local_bwd_dkdv_tc, LdkSmem, kLdkThreads, grid, d, tq, tdo, tk, tv, LSE, delta, dK_orig, dV_orig, status);
-  prof_mark("k_local_bwd_dq_tc", st);
-  MUSE_TC_LAUNCH(k_local_bwd_dq_tc, RowsSmem, kRowsThreads, grid, d, (const bf16*)Q, (const bf16*)K, (const bf16*)V, (const bf16*)dO, LSE,
-                 delta, dQacc, status);
-  return MUSE_OK;
-}
 
 int ret_bwd_pairs_tc(const Dims& d, const void* Q, const void* dO, const void* Kp, const void* Vp, const float* LSE,
                      const float* delta, const int32_t* off_k, const int32_t* goff, const int32_t* pairs, void* dq_part,

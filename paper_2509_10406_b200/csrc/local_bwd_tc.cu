@@ -1,0 +1,288 @@
+// Exact causal attention inside the spatial blocks, backward (bf16 inputs, D = 64 or 128).  With L the merged
+// log-sum-exp and delta = dO.O:   P = exp(sigma q.k - L),  G = P (dO.v - delta),
+//   k_local_bwd_dkdv_tc   128 keys per CTA:     S^T = K Q^T, dP^T = V dO^T;  dV += P^T dO,  dK += G^T Q  (times sigma)
+//   k_local_bwd_dq_tc     128 queries per CTA:  S = Q K^T,   dP = dO V^T;    dQ += G K                    (times sigma)
+// Two kernels instead of one that also adds its dQ to memory: dQ is then a sum in a fixed order, the same in every run.
+//
+// Both walk the other side in tiles of 64, which go round NW warpgroups: a warpgroup's thread owns a row (key or query)
+// of the 128 and the tile's 64 columns.  A warpgroup has 128 tensor-memory columns, S and dP, over which it writes P and
+// G as bf16; from there they are the A operands of the second products, so nothing of them passes through shared
+// memory.  While one warpgroup is at its exponentials the tensor cores work for the others.  One warp issues every
+// product, in the order ... second products of tile t, first products of tile t + NW ... (the tensor core executes a
+// CTA's products in the order they were issued, so a warpgroup's columns may be overwritten by the next ones), one warp
+// every load.
+//
+// Bound by the tensor cores: 784 / 1296 cycles per 128 x 64 tile (D = 64 / 128) for dK and dV, 588 / 1040 for dQ (an
+// N = 64 product takes 49 cycles per 16-deep step instead of 32: its A operand has to come out of memory).  NW is the
+// most that tensor memory holds beside the accumulators.  Against products issued by one thread around CTA-wide barriers,
+// with P and G through shared memory: 64k tokens in 8 blocks, D = 64, 32 heads, dK/dV 9490 -> 5650 us (780 TFLOP/s) and dQ
+// 5810 -> 3400 us (970); D = 128, 4 heads, 1540 -> 980 (1130) and 1070 -> 670 us (1230).
+#include <cuda.h>
+#include "common.cuh"
+#include "tc05.cuh"
+
+namespace muse {
+
+typedef __nv_bfloat16 bf16;
+int make_tmap_bf16_rows(void* out_map, const void* base, uint64_t rows, uint32_t cols, uint32_t box_rows);
+
+namespace lb {
+constexpr int kM = 128, kN = 64;                           // rows of a CTA; columns of a tile
+constexpr float kLog2e = 1.4426950408889634f;
+// KIND 0: dK / dV (two accumulators), 1: dQ (one)
+template <int D, int KIND> struct Lay {
+  static constexpr int kRow = kM * D * 2, kCol = kN * D * 2;             // resident tile; streamed tile
+  static constexpr int NW = D == 128 && KIND == 0 ? 2 : 3;               // warpgroups
+  static constexpr int kStages = D == 128 ? 4 : 6;
+  static constexpr int oA = 0, oB = kRow, oRing = 2 * kRow, total = oRing + kStages * 2 * kCol + 1024;
+  static constexpr int kThreads = NW * 128 + 64;
+  static constexpr uint32_t cAcc = NW * 2 * kN;                          // tensor-memory columns: NW x (S | dP) | accumulators
+};
+struct Bars { uint64_t res, full[6], empty[6], s_full[3], ready[3], done; };
+
+// 16 columns of S and dP at a time: P (or 0) and G in bf16, two columns per word
+__device__ __forceinline__ uint32_t pack2(float a, float b) {
+  __nv_bfloat162 x = __floats2bfloat162_rn(a, b);
+  return *reinterpret_cast<uint32_t*>(&x);
+}
+}  // namespace lb
+
+// What both kernels share: barriers, tensor memory, the load warp and the MMA warp.
+//   res    the CTA's resident tiles A, B (K, V or Q, dO) have landed
+//   full   a ring stage (Q, dO or K, V of 64 rows) has landed; in KIND 0 the stage's L and delta too
+template <int D, int KIND>
+__global__ void __launch_bounds__((lb::Lay<D, KIND>::kThreads), 1)
+k_local_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b, const __grid_constant__ CUtensorMap tm_c,
+               const __grid_constant__ CUtensorMap tm_d, const float* LSE, const float* delta, float* __restrict__ out0, float* __restrict__ out1,
+               int* __restrict__ status) {
+  using namespace lb;
+  typedef Lay<D, KIND> LY;
+  constexpr int kRow = LY::kRow, kCol = LY::kCol, NW = LY::NW, NS = LY::kStages, G = D / 64, MW = NW * 4;
+  extern __shared__ __align__(1024) unsigned char sm_raw[];
+  __shared__ Bars bars;
+  __shared__ uint32_t tbase_s;
+  __shared__ __align__(16) float Ls[KIND == 0 ? NS : 1][kN], ds[KIND == 0 ? NS : 1][kN];
+  const int tid = threadIdx.x, warp = tc::warp_index(), lane = tid & 31;
+  unsigned char* sm = sm_raw + ((1024u - (tc::smem_u32(sm_raw) & 1023u)) & 1023u);
+  if (warp == MW) tc::tmem_alloc(&tbase_s, 512);
+  if (tid == 0) {
+    tc::mbar_init(&bars.res, 1); tc::mbar_init(&bars.done, 1);
+    for (int s = 0; s < NS; ++s) { tc::mbar_init(&bars.full[s], KIND == 0 ? 33 : 1); tc::mbar_init(&bars.empty[s], 1); }
+    for (int w = 0; w < NW; ++w) { tc::mbar_init(&bars.s_full[w], 1); tc::mbar_init(&bars.ready[w], 128); }
+    tc::mbar_init_fence();
+  }
+  // KIND 0: early key tiles (most work) first; KIND 1: late query tiles first
+  const int tpb = cdiv(dm.Bs, kM), lin = blockIdx.x, blk = lin % dm.S, pq = blockIdx.y;
+  const int rt = KIND == 0 ? lin / dm.S : tpb - 1 - lin / dm.S;
+  const int b_ = pq / dm.Hq, h = pq % dm.Hq, pk = b_ * dm.Hkv + dm.hm.g[h];
+  const int bstart = blk * dm.Bs, bend = bstart + dm.Bs;
+  const int r0 = bstart + rt * kM, nr = min(kM, bend - r0);               // the CTA's rows
+  const int c_lo = KIND == 0 ? r0 : bstart, c_hi = KIND == 0 ? bend : r0 + nr;   // the columns they meet
+  const int T = (c_hi - c_lo + kN - 1) / kN;
+  tc::fence_before_sync();
+  __syncthreads();
+  tc::fence_after_sync();
+  const uint32_t tbase = tbase_s;
+  bool ok = true;
+  pdl_trigger();
+  pdl_wait();
+
+  if (warp == MW + 1) {                                    // ---- loads
+    const int rrow = (KIND == 0 ? pk : pq) * dm.N + r0, crow = (KIND == 0 ? pq : pk) * dm.N + c_lo;
+    if (tc::elect_one()) {
+      tc::mbar_expect_tx(&bars.res, 2 * kRow);
+#pragma unroll
+      for (int g = 0; g < G; ++g) {
+        tc::tma_load_2d(sm + LY::oA + g * kM * 128, &tm_a, 64 * g, rrow, &bars.res);
+        tc::tma_load_2d(sm + LY::oB + g * kM * 128, &tm_b, 64 * g, rrow, &bars.res);
+      }
+    }
+    float l0 = 0.f, l1 = 0.f, d0 = 0.f, d1 = 0.f;          // L (log2 units) and delta of the next tile's columns lane, lane + 32
+    auto scalars = [&](int t) {
+      if (KIND != 0 || t >= T) return;
+      const int q = c_lo + t * kN + lane;
+      const size_t at = (size_t)pq * dm.N;
+      l0 = q < bend ? LSE[at + q] * kLog2e : 0.f; d0 = q < bend ? delta[at + q] : 0.f;
+      l1 = q + 32 < bend ? LSE[at + q + 32] * kLog2e : 0.f; d1 = q + 32 < bend ? delta[at + q + 32] : 0.f;
+    };
+    scalars(0);
+    for (int t = 0, s = 0, ph = 0; t < T && ok; ++t) {
+      if (!tc::mbar_wait(&bars.empty[s], ph ^ 1)) { ok = false; break; }
+      if (tc::elect_one()) {
+        unsigned char* st = sm + LY::oRing + s * 2 * kCol;
+        tc::mbar_expect_tx(&bars.full[s], 2 * kCol);
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+          tc::tma_load_2d(st + g * kN * 128, &tm_c, 64 * g, crow + t * kN, &bars.full[s]);
+          tc::tma_load_2d(st + kCol + g * kN * 128, &tm_d, 64 * g, crow + t * kN, &bars.full[s]);
+        }
+      }
+      if (KIND == 0) {
+        Ls[s][lane] = l0; Ls[s][lane + 32] = l1; ds[s][lane] = d0; ds[s][lane + 32] = d1;
+        tc::mbar_arrive(&bars.full[s]);
+        scalars(t + 1);
+      }
+      if (++s == NS) { s = 0; ph ^= 1; }
+    }
+  } else if (warp == MW) {                                 // ---- products
+    const uint32_t id1 = tc::idesc_bf16(kM, kN, 0, 0), id2 = tc::idesc_bf16(kM, D, 0, 1);
+    const uint64_t da = tc::smem_desc_sw128(tc::smem_u32(sm + LY::oA), 16, 1024), db = tc::smem_desc_sw128(tc::smem_u32(sm + LY::oB), 16, 1024);
+    const uint64_t dk = tc::smem_desc_sw128(tc::smem_u32(sm + LY::oRing), 16, 1024),              // stage tiles, contraction over D
+                   dn = tc::smem_desc_sw128(tc::smem_u32(sm + LY::oRing), kN * 128, 1024);         // ... over their rows
+    int s1 = 0, ph1 = 0, w1 = 0;                           // stage and warpgroup of the next first products
+    auto first = [&](int t) {                              // S, dP of tile t
+      if (t >= T) return;
+      if (!tc::mbar_wait(&bars.full[s1], ph1)) { ok = false; return; }
+      tc::fence_after_sync();
+      const uint32_t c = tbase + (uint32_t)w1 * 2 * kN;
+      const uint64_t x = tc::desc_step(dk, (uint32_t)s1 * 2 * kCol), y = tc::desc_step(x, kCol);
+#pragma unroll
+      for (int ks = 0; ks < D / 16; ++ks)
+        tc::mma_bf16_ss_warp(c, tc::desc_step(da, (ks / 4) * kM * 128 + (ks % 4) * 32), tc::desc_step(x, (ks / 4) * kN * 128 + (ks % 4) * 32), id1, ks > 0);
+#pragma unroll
+      for (int ks = 0; ks < D / 16; ++ks)
+        tc::mma_bf16_ss_warp(c + kN, tc::desc_step(db, (ks / 4) * kM * 128 + (ks % 4) * 32), tc::desc_step(y, (ks / 4) * kN * 128 + (ks % 4) * 32), id1, ks > 0);
+      tc::mma_commit_warp(&bars.s_full[w1]);
+      if (++s1 == NS) { s1 = 0; ph1 ^= 1; }
+      if (++w1 == NW) w1 = 0;
+    };
+    if (!tc::mbar_wait(&bars.res, 0)) ok = false;
+    for (int t = 0; t < NW && ok; ++t) first(t);
+    for (int t = 0, s = 0, w = 0, ph = 0; t < T && ok; ++t) {
+      if (!tc::mbar_wait(&bars.ready[w], ph)) { ok = false; break; }
+      tc::fence_after_sync();
+      const uint32_t c = tbase + (uint32_t)w * 2 * kN, acc = tbase + LY::cAcc;
+      const uint64_t x = tc::desc_step(dn, (uint32_t)s * 2 * kCol), y = tc::desc_step(x, kCol);
+      if (KIND == 0) {                                     // dV += P^T dO, dK += G^T Q
+#pragma unroll
+        for (int ks = 0; ks < kN / 16; ++ks) tc::mma_bf16_ts_warp(acc, c + 8 * ks, tc::desc_step(y, ks * 16 * 128), id2, t > 0 || ks > 0);
+#pragma unroll
+        for (int ks = 0; ks < kN / 16; ++ks) tc::mma_bf16_ts_warp(acc + D, c + kN + 8 * ks, tc::desc_step(x, ks * 16 * 128), id2, t > 0 || ks > 0);
+      } else {                                             // dQ += G K
+#pragma unroll
+        for (int ks = 0; ks < kN / 16; ++ks) tc::mma_bf16_ts_warp(acc, c + 8 * ks, tc::desc_step(x, ks * 16 * 128), id2, t > 0 || ks > 0);
+      }
+      tc::mma_commit_warp(&bars.empty[s]);
+      if (++s == NS) s = 0;
+      if (++w == NW) { w = 0; ph ^= 1; }
+      first(t + NW);
+    }
+    tc::mma_commit_warp(&bars.done);
+  } else {                                                 // ---- P and G: thread = row
+    const int w = warp >> 2, row = tid & 127, u = r0 + row;
+    const uint32_t tl = tbase + ((uint32_t)((warp & 3) * 32) << 16), ts = tl + (uint32_t)w * 2 * kN;
+    const float scale2 = dm.sigma * kLog2e;
+    float L2 = 0.f, dl = 0.f;
+    if (KIND == 1 && row < nr) { L2 = LSE[(size_t)pq * dm.N + u] * kLog2e; dl = delta[(size_t)pq * dm.N + u]; }
+    int s = w % NS;
+    for (int t = w, ph = 0; t < T; t += NW, ph ^= 1) {
+      if (ok && !tc::mbar_wait(&bars.s_full[w], ph)) ok = false;
+      if constexpr (KIND == 0) {                           // L and delta of the stage (a stage always falls to the same warpgroup)
+        static_assert(NS % NW == 0, "");
+        if (ok && !tc::mbar_wait(&bars.full[s], (t / NS) & 1)) ok = false;
+      }
+      tc::fence_after_sync();
+      // columns of the tile that meet this row: [lo, hi)
+      const int c0 = c_lo + t * kN;
+      const int lo = KIND == 0 ? u - c0 : 0, hi = KIND == 0 ? bend - c0 : u - c0 + 1;
+      const bool full = KIND == 0 ? t >= 2 && bend - c0 >= kN : c0 + kN <= r0;      // all of them, for every row
+      float sv[16], dp[16];
+      tc::tmem_ld16_issue(ts, sv);
+      tc::tmem_ld16_issue(ts + kN, dp);
+#pragma unroll
+      for (int g = 0; g < 4; ++g) {
+        tc::tmem_ld_wait();
+        tc::tmem_ld_use16(sv);
+        tc::tmem_ld_use16(dp);
+        float sn[16], dn_[16];
+        if (g < 3) { tc::tmem_ld16_issue(ts + 16 * (g + 1), sn); tc::tmem_ld16_issue(ts + kN + 16 * (g + 1), dn_); }
+        uint32_t pw[8], gw[8];
+        float p[16];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          float Lc[4], dc[4];
+          if (KIND == 0) {
+            const float4 a = *reinterpret_cast<const float4*>(&Ls[s][16 * g + 4 * k]), b = *reinterpret_cast<const float4*>(&ds[s][16 * g + 4 * k]);
+            Lc[0] = a.x; Lc[1] = a.y; Lc[2] = a.z; Lc[3] = a.w; dc[0] = b.x; dc[1] = b.y; dc[2] = b.z; dc[3] = b.w;
+          }
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const int c = 4 * k + e;
+            p[c] = tc::fast_exp2(fmaf(sv[c], scale2, KIND == 0 ? -Lc[e] : -L2));
+            if (!full) p[c] = 16 * g + c >= lo && 16 * g + c < hi ? p[c] : 0.f;
+            dp[c] = p[c] * (dp[c] - (KIND == 0 ? dc[e] : dl));
+          }
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) { pw[k] = pack2(p[2 * k], p[2 * k + 1]); gw[k] = pack2(dp[2 * k], dp[2 * k + 1]); }
+        // over logits already consumed: columns [16 g, 16 g + 16) -> words [8 g, 8 g + 8)
+        if (KIND == 0) { tc::tmem_st8_issue(ts + 8 * g, pw); tc::tmem_st8_issue(ts + kN + 8 * g, gw); }
+        else tc::tmem_st8_issue(ts + 8 * g, gw);
+        if (g < 3) {
+#pragma unroll
+          for (int c = 0; c < 16; ++c) { sv[c] = sn[c]; dp[c] = dn_[c]; }
+        }
+      }
+      tc::tmem_st_wait();
+      tc::fence_before_sync();
+      tc::mbar_arrive(&bars.ready[w]);
+      s += NW;
+      if (s >= NS) s -= NS;
+    }
+    if (ok && !tc::mbar_wait(&bars.done, 0)) ok = false;
+    tc::fence_after_sync();
+    // KIND 0: warpgroup 0 writes dV, warpgroup 1 dK; KIND 1: two warpgroups write half of dQ each
+    if (w < 2) {
+      constexpr int W = KIND == 0 ? D : D / 2;
+      float* dst = (KIND == 0 && w == 1 ? out1 : out0) + ((size_t)pq * dm.N + u) * D + (KIND == 0 ? 0 : w * W);
+      const float f = KIND == 0 && w == 0 ? 1.f : dm.sigma;
+#pragma unroll
+      for (int d0 = 0; d0 < W; d0 += 32) {
+        float v[32];
+        tc::tmem_ld32(tl + LY::cAcc + w * W + d0, v);
+        if (ok && row < nr) {
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            uint32_t x[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) x[e] = __float_as_uint(v[8 * c + e] * f);
+            tc::st_global_32B(dst + d0 + 8 * c, x);
+          }
+        }
+      }
+    }
+  }
+  if (!ok && lane == 0) report_status(status, MUSE_STATUS_BWD_TIMEOUT);
+  tc::fence_before_sync();
+  __syncthreads();
+  if (warp == MW) tc::tmem_dealloc(tbase, 512);
+}
+
+template <int D>
+static int local_bwd_d(const Dims& d, const void* Q, const void* K, const void* V, const void* dO, const float* LSE, const float* delta,
+                       float* dQacc, float* dK_orig, float* dV_orig, int* status, cudaStream_t st) {
+  const uint64_t rq = (uint64_t)d.B * d.Hq * d.N, rk = (uint64_t)d.B * d.Hkv * d.N;
+  CUtensorMap q[2], o[2], k[2], v[2];                      // boxes of 128 rows (resident) and of 64 (streamed)
+  for (int i = 0; i < 2; ++i) {
+    const uint32_t rows = i == 0 ? lb::kM : lb::kN;
+    MUSE_RC(make_tmap_bf16_rows(&q[i], Q, rq, D, rows));
+    MUSE_RC(make_tmap_bf16_rows(&o[i], dO, rq, D, rows));
+    MUSE_RC(make_tmap_bf16_rows(&k[i], K, rk, D, rows));
+    MUSE_RC(make_tmap_bf16_rows(&v[i], V, rk, D, rows));
+  }
+  const dim3 grid(d.S * cdiv(d.Bs, lb::kM), d.B * d.Hq);
+  prof_mark("k_local_bwd_dkdv_tc", st);
+  MUSE_RC(launch_pdl(k_local_bwd_tc<D, 0>, grid, lb::Lay<D, 0>::kThreads, lb::Lay<D, 0>::total, st, d, k[0], v[0], q[1], o[1], LSE, delta, dV_orig,
+                     dK_orig, status));
+  prof_mark("k_local_bwd_dq_tc", st);
+  return launch_pdl(k_local_bwd_tc<D, 1>, grid, lb::Lay<D, 1>::kThreads, lb::Lay<D, 1>::total, st, d, q[0], o[0], k[1], v[1], LSE, delta, dQacc,
+                    (float*)nullptr, status);
+}
+
+int local_bwd_tc(const Dims& d, const void* Q, const void* K, const void* V, const void* dO, const float* LSE,
+                 const float* delta, float* dQacc, float* dK_orig, float* dV_orig, int* status, cudaStream_t st) {
+  return d.D == 128 ? local_bwd_d<128>(d, Q, K, V, dO, LSE, delta, dQacc, dK_orig, dV_orig, status, st)
+                    : local_bwd_d<64>(d, Q, K, V, dO, LSE, delta, dQacc, dK_orig, dV_orig, status, st);
+}
+
+}  // namespace muse
