@@ -188,16 +188,18 @@ k_local_bwd_dq(Dims dm, const T* __restrict__ Q, const T* __restrict__ K, const 
 }
 
 // ---------------------------------------------------------------------------------------------
-// Retrieval backward: one CTA per (key cluster j, head).  Key chunks are the outer loop so that
-// dK, dV of a chunk accumulate in registers over every plane and query tile that sees it; the
-// per-pair dq partials are owned by this CTA (a pair retrieves exactly one cluster).
+// Retrieval backward: one CTA per (key cluster j, head), or per (j, head, plane, share of the plane's
+// pair tiles) when that leaves most of the chip idle (planes > 1; the fp32 check layer has 16 clusters: 585 -> 101 us).
+// Key chunks are the outer loop so that dK, dV of a chunk accumulate in registers over every plane
+// and query tile of the CTA that sees it; split CTAs add them to the zeroed accumulators.  The
+// per-pair dq partials are owned by one CTA (a pair retrieves exactly one cluster).
 // ---------------------------------------------------------------------------------------------
 template <class T, int D>
 __global__ void __launch_bounds__(kFlashThreads)
 k_ret_bwd(Dims dm, const T* __restrict__ Q, const T* __restrict__ dO, const T* __restrict__ Kp,
           const T* __restrict__ Vp, const float* __restrict__ LSE, const float* __restrict__ delta,
           const int32_t* __restrict__ off_k, const int32_t* __restrict__ goff, const int32_t* __restrict__ pairs,
-          float* __restrict__ dq_part, float* __restrict__ dK_perm, float* __restrict__ dV_perm) {
+          float* __restrict__ dq_part, float* __restrict__ dK_perm, float* __restrict__ dV_perm, int planes, int shares) {
   constexpr int LD = D + Pad<T>::v;
   extern __shared__ __align__(16) unsigned char smraw[];
   T* Ks = (T*)smraw; T* Vs = Ks + kTile * LD; T* Qs = Vs + kTile * LD; T* dOs = Qs + kTile * LD;
@@ -209,24 +211,28 @@ k_ret_bwd(Dims dm, const T* __restrict__ Q, const T* __restrict__ dO, const T* _
   const int nkeys = dm.SB * dm.Ck;
   const int32_t* go = goff + (size_t)pq * (nkeys + 1);
   const int32_t* ok = off_k + (size_t)pk * (dm.Ck * dm.S + 1) + (size_t)j * dm.S;
-  const int kbeg = ok[0], kvis = ok[dm.SB];          // keys some plane can see
+  const int kbeg = ok[0];
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   const T* Qb = Q + (size_t)pq * dm.N * D; const T* dOb = dO + (size_t)pq * dm.N * D;
   const T* Kb = Kp + (size_t)pk * dm.N * D; const T* Vb = Vp + (size_t)pk * dm.N * D;
   const int32_t* pr = pairs + (size_t)pq * dm.N * dm.m;
-  for (int c0 = kbeg; c0 < kvis; c0 += kTile) {
+  const int part = blockIdx.z / shares, share = blockIdx.z % shares;      // this CTA's planes: [pl0, pl1)
+  const int pl0 = planes > 1 ? part : 0, pl1 = planes > 1 ? part + 1 : dm.SB;
+  if (go[(size_t)j * dm.SB + pl0] + share * kTile >= go[(size_t)j * dm.SB + pl1]) return;
+  const int kend = ok[pl1];                                               // keys that these planes see
+  for (int c0 = kbeg; c0 < kend; c0 += kTile) {
     __syncthreads();
-    const int nkc = min(kTile, kvis - c0);
+    const int nkc = min(kTile, kend - c0);
     load_tile<T, D>(Ks, Kb, nkc, [&](int r) { return c0 + r; }, tid);
     load_tile<T, D>(Vs, Vb, nkc, [&](int r) { return c0 + r; }, tid);
     float dk[4][D / 64][4], dv[4][D / 64][4];
     zero_acc<D>(dk); zero_acc<D>(dv);
-    for (int pl = 0; pl < dm.SB; ++pl) {
+    for (int pl = pl0; pl < pl1; ++pl) {
       const int vis_end = ok[pl + 1];
       if (c0 >= vis_end) continue;
       const int nk = min(kTile, vis_end - c0);
       const int g0 = go[(size_t)j * dm.SB + pl], g1 = go[(size_t)j * dm.SB + pl + 1];
-      for (int t0 = g0; t0 < g1; t0 += kTile) {
+      for (int t0 = g0 + share * kTile; t0 < g1; t0 += shares * kTile) {
         const int nq = min(kTile, g1 - t0);
         __syncthreads();
         if (tid < kTile) {
@@ -286,8 +292,12 @@ k_ret_bwd(Dims dm, const T* __restrict__ Q, const T* __restrict__ dO, const T* _
         const size_t u = (size_t)pq * dm.N + c0 + row;
 #pragma unroll
         for (int k = 0; k < D / 64; ++k) {
-          st4(dK_perm + u * D + tx * 4 + 64 * k, make_float4(dk[r][k][0] * dm.sigma, dk[r][k][1] * dm.sigma, dk[r][k][2] * dm.sigma, dk[r][k][3] * dm.sigma));
-          st4(dV_perm + u * D + tx * 4 + 64 * k, make_float4(dv[r][k][0], dv[r][k][1], dv[r][k][2], dv[r][k][3]));
+          const float4 a = make_float4(dk[r][k][0] * dm.sigma, dk[r][k][1] * dm.sigma, dk[r][k][2] * dm.sigma, dk[r][k][3] * dm.sigma);
+          const float4 b = make_float4(dv[r][k][0], dv[r][k][1], dv[r][k][2], dv[r][k][3]);
+          float* pa = dK_perm + u * D + tx * 4 + 64 * k;
+          float* pb = dV_perm + u * D + tx * 4 + 64 * k;
+          if (planes > 1) { atomicAdd(reinterpret_cast<float4*>(pa), a); atomicAdd(reinterpret_cast<float4*>(pb), b); }
+          else { st4(pa, a); st4(pb, b); }
         }
       }
     }
@@ -459,7 +469,9 @@ k_far_bwd(Dims dm, const T* __restrict__ Q, const T* __restrict__ dO, const floa
 }
 
 // ---------------------------------------------------------------------------------------------
-// Key-side pass through the accumulated summaries: one CTA per (key cluster j, head).
+// Key-side pass through the accumulated summaries: one CTA per (key cluster j, head), or per (j, head, bucket) when
+// that leaves most of the chip idle: a bucket's CTA runs the suffix recursion down to its own plane and takes only the
+// bucket's keys (same sums in the same order).
 // For bucket b' (keys of block b') the planes pl >= b' contain it.  With the running suffix
 //   GU(b') = sum_{pl >= b'} exp(mu(b') - mu(pl)) dkappa(pl)   (GW, GS likewise from dnu, dS)
 // and w_iu = exp(sigma qbar_i . k_u - mu_ij(b')) <= 1:
@@ -486,6 +498,8 @@ k_summ_bwd(Dims dm, const T* __restrict__ Kp, const T* __restrict__ Vp, const in
   const int32_t* oq = off_q + (size_t)pq * (dm.S * dm.Cq + 1);
   const T* Kb = Kp + (size_t)pk * dm.N * D; const T* Vb = Vp + (size_t)pk * dm.N * D;
   if (ok[0] >= ok[dm.SB]) return;                    // no key of this cluster is ever summarised
+  const int pl_last = gridDim.z > 1 ? (int)blockIdx.z : 0;
+  if (gridDim.z > 1 && ok[pl_last] >= ok[pl_last + 1]) return;
   for (int i0 = 0; i0 < dm.Cq; i0 += kTile) {
     __syncthreads();
     for (int e = tid; e < kTile * (D / 4); e += kFlashThreads) {
@@ -498,7 +512,7 @@ k_summ_bwd(Dims dm, const T* __restrict__ Kp, const T* __restrict__ Vp, const in
       st4(GW + r * LD + q * 4, make_float4(0.f, 0.f, 0.f, 0.f));
     }
     if (tid < kTile) { GS[tid] = 0.f; muref[tid] = INFINITY; }
-    for (int pl = dm.SB - 1; pl >= 0; --pl) {
+    for (int pl = dm.SB - 1; pl >= pl_last; --pl) {
       __syncthreads();
       // suffix update: G(pl) = grad(pl) + exp(mu(pl) - mu(pl+1)) G(pl+1)
       if (tid < kTile) {
@@ -533,7 +547,7 @@ k_summ_bwd(Dims dm, const T* __restrict__ Kp, const T* __restrict__ Vp, const in
         GS[tid] = g;
       }
       // keys of bucket pl
-      const int kb0 = ok[pl], kb1 = ok[pl + 1];
+      const int kb0 = ok[pl], kb1 = gridDim.z > 1 && pl != pl_last ? kb0 : ok[pl + 1];
       for (int c0 = kb0; c0 < kb1; c0 += kTile) {
         const int nk = min(kTile, kb1 - c0);
         __syncthreads();
@@ -765,8 +779,11 @@ static int attn_bwd_t(const Dims& d, int dtype, const T* Q, const T* K, const T*
       } else {
         MUSE_CUDA_OK(cudaFuncSetAttribute(k_ret_bwd<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm4));
         prof_mark("k_ret_bwd", st);
-        k_ret_bwd<T, D><<<dim3(d.Ck, pq), kFlashThreads, sm4, st>>>(d, Q, dO, Kp, Vp, LSE, w.delta, off_k, ri.goff, ri.pairs,
-                                                                  w.dq_part, w.dK_perm, w.dV_perm);
+        // fewer (cluster, head) CTAs than two rounds of the chip: split by plane, and the planes' pair tiles in two
+        const bool split = d.Ck * pq < 2 * sm_count();
+        const int planes = split && d.SB > 1 ? d.SB : 1, shares = planes > 1 ? 2 : 1;
+        k_ret_bwd<T, D><<<dim3(d.Ck, pq, planes * shares), kFlashThreads, sm4, st>>>(d, Q, dO, Kp, Vp, LSE, w.delta, off_k, ri.goff, ri.pairs,
+                                                                                   w.dq_part, w.dK_perm, w.dV_perm, planes, shares);
         MUSE_LAUNCH_OK();
       }
       use_ret = 1;
@@ -811,12 +828,12 @@ static int attn_bwd_t(const Dims& d, int dtype, const T* Q, const T* K, const T*
       typedef __nv_bfloat16 GB;
       MUSE_CUDA_OK(cudaFuncSetAttribute(k_summ_bwd<T, D, GB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssm));
       prof_mark("k_summ_bwd", st);
-      k_summ_bwd<T, D, GB><<<dim3(d.Ck, pq), kFlashThreads, ssm, st>>>(d, Kp, Vp, off_k, w.off_q, qbar, mu, (const GB*)w.dkappa,
+      k_summ_bwd<T, D, GB><<<dim3(d.Ck, pq, d.Ck * pq < 2 * sm_count() ? d.SB : 1), kFlashThreads, ssm, st>>>(d, Kp, Vp, off_k, w.off_q, qbar, mu, (const GB*)w.dkappa,
                                                                      (const GB*)w.dnu, w.dS, w.dK_perm, w.dV_perm, 0);
     } else {
       MUSE_CUDA_OK(cudaFuncSetAttribute(k_summ_bwd<T, D, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssm));
       prof_mark("k_summ_bwd", st);
-      k_summ_bwd<T, D, float><<<dim3(d.Ck, pq), kFlashThreads, ssm, st>>>(d, Kp, Vp, off_k, w.off_q, qbar, mu, w.dkappa, w.dnu, w.dS,
+      k_summ_bwd<T, D, float><<<dim3(d.Ck, pq, d.Ck * pq < 2 * sm_count() ? d.SB : 1), kFlashThreads, ssm, st>>>(d, Kp, Vp, off_k, w.off_q, qbar, mu, w.dkappa, w.dnu, w.dS,
                                                                         w.dK_perm, w.dV_perm, 0);
     }
     MUSE_LAUNCH_OK();
@@ -850,7 +867,7 @@ static int attn_bwd_t(const Dims& d, int dtype, const T* Q, const T* K, const T*
       const size_t ssm = (size_t)(5 * kTile * (D + 4) + kTile * kLDP) * sizeof(float);
       MUSE_CUDA_OK(cudaFuncSetAttribute(k_summ_bwd<T, D, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssm));
       prof_mark("k_summ_bwd", st);
-      k_summ_bwd<T, D, float><<<dim3(d.Ck, pq), kFlashThreads, ssm, st>>>(d, Kp, Vp, off_k, w.off_q, qbar, spb.mu, w.dkappa_b, w.dnu_b, w.dS_b,
+      k_summ_bwd<T, D, float><<<dim3(d.Ck, pq, d.Ck * pq < 2 * sm_count() ? d.SB : 1), kFlashThreads, ssm, st>>>(d, Kp, Vp, off_k, w.off_q, qbar, spb.mu, w.dkappa_b, w.dnu_b, w.dS_b,
                                                                         w.dK_perm, w.dV_perm, 1);
       MUSE_LAUNCH_OK();
     }

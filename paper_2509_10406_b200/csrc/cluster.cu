@@ -270,12 +270,13 @@ static int lloyd_t(LloydSides& g, const Dims& d, int nsides, int init_mode, uint
   if (init_mode == MUSE_INIT_KMEANSPP) {
     // the draws borrow two arrays that the iterations only fill later: perm as the running minimum distance
     // [problems, N] fp32, off (at least C + 1 words per problem) as the drawn indices [problems, C]
+    KmeansppSide pp[2];
     for (int k = 0; k < nsides; ++k) {
       LloydSide& s = g.s[k];
-      MUSE_RC(kmeanspp(sizeof(T) == 2 ? MUSE_BF16 : MUSE_F32, s.X, s.problems, d.N, D, s.C, s.kind, seed,
-                       reinterpret_cast<float*>(s.perm), s.off, status, st));
+      pp[k] = KmeansppSide{s.X, reinterpret_cast<float*>(s.perm), s.off, s.problems, s.C, s.kind};
       s.init_idx = s.off;
     }
+    MUSE_RC(kmeanspp(sizeof(T) == 2 ? MUSE_BF16 : MUSE_F32, pp, nsides, d.N, D, seed, status, st));
     init_mode = MUSE_INIT_INDICES;
   }
   long long centres = 0;

@@ -214,8 +214,8 @@ int assign_distances(const Dims& d, int dtype, const LloydSide& side, int* statu
 
 // the paper's own clustering: one streaming pass (state = totals, counts; n_batches < 0: to the end) and the
 // per-block assignment under a bucket-size cap (factor <= 0: plain nearest centroid)
-int kmeanspp(int dtype, const void* X, int problems, int N, int D, int C, int kind, uint64_t seed, float* mind2,
-             int32_t* idx_out, int* status, cudaStream_t st);
+struct KmeansppSide { const void* X; float* mind2; int32_t* idx_out; int problems, C, kind; };
+int kmeanspp(int dtype, const KmeansppSide* sides, int nsides, int N, int D, uint64_t seed, int* status, cudaStream_t st);
 struct StreamSide { const void* X; float *totals, *counts, *centres; int32_t* assign_stream; int problems, C, kind; };
 int stream_kmeans(const Dims& d, int dtype, const StreamSide* sides, int n, uint64_t seed, float beta, int first_batch, int n_batches,
                   int32_t* status, cudaStream_t st);

@@ -23,6 +23,7 @@ namespace cg = cooperative_groups;
 namespace muse {
 
 constexpr int kPpThreads = 256, kPpCluster = 8, kPpWarps = kPpThreads / 32;
+struct PpArgs { KmeansppSide s[2]; };
 
 __device__ __forceinline__ bool pp_better(float k, int i, float bk, int bi) { return k > bk || (k == bk && i < bi); }
 
@@ -37,11 +38,18 @@ __device__ __forceinline__ void pp_bulk_load(void* smem_dst, const void* gsrc, u
 // keeps running across draws, since every draw reads the same slice in the same order.
 template <class T, int D, int kPpStages, int kPpGroupBytes>
 __global__ void __launch_bounds__(kPpThreads)
-k_kmeanspp(const T* __restrict__ X, int N, int C, uint64_t seed, int kind, float* __restrict__ mind2,
-           int32_t* __restrict__ idx_out, int md_shared, int* __restrict__ status) {
+k_kmeanspp(const __grid_constant__ PpArgs g, int N, uint64_t seed, int md_shared, int* __restrict__ status) {
   cg::cluster_group cluster = cg::this_cluster();
   const int CS = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
-  const int prob = blockIdx.x / CS, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  int prob = blockIdx.x / CS;
+  const bool second = prob >= g.s[0].problems;            // the sides' problems run side by side
+  const KmeansppSide& sd = g.s[second ? 1 : 0];
+  if (second) prob -= g.s[0].problems;
+  const T* __restrict__ X = (const T*)sd.X;
+  float* __restrict__ mind2 = sd.mind2;
+  int32_t* __restrict__ idx_out = sd.idx_out;
+  const int C = sd.C, kind = sd.kind;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   constexpr int EPL = 16 / (int)sizeof(T);      // elements per 16-byte load
   constexpr int LPR = D / EPL, RPW = 32 / LPR;  // lanes per vector, vectors per warp and load
   constexpr int GR = (kPpGroupBytes / (D * (int)sizeof(T))) < 32 ? (kPpGroupBytes / (D * (int)sizeof(T))) : 32;   // vectors per group
@@ -242,8 +250,8 @@ static PpPlan<T, D> pp_plan(int per) {
 }
 
 template <class T, int D, int ST>
-static int kmeanspp_v(const T* X, int problems, int N, int C, int kind, uint64_t seed, float* mind2, int32_t* idx_out,
-                      int cs, int md_shared, size_t smem, bool query_only, int* max_clusters, int* status, cudaStream_t st) {
+static int kmeanspp_v(const PpArgs& g, int problems, int N, uint64_t seed, int cs, int md_shared, size_t smem, bool query_only, int* max_clusters,
+                      int* status, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -260,13 +268,15 @@ static int kmeanspp_v(const T* X, int problems, int N, int C, int kind, uint64_t
     return MUSE_OK;
   }
   prof_mark("k_kmeanspp", st);
-  MUSE_CUDA_OK(cudaLaunchKernelEx(&cfg, k_kmeanspp<T, D, ST, 8192>, X, N, C, seed, kind, mind2, idx_out, md_shared, status));
+  MUSE_CUDA_OK(cudaLaunchKernelEx(&cfg, k_kmeanspp<T, D, ST, 8192>, g, N, seed, md_shared, status));
   return MUSE_OK;
 }
 
 template <class T, int D>
-static int kmeanspp_t(const T* X, int problems, int N, int C, int kind, uint64_t seed, float* mind2, int32_t* idx_out,
-                      int* status, cudaStream_t st) {
+static int kmeanspp_t(const KmeansppSide* sides, int nsides, int N, uint64_t seed, int* status, cudaStream_t st) {
+  PpArgs g = {};
+  int problems = 0;
+  for (int k = 0; k < nsides; ++k) { g.s[k] = sides[k]; problems += sides[k].problems; }
   // CTAs per problem: the most (up to 8, slices of at least 1024 vectors) for which all problems' clusters can be resident
   // at once.  The draws are sequential, so a cluster that has to wait for a free slot doubles the stage's time; a GPU
   // whose processor groups leave no room for every cluster of 8 does better with clusters of 7 or 6.
@@ -276,27 +286,27 @@ static int kmeanspp_t(const T* X, int problems, int N, int C, int kind, uint64_t
   for (int c = cs_max; c >= 1; --c) {
     const PpPlan<T, D> pl = pp_plan<T, D>((N + c - 1) / c);
     int active = 0;
-    int rc = pl.stages == 3 ? kmeanspp_v<T, D, 3>(X, problems, N, C, kind, seed, mind2, idx_out, c, pl.md_shared, pl.smem, true, &active, status, st)
-                            : kmeanspp_v<T, D, 2>(X, problems, N, C, kind, seed, mind2, idx_out, c, pl.md_shared, pl.smem, true, &active, status, st);
+    int rc = pl.stages == 3 ? kmeanspp_v<T, D, 3>(g, problems, N, seed, c, pl.md_shared, pl.smem, true, &active, status, st)
+                            : kmeanspp_v<T, D, 2>(g, problems, N, seed, c, pl.md_shared, pl.smem, true, &active, status, st);
     if (rc != MUSE_OK) return rc;
     if (active >= problems) { cs = c; break; }
+    if (nsides == 2) {          // not every cluster of the full size resident: the sides one after the other
+      for (int k = 0; k < 2; ++k) MUSE_RC((kmeanspp_t<T, D>(sides + k, 1, N, seed, status, st)));
+      return MUSE_OK;
+    }
     if (c == 1 || active * c < 64) { cs = cs_max; break; }       // more problems than the GPU holds: several rounds either way
   }
   const PpPlan<T, D> pl = pp_plan<T, D>((N + cs - 1) / cs);
-  if (pl.stages == 3) return kmeanspp_v<T, D, 3>(X, problems, N, C, kind, seed, mind2, idx_out, cs, pl.md_shared, pl.smem, false, nullptr, status, st);
-  return kmeanspp_v<T, D, 2>(X, problems, N, C, kind, seed, mind2, idx_out, cs, pl.md_shared, pl.smem, false, nullptr, status, st);
+  if (pl.stages == 3) return kmeanspp_v<T, D, 3>(g, problems, N, seed, cs, pl.md_shared, pl.smem, false, nullptr, status, st);
+  return kmeanspp_v<T, D, 2>(g, problems, N, seed, cs, pl.md_shared, pl.smem, false, nullptr, status, st);
 }
 
-// Start indices [problems, C] of every problem; mind2 is scratch of kmeanspp_ws_floats(problems, N) floats.
-int kmeanspp(int dtype, const void* X, int problems, int N, int D, int C, int kind, uint64_t seed, float* mind2,
-             int32_t* idx_out, int* status, cudaStream_t st) {
+// Start indices [problems, C] of every problem of one or both sides; mind2 is scratch of kmeanspp_ws_floats(problems, N)
+// floats per side.
+int kmeanspp(int dtype, const KmeansppSide* sides, int nsides, int N, int D, uint64_t seed, int* status, cudaStream_t st) {
   typedef __nv_bfloat16 bf;
-  if (dtype == MUSE_F32) {
-    if (D == 64) return kmeanspp_t<float, 64>((const float*)X, problems, N, C, kind, seed, mind2, idx_out, status, st);
-    return kmeanspp_t<float, 128>((const float*)X, problems, N, C, kind, seed, mind2, idx_out, status, st);
-  }
-  if (D == 64) return kmeanspp_t<bf, 64>((const bf*)X, problems, N, C, kind, seed, mind2, idx_out, status, st);
-  return kmeanspp_t<bf, 128>((const bf*)X, problems, N, C, kind, seed, mind2, idx_out, status, st);
+  if (dtype == MUSE_F32) return D == 64 ? kmeanspp_t<float, 64>(sides, nsides, N, seed, status, st) : kmeanspp_t<float, 128>(sides, nsides, N, seed, status, st);
+  return D == 64 ? kmeanspp_t<bf, 64>(sides, nsides, N, seed, status, st) : kmeanspp_t<bf, 128>(sides, nsides, N, seed, status, st);
 }
 
 }  // namespace muse
