@@ -1,22 +1,21 @@
-// Exact retrieval, backward (Section "Exact Retrieval and Local Attention"; gradients with the selections
-// held constant, Appendix "Centroid Gradient Flow"), D = 64 or 128.  With L the merged log-sum-exp and
-// delta = dO.O:   P = exp(sigma q.k - L),  G = sigma P (dO.v - delta),
-//                 dQ = G K  (one bf16 partial row per (query, slot) pair),  dV = P^T dO,  dK = G^T Q.
-// Organised by the inverse index like the forward pass: a CTA owns one key cluster of one head (or a share
-// of it), keeps 64 of its keys and values in shared memory, and walks the retrieving pairs in tiles of 128
-// (pairs on the MMA M side), ordered by plane:
-//   S = Q K^T, dP = dO V^T            tcgen05.mma into tensor memory
-//   P, G                               one thread per pair row, written as bf16 tiles to shared memory
-//   dQ = G K                           over the tensor-memory columns that S and dP have vacated
-//   dV^T += dO^T P,  dK^T += Q^T G     [D][keys], accumulated in tensor memory over all of the CTA's tiles
-// The tiles of Q, dO, P and G fill shared memory, so only one CTA fits an SM; to keep the tensor cores, the
-// load/store unit and the arithmetic warps busy at the same time, the CTA runs TWO independent pipelines
-// ("halves") that share the key / value tiles and take alternate pair tiles.  Each half has four row warps,
-// an MMA-issuing warp and four gather warps (the Q and dO rows arrive by 16-byte asynchronous copies, whose rate
-// grows with the number of threads that issue them; no arithmetic warp spends its time on them), its own 256 tensor-memory columns, its own
-// barriers and its own dV^T / dK^T accumulators, added to global memory with float atomics at the end of a sweep.
-// A cluster with more than 64 visible keys takes further sweeps over the tiles that see them; later sweeps
-// add to the stored dQ rows.
+// Exact retrieval, backward (Section "Exact Retrieval and Local Attention"; gradients with the selections held
+// constant, Appendix "Centroid Gradient Flow"), D = 64 or 128.  With L the merged log-sum-exp and delta = dO.O:
+//   P = exp(sigma q.k - L),  G = P (dO.v - delta);   dQ = sigma G K (one bf16 partial row per (query, slot) pair),
+//   dV = P^T dO,  dK = sigma G^T Q.
+// Organised by the inverse index like the forward pass: a CTA owns one key cluster of one head, or a share of it, and the
+// pairs that retrieve the cluster come in tiles ordered by plane, so that the keys a tile sees are a prefix of the
+// cluster.  Two kernels of one structure (see the local backward): warpgroups take tiles in turn and write P and G over
+// the consumed logits in tensor memory, from where they are A operands; one warp issues every product, one the TMA loads,
+// gather warps bring the scattered Q and dO rows by 16-byte asynchronous copies.
+//   k_ret_bwd_dkdv   128 keys resident, tiles of 64 pairs gathered:  S^T = K Q^T, dP^T = V dO^T;  dV += P^T dO, dK += G^T Q
+//   k_ret_bwd_dq     128 pairs gathered (two buffers), tiles of 64 keys by TMA:  S = Q K^T, dP = dO V^T;  dQ += G K
+// A pair's rows are gathered once for dQ and once per 128 keys it sees for dK and dV, and its dQ row is written once.
+// (One kernel for all five products has to keep dK and dV of the keys at hand in tensor memory, so it takes 64 keys per
+// sweep: the rows were then gathered, and the stored dQ row read and rewritten, once per 64 keys.)
+//
+// Bound: the tensor cores where clusters are long (7 products, 784 + 588 cycles per 128 x 64 tile at D = 64), else the
+// gather of rows (23-26 B/clk per SM).  64 heads of two sequences of 64k tokens, D = 64, 512 keys per cluster, 8 slots:
+// 16.86 ms in one kernel with five products per tile (ret_bwd_short_tc.cu, which short clusters keep), 5.55 + 3.81 ms here.
 #include <cuda.h>
 #include "common.cuh"
 #include "tc05.cuh"
@@ -24,391 +23,616 @@
 namespace muse {
 
 typedef __nv_bfloat16 bf16;
+int make_tmap_bf16_rows(void* out_map, const void* base, uint64_t rows, uint32_t cols, uint32_t box_rows);
 
 namespace rb {
-constexpr int kPairs = 128, kKeys = 64;
-constexpr int kRowWarps = 4, kIssuerWarp0 = 8, kGatherWarp0 = 10, kGather = 128, kThreads = (kGatherWarp0 + 2 * kGather / 32) * 32;
-constexpr int kSplit = 4, kTilesPerCta = 16;                // a cluster with many pair tiles is shared by up to 4 CTAs
-constexpr int kOkCache = 72;
+constexpr int kM = 128, kN = 64;                           // resident rows; columns of a tile
+constexpr int kSplit = 4, kTilesPerCta = 16;               // a cluster with many 128-pair tiles is shared by up to 4 CTAs
+constexpr int kOkCache = 72;                               // bucket offsets of the cluster kept in shared memory (S + 1 <= 72)
 constexpr float kLog2e = 1.4426950408889634f;
-template <int D> struct Lay {
-  static constexpr int kTile = kPairs * D * 2, kKV = kKeys * D * 2, kPG = kPairs * kKeys * 2;
-  static constexpr int oK = 0, oV = kKV, oHalf = 2 * kKV, kHalf = 2 * kTile + 2 * kPG;   // per half: Q | dO | P | G
-  static constexpr int kSmem = oHalf + 2 * kHalf;           // 224 KB at D = 128: no slack, the kernel checks the alignment of its base
-};
-constexpr uint32_t cS = 0, cDP = 64, cDQ = 0, cDV = 128, cDK = 192, kCols = 256;   // per half; dQ reuses the columns of S and dP
-
-struct Bars { uint64_t q_full, q_empty, s_done, pg_ready, m2_done, dq_free; };
 
 __device__ __forceinline__ void cp_async16(void* smem_dst, const void* src, bool valid) {
   const int n = valid ? 16 : 0;                             // 0 source bytes: the 16 bytes are zero-filled
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(tc::smem_u32(smem_dst)), "l"(src), "r"(n) : "memory");
 }
-// K-major view of a [ROWS][D] tile at k-step ks (16 elements of D) / MN-major view at k-step ks (16 rows)
-template <int ROWS> __device__ __forceinline__ uint64_t desc_k(uint32_t base, int ks) {
-  return tc::smem_desc_sw128(base + (ks / 4) * ROWS * 128 + (ks % 4) * 32, 16, 1024);
+__device__ __forceinline__ uint32_t pack2(float a, float b) {
+  __nv_bfloat162 x = __floats2bfloat162_rn(a, b);
+  return *reinterpret_cast<uint32_t*>(&x);
 }
-template <int ROWS> __device__ __forceinline__ uint64_t desc_mn(uint32_t base, int ks) {
-  return tc::smem_desc_sw128(base + ks * 16 * 128, ROWS * 128, 1024);
-}
+
+// The pairs and keys of this CTA's cluster, or (k2 > 0, spatial block selection) of its BUCKET (cluster j, block bb): then
+// the pairs are the (query, slot, chosen block) triples that chose the block, and every one of them sees the whole bucket.
+struct Group {
+  bool bucket;
+  int j, bb, sub, pq, pk, mk, g0, g1, k0, kall, ntiles, nsub;
+  const int32_t *go, *okg;
+  __device__ __forceinline__ Group(const Dims& dm, const int32_t* goff, const int32_t* off_k) {
+    bucket = dm.k2 > 0;
+    j = bucket ? blockIdx.x / dm.SB : blockIdx.x; bb = bucket ? blockIdx.x % dm.SB : 0; sub = blockIdx.y; pq = blockIdx.z;
+    mk = dm.m * (bucket ? dm.k2 : 1);
+    const int b_ = pq / dm.Hq, h = pq % dm.Hq;
+    pk = b_ * dm.Hkv + dm.hm.g[h];
+    go = goff + (size_t)pq * (dm.SB * dm.Ck + 1) + (size_t)j * dm.SB + bb;      // plane pl's pairs: [go[pl], go[pl + 1])
+    g0 = go[0]; g1 = go[bucket ? 1 : dm.SB];
+    okg = off_k + (size_t)pk * (dm.Ck * dm.S + 1) + (size_t)j * dm.S;           // okg[b]: first key of bucket (j, b)
+    k0 = okg[bb]; kall = (bucket ? okg[bb + 1] : okg[dm.SB]) - k0;              // keys that some pair of the group sees
+    ntiles = (g1 - g0 + kM - 1) / kM;
+    nsub = min(kSplit, max(1, ntiles / kTilesPerCta));
+  }
+};
 }  // namespace rb
 
+// ================================================================================================
+// dK, dV
+// ================================================================================================
+namespace rk {
+using namespace rb;
+template <int D> struct Lay {
+  static constexpr int kRow = kM * D * 2, kCol = kN * D * 2;
+  static constexpr int NW = D == 128 ? 2 : 3, NS = D == 128 ? 4 : 6, kGather = D == 128 ? 256 : 128;
+  static constexpr int oK = 0, oV = kRow, oRing = 2 * kRow, total = oRing + NS * 2 * kCol + 1024;
+  static constexpr int kThreads = NW * 128 + 64 + kGather;
+  static constexpr uint32_t cAcc = NW * 2 * kN;
+};
+struct Bars { uint64_t res, full[6], empty[6], s_full[3], ready[3], done, acc_free; };
+constexpr int kDepth = 2;                                  // tiles whose copies are in flight beside the one being issued
+}  // namespace rk
+
 template <int D>
-__global__ void __launch_bounds__(rb::kThreads, 1)
-k_ret_bwd_pairs_tc(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ dO, const bf16* __restrict__ Kp,
-                   const bf16* __restrict__ Vp, const float* __restrict__ LSE, const float* __restrict__ delta,
-                   const int32_t* __restrict__ off_k, const int32_t* __restrict__ goff, const int32_t* __restrict__ pairs,
-                   bf16* __restrict__ dq_part, float* __restrict__ dK_perm, float* __restrict__ dV_perm, int* __restrict__ status) {
-  using namespace rb;
+__global__ void __launch_bounds__(rk::Lay<D>::kThreads, 1)
+k_ret_bwd_dkdv(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v, const bf16* __restrict__ Q,
+               const bf16* __restrict__ dO, const float* __restrict__ LSE, const float* __restrict__ delta, const int32_t* __restrict__ off_k,
+               const int32_t* __restrict__ goff, const int32_t* __restrict__ pairs, float* __restrict__ dK_perm, float* __restrict__ dV_perm,
+               int* __restrict__ status) {
+  using namespace rk;
   typedef Lay<D> LY;
-  constexpr int kTile = LY::kTile, kPG = LY::kPG, oK = LY::oK, oV = LY::oV, oHalf = LY::oHalf, kHalf = LY::kHalf;
-  extern __shared__ __align__(1024) unsigned char sm[];
-  __shared__ Bars bars[2];
+  constexpr int kRow = LY::kRow, kCol = LY::kCol, NW = LY::NW, NS = LY::NS, G = D / 64, MW = NW * 4, CPR = D / 8;
+  static_assert(NS % NW == 0, "a stage always falls to the same warpgroup");
+  extern __shared__ __align__(1024) unsigned char sm_raw[];
+  __shared__ Bars bars;
   __shared__ uint32_t tbase_s;
-  __shared__ int32_t ok_s[kOkCache];
-  __shared__ int32_t tok_s[2][kPairs];                      // tokens of the tile each half is gathering
+  __shared__ int32_t ok_s[kOkCache], tok_s[4][kN];
+  __shared__ __align__(16) float Ls[NS][kN], ds[NS][kN];
+  __shared__ __align__(16) int vs[NS][kN];                  // keys each pair of the tile sees, counted from the cluster's first
+  const Group gr(dm, goff, off_k);
+  if (gr.ntiles == 0 || gr.sub >= gr.nsub || gr.kall <= 0) return;
   const int tid = threadIdx.x, warp = tc::warp_index(), lane = tid & 31;
-  // With spatial block selection (k2 > 0) the CTA owns one BUCKET (cluster j, block bb): its pairs are the (query, slot,
-  // chosen block) triples that chose the block, and every one of them sees the whole bucket (as in the forward kernel).
-  const bool bucket = dm.k2 > 0;
-  const int j = bucket ? blockIdx.x / dm.SB : blockIdx.x, bb = bucket ? blockIdx.x % dm.SB : 0, sub = blockIdx.y, pq = blockIdx.z;
-  const int mk = dm.m * (bucket ? dm.k2 : 1);               // partial dQ rows per query
-  const int b_ = pq / dm.Hq, h = pq % dm.Hq, pk = b_ * dm.Hkv + dm.hm.g[h];
-  const int ngroups = dm.SB * dm.Ck;
-  const int32_t* go = goff + (size_t)pq * (ngroups + 1) + (size_t)j * dm.SB + bb;   // the group's pairs: plane pl is [go[pl], go[pl + 1])
-  const int g0 = go[0], g1 = go[bucket ? 1 : dm.SB];
-  const int ntiles = (g1 - g0 + kPairs - 1) / kPairs;
-  const int nsub = min(kSplit, max(1, ntiles / kTilesPerCta));            // tiles are dealt round-robin to nsub CTAs
-  const int32_t* okg = off_k + (size_t)pk * (dm.Ck * dm.S + 1) + (size_t)j * dm.S;   // okg[b]: first key of bucket (j, b)
-  const int k0 = okg[bb], kall = (bucket ? okg[bb + 1] : okg[dm.SB]) - k0;   // keys that some pair of the group sees
-  if (ntiles == 0 || sub >= nsub) return;
-  if (tc::smem_u32(sm) & 1023u) {                           // the tiles fill the whole dynamic allocation: no room to realign
-    if (tid == 0) report_status(status, MUSE_STATUS_BWD_TIMEOUT);
-    return;
-  }
-  const int32_t* ok = dm.S + 1 <= kOkCache ? ok_s : okg;
+  unsigned char* sm = sm_raw + ((1024u - (tc::smem_u32(sm_raw) & 1023u)) & 1023u);
+  const int32_t* ok = dm.S + 1 <= kOkCache ? ok_s : gr.okg;
   if (dm.S + 1 <= kOkCache)
-    for (int b = tid; b <= dm.S; b += kThreads) ok_s[b] = okg[b];
-  if (warp == 0) tc::tmem_alloc(&tbase_s, 2 * kCols);
+    for (int b = tid; b <= dm.S; b += LY::kThreads) ok_s[b] = gr.okg[b];
+  if (warp == MW) tc::tmem_alloc(&tbase_s, 512);
   if (tid == 0) {
-    for (int v = 0; v < 2; ++v) {
-      tc::mbar_init(&bars[v].q_full, kGather); tc::mbar_init(&bars[v].q_empty, 1); tc::mbar_init(&bars[v].s_done, 1);
-      tc::mbar_init(&bars[v].pg_ready, kRowWarps * 32); tc::mbar_init(&bars[v].m2_done, 1); tc::mbar_init(&bars[v].dq_free, kRowWarps * 32);
-    }
+    tc::mbar_init(&bars.res, 1); tc::mbar_init(&bars.done, 1); tc::mbar_init(&bars.acc_free, 256);
+    for (int s = 0; s < NS; ++s) { tc::mbar_init(&bars.full[s], LY::kGather); tc::mbar_init(&bars.empty[s], 1); }
+    for (int w = 0; w < NW; ++w) { tc::mbar_init(&bars.s_full[w], 1); tc::mbar_init(&bars.ready[w], 128); }
     tc::mbar_init_fence();
   }
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
-  const bf16* Qb = Q + (size_t)pq * dm.N * D;
-  const bf16* dOb = dO + (size_t)pq * dm.N * D;
-  const bf16* Kb = Kp + ((size_t)pk * dm.N + k0) * D;
-  const bf16* Vb = Vp + ((size_t)pk * dm.N + k0) * D;
-  const int32_t* pr = pairs + (size_t)pq * dm.N * mk;
-  const size_t pbase = (size_t)pq * dm.N * mk;
-  // role of this warp: half v, and row / issuing / gather warp
-  const bool roww = warp < 2 * kRowWarps, issw = warp >= kIssuerWarp0 && warp < kIssuerWarp0 + 2, gatw = warp >= kGatherWarp0;
-  const int v = roww ? warp / kRowWarps : issw ? warp - kIssuerWarp0 : (warp - kGatherWarp0) / (kGather / 32);
-  Bars& B = bars[v];
-  unsigned char* hb = sm + oHalf + v * kHalf;               // this half's Q | dO | P | G tiles
-  const uint32_t tbase = tbase_s + v * kCols;
-  bool ok_ = true;                                          // false once a bounded wait ran out (every role still walks all its tiles)
+  const uint32_t tbase = tbase_s;
+  bool ok_ = true;
   auto wait = [&](uint64_t* bar, uint32_t parity) { if (ok_ && !tc::mbar_wait(bar, parity)) ok_ = false; };
-  // keys of sweep `kc` that the query of pair `pid` sees (its block's prefix of the cluster)
-  auto visible = [&](int pid, int kc) {
-    if (bucket) return min(kKeys, max(0, kall - kc));
-    const int tok = pid / dm.m;
-    return min(kKeys, max(0, ok[dm.causal ? tok / dm.Bs : 1] - k0 - kc));
-  };
-
-  uint32_t np = 0;                                          // tiles this half has processed: the phase count of its barriers
-#ifdef MUSE_PHASE_CLOCKS
-  long long pc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  const long long t_in_ = clock64();
-  long long z_ = t_in_;
-#define RBCLK(k) { long long n_ = clock64(); pc[k] += n_ - z_; z_ = n_; }
-#else
-#define RBCLK(k)
-#endif
-  // (a cluster none of whose keys is visible, possible with forced selections, still takes one sweep: its dQ rows are zeros)
-  for (int kc = 0; kc == 0 || kc < kall; kc += kKeys) {
-    const bool first = kc == 0;
-    const int nkc = max(0, min(kKeys, kall - kc));
-    // later sweeps pass over the tiles of planes that see none of the sweep's keys (a prefix of the cluster's tiles)
-    int tile_lo = 0;
-    if (!first && !bucket) {
+  // the 64-pair tiles of this CTA that see keys from `kc` on: every nsub-th of a suffix of the cluster's
+  const int nt64 = (gr.g1 - gr.g0 + kN - 1) / kN;
+  auto first_tile = [&](int kc) {
+    int lo = 0;
+    if (kc > 0 && !gr.bucket) {
       int pl = 0;
-      while (pl + 1 < dm.SB && ok[pl + 1] - k0 <= kc) ++pl;
-      tile_lo = (go[pl] - g0) / kPairs;
+      while (pl + 1 < dm.SB && ok[pl + 1] - gr.k0 <= kc) ++pl;
+      lo = (gr.go[pl] - gr.g0) / kN;
     }
-    const int tile0 = tile_lo + ((sub - tile_lo % nsub) + nsub) % nsub + v * nsub;   // this half's first tile; it takes every second of the CTA's
-    const int tstep = 2 * nsub;
-    __syncthreads();                                        // the previous sweep's products are complete, its accumulators read
-    // the sweep's keys and values as [2][64 rows][128 B] swizzled tiles (K-major and MN-major operands); rows past the cluster are zeros
-    for (int e = tid; e < kKeys * (D / 8); e += kThreads) {
-      const int r = e / (D / 8), ck = e % (D / 8);
-      uint4 a = make_uint4(0u, 0u, 0u, 0u), b = a;
-      if (r < nkc && MUSE_IN_RANGE(k0 + kc + r, dm.N)) {
-        a = reinterpret_cast<const uint4*>(Kb + (size_t)(kc + r) * D)[ck];
-        b = reinterpret_cast<const uint4*>(Vb + (size_t)(kc + r) * D)[ck];
-      }
-      const uint32_t off = (ck >> 3) * kKeys * 128 + tc::sw128_off(r, ck & 7);
-      if (!MUSE_IN_RANGE(off, kKeys * D * 2 - 15)) continue;
-      *reinterpret_cast<uint4*>(sm + oK + off) = a;
-      *reinterpret_cast<uint4*>(sm + oV + off) = b;
-    }
-    tc::fence_async_smem();                                 // the tensor cores read the tiles through the async proxy
-    __syncthreads();
+    return lo + ((gr.sub - lo % gr.nsub) + gr.nsub) % gr.nsub;
+  };
+  const int32_t* pr = pairs + (size_t)gr.pq * dm.N * gr.mk;
 
-    if (roww) {
-      // ================= P, G and the dQ rows: thread = pair row =================
-      const int row = tid & 127;
-      const uint32_t tl = tbase + ((uint32_t)((warp & 3) * 32) << 16);
-      const float scale2 = dm.sigma * kLog2e;
-      // pair ids two tiles ahead and the rows' L, delta one tile ahead: no dependent global load at the top of a tile
-      auto ld_pid = [&](int t) {
-        const int t0 = g0 + t * kPairs;
-        const int id = (t < ntiles && t0 + row < g1) ? __ldg(pr + t0 + row) : -1;
-        return id >= 0 && !MUSE_IN_RANGE(id, (long long)dm.N * mk) ? -1 : id;
-      };
-      int pid = ld_pid(tile0), pid_n = ld_pid(tile0 + tstep);
-      float L2 = 0.f, dl = 0.f, L2_n = 0.f, dl_n = 0.f;
-      auto ld_scalars = [&](int p, float& l2, float& d_) {
-        const size_t tt = (size_t)pq * dm.N + max(p, 0) / mk;
-        l2 = p >= 0 ? LSE[tt] * kLog2e : 0.f;
-        d_ = p >= 0 ? delta[tt] : 0.f;
-      };
-      ld_scalars(pid, L2, dl);
-      bool started = false;
-      for (int tile = tile0; tile < ntiles; tile += tstep, ++np) {
-        const int pid_nn = ld_pid(tile + 2 * tstep);
-        ld_scalars(pid_n, L2_n, dl_n);
-        if (!first && pid_n >= 0) {                         // a later sweep adds to the stored dQ row: have the next tile's row on its way
-          const char* pf = reinterpret_cast<const char*>(dq_part + (pbase + pid_n) * D);
-#pragma unroll
-          for (int o = 0; o < D * 2; o += 128) asm volatile("prefetch.global.L2 [%0];" ::"l"(pf + o));
+  if (warp > MW + 1) {                                     // ---- gather of the Q and dO rows
+    const int g = tid - (MW + 2) * 32, ck = g % CPR;
+    constexpr int RPP = LY::kGather / CPR;                 // rows per pass
+    const bf16* Qb = Q + (size_t)gr.pq * dm.N * D + ck * 8;
+    const bf16* Ob = dO + (size_t)gr.pq * dm.N * D + ck * 8;
+    const float* Lp = LSE + (size_t)gr.pq * dm.N;
+    const float* dp = delta + (size_t)gr.pq * dm.N;
+    auto ld_pid = [&](int t) {
+      const int at = gr.g0 + t * kN + g;
+      const int id = g < kN && t < nt64 && at < gr.g1 ? __ldg(pr + at) : -1;
+      return id >= 0 && !MUSE_IN_RANGE(id, (long long)dm.N * gr.mk) ? -1 : id;
+    };
+    int n = 0;                                             // tiles issued
+    auto publish = [&](int k) { tc::fence_async_smem(); tc::mbar_arrive(&bars.full[k % NS]); };
+    for (int kc = 0; kc < gr.kall; kc += kM) {
+      int t = first_tile(kc);
+      // pair ids two tiles ahead, the rows' L and delta one ahead: no dependent load in front of the copies
+      int tok = ld_pid(t), tok_n = ld_pid(t + gr.nsub);
+      tok = tok >= 0 ? tok / gr.mk : -1; tok_n = tok_n >= 0 ? tok_n / gr.mk : -1;
+      float L = tok >= 0 ? Lp[tok] : 0.f, d_ = tok >= 0 ? dp[tok] : 0.f;
+      for (; t < nt64; t += gr.nsub, ++n) {
+        const int pid2 = ld_pid(t + 2 * gr.nsub);
+        const float L_n = tok_n >= 0 ? Lp[tok_n] : 0.f, d_n = tok_n >= 0 ? dp[tok_n] : 0.f;
+        const int s = n % NS;
+        wait(&bars.empty[s], ((n / NS) & 1) ^ 1);
+        if (g < kN) {
+          tok_s[n & 3][g] = tok;
+          Ls[s][g] = L * kLog2e; ds[s][g] = d_;
+          vs[s][g] = tok < 0 ? 0 : gr.bucket ? gr.kall : ok[dm.causal ? tok / dm.Bs : 1] - gr.k0;
         }
-        const int vis = pid >= 0 ? visible(pid, kc) : 0;
-        const uint32_t ph = np & 1;
-        RBCLK(0)
-        wait(&B.s_done, ph);
-        tc::fence_after_sync();
-        RBCLK(1)
+        tc::named_bar_sync(1, LY::kGather);
+        unsigned char* qd = sm + LY::oRing + s * 2 * kCol + (ck >> 3) * kN * 128;
 #pragma unroll
-        for (int hf = 0; hf < 2; ++hf) {                    // 32 key columns at a time
-          float sv[32], dp[32];
-          tc::tmem_ld32(tl + cS + 32 * hf, sv);
-          tc::tmem_ld32(tl + cDP + 32 * hf, dp);
-          uint32_t pw[16], gw[16];
-#pragma unroll
-          for (int i = 0; i < 32; i += 2) {
-            const float e0 = 32 * hf + i < vis ? tc::fast_exp2(fmaf(sv[i], scale2, -L2)) : 0.f;
-            const float e1 = 32 * hf + i + 1 < vis ? tc::fast_exp2(fmaf(sv[i + 1], scale2, -L2)) : 0.f;
-            __nv_bfloat162 pb = __floats2bfloat162_rn(e0, e1);
-            __nv_bfloat162 gb = __floats2bfloat162_rn(e0 * (dp[i] - dl) * dm.sigma, e1 * (dp[i + 1] - dl) * dm.sigma);   // (sigma rides on G: dQ and dK come out scaled)
-            pw[i / 2] = *reinterpret_cast<uint32_t*>(&pb);
-            gw[i / 2] = *reinterpret_cast<uint32_t*>(&gb);
-          }
-#pragma unroll
-          for (int c4 = 0; c4 < 4; ++c4) {
-            const uint32_t off = tc::sw128_off(row, 4 * hf + c4);
-            *reinterpret_cast<uint4*>(hb + 2 * kTile + off) = make_uint4(pw[4 * c4], pw[4 * c4 + 1], pw[4 * c4 + 2], pw[4 * c4 + 3]);
-            *reinterpret_cast<uint4*>(hb + 2 * kTile + kPG + off) = make_uint4(gw[4 * c4], gw[4 * c4 + 1], gw[4 * c4 + 2], gw[4 * c4 + 3]);
-          }
-        }
-        tc::fence_async_smem();                             // P and G are read by the tensor cores
-        tc::fence_before_sync();
-        tc::mbar_arrive(&B.pg_ready);
-        RBCLK(2)
-        wait(&B.m2_done, ph);
-        tc::fence_after_sync();
-        RBCLK(3)
-        started = true;
-        const bool live = pid >= 0 && ok_;
-        bf16* drow = dq_part + (pbase + max(pid, 0)) * D;
-#pragma unroll
-        for (int d0 = 0; d0 < D; d0 += 32) {
-          float x[32];
-          tc::tmem_ld32(tl + cDQ + d0, x);                  // (warp-wide: every thread takes part, rows past the tile's end do not store)
-          if (d0 + 32 == D) {                               // the columns may be overwritten by the next tile's S and dP
-            tc::fence_before_sync();
-            tc::mbar_arrive(&B.dq_free);
-          }
-          if (live) {
-#pragma unroll
-            for (int c = 0; c < 2; ++c) {                   // 16 columns = 32 bytes per store
-              uint32_t w[8];
-              if (!first) {
-                tc::ld_global_32B(drow + d0 + 16 * c, w);
-#pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                  const __nv_bfloat162 o2 = *reinterpret_cast<const __nv_bfloat162*>(&w[e]);
-                  __nv_bfloat162 b2 = __floats2bfloat162_rn(x[16 * c + 2 * e] + __low2float(o2), x[16 * c + 2 * e + 1] + __high2float(o2));
-                  w[e] = *reinterpret_cast<uint32_t*>(&b2);
-                }
-              } else {
-#pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                  __nv_bfloat162 b2 = __floats2bfloat162_rn(x[16 * c + 2 * e], x[16 * c + 2 * e + 1]);
-                  w[e] = *reinterpret_cast<uint32_t*>(&b2);
-                }
-              }
-              tc::st_global_32B(drow + d0 + 16 * c, w);
-            }
-          }
-        }
-        pid = pid_n; pid_n = pid_nn; L2 = L2_n; dl = dl_n;
-        RBCLK(4)
-#ifdef MUSE_PHASE_CLOCKS
-        pc[7] += 1;
-#endif
-      }
-      // dV^T and dK^T of this sweep's keys: thread = output dim, one key per column; the other half of the CTA
-      // (and other CTAs that share the cluster) add theirs to the same rows
-      if (started && (warp & 3) * 32 < D) {                  // (warp-uniform: the lanes of a warp hold 32 consecutive dims)
-        const int dd = (warp & 3) * 32 + lane;
-#pragma unroll
-        for (int w2 = 0; w2 < 2; ++w2) {
-          float* dst = (w2 == 0 ? dV_perm : dK_perm) + ((size_t)pq * dm.N + k0 + kc) * D + dd;
-#pragma unroll
-          for (int u0 = 0; u0 < kKeys; u0 += 32) {
-            float x[32];
-            tc::tmem_ld32(tl + (w2 == 0 ? cDV : cDK) + u0, x);
-            if (ok_) {
-#pragma unroll
-              for (int u = 0; u < 32; ++u)
-                if (u0 + u < nkc && MUSE_IN_RANGE(k0 + kc + u0 + u, dm.N)) atomicAdd(dst + (size_t)(u0 + u) * D, x[u]);      // (result unused: no round trip)
-            }
-          }
-        }
-      }
-    } else if (issw) {
-      // ================= MMA issue =================
-      const uint32_t qa = tc::smem_u32(hb), da = qa + kTile, pa = da + kTile, ga = pa + kPG;
-      const uint32_t ka = tc::smem_u32(sm + oK), va = tc::smem_u32(sm + oV);
-      const uint32_t np0 = np;
-      for (int tile = tile0; tile < ntiles; tile += tstep, ++np) {
-        {
-          const uint32_t ph = np & 1;
-          RBCLK(0)
-          wait(&B.q_full, ph);                               // the tile's Q and dO rows are in shared memory
-          RBCLK(1)
-          if (np > 0) wait(&B.dq_free, ph ^ 1);              // the previous dQ rows have been read out of the columns S and dP go to
-          tc::fence_after_sync();
-          RBCLK(2)
-          const uint32_t id1 = tc::idesc_bf16(kPairs, kKeys, 0, 0);
-#pragma unroll
-          for (int ks = 0; ks < D / 16; ++ks) tc::mma_bf16_ss_warp(tbase + cS, desc_k<kPairs>(qa, ks), desc_k<kKeys>(ka, ks), id1, ks > 0);
-#pragma unroll
-          for (int ks = 0; ks < D / 16; ++ks) tc::mma_bf16_ss_warp(tbase + cDP, desc_k<kPairs>(da, ks), desc_k<kKeys>(va, ks), id1, ks > 0);
-          tc::mma_commit_warp(&B.s_done);
-          RBCLK(3)
-          wait(&B.pg_ready, ph);                             // P and G are in shared memory, S and dP consumed
-          tc::fence_after_sync();
-          RBCLK(4)
-          const uint32_t id_dq = tc::idesc_bf16(kPairs, D, 0, 1);        // A = G (contraction over keys), B = key rows MN-major
-          // A = dO / Q tile and B = P / G tile, both contracted over pairs.  M = 128 output dims even when D = 64: the second
-          // 64-dim group of the A operand is then the tile that follows in shared memory, and lanes 64..127 hold numbers nobody reads
-          const uint32_t id_t = tc::idesc_bf16(128, kKeys, 1, 1);
-          const bool acc = np > np0;                                     // the accumulators start at zero in every sweep
-#pragma unroll
-          for (int ks = 0; ks < kKeys / 16; ++ks)
-            tc::mma_bf16_ss_warp(tbase + cDQ, tc::smem_desc_sw128(ga + ks * 32, 16, 1024), desc_mn<kKeys>(ka, ks), id_dq, ks > 0);
-#pragma unroll
-          for (int ks = 0; ks < kPairs / 16; ++ks)
-            tc::mma_bf16_ss_warp(tbase + cDV, desc_mn<kPairs>(da, ks), tc::smem_desc_sw128(pa + ks * 16 * 128, kPairs * 128, 1024), id_t, acc || ks > 0);
-#pragma unroll
-          for (int ks = 0; ks < kPairs / 16; ++ks)
-            tc::mma_bf16_ss_warp(tbase + cDK, desc_mn<kPairs>(qa, ks), tc::smem_desc_sw128(ga + ks * 16 * 128, kPairs * 128, 1024), id_t, acc || ks > 0);
-          tc::mma_commit_warp(&B.m2_done);
-          tc::mma_commit_warp(&B.q_empty);                        // ... and the Q / dO tiles refilled
-          RBCLK(5)
-#ifdef MUSE_PHASE_CLOCKS
-          pc[7] += 1;
-#endif
-        }
-        __syncwarp();
-      }
-      if (np > np0) {                           // all products done before the key tiles are replaced or the CTA ends
-        wait(&B.m2_done, (np - 1) & 1);
-        tc::fence_after_sync();
-      }
-    } else if (gatw) {
-      // ================= gather of the Q and dO rows =================
-      const int g = tid - (kGatherWarp0 + (kGather / 32) * v) * 32, ck = g % (D / 8);
-      constexpr int RPP = kGather / (D / 8);                // rows per pass
-      static_assert(kGather == kPairs, "one gather thread per pair row looks up its token");
-      unsigned char* qd = hb + (ck >> 3) * kPairs * 128;
-      unsigned char* od = hb + kTile + (ck >> 3) * kPairs * 128;
-      auto ld1 = [&](int t) {                                // id of row g
-        const int t0 = g0 + t * kPairs;
-        return (t < ntiles && t0 + g < g1) ? __ldg(pr + t0 + g) : -1;
-      };
-      int pa_ = ld1(tile0);
-      for (int tile = tile0; tile < ntiles; tile += tstep, ++np) {
-        const int pa_n = ld1(tile + tstep);
-        RBCLK(0)
-        if (np > 0) wait(&B.q_empty, (np - 1) & 1);          // the previous tile's products have read the buffers
-        RBCLK(1)
-        tok_s[v][g] = pa_ >= 0 ? pa_ / mk : -1;
-        tc::named_bar_sync(1 + v, kGather);
-#pragma unroll 4
-        for (int r = g / (D / 8); r < kPairs; r += RPP) {
-          const int tok = tok_s[v][r];
-          const size_t at = (size_t)max(tok, 0) * D + ck * 8;
-          if (!MUSE_IN_RANGE(tok + 1, dm.N + 1) || !MUSE_IN_RANGE((ck >> 3) * kPairs * 128 + tc::sw128_off(r, ck & 7), kPairs * D * 2 - 15)) continue;
-          cp_async16(qd + tc::sw128_off(r, ck & 7), Qb + at, tok >= 0);
-          cp_async16(od + tc::sw128_off(r, ck & 7), dOb + at, tok >= 0);
+        for (int r = g / CPR; r < kN; r += RPP) {
+          const int tk = tok_s[n & 3][r];
+          if (!MUSE_IN_RANGE(tk + 1, dm.N + 1)) continue;
+          const size_t at = (size_t)max(tk, 0) * D;
+          cp_async16(qd + tc::sw128_off(r, ck & 7), Qb + at, tk >= 0);
+          cp_async16(qd + kCol + tc::sw128_off(r, ck & 7), Ob + at, tk >= 0);
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
-        RBCLK(2)
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
-        tc::fence_async_smem();                              // the tensor cores read the rows through the async proxy
-        tc::mbar_arrive(&B.q_full);
-        RBCLK(3)
-        tc::named_bar_sync(1 + v, kGather);                  // tok_s may be rewritten
-        pa_ = pa_n;
-#ifdef MUSE_PHASE_CLOCKS
-        pc[7] += 1;
-#endif
+        if (n >= kDepth) { asm volatile("cp.async.wait_group %0;" ::"n"(kDepth) : "memory"); publish(n - kDepth); }
+        tok = tok_n; L = L_n; d_ = d_n;
+        tok_n = pid2 >= 0 ? pid2 / gr.mk : -1;
       }
     }
-    tc::fence_before_sync();
-  }
-#ifdef MUSE_PHASE_CLOCKS
-  // (instrumented builds only: words 8..22 of the status block, five per role, in units of 16 clocks)
-  if (pc[7] >= 20 && lane == 0 && v == 0 && (warp == 0 || warp == kIssuerWarp0 || warp == kGatherWarp0)) {
-    const int slot = warp == 0 ? 0 : warp == kIssuerWarp0 ? 1 : 2;
-    if (atomicCAS(status + 5 + slot, 0, 1) == 0) {
-      int* o = status + 8 + 5 * slot;
-      if (slot == 0) { o[0] = (int)(pc[1] / 16); o[1] = (int)(pc[2] / 16); o[2] = (int)(pc[3] / 16); o[3] = (int)(pc[4] / 16); o[4] = (int)pc[7]; }
-      if (slot == 1) { o[0] = (int)(pc[1] / 16); o[1] = (int)(pc[2] / 16); o[2] = (int)(pc[4] / 16); o[3] = (int)(pc[5] / 16); o[4] = (int)((clock64() - t_in_) / 16); }
-      if (slot == 2) { o[0] = (int)(pc[1] / 16); o[1] = (int)(pc[2] / 16); o[2] = (int)(pc[3] / 16); o[3] = (int)pc[7]; o[4] = kall; }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    for (int k = max(0, n - kDepth); k < n; ++k) publish(k);
+  } else if (warp == MW + 1) {                             // ---- the sweep's keys and values
+    int sweep = 0;
+    for (int kc = 0; kc < gr.kall; kc += kM) {
+      if (first_tile(kc) >= nt64) continue;
+      if (sweep > 0) wait(&bars.done, (sweep - 1) & 1);    // the previous sweep's products have read the tiles
+      if (tc::elect_one()) {
+        tc::mbar_expect_tx(&bars.res, 2 * kRow);
+        const int row = gr.pk * dm.N + gr.k0 + kc;         // (rows past the cluster are other keys; their results are dropped)
+#pragma unroll
+        for (int q = 0; q < G; ++q) {
+          tc::tma_load_2d(sm + LY::oK + q * kM * 128, &tm_k, 64 * q, row, &bars.res);
+          tc::tma_load_2d(sm + LY::oV + q * kM * 128, &tm_v, 64 * q, row, &bars.res);
+        }
+      }
+      ++sweep;
+    }
+  } else if (warp == MW) {                                 // ---- products
+    const uint32_t id1 = tc::idesc_bf16(kM, kN, 0, 0), id2 = tc::idesc_bf16(kM, D, 0, 1);
+    const uint64_t da = tc::smem_desc_sw128(tc::smem_u32(sm + LY::oK), 16, 1024), db = tc::smem_desc_sw128(tc::smem_u32(sm + LY::oV), 16, 1024);
+    const uint64_t dk = tc::smem_desc_sw128(tc::smem_u32(sm + LY::oRing), 16, 1024), dn = tc::smem_desc_sw128(tc::smem_u32(sm + LY::oRing), kN * 128, 1024);
+    const uint32_t acc = tbase + LY::cAcc;
+    int n1 = 0, n2 = 0, sweep = 0;                         // tiles whose first / second products have been issued
+    for (int kc = 0; kc < gr.kall; kc += kM) {
+      const int t0 = first_tile(kc);
+      if (t0 >= nt64) continue;
+      const int cnt = (nt64 - t0 + gr.nsub - 1) / gr.nsub, end = n2 + cnt;
+      auto first = [&]() {
+        const int s = n1 % NS;
+        wait(&bars.full[s], (n1 / NS) & 1);
+        tc::fence_after_sync();
+        const uint32_t c = tbase + (uint32_t)(n1 % NW) * 2 * kN;
+        const uint64_t x = tc::desc_step(dk, (uint32_t)s * 2 * kCol), y = tc::desc_step(x, kCol);
+#pragma unroll
+        for (int ks = 0; ks < D / 16; ++ks)
+          tc::mma_bf16_ss_warp(c, tc::desc_step(da, (ks / 4) * kM * 128 + (ks % 4) * 32), tc::desc_step(x, (ks / 4) * kN * 128 + (ks % 4) * 32), id1, ks > 0);
+#pragma unroll
+        for (int ks = 0; ks < D / 16; ++ks)
+          tc::mma_bf16_ss_warp(c + kN, tc::desc_step(db, (ks / 4) * kM * 128 + (ks % 4) * 32), tc::desc_step(y, (ks / 4) * kN * 128 + (ks % 4) * 32), id1, ks > 0);
+        tc::mma_commit_warp(&bars.s_full[n1 % NW]);
+        ++n1;
+      };
+      wait(&bars.res, sweep & 1);
+      for (int k = 0; k < NW && n1 < end; ++k) first();
+      if (sweep > 0) wait(&bars.acc_free, (sweep - 1) & 1);
+      for (bool acc_in = false; n2 < end; ++n2, acc_in = true) {
+        const int s = n2 % NS, w = n2 % NW;
+        wait(&bars.ready[w], (n2 / NW) & 1);
+        tc::fence_after_sync();
+        const uint32_t c = tbase + (uint32_t)w * 2 * kN;
+        const uint64_t x = tc::desc_step(dn, (uint32_t)s * 2 * kCol), y = tc::desc_step(x, kCol);
+#pragma unroll
+        for (int ks = 0; ks < kN / 16; ++ks) tc::mma_bf16_ts_warp(acc, c + 8 * ks, tc::desc_step(y, ks * 16 * 128), id2, acc_in || ks > 0);
+#pragma unroll
+        for (int ks = 0; ks < kN / 16; ++ks) tc::mma_bf16_ts_warp(acc + D, c + kN + 8 * ks, tc::desc_step(x, ks * 16 * 128), id2, acc_in || ks > 0);
+        tc::mma_commit_warp(&bars.empty[s]);
+        if (n1 < end) first();
+      }
+      tc::mma_commit_warp(&bars.done);
+      ++sweep;
+    }
+  } else {                                                 // ---- P and G: thread = key
+    const int w = warp >> 2, row = tid & 127;
+    const uint32_t tl = tbase + ((uint32_t)((warp & 3) * 32) << 16), ts = tl + (uint32_t)w * 2 * kN;
+    const float scale2 = dm.sigma * kLog2e;
+    int n = 0, sweep = 0;
+    for (int kc = 0; kc < gr.kall; kc += kM) {
+      const int t0 = first_tile(kc);
+      if (t0 >= nt64) continue;
+      for (int t = t0; t < nt64; t += gr.nsub, ++n) {
+        if (n % NW != w) continue;
+        const int s = n % NS;
+        wait(&bars.s_full[w], (n / NW) & 1);
+        wait(&bars.full[s], (n / NS) & 1);                 // (the stage's L, delta and vs)
+        tc::fence_after_sync();
+        // the tile's first pair sees the fewest keys: do all pairs see all of this sweep's?
+        const int v0 = vs[s][0];
+        const bool full = gr.g0 + t * kN + kN <= gr.g1 && (v0 >= kc + kM || v0 >= gr.kall);
+        float sv[16], dp[16];
+        tc::tmem_ld16_issue(ts, sv);
+        tc::tmem_ld16_issue(ts + kN, dp);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          tc::tmem_ld_wait();
+          tc::tmem_ld_use16(sv);
+          tc::tmem_ld_use16(dp);
+          float sn[16], dn_[16];
+          if (q < 3) { tc::tmem_ld16_issue(ts + 16 * (q + 1), sn); tc::tmem_ld16_issue(ts + kN + 16 * (q + 1), dn_); }
+          float p[16];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const float4 a = *reinterpret_cast<const float4*>(&Ls[s][16 * q + 4 * k]), b = *reinterpret_cast<const float4*>(&ds[s][16 * q + 4 * k]);
+            const float Lc[4] = {a.x, a.y, a.z, a.w}, dc[4] = {b.x, b.y, b.z, b.w};
+            int4 vv = make_int4(0x7fffffff, 0x7fffffff, 0x7fffffff, 0x7fffffff);
+            if (!full) vv = *reinterpret_cast<const int4*>(&vs[s][16 * q + 4 * k]);
+            const int vc[4] = {vv.x, vv.y, vv.z, vv.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const int c = 4 * k + e;
+              p[c] = tc::fast_exp2(fmaf(sv[c], scale2, -Lc[e]));
+              if (!full) p[c] = kc + row < vc[e] ? p[c] : 0.f;
+              dp[c] = p[c] * (dp[c] - dc[e]);
+            }
+          }
+          uint32_t pw[8], gw[8];
+#pragma unroll
+          for (int k = 0; k < 8; ++k) { pw[k] = pack2(p[2 * k], p[2 * k + 1]); gw[k] = pack2(dp[2 * k], dp[2 * k + 1]); }
+          tc::tmem_st8_issue(ts + 8 * q, pw);              // over logits already consumed
+          tc::tmem_st8_issue(ts + kN + 8 * q, gw);
+          if (q < 3) {
+#pragma unroll
+            for (int c = 0; c < 16; ++c) { sv[c] = sn[c]; dp[c] = dn_[c]; }
+          }
+        }
+        tc::tmem_st_wait();
+        tc::fence_before_sync();
+        tc::mbar_arrive(&bars.ready[w]);
+      }
+      // dV (warpgroup 0) and dK (warpgroup 1) of the sweep's keys; other CTAs that share the cluster add theirs to the same rows
+      if (w < 2) {
+        wait(&bars.done, sweep & 1);
+        tc::fence_after_sync();
+        const bool live = ok_ && kc + row < gr.kall && MUSE_IN_RANGE(gr.k0 + kc + row, dm.N);
+        float* dst = (w == 0 ? dV_perm : dK_perm) + ((size_t)gr.pq * dm.N + gr.k0 + kc + row) * D;
+        const float f = w == 0 ? 1.f : dm.sigma;
+#pragma unroll
+        for (int d0 = 0; d0 < D; d0 += 32) {
+          float v[32];
+          tc::tmem_ld32(tl + LY::cAcc + w * D + d0, v);
+          if (d0 + 32 == D) { tc::fence_before_sync(); tc::mbar_arrive(&bars.acc_free); }
+          if (live) {
+#pragma unroll
+            for (int c = 0; c < 32; c += 4)
+              atomicAdd(reinterpret_cast<float4*>(dst + d0 + c), make_float4(v[c] * f, v[c + 1] * f, v[c + 2] * f, v[c + 3] * f));
+          }
+        }
+      }
+      ++sweep;
     }
   }
-#endif
+  if (!ok_ && lane == 0) report_status(status, MUSE_STATUS_BWD_TIMEOUT);
   tc::fence_before_sync();
   __syncthreads();
-  if (warp == 0) tc::tmem_dealloc(tbase_s, 2 * kCols);
-  if (!ok_ && lane == 0) report_status(status, MUSE_STATUS_BWD_TIMEOUT);
+  if (warp == MW) tc::tmem_dealloc(tbase, 512);
 }
 
+// ================================================================================================
+// dQ
+// ================================================================================================
+namespace rq {
+using namespace rb;
+template <int D> struct Lay {
+  static constexpr int kRow = kM * D * 2, kCol = kN * D * 2;
+  static constexpr int NW = D == 128 ? 2 : 3, NSK = D == 128 ? 3 : 5, NSV = D == 128 ? 2 : 4, kGather = D == 128 ? 256 : 128;
+  static constexpr int oQ = 0, oO = 2 * kRow, oK = 4 * kRow, oV = oK + NSK * kCol, total = oV + NSV * kCol + 1024;   // Q, dO: two buffers each
+  static constexpr int kThreads = NW * 128 + 128 + 64 + kGather;                     // + an epilogue warpgroup
+  static constexpr uint32_t cAcc = NW * 2 * kN;            // two accumulators follow
+};
+struct Bars { uint64_t q_full[2], q_empty[2], k_full[5], k_empty[5], v_full[4], v_empty[4], s_full[3], ready[3], acc_done[2], acc_free[2]; };
+}  // namespace rq
+
+template <int D>
+__global__ void __launch_bounds__(rq::Lay<D>::kThreads, 1)
+k_ret_bwd_dq(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v, const bf16* __restrict__ Q,
+             const bf16* __restrict__ dO, const float* __restrict__ LSE, const float* __restrict__ delta, const int32_t* __restrict__ off_k,
+             const int32_t* __restrict__ goff, const int32_t* __restrict__ pairs, bf16* __restrict__ dq_part, int* __restrict__ status) {
+  using namespace rq;
+  typedef Lay<D> LY;
+  constexpr int kRow = LY::kRow, kCol = LY::kCol, NW = LY::NW, NSK = LY::NSK, NSV = LY::NSV, G = D / 64, CPR = D / 8;
+  constexpr int EW = NW * 4, MW = EW + 4, kReaders = 128 * (NW + 1);         // epilogue warps, MMA warp; threads that read a tile's scalars
+  extern __shared__ __align__(1024) unsigned char sm_raw[];
+  __shared__ Bars bars;
+  __shared__ uint32_t tbase_s;
+  __shared__ int32_t ok_s[kOkCache], tok_s[2][kM], pid_s[2][kM], vs[2][kM], T_s[2];
+  __shared__ float Ls[2][kM], ds[2][kM];
+  const Group gr(dm, goff, off_k);
+  if (gr.ntiles == 0 || gr.sub >= gr.nsub) return;
+  const int tid = threadIdx.x, warp = tc::warp_index(), lane = tid & 31;
+  unsigned char* sm = sm_raw + ((1024u - (tc::smem_u32(sm_raw) & 1023u)) & 1023u);
+  const int32_t* ok = dm.S + 1 <= kOkCache ? ok_s : gr.okg;
+  if (dm.S + 1 <= kOkCache)
+    for (int b = tid; b <= dm.S; b += LY::kThreads) ok_s[b] = gr.okg[b];
+  if (warp == MW) tc::tmem_alloc(&tbase_s, 512);
+  if (tid == 0) {
+    for (int b = 0; b < 2; ++b) {
+      tc::mbar_init(&bars.q_full[b], LY::kGather); tc::mbar_init(&bars.q_empty[b], 1 + kReaders);
+      tc::mbar_init(&bars.acc_done[b], 1); tc::mbar_init(&bars.acc_free[b], 128);
+    }
+    for (int s = 0; s < NSK; ++s) { tc::mbar_init(&bars.k_full[s], 1); tc::mbar_init(&bars.k_empty[s], 1); }
+    for (int s = 0; s < NSV; ++s) { tc::mbar_init(&bars.v_full[s], 1); tc::mbar_init(&bars.v_empty[s], 1); }
+    for (int w = 0; w < NW; ++w) { tc::mbar_init(&bars.s_full[w], 1); tc::mbar_init(&bars.ready[w], 128); }
+    tc::mbar_init_fence();
+  }
+  tc::fence_before_sync();
+  __syncthreads();
+  tc::fence_after_sync();
+  const uint32_t tbase = tbase_s;
+  bool ok_ = true;
+  auto wait = [&](uint64_t* bar, uint32_t parity) { if (ok_ && !tc::mbar_wait(bar, parity)) ok_ = false; };
+  const int32_t* pr = pairs + (size_t)gr.pq * dm.N * gr.mk;
+  auto visible = [&](int tok) { return tok < 0 ? 0 : gr.bucket ? max(gr.kall, 0) : max(0, ok[dm.causal ? tok / dm.Bs : 1] - gr.k0); };
+  auto ld_pid = [&](int at) {
+    const int id = at < gr.g1 ? __ldg(pr + at) : -1;
+    return id >= 0 && !MUSE_IN_RANGE(id, (long long)dm.N * gr.mk) ? -1 : id;
+  };
+  const int cnt = gr.ntiles > gr.sub ? (gr.ntiles - gr.sub + gr.nsub - 1) / gr.nsub : 0;      // pair tiles of this CTA; the i-th is sub + i * nsub
+
+  if (warp > MW + 1) {                                     // ---- gather of the Q and dO rows
+    const int g = tid - (MW + 2) * 32, ck = g % CPR;
+    constexpr int RPP = LY::kGather / CPR;
+    const bf16* Qb = Q + (size_t)gr.pq * dm.N * D + ck * 8;
+    const bf16* Ob = dO + (size_t)gr.pq * dm.N * D + ck * 8;
+    const float* Lp = LSE + (size_t)gr.pq * dm.N;
+    const float* dp = delta + (size_t)gr.pq * dm.N;
+    int pid = g < kM ? ld_pid(gr.g0 + gr.sub * kM + g) : -1;
+    for (int i = 0; i < cnt; ++i) {
+      const int b = i & 1, at = gr.g0 + (gr.sub + i * gr.nsub) * kM;
+      const int pid_n = g < kM && i + 1 < cnt ? ld_pid(at + gr.nsub * kM + g) : -1;
+      const int tok = pid >= 0 ? pid / gr.mk : -1;
+      const float L = tok >= 0 ? Lp[tok] * kLog2e : 0.f, d_ = tok >= 0 ? dp[tok] : 0.f;
+      wait(&bars.q_empty[b], ((i >> 1) & 1) ^ 1);
+      if (g < kM) {
+        const int v = visible(tok);
+        tok_s[b][g] = tok; pid_s[b][g] = pid; vs[b][g] = v;
+        if (g == min(kM, gr.g1 - at) - 1) T_s[b] = (v + kN - 1) / kN;          // (the tile's last pair sees the most keys)
+      }
+      tc::named_bar_sync(1, LY::kGather);
+#pragma unroll 4
+      for (int r = g / CPR; r < kM; r += RPP) {
+        const int tk = tok_s[b][r];
+        if (!MUSE_IN_RANGE(tk + 1, dm.N + 1)) continue;
+        const size_t src = (size_t)max(tk, 0) * D;
+        const uint32_t off = (uint32_t)(b * kRow + (ck >> 3) * kM * 128) + tc::sw128_off(r, ck & 7);
+        cp_async16(sm + LY::oQ + off, Qb + src, tk >= 0);
+        cp_async16(sm + LY::oO + off, Ob + src, tk >= 0);
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+      if (g < kM) { Ls[b][g] = L; ds[b][g] = d_; }
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+      tc::fence_async_smem();
+      tc::mbar_arrive(&bars.q_full[b]);
+      pid = pid_n;
+    }
+  } else if (warp == MW + 1) {                             // ---- key and value tiles
+    int sk = 0, phk = 0, sv = 0, phv = 0;
+    auto last_pid = [&](int i) { return i < cnt ? ld_pid(min(gr.g1, gr.g0 + (gr.sub + i * gr.nsub + 1) * kM) - 1) : -1; };
+    int pid = last_pid(0);
+    for (int i = 0; i < cnt && ok_; ++i) {
+      const int pid_n = last_pid(i + 1);
+      const int T = (visible(pid >= 0 ? pid / gr.mk : -1) + kN - 1) / kN;
+      pid = pid_n;
+      for (int t = 0; t < T && ok_; ++t) {
+        const int row = gr.pk * dm.N + gr.k0 + t * kN;     // (rows past the cluster are other keys; they are masked)
+        wait(&bars.k_empty[sk], phk ^ 1);
+        if (tc::elect_one()) {
+          tc::mbar_expect_tx(&bars.k_full[sk], kCol);
+#pragma unroll
+          for (int q = 0; q < G; ++q) tc::tma_load_2d(sm + LY::oK + sk * kCol + q * kN * 128, &tm_k, 64 * q, row, &bars.k_full[sk]);
+        }
+        if (++sk == NSK) { sk = 0; phk ^= 1; }
+        wait(&bars.v_empty[sv], phv ^ 1);
+        if (tc::elect_one()) {
+          tc::mbar_expect_tx(&bars.v_full[sv], kCol);
+#pragma unroll
+          for (int q = 0; q < G; ++q) tc::tma_load_2d(sm + LY::oV + sv * kCol + q * kN * 128, &tm_v, 64 * q, row, &bars.v_full[sv]);
+        }
+        if (++sv == NSV) { sv = 0; phv ^= 1; }
+      }
+    }
+  } else if (warp == MW) {                                 // ---- products
+    const uint32_t id1 = tc::idesc_bf16(kM, kN, 0, 0), id2 = tc::idesc_bf16(kM, D, 0, 1);
+    const uint64_t dq0 = tc::smem_desc_sw128(tc::smem_u32(sm + LY::oQ), 16, 1024), do0 = tc::smem_desc_sw128(tc::smem_u32(sm + LY::oO), 16, 1024),
+                   dk0 = tc::smem_desc_sw128(tc::smem_u32(sm + LY::oK), 16, 1024), dv0 = tc::smem_desc_sw128(tc::smem_u32(sm + LY::oV), 16, 1024),
+                   dkn = tc::smem_desc_sw128(tc::smem_u32(sm + LY::oK), kN * 128, 1024);
+    // first products run up to NW tiles ahead, across pair tiles: (ia, ka) = pair tile and key tile of the next ones
+    int ia = 0, ka = 0, Ta = -1, n1 = 0, n2 = 0, sk1 = 0, phk1 = 0, sv1 = 0, phv1 = 0;
+    auto first = [&](bool must) {                          // false: nothing left, or (unless `must`) the next rows are still on their way
+      while (ia < cnt) {
+        if (Ta < 0) {
+          if (!must && !tc::mbar_try_wait(&bars.q_full[ia & 1], (ia >> 1) & 1)) return false;
+          wait(&bars.q_full[ia & 1], (ia >> 1) & 1);
+          Ta = T_s[ia & 1];
+          ka = 0;
+        }
+        if (ka < Ta) break;
+        ++ia;
+        Ta = -1;
+      }
+      if (ia >= cnt) return false;
+      wait(&bars.k_full[sk1], phk1);
+      wait(&bars.v_full[sv1], phv1);
+      tc::fence_after_sync();
+      const uint32_t c = tbase + (uint32_t)(n1 % NW) * 2 * kN;
+      const uint64_t a = tc::desc_step(dq0, (uint32_t)(ia & 1) * kRow), o = tc::desc_step(do0, (uint32_t)(ia & 1) * kRow);
+      const uint64_t x = tc::desc_step(dk0, (uint32_t)sk1 * kCol), y = tc::desc_step(dv0, (uint32_t)sv1 * kCol);
+#pragma unroll
+      for (int ks = 0; ks < D / 16; ++ks)
+        tc::mma_bf16_ss_warp(c, tc::desc_step(a, (ks / 4) * kM * 128 + (ks % 4) * 32), tc::desc_step(x, (ks / 4) * kN * 128 + (ks % 4) * 32), id1, ks > 0);
+#pragma unroll
+      for (int ks = 0; ks < D / 16; ++ks)
+        tc::mma_bf16_ss_warp(c + kN, tc::desc_step(o, (ks / 4) * kM * 128 + (ks % 4) * 32), tc::desc_step(y, (ks / 4) * kN * 128 + (ks % 4) * 32), id1, ks > 0);
+      tc::mma_commit_warp(&bars.s_full[n1 % NW]);
+      tc::mma_commit_warp(&bars.v_empty[sv1]);
+      if (++sk1 == NSK) { sk1 = 0; phk1 ^= 1; }
+      if (++sv1 == NSV) { sv1 = 0; phv1 ^= 1; }
+      ++ka; ++n1;
+      return true;
+    };
+    uint32_t used = 3u;                                    // bit b: parity to wait for before accumulator b is overwritten
+    for (int i = 0, sk = 0; i < cnt && ok_; ++i) {
+      const int b = i & 1;
+      wait(&bars.q_full[b], (i >> 1) & 1);
+      const int T = T_s[b];
+      if (T > 0) { wait(&bars.acc_free[b], (used >> b) & 1u); used ^= 1u << b; }
+      for (int t = 0; t < T && ok_; ++t, ++n2) {
+        while (n1 - n2 < NW && first(n1 == n2)) {}
+        const int w = n2 % NW;
+        wait(&bars.ready[w], (n2 / NW) & 1);
+        tc::fence_after_sync();
+        const uint32_t c = tbase + (uint32_t)w * 2 * kN, acc = tbase + LY::cAcc + (uint32_t)b * D;
+        const uint64_t x = tc::desc_step(dkn, (uint32_t)sk * kCol);
+#pragma unroll
+        for (int ks = 0; ks < kN / 16; ++ks) tc::mma_bf16_ts_warp(acc, c + 8 * ks, tc::desc_step(x, ks * 16 * 128), id2, t > 0 || ks > 0);
+        tc::mma_commit_warp(&bars.k_empty[sk]);
+        if (++sk == NSK) sk = 0;
+      }
+      tc::mma_commit_warp(&bars.acc_done[b]);
+      tc::mma_commit_warp(&bars.q_empty[b]);
+    }
+  } else if (warp >= EW) {                                 // ---- the finished rows: thread = pair
+    const int row = tid & 127;
+    const uint32_t tl = tbase + ((uint32_t)((warp & 3) * 32) << 16);
+    for (int i = 0; i < cnt; ++i) {
+      const int b = i & 1;
+      wait(&bars.q_full[b], (i >> 1) & 1);
+      const int pid = pid_s[b][row], T = T_s[b];
+      wait(&bars.acc_done[b], (i >> 1) & 1);
+      tc::fence_after_sync();
+      const bool live = ok_ && pid >= 0;
+      bf16* dst = dq_part + ((size_t)gr.pq * dm.N * gr.mk + max(pid, 0)) * D;
+#pragma unroll
+      for (int d0 = 0; d0 < D; d0 += 32) {
+        float v[32];
+        if (T > 0) tc::tmem_ld32(tl + LY::cAcc + b * D + d0, v);
+        else {                                             // (no visible key, possible with forced selections: a row of zeros)
+#pragma unroll
+          for (int c = 0; c < 32; ++c) v[c] = 0.f;
+        }
+        if (d0 + 32 == D) {
+          tc::fence_before_sync();
+          if (T > 0) tc::mbar_arrive(&bars.acc_free[b]);
+          tc::mbar_arrive(&bars.q_empty[b]);
+        }
+        if (live) {
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {                    // 16 columns = 32 bytes per store
+            uint32_t x[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) x[e] = pack2(v[16 * c + 2 * e] * dm.sigma, v[16 * c + 2 * e + 1] * dm.sigma);
+            tc::st_global_32B(dst + d0 + 16 * c, x);
+          }
+        }
+      }
+    }
+  } else {                                                 // ---- G: thread = pair row
+    const int w = warp >> 2, row = tid & 127;
+    const uint32_t ts = tbase + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)w * 2 * kN;
+    const float scale2 = dm.sigma * kLog2e;
+    int n = 0;
+    for (int i = 0; i < cnt; ++i) {
+      const int b = i & 1;
+      wait(&bars.q_full[b], (i >> 1) & 1);
+      const int T = T_s[b], vis = vs[b][row], vmin = vs[b][0];                 // (the first pair sees the fewest keys)
+      const bool whole = pid_s[b][kM - 1] >= 0;
+      const float L2 = Ls[b][row], dl = ds[b][row];
+      tc::mbar_arrive(&bars.q_empty[b]);                   // (the scalars are in registers; the rows are the products' concern)
+      for (int t = 0; t < T; ++t, ++n) {
+        if (n % NW != w) continue;
+        wait(&bars.s_full[w], (n / NW) & 1);
+        tc::fence_after_sync();
+        const int v = vis - t * kN;
+        const bool full = whole && vmin - t * kN >= kN;
+        float sv[16], dp[16];
+        tc::tmem_ld16_issue(ts, sv);
+        tc::tmem_ld16_issue(ts + kN, dp);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          tc::tmem_ld_wait();
+          tc::tmem_ld_use16(sv);
+          tc::tmem_ld_use16(dp);
+          float sn[16], dn_[16];
+          if (q < 3) { tc::tmem_ld16_issue(ts + 16 * (q + 1), sn); tc::tmem_ld16_issue(ts + kN + 16 * (q + 1), dn_); }
+#pragma unroll
+          for (int c = 0; c < 16; ++c) {
+            float p = tc::fast_exp2(fmaf(sv[c], scale2, -L2));
+            if (!full) p = 16 * q + c < v ? p : 0.f;
+            dp[c] = p * (dp[c] - dl);
+          }
+          uint32_t gw[8];
+#pragma unroll
+          for (int k = 0; k < 8; ++k) gw[k] = pack2(dp[2 * k], dp[2 * k + 1]);
+          tc::tmem_st8_issue(ts + 8 * q, gw);              // over logits already consumed
+          if (q < 3) {
+#pragma unroll
+            for (int c = 0; c < 16; ++c) { sv[c] = sn[c]; dp[c] = dn_[c]; }
+          }
+        }
+        tc::tmem_st_wait();
+        tc::fence_before_sync();
+        tc::mbar_arrive(&bars.ready[w]);
+      }
+    }
+  }
+  if (!ok_ && lane == 0) report_status(status, MUSE_STATUS_BWD_TIMEOUT);
+  tc::fence_before_sync();
+  __syncthreads();
+  if (warp == MW) tc::tmem_dealloc(tbase, 512);
+}
+
+template <int D>
+static int ret_bwd_d(const Dims& d, const void* Q, const void* dO, const void* Kp, const void* Vp, const float* LSE, const float* delta,
+                     const int32_t* off_k, const int32_t* goff, const int32_t* pairs, void* dq_part, float* dK_perm, float* dV_perm, int* status,
+                     cudaStream_t st) {
+  const uint64_t rk = (uint64_t)d.B * d.Hkv * d.N;
+  CUtensorMap k[2], v[2];                                  // boxes of 128 keys (resident) and of 64 (streamed)
+  for (int i = 0; i < 2; ++i) {
+    MUSE_RC(make_tmap_bf16_rows(&k[i], Kp, rk, D, i == 0 ? rb::kM : rb::kN));
+    MUSE_RC(make_tmap_bf16_rows(&v[i], Vp, rk, D, i == 0 ? rb::kM : rb::kN));
+  }
+  const dim3 grid(d.k2 > 0 ? d.Ck * d.SB : d.Ck, rb::kSplit, d.B * d.Hq);      // one CTA (or a few) per key cluster, or per bucket
+  prof_mark("k_ret_bwd_pairs_tc", st);
+  MUSE_CUDA_OK(cudaFuncSetAttribute(k_ret_bwd_dkdv<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, rk::Lay<D>::total));
+  k_ret_bwd_dkdv<D><<<grid, rk::Lay<D>::kThreads, rk::Lay<D>::total, st>>>(d, k[0], v[0], (const bf16*)Q, (const bf16*)dO, LSE, delta, off_k, goff, pairs,
+                                                                       dK_perm, dV_perm, status);
+  MUSE_LAUNCH_OK();
+  prof_mark("k_ret_bwd_dq", st);
+  MUSE_CUDA_OK(cudaFuncSetAttribute(k_ret_bwd_dq<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, rq::Lay<D>::total));
+  k_ret_bwd_dq<D><<<grid, rq::Lay<D>::kThreads, rq::Lay<D>::total, st>>>(d, k[1], v[1], (const bf16*)Q, (const bf16*)dO, LSE, delta, off_k, goff, pairs,
+                                                                     (bf16*)dq_part, status);
+  MUSE_LAUNCH_OK();
+  return MUSE_OK;
+}
+
+int ret_bwd_short_tc(const Dims& d, const void* Q, const void* dO, const void* Kp, const void* Vp, const float* LSE,
+                     const float* delta, const int32_t* off_k, const int32_t* goff, const int32_t* pairs, void* dq_part,
+                     float* dK_perm, float* dV_perm, int* status, cudaStream_t st);
+
+// Two kernels, or one with five products per tile?  By the mean number of keys of a cluster: the fused kernel gathers a pair's
+// rows once per 64 keys and reads back the stored dQ row from the second time on, the two kernels gather it once more than
+// they have to when one sweep would have done.  Measured, fused | dK, dV + dQ, us:
+//   D = 64:   64 keys 566 | 311 + 569,  128 keys 469 | 233 + 293,  256 keys 1331 | 543 + 501,  512 keys 16860 | 5549 + 3808
+//   D = 128:  64 keys 850 | 484 + 438,  128 keys 684 | 353 + 261,  256 keys 1875 | 802 + 514
 int ret_bwd_pairs_tc(const Dims& d, const void* Q, const void* dO, const void* Kp, const void* Vp, const float* LSE,
                      const float* delta, const int32_t* off_k, const int32_t* goff, const int32_t* pairs, void* dq_part,
                      float* dK_perm, float* dV_perm, int* status, cudaStream_t st) {
-  prof_mark("k_ret_bwd_pairs_tc", st);
-  const dim3 grid(d.k2 > 0 ? d.Ck * d.SB : d.Ck, rb::kSplit, d.B * d.Hq);      // one CTA (or a few) per key cluster, or per bucket
-  if (d.D == 128) {
-    MUSE_CUDA_OK(cudaFuncSetAttribute(k_ret_bwd_pairs_tc<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, rb::Lay<128>::kSmem));
-    k_ret_bwd_pairs_tc<128><<<grid, rb::kThreads, rb::Lay<128>::kSmem, st>>>(
-        d, (const bf16*)Q, (const bf16*)dO, (const bf16*)Kp, (const bf16*)Vp, LSE, delta, off_k, goff, pairs, (bf16*)dq_part, dK_perm, dV_perm, status);
-  } else {
-    MUSE_CUDA_OK(cudaFuncSetAttribute(k_ret_bwd_pairs_tc<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, rb::Lay<64>::kSmem));
-    k_ret_bwd_pairs_tc<64><<<grid, rb::kThreads, rb::Lay<64>::kSmem, st>>>(
-        d, (const bf16*)Q, (const bf16*)dO, (const bf16*)Kp, (const bf16*)Vp, LSE, delta, off_k, goff, pairs, (bf16*)dq_part, dK_perm, dV_perm, status);
-  }
-  MUSE_LAUNCH_OK();
-  return MUSE_OK;
+  if (d.N / d.Ck < (d.D == 128 ? 128 : 256))
+    return ret_bwd_short_tc(d, Q, dO, Kp, Vp, LSE, delta, off_k, goff, pairs, dq_part, dK_perm, dV_perm, status, st);
+  return d.D == 128 ? ret_bwd_d<128>(d, Q, dO, Kp, Vp, LSE, delta, off_k, goff, pairs, dq_part, dK_perm, dV_perm, status, st)
+                    : ret_bwd_d<64>(d, Q, dO, Kp, Vp, LSE, delta, off_k, goff, pairs, dq_part, dK_perm, dV_perm, status, st);
 }
 
 }  // namespace muse

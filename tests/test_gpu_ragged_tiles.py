@@ -4,8 +4,8 @@ import numpy as np
 import pytest
 import torch
 
-from tests.gpu_util import to_np
-from tests.test_gpu_backward import _backward_parity
+from tests.gpu_util import kernels_launched, to_np
+from tests.test_gpu_backward import _backward_parity, _backward_parity_run
 from tests.test_gpu_cluster import CASES
 from tests.test_gpu_forward import TC_BWD_KERNELS, TC_FWD_KERNELS, _forward_parity
 
@@ -47,3 +47,13 @@ def test_streaming_both_sides_at_once_equals_each_side_alone(Hq, Hkv, D, Cq, Ck,
         assert np.array_equal(to_np(c1), to_np(cen)) and np.array_equal(to_np(a1), to_np(assign))
         size = np.bincount(to_np(a1)[0, 0, :N // S], minlength=C)
         assert size.sum() == N // S and size.max() <= max(1, int(np.ceil(cap * (N // S) / C)))
+
+
+@pytest.mark.parametrize("base,Ck,two_kernels", [("d64", 7, True), ("d64", 8, False), ("d64", 2, True), ("d128", 15, True), ("d128", 16, False),
+                                                 ("d128", 3, True)])
+def test_retrieval_backward_on_both_sides_of_the_cluster_length_rule(base, Ck, two_kernels):
+    """2040 keys: clusters of 255 (D = 64) or 127 keys (D = 128) and shorter take the fused kernel."""
+    w = CASES[base].with_(Hq=2, Hkv=1, N=2040, S=4, Cq=9, Ck=Ck, m=min(Ck, 3), components=64)
+    with kernels_launched() as rec:
+        _backward_parity_run(w, 128.0)
+    assert "k_ret_bwd_pairs_tc" in rec.names and ("k_ret_bwd_dq" in rec.names) == two_kernels
