@@ -8,7 +8,7 @@
 
 namespace muse {
 
-int near_bwd(const Dims& d, int dtype, const void* Q, const void* dO, const float* qbar, const float* LSE, const float* delta,
+int near_bwd(const Dims& d, const void* Q, const void* dO, const float* qbar, const float* LSE, const float* delta,
              const int32_t* off_q, const int32_t* perm_q, const int32_t* sel, const int32_t* bsel, const SummPtrs& sp, float* dQacc,
              float* dkappa_b, float* dnu_b, float* dS_b, int grad_ji, cudaStream_t st);
 int grad_to_bf16(const float* in, size_t n, void* out, cudaStream_t st);
@@ -852,7 +852,7 @@ static int attn_bwd_t(const Dims& d, int dtype, const T* Q, const T* K, const T*
     MUSE_CUDA_OK(cudaMemsetAsync(w.dS_b, 0, ent * sizeof(float), st));
     const SummPtrs spb = summ_ptrs_blk(L, base);
     const bool tcb = summ_bwd_tc_supported(d, dtype) && !path_forced(kForceSummBwdSimt);
-    int rc = near_bwd(d, dtype, Q, dO, qbar, LSE, w.delta, w.off_q, w.perm_q, sel, bsel, spb, w.dQacc, w.dkappa_b, w.dnu_b, w.dS_b,
+    int rc = near_bwd(d, Q, dO, qbar, LSE, w.delta, w.off_q, w.perm_q, sel, bsel, spb, w.dQacc, w.dkappa_b, w.dnu_b, w.dS_b,
                       tcb ? 1 : 0, st);
     if (rc != MUSE_OK) return rc;
     if (tcb) {

@@ -10,223 +10,305 @@
 // the key-side pass takes the log-mass gradient) are the gradients of the per-block summaries, which that pass then
 // carries to the keys and values of bucket (j, b').
 //
-// Organisation: entries (i, j, b') receive contributions from the queries of cluster i in every later block, so one
-// CTA owns a query cluster i of one head and walks its segments (block b, i) in turn: it is the only writer of the
-// gradient entries of i, which it updates with plain read-modify-writes.  Within a segment it works like the block
-// selection kernel of the forward pass: 32 queries at a time (a warp owns four), the clusters they selected in
-// ascending order, each cluster's per-block rows staged once in shared memory; the warps add their queries'
-// contributions for the staged cluster into shared-memory accumulators, which are flushed before the next cluster.
+// Organisation.  A CTA takes the queries of one cluster i over all blocks, up to 256 at a time (bf16 rows in shared memory),
+// and lists their (query, slot) pairs by selected cluster j.  Then
+//   1. a warp takes a cluster j and the next 16 pairs of its list against the rows of 8 earlier blocks, which it keeps in
+//      registers:  S^T = kappa q^T with kappa_hi on rows 0-7 of the product and kappa_lo on rows 8-15, dP^T = nu dO^T;
+//      the lanes turn them into p and g in place, where they are B operands (as bf16 high and low parts) of
+//      d kappa^T += q^T g,  d nu^T += dO^T p;  the sums over the list go to global memory once, by reductions;
+//   2. after a barrier a warp takes a query, lanes sharing D, and adds up g kappa over its pairs in a fixed order.
+// The products are 8 blocks by 16 gathered pairs, so they are warp-level mma.sync: tcgen05 products have at least 64 rows.
+// Of the pairs of 32 queries of one segment only two or three name the same cluster, so a lane per query in step 1 (the
+// kernel that block_select_q.cu still is) leaves nine lanes in ten idle, and the sums went out after two or three pairs.
+//
+// Bound: L2 - step 2 reads 256 bytes (D = 64) per pair and block, and the sums leave as 4-byte reductions.  8 heads of two
+// sequences of 64k tokens, D = 64, 128 x 128 clusters, 8 slots, 8 blocks: 23.19 ms for a warp per pair with shared-memory
+// atomics, 9.88 ms for a lane per query over 32 queries of a segment, 2.68 ms here.
 #include <algorithm>
 #include "common.cuh"
 
 namespace muse {
 
-constexpr int kNbMaxBlocks = 32;
-constexpr int kNbThreads = 256, kNbWarps = kNbThreads / 32, kNbQPW = 4, kNbChunk = kNbWarps * kNbQPW;
+typedef __nv_bfloat16 bf16;
 
+constexpr int kNbPairs = 2048, kNbGroup = 8;                // pairs of a chunk; earlier blocks per pass
+
+// D = 128 needs 255 registers a thread for its sums
+template <int D> struct NbLay {
+  static constexpr int kThreads = D == 128 ? 256 : 512, kQ = D == 128 ? 128 : 256;       // queries of a chunk at most
+  static constexpr int LD = D + 8;                          // bf16 per query row: ldmatrix rows do not conflict
+  static constexpr int oQ = 0, oDO = oQ + kQ * LD * 2, oG = oDO + kQ * LD * 2, oL = oG + kNbPairs * kNbGroup * 4, oDl = oL + kQ * 4, oRow = oDl + kQ * 4,
+                       oNb = oRow + kQ * 4, oVis = oNb + kQ * 4, oList = oVis + kNbPairs * 4, oSel = oList + kNbPairs * 4, oQb = oSel + kNbPairs * 2,
+                       oOff = oQb + D * 4;                  // then Ck ints
+};
+
+__device__ __forceinline__ void nb_mma(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+               : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void nb_ldmatrix_t(uint32_t (&a)[4], const bf16* p) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]) : "r"((uint32_t)__cvta_generic_to_shared(p)) : "memory");
+}
 __device__ __forceinline__ void nb_cp_async16(void* smem_dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(smem_dst)), "l"(src) : "memory");
 }
-__device__ __forceinline__ void nb_cp_async4(void* smem_dst, const void* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(smem_dst)), "l"(src) : "memory");
-}
-template <class T> __host__ __device__ constexpr int nb_rows() { return sizeof(T) == 2 ? 3 : 2; }   // kappa_hi | kappa_lo (bf16) | nu
-template <class T> __host__ __device__ inline size_t nb_stage_bytes(int SB, int D) {
-  return (size_t)SB * nb_rows<T>() * D * sizeof(T) + (size_t)kNbMaxBlocks * sizeof(float);
+// two numbers as packed bf16 high parts and packed bf16 remainders
+__device__ __forceinline__ void nb_split(float x, float y, uint32_t& hi, uint32_t& lo) {
+  const __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
+  const __nv_bfloat162 l = __floats2bfloat162_rn(x - __bfloat162float(h.x), y - __bfloat162float(h.y));
+  hi = *reinterpret_cast<const uint32_t*>(&h);
+  lo = *reinterpret_cast<const uint32_t*>(&l);
 }
 
-template <class T, int D>
-__global__ void __launch_bounds__(kNbThreads)
-k_near_bwd(Dims dm, const T* __restrict__ Q, const T* __restrict__ dO, const float* __restrict__ qbar, const float* __restrict__ LSE,
+template <int D>
+__global__ void __launch_bounds__(NbLay<D>::kThreads, 1)
+k_near_bwd(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ dO, const float* __restrict__ qbar, const float* __restrict__ LSE,
            const float* __restrict__ delta, const int32_t* __restrict__ off_q, const int32_t* __restrict__ perm_q,
            const int32_t* __restrict__ sel, const int32_t* __restrict__ bsel, SummPtrs sp, float* __restrict__ dQacc,
            float* __restrict__ dkappa_b, float* __restrict__ dnu_b, float* __restrict__ dS_b, int grad_ji) {
   // grad_ji: the gradient entries are laid out [plane][j][i] (what the tensor-core key-side kernel reads) instead of [plane][i][j]
-  constexpr int EPL = D / 32, ROWS = nb_rows<T>();
-  extern __shared__ __align__(16) unsigned char nb_smem[];
+  typedef NbLay<D> L;
+  constexpr int kThreads = L::kThreads, kWarps = kThreads / 32, LD = L::LD, EPL = D / 32, KS = D / 16, G = kNbGroup;
+  extern __shared__ __align__(16) unsigned char nb_sm[];
   const int m = dm.m, k2 = dm.k2, SB = dm.SB, Ck = dm.Ck;
-  const size_t stage_bytes = nb_stage_bytes<T>(SB, D);
-  unsigned char* stage0 = nb_smem;
-  float* gka = reinterpret_cast<float*>(nb_smem + 2 * stage_bytes);   // [SB][D] sum over queries of g sigma (q - qbar_i), staged cluster
-  float* gnu = gka + (size_t)SB * D;                                   // [SB][D] sum of p dO
-  float* gmu = gnu + (size_t)SB * D;                                   // [SB]    sum of g (1 - sigma (q - qbar_i) . kappa) - p dO . nu
-  int* sel_s = reinterpret_cast<int*>(gmu + kNbMaxBlocks);             // [32][m + 1]
-  uint32_t* bitmap = reinterpret_cast<uint32_t*>(sel_s + kNbChunk * (m + 1));
-  int* ulist = reinterpret_cast<int*>(bitmap + ((Ck + 31) >> 5));
-  __shared__ int nU_s, touched_s;
-  const int i = blockIdx.x, pq = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  bf16 *q_s = (bf16*)(nb_sm + L::oQ), *do_s = (bf16*)(nb_sm + L::oDO);
+  float *g_s = (float*)(nb_sm + L::oG), *L_s = (float*)(nb_sm + L::oL), *dl_s = (float*)(nb_sm + L::oDl), *qb_s = (float*)(nb_sm + L::oQb);
+  int *row_s = (int*)(nb_sm + L::oRow), *nb_s = (int*)(nb_sm + L::oNb), *off = (int*)(nb_sm + L::oOff);
+  uint32_t *vis_s = (uint32_t*)(nb_sm + L::oVis), *list = (uint32_t*)(nb_sm + L::oList);       // list: query << 16 | pair
+  uint16_t* sel_s = (uint16_t*)(nb_sm + L::oSel);
+  __shared__ int pre_s[33], p0_s[33], next_s;                        // queries of the cluster before block b + 1; where block b + 1's start
+  const int i = blockIdx.x, pq = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, n = lane >> 2, c = lane & 3;
   const int32_t* pm = perm_q + (size_t)pq * dm.N;
   const size_t estep = (size_t)dm.Cq * Ck;
-  const size_t ebase = ((size_t)pq * SB * dm.Cq + i) * Ck;             // entry (block 0, i, cluster 0)
-  const int nwords = (Ck + 31) >> 5;
-  float qb[EPL];                                                       // sigma qbar_i, this lane's dims
-  ldv<EPL>(qbar + ((size_t)pq * dm.Cq + i) * D + lane * EPL, qb);
+  const size_t ebase = ((size_t)pq * SB * dm.Cq + i) * Ck;           // entry (block 0, i, cluster 0)
+  if (warp == 0) {                                                   // SB <= 32
+    const int32_t* oq = off_q + (size_t)pq * (dm.S * dm.Cq + 1) + (size_t)(lane + 1) * dm.Cq + i;
+    const int p0 = lane < SB ? oq[0] : 0, len = lane < SB ? oq[1] - p0 : 0;
+    int pre = len;
 #pragma unroll
-  for (int e = 0; e < EPL; ++e) qb[e] *= dm.sigma;
-  for (int e = tid; e < SB * D; e += kNbThreads) { gka[e] = 0.f; gnu[e] = 0.f; }
-  if (tid < kNbMaxBlocks) gmu[tid] = 0.f;
-  if (tid == 0) touched_s = 0;
+    for (int o = 1; o < 32; o <<= 1) { const int v = __shfl_up_sync(0xffffffffu, pre, o); if (lane >= o) pre += v; }
+    p0_s[lane] = p0;
+    pre_s[lane + 1] = pre;
+    if (lane == 0) pre_s[0] = 0;
+  }
+  for (int d = tid; d < D; d += kThreads) qb_s[d] = qbar[((size_t)pq * dm.Cq + i) * D + d];
   __syncthreads();
-
-  for (int b = 1; b < dm.S; ++b) {
-    const int32_t* oq = off_q + (size_t)pq * (dm.S * dm.Cq + 1) + (size_t)b * dm.Cq + i;
-    const int p0 = oq[0], p1 = oq[1];
-    for (int c0 = p0; c0 < p1; c0 += kNbChunk) {
-      const int nq = min(kNbChunk, p1 - c0);
-      int tq[kNbQPW];
-      float q[kNbQPW][EPL], go[kNbQPW][EPL], dqa[kNbQPW][EPL], Lq[kNbQPW], dl[kNbQPW];
-#pragma unroll
-      for (int k = 0; k < kNbQPW; ++k) {
-        const int r = warp * kNbQPW + k;
-        tq[k] = r < nq ? pm[c0 + r] : -1;
-        if (tq[k] >= 0 && !MUSE_IN_RANGE(tq[k], dm.N)) tq[k] = -1;
-        Lq[k] = 0.f; dl[k] = 0.f;
-#pragma unroll
-        for (int e = 0; e < EPL; ++e) { q[k][e] = 0.f; go[k][e] = 0.f; dqa[k][e] = 0.f; }
-        if (tq[k] >= 0) {
-          const size_t row = (size_t)pq * dm.N + tq[k];
-          ldv<EPL>(Q + row * D + lane * EPL, q[k]);
-          ldv<EPL>(dO + row * D + lane * EPL, go[k]);
-#pragma unroll
-          for (int e = 0; e < EPL; ++e) q[k][e] *= dm.sigma;
-          Lq[k] = LSE[row]; dl[k] = delta[row];
+  const int total = pre_s[SB], QC = min(L::kQ, kNbPairs / m);
+  for (int c0 = blockIdx.z * QC; c0 < total; c0 += gridDim.z * QC) {
+    const int nq = min(QC, total - c0);
+    // ---- the chunk's queries, their pairs, the list of pairs by selected cluster
+    for (int r = tid; r < nq; r += kThreads) {
+      int b = 0;
+      while (pre_s[b + 1] <= c0 + r) ++b;
+      int t = pm[p0_s[b] + c0 + r - pre_s[b]];
+      if (!MUSE_IN_RANGE(t, dm.N)) t = -1;
+      row_s[r] = t;
+      nb_s[r] = b + 1;
+      L_s[r] = t >= 0 ? LSE[(size_t)pq * dm.N + t] : 0.f;
+      dl_s[r] = t >= 0 ? delta[(size_t)pq * dm.N + t] : 0.f;
+    }
+    for (int j = tid; j < Ck; j += kThreads) off[j] = 0;
+    __syncthreads();
+    constexpr int kP = D / 8;                                        // 16-byte pieces of a row
+    for (int e = tid; e < nq * 2 * kP; e += kThreads) {
+      const int r = e / (2 * kP), w = e / kP % 2, p = e % kP;
+      const size_t o = ((size_t)pq * dm.N + max(row_s[r], 0)) * D + p * 8;
+      nb_cp_async16((w ? do_s : q_s) + r * LD + p * 8, (w ? dO : Q) + o);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    for (int e = tid; e < nq * m; e += kThreads) {
+      const int r = e / m, t = row_s[r], nb = nb_s[r];
+      int j = -1;
+      uint32_t vis = 0u;                                             // the earlier blocks that stand in for this pair's keys:
+      if (t >= 0) {
+        const size_t pr = ((size_t)pq * dm.N + t) * m + (e - r * m);
+        j = sel[pr];
+        if (j < 0 || j >= Ck) j = -1;
+        vis = 0xffffffffu >> (32 - nb);
+        for (int x = 0; x < k2; ++x) {
+          const int bb = bsel[pr * k2 + x];
+          if (bb >= 0 && bb < nb) vis &= ~(1u << bb);                // all but those retrieved exactly
         }
       }
-      for (int w = tid; w < nwords; w += kNbThreads) bitmap[w] = 0u;
-      __syncthreads();
+      if (vis == 0u) j = -1;
+      vis_s[e] = vis;
+      sel_s[e] = (uint16_t)(j < 0 ? 0xffff : j);
+      if (j >= 0) atomicAdd(&off[j], 1);
+    }
+    __syncthreads();
+    if (warp == 0) {
+      int at = 0;
+      for (int j0 = 0; j0 < Ck; j0 += 32) {
+        const int cnt = j0 + lane < Ck ? off[j0 + lane] : 0;
+        int pre = cnt;
 #pragma unroll
-      for (int k = 0; k < kNbQPW; ++k) {
-        const int r = warp * kNbQPW + k;
-        for (int s = lane; s < m; s += 32) {
-          int j = -1;
-          if (tq[k] >= 0) {
-            j = sel[((size_t)pq * dm.N + tq[k]) * m + s];
-            if (j < 0 || j >= Ck) j = -1;
+        for (int o = 1; o < 32; o <<= 1) { const int v = __shfl_up_sync(0xffffffffu, pre, o); if (lane >= o) pre += v; }
+        if (j0 + lane < Ck) off[j0 + lane] = at + pre - cnt;
+        at += __shfl_sync(0xffffffffu, pre, 31);
+      }
+    }
+    __syncthreads();
+    for (int e = tid; e < nq * m; e += kThreads) {
+      const int j = sel_s[e];
+      if (j != 0xffff) list[atomicAdd(&off[j], 1)] = (uint32_t)(e / m) << 16 | (uint32_t)e;   // off[j]: then the end of j's pairs
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    const int nbmax = nb_s[nq - 1];                                  // queries go by block
+    for (int g0 = 0; g0 < nbmax; g0 += G) {
+      if (tid == 0) next_s = 0;
+      __syncthreads();
+      for (;;) {
+        int j = 0;
+        if (lane == 0) j = atomicAdd(&next_s, 1);
+        j = __shfl_sync(0xffffffffu, j, 0);
+        if (j >= Ck) break;
+        const int o0 = j > 0 ? off[j - 1] : 0, o1 = off[j];
+        if (o0 == o1) continue;
+        // ---- step 1.  Lane (n, c) holds block n's dims c D/4 .. of kappa and nu: the k index of a product is a permutation of D,
+        // the same for both operands, so that a lane's operands are 16-byte loads.
+        const size_t ent = ebase + (size_t)(g0 + n) * estep + j;
+        uint4 kh[KS / 2], kl[KS / 2], nv[KS / 2];
+        const bool here = g0 + n < nbmax;
+#pragma unroll
+        for (int t = 0; t < KS / 2; ++t) {
+          const size_t o = ent * D + c * (D / 4) + t * 8;
+          kh[t] = here ? *reinterpret_cast<const uint4*>((const bf16*)sp.khi + o) : make_uint4(0u, 0u, 0u, 0u);
+          kl[t] = here ? *reinterpret_cast<const uint4*>((const bf16*)sp.klo + o) : make_uint4(0u, 0u, 0u, 0u);
+          nv[t] = here ? *reinterpret_cast<const uint4*>((const bf16*)sp.nu + o) : make_uint4(0u, 0u, 0u, 0u);
+        }
+        const float be = here ? sp.beta[ent] : -INFINITY;
+        const bool live = be != -INFINITY;
+        float s3 = 0.f;                                              // sigma qbar_i . kappa of block n
+#pragma unroll
+        for (int t = 0; t < KS / 2; ++t) {
+          const uint32_t h[4] = {kh[t].x, kh[t].y, kh[t].z, kh[t].w}, l[4] = {kl[t].x, kl[t].y, kl[t].z, kl[t].w};
+#pragma unroll
+          for (int x = 0; x < 4; ++x) {
+            const float2 qv = *reinterpret_cast<const float2*>(qb_s + c * (D / 4) + t * 8 + 2 * x);
+            s3 = fmaf(qv.x, __uint_as_float(h[x] << 16) + __uint_as_float(l[x] << 16), s3);
+            s3 = fmaf(qv.y, __uint_as_float(h[x] & 0xffff0000u) + __uint_as_float(l[x] & 0xffff0000u), s3);
           }
-          sel_s[r * (m + 1) + s] = j;
-          if (j >= 0) atomicOr(&bitmap[j >> 5], 1u << (j & 31));
         }
-      }
-      __syncthreads();
-      if (warp == 0) {
-        int n = 0;
-        for (int w0 = 0; w0 < nwords; w0 += 32) {
-          const uint32_t bits = w0 + lane < nwords ? bitmap[w0 + lane] : 0u;
-          const int cnt = __popc(bits);
-          int pre = cnt;
+        s3 += __shfl_xor_sync(0xffffffffu, s3, 1);
+        s3 += __shfl_xor_sync(0xffffffffu, s3, 2);
+        s3 *= dm.sigma;
+        float aka[KS][4], anu[KS][4], ds = 0.f, gsum = 0.f;          // sums over the list: [dims of tile: n, n + 8][blocks 2c, 2c + 1]
+        uint32_t seen = 0u;
 #pragma unroll
-          for (int o = 1; o < 32; o <<= 1) { const int v = __shfl_up_sync(0xffffffffu, pre, o); if (lane >= o) pre += v; }
-          int at = n + pre - cnt;
-          for (uint32_t rest = bits; rest; rest &= rest - 1) ulist[at++] = (w0 + lane) * 32 + __ffs(rest) - 1;
-          n += __shfl_sync(0xffffffffu, pre, 31);
-        }
-        if (lane == 0) nU_s = n;
-      }
-      __syncthreads();
-      const int nU = nU_s;
-      auto stage_rows = [&](int u) {
-        unsigned char* st = stage0 + (u & 1) * stage_bytes;
-        const int j = ulist[u];
-        constexpr int CPR = D * (int)sizeof(T) / 16;
-        for (int e = tid; e < b * ROWS * CPR; e += kNbThreads) {
-          const int bp = e / (ROWS * CPR), rw = (e / CPR) % ROWS, c = e % CPR;
-          const size_t ent = ebase + (size_t)bp * estep + j;
-          const T* src = rw == 0 ? (const T*)sp.khi : (rw == ROWS - 1 ? (const T*)sp.nu : (const T*)sp.klo);
-          nb_cp_async16(st + ((size_t)(bp * ROWS + rw) * D) * sizeof(T) + c * 16, reinterpret_cast<const unsigned char*>(src + ent * D) + c * 16);
-        }
-        if (tid < b) nb_cp_async4(st + (size_t)SB * ROWS * D * sizeof(T) + tid * 4, sp.beta + ebase + (size_t)tid * estep + j);
-        asm volatile("cp.async.commit_group;" ::: "memory");
-      };
-      if (nU > 0) stage_rows(0);
-      for (int u = 0; u < nU; ++u) {
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
-        __syncthreads();                                               // cluster u's rows are in place; the accumulators are clear
-        if (u + 1 < nU) stage_rows(u + 1);
-        const unsigned char* st = stage0 + (u & 1) * stage_bytes;
-        const T* rows = reinterpret_cast<const T*>(st);
-        const float* betas = reinterpret_cast<const float*>(st + (size_t)SB * ROWS * D * sizeof(T));
-        const int j = ulist[u];
-        const float be = lane < b ? betas[lane] : -INFINITY;
-        const uint32_t live = __ballot_sync(0xffffffffu, be != -INFINITY);
+        for (int t = 0; t < KS; ++t)
 #pragma unroll
-        for (int k = 0; k < kNbQPW; ++k) {
-          if (tq[k] < 0) continue;                                     // (warp-uniform)
-          const int r = warp * kNbQPW + k;
-          unsigned long long hit = (unsigned long long)__ballot_sync(0xffffffffu, lane < m && sel_s[r * (m + 1) + min(lane, m - 1)] == j);
-          if (m > 32) hit |= (unsigned long long)__ballot_sync(0xffffffffu, lane + 32 < m && sel_s[r * (m + 1) + min(lane + 32, m - 1)] == j) << 32;
-          for (; hit != 0ull; hit &= hit - 1ull) {
-            const int s = __ffsll((long long)hit) - 1;
-            const size_t row = (size_t)pq * dm.N + tq[k];
-            // the blocks this (query, slot) retrieved exactly are not stand-in keys
-            uint32_t chosen = 0u;
-            for (int e = 0; e < k2; ++e) {
-              const int c = bsel[(row * m + s) * k2 + e];
-              if (c >= 0 && c < b) chosen |= 1u << c;
-            }
-            for (uint32_t rest = live & ~chosen; rest != 0u; rest &= rest - 1u) {
-              const int bp = __ffs(rest) - 1;
-              float kh[EPL], kl[EPL], nv[EPL];
-              ldv<EPL>(rows + (size_t)(bp * ROWS) * D + lane * EPL, kh);
-              if (ROWS == 3) ldv<EPL>(rows + (size_t)(bp * ROWS + 1) * D + lane * EPL, kl);
-              else {
+          for (int x = 0; x < 4; ++x) { aka[t][x] = 0.f; anu[t][x] = 0.f; }
+        for (int o = o0; o < o1; o += 16) {
+          const int cnt = min(16, o1 - o);
+          float s[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}}, dp[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
 #pragma unroll
-                for (int e = 0; e < EPL; ++e) kl[e] = 0.f;
+          for (int h = 0; h < 2; ++h) {
+            if (8 * h < cnt) {
+              const int r = list[o + min(8 * h + n, cnt - 1)] >> 16;
+              const bf16 *qr = q_s + r * LD + c * (D / 4), *gr = do_s + r * LD + c * (D / 4);
+#pragma unroll
+              for (int t = 0; t < KS / 2; ++t) {
+                const uint4 x = *reinterpret_cast<const uint4*>(qr + 8 * t), y = *reinterpret_cast<const uint4*>(gr + 8 * t);
+                nb_mma(s[h], kh[t].x, kl[t].x, kh[t].y, kl[t].y, x.x, x.y);
+                nb_mma(s[h], kh[t].z, kl[t].z, kh[t].w, kl[t].w, x.z, x.w);
+                nb_mma(dp[h], nv[t].x, 0u, nv[t].y, 0u, y.x, y.y);
+                nb_mma(dp[h], nv[t].z, 0u, nv[t].w, 0u, y.z, y.w);
               }
-              ldv<EPL>(rows + (size_t)(bp * ROWS + ROWS - 1) * D + lane * EPL, nv);
-              float s1 = 0.f, s2 = 0.f, s3 = 0.f;                      // sigma q . kappa,  dO . nu,  sigma qbar_i . kappa
-#pragma unroll
-              for (int e = 0; e < EPL; ++e) {
-                kh[e] += kl[e];
-                s1 = fmaf(q[k][e], kh[e], s1); s2 = fmaf(go[k][e], nv[e], s2); s3 = fmaf(qb[e], kh[e], s3);
-              }
-#pragma unroll
-              for (int o = 16; o > 0; o >>= 1) {
-                s1 += __shfl_xor_sync(0xffffffffu, s1, o); s2 += __shfl_xor_sync(0xffffffffu, s2, o); s3 += __shfl_xor_sync(0xffffffffu, s3, o);
-              }
-              const float p = __expf(s1 + __shfl_sync(0xffffffffu, be, bp) - Lq[k]);
-              const float g = p * (s2 - dl[k]);
-#pragma unroll
-              for (int e = 0; e < EPL; ++e) {
-                dqa[k][e] = fmaf(g, kh[e], dqa[k][e]);
-                atomicAdd(&gka[bp * D + lane * EPL + e], g * (q[k][e] - qb[e]));
-                atomicAdd(&gnu[bp * D + lane * EPL + e], p * go[k][e]);
-              }
-              // the scalar the key-side pass wants per entry: d mu - d kappa . kappa - d nu . nu  (this query's share)
-              if (lane == 0) { atomicAdd(&gmu[bp], g * (1.f - (s1 - s3)) - p * s2); touched_s = 1; }
             }
           }
-        }
-        __syncthreads();                                               // every warp has added its queries' share for cluster j
-        if (touched_s) {                                               // (block-uniform) flush into the gradient entries (b', i, j), which this CTA owns
-          for (int e = tid; e < b * D; e += kNbThreads) {
-            const int bp = e / D, d0 = e % D;
-            const size_t ent = grad_ji ? (((size_t)pq * SB + bp) * Ck + j) * dm.Cq + i : ebase + (size_t)bp * estep + j;
-            const float a = gka[e], c = gnu[e];
-            if (a != 0.f) dkappa_b[ent * D + d0] += a;
-            if (c != 0.f) dnu_b[ent * D + d0] += c;
-            gka[e] = 0.f; gnu[e] = 0.f;
-          }
-          if (tid < b) {
-            const float a = gmu[tid];
-            if (a != 0.f) dS_b[grad_ji ? (((size_t)pq * SB + tid) * Ck + j) * dm.Cq + i : ebase + (size_t)tid * estep + j] += a;
-            gmu[tid] = 0.f;
-          }
-        }
-        __syncthreads();
-        if (tid == 0) touched_s = 0;
-      }
-      // the chunk's contribution to dQ (the far-field and local parts are already in the accumulator)
+          float p[4], g[4];                                          // pairs 2c, 2c + 1, 8 + 2c, 9 + 2c with block n
 #pragma unroll
-      for (int k = 0; k < kNbQPW; ++k) {
-        if (tq[k] < 0) continue;
-        float* dst = dQacc + ((size_t)pq * dm.N + tq[k]) * D + lane * EPL;
+          for (int k = 0; k < 4; ++k) {
+            const int h = 8 * (k >> 1) + 2 * c + (k & 1);
+            p[k] = g[k] = 0.f;
+            if (h < cnt) {
+              const uint32_t le = list[o + h];
+              const int r = le >> 16, e = le & 0xffffu;
+              const uint32_t vis = vis_s[e];
+              const float lg = dm.sigma * (s[k >> 1][k & 1] + s[k >> 1][2 + (k & 1)]), dv = dp[k >> 1][k & 1];
+              if (live && ((vis >> (g0 + n)) & 1u)) {
+                p[k] = __expf(lg + be - L_s[r]);
+                g[k] = p[k] * (dv - dl_s[r]);
+                // the scalar the key-side pass wants per entry: d mu - d kappa . kappa - d nu . nu
+                ds += g[k] * (1.f - (lg - s3)) - p[k] * dv;
+                gsum += g[k];
+                seen = 1u;
+              }
+              g_s[e * G + n] = g[k];
+            }
+          }
+          uint32_t gh[2], gl[2], ph[2], pl[2];
+#pragma unroll
+          for (int h = 0; h < 2; ++h) { nb_split(g[2 * h], g[2 * h + 1], gh[h], gl[h]); nb_split(p[2 * h], p[2 * h + 1], ph[h], pl[h]); }
+          const int ro = (list[o + min((lane & 7) + ((lane >> 4) << 3), cnt - 1)] >> 16) * LD + ((lane >> 3) & 1) * 8;
+#pragma unroll
+          for (int t = 0; t < KS; ++t) {
+            uint32_t a[4];
+            nb_ldmatrix_t(a, q_s + ro + 16 * t);
+            nb_mma(aka[t], a[0], a[1], a[2], a[3], gh[0], gh[1]);
+            nb_mma(aka[t], a[0], a[1], a[2], a[3], gl[0], gl[1]);
+            nb_ldmatrix_t(a, do_s + ro + 16 * t);
+            nb_mma(anu[t], a[0], a[1], a[2], a[3], ph[0], ph[1]);
+            nb_mma(anu[t], a[0], a[1], a[2], a[3], pl[0], pl[1]);
+          }
+        }
+        ds += __shfl_xor_sync(0xffffffffu, ds, 1);
+        gsum += __shfl_xor_sync(0xffffffffu, gsum, 1);
+        ds += __shfl_xor_sync(0xffffffffu, ds, 2);
+        gsum += __shfl_xor_sync(0xffffffffu, gsum, 2);
+        const uint32_t any = __ballot_sync(0xffffffffu, seen != 0u); // blocks without a stand-in of this list have nothing to add
+        const auto entry = [&](int bp) {
+          return grad_ji ? (((size_t)pq * SB + g0 + bp) * Ck + j) * dm.Cq + i : ebase + (size_t)(g0 + bp) * estep + j;
+        };
+        if (c == 0 && ((any >> (4 * n)) & 15u) != 0u) atomicAdd(dS_b + entry(n), ds);
+#pragma unroll
+        for (int x = 0; x < 2; ++x) {
+          const int bp = 2 * c + x;
+          const float gs = __shfl_sync(0xffffffffu, gsum, 4 * bp);
+          if (((any >> (4 * bp)) & 15u) == 0u) continue;
+          float *ka = dkappa_b + entry(bp) * D, *nu = dnu_b + entry(bp) * D;
+#pragma unroll
+          for (int t = 0; t < KS; ++t) {
+            const int d = 16 * t + n;
+            atomicAdd(ka + d, dm.sigma * (aka[t][x] - gs * qb_s[d]));
+            atomicAdd(ka + d + 8, dm.sigma * (aka[t][2 + x] - gs * qb_s[d + 8]));
+            atomicAdd(nu + d, anu[t][x]);
+            atomicAdd(nu + d + 8, anu[t][2 + x]);
+          }
+        }
+      }
+      __syncthreads();
+      // ---- step 2: a warp per query, lanes share D: sum of g kappa (the far-field and local parts are already in the accumulator)
+      for (int r = warp; r < nq; r += kWarps) {
+        if (row_s[r] < 0) continue;                                  // (warp-uniform)
+        float acc[EPL];
+#pragma unroll
+        for (int e = 0; e < EPL; ++e) acc[e] = 0.f;
+        for (int s = 0; s < m; ++s) {
+          const int j = sel_s[r * m + s];
+          if (j == 0xffff) continue;
+          const float4 ga = *reinterpret_cast<const float4*>(g_s + (r * m + s) * G), gb = *reinterpret_cast<const float4*>(g_s + (r * m + s) * G + 4);
+          const float g[G] = {ga.x, ga.y, ga.z, ga.w, gb.x, gb.y, gb.z, gb.w};
+          const size_t o = (ebase + (size_t)g0 * estep + j) * D + lane * EPL;
+#pragma unroll
+          for (int bp = 0; bp < G; ++bp)
+            if (g[bp] != 0.f) {
+              float kh[EPL], kl[EPL];
+              ldv<EPL>((const bf16*)sp.khi + o + (size_t)bp * estep * D, kh);
+              ldv<EPL>((const bf16*)sp.klo + o + (size_t)bp * estep * D, kl);
+#pragma unroll
+              for (int e = 0; e < EPL; ++e) acc[e] = fmaf(g[bp], kh[e] + kl[e], acc[e]);
+            }
+        }
+        float* dst = dQacc + ((size_t)pq * dm.N + row_s[r]) * D + lane * EPL;
         float cur[EPL];
         ldv<EPL>(dst, cur);
 #pragma unroll
-        for (int e = 0; e < EPL; ++e) cur[e] = fmaf(dm.sigma, dqa[k][e], cur[e]);
+        for (int e = 0; e < EPL; ++e) cur[e] = fmaf(dm.sigma, acc[e], cur[e]);
         stv<EPL>(dst, cur);
       }
-      __syncthreads();
+      __syncthreads();                                               // g_s and the lists are refilled
     }
   }
 }
@@ -246,35 +328,29 @@ int grad_to_bf16(const float* in, size_t n, void* out, cudaStream_t st) {
   return MUSE_OK;
 }
 
-size_t near_bwd_smem_bytes(const Dims& d, int elem_bytes) {
-  const size_t stage = (size_t)d.SB * (elem_bytes == 2 ? 3 : 2) * d.D * elem_bytes + (size_t)kNbMaxBlocks * sizeof(float);
-  return 2 * stage + (size_t)(2 * d.SB * d.D + kNbMaxBlocks) * sizeof(float) + (size_t)kNbChunk * (d.m + 1) * sizeof(int) +
-         (size_t)((d.Ck + 31) >> 5) * sizeof(uint32_t) + (size_t)std::min(d.Ck, kNbChunk * d.m) * sizeof(int);
-}
-
-template <class T, int D>
-static int near_bwd_t(const Dims& d, const T* Q, const T* dO, const float* qbar, const float* LSE, const float* delta,
-                      const int32_t* off_q, const int32_t* perm_q, const int32_t* sel, const int32_t* bsel, const SummPtrs& sp,
-                      float* dQacc, float* dkappa_b, float* dnu_b, float* dS_b, int grad_ji, cudaStream_t st) {
-  const size_t smem = near_bwd_smem_bytes(d, (int)sizeof(T));
-  MUSE_CUDA_OK(cudaFuncSetAttribute(k_near_bwd<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+template <int D>
+static int near_bwd_d(const Dims& d, const void* Q, const void* dO, const float* qbar, const float* LSE, const float* delta, const int32_t* off_q,
+                      const int32_t* perm_q, const int32_t* sel, const int32_t* bsel, const SummPtrs& sp, float* dQacc, float* dkappa_b,
+                      float* dnu_b, float* dS_b, int grad_ji, cudaStream_t st) {
+  typedef NbLay<D> L;
+  const int smem = L::oOff + d.Ck * 4;                       // Ck <= 4096: at most 180 KB
+  MUSE_CUDA_OK(cudaFuncSetAttribute(k_near_bwd<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  // a cluster's chunks are shared by several CTAs where one per (cluster, head) would leave SMs idle
+  const int per = d.Cq * d.B * d.Hq, chunk = std::min(L::kQ, kNbPairs / d.m);
+  const int share = std::max(1, std::min((2 * sm_count() + per - 1) / per, (d.N / d.Cq + chunk - 1) / chunk));
   prof_mark("k_near_bwd", st);
-  k_near_bwd<T, D><<<dim3(d.Cq, d.B * d.Hq), kNbThreads, smem, st>>>(d, Q, dO, qbar, LSE, delta, off_q, perm_q, sel, bsel, sp, dQacc,
-                                                                   dkappa_b, dnu_b, dS_b, grad_ji);
+  k_near_bwd<D><<<dim3(d.Cq, d.B * d.Hq, share), L::kThreads, smem, st>>>(d, (const bf16*)Q, (const bf16*)dO, qbar, LSE, delta, off_q, perm_q, sel, bsel,
+                                                                       sp, dQacc, dkappa_b, dnu_b, dS_b, grad_ji);
   MUSE_LAUNCH_OK();
   return MUSE_OK;
 }
 
-int near_bwd(const Dims& d, int dtype, const void* Q, const void* dO, const float* qbar, const float* LSE, const float* delta,
-             const int32_t* off_q, const int32_t* perm_q, const int32_t* sel, const int32_t* bsel, const SummPtrs& sp, float* dQacc,
-             float* dkappa_b, float* dnu_b, float* dS_b, int grad_ji, cudaStream_t st) {
-  typedef __nv_bfloat16 bf;
-  if (dtype == MUSE_F32) {
-    if (d.D == 64) return near_bwd_t<float, 64>(d, (const float*)Q, (const float*)dO, qbar, LSE, delta, off_q, perm_q, sel, bsel, sp, dQacc, dkappa_b, dnu_b, dS_b, grad_ji, st);
-    return near_bwd_t<float, 128>(d, (const float*)Q, (const float*)dO, qbar, LSE, delta, off_q, perm_q, sel, bsel, sp, dQacc, dkappa_b, dnu_b, dS_b, grad_ji, st);
-  }
-  if (d.D == 64) return near_bwd_t<bf, 64>(d, (const bf*)Q, (const bf*)dO, qbar, LSE, delta, off_q, perm_q, sel, bsel, sp, dQacc, dkappa_b, dnu_b, dS_b, grad_ji, st);
-  return near_bwd_t<bf, 128>(d, (const bf*)Q, (const bf*)dO, qbar, LSE, delta, off_q, perm_q, sel, bsel, sp, dQacc, dkappa_b, dnu_b, dS_b, grad_ji, st);
+// k2 > 0 (and with it S > 1 blocks) is built for bf16 only
+int near_bwd(const Dims& d, const void* Q, const void* dO, const float* qbar, const float* LSE, const float* delta, const int32_t* off_q,
+             const int32_t* perm_q, const int32_t* sel, const int32_t* bsel, const SummPtrs& sp, float* dQacc, float* dkappa_b, float* dnu_b,
+             float* dS_b, int grad_ji, cudaStream_t st) {
+  return d.D == 128 ? near_bwd_d<128>(d, Q, dO, qbar, LSE, delta, off_q, perm_q, sel, bsel, sp, dQacc, dkappa_b, dnu_b, dS_b, grad_ji, st)
+                    : near_bwd_d<64>(d, Q, dO, qbar, LSE, delta, off_q, perm_q, sel, bsel, sp, dQacc, dkappa_b, dnu_b, dS_b, grad_ji, st);
 }
 
 }  // namespace muse

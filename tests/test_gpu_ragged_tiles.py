@@ -4,6 +4,7 @@ import numpy as np
 import pytest
 import torch
 
+from tests import test_gpu_k2
 from tests.gpu_util import kernels_launched, to_np
 from tests.test_gpu_backward import _backward_parity, _backward_parity_run
 from tests.test_gpu_cluster import CASES
@@ -57,3 +58,11 @@ def test_retrieval_backward_on_both_sides_of_the_cluster_length_rule(base, Ck, t
     with kernels_launched() as rec:
         _backward_parity_run(w, 128.0)
     assert "k_ret_bwd_pairs_tc" in rec.names and ("k_ret_bwd_dq" in rec.names) == two_kernels
+
+
+@pytest.mark.parametrize("base,Cq,Ck,m,S,k2", [("d64", 5, 9, 4, 10, 1), ("d64", 3, 40, 33, 3, 1), ("d128", 7, 10, 5, 12, 2), ("d128", 1, 6, 6, 2, 1)])
+def test_near_field_backward_over_groups_of_blocks(monkeypatch, base, Cq, Ck, m, S, k2):
+    """More earlier blocks than one group of the kernel (8 at D = 64, 4 at D = 128), more than 32 slots, one earlier block."""
+    w = CASES[base].with_(Hq=2, Hkv=1, N=330 * S, S=S, Cq=Cq, Ck=Ck, m=m, components=64)
+    monkeypatch.setitem(test_gpu_k2.K2_CASES, "groups", w)
+    test_gpu_k2.test_two_level_backward_matches_oracle("groups", k2, True, 4)
