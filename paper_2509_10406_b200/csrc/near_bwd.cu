@@ -18,20 +18,19 @@
 //      d kappa^T += q^T g,  d nu^T += dO^T p;  the sums over the list go to global memory once, by reductions;
 //   2. after a barrier a warp takes a query, lanes sharing D, and adds up g kappa over its pairs in a fixed order.
 // The products are 8 blocks by 16 gathered pairs, so they are warp-level mma.sync: tcgen05 products have at least 64 rows.
-// Of the pairs of 32 queries of one segment only two or three name the same cluster, so a lane per query in step 1 (the
-// kernel that block_select_q.cu still is) leaves nine lanes in ten idle, and the sums went out after two or three pairs.
+// Of the pairs of 32 queries of one segment only two or three name the same cluster: a lane per query in step 1 left nine
+// lanes in ten idle, and the sums went out after two or three pairs.
 //
 // Bound: L2 - step 2 reads 256 bytes (D = 64) per pair and block, and the sums leave as 4-byte reductions.  8 heads of two
 // sequences of 64k tokens, D = 64, 128 x 128 clusters, 8 slots, 8 blocks: 23.19 ms for a warp per pair with shared-memory
 // atomics, 9.88 ms for a lane per query over 32 queries of a segment, 2.68 ms here.
 #include <algorithm>
 #include "common.cuh"
+#include "near.cuh"
 
 namespace muse {
 
 typedef __nv_bfloat16 bf16;
-
-constexpr int kNbPairs = 2048, kNbGroup = 8;                // pairs of a chunk; earlier blocks per pass
 
 // D = 128 needs 255 registers a thread for its sums
 template <int D> struct NbLay {
@@ -42,16 +41,9 @@ template <int D> struct NbLay {
                        oOff = oQb + D * 4;                  // then Ck ints
 };
 
-__device__ __forceinline__ void nb_mma(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
-  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-               : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
 __device__ __forceinline__ void nb_ldmatrix_t(uint32_t (&a)[4], const bf16* p) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
                : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]) : "r"((uint32_t)__cvta_generic_to_shared(p)) : "memory");
-}
-__device__ __forceinline__ void nb_cp_async16(void* smem_dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(smem_dst)), "l"(src) : "memory");
 }
 // two numbers as packed bf16 high parts and packed bf16 remainders
 __device__ __forceinline__ void nb_split(float x, float y, uint32_t& hi, uint32_t& lo) {
@@ -137,17 +129,7 @@ k_near_bwd(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ dO, con
       if (j >= 0) atomicAdd(&off[j], 1);
     }
     __syncthreads();
-    if (warp == 0) {
-      int at = 0;
-      for (int j0 = 0; j0 < Ck; j0 += 32) {
-        const int cnt = j0 + lane < Ck ? off[j0 + lane] : 0;
-        int pre = cnt;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) { const int v = __shfl_up_sync(0xffffffffu, pre, o); if (lane >= o) pre += v; }
-        if (j0 + lane < Ck) off[j0 + lane] = at + pre - cnt;
-        at += __shfl_sync(0xffffffffu, pre, 31);
-      }
-    }
+    if (warp == 0) nb_scan(off, Ck, lane);
     __syncthreads();
     for (int e = tid; e < nq * m; e += kThreads) {
       const int j = sel_s[e];
