@@ -1,0 +1,378 @@
+// Exact retrieval, forward, where key clusters are long (ret_fwd_tc.cu has the definitions and the kernel for short ones).
+// A CTA owns one key cluster of one head, or a share of its pairs, and walks units of two tiles of 128 retrieving pairs
+// (ordered by plane, so that the keys a tile sees are a prefix of the cluster) over the cluster's keys in tiles of 128, by
+// the scheme of the local forward kernel:
+//   S_q = Q_q K^T        Q rows gathered once per tile by 16-byte asynchronous copies, keys and values streamed by TMA
+//   P_q                  two threads per pair row at D = 64, one at D = 128; bf16 over the consumed logits in tensor memory
+//   O_q += P_q V         accumulated in tensor memory over the tile's keys, rescaled lazily
+// The (pair tile, key tile) products, numbered n over all units, go through NB logit buffers; products are issued in the
+// order ... O += P(n) V, S(n + NB) = Q K ..., which the tensor core keeps, so S(n + NB) may overwrite P(n) and the tensor
+// cores need not wait at a unit's end.  A pair's partial row is written once.
+//
+// Bound by the exponentials (16 per clock and SM) and the latency of a warp's pass over its logits.  64 heads of two
+// sequences of 64k tokens, D = 64, 512 keys per cluster, 8 slots: 7.32 ms with 128 resident keys per sweep, 4.47 ms here.
+#include <cuda.h>
+#include "common.cuh"
+#include "tc05.cuh"
+
+namespace muse {
+
+typedef __nv_bfloat16 bf16;
+int make_tmap_bf16_rows(void* out_map, const void* base, uint64_t rows, uint32_t cols, uint32_t box_rows);
+
+namespace rl {
+constexpr int kPairs = 128, kKeys = 128;
+constexpr int kSplit = 4, kUnitsPerCta = 8;                // a cluster with many units is shared by up to 4 CTAs
+constexpr int kOkCache = 72;                               // bucket offsets of the cluster kept in shared memory (S + 1 <= 72)
+template <int D> struct Lay {
+  static constexpr int kTile = 128 * D * 2, NS = D == 128 ? 2 : 3, NB = D == 128 ? 2 : 3, NQ = D == 128 ? 3 : 4;
+  static constexpr int H = D == 128 ? 1 : 2, kSoft = 256 * H, kGather = 64, kThreads = kSoft + 64 + kGather;
+  static constexpr int oQ = 0, oK = NQ * kTile, oV = oK + NS * kTile, total = oV + NS * kTile + 1024;
+};
+struct Bars { uint64_t q_full[4], q_empty[4], k_full[3], k_empty[3], v_full[3], v_empty[3], s_full[2][2], p_ready[2][2], pv_done[2]; };
+
+__device__ __forceinline__ void cp_async16(void* smem_dst, const void* src, bool valid) {
+  const int n = valid ? 16 : 0;                            // 0 source bytes: the 16 bytes are zero-filled
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(tc::smem_u32(smem_dst)), "l"(src), "r"(n) : "memory");
+}
+// barrier among `count` threads with an OR of their predicates
+__device__ __forceinline__ bool bar_or(int id, int count, bool p) {
+  uint32_t r;
+  asm volatile("{\n.reg .pred p, q;\nsetp.ne.u32 p, %1, 0;\nbarrier.cta.red.or.pred q, %2, %3, p;\nselp.u32 %0, 1, 0, q;\n}\n"
+               : "=r"(r) : "r"((uint32_t)p), "r"(id), "r"(count) : "memory");
+  return r != 0;
+}
+}  // namespace rl
+
+template <int D>
+__global__ void __launch_bounds__(rl::Lay<D>::kThreads, 1)
+k_ret_fwd_long(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v, const bf16* __restrict__ Q,
+               const int32_t* __restrict__ off_k, const int32_t* __restrict__ goff, const int32_t* __restrict__ pairs,
+               bf16* __restrict__ o_part, float* __restrict__ l_part, int* __restrict__ status) {
+  using namespace rl;
+  typedef Lay<D> LY;
+  constexpr int kTile = LY::kTile, NS = LY::NS, NB = LY::NB, NQ = LY::NQ, H = LY::H, kSoft = LY::kSoft, MW = kSoft / 32, G = D / 64, CPR = D / 8;
+  constexpr uint32_t cO = NB * kKeys;                      // tensor-memory columns: NB logit buffers | O_0 | O_1
+  extern __shared__ __align__(1024) unsigned char sm_raw[];
+  __shared__ Bars bars;
+  __shared__ uint32_t tbase_s;
+  __shared__ int32_t ok_s[kOkCache], tok_s[kPairs];
+  __shared__ float mx_s[2][2][kPairs];
+  const int tid = threadIdx.x, warp = tc::warp_index(), lane = tid & 31;
+  const int j = blockIdx.x, sub = blockIdx.y, pq = blockIdx.z, b_ = pq / dm.Hq, h = pq % dm.Hq, pk = b_ * dm.Hkv + dm.hm.g[h];
+  const int32_t* go = goff + (size_t)pq * (dm.SB * dm.Ck + 1) + (size_t)j * dm.SB;      // plane pl's pairs: [go[pl], go[pl + 1])
+  const int g0 = go[0], g1 = go[dm.SB], ntiles = (g1 - g0 + kPairs - 1) / kPairs, nunits = (ntiles + 1) / 2;
+  const int nsub = min(kSplit, max(1, nunits / kUnitsPerCta));            // units are dealt round-robin to nsub CTAs
+  if (ntiles == 0 || sub >= nsub) return;
+  const int32_t* okg = off_k + (size_t)pk * (dm.Ck * dm.S + 1) + (size_t)j * dm.S;      // okg[b]: first key of bucket (j, b)
+  const int k0 = okg[0];
+  const int32_t* ok = dm.S + 1 <= kOkCache ? ok_s : okg;
+  if (dm.S + 1 <= kOkCache)
+    for (int b = tid; b <= dm.S; b += LY::kThreads) ok_s[b] = okg[b];
+  unsigned char* sm = sm_raw + ((1024u - (tc::smem_u32(sm_raw) & 1023u)) & 1023u);
+  if (warp == MW) tc::tmem_alloc(&tbase_s, 512);
+  if (tid == 0) {
+    for (int q = 0; q < 2; ++q) {
+      for (int e = 0; e < 2; ++e) { tc::mbar_init(&bars.s_full[q][e], 1); tc::mbar_init(&bars.p_ready[q][e], kSoft / 2); }
+      tc::mbar_init(&bars.pv_done[q], 1);
+    }
+    for (int s = 0; s < NQ; ++s) { tc::mbar_init(&bars.q_full[s], LY::kGather); tc::mbar_init(&bars.q_empty[s], 1); }
+    for (int s = 0; s < NS; ++s) {
+      tc::mbar_init(&bars.k_full[s], 1); tc::mbar_init(&bars.k_empty[s], 1); tc::mbar_init(&bars.v_full[s], 1); tc::mbar_init(&bars.v_empty[s], 1);
+    }
+    tc::mbar_init_fence();
+  }
+  tc::fence_before_sync();
+  __syncthreads();
+  tc::fence_after_sync();
+  const uint32_t tbase = tbase_s;
+  bool ok_ = true;                                         // false once a bounded wait ran out (every role still walks all its units)
+  auto wait = [&](uint64_t* bar, uint32_t parity) { if (ok_ && !tc::mbar_wait(bar, parity)) ok_ = false; };
+  const int32_t* pr = pairs + (size_t)pq * dm.N * dm.m + g0;
+  const int np = g1 - g0;
+  const size_t pbase = (size_t)pq * dm.N * dm.m;
+  auto ld_pid = [&](int at) {                              // the pair at position `at` of the cluster's list
+    const int id = at < np ? __ldg(pr + at) : -1;
+    return id >= 0 && !MUSE_IN_RANGE(id, (long long)dm.N * dm.m) ? -1 : id;
+  };
+  auto ld_last = [&](int tile) { return ld_pid(min(tile * kPairs + kPairs, np) - 1 + (tile * kPairs < np ? 0 : np)); };   // -1 past the last tile
+  auto visible = [&](int pid) { return pid < 0 ? 0 : ok[dm.causal ? pid / dm.m / dm.Bs : 1] - k0; };     // keys the query of a pair sees
+  auto key_tiles = [&](int last) { return (visible(last) + kKeys - 1) / kKeys; };        // (a tile's last pair sees the most)
+
+  if (warp > MW + 1) {                                     // ---- gather of the Q rows
+    const int g = tid - (MW + 2) * 32, ck = g % CPR;
+    constexpr int RPP = LY::kGather / CPR, RPT = kPairs / LY::kGather;
+    const bf16* Qb = Q + (size_t)pq * dm.N * D + ck * 8;
+    int o = 0;                                             // tiles filled
+    for (int u = sub; u < nunits; u += nsub) {
+      int pa[2][RPT];
+#pragma unroll
+      for (int q = 0; q < 2; ++q)
+#pragma unroll
+        for (int x = 0; x < RPT; ++x) pa[q][x] = ld_pid((2 * u + q) * kPairs + g + x * LY::kGather);
+#pragma unroll
+      for (int q = 0; q < 2; ++q, ++o) {
+        const int s = o % NQ;
+#pragma unroll
+        for (int x = 0; x < RPT; ++x) tok_s[g + x * LY::kGather] = pa[q][x] >= 0 ? pa[q][x] / dm.m : -1;
+        wait(&bars.q_empty[s], ((o / NQ) & 1) ^ 1);
+        tc::named_bar_sync(5, LY::kGather);
+        unsigned char* qd = sm + LY::oQ + s * kTile + (ck >> 3) * kPairs * 128;
+#pragma unroll 8
+        for (int r = g / CPR; r < kPairs; r += RPP) {
+          const int tok = tok_s[r];
+          if (!MUSE_IN_RANGE(tok + 1, dm.N + 1)) continue;
+          cp_async16(qd + tc::sw128_off(r, ck & 7), Qb + (size_t)max(tok, 0) * D, tok >= 0);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        tc::fence_async_smem();                            // the tensor cores read the rows through the async proxy
+        tc::mbar_arrive(&bars.q_full[s]);
+        tc::named_bar_sync(5, LY::kGather);                // tok_s may be rewritten
+      }
+    }
+  } else if (warp == MW + 1) {                             // ---- keys and values
+    auto load = [&](unsigned char* dst, const void* map, int row, uint64_t* bar) {
+      if (tc::elect_one()) {
+        tc::mbar_expect_tx(bar, kTile);
+#pragma unroll
+        for (int g = 0; g < G; ++g) tc::tma_load_2d(dst + g * 128 * 128, map, 64 * g, row, bar);
+      }
+    };
+    int s = 0, ph = 0, l0 = ld_last(2 * sub), l1 = ld_last(2 * sub + 1);
+    for (int u = sub; u < nunits; u += nsub) {
+      const int T = max(key_tiles(l0), key_tiles(l1));
+      l0 = ld_last(2 * (u + nsub)); l1 = ld_last(2 * (u + nsub) + 1);
+      for (int t = 0; t < T; ++t) {                        // (rows past the keys that the tile sees are loaded too; they are masked)
+        const int row = pk * dm.N + k0 + t * kKeys;
+        wait(&bars.k_empty[s], ph ^ 1);
+        if (ok_) load(sm + LY::oK + s * kTile, &tm_k, row, &bars.k_full[s]);
+        wait(&bars.v_empty[s], ph ^ 1);
+        if (ok_) load(sm + LY::oV + s * kTile, &tm_v, row, &bars.v_full[s]);
+        if (++s == NS) { s = 0; ph ^= 1; }
+      }
+    }
+  } else if (warp == MW) {                                 // ---- products
+    const uint32_t id_s = tc::idesc_bf16(kPairs, kKeys, 0, 0), id_o = tc::idesc_bf16(kPairs, D, 0, 1);
+    const uint64_t dq = tc::smem_desc_sw128(tc::smem_u32(sm + LY::oQ), 16, 1024), dk = tc::smem_desc_sw128(tc::smem_u32(sm + LY::oK), 16, 1024),
+                   dv = tc::smem_desc_sw128(tc::smem_u32(sm + LY::oV), kKeys * 128, 1024);
+    // a cursor over the sequence of products (unit, key tile t, pair tile q); T: key tiles of the unit's two pair tiles
+    struct Cur { int u, t, q, T0, T1, T, l0, l1, n, e0, e1, o; };
+    auto enter = [&](Cur& c) {                             // the unit's numbers of key tiles; its successor's last pairs are on their way
+      c.T0 = key_tiles(c.l0); c.T1 = key_tiles(c.l1); c.T = max(c.T0, c.T1);
+      c.l0 = ld_last(2 * (c.u + nsub)); c.l1 = ld_last(2 * (c.u + nsub) + 1);
+      c.t = c.q = 0;
+    };
+    auto begin = [&](Cur& c) {
+      c.u = sub; c.n = c.e0 = c.e1 = c.o = 0;
+      c.l0 = ld_last(2 * sub); c.l1 = ld_last(2 * sub + 1);
+      enter(c);
+    };
+    Cur cs, cp;
+    begin(cs); begin(cp);
+    int sk = 0, phk = 0, sv = 0, phv = 0;
+    auto issue_s = [&]() {                                 // the next S of the sequence, where the pair exists
+      for (; cs.u < nunits && cs.t >= cs.T;) {          // (a unit that sees no keys: its rows are gathered all the same)
+        if (cs.t == 0)
+          for (int q = 0; q < 2; ++q) { wait(&bars.q_full[(cs.o + q) % NQ], ((cs.o + q) / NQ) & 1); tc::mma_commit_warp(&bars.q_empty[(cs.o + q) % NQ]); }
+        cs.u += nsub; cs.o += 2;
+        if (cs.u < nunits) enter(cs);
+      }
+      if (cs.u >= nunits) return;
+      const int q = cs.q, o = cs.o + q, Tq = q == 0 ? cs.T0 : cs.T1;
+      if (q == 0) { wait(&bars.k_full[sk], phk); tc::fence_after_sync(); }
+      if (cs.t == 0) { wait(&bars.q_full[o % NQ], (o / NQ) & 1); tc::fence_after_sync(); }
+      if (cs.t < Tq) {
+        const uint32_t c = tbase + (uint32_t)(cs.n % NB) * kKeys;
+        const uint64_t a = tc::desc_step(dq, (o % NQ) * kTile), b = tc::desc_step(dk, (uint32_t)sk * kTile);
+#pragma unroll
+        for (int ks = 0; ks < D / 16; ++ks)
+          tc::mma_bf16_ss_warp(c, tc::desc_step(a, (ks / 4) * 128 * 128 + (ks % 4) * 32), tc::desc_step(b, (ks / 4) * 128 * 128 + (ks % 4) * 32),
+                               id_s, ks > 0);
+        tc::mma_commit_warp(&bars.s_full[q][(q == 0 ? cs.e0++ : cs.e1++) & 1]);
+      }
+      if (cs.t == max(Tq - 1, 0)) tc::mma_commit_warp(&bars.q_empty[o % NQ]);
+      ++cs.n;
+      if (q == 1) { tc::mma_commit_warp(&bars.k_empty[sk]); if (++sk == NS) { sk = 0; phk ^= 1; } ++cs.t; }
+      cs.q ^= 1;
+    };
+    for (int n = 0; n < NB; ++n) issue_s();
+    for (;;) {
+      while (cp.u < nunits && cp.t >= cp.T) { cp.u += nsub; if (cp.u < nunits) enter(cp); }
+      if (cp.u >= nunits) break;
+      const int q = cp.q;
+      if (q == 0) { wait(&bars.v_full[sv], phv); tc::fence_after_sync(); }
+      if (cp.t < (q == 0 ? cp.T0 : cp.T1)) {
+        const int e = q == 0 ? cp.e0++ : cp.e1++;
+        wait(&bars.p_ready[q][e & 1], (e >> 1) & 1);
+        tc::fence_after_sync();
+        const uint64_t b = tc::desc_step(dv, (uint32_t)sv * kTile);
+        const uint32_t c = tbase + (uint32_t)(cp.n % NB) * kKeys;
+#pragma unroll
+        for (int ks = 0; ks < kKeys / 16; ++ks)
+          tc::mma_bf16_ts_warp(tbase + cO + q * D, c + 8 * ks, tc::desc_step(b, ks * 16 * 128), id_o, cp.t > 0 || ks > 0);
+        tc::mma_commit_warp(&bars.pv_done[q]);
+      }
+      issue_s();
+      ++cp.n;
+      if (q == 1) { tc::mma_commit_warp(&bars.v_empty[sv]); if (++sv == NS) { sv = 0; phv ^= 1; } ++cp.t; }
+      cp.q ^= 1;
+    }
+  } else {                                                 // ---- softmax: thread = pair row, or (pair row, half of the tile's keys)
+    constexpr int W = kKeys / H, OD = D / H;               // logits and output dims of a thread
+    const int q = warp / (4 * H), half = H == 2 ? (warp >> 2) & 1 : 0, row = tid & 127;
+    const uint32_t tl = tbase + ((uint32_t)((warp & 3) * 32) << 16), to = tl + cO + q * D + half * OD;
+    const float scale2 = dm.sigma * 1.4426950408889634f;
+    constexpr float kLazy = 8.f;                           // see the local forward kernel
+    int e = 0, n0 = q;                                     // products of this pair tile so far; number of the unit's first
+    struct Ids { int pid, first, l0, l1; };
+    auto ld_ids = [&](int u) {                             // one unit ahead: no global-memory latency at the top of a unit
+      const int t0 = (2 * u + q) * kPairs;
+      return Ids{ld_pid(t0 + row), ld_pid(t0), ld_last(2 * u), ld_last(2 * u + 1)};
+    };
+    Ids nx = ld_ids(sub);
+    for (int u = sub; u < nunits; u += nsub) {
+      const Ids id = nx;
+      nx = ld_ids(u + nsub);
+      const int T0 = key_tiles(id.l0), T1 = key_tiles(id.l1), Tq = q == 0 ? T0 : T1;
+      const int nk = visible(id.pid);                      // keys this row sees: a prefix of the cluster's
+      const int nfull = (2 * u + q) * kPairs + kPairs <= np ? visible(id.first) : 0;     // ... and every row of the tile
+      float m2 = -INFINITY, l = 0.f;
+      for (int t = 0; t < Tq; ++t, ++e) {
+        wait(&bars.s_full[q][e & 1], (e >> 1) & 1);
+        tc::fence_after_sync();
+        const uint32_t ts = tl + (uint32_t)((n0 + 2 * t) % NB) * kKeys;
+        float s[W / 16][16];
+#pragma unroll
+        for (int g = 0; g < W / 16; ++g) tc::tmem_ld16_issue(ts + W * half + 16 * g, s[g]);
+        tc::tmem_ld_wait();
+#pragma unroll
+        for (int g = 0; g < W / 16; ++g) tc::tmem_ld_use16(s[g]);
+        if (nfull < (t + 1) * kKeys) {
+          const int lim = nk - t * kKeys - W * half;
+#pragma unroll
+          for (int g = 0; g < W / 16; ++g)
+#pragma unroll
+            for (int i = 0; i < 16; ++i) s[g][i] = 16 * g + i < lim ? s[g][i] : -INFINITY;
+        }
+        float mx[4];
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+          mx[g] = s[g][0];
+#pragma unroll
+          for (int k = g; k < W / 16; k += 4)
+#pragma unroll
+            for (int i = 0; i < 16; ++i) mx[g] = fmaxf(mx[g], s[k][i]);
+        }
+        const float mt = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * scale2;
+        // (also: both halves have read their logits before either writes P over them)
+        const bool grow = t == 0 || mt > m2 + kLazy;
+        if (H == 2 ? bar_or(1 + q, kSoft / 2, grow) : __any_sync(0xffffffffu, grow)) {
+          float mr = mt;
+          if (H == 2) {
+            mx_s[q][half][row] = mt;
+            tc::named_bar_sync(1 + q, kSoft / 2);
+            mr = fmaxf(mt, mx_s[q][half ^ 1][row]);
+          }
+          const float mn = mr > m2 + kLazy ? mr : m2;      // rows that did not grow keep their base; -inf: a row that sees no key
+          if (t > 0) {
+            wait(&bars.pv_done[q], (e - 1) & 1);           // (complete ever since: the wait below returns at once)
+            tc::fence_after_sync();
+            const float resc = mn == -INFINITY ? 1.f : tc::fast_exp2(m2 - mn);
+#pragma unroll
+            for (int d0 = 0; d0 < OD; d0 += 32) {
+              float v[32];
+              tc::tmem_ld32(to + d0, v);
+#pragma unroll
+              for (int i = 0; i < 32; ++i) v[i] *= resc;
+              tc::tmem_st32(to + d0, v);
+            }
+            l *= resc;
+          }
+          m2 = mn;
+        }
+        const float base = m2 == -INFINITY ? 0.f : m2;
+        float rs[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int g = 0; g < W / 16; ++g) {
+          uint32_t pk2[8];
+#pragma unroll
+          for (int i = 0; i < 16; i += 2) {
+            __nv_bfloat162 e2 = __floats2bfloat162_rn(tc::fast_exp2(fmaf(s[g][i], scale2, -base)), tc::fast_exp2(fmaf(s[g][i + 1], scale2, -base)));
+            rs[(i / 2) & 3] += __low2float(e2) + __high2float(e2);            // the rounded values, as the P V product sees them
+            pk2[i / 2] = *reinterpret_cast<uint32_t*>(&e2);
+          }
+          tc::tmem_st8_issue(ts + W / 2 * half + 8 * g, pk2);
+        }
+        l += (rs[0] + rs[1]) + (rs[2] + rs[3]);
+        if (e > 0) wait(&bars.pv_done[q], (e - 1) & 1);    // every phase is waited for, before the next one can complete
+        tc::tmem_st_wait();
+        tc::fence_before_sync();
+        tc::mbar_arrive(&bars.p_ready[q][e & 1]);
+      }
+      n0 += 2 * max(T0, T1);
+      if (H == 2) {
+        tc::named_bar_sync(1 + q, kSoft / 2);
+        mx_s[q][half][row] = l;
+        tc::named_bar_sync(1 + q, kSoft / 2);
+        l += mx_s[q][half ^ 1][row];
+        tc::named_bar_sync(1 + q, kSoft / 2);              // mx_s is written again by the next unit
+      }
+      if (Tq > 0) {
+        wait(&bars.pv_done[q], (e - 1) & 1);
+        tc::fence_after_sync();
+      }
+      const bool live = ok_ && id.pid >= 0;
+      const float inv = l > 0.f ? 1.f / l : 0.f;
+      bf16* orow = o_part + (pbase + max(id.pid, 0)) * D + half * OD;
+#pragma unroll
+      for (int d0 = 0; d0 < OD; d0 += 32) {
+        float v[32];
+        if (Tq > 0) tc::tmem_ld32(to + d0, v);
+        else {
+#pragma unroll
+          for (int i = 0; i < 32; ++i) v[i] = 0.f;
+        }
+        if (live) {
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {                    // 16 columns = 32 bytes per store
+            uint32_t w[8];
+#pragma unroll
+            for (int x = 0; x < 8; ++x) {
+              __nv_bfloat162 b2 = __floats2bfloat162_rn(v[16 * c + 2 * x] * inv, v[16 * c + 2 * x + 1] * inv);
+              w[x] = *reinterpret_cast<uint32_t*>(&b2);
+            }
+            tc::st_global_32B(orow + d0 + 16 * c, w);
+          }
+        }
+      }
+      if (live && half == 0) l_part[pbase + id.pid] = l > 0.f ? (m2 + log2f(l)) * 0.6931471805599453f : -INFINITY;
+    }
+  }
+  if (!ok_ && lane == 0) report_status(status, MUSE_STATUS_FWD_TIMEOUT);
+  tc::fence_before_sync();
+  __syncthreads();
+  if (warp == MW) tc::tmem_dealloc(tbase, 512);
+}
+
+template <int D>
+static int ret_fwd_long_d(const Dims& d, const void* Q, const void* Kp, const void* Vp, const int32_t* off_k, const int32_t* goff, const int32_t* pairs,
+                          void* o_part, float* l_part, int* status, cudaStream_t st) {
+  CUtensorMap k, v;
+  MUSE_RC(make_tmap_bf16_rows(&k, Kp, (uint64_t)d.B * d.Hkv * d.N, D, rl::kKeys));
+  MUSE_RC(make_tmap_bf16_rows(&v, Vp, (uint64_t)d.B * d.Hkv * d.N, D, rl::kKeys));
+  MUSE_CUDA_OK(cudaFuncSetAttribute(k_ret_fwd_long<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, rl::Lay<D>::total));
+  prof_mark("k_ret_fwd_pairs_tc", st);
+  k_ret_fwd_long<D><<<dim3(d.Ck, rl::kSplit, d.B * d.Hq), rl::Lay<D>::kThreads, rl::Lay<D>::total, st>>>(d, k, v, (const bf16*)Q, off_k, goff, pairs,
+                                                                                                  (bf16*)o_part, l_part, status);
+  MUSE_LAUNCH_OK();
+  return MUSE_OK;
+}
+
+int ret_fwd_long_tc(const Dims& d, const void* Q, const void* Kp, const void* Vp, const int32_t* off_k, const int32_t* goff,
+                    const int32_t* pairs, void* o_part, float* l_part, int* status, cudaStream_t st) {
+  return d.D == 128 ? ret_fwd_long_d<128>(d, Q, Kp, Vp, off_k, goff, pairs, o_part, l_part, status, st)
+                    : ret_fwd_long_d<64>(d, Q, Kp, Vp, off_k, goff, pairs, o_part, l_part, status, st);
+}
+
+}  // namespace muse

@@ -370,8 +370,18 @@ k_ret_fwd_pairs_tc(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__
   if (!ok_ && lane == 0) report_status(status, MUSE_STATUS_FWD_TIMEOUT);
 }
 
+int ret_fwd_long_tc(const Dims& d, const void* Q, const void* Kp, const void* Vp, const int32_t* off_k, const int32_t* goff,
+                    const int32_t* pairs, void* o_part, float* l_part, int* status, cudaStream_t st);
+
+// The kernel here keeps 128 keys resident and two CTAs on an SM, but a cluster of more keys takes sweeps that gather the rows again and
+// read back the stored ones; the other streams the keys, and a tile of few keys pays for its longer pipeline.  Measured,
+// resident | streamed, us:
+//   D = 64:   64 keys 258 | 403,  128 keys 249 | 260 (sharp selections 219 | 275),  256 keys 727 | 544,  512 keys 7320 | 4470
+//   D = 128:  64 keys 408 | 506,  128 keys 366 | 319,  256 keys 993 | 665
 int ret_fwd_pairs_tc(const Dims& d, const void* Q, const void* Kp, const void* Vp, const int32_t* off_k, const int32_t* goff,
                      const int32_t* pairs, void* o_part, float* l_part, int* status, cudaStream_t st) {
+  if (d.k2 == 0 && d.N / d.Ck >= (d.D == 128 ? 128 : 256))             // mean keys of a cluster
+    return ret_fwd_long_tc(d, Q, Kp, Vp, off_k, goff, pairs, o_part, l_part, status, st);
   const dim3 grid(d.k2 > 0 ? d.Ck * d.SB : d.Ck, rf::kSplit, d.B * d.Hq);     // one CTA (or a few) per key cluster, or per bucket
   prof_mark("k_ret_fwd_pairs_tc", st);
   if (d.D == 128) {

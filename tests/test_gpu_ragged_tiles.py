@@ -52,8 +52,9 @@ def test_streaming_both_sides_at_once_equals_each_side_alone(Hq, Hkv, D, Cq, Ck,
 
 @pytest.mark.parametrize("base,Ck,two_kernels", [("d64", 7, True), ("d64", 8, False), ("d64", 2, True), ("d128", 15, True), ("d128", 16, False),
                                                  ("d128", 3, True)])
-def test_retrieval_backward_on_both_sides_of_the_cluster_length_rule(base, Ck, two_kernels):
-    """2040 keys: clusters of 255 (D = 64) or 127 keys (D = 128) and shorter take the fused kernel."""
+def test_retrieval_on_both_sides_of_the_cluster_length_rule(base, Ck, two_kernels):
+    """2040 keys: clusters of 255 (D = 64) or 127 keys (D = 128) and shorter take the fused kernel (and, before it, the forward
+    kernel with resident keys)."""
     w = CASES[base].with_(Hq=2, Hkv=1, N=2040, S=4, Cq=9, Ck=Ck, m=min(Ck, 3), components=64)
     with kernels_launched() as rec:
         _backward_parity_run(w, 128.0)
