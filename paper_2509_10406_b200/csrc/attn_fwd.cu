@@ -25,117 +25,6 @@ int block_select(const Dims& d, int dtype, const void* Q, const int32_t* off_q, 
 __device__ __forceinline__ int query_plane(const Dims& d, int t) { return d.causal ? t / d.Bs - 1 : 0; }
 
 // ---------------------------------------------------------------------------------------------
-// Inverse index for retrieval (Section "Exact Retrieval and Local Attention"): for every
-// (key cluster, plane) the list of (query, slot) pairs that retrieve it.  Group key = cluster * SB + plane,
-// so that the pairs of one cluster over all planes form one run, ordered by plane.
-// ---------------------------------------------------------------------------------------------
-// Thread e handles (slot = e / N, query = e % N): the lanes of a warp are consecutive queries,
-// which often retrieve the same cluster in the same slot, so equal keys are combined with a warp
-// match and only one atomic per distinct key and warp reaches memory.
-// With spatial block selection (bsel != nullptr, k2 > 0) a pair is (query, slot, chosen block e2), its group the
-// BUCKET (cluster, chosen block) and its id (query * m + slot) * k2 + e2: the retrieval kernel then keeps one bucket
-// resident and every pair of the group sees all of it.
-__device__ __forceinline__ void ret_pair_key(const Dims& d, const int32_t* sel, const int32_t* bsel, int pq, long long e, int e2,
-                                             int& key, int& pid) {
-  key = -1; pid = 0;
-  if (e >= (long long)d.N * d.m) return;
-  const int t = (int)(e % d.N), k = (int)(e / d.N);
-  const size_t slot = ((size_t)pq * d.N + t) * d.m + k;
-  const int c = sel[slot];
-  const int pl = query_plane(d, t);
-  if (c < 0 || c >= d.Ck || pl < 0) return;                // entries outside [0, Ck) count as "none"
-  if (bsel == nullptr) { key = c * d.SB + pl; pid = t * d.m + k; return; }
-  const int bb = bsel[slot * d.k2 + e2];
-  if (bb < 0 || bb > pl) return;                           // (block bb is earlier than the query's block pl + 1)
-  key = c * d.SB + bb; pid = (t * d.m + k) * d.k2 + e2;
-}
-
-__global__ void k_ret_count(Dims d, const int32_t* __restrict__ sel, const int32_t* __restrict__ bsel, int32_t* __restrict__ cnt) {
-  const int pq = blockIdx.y;
-  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const int lane = threadIdx.x & 31;
-  for (int e2 = 0; e2 < (bsel ? d.k2 : 1); ++e2) {
-    int key, pid;
-    ret_pair_key(d, sel, bsel, pq, e, e2, key, pid);
-    const unsigned peers = __match_any_sync(0xffffffffu, key);
-    if (key >= 0 && lane == __ffs(peers) - 1) atomicAdd(&cnt[(size_t)pq * d.SB * d.Ck + key], __popc(peers));
-  }
-}
-
-__global__ void k_ret_fill(Dims d, const int32_t* __restrict__ sel, const int32_t* __restrict__ bsel, int32_t* __restrict__ cursor,
-                           int32_t* __restrict__ pairs) {
-  const int pq = blockIdx.y;
-  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const int lane = threadIdx.x & 31;
-  const size_t npairs = (size_t)d.N * d.m * (bsel ? d.k2 : 1);
-  for (int e2 = 0; e2 < (bsel ? d.k2 : 1); ++e2) {
-    int key, pid;
-    ret_pair_key(d, sel, bsel, pq, e, e2, key, pid);
-    const unsigned peers = __match_any_sync(0xffffffffu, key);
-    const int leader = __ffs(peers) - 1;
-    int base = 0;
-    if (key >= 0 && lane == leader) base = atomicAdd(&cursor[(size_t)pq * d.SB * d.Ck + key], __popc(peers));
-    base = __shfl_sync(0xffffffffu, base, leader);
-    if (key >= 0 && MUSE_IN_RANGE(base + __popc(peers & ((1u << lane) - 1u)), npairs))
-      pairs[(size_t)pq * npairs + base + __popc(peers & ((1u << lane) - 1u))] = pid;
-  }
-}
-
-// Exclusive scan of a head's counts; off[key] = start of the key's run.
-__global__ void __launch_bounds__(1024)
-k_ret_scan(int32_t* __restrict__ cnt, int nkeys, int32_t* __restrict__ off) {
-  __shared__ int32_t wsum[32];
-  const int prob = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  int32_t* c = cnt + (size_t)prob * nkeys;
-  int32_t* o = off + (size_t)prob * (nkeys + 1);
-  int carry = 0;
-  for (int e0 = 0; e0 < nkeys; e0 += 1024) {
-    const int e = e0 + tid, v = e < nkeys ? c[e] : 0;
-    int inc = v;
-#pragma unroll
-    for (int s = 1; s < 32; s <<= 1) { const int x = __shfl_up_sync(0xffffffffu, inc, s); if (lane >= s) inc += x; }
-    if (lane == 31) wsum[warp] = inc;
-    __syncthreads();
-    int base = carry, all = 0;
-    for (int w = 0; w < 32; ++w) { const int x = wsum[w]; if (w < warp) base += x; all += x; }
-    if (e < nkeys) { c[e] = base + inc - v; o[e] = base + inc - v; }
-    carry += all;
-    __syncthreads();
-  }
-  if (tid == 0) o[nkeys] = carry;
-}
-
-size_t ret_index_elems(const Dims& d) {
-  // cursor [SB*Ck] + goff [SB*Ck+1] + pairs [N*m*max(k2,1)], each rounded up to 64 ints
-  auto up = [](size_t x) { return (x + 63) & ~size_t(63); };
-  return up((size_t)d.SB * d.Ck) + up((size_t)d.SB * d.Ck + 1) + up((size_t)d.N * d.m * (d.k2 > 0 ? d.k2 : 1));
-}
-
-int build_ret_index(const Dims& d, const int32_t* sel, const int32_t* bsel, int32_t* scratch, RetIndex* out, cudaStream_t st) {
-  auto up = [](size_t x) { return (x + 63) & ~size_t(63); };
-  const int pq = d.B * d.Hq, nkeys = d.SB * d.Ck;
-  out->cursor = scratch;
-  out->goff = scratch + (size_t)pq * up(nkeys);
-  out->pairs = out->goff + (size_t)pq * up((size_t)nkeys + 1);
-  // note: cursor / goff are indexed with their natural strides (nkeys, nkeys + 1); the padded
-  // region sizes above only reserve space
-  if (d.m == 0 || nkeys == 0) return MUSE_OK;
-  prof_mark("memset", st);
-  MUSE_CUDA_OK(cudaMemsetAsync(out->cursor, 0, (size_t)pq * nkeys * sizeof(int32_t), st));
-  dim3 grid(cdiv((long long)d.N * d.m > 0 ? d.N * d.m : 1, 256), pq);
-  prof_mark("k_ret_count", st);
-  k_ret_count<<<grid, 256, 0, st>>>(d, sel, bsel, out->cursor);
-  MUSE_LAUNCH_OK();
-  prof_mark("k_ret_scan", st);
-  k_ret_scan<<<pq, 1024, 0, st>>>(out->cursor, nkeys, out->goff);
-  MUSE_LAUNCH_OK();
-  prof_mark("k_ret_fill", st);
-  k_ret_fill<<<grid, 256, 0, st>>>(d, sel, bsel, out->cursor, out->pairs);
-  MUSE_LAUNCH_OK();
-  return MUSE_OK;
-}
-
-// ---------------------------------------------------------------------------------------------
 // Far field: scores against all accumulated cluster summaries, top-m, approximate attention
 // over the rest.  One CTA per (query cluster i, plane, head) segment.
 // ---------------------------------------------------------------------------------------------
