@@ -153,6 +153,7 @@ void prof_mark(const char* name, cudaStream_t st);
 // MUSE_STATUS_* code a kernel reported (0 = none); the entry points clear the words once per call.
 // Words from 8 up carry diagnostics of instrumented builds only.
 constexpr int kStatusWords = 64;
+constexpr int kItemWord = 4;               // work counter of the persistent summary kernel (zeroed by the kernel before it)
 __device__ __forceinline__ void report_status(int* status, int code) { atomicCAS(status, 0, code); }
 
 // Bounds-checked build (compiled with -DMUSE_DEBUG into a second library): every index that a kernel derives from data
@@ -232,7 +233,7 @@ size_t summarize_ws_bytes(const Dims& d, int dtype);
 
 // sigma * qbar as two bf16 planes (hi + lo keeps ~16 mantissa bits), [B*Hq*Cq][D] each: the tensor-core
 // summary kernels load their centroid tiles from these by TMA instead of converting them per CTA
-int split_qbar(const Dims& d, const float* qbar, void* qhi, void* qlo, cudaStream_t st);
+int split_qbar(const Dims& d, const float* qbar, void* qhi, void* qlo, int* dealt, cudaStream_t st);   // dealt: zeroed, if given
 
 
 // Byte offsets inside the caller's summaries buffer.  Per entry (b, h, plane, i, j):

@@ -1,15 +1,20 @@
-// Accumulated tilted summaries on the tensor cores (bf16 mode, D = 128): Eq. 3-5 and the
-// exclusive causal accumulation of Algorithm 1 in one online-softmax walk over the buckets of a
-// key cluster.  One CTA = (key cluster j, 128 query clusters, head), 256 threads: thread
-// (row i, warpgroup w) keeps the running max / mass of centroid i and 128 fp32 accumulators:
-// dims [64 w, 64 w + 64) of kappa and of nu.
-//   L   = sigma qbar K^T        tcgen05, qbar as bf16 hi + lo, keys TMA-loaded 64 at a time
-//   w_u = exp(l_u - running max)  per thread, written as a bf16 hi + lo operand pair
-//   U   = W [K | V]             tcgen05 (keys contracted), folded into the accumulators with the
-//                               online-softmax rescale
-// After each bucket the normalised snapshot (mu, beta, kappa hi/lo, nu) of plane = bucket index
-// is staged in shared memory as three swizzled tiles that leave by TMA stores while the next
-// plane is being computed.
+// Accumulated tilted summaries on the tensor cores (bf16 mode, D = 64 or 128): Eq. 3-5 and the exclusive causal
+// accumulation of Algorithm 1 in one online-softmax walk over the buckets of a key cluster.  An item is (key cluster j, 128
+// query clusters, head); a CTA walks the planes of a contiguous range of items, so that the rows it writes and its logits'
+// query operand stay close.  A bucket comes in steps of at most 64 keys:
+//   L   = sigma qbar K^T        query clusters as bf16 hi + lo; keys and values of a step by TMA through a ring
+//   w_u = exp(l_u - base)       thread = query cluster; bf16 hi + lo over the consumed logits in tensor memory, A operands of
+//   U  += W [K | V]             accumulated in tensor memory over the whole cluster; rescaled only when a logit exceeds the
+//                               base by more than kLazy
+// and after a bucket the normalised snapshot (mu, beta, kappa hi / lo, nu) of its plane goes from tensor memory to global
+// memory.  Four roles run this as a pipeline over all steps of all items: one warp loads, one issues products (the logits
+// of a step before the sums of the one before it), four warps make weights, sixteen write snapshots; a snapshot's writers
+// give the accumulators back as soon as they hold them in registers.
+//
+// Bound by the snapshot writes, 6 D bytes per (query cluster, key cluster, plane), at D = 128 (3.5 TB/s; a memset reaches 4),
+// and at D = 64 by the weights of one step after the other.  Against one CTA per item with every phase behind a CTA barrier,
+// accumulators in registers and snapshots staged for TMA: 64k tokens, 128 x 128 clusters, D = 64, 32 heads 1499 -> 639 us;
+// 8k tokens, 64 x 128, 16 heads 304 -> 159; 64k, 256 x 1024, D = 128, 4 heads 1696 -> 1592; 128k, 512 x 2048 6.52 -> 6.28 ms.
 #include <cuda.h>
 #include "common.cuh"
 #include "tc05.cuh"
@@ -18,23 +23,25 @@ namespace muse {
 
 typedef __nv_bfloat16 bf16;
 int make_tmap_bf16_rows(void* out_map, const void* base, uint64_t rows, uint32_t cols, uint32_t box_rows);
-int make_tmap_bf16_nd(void* out_map, const void* base, int rank, const uint64_t* dims, const uint64_t* strides_bytes,
-                      const uint32_t* box);
 
 namespace st {
-constexpr int TI = 128, NU = 64, THREADS = 256;
-template <int D> struct Lay {                     // shared-memory offsets and TMEM columns for head dimension D (64 or 128)
-  static constexpr int G = D / 64;                // 64-element (128-byte) column groups of a row
-  static constexpr int kTile = TI * D * 2, kKeys = NU * D * 2, kW = TI * NU * 2;
-  static constexpr int oQhi = 0, oQlo = oQhi + kTile, oK = oQlo + kTile, oV = oK + kKeys, oWhi = oV + kKeys, oWlo = oWhi + kW;
-  static constexpr int oStage = oWlo + kW;        // three snapshot tiles (kappa hi, kappa lo, nu) leaving by TMA
-  static constexpr int total = oStage + 3 * kTile + 1024;
-  static constexpr uint32_t cL = 0, cUk = 64, cUv = 64 + D;
+constexpr int TI = 128, NU = 64, NS = 4;                   // query clusters of an item; keys of a step; steps in the ring
+constexpr int kSnapWarps = 16, kWeightWarp0 = 16, kMmaWarp = 20, kLoadWarp = 21, kDealWarp = 22, kThreads = 23 * 32;
+constexpr int kRing = 2, kTakers = kSnapWarps + 6;           // item ranges handed out ahead; warps that take each of them
+constexpr float kLazy = 8.f, kNever = -1e30f, kLog2e = 1.4426950408889634f;
+template <int D> struct Lay {                              // shared-memory offsets and TMEM columns for head dimension D
+  static constexpr int G = D / 64;                         // 64-element (128-byte) column groups of a row
+  static constexpr int NG = 128 / D;                       // groups of snapshot warps that take planes in turn (2 or 4 threads per row)
+  static constexpr int kTile = TI * D * 2, kKeys = NU * D * 2;
+  static constexpr int oQhi = 0, oQlo = kTile, oKV = 2 * kTile, total = oKV + NS * 2 * kKeys + 1024;
+  static constexpr uint32_t cUk = 0, cUv = D, cL = 2 * D, cLo = 2 * D + 2 * NU, cols = 512;
 };
+struct Bars { uint64_t q_full, q_free, kv_full[NS], kv_empty[NS], l_full[2], w_ready, u_step, u_done[2], acc_free[2], item_full[kRing], item_free[kRing]; };
 }  // namespace st
 
-__global__ void k_split_qbar(const float* __restrict__ qbar, long long n, float sigma, bf16* __restrict__ hi, bf16* __restrict__ lo) {
+__global__ void k_split_qbar(const float* __restrict__ qbar, long long n, float sigma, bf16* __restrict__ hi, bf16* __restrict__ lo, int* dealt) {
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e == 0 && dealt != nullptr) *dealt = 0;              // the item counter of the kernel that follows
   if (e >= n) return;
   const float x = qbar[e] * sigma;
   const bf16 h = __float2bfloat16_rn(x);
@@ -42,238 +49,340 @@ __global__ void k_split_qbar(const float* __restrict__ qbar, long long n, float 
   lo[e] = __float2bfloat16_rn(x - __bfloat162float(h));
 }
 
-int split_qbar(const Dims& d, const float* qbar, void* qhi, void* qlo, cudaStream_t st) {
+int split_qbar(const Dims& d, const float* qbar, void* qhi, void* qlo, int* dealt, cudaStream_t st) {
   const long long n = (long long)d.B * d.Hq * d.Cq * d.D;
   prof_mark("k_split_qbar", st);
-  k_split_qbar<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(qbar, n, d.sigma, (bf16*)qhi, (bf16*)qlo);
+  k_split_qbar<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(qbar, n, d.sigma, (bf16*)qhi, (bf16*)qlo, dealt);
   MUSE_LAUNCH_OK();
   return MUSE_OK;
 }
 
 template <int D>
-__global__ void __launch_bounds__(st::THREADS, 1)
+__global__ void __launch_bounds__(st::kThreads, 1)
 k_summarize_tc(Dims dm, const __grid_constant__ CUtensorMap tm_K, const __grid_constant__ CUtensorMap tm_V,
-               const __grid_constant__ CUtensorMap tm_okhi, const __grid_constant__ CUtensorMap tm_oklo,
-               const __grid_constant__ CUtensorMap tm_onu, const __grid_constant__ CUtensorMap tm_qhi,
-               const __grid_constant__ CUtensorMap tm_qlo, const int32_t* __restrict__ off_k, SummPtrs sp, int per_block,
-               int* __restrict__ status) {
-  using namespace st;
+               const __grid_constant__ CUtensorMap tm_qhi, const __grid_constant__ CUtensorMap tm_qlo, const int32_t* __restrict__ off_k,
+               SummPtrs sp, int per_block, int per, int* __restrict__ dealt, int* __restrict__ status) {
+  using namespace st;   // per: items of a CTA, or 1: they are dealt out one by one; dealt: those dealt so far
   typedef Lay<D> LY;
-  constexpr int G = LY::G, HD = D / 2, kTile = LY::kTile;
-  constexpr int oQhi = LY::oQhi, oQlo = LY::oQlo, oK = LY::oK, oV = LY::oV, oWhi = LY::oWhi, oWlo = LY::oWlo, oStage = LY::oStage;
-  constexpr uint32_t cL = LY::cL, cUk = LY::cUk, cUv = LY::cUv;
+  constexpr int G = LY::G, NG = LY::NG, kKeys = LY::kKeys;
   extern __shared__ __align__(1024) unsigned char sm_raw[];
-  __shared__ uint64_t bar_kv, bar_q, bar1, bar2;
+  __shared__ Bars bars;
   __shared__ uint32_t tbase_s;
-  const int j = blockIdx.x, i0 = blockIdx.y * TI, pq = blockIdx.z;
-  const int b_ = pq / dm.Hq, h = pq % dm.Hq, pk = b_ * dm.Hkv + dm.hm.g[h];
-  const int tid = threadIdx.x, warp = tc::warp_index(), wg = tid >> 7, row = tid & 127, i = i0 + row;
+  __shared__ int item_s[kRing];
+  __shared__ float base_s[4][TI], s_s[4][TI], T_s[4][TI];  // of the last snapshots: base (log2), mass and sum of w * logit (log2), relative to the base
+  const int tid = threadIdx.x, warp = tc::warp_index(), lane = tid & 31;
   unsigned char* sm = sm_raw + ((1024u - (tc::smem_u32(sm_raw) & 1023u)) & 1023u);
-  const int32_t* off = off_k + (size_t)pk * (dm.Ck * dm.S + 1) + (size_t)j * dm.S;
-  if (warp == 0) tc::tmem_alloc(&tbase_s, 512);
-  if (tid == 0) { tc::mbar_init(&bar_kv, 1); tc::mbar_init(&bar_q, 1); tc::mbar_init(&bar1, 1); tc::mbar_init(&bar2, 1); tc::mbar_init_fence(); }
+  if (warp == kMmaWarp) tc::tmem_alloc(&tbase_s, LY::cols);
+  if (tid == 0) {
+    for (int r = 0; r < kRing; ++r) { tc::mbar_init(&bars.item_full[r], 1); tc::mbar_init(&bars.item_free[r], kTakers); }
+    tc::mbar_init(&bars.q_full, 1); tc::mbar_init(&bars.q_free, 1); tc::mbar_init(&bars.w_ready, TI); tc::mbar_init(&bars.u_step, 1);
+    for (int s = 0; s < NS; ++s) { tc::mbar_init(&bars.kv_full[s], 1); tc::mbar_init(&bars.kv_empty[s], 1); }
+    for (int g = 0; g < 2; ++g) { tc::mbar_init(&bars.l_full[g], 1); tc::mbar_init(&bars.u_done[g], 1); tc::mbar_init(&bars.acc_free[g], kSnapWarps * 32 / NG); }
+    tc::mbar_init_fence();
+  }
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
-  // sigma * qbar tile as bf16 hi and lo operands, split once per layer and loaded here by TMA
-  if (warp == 0) {
-    tc::mbar_expect_tx_warp(&bar_q, 2 * kTile);
-    const int r = pq * dm.Cq + i0;
-    for (int g = 0; g < G; ++g) {
-      tc::tma_load_2d_warp(sm + oQhi + g * TI * 128, &tm_qhi, 64 * g, r, &bar_q);
-      tc::tma_load_2d_warp(sm + oQlo + g * TI * 128, &tm_qlo, 64 * g, r, &bar_q);
-    }
-  }
-  const uint32_t tbase = tbase_s, tlane = tbase + ((uint32_t)((warp & 3) * 32) << 16);
-  const uint32_t aQhi = tc::smem_u32(sm + oQhi), aQlo = tc::smem_u32(sm + oQlo), aK = tc::smem_u32(sm + oK),
-                 aV = tc::smem_u32(sm + oV), aWhi = tc::smem_u32(sm + oWhi), aWlo = tc::smem_u32(sm + oWlo);
-  uint32_t ph_kv = 0, ph1 = 0, ph2 = 0;
-  bool ok = true, q_ready = false;
-  float acc[D];
-#pragma unroll
-  for (int d = 0; d < D; ++d) acc[d] = 0.f;
-  float M = -INFINITY, s = 0.f, T = 0.f;           // running max, mass and sum of w * logit (all relative to M)
-#ifdef MUSE_PHASE_CLOCKS
-  long long pc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  long long t_ = clock64();
-#define PCLK(k) { long long n_ = clock64(); pc[k] += n_ - t_; t_ = n_; }
-#else
-#define PCLK(k)
-#endif
+  const uint32_t tbase = tbase_s;
+  const int NI = (dm.Cq + TI - 1) / TI, items = NI * dm.Ck * dm.B * dm.Hq;             // (head, tile of query clusters, key cluster), in this order
+  bool ok = true;                                          // false once a bounded wait ran out (every role then runs off the end of its items)
+  auto wait = [&](uint64_t* bar, uint32_t parity) { if (ok && !tc::mbar_wait(bar, parity)) ok = false; };
+  // one plane of one item: its key cluster, tile, head, and its bucket's keys [p0, p1); taken: ranges of items so far
+  struct Plane { int it, end, taken, pl, j, i0, pq, pk, p0, p1; };
+  auto take = [&](Plane& P) {                              // the next item
+    if (++P.it < P.end) return;
+    const int r = P.taken % kRing;
+    wait(&bars.item_full[r], (P.taken / kRing) & 1);
+    P.it = ok ? item_s[r] : items;
+    P.end = min(P.it + per, items);
+    ++P.taken;
+    __syncwarp();
+    if (lane == 0) tc::mbar_arrive(&bars.item_free[r]);
+  };
+  auto place = [&](Plane& P) {
+    P.pl = 0;
+    P.j = P.it % dm.Ck;
+    P.i0 = P.it / dm.Ck % NI * TI;
+    P.pq = P.it / dm.Ck / NI;
+    P.pk = P.pq / dm.Hq * dm.Hkv + dm.hm.g[P.pq % dm.Hq];
+  };
+  auto advance = [&](Plane& P) {                           // the next plane (fetched one ahead of its use)
+    if (++P.pl == dm.SB) { take(P); if (P.it < items) place(P); }
+    if (P.it >= items) return;
+    const int32_t* off = off_k + (size_t)P.pk * (dm.Ck * dm.S + 1) + (size_t)P.j * dm.S + P.pl;
+    P.p0 = __ldg(off);
+    P.p1 = __ldg(off + 1);
+    (void)MUSE_IN_RANGE(P.p1, dm.N + 1); (void)MUSE_IN_RANGE(P.p0, P.p1 + 1);          // (the tiles come through tensor maps, which clip)
+  };
+  struct Walk { Plane cur, nxt; };
+  auto start = [&](Walk& w) {
+    w.cur = Plane{-1, 0, 0, dm.SB - 1, 0, 0, 0, 0, 0, 0};
+    advance(w.cur);
+    w.nxt = w.cur;
+    if (w.nxt.it < items) advance(w.nxt);
+  };
+  auto next = [&](Walk& w) { w.cur = w.nxt; if (w.nxt.it < items) advance(w.nxt); };
+  pdl_trigger();
+  pdl_wait();
 
-  // The cluster's keys are contiguous in bucket order, so its chunks (at most 64 keys, never across a
-  // bucket boundary) form one sequence; thread 32 starts the load of chunk n + 1 as soon as the MMAs of
-  // chunk n have released the key / value tiles, so that it lands while the snapshot is written.
-  // A bucket usually holds far fewer than 64 keys: only the 16-key groups in use are loaded and contracted.
-  auto issue_kv = [&](int c0, int nk) {
-    const int ng_ = (nk + 15) >> 4;
-    tc::mbar_expect_tx_warp(&bar_kv, ng_ * 2 * G * (16 * 128));
-    const int r = (int)((size_t)pk * dm.N + c0);
-    for (int g = 0; g < ng_; ++g)
-      for (int cg = 0; cg < G; ++cg) {
-        tc::tma_load_2d_warp(sm + oK + cg * NU * 128 + g * 16 * 128, &tm_K, 64 * cg, r + 16 * g, &bar_kv);
-        tc::tma_load_2d_warp(sm + oV + cg * NU * 128 + g * 16 * 128, &tm_V, 64 * cg, r + 16 * g, &bar_kv);
-      }
-  };
-  auto issue_after = [&](int c_end) {                  // the chunk that starts at key c_end, if any
-    int npl = 0;
-    while (npl < dm.SB && off[npl + 1] <= c_end) ++npl;
-    if (npl < dm.SB) issue_kv(c_end, min(NU, off[npl + 1] - c_end));
-  };
-  if (warp == 1) issue_after(off[0]);
-  for (int pl = 0; pl < dm.SB && ok; ++pl) {
-    const int p0 = off[pl], p1 = off[pl + 1];
-    (void)MUSE_IN_RANGE(p1, dm.N + 1); (void)MUSE_IN_RANGE(p0, p1 + 1);     // (the tiles come through tensor maps, which clip)
-    if (per_block) {                                     // the summary of block pl alone: the running state starts afresh
-      M = -INFINITY; s = 0.f; T = 0.f;
-#pragma unroll
-      for (int d = 0; d < D; ++d) acc[d] = 0.f;
+  if (warp == kDealWarp) {                                 // ---- hands out ranges of items
+    for (int n = 0, it = 0; it < items && ok; ++n) {       // (a short ring: what a CTA has taken no other can)
+      const int r = n % kRing;
+      if (lane == 0) it = per > 1 ? (n == 0 ? min((int)blockIdx.x * per, items) : items) : min(atomicAdd(dealt, 1), items);
+      it = __shfl_sync(0xffffffffu, it, 0);
+      wait(&bars.item_free[r], ((n / kRing) & 1) ^ 1);
+      if (lane == 0) { item_s[r] = it; tc::mbar_arrive(&bars.item_full[r]); }
     }
-    for (int c0 = p0; c0 < p1 && ok; c0 += NU) {
-      const int nk = min(NU, p1 - c0);
-      PCLK(0)
-      __syncthreads();
-      const int ng = (nk + 15) >> 4;
-      if (warp == 0) {
-        if (!q_ready) { if (!tc::mbar_wait(&bar_q, 0)) ok = false; q_ready = true; }
-        if (!tc::mbar_wait(&bar_kv, ph_kv)) ok = false;
-        tc::fence_after_sync();
-        const uint32_t idesc = tc::idesc_bf16(TI, 16 * ng, 0, 0);
-#pragma unroll
-        for (int ks = 0; ks < D / 16; ++ks)
-          tc::mma_bf16_ss_warp(tbase + cL, tc::smem_desc_sw128(aQhi + (ks / 4) * TI * 128 + (ks % 4) * 32, 16, 1024),
-                          tc::smem_desc_sw128(aK + (ks / 4) * NU * 128 + (ks % 4) * 32, 16, 1024), idesc, ks > 0);
-#pragma unroll
-        for (int ks = 0; ks < D / 16; ++ks)
-          tc::mma_bf16_ss_warp(tbase + cL, tc::smem_desc_sw128(aQlo + (ks / 4) * TI * 128 + (ks % 4) * 32, 16, 1024),
-                          tc::smem_desc_sw128(aK + (ks / 4) * NU * 128 + (ks % 4) * 32, 16, 1024), idesc, 1);
-        tc::mma_commit_warp(&bar1);
+  } else if (warp == kLoadWarp) {                          // ---- loads
+    Walk w;
+    start(w);
+    int n = 0, nq = 0, tile = -1;
+    for (; w.cur.it < items; next(w)) {
+      if (w.cur.pl == 0 && w.cur.it / dm.Ck != tile) {        // another tile of query clusters
+        tile = w.cur.it / dm.Ck;
+        if (nq > 0) wait(&bars.q_free, (nq - 1) & 1);
+        ++nq;
+        if (ok) {
+          tc::mbar_expect_tx_warp(&bars.q_full, 2 * LY::kTile);
+          const int r = w.cur.pq * dm.Cq + w.cur.i0;
+          for (int g = 0; g < G; ++g) {
+            tc::tma_load_2d_warp(sm + LY::oQhi + g * TI * 128, &tm_qhi, 64 * g, r, &bars.q_full);
+            tc::tma_load_2d_warp(sm + LY::oQlo + g * TI * 128, &tm_qlo, 64 * g, r, &bars.q_full);
+          }
+        }
       }
-      ph_kv ^= 1;
-      __syncwarp();
-      if (!tc::mbar_wait(&bar1, ph1)) ok = false;
-      ph1 ^= 1;
+      for (int c0 = w.cur.p0; c0 < w.cur.p1; c0 += NU, ++n) {
+        const int s = n % NS, ng = (min(NU, w.cur.p1 - c0) + 15) >> 4;   // a bucket often holds far fewer than 64 keys: only the 16-key groups in use
+        wait(&bars.kv_empty[s], ((n / NS) & 1) ^ 1);
+        if (!ok) continue;
+        tc::mbar_expect_tx_warp(&bars.kv_full[s], ng * 2 * G * (16 * 128));
+        const int r = w.cur.pk * dm.N + c0;
+        unsigned char* kv = sm + LY::oKV + s * 2 * kKeys;
+        for (int g = 0; g < ng; ++g)
+          for (int cg = 0; cg < G; ++cg) {
+            tc::tma_load_2d_warp(kv + cg * NU * 128 + g * 16 * 128, &tm_K, 64 * cg, r + 16 * g, &bars.kv_full[s]);
+            tc::tma_load_2d_warp(kv + kKeys + cg * NU * 128 + g * 16 * 128, &tm_V, 64 * cg, r + 16 * g, &bars.kv_full[s]);
+          }
+      }
+    }
+  } else if (warp == kMmaWarp) {                           // ---- products
+    const uint64_t dqh = tc::smem_desc_sw128(tc::smem_u32(sm + LY::oQhi), 16, 1024), dql = tc::smem_desc_sw128(tc::smem_u32(sm + LY::oQlo), 16, 1024),
+                   dk = tc::smem_desc_sw128(tc::smem_u32(sm + LY::oKV), 16, 1024), dn = tc::smem_desc_sw128(tc::smem_u32(sm + LY::oKV), NU * 128, 1024);
+    int el = 0, nq = 0, tile = -1;                         // non-empty steps whose logits have been issued, tiles so far
+    auto issue_l = [&](int it, int pl, int c, int p1) {    // the logits of the step that starts at key c of a bucket that ends at p1
+      if (pl == 0 && it / dm.Ck != tile) {
+        tile = it / dm.Ck;
+        if (nq > 0) tc::mma_commit_warp(&bars.q_free);
+        wait(&bars.q_full, nq & 1);
+        ++nq;
+      }
+      if (c >= p1) return;
+      const int s = el % NS, ng = (min(NU, p1 - c) + 15) >> 4;
+      wait(&bars.kv_full[s], (el / NS) & 1);
       tc::fence_after_sync();
-      PCLK(1)
-      // two sweeps over the logits in TMEM (max, then weights) keep the register footprint small
-      float cm = -INFINITY;
-      for (int g = 0; g < ng; ++g) {
-        float v[16];
-        tc::tmem_ld16(tlane + cL + 16 * g, v);
+      const uint32_t idesc = tc::idesc_bf16(TI, 16 * ng, 0, 0), tl = tbase + LY::cL + (el & 1) * NU;
+      const uint64_t k = tc::desc_step(dk, (uint32_t)s * 2 * kKeys);
 #pragma unroll
-        for (int u = 0; u < 16; ++u) if (16 * g + u < nk) cm = fmaxf(cm, v[u]);
-      }
-      const float Mn = fmaxf(M, cm);
-      const float sc = __expf(M - Mn);                 // 0 on the first keys (M = -inf)
-      float ws = 0.f, wl = 0.f;
-      for (int g = 0; g < ng; ++g) {
-        float v[16];
-        tc::tmem_ld16(tlane + cL + 16 * g, v);
-        uint32_t pk_[8];
+      for (int ks = 0; ks < D / 16; ++ks)
+        tc::mma_bf16_ss_warp(tl, tc::desc_step(dqh, (ks / 4) * TI * 128 + (ks % 4) * 32), tc::desc_step(k, (ks / 4) * NU * 128 + (ks % 4) * 32), idesc, ks > 0);
 #pragma unroll
-        for (int u = 0; u < 16; u += 2) {
-          const bool in0 = 16 * g + u < nk, in1 = 16 * g + u + 1 < nk;
-          const float w0 = in0 ? __expf(v[u] - Mn) : 0.f, w1 = in1 ? __expf(v[u + 1] - Mn) : 0.f;
-          ws += w0 + w1;
-          wl += (in0 ? w0 * v[u] : 0.f) + (in1 ? w1 * v[u + 1] : 0.f);
-          __nv_bfloat162 hb = __floats2bfloat162_rn(w0, w1);
-          __nv_bfloat162 lb = __floats2bfloat162_rn(w0 - __low2float(hb), w1 - __high2float(hb));
-          pk_[u >> 1] = wg == 0 ? *reinterpret_cast<uint32_t*>(&hb) : *reinterpret_cast<uint32_t*>(&lb);
-        }
-#pragma unroll
-        for (int ch = 0; ch < 2; ++ch)
-          *reinterpret_cast<uint4*>(sm + (wg == 0 ? oWhi : oWlo) + tc::sw128_off(row, 2 * g + ch)) = make_uint4(pk_[4 * ch], pk_[4 * ch + 1], pk_[4 * ch + 2], pk_[4 * ch + 3]);
-      }
-      s = s * sc + ws; T = T * sc + wl; M = Mn;
-      tc::fence_async_smem();
-      tc::fence_before_sync();
-      __syncthreads();
-      PCLK(2)
-      if (warp == 0) {
+      for (int ks = 0; ks < D / 16; ++ks)
+        tc::mma_bf16_ss_warp(tl, tc::desc_step(dql, (ks / 4) * TI * 128 + (ks % 4) * 32), tc::desc_step(k, (ks / 4) * NU * 128 + (ks % 4) * 32), idesc, 1);
+      tc::mma_commit_warp(&bars.l_full[el & 1]);
+      ++el;
+    };
+    const uint32_t idesc = tc::idesc_bf16(TI, D, 0, 1);    // A = W in tensor memory, B = key or value rows (MN-major)
+    Walk w;
+    start(w);
+    int n = -1, e = 0, k = 0;                              // steps (-1: only the first step's logits), non-empty steps, snapshots
+    bool acc_in = false, held = false;                     // held: snapshot k - 1 has not been waited for
+    int c0 = w.cur.p0;
+    while (w.cur.it < items) {
+      // the next step's logits, before this step's sums (an empty bucket is one step without keys)
+      const bool same = n < 0 || c0 + NU < w.cur.p1;
+      const int cn = n < 0 ? c0 : same ? c0 + NU : w.nxt.p0;
+      if (same || w.nxt.it < items) issue_l(same ? w.cur.it : w.nxt.it, same ? w.cur.pl : w.nxt.pl, cn, same ? w.cur.p1 : w.nxt.p1);
+      if (n < 0) { n = 0; continue; }
+      const int nk = min(NU, w.cur.p1 - c0);
+      if (c0 == w.cur.p0 && (w.cur.pl == 0 || per_block)) acc_in = false;
+      wait(&bars.w_ready, n & 1);
+      ++n;
+      if (nk > 0) {
+        if (held) { wait(&bars.acc_free[(k - 1) % NG], ((k - 1) / NG) & 1); held = false; }
         tc::fence_after_sync();
-        const uint32_t idesc = tc::idesc_bf16(TI, D, 0, 1);          // A = W (K-major over keys), B = key rows (MN-major)
+        const int s = e % NS, ng = (nk + 15) >> 4;
+        const uint32_t hi = tbase + LY::cL + (e & 1) * NU, lo = tbase + LY::cLo + (e & 1) * (NU / 2);
+        const uint64_t x = tc::desc_step(dn, (uint32_t)s * 2 * kKeys), y = tc::desc_step(x, kKeys);
+#pragma unroll 1
         for (int ks = 0; ks < ng; ++ks) {
-          tc::mma_bf16_ss_warp(tbase + cUk, tc::smem_desc_sw128(aWhi + ks * 32, 16, 1024), tc::smem_desc_sw128(aK + ks * 16 * 128, NU * 128, 1024), idesc, ks > 0);
-          tc::mma_bf16_ss_warp(tbase + cUv, tc::smem_desc_sw128(aWhi + ks * 32, 16, 1024), tc::smem_desc_sw128(aV + ks * 16 * 128, NU * 128, 1024), idesc, ks > 0);
+          tc::mma_bf16_ts_warp(tbase + LY::cUk, hi + 8 * ks, tc::desc_step(x, ks * 16 * 128), idesc, acc_in || ks > 0);
+          tc::mma_bf16_ts_warp(tbase + LY::cUv, hi + 8 * ks, tc::desc_step(y, ks * 16 * 128), idesc, acc_in || ks > 0);
+          tc::mma_bf16_ts_warp(tbase + LY::cUk, lo + 8 * ks, tc::desc_step(x, ks * 16 * 128), idesc, 1);
+          tc::mma_bf16_ts_warp(tbase + LY::cUv, lo + 8 * ks, tc::desc_step(y, ks * 16 * 128), idesc, 1);
         }
-        for (int ks = 0; ks < ng; ++ks) {
-          tc::mma_bf16_ss_warp(tbase + cUk, tc::smem_desc_sw128(aWlo + ks * 32, 16, 1024), tc::smem_desc_sw128(aK + ks * 16 * 128, NU * 128, 1024), idesc, 1);
-          tc::mma_bf16_ss_warp(tbase + cUv, tc::smem_desc_sw128(aWlo + ks * 32, 16, 1024), tc::smem_desc_sw128(aV + ks * 16 * 128, NU * 128, 1024), idesc, 1);
-        }
-        tc::mma_commit_warp(&bar2);
+        acc_in = true;
+        tc::mma_commit_warp(&bars.kv_empty[s]);
+        ++e;
       }
-      __syncwarp();
-      if (!tc::mbar_wait(&bar2, ph2)) ok = false;
-      ph2 ^= 1;
-      tc::fence_after_sync();
-      if (warp == 1 && ok) issue_after(c0 + nk);         // key / value tiles are free again (not thread 0: it issues the MMAs)
-      PCLK(3)
+      const bool last = !(c0 + NU < w.cur.p1);
+      if (last) {
+        if (held) wait(&bars.acc_free[(k - 1) % NG], ((k - 1) / NG) & 1);              // (a wait never skips a phase)
+        tc::mma_commit_warp(&bars.u_done[k % NG]);
+        ++k;
+        held = true;
+      }
+      tc::mma_commit_warp(&bars.u_step);
+      c0 += NU;
+      if (last) { next(w); c0 = w.cur.p0; }
+    }
+    if (held) wait(&bars.acc_free[(k - 1) % NG], ((k - 1) / NG) & 1);
+    if (n > 0) wait(&bars.u_step, (n - 1) & 1);
+  } else if (warp >= kWeightWarp0) {                       // ---- weights: thread = query cluster
+    const int row = tid - kWeightWarp0 * 32;
+    const uint32_t tl = tbase + ((uint32_t)((warp & 3) * 32) << 16);
+    Walk w;
+    start(w);
+    int n = 0, e = 0, k = 0;
+    float base = -INFINITY, s = 0.f, T = 0.f;              // (log2 units) mass and sum of w * logit, relative to the base
+    for (; w.cur.it < items; next(w)) {
+      if (w.cur.pl == 0 || per_block) { base = -INFINITY; s = 0.f; T = 0.f; }
+      int c0 = w.cur.p0;
+      do {
+        const int nk = min(NU, w.cur.p1 - c0), ng = nk > 0 ? (nk + 15) >> 4 : 0;
+        bool stepped = n == 0;                             // the previous step's products have been waited for
+        if (nk > 0) {
+          wait(&bars.l_full[e & 1], (e >> 1) & 1);
+          tc::fence_after_sync();
+          const uint32_t tL = tl + LY::cL + (e & 1) * NU, tLo = tl + LY::cLo + (e & 1) * (NU / 2);
+          // two sweeps over the logits in tensor memory (maximum, then weights); columns past the bucket's keys count as kNever
+          auto mask = [&](float (&v)[16], int g) {
+            if (16 * g + 16 > nk) {
 #pragma unroll
-      for (int d0 = 0; d0 < D; d0 += 32) {              // acc[0..D/2): kappa dims (D/2) wg.., acc[D/2..D): nu dims (D/2) wg..
+              for (int u = 0; u < 16; ++u) v[u] = 16 * g + u < nk ? v[u] : kNever;
+            }
+          };
+          float cm = kNever;
+#pragma unroll 1
+          for (int g = 0; g < ng; ++g) {
+            float v[16];
+            tc::tmem_ld16(tL + 16 * g, v);
+            mask(v, g);
+            float m4[4] = {v[0], v[1], v[2], v[3]};
+#pragma unroll
+            for (int u = 4; u < 16; ++u) m4[u & 3] = fmaxf(m4[u & 3], v[u]);
+            cm = fmaxf(cm, fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])));
+          }
+          cm *= kLog2e;
+          const bool fresh = base == -INFINITY;            // (the same in every thread)
+          const float nb = fresh || cm > base + kLazy ? cm : base;
+          if (__any_sync(0xffffffffu, !fresh && nb != base)) {
+            if (!stepped) { wait(&bars.u_step, (n - 1) & 1); stepped = true; }
+            if (k > 0) wait(&bars.acc_free[(k - 1) % NG], ((k - 1) / NG) & 1);
+            tc::fence_after_sync();
+            const float sc = tc::fast_exp2(base - nb);
+            s *= sc; T *= sc;
+#pragma unroll 1
+            for (int d0 = 0; d0 < 2 * D; d0 += 16) {
+              float v[16];
+              uint32_t x[16];
+              tc::tmem_ld16(tl + LY::cUk + d0, v);
+#pragma unroll
+              for (int u = 0; u < 16; ++u) x[u] = __float_as_uint(v[u] * sc);
+              tc::tmem_st16_issue(tl + LY::cUk + d0, x);
+            }
+          }
+          base = nb;
+          float ws[2] = {0.f, 0.f}, wl[2] = {0.f, 0.f};
+#pragma unroll 1
+          for (int g = 0; g < ng; ++g) {
+            float v[16];
+            tc::tmem_ld16(tL + 16 * g, v);
+            mask(v, g);
+            uint32_t hw[8], lw[8];
+#pragma unroll
+            for (int u = 0; u < 16; u += 2) {
+              const float w0 = tc::fast_exp2(fmaf(v[u], kLog2e, -base)), w1 = tc::fast_exp2(fmaf(v[u + 1], kLog2e, -base));
+              ws[0] += w0; ws[1] += w1;
+              wl[0] = fmaf(w0, v[u], wl[0]);
+              wl[1] = fmaf(w1, v[u + 1], wl[1]);
+              const __nv_bfloat162 hb = __floats2bfloat162_rn(w0, w1);
+              const uint32_t hu = *reinterpret_cast<const uint32_t*>(&hb);
+              const __nv_bfloat162 lb = __floats2bfloat162_rn(w0 - __uint_as_float(hu << 16), w1 - __uint_as_float(hu & 0xffff0000u));
+              hw[u >> 1] = hu;
+              lw[u >> 1] = *reinterpret_cast<const uint32_t*>(&lb);
+            }
+            tc::tmem_st8_issue(tL + 8 * g, hw);            // over logits already consumed
+            tc::tmem_st8_issue(tLo + 8 * g, lw);
+          }
+          s += ws[0] + ws[1]; T += wl[0] + wl[1];
+          ++e;
+        }
+        c0 += NU;
+        if (c0 >= w.cur.p1) { base_s[k & 3][row] = base; s_s[k & 3][row] = s; T_s[k & 3][row] = T; ++k; }
+        if (!stepped) wait(&bars.u_step, (n - 1) & 1);     // (no more than one step ahead of the products)
+        tc::tmem_st_wait();
+        tc::fence_before_sync();
+        tc::mbar_arrive(&bars.w_ready);
+        ++n;
+      } while (c0 < w.cur.p1);
+    }
+  } else {                                                 // ---- snapshots: thread = (query cluster, 32 dims of kappa and of nu)
+    const int row = (warp & 3) * 32 + lane, part = (warp >> 2) & (D / 32 - 1), grp = NG == 2 ? warp >> 3 : 0;
+    const uint32_t tl = tbase + ((uint32_t)((warp & 3) * 32) << 16) + 32 * part;
+    int k = 0;
+    Plane P{-1, 0, 0, 0, 0, 0, 0, 0, 0, 0};
+    for (take(P); P.it < items; take(P)) {
+      place(P);
+      const int j = P.j, i = P.i0 + row, pq = P.pq;
+      for (int pl = 0; pl < dm.SB; ++pl, ++k) {
+        if (k % NG != grp) continue;
+        wait(&bars.u_done[grp], (k / NG) & 1);
+        tc::fence_after_sync();
+        const float mass = s_s[k & 3][row], inv = mass > 0.f ? 1.f / mass : 0.f, base = base_s[k & 3][row], T = T_s[k & 3][row];
+        uint32_t hw[16], lw[16], nw[16];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          float v[16];
+          tc::tmem_ld16(tl + LY::cUk + 16 * h, v);
+#pragma unroll
+          for (int u = 0; u < 16; u += 2) {
+            const float x0 = inv > 0.f ? v[u] * inv : 0.f, x1 = inv > 0.f ? v[u + 1] * inv : 0.f;
+            const __nv_bfloat162 hb = __floats2bfloat162_rn(x0, x1);
+            const __nv_bfloat162 lb = __floats2bfloat162_rn(x0 - __low2float(hb), x1 - __high2float(hb));
+            hw[8 * h + u / 2] = *reinterpret_cast<const uint32_t*>(&hb);
+            lw[8 * h + u / 2] = *reinterpret_cast<const uint32_t*>(&lb);
+          }
+        }
         float v[32];
-        tc::tmem_ld32(tlane + (d0 < D / 2 ? cUk : cUv) + (D / 2) * wg + (d0 & (D / 2 - 1)), v);
+        tc::tmem_ld32(tl + LY::cUv, v);
+        tc::fence_before_sync();
+        tc::mbar_arrive(&bars.acc_free[grp]);
 #pragma unroll
-        for (int e = 0; e < 32; ++e) acc[d0 + e] = fmaf(acc[d0 + e], sc, v[e]);
-      }
-      tc::fence_before_sync();
-      PCLK(4)
-#ifdef MUSE_PHASE_CLOCKS
-      pc[7] += 1;
-#endif
-    }
-    // ---- snapshot of plane pl: three 128 x 256-byte row tiles (kappa hi, kappa lo, nu) staged in the W region
-    const bool some = s > 0.f;
-    const float inv = some ? 1.f / s : 0.f;
-    const size_t ent_row0 = ((size_t)pq * dm.SB + pl) * dm.Cq;       // entry = (ent_row0 + i) * Ck + j
-    if (wg == 0 && i < dm.Cq) {
-      const float m_ = some ? M + __logf(s) : -INFINITY;
-      const size_t ent = (ent_row0 + i) * dm.Ck + j;
-      sp.mu[ent] = m_;
-      sp.beta[ent] = some ? m_ - T * inv : -INFINITY;
-    }
-    // kappa hi / lo (warpgroup 0) and nu (warpgroup 1) as swizzled [128 rows][2 x 128 B] tiles; they leave
-    // by TMA (rows of consecutive query clusters are Ck entries apart in memory) while the next plane is computed
-    if (warp == 0) tc::tma_store_wait_read_warp();                           // the previous plane's stores have read the tiles
-    __syncthreads();
-    // this warpgroup's half of the row (dims [HD wg, HD wg + HD)) in 16-byte chunks of 8 dims: chunk c of column group gq
+        for (int u = 0; u < 32; u += 2) {
+          const __nv_bfloat162 nb = __floats2bfloat162_rn(inv > 0.f ? v[u] * inv : 0.f, inv > 0.f ? v[u + 1] * inv : 0.f);
+          nw[u / 2] = *reinterpret_cast<const uint32_t*>(&nb);
+        }
+        if (i < dm.Cq && ok) {                             // 32-byte stores: whole sectors
+          const size_t ent = (((size_t)pq * dm.SB + pl) * dm.Cq + i) * dm.Ck + j, at = ent * D + 32 * part;
+          if (part == 0) {
+            const float m_ = mass > 0.f ? (base + log2f(mass)) * 0.6931471805599453f : -INFINITY;
+            sp.mu[ent] = m_;
+            sp.beta[ent] = mass > 0.f ? m_ - T * inv : -INFINITY;
+          }
 #pragma unroll
-    for (int ck = 0; ck < HD / 8; ++ck) {
-      uint32_t w[4], wl_[4], wn[4];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float x0 = acc[ck * 8 + 2 * e] * inv, x1 = acc[ck * 8 + 2 * e + 1] * inv;
-        __nv_bfloat162 hh = __floats2bfloat162_rn(x0, x1);
-        __nv_bfloat162 ll = __floats2bfloat162_rn(x0 - __low2float(hh), x1 - __high2float(hh));
-        __nv_bfloat162 nn = __floats2bfloat162_rn(acc[HD + ck * 8 + 2 * e] * inv, acc[HD + ck * 8 + 2 * e + 1] * inv);
-        w[e] = *reinterpret_cast<uint32_t*>(&hh); wl_[e] = *reinterpret_cast<uint32_t*>(&ll); wn[e] = *reinterpret_cast<uint32_t*>(&nn);
+          for (int c = 0; c < 2; ++c) {
+            tc::st_global_32B((bf16*)sp.khi + at + 16 * c, reinterpret_cast<uint32_t(&)[8]>(hw[8 * c]));
+            tc::st_global_32B((bf16*)sp.klo + at + 16 * c, reinterpret_cast<uint32_t(&)[8]>(lw[8 * c]));
+            tc::st_global_32B((bf16*)sp.nu + at + 16 * c, reinterpret_cast<uint32_t(&)[8]>(nw[8 * c]));
+          }
+        }
       }
-      const int dch = wg * (HD / 8) + ck;                                  // 16-byte chunk of the whole row
-      const uint32_t off = (dch >> 3) * TI * 128 + tc::sw128_off(row, dch & 7);
-      *reinterpret_cast<uint4*>(sm + oStage + off) = make_uint4(w[0], w[1], w[2], w[3]);
-      *reinterpret_cast<uint4*>(sm + oStage + kTile + off) = make_uint4(wl_[0], wl_[1], wl_[2], wl_[3]);
-      *reinterpret_cast<uint4*>(sm + oStage + 2 * kTile + off) = make_uint4(wn[0], wn[1], wn[2], wn[3]);
     }
-    tc::fence_async_smem();
-    __syncthreads();
-    if (warp == 0 && ok) {
-      const int P = pq * dm.SB + pl;
-      for (int g = 0; g < G; ++g) {
-        tc::tma_store_4d_warp(&tm_okhi, sm + oStage + g * TI * 128, 64 * g, j, i0, P);
-        tc::tma_store_4d_warp(&tm_oklo, sm + oStage + kTile + g * TI * 128, 64 * g, j, i0, P);
-        tc::tma_store_4d_warp(&tm_onu, sm + oStage + 2 * kTile + g * TI * 128, 64 * g, j, i0, P);
-      }
-      tc::tma_store_commit_warp();
-    }
-    PCLK(5)
   }
-#ifdef MUSE_PHASE_CLOCKS
-  if (tid == 0 && blockIdx.x == 5 && blockIdx.y == 0 && blockIdx.z == 0) for (int k = 0; k < 8; ++k) status[56 + k] = (int)pc[k];
-#endif
-  if (warp == 0) tc::tma_store_wait_all_warp();
+  if (!ok && lane == 0) report_status(status, 7);
   tc::fence_before_sync();
   __syncthreads();
-  if (warp == 0) tc::tmem_dealloc(tbase, 512);
-  if (!ok && tid == 0) report_status(status, 7);
+  if (warp == kMmaWarp) tc::tmem_dealloc(tbase, LY::cols);
 }
 
 bool summarize_tc_supported(const Dims& d, int dtype) { return dtype == MUSE_BF16 && (d.D == 64 || d.D == 128); }
@@ -283,7 +392,7 @@ int summarize_tc(const Dims& d, const void* Kp, const void* Vp, const int32_t* o
   // qsplit: 2 * B*Hq*Cq*D bf16 of scratch for the split centroids
   bf16* qhi = (bf16*)qsplit;
   bf16* qlo = qhi + (size_t)d.B * d.Hq * d.Cq * d.D;
-  int rcq = split_qbar(d, qbar, qhi, qlo, stream);
+  int rcq = split_qbar(d, qbar, qhi, qlo, status + kItemWord, stream);
   if (rcq != MUSE_OK) return rcq;
   CUtensorMap tqh, tql;
   rcq = make_tmap_bf16_rows(&tqh, qhi, (uint64_t)d.B * d.Hq * d.Cq, d.D, st::TI);
@@ -292,26 +401,17 @@ int summarize_tc(const Dims& d, const void* Kp, const void* Vp, const int32_t* o
   CUtensorMap tK, tV;
   int rc = make_tmap_bf16_rows(&tK, Kp, (uint64_t)d.B * d.Hkv * d.N, d.D, 16);       // boxes of 16 keys
   if (rc == MUSE_OK) rc = make_tmap_bf16_rows(&tV, Vp, (uint64_t)d.B * d.Hkv * d.N, d.D, 16);
-  // outputs as 4-D tensors (d, j, i, head * planes + plane); a box is 128 query clusters of one key cluster
-  CUtensorMap okhi, oklo, onu;
-  const uint64_t dims[4] = {(uint64_t)d.D, (uint64_t)d.Ck, (uint64_t)d.Cq, (uint64_t)d.B * d.Hq * d.SB};
-  const uint64_t strides[3] = {(uint64_t)d.D * 2, (uint64_t)d.Ck * d.D * 2, (uint64_t)d.Cq * d.Ck * d.D * 2};
-  const uint32_t box[4] = {64, 1, (uint32_t)st::TI, 1};
-  if (rc == MUSE_OK) rc = make_tmap_bf16_nd(&okhi, sp.khi, 4, dims, strides, box);
-  if (rc == MUSE_OK) rc = make_tmap_bf16_nd(&oklo, sp.klo, 4, dims, strides, box);
-  if (rc == MUSE_OK) rc = make_tmap_bf16_nd(&onu, sp.nu, 4, dims, strides, box);
   if (rc != MUSE_OK) return rc;
   prof_mark("k_summarize_tc", stream);
-  const dim3 grid(d.Ck, cdiv(d.Cq, st::TI), d.B * d.Hq);
-  if (d.D == 128) {
-    MUSE_CUDA_OK(cudaFuncSetAttribute(k_summarize_tc<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, st::Lay<128>::total));
-    k_summarize_tc<128><<<grid, st::THREADS, st::Lay<128>::total, stream>>>(d, tK, tV, okhi, oklo, onu, tqh, tql, off_k, sp, per_block, status);
-  } else {
-    MUSE_CUDA_OK(cudaFuncSetAttribute(k_summarize_tc<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, st::Lay<64>::total));
-    k_summarize_tc<64><<<grid, st::THREADS, st::Lay<64>::total, stream>>>(d, tK, tV, okhi, oklo, onu, tqh, tql, off_k, sp, per_block, status);
-  }
-  MUSE_LAUNCH_OK();
-  return MUSE_OK;
+  const long long items = (long long)d.Ck * cdiv(d.Cq, st::TI) * d.B * d.Hq;
+  const int grid = (int)(items < sm_count() ? items : sm_count());
+  // With many key clusters per tile the items are dealt out one by one, in order: all CTAs then write neighbouring rows at a time,
+  // which is what DRAM wants (128k tokens, 512 x 2048 clusters, 22 GB of summaries: 9.1 ms in one range per CTA, 6.3 ms dealt).
+  // With few, every item would change the tile.
+  const int per = d.Ck >= grid ? 1 : (int)((items + grid - 1) / grid);
+  int* dealt = status + kItemWord;
+  if (d.D == 128) return launch_pdl(k_summarize_tc<128>, dim3(grid), st::kThreads, st::Lay<128>::total, stream, d, tK, tV, tqh, tql, off_k, sp, per_block, per, dealt, status);
+  return launch_pdl(k_summarize_tc<64>, dim3(grid), st::kThreads, st::Lay<64>::total, stream, d, tK, tV, tqh, tql, off_k, sp, per_block, per, dealt, status);
 }
 
 }  // namespace muse
