@@ -548,8 +548,14 @@ bool far_fwd_tc_supported(const Dims& d, int dtype) {
   return dtype == MUSE_BF16 && (d.D == 64 || d.D == 128) && d.Ck <= 2048;
 }
 
+bool far_fwd_small_supported(const Dims& d, bool sel_given);
+int far_fwd_small(const Dims& d, const SummPtrs& sp, const void* Q, const int32_t* off_q, const int32_t* perm_q, const int32_t* sel_in,
+                  int32_t* sel_out, float* o_far, float* lse_far, int* status, cudaStream_t st);
+
 int far_fwd_tc(const Dims& d, const SummPtrs& sp, const void* Q, const int32_t* off_q, const int32_t* perm_q,
                const int32_t* sel_in, int32_t* sel_out, float* o_far, float* lse_far, int* status, cudaStream_t st) {
+  // four threads per query hold their scores and a sorted list of the largest in registers up to 256 clusters and lists of 16
+  if (far_fwd_small_supported(d, sel_in != nullptr)) return far_fwd_small(d, sp, Q, off_q, perm_q, sel_in, sel_out, o_far, lse_far, status, st);
   // [segments][Ck][D]
   const uint64_t dims[3] = {(uint64_t)d.D, (uint64_t)d.Ck, (uint64_t)d.B * d.Hq * d.SB * d.Cq};
   const uint64_t strides[2] = {(uint64_t)d.D * 2, (uint64_t)d.Ck * d.D * 2};
