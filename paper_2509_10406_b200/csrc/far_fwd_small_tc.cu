@@ -1,17 +1,18 @@
 // Far-field forward on the tensor cores for few key clusters (Ck <= 256) and short selections (m <= 16, or selections that
 // are given); far_fwd_tc.cu has the definitions and the kernel for the rest.  One CTA per (query cluster i, plane, head)
-// segment, 64 of its queries per pass:
-//   A  scores^T[j][r] = (kappa_hi[j] + kappa_lo[j]) . q[r]   clusters on the M side (tiles of 128), queries on the N side;
-//      all of the segment's kappa and nu tiles arrive by TMA at the start
-//   B  tensor memory -> shared memory, transposed to [r][j] fp32, beta added
-//   C  four threads per query, a quarter of its scores each in registers: a running sorted list of the largest (branch-free
-//      max / min steps) per thread, two merges, and everything above the m-th largest is selected (ties: lowest cluster
-//      first); softmax over the rest, P written as a bf16 operand
+// segment, 64 of its queries per pass (32 above 128 clusters):
+//   A  scores^T[j][r] = (kappa_hi[j] + kappa_lo[j]) . q[r]   clusters on the M side (tiles of 128), queries on the N side
+//   B  tensor memory -> shared memory, transposed to [r][j] fp32, beta added; the nu tiles are on their way meanwhile
+//   C  32 scores per thread, in registers (four threads per query up to 128 clusters, eight above): groups of 8 or 16 sorted by
+//      a branch-free network, merged to the thread's and then the query's largest m; all scores from the m-th largest up are
+//      selected (ties beyond m: lowest cluster first); softmax over the rest, P written as a bf16 operand
 //   D  out^T[d][r] = sum_j nu[j][d] P[r][j]
 // A warp per query, which the other kernel has, takes some thousand instructions per query for the bisection to the m-th
-// largest score and its votes; four threads per query take 2 * Ck / 4 * 8 (or 16) max / min steps for eight queries at once.
+// largest score and its votes; here 500 to 700 serve eight or four queries at once.
 //
-// Bound by the latency of the phases; several CTAs share an SM.  MEASURED
+// Bound by instruction issue and the latency of the phases; two or three CTAs share an SM.  Against the other kernel: 32 heads
+// of 64k tokens, D = 64, 128 x 128 clusters, 8 slots 3130 -> 934 us; 32 heads of 16k, 128 x 256, 16 slots 1562 -> 686; 16 heads
+// of 8k, 64 x 128 367 -> 131; 6 heads of 9k, D = 128, 50 x 200, 10 slots 230 -> 94.
 #include <cuda.h>
 #include "common.cuh"
 #include "tc05.cuh"
@@ -22,15 +23,39 @@ typedef __nv_bfloat16 bf16;
 int make_tmap_bf16_nd(void* out_map, const void* base, int rank, const uint64_t* dims, const uint64_t* strides_bytes, const uint32_t* box);
 
 namespace fs {
-constexpr int kJ = 128, kR = 64, kThreads = 256;           // clusters of a tile, queries of a pass
+constexpr int kJ = 128, kThreads = 256, NV = 32;           // clusters of a tile; scores per thread
 template <int D, int CT> struct Lay {                      // CT: tiles of clusters
+  static constexpr int kR = 64 / CT, TQ = 4 * CT;          // queries of a pass, threads per query
   static constexpr int kTile = kJ * D * 2, LD = CT * kJ + 4;                  // LD: floats per score row (16-byte reads of 8 rows do not conflict)
-  static constexpr int kKappa = 2 * CT * kTile, kScore = kR * LD * 4, kArea = kKappa > kScore ? kKappa : (kScore + 1023) / 1024 * 1024;
-  // at D = 64 the 128-row products of phase D read one tile past nu, into the area behind it, and ignore the result
-  static constexpr int oNu = 0, oArea = CT * kTile, oQ = oArea + kArea, total = oQ + kR * D * 2 + 1024;
-  static constexpr int kMin = total <= 75 * 1024 ? 3 : total <= 113 * 1024 ? 2 : 1;      // CTAs per SM
+  // phase A: a ring of kappa tiles; then the nu tiles, and behind them the scores, later P.  (At D = 64 the 128-row products of
+  // phase D read one tile past nu, and ignore the result.)
+  static constexpr int kScore = (kR * LD * 4 + 1023) / 1024 * 1024, kArea0 = CT * kTile + (kScore > kTile ? kScore : kTile);
+  static constexpr int NS = kArea0 / kTile < 2 * CT ? kArea0 / kTile : 2 * CT, kArea = kArea0;
+  static constexpr int oNu = 0, oScore = CT * kTile, oQ = kArea, total = oQ + kR * D * 2 + 1024;
+  static constexpr int kMin = total <= 75 * 1024 ? 3 : 2;  // CTAs per SM
 };
-struct Bars { uint64_t kappa, nu, done; };
+// descending sorting network (Batcher's odd-even merge) over N registers at a[o ..); P, K: the stage
+template <int N, int P = 1, int K = 1> __device__ __forceinline__ void sort_desc(float* a) {
+#pragma unroll
+  for (int e = 0; e + K < N; ++e)
+    if (e >= K % P && (e - K % P) % (2 * K) < K && e / (2 * P) == (e + K) / (2 * P)) {
+      const float hi = fmaxf(a[e], a[e + K]), lo = fminf(a[e], a[e + K]);
+      a[e] = hi; a[e + K] = lo;
+    }
+  if constexpr (K > 1) sort_desc<N, P, K / 2>(a);
+  else if constexpr (2 * P < N) sort_desc<N, 2 * P, 2 * P>(a);
+}
+// the larger half of two descending lists, descending, into a (b in the order it is given)
+template <int N> __device__ __forceinline__ void merge_desc(float* a, const float* b) {
+#pragma unroll
+  for (int k = 0; k < N; ++k) a[k] = fmaxf(a[k], b[N - 1 - k]);        // a bitonic sequence
+#pragma unroll
+  for (int d = N / 2; d > 0; d >>= 1)
+#pragma unroll
+    for (int k = 0; k < N; ++k)
+      if ((k & d) == 0) { const float hi = fmaxf(a[k], a[k + d]), lo = fminf(a[k], a[k + d]); a[k] = hi; a[k + d] = lo; }
+}
+struct Bars { uint64_t full[4], empty[4], nu, done; };
 }  // namespace fs
 
 template <int D, int CT, int ML>
@@ -41,8 +66,8 @@ k_far_fwd_small(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __gri
                 float* __restrict__ lse_far, int* __restrict__ status) {
   using namespace fs;
   typedef Lay<D, CT> LY;
-  constexpr int G = D / 64, kTile = LY::kTile, LD = LY::LD, NV = 32 * CT;     // NV: scores per thread
-  constexpr uint32_t kCols = 64 * CT;
+  constexpr int G = D / 64, kTile = LY::kTile, LD = LY::LD, kR = LY::kR, TQ = LY::TQ, NS = LY::NS;
+  constexpr uint32_t kCols = 64;
   extern __shared__ __align__(1024) unsigned char sm_raw[];
   __shared__ Bars bars;
   __shared__ uint32_t tbase_s;
@@ -51,10 +76,13 @@ k_far_fwd_small(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __gri
   const int i = blockIdx.x, pl = blockIdx.y, pq = blockIdx.z, blk = dm.causal ? pl + 1 : 0, Ck = dm.Ck, m = dm.m;
   const int tid = threadIdx.x, warp = tc::warp_index(), lane = tid & 31;
   unsigned char* sm = sm_raw + ((1024u - (tc::smem_u32(sm_raw) & 1023u)) & 1023u);
-  float* sc = reinterpret_cast<float*>(sm + LY::oArea);
-  unsigned char *Pm = sm + LY::oArea, *Qs = sm + LY::oQ;
+  float* sc = reinterpret_cast<float*>(sm + LY::oScore);
+  unsigned char *Pm = sm + LY::oScore, *Qs = sm + LY::oQ;
   if (warp == 0) tc::tmem_alloc(&tbase_s, kCols);
-  if (tid == 0) { tc::mbar_init(&bars.kappa, 1); tc::mbar_init(&bars.nu, 1); tc::mbar_init(&bars.done, 1); tc::mbar_init_fence(); }
+  if (tid == 0) {
+    for (int t = 0; t < NS; ++t) { tc::mbar_init(&bars.full[t], 1); tc::mbar_init(&bars.empty[t], 1); }
+    tc::mbar_init(&bars.nu, 1); tc::mbar_init(&bars.done, 1); tc::mbar_init_fence();
+  }
   pdl_trigger();
   pdl_wait();
   const int32_t* oq = off_q + (size_t)pq * (dm.S * dm.Cq + 1) + (size_t)blk * dm.Cq + i;
@@ -89,25 +117,20 @@ k_far_fwd_small(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __gri
   tc::fence_after_sync();
   const uint32_t tbase = tbase_s;
   bool ok = true;
-  uint32_t done_ph = 0, k_ph = 0;
+  uint32_t done_ph = 0, nu_ph = 0, cnt = 0;                // cnt: kappa tiles of earlier passes
   for (int r0 = p0; r0 < p1 && ok; r0 += kR) {
     const int n = min(kR, p1 - r0), n16 = (n + 15) & ~15;
+    auto load_kappa = [&](int t) {                         // tile t: hi and lo of 128 clusters in turn
+      const int s = (cnt + t) % NS;
+      if (!tc::mbar_wait(&bars.empty[s], (((cnt + t) / NS) & 1) ^ 1)) { ok = false; return; }
+      tc::mbar_expect_tx_warp(&bars.full[s], kTile);
+      const void* map = (t & 1) ? (const void*)&tm_klo : (const void*)&tm_khi;
+#pragma unroll
+      for (int g = 0; g < G; ++g) tc::tma_load_3d_warp(sm + s * kTile + g * kJ * 128, map, 64 * g, (t >> 1) * kJ, seg, &bars.full[s]);
+    };
     if (warp == 0) {                                       // ---- A
-      tc::mbar_expect_tx_warp(&bars.kappa, 2 * CT * kTile);
-#pragma unroll
-      for (int t = 0; t < CT; ++t)
-#pragma unroll
-        for (int g = 0; g < G; ++g) {
-          tc::tma_load_3d_warp(sm + LY::oArea + 2 * t * kTile + g * kJ * 128, &tm_khi, 64 * g, t * kJ, seg, &bars.kappa);
-          tc::tma_load_3d_warp(sm + LY::oArea + (2 * t + 1) * kTile + g * kJ * 128, &tm_klo, 64 * g, t * kJ, seg, &bars.kappa);
-        }
-      if (r0 == p0) {
-        tc::mbar_expect_tx_warp(&bars.nu, CT * kTile);
-#pragma unroll
-        for (int t = 0; t < CT; ++t)
-#pragma unroll
-          for (int g = 0; g < G; ++g) tc::tma_load_3d_warp(sm + LY::oNu + t * kTile + g * kJ * 128, &tm_nu, 64 * g, t * kJ, seg, &bars.nu);
-      }
+#pragma unroll 1
+      for (int t = 0; t < NS; ++t) load_kappa(t);
     }
     if (tid < kR) {
       int t = tid < n ? pm[r0 + tid] : -1;
@@ -121,53 +144,77 @@ k_far_fwd_small(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __gri
       if (r < n && MUSE_IN_RANGE(pm[r0 + r], dm.N)) v = reinterpret_cast<const uint4*>(Qp + (size_t)pm[r0 + r] * D)[ck];
       *reinterpret_cast<uint4*>(Qs + (ck >> 3) * kR * 128 + tc::sw128_off(r, ck & 7)) = v;
     }
-    float bq[CT];                                          // beta of this thread's clusters (lane = cluster in phase B)
-#pragma unroll
-    for (int t = 0; t < CT; ++t) { const int j = t * kJ + (tid & 127); bq[t] = j < Ck ? beta[ent0 + j] : -INFINITY; }
+    const int jb = (CT == 2 ? (warp >> 2) * kJ : 0) + (tid & 127);
+    const float bq = jb < Ck ? beta[ent0 + jb] : -INFINITY;  // beta of this thread's cluster in phase B
     tc::fence_async_smem();
     __syncthreads();
-    if (warp == 1) {
-      if (!tc::mbar_wait(&bars.kappa, k_ph)) ok = false;
-      tc::fence_after_sync();
+    if (warp == 0) {
+#pragma unroll 1
+      for (int t = NS; t < 2 * CT; ++t) load_kappa(t);
+#pragma unroll 1
+      for (int t = 0; r0 == p0 && t < CT; ++t)             // nu into L2 (it arrives when the ring has been consumed)
+        for (int g = 0; g < G; ++g) tc::tma_prefetch_3d_warp(&tm_nu, 64 * g, t * kJ, seg);
+    } else if (warp == 1) {
       const uint32_t idesc = tc::idesc_bf16(kJ, n16, 0, 0);
-      const uint64_t dq = tc::smem_desc_sw128(tc::smem_u32(Qs), 16, 1024), da = tc::smem_desc_sw128(tc::smem_u32(sm + LY::oArea), 16, 1024);
-#pragma unroll
-      for (int t = 0; t < 2 * CT; ++t)
+      const uint64_t dq = tc::smem_desc_sw128(tc::smem_u32(Qs), 16, 1024), da = tc::smem_desc_sw128(tc::smem_u32(sm), 16, 1024);
+#pragma unroll 1
+      for (int t = 0; t < 2 * CT; ++t) {
+        const int s = (cnt + t) % NS;
+        if (!tc::mbar_wait(&bars.full[s], ((cnt + t) / NS) & 1)) ok = false;
+        tc::fence_after_sync();
 #pragma unroll
         for (int ks = 0; ks < D / 16; ++ks)
-          tc::mma_bf16_ss_warp(tbase + (t >> 1) * kR, tc::desc_step(da, t * kTile + (ks / 4) * kJ * 128 + (ks % 4) * 32),
+          tc::mma_bf16_ss_warp(tbase + (t >> 1) * kR, tc::desc_step(da, s * kTile + (ks / 4) * kJ * 128 + (ks % 4) * 32),
                                tc::desc_step(dq, (ks / 4) * kR * 128 + (ks % 4) * 32), idesc, (t & 1) || ks > 0);
+        tc::mma_commit_warp(&bars.empty[s]);
+      }
       tc::mma_commit_warp(&bars.done);
       if (!tc::mbar_wait(&bars.done, done_ph)) ok = false;
       tc::fence_before_sync();
     }
-    k_ph ^= 1;
+    cnt += 2 * CT;
     ok = __syncthreads_and(ok);
     done_ph ^= 1;
     tc::fence_after_sync();
-    // ---- B: the kappa tiles have been read, the scores take their place.  Warps 0-3: queries 0-31, warps 4-7: the others
+    // ---- B: the kappa tiles have been read, nu and the scores take their place.  The two groups of four warps take half of the
+    // queries each, or a tile of clusters each
+    if (warp == 0) {
+      tc::mbar_expect_tx_warp(&bars.nu, CT * kTile);
 #pragma unroll
-    for (int t = 0; t < CT; ++t)
+      for (int t = 0; t < CT; ++t)
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int c0 = 32 * (warp >> 2) + 16 * h;
-        if (c0 < n16) {
-          float v[16];
-          tc::tmem_ld16(tbase + ((uint32_t)((warp & 3) * 32) << 16) + t * kR + c0, v);
+        for (int g = 0; g < G; ++g) tc::tma_load_3d_warp(sm + LY::oNu + t * kTile + g * kJ * 128, &tm_nu, 64 * g, t * kJ, seg, &bars.nu);
+    }
 #pragma unroll
-          for (int r = 0; r < 16; ++r) sc[(c0 + r) * LD + t * kJ + (tid & 127)] = bq[t] == -INFINITY ? -INFINITY : fmaf(v[r], dm.sigma, bq[t]);
-        }
+    for (int h = 0; h < 2; ++h) {
+      const int t = CT == 2 ? warp >> 2 : 0, c0 = (CT == 2 ? 0 : 32 * (warp >> 2)) + 16 * h, j = t * kJ + (tid & 127);
+      if (c0 < n16) {
+        const float b = bq;
+        float v[16];
+        tc::tmem_ld16(tbase + ((uint32_t)((warp & 3) * 32) << 16) + t * kR + c0, v);
+#pragma unroll
+        for (int r = 0; r < 16; ++r) sc[(c0 + r) * LD + j] = b == -INFINITY ? -INFINITY : fmaf(v[r], dm.sigma, b);
       }
+    }
     tc::fence_before_sync();
     __syncthreads();
-    // ---- C: thread q of a query's four has its chunks q, q + 4, ... of eight clusters
-    const int r = warp * 8 + (lane >> 2), q = lane & 3;
-    const bool live = r < n && rows[r] >= 0;
+    // ---- C: thread q of a query's TQ has its chunks q, q + TQ, ... of eight clusters
+    constexpr int RW = 32 / TQ;                            // queries of a warp
+    const int r = warp * RW + lane / TQ, q = lane % TQ;
+    const bool live = r < n && rows[r] >= 0, work = warp * RW < n;
+    auto cluster_of = [&](int e) { return 8 * (q + TQ * (e >> 3)) + (e & 7); };
+    auto red = [&](auto x, auto op) {                      // over the threads of a query
+#pragma unroll
+      for (int o = 1; o < TQ; o <<= 1) x = op(x, __shfl_xor_sync(0xffffffffu, x, o));
+      return x;
+    };
+    const auto add = [](int a, int b) { return a + b; };
+    const auto fmx = [](float a, float b) { return fmaxf(a, b); };
     int32_t* so = sel_out + ((size_t)pq * dm.N + max(r < n ? rows[r] : 0, 0)) * m;
     float* s = sc + r * LD;
-    if (warp * 8 < n && (sel_in != nullptr || percluster)) {
+    if (work && (sel_in != nullptr || percluster)) {
       if (live)
-        for (int k = q; k < m; k += 4) {
+        for (int k = q; k < m; k += TQ) {
           int c = percluster ? selq[k] : sel_in[((size_t)pq * dm.N + rows[r]) * m + k];
           c = c >= 0 && c < Ck ? c : -1;
           so[k] = c;
@@ -176,121 +223,97 @@ k_far_fwd_small(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __gri
       __syncwarp();
     }
     float v[NV];
-    if (warp * 8 < n) {
+    if (work) {
 #pragma unroll
       for (int t = 0; t < NV / 8; ++t) {
-        const float4 a = *reinterpret_cast<const float4*>(s + 8 * (q + 4 * t)), b = *reinterpret_cast<const float4*>(s + 8 * (q + 4 * t) + 4);
+        const float4 a = *reinterpret_cast<const float4*>(s + 8 * (q + TQ * t)), b = *reinterpret_cast<const float4*>(s + 8 * (q + TQ * t) + 4);
         v[8 * t] = a.x; v[8 * t + 1] = a.y; v[8 * t + 2] = a.z; v[8 * t + 3] = a.w;
         v[8 * t + 4] = b.x; v[8 * t + 5] = b.y; v[8 * t + 6] = b.z; v[8 * t + 7] = b.w;
       }
       if (sel_in == nullptr && !percluster && m > 0) {     // (the same in every thread)
-        float a[ML];                                       // the largest so far, descending
+        float T;                                           // the m-th largest score
+        {
+          float a[NV];
 #pragma unroll
-        for (int k = 0; k < ML; ++k) a[k] = -INFINITY;
+          for (int e = 0; e < NV; ++e) a[e] = v[e];
 #pragma unroll
-        for (int e = 0; e < NV; ++e) {
-          float x = v[e];
+          for (int g = 0; g < NV / ML; ++g) sort_desc<ML>(a + g * ML);
 #pragma unroll
-          for (int k = 0; k < ML; ++k) { const float hi = fmaxf(a[k], x); x = fminf(a[k], x); a[k] = hi; }
-        }
+          for (int w = NV / ML / 2; w > 0; w >>= 1)
 #pragma unroll
-        for (int o = 1; o <= 2; o <<= 1) {                 // merge with the neighbour's list: the larger halves form a bitonic sequence
-          float b[ML];
+            for (int g = 0; g < w; ++g) merge_desc<ML>(a + g * ML, a + (g + w) * ML);
 #pragma unroll
-          for (int k = 0; k < ML; ++k) b[k] = __shfl_xor_sync(0xffffffffu, a[k], o);
+          for (int o = 1; o < TQ; o <<= 1) {
+            float b[ML];
 #pragma unroll
-          for (int k = 0; k < ML; ++k) a[k] = fmaxf(a[k], b[ML - 1 - k]);
-#pragma unroll
-          for (int d = ML / 2; d > 0; d >>= 1)
-#pragma unroll
-            for (int k = 0; k < ML; ++k)
-              if ((k & d) == 0) { const float hi = fmaxf(a[k], a[k + d]), lo = fminf(a[k], a[k + d]); a[k] = hi; a[k + d] = lo; }
-        }
-        float T = a[0];
-#pragma unroll
-        for (int k = 1; k < ML; ++k) T = k == m - 1 ? a[k] : T;
-        uint32_t gt[CT], eq[CT];                           // above the m-th largest; equal to it (none if fewer than m are finite)
-        int cnt = 0;                                       // both counts, 16 bits each
-#pragma unroll
-        for (int w = 0; w < CT; ++w) {
-          gt[w] = eq[w] = 0u;
-#pragma unroll
-          for (int e = 0; e < 32; ++e) {
-            gt[w] |= v[32 * w + e] > T ? 1u << e : 0u;
-            eq[w] |= v[32 * w + e] == T ? 1u << e : 0u;
+            for (int k = 0; k < ML; ++k) b[k] = __shfl_xor_sync(0xffffffffu, a[k], o);
+            merge_desc<ML>(a, b);
           }
-          if (T == -INFINITY) eq[w] = 0u;
-          cnt += __popc(gt[w]) | __popc(eq[w]) << 16;
+          T = -INFINITY;                                   // (written so that the list stays in registers)
+#pragma unroll
+          for (int k = 0; k < ML; ++k) T = fmaxf(T, k >= m - 1 ? a[k] : -INFINITY);
         }
-        int all = cnt + __shfl_xor_sync(0xffffffffu, cnt, 1);
-        all += __shfl_xor_sync(0xffffffffu, all, 2);
-        int need = m - (all & 0xffff);                     // ties still to take
-        bool few = (all >> 16) <= need;
-        if (few) {
+        uint32_t take = 0u;
 #pragma unroll
-          for (int w = 0; w < CT; ++w) gt[w] |= eq[w];
-        }
-        while (__any_sync(0xffffffffu, !few && need > 0)) {            // more ties than places: lowest cluster first
-          int jm = 0x7fffffff;                             // (bit e of word w is cluster 8 (q + 4 (4 w + e / 8)) + e % 8: ascending)
+        for (int e = 0; e < NV; ++e) take |= v[e] >= T ? 1u << e : 0u;
+        if (__any_sync(0xffffffffu, red(__popc(take), add) != m)) {            // ties at T beyond m places, or fewer than m finite scores
+          uint32_t gt = 0u;
 #pragma unroll
-          for (int w = CT - 1; w >= 0; --w)
-            if ((eq[w] & ~gt[w]) != 0u) { const int e = __ffs((int)(eq[w] & ~gt[w])) - 1; jm = 8 * (q + 4 * (4 * w + (e >> 3))) + (e & 7); }
-          int jq = min(jm, __shfl_xor_sync(0xffffffffu, jm, 1));
-          jq = min(jq, __shfl_xor_sync(0xffffffffu, jq, 2));
-          if (!few && need > 0 && jm == jq) {
-            const int ch = jm >> 5, e = (ch & 3) * 8 + (jm & 7);       // chunk (jm >> 3) = q + 4 ch
-#pragma unroll
-            for (int w = 0; w < CT; ++w) if ((ch >> 2) == w) gt[w] |= 1u << e;
+          for (int e = 0; e < NV; ++e) gt |= v[e] > T ? 1u << e : 0u;
+          uint32_t eq = T == -INFINITY ? 0u : take & ~gt;
+          int need = m - red(__popc(gt), add);
+          if (red(__popc(eq), add) <= need) { gt |= eq; eq = 0u; need = 0; }
+          while (__any_sync(0xffffffffu, eq != 0u && need > 0)) {              // lowest cluster first
+            const int jm = eq != 0u ? cluster_of(__ffs((int)eq) - 1) : 0x7fffffff;
+            const int jq = red(jm, [](int a, int b) { return min(a, b); });
+            if (need > 0 && jm == jq && eq != 0u) { gt |= eq & (0u - eq); eq &= eq - 1u; }
+            --need;
           }
-          --need;
+          take = gt;
         }
-        int mine = 0;
-#pragma unroll
-        for (int w = 0; w < CT; ++w) mine += __popc(gt[w]);
+        const int mine = __popc(take);
         int inc = mine;
-        { const int x = __shfl_up_sync(0xffffffffu, inc, 1, 4); if (q >= 1) inc += x; }
-        { const int x = __shfl_up_sync(0xffffffffu, inc, 2, 4); if (q >= 2) inc += x; }
-        const int tot = __shfl_sync(0xffffffffu, inc, 3, 4);
+#pragma unroll
+        for (int o = 1; o < TQ; o <<= 1) { const int x = __shfl_up_sync(0xffffffffu, inc, o, TQ); if (q >= o) inc += x; }
+        const int tot = __shfl_sync(0xffffffffu, inc, TQ - 1, TQ);
         if (live) {
           int at = inc - mine;
-#pragma unroll
-          for (int w = 0; w < CT; ++w)
-            for (uint32_t b = gt[w]; b != 0u; b &= b - 1u) {
-              const int e = __ffs((int)b) - 1;
-              if (at < m) so[at] = 8 * (q + 4 * (4 * w + (e >> 3))) + (e & 7);
-              ++at;
-            }
-          for (int k = tot + q; k < m; k += 4) so[k] = -1;
+          for (uint32_t b = take; b != 0u; b &= b - 1u, ++at)
+            if (at < m) so[at] = cluster_of(__ffs((int)b) - 1);
+          for (int k = tot + q; k < m; k += TQ) so[k] = -1;
         }
 #pragma unroll
-        for (int e = 0; e < NV; ++e) v[e] = (gt[e >> 5] >> (e & 31)) & 1u ? -INFINITY : v[e];
+        for (int e = 0; e < NV; ++e) v[e] = (take >> e) & 1u ? -INFINITY : v[e];
       }
     }
     __syncthreads();                                       // every score has been read: P takes their place
-    if (warp * 8 < n16) {
+    if (warp * RW < n16) {
       float mx = -INFINITY, sum = 0.f;
       if (live) {
+        float m4[4] = {v[0], v[1], v[2], v[3]};
 #pragma unroll
-        for (int e = 0; e < NV; ++e) mx = fmaxf(mx, v[e]);
+        for (int e = 4; e < NV; ++e) m4[e & 3] = fmaxf(m4[e & 3], v[e]);
+        mx = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
       }
-      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+      mx = red(mx, fmx);
+      const float mx2 = mx * 1.4426950408889634f;
+      const bool some = mx != -INFINITY;
 #pragma unroll
       for (int t = 0; t < NV / 8; ++t) {
         uint32_t w[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-          float a = 0.f, b = 0.f;
-          if (mx != -INFINITY) { a = __expf(v[8 * t + 2 * k] - mx); b = __expf(v[8 * t + 2 * k + 1] - mx); }
+          const float a = some ? tc::fast_exp2(fmaf(v[8 * t + 2 * k], 1.4426950408889634f, -mx2)) : 0.f;
+          const float b = some ? tc::fast_exp2(fmaf(v[8 * t + 2 * k + 1], 1.4426950408889634f, -mx2)) : 0.f;
           const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
           sum += __low2float(h) + __high2float(h);
           w[k] = *reinterpret_cast<const uint32_t*>(&h);
         }
-        const int ch = q + 4 * t;
+        const int ch = q + TQ * t;
         *reinterpret_cast<uint4*>(Pm + (ch >> 3) * (kR * 128) + tc::sw128_off(r, ch & 7)) = make_uint4(w[0], w[1], w[2], w[3]);
       }
-      sum += __shfl_xor_sync(0xffffffffu, sum, 1);
-      sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+#pragma unroll
+      for (int o = 1; o < TQ; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
       if (q == 0) {
         rinv[r] = sum > 0.f ? 1.f / sum : 0.f;
         if (live) lse_far[(size_t)pq * dm.N + rows[r]] = sum > 0.f ? mx + logf(sum) : -INFINITY;
@@ -300,7 +323,7 @@ k_far_fwd_small(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __gri
     __syncthreads();
     // ---- D (all threads' reads of the scores in tensor memory are behind them)
     if (warp == 1) {
-      if (r0 == p0 && !tc::mbar_wait(&bars.nu, 0)) ok = false;
+      if (!tc::mbar_wait(&bars.nu, nu_ph)) ok = false;
       tc::fence_after_sync();
       const uint32_t idesc = tc::idesc_bf16(128, n16, 1, 0);
       const uint64_t dp = tc::smem_desc_sw128(tc::smem_u32(Pm), 16, 1024), dn = tc::smem_desc_sw128(tc::smem_u32(sm + LY::oNu), kJ * 128, 1024);
@@ -316,16 +339,22 @@ k_far_fwd_small(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __gri
     }
     ok = __syncthreads_and(ok);
     done_ph ^= 1;
+    nu_ph ^= 1;
     tc::fence_after_sync();
-    // ---- E: thread = output dim; warps 0-3 queries 0-31, warps 4-7 the others
-    if (32 * (warp >> 2) < n && (warp & 3) * 32 < D) {
-      const int h = 32 * (warp >> 2);
-      float x[32];
-      tc::tmem_ld32(tbase + ((uint32_t)((warp & 3) * 32) << 16) + h, x);
-      if (ok) {
+    // ---- E: thread = output dim; the two groups of four warps take half of the queries each
+    if ((warp & 3) * 32 < D) {
 #pragma unroll
-        for (int k = 0; k < 32; ++k)
-          if (h + k < n && rows[h + k] >= 0) o_far[((size_t)pq * dm.N + rows[h + k]) * D + (tid & 127)] = x[k] * rinv[h + k];
+      for (int c = 0; c < kR / 32; ++c) {
+        const int h = (warp >> 2) * (kR / 2) + 16 * c;
+        if (h < n) {
+          float x[16];
+          tc::tmem_ld16(tbase + ((uint32_t)((warp & 3) * 32) << 16) + h, x);
+          if (ok) {
+#pragma unroll
+            for (int k = 0; k < 16; ++k)
+              if (h + k < n && rows[h + k] >= 0) o_far[((size_t)pq * dm.N + rows[h + k]) * D + (tid & 127)] = x[k] * rinv[h + k];
+          }
+        }
       }
     }
     tc::fence_before_sync();

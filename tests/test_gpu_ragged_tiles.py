@@ -67,3 +67,10 @@ def test_near_field_backward_over_groups_of_blocks(monkeypatch, base, Cq, Ck, m,
     w = CASES[base].with_(Hq=2, Hkv=1, N=330 * S, S=S, Cq=Cq, Ck=Ck, m=m, components=64)
     monkeypatch.setitem(test_gpu_k2.K2_CASES, "groups", w)
     test_gpu_k2.test_two_level_backward_matches_oracle("groups", k2, True, 4)
+
+
+@pytest.mark.parametrize("base,Cq,Ck,m", [("d64", 2, 256, 16), ("d64", 3, 128, 9), ("d64", 5, 2, 1), ("d128", 2, 256, 8), ("d128", 3, 127, 16), ("d64", 4, 256, 17)])
+def test_selection_and_far_field_of_few_clusters(base, Cq, Ck, m):
+    """Lists of 8 and 16 (and one more, which another kernel takes), one and two tiles of clusters, several passes over a segment."""
+    w = CASES[base].with_(Hq=2, Hkv=1, N=1020, S=4, Cq=Cq, Ck=Ck, m=m, components=64)
+    _forward_parity(w, 128.0, expect_kernels=TC_FWD_KERNELS)
