@@ -1,4 +1,4 @@
-// Far-field backward on the tensor cores (bf16 mode, D = 64 or 128, Ck a multiple of 128, <= 2048).
+// Far-field backward on the tensor cores (bf16 mode, D = 64 or 128, Ck <= 2048).
 // One CTA per (query cluster i, plane, head) segment.  Clusters sit on the MMA M side (128 per
 // tile, one TMEM lane each), the segment's queries on the N side (64 per sweep; a longer segment
 // takes further sweeps that add to the stored gradients).  Per cluster tile, with L the merged log-sum-exp and delta = dO.O:
@@ -8,6 +8,11 @@
 //   dkappa = dkappa_raw - sigma (sum_r g) qbar_i
 //   dS = sum_r g - dkappa.kappa - dnu.nu = sum_r g (1 + mu - score) - sum_r p dPnu   (no row dot products)
 // dkappa and dnu are stored as bf16 rows for the key-side pass, dS as fp32.
+// A segment of few queries pays for its own rows only (multiples of 16), not for 64.  At D = 64 dnu and dkappa take the
+// tensor-memory columns of the consumed scores and are staged in the consumed P and G tiles, so that two CTAs fill each
+// other's waits on an SM.  Bound by DRAM at D = 128 (4.1 TB/s of reads and writes at 4 heads of 64k tokens, 256 x 1024
+// clusters), by the phases' latency at D = 64.  Measured, before | after: 32 heads of 64k tokens, 128 x 128 clusters, D = 64
+// 3243 | 1778 us; 32 heads of 16k, 128 x 256 2490 | 1330; 16 heads of 8k, 64 x 128 488 | 267; 4 heads, D = 128 2425 | 2274.
 #include <cuda.h>
 #include "common.cuh"
 #include "tc05.cuh"
@@ -31,10 +36,13 @@ template <int D> struct Lay {
   static constexpr int oPt = oDO + NP * kRows, oGt = oPt + TJ * NR * 2;
   // gradient rows on their way out: dkappa is staged in the (consumed) P / G tiles, dnu in a tile of its own,
   // so that the three operand tiles are free for the next cluster tile as soon as the MMAs have finished
-  static constexpr int oStK = oPt, oStN = oGt + TJ * NR * 2;
+  // (at D = 64: dkappa in the P tile, dnu in the G tile once the dq products have read it; two CTAs then fit an SM)
+  static constexpr int oStK = oPt, oStN = D == 64 ? oGt : oGt + TJ * NR * 2;
   static constexpr int oMask = oStN + kTile;      // [NP*NR rows][Ck/32] words follow
+  // TMEM columns; at D = 64 dnu and dkappa take the place of the consumed S and dPnu
+  static constexpr uint32_t cS = 0, cDP = 64, cDNU = D == 64 ? 0 : 128, cDKA = D == 64 ? 64 : 256, cDQ = D == 64 ? 128 : 384, cols = D == 64 ? 256 : 512;
+  static constexpr int kMin = D == 64 ? 2 : 1;    // CTAs per SM
 };
-constexpr uint32_t cS = 0, cDP = 64, cDNU = 128, cDKA = 256, cDQ = 384;   // TMEM columns
 constexpr float kLog2e = 1.4426950408889634f;
 }  // namespace fb
 
@@ -45,7 +53,7 @@ __device__ __forceinline__ float fast_exp2(float x) {
 }
 
 template <int D>
-__global__ void __launch_bounds__(fb::THREADS, 1)
+__global__ void __launch_bounds__(fb::THREADS, fb::Lay<D>::kMin)
 k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_constant__ CUtensorMap tm_klo,
              const __grid_constant__ CUtensorMap tm_nu, const __grid_constant__ CUtensorMap tm_gka,
              const __grid_constant__ CUtensorMap tm_gnu, const bf16* __restrict__ Q, const bf16* __restrict__ dO,
@@ -57,6 +65,7 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
   typedef Lay<D> LY;
   constexpr int kTile = LY::kTile, kRows = LY::kRows, oHi = LY::oHi, oLo = LY::oLo, oNu = LY::oNu, oQ = LY::oQ, oDO = LY::oDO,
                 oPt = LY::oPt, oGt = LY::oGt, oStK = LY::oStK, oStN = LY::oStN, oMask = LY::oMask, G = D / 64, CPR = D / 8;
+  constexpr uint32_t cS = LY::cS, cDP = LY::cDP, cDNU = LY::cDNU, cDKA = LY::cDKA, cDQ = LY::cDQ;
   extern __shared__ __align__(1024) unsigned char sm_raw[];
   // bar_full: kappa tiles landed; bar_nu: nu tile landed; bar1: S / dPnu products done; bar2: dnu / dkappa
   // products done; bar3: dq products done as well; bar_st: the previous tile's stores have read their staging
@@ -95,7 +104,7 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
   const bf16* dOp = dO + (size_t)pq * dm.N * D;
   const int32_t* pm = perm_q + (size_t)pq * dm.N;
 
-  if (warp == 0) tc::tmem_alloc(&tbase_s, 512);
+  if (warp == 0) tc::tmem_alloc(&tbase_s, LY::cols);
   if (tid == 0) { tc::mbar_init(&bar_full, 1); tc::mbar_init(&bar1, 1); tc::mbar_init(&bar2, 1); tc::mbar_init(&bar3, 1);
                   tc::mbar_init(&bar_nu, 1); tc::mbar_init(&bar_st, 1); tc::mbar_init_fence(); }
   if (tid < D) qb[tid] = qbar[((size_t)pq * dm.Cq + i) * D + tid];
@@ -122,6 +131,8 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
   };
   for (int s0 = p0; s0 < p1 && ok; s0 += NP * NR) {        // sweep: up to 64 rows
     const int ns = min(NP * NR, p1 - s0), np = (ns + NR - 1) / NR;
+    // the products take only as many rows as there are: nc of them (a multiple of 8) per warpgroup, nr in all
+    const int nc = ((ns + 1) / 2 + 7) & ~7, nr = 2 * nc;
     __syncthreads();
     // the operand tiles are free (every product of the previous sweep has completed): the first cluster
     // tile travels while the rows are gathered
@@ -135,7 +146,7 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
     }
     for (int e = tid; e < 2 * NJ * TJ; e += THREADS) smask[e] = 0u;
     __syncthreads();
-    for (int e = tid; e < NP * NR * CPR; e += THREADS) {
+    for (int e = tid; e < nr * CPR; e += THREADS) {
       const int r = e / CPR, ck = e % CPR, kb = ck >> 3, c = ck & 7, p = r / NR, rr = r % NR;
       uint4 a = make_uint4(0u, 0u, 0u, 0u), b = a;
       if (r < ns && rows[r] >= 0) {
@@ -156,15 +167,7 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
 #ifdef MUSE_PHASE_CLOCKS
     long long pc[6] = {0, 0, 0, 0, 0, 0};
 #endif
-    // L and delta of this warpgroup's 32 rows stay in registers for the whole sweep
     static_assert(NP == 1, "one pass per sweep");
-    float Lc[32], dc[32];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const float4 a = *reinterpret_cast<const float4*>(Ls + 32 * (wg & 1) + 4 * k), b = *reinterpret_cast<const float4*>(ds + 32 * (wg & 1) + 4 * k);
-      Lc[4 * k] = a.x; Lc[4 * k + 1] = a.y; Lc[4 * k + 2] = a.z; Lc[4 * k + 3] = a.w;
-      dc[4 * k] = b.x; dc[4 * k + 1] = b.y; dc[4 * k + 2] = b.z; dc[4 * k + 3] = b.w;
-    }
     float bnext = L < Ck ? beta[ent0 + L] : -INFINITY;
     const bool later_sweep = s0 > p0;                       // gradients of earlier sweeps are already stored: add to them
     if (later_sweep) {
@@ -193,7 +196,7 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
             if (!tc::mbar_wait(&bar_nu, ph_full)) ok = false;
           }
           tc::fence_after_sync();
-          const uint32_t idesc = tc::idesc_bf16(TJ, NR, 0, 0);
+          const uint32_t idesc = tc::idesc_bf16(TJ, nr, 0, 0);
 #pragma unroll
           for (int ks = 0; ks < D / 16; ++ks)
             tc::mma_bf16_ss_warp(tbase + cS, tc::smem_desc_sw128(aHi + (ks / 4) * TJ * 128 + (ks % 4) * 32, 16, 1024),
@@ -221,46 +224,60 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
         if (p == 0) k1_ = clock64();
 #endif
         if (cw) {
-          float s[32], dp[32];
-          tc::tmem_ld32(tlane + cS + 32 * wg, s);
-          tc::tmem_ld32(tlane + cDP + 32 * wg, dp);
-#ifdef MUSE_PHASE_CLOCKS
-          if (p == 0 && tid == 0 && blockIdx.x == 5 && blockIdx.y == 3 && blockIdx.z == 0 && jt == 3) status[32] = (int)(clock64() - k1_);
-#endif
-          uint32_t pw[16], gw[16];
-          // bit r of `near`: row r of this warpgroup's 32 is not in the far set of cluster j (retrieved,
-          // past the end of the segment, or the cluster is empty)
-          const int nv = ns - (p * NR + 32 * wg);
-          const uint32_t near = alive ? (smask[2 * j + wg] | (nv >= 32 ? 0u : nv <= 0 ? 0xffffffffu : 0xffffffffu << nv)) : 0xffffffffu;
-#pragma unroll
-          for (int c = 0; c < 32; c += 2) {
-            float pv[2], gv[2];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              const float t2 = fmaf(s[c + h], sig2, bj2);                 // Eq. 6 score in log2 units
-              const float e = fast_exp2(t2 - Lc[c + h]);
-              pv[h] = (near >> (c + h)) & 1u ? 0.f : e;
-              gv[h] = pv[h] * (dp[c + h] - dc[c + h]);
-              gsum += gv[h];
-              gt2 = fmaf(gv[h], t2, gt2);
-              pdp = fmaf(pv[h], dp[c + h], pdp);
-            }
-            __nv_bfloat162 a = __floats2bfloat162_rn(pv[0], pv[1]), b = __floats2bfloat162_rn(dm.sigma * gv[0], dm.sigma * gv[1]);
-            pw[c >> 1] = *reinterpret_cast<uint32_t*>(&a);
-            gw[c >> 1] = *reinterpret_cast<uint32_t*>(&b);
-          }
-#ifdef MUSE_PHASE_CLOCKS
-          if (p == 0 && tid == 0 && blockIdx.x == 5 && blockIdx.y == 3 && blockIdx.z == 0 && jt == 3) status[33] = (int)(clock64() - k1_);
-#endif
-          if (p == 0) {
+          // bit r of `near`: row r of this warpgroup's nc is not in the far set of cluster j (retrieved, past the end of the
+          // segment, or the cluster is empty)
+          const int nv = ns - wg * nc;
+          const unsigned long long m64 = smask[2 * j] | (unsigned long long)smask[2 * j + 1] << 32;
+          const uint32_t near = alive ? ((uint32_t)(m64 >> (wg * nc)) | (nv >= 32 ? 0u : nv <= 0 ? 0xffffffffu : 0xffffffffu << nv)) : 0xffffffffu;
+          if (p == 0) {                                    // (the previous tile's stores have read the staging tiles)
             if (!tc::mbar_wait(&bar_st, ph_st)) ok = false;
             ph_st ^= 1;
           }
+          float gs2[2] = {0.f, 0.f}, gt[2] = {0.f, 0.f}, pd[2] = {0.f, 0.f};
+          float s[8], dp[8];
+          tc::tmem_ld8_issue(tlane + cS + wg * nc, s);
+          tc::tmem_ld8_issue(tlane + cDP + wg * nc, dp);
+          tc::tmem_ld_wait();
+          tc::tmem_ld_use8(s);
+          tc::tmem_ld_use8(dp);
+#pragma unroll 1
+          for (int c0 = 0; c0 < nc; c0 += 8) {
+            float sn[8], dn[8];
+            const int cx = wg * nc + (c0 + 8 < nc ? c0 + 8 : c0);      // (the last turn loads its own columns again)
+            tc::tmem_ld8_issue(tlane + cS + cx, sn);
+            tc::tmem_ld8_issue(tlane + cDP + cx, dn);
+            const float4 La = *reinterpret_cast<const float4*>(Ls + wg * nc + c0), Lb = *reinterpret_cast<const float4*>(Ls + wg * nc + c0 + 4);
+            const float4 da = *reinterpret_cast<const float4*>(ds + wg * nc + c0), db = *reinterpret_cast<const float4*>(ds + wg * nc + c0 + 4);
+            const float Lc[8] = {La.x, La.y, La.z, La.w, Lb.x, Lb.y, Lb.z, Lb.w}, dc[8] = {da.x, da.y, da.z, da.w, db.x, db.y, db.z, db.w};
+            const uint32_t nb = near >> c0;
+            uint32_t pw[4], gw[4];
 #pragma unroll
-          for (int ch = 0; ch < 4; ++ch) {
-            *reinterpret_cast<uint4*>(sm + oPt + tc::sw128_off(L, 4 * wg + ch)) = make_uint4(pw[4 * ch], pw[4 * ch + 1], pw[4 * ch + 2], pw[4 * ch + 3]);
-            *reinterpret_cast<uint4*>(sm + oGt + tc::sw128_off(L, 4 * wg + ch)) = make_uint4(gw[4 * ch], gw[4 * ch + 1], gw[4 * ch + 2], gw[4 * ch + 3]);
+            for (int c = 0; c < 8; c += 2) {
+              float pv[2], gv[2];
+#pragma unroll
+              for (int h = 0; h < 2; ++h) {
+                const float t2 = fmaf(s[c + h], sig2, bj2);            // Eq. 6 score in log2 units
+                const float e = fast_exp2(t2 - Lc[c + h]);
+                pv[h] = (nb >> (c + h)) & 1u ? 0.f : e;
+                gv[h] = pv[h] * (dp[c + h] - dc[c + h]);
+                gs2[h] += gv[h];
+                gt[h] = fmaf(gv[h], t2, gt[h]);
+                pd[h] = fmaf(pv[h], dp[c + h], pd[h]);
+              }
+              __nv_bfloat162 a = __floats2bfloat162_rn(pv[0], pv[1]), b = __floats2bfloat162_rn(dm.sigma * gv[0], dm.sigma * gv[1]);
+              pw[c >> 1] = *reinterpret_cast<uint32_t*>(&a);
+              gw[c >> 1] = *reinterpret_cast<uint32_t*>(&b);
+            }
+            const uint32_t at = tc::sw128_off(L, (wg * nc + c0) >> 3);
+            *reinterpret_cast<uint4*>(sm + oPt + at) = make_uint4(pw[0], pw[1], pw[2], pw[3]);
+            *reinterpret_cast<uint4*>(sm + oGt + at) = make_uint4(gw[0], gw[1], gw[2], gw[3]);
+            tc::tmem_ld_wait();
+            tc::tmem_ld_use8(sn);
+            tc::tmem_ld_use8(dn);
+#pragma unroll
+            for (int c = 0; c < 8; ++c) { s[c] = sn[c]; dp[c] = dn[c]; }
           }
+          gsum += gs2[0] + gs2[1]; gt2 += gt[0] + gt[1]; pdp += pd[0] + pd[1];
         }
 #ifdef MUSE_PHASE_CLOCKS
         if (p == 0) k2_ = clock64();
@@ -273,13 +290,13 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
           const uint32_t id_row = tc::idesc_bf16(TJ, D, 0, 1);      // A K-major (P / G), B = query rows, MN-major
           // A = kappa tile MN-major, B = G MN-major.  M = 128 output dims even when D = 64: the second 64-dim group of the
           // operand is then the tile that follows in shared memory, and output lanes 64..127 hold numbers that nobody reads
-          const uint32_t id_dq = tc::idesc_bf16(128, NR, 1, 1);
+          const uint32_t id_dq = tc::idesc_bf16(128, nr, 1, 1);
 #pragma unroll
-          for (int ks = 0; ks < NR / 16; ++ks)
+          for (int ks = 0; ks < NR / 16; ++ks) if (16 * ks < nr)
             tc::mma_bf16_ss_warp(tbase + cDNU, tc::smem_desc_sw128(aPt + ks * 32, 16, 1024),
                             tc::smem_desc_sw128(aDO + ks * 16 * 128, NR * 128, 1024), id_row, !(p == 0 && ks == 0));
 #pragma unroll
-          for (int ks = 0; ks < NR / 16; ++ks)
+          for (int ks = 0; ks < NR / 16; ++ks) if (16 * ks < nr)
             tc::mma_bf16_ss_warp(tbase + cDKA, tc::smem_desc_sw128(aGt + ks * 32, 16, 1024),
                             tc::smem_desc_sw128(aQ + ks * 16 * 128, NR * 128, 1024), id_row, !(p == 0 && ks == 0));
           tc::mma_commit_warp(&bar2);              // the read-out of dnu / dkappa can start while the dq products still run
@@ -334,8 +351,8 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
         for (int u = 0; u < D / 32; ++u) {
           float x[32];
           tc::tmem_ld32(tsrc + 32 * u, x);
-          // the second half of the dkappa staging is the G tile, which the dq products read
-          if (u == 2 && wg == 1 && !tc::mbar_wait(&bar3, ph3 ^ 1)) ok = false;
+          // the second half of the dkappa staging (at D = 64: the dnu staging) is the G tile, which the dq products read
+          if (D == 128 ? u == 2 && wg == 1 : u == 0 && wg == 0) { if (!tc::mbar_wait(&bar3, ph3 ^ 1)) ok = false; }
           if (wg == 1) {
 #pragma unroll
             for (int ch = 0; ch < 8; ++ch) {
@@ -415,7 +432,7 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
   tc::fence_before_sync();
   __syncthreads();
   if (warp == ISSUER / 32) tc::tma_store_wait_read_warp();             // the staging tiles must outlive the stores' reads only
-  if (warp == 0) tc::tmem_dealloc(tbase, 512);
+  if (warp == 0) tc::tmem_dealloc(tbase, LY::cols);
   if (!ok && tid == 0) report_status(status, 4);
 #ifdef MUSE_PHASE_CLOCKS
   if (tid == 0 && blockIdx.x == 5 && blockIdx.y == 3 && blockIdx.z == 0) {
