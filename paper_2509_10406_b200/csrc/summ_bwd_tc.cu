@@ -8,7 +8,8 @@
 // (the shared-memory qbar tiles already carry the factor sigma)
 // Query clusters sit on the MMA M side for the three D-contractions (one thread per i computes
 // w and w*c) and on the K side for the three i-contractions, whose outputs are transposed
-// ([d][u]) so that the read-out is coalesced over d.  Planes are handled independently and
+// ([d][u]) so that the read-out is coalesced over d.  The centroids are the same for every plane, so w c is summed over
+// the planes in registers and contracted with them once.  Planes are handled independently and
 // accumulate, together with the query-cluster tiles, in tensor memory; the far-field backward
 // stores its gradients [plane][j][i] so that each (plane, j, 128 i) tile is one contiguous TMA box.
 #include <cuda.h>
@@ -28,17 +29,17 @@ template <int D> struct Lay {
   // The low half of the centroid tile is only needed for the tilt logits, which do not depend on
   // the plane: once they are in TMEM its space serves as the second dkappa buffer.
   static constexpr int oQhi = 0, oQlo = oQhi + kTile, oDka0 = oQlo + kTile, oDnu0 = oDka0 + kTile, oDnu1 = oDnu0 + kTile;
-  static constexpr int oK = oDnu1 + kTile, oV = oK + kKeys, oW = oV + kKeys, oWc = oW + TI * NU * 2;
-  static constexpr int total = oWc + TI * NU * 2 + 1024;
+  static constexpr int oK = oDnu1 + kTile, oV = oK + kKeys, oW = oV + kKeys;
+  static constexpr int total = oW + TI * NU * 2;           // 112 KB at D = 64, two CTAs per SM: no slack, the kernel checks the alignment of its base
 };
-constexpr uint32_t cL = 0, cX1 = 64, cX2 = 128, cDK = 192, cDV = 256;
+constexpr uint32_t cL = 0, cX1 = 0, cX2 = 64, cDK = 128, cDV = 192, cols = 256;        // (X1 over the tilt logits, which go to registers)
 }  // namespace sb
 
 // 2-D tensor map over a bf16 matrix with an arbitrary row pitch (bytes), 128B swizzle, box [box_rows][64]
 int make_tmap_bf16_pitched(void* out_map, const void* base, uint64_t rows, uint64_t cols, uint64_t pitch_bytes, uint32_t box_rows);
 
 template <int D>
-__global__ void __launch_bounds__(sb::THREADS, 1)
+__global__ void __launch_bounds__(sb::THREADS, D == 64 ? 2 : 1)
 k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_constant__ CUtensorMap tm_dnu,
               const __grid_constant__ CUtensorMap tm_K, const __grid_constant__ CUtensorMap tm_V,
               const __grid_constant__ CUtensorMap tm_qhi, const __grid_constant__ CUtensorMap tm_qlo,
@@ -51,7 +52,7 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
   using namespace sb;
   typedef Lay<D> LY;
   constexpr int kTile = LY::kTile, kKeys = LY::kKeys, oQhi = LY::oQhi, oQlo = LY::oQlo, oDka0 = LY::oDka0, oDnu0 = LY::oDnu0,
-                oDnu1 = LY::oDnu1, oK = LY::oK, oV = LY::oV, oW = LY::oW, oWc = LY::oWc, G = D / 64;
+                oDnu1 = LY::oDnu1, oK = LY::oK, oV = LY::oV, oW = LY::oW, G = D / 64;
   extern __shared__ __align__(1024) unsigned char sm_raw[];
   __shared__ uint64_t bar_g[2], bar_kv, bar_q, bar_l, bar1, bar2;
   __shared__ uint32_t tbase_s;
@@ -64,8 +65,12 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
   const int kbeg = ok_[0];
   (void)MUSE_IN_RANGE(ok_[dm.SB], dm.N + 1); (void)MUSE_IN_RANGE(kbeg, ok_[dm.SB] + 1);   // (the tiles come through tensor maps, which clip)
   if (kbeg >= ok_[dm.SB]) return;                       // no key of this cluster is ever summarised
-  unsigned char* sm = sm_raw + ((1024u - (tc::smem_u32(sm_raw) & 1023u)) & 1023u);
-  if (warp == 0) tc::tmem_alloc(&tbase_s, 512);
+  unsigned char* sm = sm_raw;
+  if ((tc::smem_u32(sm_raw) & 1023u) != 0u) {              // (the toolchain honours the declared alignment)
+    if (tid == 0) report_status(status, 5);
+    return;
+  }
+  if (warp == 0) tc::tmem_alloc(&tbase_s, cols);
   if (tid == 0) {
     tc::mbar_init(&bar_g[0], 1); tc::mbar_init(&bar_g[1], 1); tc::mbar_init(&bar_kv, 1); tc::mbar_init(&bar_q, 1); tc::mbar_init(&bar_l, 1);
     tc::mbar_init(&bar1, 1); tc::mbar_init(&bar2, 1); tc::mbar_init_fence();
@@ -77,7 +82,7 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
   uint32_t ph_g[2] = {0, 0}, ph_kv = 0, ph_q = 0, ph_l = 0, ph1 = 0, ph2 = 0;
   bool ok = true;
   const uint32_t aQhi = tc::smem_u32(sm + oQhi), aQlo = tc::smem_u32(sm + oQlo), aK = tc::smem_u32(sm + oK),
-                 aV = tc::smem_u32(sm + oV), aW = tc::smem_u32(sm + oW), aWc = tc::smem_u32(sm + oWc);
+                 aV = tc::smem_u32(sm + oV), aW = tc::smem_u32(sm + oW);
 
   const int kvis = ok_[dm.SB];
 #ifdef MUSE_PHASE_CLOCKS
@@ -163,6 +168,12 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
 #pragma unroll
         for (int c = 0; c < 32; ++c) lg[c] *= 1.4426950408889634f;
       }
+      float wc[32];                                               // sum over the planes of w c: contracted with the centroids once, below
+#pragma unroll
+      for (int c = 0; c < 32; ++c) wc[c] = 0.f;
+      tc::fence_before_sync();
+      __syncthreads();                                            // the products of the first plane overwrite the logits
+      tc::fence_after_sync();
       // per-plane scalars, loaded one plane ahead
       auto ent_of = [&](int pl) { return (((size_t)pq * dm.SB + pl) * dm.Cq + ic) * dm.Ck + j; };        // summaries: [plane][i][j]
       auto gent_of = [&](int pl) { return (((size_t)pq * dm.SB + pl) * dm.Ck + j) * dm.Cq + ic; };      // gradients: [plane][j][i]
@@ -179,7 +190,7 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
         if (pl + 1 < pl_end && ((livemask >> (pl + 1)) & 1u)) { mu_n = mu[ent_of(pl + 1)]; dS_n = dS[gent_of(pl + 1)]; }
         // The far-field pass wrote every row of the gradient tensors (zeros for an empty segment), so the
         // tiles go to the tensor cores as they land.  The D-contractions of this plane do not depend on the
-        // previous plane's i-contractions: they are issued first, and only the W / Wc tiles and the other
+        // previous plane's i-contractions: they are issued first, and only the W tile and the other
         // gradient buffer wait for those.
         if (warp == ISSUER / 32) {
           if (!tc::mbar_wait(&bar_g[buf], ph_g[buf])) ok = false;
@@ -204,23 +215,32 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
         tc::fence_after_sync();
         PCLK(3)
         if (cw) {
-          float x1[32], x2[32];
-          tc::tmem_ld32(tlane + cX1 + 32 * wg, x1);
-          tc::tmem_ld32(tlane + cX2 + 32 * wg, x2);
-          uint32_t ww[16], wc[16];
+          const int lo = live ? klo - 32 * wg : 32, hi = live ? nk - 32 * wg : 0;      // this thread's keys of the plane: [lo, hi)
+          const bool whole = lo <= 0 && hi >= 32;
+          if (k > 0 && !tc::mbar_wait(&bar2, ph2)) ok = false;      // the previous plane's MMAs have read W
 #pragma unroll
-          for (int c = 0; c < 32; c += 2) {
-            float w0 = 0.f, w1 = 0.f, c0_ = 0.f, c1_ = 0.f;
-            if (live && 32 * wg + c < nk && 32 * wg + c >= klo) { w0 = tc::fast_exp2(lg[c] - mu_i); c0_ = w0 * (dS_i + x1[c] + x2[c]); }
-            if (live && 32 * wg + c + 1 < nk && 32 * wg + c + 1 >= klo) { w1 = tc::fast_exp2(lg[c + 1] - mu_i); c1_ = w1 * (dS_i + x1[c + 1] + x2[c + 1]); }
-            __nv_bfloat162 a = __floats2bfloat162_rn(w0, w1), b = __floats2bfloat162_rn(c0_, c1_);
-            ww[c >> 1] = *reinterpret_cast<uint32_t*>(&a); wc[c >> 1] = *reinterpret_cast<uint32_t*>(&b);
-          }
-          if (k > 0 && !tc::mbar_wait(&bar2, ph2)) ok = false;      // the previous plane's MMAs have read W / Wc
+          for (int g = 0; g < 4; ++g) {
+            float x1[8], x2[8];
+            tc::tmem_ld8_issue(tlane + cX1 + 32 * wg + 8 * g, x1);
+            tc::tmem_ld8_issue(tlane + cX2 + 32 * wg + 8 * g, x2);
+            tc::tmem_ld_wait();
+            tc::tmem_ld_use8(x1);
+            tc::tmem_ld_use8(x2);
+            uint32_t ww[4];
 #pragma unroll
-          for (int ch = 0; ch < 4; ++ch) {
-            *reinterpret_cast<uint4*>(sm + oW + tc::sw128_off(L, 4 * wg + ch)) = make_uint4(ww[4 * ch], ww[4 * ch + 1], ww[4 * ch + 2], ww[4 * ch + 3]);
-            *reinterpret_cast<uint4*>(sm + oWc + tc::sw128_off(L, 4 * wg + ch)) = make_uint4(wc[4 * ch], wc[4 * ch + 1], wc[4 * ch + 2], wc[4 * ch + 3]);
+            for (int c = 0; c < 8; c += 2) {
+              float w[2];
+#pragma unroll
+              for (int e = 0; e < 2; ++e) {
+                const int u = 8 * g + c + e;
+                w[e] = tc::fast_exp2(lg[u] - mu_i);
+                if (!whole) w[e] = u >= lo && u < hi ? w[e] : 0.f;
+                wc[u] = fmaf(w[e], dS_i + x1[c + e] + x2[c + e], wc[u]);
+              }
+              const __nv_bfloat162 a = __floats2bfloat162_rn(w[0], w[1]);
+              ww[c / 2] = *reinterpret_cast<const uint32_t*>(&a);
+            }
+            *reinterpret_cast<uint4*>(sm + oW + tc::sw128_off(L, 4 * wg + g)) = make_uint4(ww[0], ww[1], ww[2], ww[3]);
           }
         }
         if (k > 0) ph2 ^= 1;
@@ -236,12 +256,6 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
           for (int ks = 0; ks < TI / 16; ++ks)
             tc::mma_bf16_ss_warp(tbase + cDK, tc::smem_desc_sw128(aDka + ks * 16 * 128, TI * 128, 1024),
                             tc::smem_desc_sw128(aW + ks * 16 * 128, TI * 128, 1024), idesc, started || ks > 0);
-          if (dm.agg_grad) {
-#pragma unroll
-            for (int ks = 0; ks < TI / 16; ++ks)
-              tc::mma_bf16_ss_warp(tbase + cDK, tc::smem_desc_sw128(aQhi + ks * 16 * 128, TI * 128, 1024),
-                              tc::smem_desc_sw128(aWc + ks * 16 * 128, TI * 128, 1024), idesc, 1);
-          }
 #pragma unroll
           for (int ks = 0; ks < TI / 16; ++ks)
             tc::mma_bf16_ss_warp(tbase + cDV, tc::smem_desc_sw128(aDnu + ks * 16 * 128, TI * 128, 1024),
@@ -259,6 +273,36 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
         if (!tc::mbar_wait(&bar2, ph2)) ok = false;
         ph2 ^= 1;
         tc::fence_after_sync();
+        if (dm.agg_grad) {                                // dK^T += qbar^T (sum over the planes of w c), in the place of W
+          if (cw) {
+#pragma unroll
+            for (int ch = 0; ch < 4; ++ch) {
+              uint32_t x[4];
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                const __nv_bfloat162 a = __floats2bfloat162_rn(wc[8 * ch + 2 * e], wc[8 * ch + 2 * e + 1]);
+                x[e] = *reinterpret_cast<const uint32_t*>(&a);
+              }
+              *reinterpret_cast<uint4*>(sm + oW + tc::sw128_off(L, 4 * wg + ch)) = make_uint4(x[0], x[1], x[2], x[3]);
+            }
+          }
+          tc::fence_async_smem();
+          tc::fence_before_sync();
+          __syncthreads();
+          if (warp == ISSUER / 32) {
+            tc::fence_after_sync();
+            const uint32_t idesc = tc::idesc_bf16(128, NU, 1, 1);
+#pragma unroll
+            for (int ks = 0; ks < TI / 16; ++ks)
+              tc::mma_bf16_ss_warp(tbase + cDK, tc::smem_desc_sw128(aQhi + ks * 16 * 128, TI * 128, 1024),
+                                   tc::smem_desc_sw128(aW + ks * 16 * 128, TI * 128, 1024), idesc, 1);
+            tc::mma_commit_warp(&bar2);
+          }
+          __syncwarp();
+          if (!tc::mbar_wait(&bar2, ph2)) ok = false;
+          ph2 ^= 1;
+          tc::fence_after_sync();
+        }
       }
     }
     PCLK(5)
@@ -283,7 +327,7 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
   }
   tc::fence_before_sync();
   __syncthreads();
-  if (warp == 0) tc::tmem_dealloc(tbase, 512);
+  if (warp == 0) tc::tmem_dealloc(tbase, cols);
 #ifdef MUSE_PHASE_CLOCKS
   if (tid == 0 && blockIdx.x == 5 && blockIdx.y == 0) for (int k = 0; k < 8; ++k) status[56 + k] = (int)pc[k];
 #endif
