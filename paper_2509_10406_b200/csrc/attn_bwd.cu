@@ -672,7 +672,7 @@ __global__ void k_final_dkv(Dims dm, const int32_t* __restrict__ perm_k, const f
 int local_bwd_tc(const Dims& d, const void* Q, const void* K, const void* V, const void* dO, const float* LSE,
                  const float* delta, float* dQacc, float* dK_orig, float* dV_orig, int* status, cudaStream_t st);
 int ret_bwd_tc(const Dims& d, const void* Q, const void* dO, const void* Kp, const void* Vp, const float* LSE,
-               const float* delta, const int32_t* off_k, const int32_t* goff, const int32_t* pairs, void* dq_part,
+               const float* delta, const int32_t* off_k, const RetIndex& ri, void* dq_part,
                float* dK_perm, float* dV_perm, int* status, cudaStream_t st);
 
 bool far_bwd_tc_supported(const Dims& d, int dtype);
@@ -774,7 +774,7 @@ static int attn_bwd_t(const Dims& d, int dtype, const T* Q, const T* K, const T*
       rc = build_ret_index(d, sel, bsel, w.ret_scratch, &ri, st);
       if (rc != MUSE_OK) return rc;
       if (kTensor) {
-        rc = ret_bwd_tc(d, Q, dO, Kp, Vp, LSE, w.delta, off_k, ri.goff, ri.pairs, w.dq_part, w.dK_perm, w.dV_perm, w.status, st);
+        rc = ret_bwd_tc(d, Q, dO, Kp, Vp, LSE, w.delta, off_k, ri, w.dq_part, w.dK_perm, w.dV_perm, w.status, st);
         if (rc != MUSE_OK) return rc;
       } else {
         MUSE_CUDA_OK(cudaFuncSetAttribute(k_ret_bwd<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm4));

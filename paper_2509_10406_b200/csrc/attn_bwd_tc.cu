@@ -499,21 +499,21 @@ k_ret_bwd_dkdv_tc(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ 
   } while (0)
 
 int ret_bwd_pairs_tc(const Dims& d, const void* Q, const void* dO, const void* Kp, const void* Vp, const float* LSE,
-                     const float* delta, const int32_t* off_k, const int32_t* goff, const int32_t* pairs, void* dq_part,
+                     const float* delta, const int32_t* off_k, const RetIndex& ri, void* dq_part,
                      float* dK_perm, float* dV_perm, int* status, cudaStream_t st);
 
 int ret_bwd_tc(const Dims& d, const void* Q, const void* dO, const void* Kp, const void* Vp, const float* LSE,
-               const float* delta, const int32_t* off_k, const int32_t* goff, const int32_t* pairs, void* dq_part,
+               const float* delta, const int32_t* off_k, const RetIndex& ri, void* dq_part,
                float* dK_perm, float* dV_perm, int* status, cudaStream_t st) {
   const int pq = d.B * d.Hq;
   if (!path_forced(kForceRetBwdSplit) || d.k2 > 0)
-    return ret_bwd_pairs_tc(d, Q, dO, Kp, Vp, LSE, delta, off_k, goff, pairs, dq_part, dK_perm, dV_perm, status, st);
+    return ret_bwd_pairs_tc(d, Q, dO, Kp, Vp, LSE, delta, off_k, ri, dq_part, dK_perm, dV_perm, status, st);
   prof_mark("k_ret_bwd_dkdv_tc", st);
   MUSE_TC_LAUNCH(k_ret_bwd_dkdv_tc, KeysSmem, kKeysThreads, dim3(d.Ck, d.SB * kRetSplit, pq), d, (const bf16*)Q, (const bf16*)dO, (const bf16*)Kp,
-                 (const bf16*)Vp, LSE, delta, off_k, goff, pairs, dK_perm, dV_perm, status);
+                 (const bf16*)Vp, LSE, delta, off_k, ri.goff, ri.pairs, dK_perm, dV_perm, status);
   prof_mark("k_ret_bwd_dq_tc", st);
   MUSE_TC_LAUNCH(k_ret_bwd_dq_tc, RowsSmem, kRowsThreads, dim3(d.Ck, d.SB * kRetSplitRows, pq), d, (const bf16*)Q, (const bf16*)dO, (const bf16*)Kp,
-                 (const bf16*)Vp, LSE, delta, off_k, goff, pairs, (bf16*)dq_part, status);
+                 (const bf16*)Vp, LSE, delta, off_k, ri.goff, ri.pairs, (bf16*)dq_part, status);
   return MUSE_OK;
 }
 

@@ -12,8 +12,7 @@ int local_fwd_tc(const Dims& d, const void* Q, const void* K, const void* V, flo
 bool far_fwd_tc_supported(const Dims& d, int dtype);
 int far_fwd_tc(const Dims& d, const SummPtrs& sp, const void* Q, const int32_t* off_q, const int32_t* perm_q,
                const int32_t* sel_in, int32_t* sel_out, float* o_far, float* lse_far, int* status, cudaStream_t st);
-int ret_fwd_tc(const Dims& d, const void* Q, const void* Kp, const void* Vp, const int32_t* off_k, const int32_t* goff,
-               const int32_t* pairs, void* o_part, float* l_part, int* status, cudaStream_t st);
+int ret_fwd_tc(const Dims& d, const void* Q, const void* Kp, const void* Vp, const int32_t* off_k, const RetIndex& ri, void* o_part, float* l_part, int* status, cudaStream_t st);
 bool block_select_q_supported(const Dims& d, int dtype);
 int block_select_q(const Dims& d, const void* Q, const int32_t* off_q, const int32_t* perm_q, const int32_t* sel, const SummPtrs& sp,
                    const int32_t* bsel_in, int32_t* bsel_out, float* o_near, float* lse_near, cudaStream_t st);
@@ -556,7 +555,7 @@ static int attn_fwd_t(const Dims& d, const T* Q, const T* K, const T* V, const i
         if (rc != MUSE_OK) return rc;
       }
       if (kTensor) {
-        rc = ret_fwd_tc(d, Q, Kp, Vp, off_k, ri.goff, ri.pairs, w.o_part, w.l_part, w.status, st);
+        rc = ret_fwd_tc(d, Q, Kp, Vp, off_k, ri, w.o_part, w.l_part, w.status, st);
         if (rc != MUSE_OK) return rc;
       } else {
         MUSE_CUDA_OK(cudaFuncSetAttribute(k_ret_fwd<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fl_smem));

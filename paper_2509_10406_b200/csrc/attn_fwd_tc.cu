@@ -226,22 +226,20 @@ k_ret_fwd_tc(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ Kp, c
   tc_teardown<D>(c, tid, status);
 }
 
-int ret_fwd_pairs_tc(const Dims& d, const void* Q, const void* Kp, const void* Vp, const int32_t* off_k, const int32_t* goff,
-                     const int32_t* pairs, void* o_part, float* l_part, int* status, cudaStream_t st);
+int ret_fwd_pairs_tc(const Dims& d, const void* Q, const void* Kp, const void* Vp, const int32_t* off_k, const RetIndex& ri, void* o_part, float* l_part, int* status, cudaStream_t st);
 
-int ret_fwd_tc(const Dims& d, const void* Q, const void* Kp, const void* Vp, const int32_t* off_k, const int32_t* goff,
-               const int32_t* pairs, void* o_part, float* l_part, int* status, cudaStream_t st) {
+int ret_fwd_tc(const Dims& d, const void* Q, const void* Kp, const void* Vp, const int32_t* off_k, const RetIndex& ri, void* o_part, float* l_part, int* status, cudaStream_t st) {
   dim3 grid(d.Ck, d.SB * kRetFwdSplit, d.B * d.Hq);
   const int min_keys = 0;
   if (!path_forced(kForceRetFwdStream) || d.k2 > 0)           // (block selection exists in the pair kernel only)
-    return ret_fwd_pairs_tc(d, Q, Kp, Vp, off_k, goff, pairs, o_part, l_part, status, st);
+    return ret_fwd_pairs_tc(d, Q, Kp, Vp, off_k, ri, o_part, l_part, status, st);
   prof_mark("k_ret_fwd_tc", st);
   if (d.D == 128) {
     MUSE_CUDA_OK(cudaFuncSetAttribute(k_ret_fwd_tc<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdTcSmem<128>::total));
-    k_ret_fwd_tc<128><<<grid, 128, FwdTcSmem<128>::total, st>>>(d, (const bf16*)Q, (const bf16*)Kp, (const bf16*)Vp, off_k, goff, pairs, (bf16*)o_part, l_part, min_keys, status);
+    k_ret_fwd_tc<128><<<grid, 128, FwdTcSmem<128>::total, st>>>(d, (const bf16*)Q, (const bf16*)Kp, (const bf16*)Vp, off_k, ri.goff, ri.pairs, (bf16*)o_part, l_part, min_keys, status);
   } else {
     MUSE_CUDA_OK(cudaFuncSetAttribute(k_ret_fwd_tc<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, FwdTcSmem<64>::total));
-    k_ret_fwd_tc<64><<<grid, 128, FwdTcSmem<64>::total, st>>>(d, (const bf16*)Q, (const bf16*)Kp, (const bf16*)Vp, off_k, goff, pairs, (bf16*)o_part, l_part, min_keys, status);
+    k_ret_fwd_tc<64><<<grid, 128, FwdTcSmem<64>::total, st>>>(d, (const bf16*)Q, (const bf16*)Kp, (const bf16*)Vp, off_k, ri.goff, ri.pairs, (bf16*)o_part, l_part, min_keys, status);
   }
   MUSE_LAUNCH_OK();
   return MUSE_OK;

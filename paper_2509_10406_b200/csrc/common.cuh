@@ -331,7 +331,10 @@ size_t attn_bwd_ws_bytes(const Dims& d, int dtype);
 
 // retrieval inverse index, shared by forward and backward: groups the (query, slot) pairs by
 // (query block - 1, key cluster).  pair id = t * m + slot.
-struct RetIndex { int32_t* goff; int32_t* pairs; };
+// The tensor-core kernels take the pairs of a group (a key cluster, or a bucket) in shares of `share` tiles of 128: items, for each head,
+// lists (group, share | shares << 16).
+constexpr int kRetTile = 128, kMinShare = 4, kMaxShare = 16;
+struct RetIndex { int32_t* goff; int32_t* pairs; int2* items; int32_t* nitems; int cap, share; };
 size_t ret_index_elems(const Dims& d);     // int32 elements per query head
 // bsel != nullptr (k2 > 0): groups are the (cluster, chosen block) buckets, pair id = (t * m + slot) * k2 + e
 int build_ret_index(const Dims& d, const int32_t* sel, const int32_t* bsel, int32_t* scratch, RetIndex* out, cudaStream_t st);

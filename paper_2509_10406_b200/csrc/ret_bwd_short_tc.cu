@@ -28,7 +28,6 @@ typedef __nv_bfloat16 bf16;
 namespace rs {
 constexpr int kPairs = 128, kKeys = 64;
 constexpr int kRowWarps = 4, kIssuerWarp0 = 8, kGatherWarp0 = 10, kGather = 128, kThreads = (kGatherWarp0 + 2 * kGather / 32) * 32;
-constexpr int kSplit = 4, kTilesPerCta = 16;                // a cluster with many pair tiles is shared by up to 4 CTAs
 constexpr int kOkCache = 72;
 constexpr float kLog2e = 1.4426950408889634f;
 template <int D> struct Lay {
@@ -57,7 +56,7 @@ template <int D>
 __global__ void __launch_bounds__(rs::kThreads, 1)
 k_ret_bwd_sweeps(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ dO, const bf16* __restrict__ Kp,
                    const bf16* __restrict__ Vp, const float* __restrict__ LSE, const float* __restrict__ delta,
-                   const int32_t* __restrict__ off_k, const int32_t* __restrict__ goff, const int32_t* __restrict__ pairs,
+                   const int32_t* __restrict__ off_k, const __grid_constant__ RetIndex ri,
                    bf16* __restrict__ dq_part, float* __restrict__ dK_perm, float* __restrict__ dV_perm, int* __restrict__ status) {
   using namespace rs;
   typedef Lay<D> LY;
@@ -71,17 +70,18 @@ k_ret_bwd_sweeps(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ d
   // With spatial block selection (k2 > 0) the CTA owns one BUCKET (cluster j, block bb): its pairs are the (query, slot,
   // chosen block) triples that chose the block, and every one of them sees the whole bucket (as in the forward kernel).
   const bool bucket = dm.k2 > 0;
-  const int j = bucket ? blockIdx.x / dm.SB : blockIdx.x, bb = bucket ? blockIdx.x % dm.SB : 0, sub = blockIdx.y, pq = blockIdx.z;
+  const int pq = blockIdx.y;
+  if ((int)blockIdx.x >= ri.nitems[pq]) return;
+  const int2 item = ri.items[(size_t)pq * ri.cap + blockIdx.x];               // group, share of its tiles (dealt round-robin)
+  const int j = bucket ? item.x / dm.SB : item.x, bb = bucket ? item.x % dm.SB : 0, sub = item.y & 0xffff, nsub = item.y >> 16;
   const int mk = dm.m * (bucket ? dm.k2 : 1);               // partial dQ rows per query
   const int b_ = pq / dm.Hq, h = pq % dm.Hq, pk = b_ * dm.Hkv + dm.hm.g[h];
   const int ngroups = dm.SB * dm.Ck;
-  const int32_t* go = goff + (size_t)pq * (ngroups + 1) + (size_t)j * dm.SB + bb;   // the group's pairs: plane pl is [go[pl], go[pl + 1])
+  const int32_t* go = ri.goff + (size_t)pq * (ngroups + 1) + (size_t)j * dm.SB + bb;   // the group's pairs: plane pl is [go[pl], go[pl + 1])
   const int g0 = go[0], g1 = go[bucket ? 1 : dm.SB];
   const int ntiles = (g1 - g0 + kPairs - 1) / kPairs;
-  const int nsub = min(kSplit, max(1, ntiles / kTilesPerCta));            // tiles are dealt round-robin to nsub CTAs
   const int32_t* okg = off_k + (size_t)pk * (dm.Ck * dm.S + 1) + (size_t)j * dm.S;   // okg[b]: first key of bucket (j, b)
   const int k0 = okg[bb], kall = (bucket ? okg[bb + 1] : okg[dm.SB]) - k0;   // keys that some pair of the group sees
-  if (ntiles == 0 || sub >= nsub) return;
   if (tc::smem_u32(sm) & 1023u) {                           // the tiles fill the whole dynamic allocation: no room to realign
     if (tid == 0) report_status(status, MUSE_STATUS_BWD_TIMEOUT);
     return;
@@ -104,7 +104,7 @@ k_ret_bwd_sweeps(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ d
   const bf16* dOb = dO + (size_t)pq * dm.N * D;
   const bf16* Kb = Kp + ((size_t)pk * dm.N + k0) * D;
   const bf16* Vb = Vp + ((size_t)pk * dm.N + k0) * D;
-  const int32_t* pr = pairs + (size_t)pq * dm.N * mk;
+  const int32_t* pr = ri.pairs + (size_t)pq * dm.N * mk;
   const size_t pbase = (size_t)pq * dm.N * mk;
   // role of this warp: half v, and row / issuing / gather warp
   const bool roww = warp < 2 * kRowWarps, issw = warp >= kIssuerWarp0 && warp < kIssuerWarp0 + 2, gatw = warp >= kGatherWarp0;
@@ -394,18 +394,18 @@ k_ret_bwd_sweeps(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ d
 }
 
 int ret_bwd_short_tc(const Dims& d, const void* Q, const void* dO, const void* Kp, const void* Vp, const float* LSE,
-                     const float* delta, const int32_t* off_k, const int32_t* goff, const int32_t* pairs, void* dq_part,
+                     const float* delta, const int32_t* off_k, const RetIndex& ri, void* dq_part,
                      float* dK_perm, float* dV_perm, int* status, cudaStream_t st) {
   prof_mark("k_ret_bwd_pairs_tc", st);
-  const dim3 grid(d.k2 > 0 ? d.Ck * d.SB : d.Ck, rs::kSplit, d.B * d.Hq);      // one CTA (or a few) per key cluster, or per bucket
+  const dim3 grid(ri.cap, d.B * d.Hq);
   if (d.D == 128) {
     MUSE_CUDA_OK(cudaFuncSetAttribute(k_ret_bwd_sweeps<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, rs::Lay<128>::kSmem));
     k_ret_bwd_sweeps<128><<<grid, rs::kThreads, rs::Lay<128>::kSmem, st>>>(
-        d, (const bf16*)Q, (const bf16*)dO, (const bf16*)Kp, (const bf16*)Vp, LSE, delta, off_k, goff, pairs, (bf16*)dq_part, dK_perm, dV_perm, status);
+        d, (const bf16*)Q, (const bf16*)dO, (const bf16*)Kp, (const bf16*)Vp, LSE, delta, off_k, ri, (bf16*)dq_part, dK_perm, dV_perm, status);
   } else {
     MUSE_CUDA_OK(cudaFuncSetAttribute(k_ret_bwd_sweeps<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, rs::Lay<64>::kSmem));
     k_ret_bwd_sweeps<64><<<grid, rs::kThreads, rs::Lay<64>::kSmem, st>>>(
-        d, (const bf16*)Q, (const bf16*)dO, (const bf16*)Kp, (const bf16*)Vp, LSE, delta, off_k, goff, pairs, (bf16*)dq_part, dK_perm, dV_perm, status);
+        d, (const bf16*)Q, (const bf16*)dO, (const bf16*)Kp, (const bf16*)Vp, LSE, delta, off_k, ri, (bf16*)dq_part, dK_perm, dV_perm, status);
   }
   MUSE_LAUNCH_OK();
   return MUSE_OK;

@@ -27,7 +27,6 @@ int make_tmap_bf16_rows(void* out_map, const void* base, uint64_t rows, uint32_t
 
 namespace rb {
 constexpr int kM = 128, kN = 64;                           // resident rows; columns of a tile
-constexpr int kSplit = 4, kTilesPerCta = 16;               // a cluster with many 128-pair tiles is shared by up to 4 CTAs
 constexpr int kOkCache = 72;                               // bucket offsets of the cluster kept in shared memory (S + 1 <= 72)
 constexpr float kLog2e = 1.4426950408889634f;
 
@@ -46,18 +45,19 @@ struct Group {
   bool bucket;
   int j, bb, sub, pq, pk, mk, g0, g1, k0, kall, ntiles, nsub;
   const int32_t *go, *okg;
-  __device__ __forceinline__ Group(const Dims& dm, const int32_t* goff, const int32_t* off_k) {
+  __device__ __forceinline__ Group(const Dims& dm, const RetIndex& ri, const int32_t* off_k) {
     bucket = dm.k2 > 0;
-    j = bucket ? blockIdx.x / dm.SB : blockIdx.x; bb = bucket ? blockIdx.x % dm.SB : 0; sub = blockIdx.y; pq = blockIdx.z;
+    pq = blockIdx.y;
+    const int2 item = ri.items[(size_t)pq * ri.cap + blockIdx.x];             // group, share of its tiles (dealt round-robin)
+    j = bucket ? item.x / dm.SB : item.x; bb = bucket ? item.x % dm.SB : 0; sub = item.y & 0xffff; nsub = item.y >> 16;
     mk = dm.m * (bucket ? dm.k2 : 1);
     const int b_ = pq / dm.Hq, h = pq % dm.Hq;
     pk = b_ * dm.Hkv + dm.hm.g[h];
-    go = goff + (size_t)pq * (dm.SB * dm.Ck + 1) + (size_t)j * dm.SB + bb;      // plane pl's pairs: [go[pl], go[pl + 1])
+    go = ri.goff + (size_t)pq * (dm.SB * dm.Ck + 1) + (size_t)j * dm.SB + bb;      // plane pl's pairs: [go[pl], go[pl + 1])
     g0 = go[0]; g1 = go[bucket ? 1 : dm.SB];
     okg = off_k + (size_t)pk * (dm.Ck * dm.S + 1) + (size_t)j * dm.S;           // okg[b]: first key of bucket (j, b)
     k0 = okg[bb]; kall = (bucket ? okg[bb + 1] : okg[dm.SB]) - k0;              // keys that some pair of the group sees
     ntiles = (g1 - g0 + kM - 1) / kM;
-    nsub = min(kSplit, max(1, ntiles / kTilesPerCta));
   }
 };
 }  // namespace rb
@@ -82,7 +82,7 @@ template <int D>
 __global__ void __launch_bounds__(rk::Lay<D>::kThreads, 1)
 k_ret_bwd_dkdv(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v, const bf16* __restrict__ Q,
                const bf16* __restrict__ dO, const float* __restrict__ LSE, const float* __restrict__ delta, const int32_t* __restrict__ off_k,
-               const int32_t* __restrict__ goff, const int32_t* __restrict__ pairs, float* __restrict__ dK_perm, float* __restrict__ dV_perm,
+               const __grid_constant__ RetIndex ri, float* __restrict__ dK_perm, float* __restrict__ dV_perm,
                int* __restrict__ status) {
   using namespace rk;
   typedef Lay<D> LY;
@@ -94,8 +94,9 @@ k_ret_bwd_dkdv(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_c
   __shared__ int32_t ok_s[kOkCache], tok_s[4][kN];
   __shared__ __align__(16) float Ls[NS][kN], ds[NS][kN];
   __shared__ __align__(16) int vs[NS][kN];                  // keys each pair of the tile sees, counted from the cluster's first
-  const Group gr(dm, goff, off_k);
-  if (gr.ntiles == 0 || gr.sub >= gr.nsub || gr.kall <= 0) return;
+  if ((int)blockIdx.x >= ri.nitems[blockIdx.y]) return;
+  const Group gr(dm, ri, off_k);
+  if (gr.kall <= 0) return;
   const int tid = threadIdx.x, warp = tc::warp_index(), lane = tid & 31;
   unsigned char* sm = sm_raw + ((1024u - (tc::smem_u32(sm_raw) & 1023u)) & 1023u);
   const int32_t* ok = dm.S + 1 <= kOkCache ? ok_s : gr.okg;
@@ -125,7 +126,7 @@ k_ret_bwd_dkdv(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_c
     }
     return lo + ((gr.sub - lo % gr.nsub) + gr.nsub) % gr.nsub;
   };
-  const int32_t* pr = pairs + (size_t)gr.pq * dm.N * gr.mk;
+  const int32_t* pr = ri.pairs + (size_t)gr.pq * dm.N * gr.mk;
 
   if (warp > MW + 1) {                                     // ---- gather of the Q and dO rows
     const int g = tid - (MW + 2) * 32, ck = g % CPR;
@@ -339,7 +340,7 @@ template <int D>
 __global__ void __launch_bounds__(rq::Lay<D>::kThreads, 1)
 k_ret_bwd_dq(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v, const bf16* __restrict__ Q,
              const bf16* __restrict__ dO, const float* __restrict__ LSE, const float* __restrict__ delta, const int32_t* __restrict__ off_k,
-             const int32_t* __restrict__ goff, const int32_t* __restrict__ pairs, bf16* __restrict__ dq_part, int* __restrict__ status) {
+             const __grid_constant__ RetIndex ri, bf16* __restrict__ dq_part, int* __restrict__ status) {
   using namespace rq;
   typedef Lay<D> LY;
   constexpr int kRow = LY::kRow, kCol = LY::kCol, NW = LY::NW, NSK = LY::NSK, NSV = LY::NSV, G = D / 64, CPR = D / 8;
@@ -349,8 +350,9 @@ k_ret_bwd_dq(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_con
   __shared__ uint32_t tbase_s;
   __shared__ int32_t ok_s[kOkCache], tok_s[2][kM], pid_s[2][kM], vs[2][kM], T_s[2];
   __shared__ float Ls[2][kM], ds[2][kM];
-  const Group gr(dm, goff, off_k);
-  if (gr.ntiles == 0 || gr.sub >= gr.nsub) return;
+  if ((int)blockIdx.x >= ri.nitems[blockIdx.y]) return;
+  const Group gr(dm, ri, off_k);
+  if (gr.ntiles == 0) return;
   const int tid = threadIdx.x, warp = tc::warp_index(), lane = tid & 31;
   unsigned char* sm = sm_raw + ((1024u - (tc::smem_u32(sm_raw) & 1023u)) & 1023u);
   const int32_t* ok = dm.S + 1 <= kOkCache ? ok_s : gr.okg;
@@ -373,7 +375,7 @@ k_ret_bwd_dq(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_con
   const uint32_t tbase = tbase_s;
   bool ok_ = true;
   auto wait = [&](uint64_t* bar, uint32_t parity) { if (ok_ && !tc::mbar_wait(bar, parity)) ok_ = false; };
-  const int32_t* pr = pairs + (size_t)gr.pq * dm.N * gr.mk;
+  const int32_t* pr = ri.pairs + (size_t)gr.pq * dm.N * gr.mk;
   auto visible = [&](int tok) { return tok < 0 ? 0 : gr.bucket ? max(gr.kall, 0) : max(0, ok[dm.causal ? tok / dm.Bs : 1] - gr.k0); };
   auto ld_pid = [&](int at) {
     const int id = at < gr.g1 ? __ldg(pr + at) : -1;
@@ -595,7 +597,7 @@ k_ret_bwd_dq(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_con
 
 template <int D>
 static int ret_bwd_d(const Dims& d, const void* Q, const void* dO, const void* Kp, const void* Vp, const float* LSE, const float* delta,
-                     const int32_t* off_k, const int32_t* goff, const int32_t* pairs, void* dq_part, float* dK_perm, float* dV_perm, int* status,
+                     const int32_t* off_k, const RetIndex& ri, void* dq_part, float* dK_perm, float* dV_perm, int* status,
                      cudaStream_t st) {
   const uint64_t rk = (uint64_t)d.B * d.Hkv * d.N;
   CUtensorMap k[2], v[2];                                  // boxes of 128 keys (resident) and of 64 (streamed)
@@ -603,22 +605,22 @@ static int ret_bwd_d(const Dims& d, const void* Q, const void* dO, const void* K
     MUSE_RC(make_tmap_bf16_rows(&k[i], Kp, rk, D, i == 0 ? rb::kM : rb::kN));
     MUSE_RC(make_tmap_bf16_rows(&v[i], Vp, rk, D, i == 0 ? rb::kM : rb::kN));
   }
-  const dim3 grid(d.k2 > 0 ? d.Ck * d.SB : d.Ck, rb::kSplit, d.B * d.Hq);      // one CTA (or a few) per key cluster, or per bucket
+  const dim3 grid(ri.cap, d.B * d.Hq);
   prof_mark("k_ret_bwd_pairs_tc", st);
   MUSE_CUDA_OK(cudaFuncSetAttribute(k_ret_bwd_dkdv<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, rk::Lay<D>::total));
-  k_ret_bwd_dkdv<D><<<grid, rk::Lay<D>::kThreads, rk::Lay<D>::total, st>>>(d, k[0], v[0], (const bf16*)Q, (const bf16*)dO, LSE, delta, off_k, goff, pairs,
+  k_ret_bwd_dkdv<D><<<grid, rk::Lay<D>::kThreads, rk::Lay<D>::total, st>>>(d, k[0], v[0], (const bf16*)Q, (const bf16*)dO, LSE, delta, off_k, ri,
                                                                        dK_perm, dV_perm, status);
   MUSE_LAUNCH_OK();
   prof_mark("k_ret_bwd_dq", st);
   MUSE_CUDA_OK(cudaFuncSetAttribute(k_ret_bwd_dq<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, rq::Lay<D>::total));
-  k_ret_bwd_dq<D><<<grid, rq::Lay<D>::kThreads, rq::Lay<D>::total, st>>>(d, k[1], v[1], (const bf16*)Q, (const bf16*)dO, LSE, delta, off_k, goff, pairs,
+  k_ret_bwd_dq<D><<<grid, rq::Lay<D>::kThreads, rq::Lay<D>::total, st>>>(d, k[1], v[1], (const bf16*)Q, (const bf16*)dO, LSE, delta, off_k, ri,
                                                                      (bf16*)dq_part, status);
   MUSE_LAUNCH_OK();
   return MUSE_OK;
 }
 
 int ret_bwd_short_tc(const Dims& d, const void* Q, const void* dO, const void* Kp, const void* Vp, const float* LSE,
-                     const float* delta, const int32_t* off_k, const int32_t* goff, const int32_t* pairs, void* dq_part,
+                     const float* delta, const int32_t* off_k, const RetIndex& ri, void* dq_part,
                      float* dK_perm, float* dV_perm, int* status, cudaStream_t st);
 
 // Two kernels, or one with five products per tile?  By the mean number of keys of a cluster: the fused kernel gathers a pair's
@@ -627,12 +629,12 @@ int ret_bwd_short_tc(const Dims& d, const void* Q, const void* dO, const void* K
 //   D = 64:   64 keys 566 | 311 + 569,  128 keys 469 | 233 + 293,  256 keys 1331 | 543 + 501,  512 keys 16860 | 5549 + 3808
 //   D = 128:  64 keys 850 | 484 + 438,  128 keys 684 | 353 + 261,  256 keys 1875 | 802 + 514
 int ret_bwd_pairs_tc(const Dims& d, const void* Q, const void* dO, const void* Kp, const void* Vp, const float* LSE,
-                     const float* delta, const int32_t* off_k, const int32_t* goff, const int32_t* pairs, void* dq_part,
+                     const float* delta, const int32_t* off_k, const RetIndex& ri, void* dq_part,
                      float* dK_perm, float* dV_perm, int* status, cudaStream_t st) {
   if (d.N / d.Ck < (d.D == 128 ? 128 : 256))
-    return ret_bwd_short_tc(d, Q, dO, Kp, Vp, LSE, delta, off_k, goff, pairs, dq_part, dK_perm, dV_perm, status, st);
-  return d.D == 128 ? ret_bwd_d<128>(d, Q, dO, Kp, Vp, LSE, delta, off_k, goff, pairs, dq_part, dK_perm, dV_perm, status, st)
-                    : ret_bwd_d<64>(d, Q, dO, Kp, Vp, LSE, delta, off_k, goff, pairs, dq_part, dK_perm, dV_perm, status, st);
+    return ret_bwd_short_tc(d, Q, dO, Kp, Vp, LSE, delta, off_k, ri, dq_part, dK_perm, dV_perm, status, st);
+  return d.D == 128 ? ret_bwd_d<128>(d, Q, dO, Kp, Vp, LSE, delta, off_k, ri, dq_part, dK_perm, dV_perm, status, st)
+                    : ret_bwd_d<64>(d, Q, dO, Kp, Vp, LSE, delta, off_k, ri, dq_part, dK_perm, dV_perm, status, st);
 }
 
 }  // namespace muse

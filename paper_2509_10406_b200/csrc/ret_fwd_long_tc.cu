@@ -22,7 +22,6 @@ int make_tmap_bf16_rows(void* out_map, const void* base, uint64_t rows, uint32_t
 
 namespace rl {
 constexpr int kPairs = 128, kKeys = 128;
-constexpr int kSplit = 4, kUnitsPerCta = 8;                // a cluster with many units is shared by up to 4 CTAs
 constexpr int kOkCache = 72;                               // bucket offsets of the cluster kept in shared memory (S + 1 <= 72)
 template <int D> struct Lay {
   static constexpr int kTile = 128 * D * 2, NS = D == 128 ? 2 : 3, NB = D == 128 ? 2 : 3, NQ = D == 128 ? 3 : 4;
@@ -47,8 +46,8 @@ __device__ __forceinline__ bool bar_or(int id, int count, bool p) {
 template <int D>
 __global__ void __launch_bounds__(rl::Lay<D>::kThreads, 1)
 k_ret_fwd_long(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v, const bf16* __restrict__ Q,
-               const int32_t* __restrict__ off_k, const int32_t* __restrict__ goff, const int32_t* __restrict__ pairs,
-               bf16* __restrict__ o_part, float* __restrict__ l_part, int* __restrict__ status) {
+               const int32_t* __restrict__ off_k, const __grid_constant__ RetIndex ri, bf16* __restrict__ o_part, float* __restrict__ l_part,
+               int* __restrict__ status) {
   using namespace rl;
   typedef Lay<D> LY;
   constexpr int kTile = LY::kTile, NS = LY::NS, NB = LY::NB, NQ = LY::NQ, H = LY::H, kSoft = LY::kSoft, MW = kSoft / 32, G = D / 64, CPR = D / 8;
@@ -59,11 +58,12 @@ k_ret_fwd_long(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_c
   __shared__ int32_t ok_s[kOkCache], tok_s[kPairs];
   __shared__ float mx_s[2][2][kPairs];
   const int tid = threadIdx.x, warp = tc::warp_index(), lane = tid & 31;
-  const int j = blockIdx.x, sub = blockIdx.y, pq = blockIdx.z, b_ = pq / dm.Hq, h = pq % dm.Hq, pk = b_ * dm.Hkv + dm.hm.g[h];
-  const int32_t* go = goff + (size_t)pq * (dm.SB * dm.Ck + 1) + (size_t)j * dm.SB;      // plane pl's pairs: [go[pl], go[pl + 1])
+  const int pq = blockIdx.y;
+  if ((int)blockIdx.x >= ri.nitems[pq]) return;
+  const int2 item = ri.items[(size_t)pq * ri.cap + blockIdx.x];              // key cluster, share of its units (dealt round-robin)
+  const int j = item.x, sub = item.y & 0xffff, nsub = item.y >> 16, b_ = pq / dm.Hq, h = pq % dm.Hq, pk = b_ * dm.Hkv + dm.hm.g[h];
+  const int32_t* go = ri.goff + (size_t)pq * (dm.SB * dm.Ck + 1) + (size_t)j * dm.SB;      // plane pl's pairs: [go[pl], go[pl + 1])
   const int g0 = go[0], g1 = go[dm.SB], ntiles = (g1 - g0 + kPairs - 1) / kPairs, nunits = (ntiles + 1) / 2;
-  const int nsub = min(kSplit, max(1, nunits / kUnitsPerCta));            // units are dealt round-robin to nsub CTAs
-  if (ntiles == 0 || sub >= nsub) return;
   const int32_t* okg = off_k + (size_t)pk * (dm.Ck * dm.S + 1) + (size_t)j * dm.S;      // okg[b]: first key of bucket (j, b)
   const int k0 = okg[0];
   const int32_t* ok = dm.S + 1 <= kOkCache ? ok_s : okg;
@@ -88,7 +88,7 @@ k_ret_fwd_long(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_c
   const uint32_t tbase = tbase_s;
   bool ok_ = true;                                         // false once a bounded wait ran out (every role still walks all its units)
   auto wait = [&](uint64_t* bar, uint32_t parity) { if (ok_ && !tc::mbar_wait(bar, parity)) ok_ = false; };
-  const int32_t* pr = pairs + (size_t)pq * dm.N * dm.m + g0;
+  const int32_t* pr = ri.pairs + (size_t)pq * dm.N * dm.m + g0;
   const int np = g1 - g0;
   const size_t pbase = (size_t)pq * dm.N * dm.m;
   auto ld_pid = [&](int at) {                              // the pair at position `at` of the cluster's list
@@ -356,23 +356,20 @@ k_ret_fwd_long(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_c
 }
 
 template <int D>
-static int ret_fwd_long_d(const Dims& d, const void* Q, const void* Kp, const void* Vp, const int32_t* off_k, const int32_t* goff, const int32_t* pairs,
-                          void* o_part, float* l_part, int* status, cudaStream_t st) {
+static int ret_fwd_long_d(const Dims& d, const void* Q, const void* Kp, const void* Vp, const int32_t* off_k, const RetIndex& ri, void* o_part, float* l_part, int* status, cudaStream_t st) {
   CUtensorMap k, v;
   MUSE_RC(make_tmap_bf16_rows(&k, Kp, (uint64_t)d.B * d.Hkv * d.N, D, rl::kKeys));
   MUSE_RC(make_tmap_bf16_rows(&v, Vp, (uint64_t)d.B * d.Hkv * d.N, D, rl::kKeys));
   MUSE_CUDA_OK(cudaFuncSetAttribute(k_ret_fwd_long<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, rl::Lay<D>::total));
   prof_mark("k_ret_fwd_pairs_tc", st);
-  k_ret_fwd_long<D><<<dim3(d.Ck, rl::kSplit, d.B * d.Hq), rl::Lay<D>::kThreads, rl::Lay<D>::total, st>>>(d, k, v, (const bf16*)Q, off_k, goff, pairs,
-                                                                                                  (bf16*)o_part, l_part, status);
+  k_ret_fwd_long<D><<<dim3(ri.cap, d.B * d.Hq), rl::Lay<D>::kThreads, rl::Lay<D>::total, st>>>(d, k, v, (const bf16*)Q, off_k, ri, (bf16*)o_part, l_part, status);
   MUSE_LAUNCH_OK();
   return MUSE_OK;
 }
 
-int ret_fwd_long_tc(const Dims& d, const void* Q, const void* Kp, const void* Vp, const int32_t* off_k, const int32_t* goff,
-                    const int32_t* pairs, void* o_part, float* l_part, int* status, cudaStream_t st) {
-  return d.D == 128 ? ret_fwd_long_d<128>(d, Q, Kp, Vp, off_k, goff, pairs, o_part, l_part, status, st)
-                    : ret_fwd_long_d<64>(d, Q, Kp, Vp, off_k, goff, pairs, o_part, l_part, status, st);
+int ret_fwd_long_tc(const Dims& d, const void* Q, const void* Kp, const void* Vp, const int32_t* off_k, const RetIndex& ri, void* o_part, float* l_part, int* status, cudaStream_t st) {
+  return d.D == 128 ? ret_fwd_long_d<128>(d, Q, Kp, Vp, off_k, ri, o_part, l_part, status, st)
+                    : ret_fwd_long_d<64>(d, Q, Kp, Vp, off_k, ri, o_part, l_part, status, st);
 }
 
 }  // namespace muse

@@ -29,7 +29,6 @@ typedef __nv_bfloat16 bf16;
 namespace rf {
 constexpr int kRowThreads = 128, kIssuerWarp = 4, kGather0 = 160, kGather = 64, kThreads = kGather0 + kGather;
 constexpr int kPairs = 128, kKeys = 128;
-constexpr int kSplit = 4, kTilesPerCta = 8;                // a cluster with many pair tiles is shared by up to 4 CTAs
 constexpr int kOkCache = 72;                               // bucket offsets of the cluster kept in shared memory (S + 1 <= 72)
 
 template <int D> struct Smem {
@@ -49,8 +48,8 @@ __device__ __forceinline__ void cp_async16(void* smem_dst, const void* src, bool
 template <int D>
 __global__ void __launch_bounds__(rf::kThreads, 2)
 k_ret_fwd_pairs_tc(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ Kp, const bf16* __restrict__ Vp,
-                   const int32_t* __restrict__ off_k, const int32_t* __restrict__ goff, const int32_t* __restrict__ pairs,
-                   bf16* __restrict__ o_part, float* __restrict__ l_part, int* __restrict__ status) {
+                   const int32_t* __restrict__ off_k, const __grid_constant__ RetIndex ri, bf16* __restrict__ o_part,
+                   float* __restrict__ l_part, int* __restrict__ status) {
   using namespace rf;
   typedef Smem<D> SM;
   constexpr int CPR = D / 8;                               // 16-byte chunks per row
@@ -64,15 +63,16 @@ k_ret_fwd_pairs_tc(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__
   // keys of the earlier blocks).  With it (k2 > 0) the CTA owns one BUCKET (cluster, block bb): its pairs are the
   // (query, slot, chosen block) triples that chose this block, and every one of them sees the whole bucket.
   const bool bucket = dm.k2 > 0;
-  const int j = bucket ? blockIdx.x / dm.SB : blockIdx.x, bb = bucket ? blockIdx.x % dm.SB : 0, sub = blockIdx.y, pq = blockIdx.z;
+  const int pq = blockIdx.y;
+  if ((int)blockIdx.x >= ri.nitems[pq]) return;
+  const int2 item = ri.items[(size_t)pq * ri.cap + blockIdx.x];              // group, share of its tiles (dealt round-robin)
+  const int j = bucket ? item.x / dm.SB : item.x, bb = bucket ? item.x % dm.SB : 0, sub = item.y & 0xffff, nsub = item.y >> 16;
   const int mk = dm.m * (bucket ? dm.k2 : 1);              // partial results per query
   const int b_ = pq / dm.Hq, h = pq % dm.Hq, pk = b_ * dm.Hkv + dm.hm.g[h];
   const int ngroups = dm.SB * dm.Ck;
-  const int32_t* go = goff + (size_t)pq * (ngroups + 1) + (size_t)j * dm.SB + bb;   // the group's pairs: plane pl is [go[pl], go[pl + 1])
+  const int32_t* go = ri.goff + (size_t)pq * (ngroups + 1) + (size_t)j * dm.SB + bb;   // the group's pairs: plane pl is [go[pl], go[pl + 1])
   const int g0 = go[0], g1 = go[bucket ? 1 : dm.SB];
   const int ntiles = (g1 - g0 + kPairs - 1) / kPairs;
-  const int nsub = min(kSplit, max(1, ntiles / kTilesPerCta));           // tiles are dealt round-robin to nsub CTAs
-  if (ntiles == 0 || sub >= nsub) return;
   const int32_t* okg = off_k + (size_t)pk * (dm.Ck * dm.S + 1) + (size_t)j * dm.S;   // okg[b]: first key of bucket (j, b)
   const int k0 = okg[bb], kall = (bucket ? okg[bb + 1] : okg[dm.SB]) - k0;   // keys that some pair of the group sees
   const int32_t* ok = dm.S + 1 <= kOkCache ? ok_s : okg;
@@ -93,7 +93,7 @@ k_ret_fwd_pairs_tc(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__
   const bf16* Qb = Q + (size_t)pq * dm.N * D;
   const bf16* Kb = Kp + ((size_t)pk * dm.N + k0) * D;
   const bf16* Vb = Vp + ((size_t)pk * dm.N + k0) * D;
-  const int32_t* pr = pairs + (size_t)pq * dm.N * mk;
+  const int32_t* pr = ri.pairs + (size_t)pq * dm.N * mk;
   const size_t pbase = (size_t)pq * dm.N * mk;
   bool ok_ = true;                                         // false once a bounded wait ran out (every role still walks all its tiles)
   auto wait = [&](uint64_t* bar, uint32_t parity) { if (ok_ && !tc::mbar_wait(bar, parity)) ok_ = false; };
@@ -370,28 +370,24 @@ k_ret_fwd_pairs_tc(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__
   if (!ok_ && lane == 0) report_status(status, MUSE_STATUS_FWD_TIMEOUT);
 }
 
-int ret_fwd_long_tc(const Dims& d, const void* Q, const void* Kp, const void* Vp, const int32_t* off_k, const int32_t* goff,
-                    const int32_t* pairs, void* o_part, float* l_part, int* status, cudaStream_t st);
+int ret_fwd_long_tc(const Dims& d, const void* Q, const void* Kp, const void* Vp, const int32_t* off_k, const RetIndex& ri, void* o_part, float* l_part, int* status, cudaStream_t st);
 
 // The kernel here keeps 128 keys resident and two CTAs on an SM, but a cluster of more keys takes sweeps that gather the rows again and
 // read back the stored ones; the other streams the keys, and a tile of few keys pays for its longer pipeline.  Measured,
 // resident | streamed, us:
 //   D = 64:   64 keys 258 | 403,  128 keys 249 | 260 (sharp selections 219 | 275),  256 keys 727 | 544,  512 keys 7320 | 4470
 //   D = 128:  64 keys 408 | 506,  128 keys 366 | 319,  256 keys 993 | 665
-int ret_fwd_pairs_tc(const Dims& d, const void* Q, const void* Kp, const void* Vp, const int32_t* off_k, const int32_t* goff,
-                     const int32_t* pairs, void* o_part, float* l_part, int* status, cudaStream_t st) {
+int ret_fwd_pairs_tc(const Dims& d, const void* Q, const void* Kp, const void* Vp, const int32_t* off_k, const RetIndex& ri, void* o_part, float* l_part, int* status, cudaStream_t st) {
   if (d.k2 == 0 && d.N / d.Ck >= (d.D == 128 ? 128 : 256))             // mean keys of a cluster
-    return ret_fwd_long_tc(d, Q, Kp, Vp, off_k, goff, pairs, o_part, l_part, status, st);
-  const dim3 grid(d.k2 > 0 ? d.Ck * d.SB : d.Ck, rf::kSplit, d.B * d.Hq);     // one CTA (or a few) per key cluster, or per bucket
+    return ret_fwd_long_tc(d, Q, Kp, Vp, off_k, ri, o_part, l_part, status, st);
+  const dim3 grid(ri.cap, d.B * d.Hq);
   prof_mark("k_ret_fwd_pairs_tc", st);
   if (d.D == 128) {
     MUSE_CUDA_OK(cudaFuncSetAttribute(k_ret_fwd_pairs_tc<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, rf::Smem<128>::total));
-    k_ret_fwd_pairs_tc<128><<<grid, rf::kThreads, rf::Smem<128>::total, st>>>(d, (const bf16*)Q, (const bf16*)Kp, (const bf16*)Vp, off_k, goff, pairs,
-                                                                          (bf16*)o_part, l_part, status);
+    k_ret_fwd_pairs_tc<128><<<grid, rf::kThreads, rf::Smem<128>::total, st>>>(d, (const bf16*)Q, (const bf16*)Kp, (const bf16*)Vp, off_k, ri, (bf16*)o_part, l_part, status);
   } else {
     MUSE_CUDA_OK(cudaFuncSetAttribute(k_ret_fwd_pairs_tc<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, rf::Smem<64>::total));
-    k_ret_fwd_pairs_tc<64><<<grid, rf::kThreads, rf::Smem<64>::total, st>>>(d, (const bf16*)Q, (const bf16*)Kp, (const bf16*)Vp, off_k, goff, pairs,
-                                                                        (bf16*)o_part, l_part, status);
+    k_ret_fwd_pairs_tc<64><<<grid, rf::kThreads, rf::Smem<64>::total, st>>>(d, (const bf16*)Q, (const bf16*)Kp, (const bf16*)Vp, off_k, ri, (bf16*)o_part, l_part, status);
   }
   MUSE_LAUNCH_OK();
   return MUSE_OK;

@@ -5,7 +5,8 @@
 //
 // One launch: a head is one thread-block cluster, a CTA owns a stretch of its tokens.  Every CTA counts its pairs by key in
 // shared memory; the CTAs split the keys, read each other's counts through distributed shared memory and write back where
-// in the list each CTA's pairs of a key start; then every CTA goes over its pairs again and places them.
+// in the list each CTA's pairs of a key start; then every CTA goes over its pairs again and places them.  The first CTA also lists
+// the shares in which the tensor-core kernels take the groups.
 //
 // Bound by the scattered 4-byte stores of the last pass (a store per lane) and shared-memory atomics.  32 heads of 64k tokens,
 // 8 slots, 128 clusters, 8 blocks: 220 us; a memset, a counting kernel, a scan and a placing kernel that combined equal keys
@@ -19,7 +20,7 @@ namespace muse {
 
 constexpr int kRiThreads = 1024, kRiMaxCluster = 16, kRiMinPairs = 2048;
 
-struct RiArgs { const int32_t *sel, *bsel; int32_t *goff, *pairs; int nkeys; };
+struct RiArgs { const int32_t *sel, *bsel; RetIndex ri; int nkeys; };
 
 __global__ void __launch_bounds__(kRiThreads)
 k_ret_index(Dims d, const __grid_constant__ RiArgs g) {
@@ -59,7 +60,7 @@ k_ret_index(Dims d, const __grid_constant__ RiArgs g) {
   cluster.sync();
   // this CTA's share of the keys: totals over the CTAs, their exclusive prefix within the share
   const int kper = (nkeys + CL - 1) / CL, ka = min(nkeys, rank * kper), kb = min(nkeys, ka + kper);
-  int32_t* goff = g.goff + (size_t)pq * (nkeys + 1);
+  int32_t* goff = g.ri.goff + (size_t)pq * (nkeys + 1);
   int share = 0;
   for (int k = ka + tid; k < kb; k += kRiThreads)
     for (int c = 0; c < CL; ++c) share += cluster.map_shared_rank(hist, c)[k];
@@ -101,8 +102,28 @@ k_ret_index(Dims d, const __grid_constant__ RiArgs g) {
   }
   if (rank == CL - 1 && tid == 0) goff[nkeys] = carry;
   cluster.sync();
+  if (rank == 0) {                                         // the shares of every group's pairs (this CTA has the tokens of block 0, which have no pairs)
+    const int stride = g.bsel ? 1 : d.SB, G = nkeys / stride;
+    int2* items = g.ri.items + (size_t)pq * g.ri.cap;
+    int carry2 = 0;
+    for (int k0 = 0; k0 < G; k0 += kRiThreads) {
+      const int k = k0 + tid, np = k < G ? __ldcg(goff + (k + 1) * stride) - __ldcg(goff + k * stride) : 0;
+      const int tiles = (np + kRetTile - 1) / kRetTile, ns = min(32767, (tiles + g.ri.share - 1) / g.ri.share);
+      int inc = ns;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) { const int v = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += v; }
+      __syncthreads();
+      if (lane == 31) wsum[warp] = inc;
+      __syncthreads();
+      int at = carry2 + inc - ns;
+      for (int w = 0; w < 32; ++w) { const int v = wsum[w]; if (w < warp) at += v; carry2 += v; }
+      for (int s = 0; s < ns; ++s)
+        if (MUSE_IN_RANGE(at + s, g.ri.cap)) items[at + s] = make_int2(k, s | ns << 16);
+    }
+    if (tid == 0) g.ri.nitems[pq] = carry2;
+  }
   const size_t npairs = (size_t)d.N * d.m * ke;
-  int32_t* pairs = g.pairs + (size_t)pq * npairs;
+  int32_t* pairs = g.ri.pairs + (size_t)pq * npairs;
   for (int e0 = tid; e0 < n; e0 += U * kRiThreads) {
     int c[U];
 #pragma unroll
@@ -118,23 +139,34 @@ k_ret_index(Dims d, const __grid_constant__ RiArgs g) {
   }
 }
 
+static size_t up64(size_t x) { return (x + 63) & ~size_t(63); }
+static int item_cap(const Dims& d, int share) {
+  const int groups = d.k2 > 0 ? d.Ck * d.SB : d.Ck;
+  return (int)((long long)d.N * d.m * (d.k2 > 0 ? d.k2 : 1) / (kRetTile * share)) + groups;
+}
+
 size_t ret_index_elems(const Dims& d) {
-  // goff [SB*Ck+1] + pairs [N*m*max(k2,1)], each rounded up to 64 ints
-  auto up = [](size_t x) { return (x + 63) & ~size_t(63); };
-  return up((size_t)d.SB * d.Ck + 1) + up((size_t)d.N * d.m * (d.k2 > 0 ? d.k2 : 1));
+  // goff [SB*Ck+1] + pairs [N*m*max(k2,1)] + items (2 each) + their number, each rounded up to 64 ints
+  return up64((size_t)d.SB * d.Ck + 1) + up64((size_t)d.N * d.m * (d.k2 > 0 ? d.k2 : 1)) + up64(2 * (size_t)item_cap(d, kMinShare)) + 64;
 }
 
 int build_ret_index(const Dims& d, const int32_t* sel, const int32_t* bsel, int32_t* scratch, RetIndex* out, cudaStream_t st) {
-  auto up = [](size_t x) { return (x + 63) & ~size_t(63); };
-  const int pq = d.B * d.Hq, nkeys = d.SB * d.Ck;          // nkeys <= 32768
+  const int pq = d.B * d.Hq, nkeys = d.SB * d.Ck, mk = d.m * (bsel ? d.k2 : 1);        // nkeys <= 32768
+  // Shares of 16 tiles; fewer where that would leave SMs without work (selections crowd on few clusters: one may have all of a head's
+  // queries), not below 4 (a share loads its keys and adds its gradients once).
+  const long long tiles = (long long)d.N * mk * pq / kRetTile, want = tiles / (8 * sm_count());
+  out->share = (int)(want < kMinShare ? kMinShare : want > kMaxShare ? kMaxShare : want);
+  out->cap = item_cap(d, out->share);
   out->goff = scratch;                                     // (indexed with its natural stride, nkeys + 1)
-  out->pairs = scratch + (size_t)pq * up((size_t)nkeys + 1);
+  out->pairs = out->goff + (size_t)pq * up64((size_t)nkeys + 1);
+  out->items = (int2*)(out->pairs + (size_t)pq * up64((size_t)d.N * mk));
+  out->nitems = (int32_t*)(out->items + (size_t)pq * up64(2 * (size_t)item_cap(d, kMinShare)) / 2);
   if (d.m == 0 || nkeys == 0) return MUSE_OK;
   // CTAs of a head: enough to fill the chip, of 2048 pairs or more
   int cl = 1;
   while (cl < kRiMaxCluster && cl * pq < 2 * sm_count() && (long long)d.N * d.m >= 2LL * cl * kRiMinPairs) cl *= 2;
   const size_t smem = (size_t)nkeys * sizeof(int32_t);
-  const RiArgs g = {sel, bsel, out->goff, out->pairs, nkeys};
+  const RiArgs g = {sel, bsel, *out, nkeys};
   if (cl > 8) MUSE_CUDA_OK(cudaFuncSetAttribute(k_ret_index, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
   prof_mark("k_ret_index", st);
   return launch_pdl_cluster(k_ret_index, dim3(pq * cl), kRiThreads, smem, cl, st, d, g);
