@@ -333,7 +333,7 @@ size_t attn_bwd_ws_bytes(const Dims& d, int dtype);
 // (query block - 1, key cluster).  pair id = t * m + slot.
 // The tensor-core kernels take the pairs of a group (a key cluster, or a bucket) in shares of `share` tiles of 128: items, for each head,
 // lists (group, share | shares << 16).
-constexpr int kRetTile = 128, kMinShare = 4, kMaxShare = 16;
+constexpr int kRetTile = 128, kMinShare = 4, kMaxShare = 32;
 struct RetIndex { int32_t* goff; int32_t* pairs; int2* items; int32_t* nitems; int cap, share; };
 size_t ret_index_elems(const Dims& d);     // int32 elements per query head
 // bsel != nullptr (k2 > 0): groups are the (cluster, chosen block) buckets, pair id = (t * m + slot) * k2 + e

@@ -8,14 +8,14 @@
 // the consumed logits in tensor memory, from where they are A operands; one warp issues every product, one the TMA loads,
 // gather warps bring the scattered Q and dO rows by 16-byte asynchronous copies.
 //   k_ret_bwd_dkdv   128 keys resident, tiles of 64 pairs gathered:  S^T = K Q^T, dP^T = V dO^T;  dV += P^T dO, dK += G^T Q
-//   k_ret_bwd_dq     128 pairs gathered (two buffers), tiles of 64 keys by TMA:  S = Q K^T, dP = dO V^T;  dQ += G K
+//   k_ret_bwd_dq     128 pairs gathered (four buffers at D = 64, two at D = 128), tiles of 64 keys by TMA:  S = Q K^T, dP = dO V^T;  dQ += G K
 // A pair's rows are gathered once for dQ and once per 128 keys it sees for dK and dV, and its dQ row is written once.
 // (One kernel for all five products has to keep dK and dV of the keys at hand in tensor memory, so it takes 64 keys per
 // sweep: the rows were then gathered, and the stored dQ row read and rewritten, once per 64 keys.)
 //
 // Bound: the tensor cores where clusters are long (7 products, 784 + 588 cycles per 128 x 64 tile at D = 64), else the
 // gather of rows (23-26 B/clk per SM).  64 heads of two sequences of 64k tokens, D = 64, 512 keys per cluster, 8 slots:
-// 16.86 ms in one kernel with five products per tile (ret_bwd_short_tc.cu, which short clusters keep), 5.55 + 3.81 ms here.
+// 16.86 ms in one kernel with five products per tile (ret_bwd_short_tc.cu, which short clusters keep), 5.41 + 3.61 ms here.
 #include <cuda.h>
 #include "common.cuh"
 #include "tc05.cuh"
@@ -328,12 +328,12 @@ namespace rq {
 using namespace rb;
 template <int D> struct Lay {
   static constexpr int kRow = kM * D * 2, kCol = kN * D * 2;
-  static constexpr int NW = D == 128 ? 2 : 3, NSK = D == 128 ? 3 : 5, NSV = D == 128 ? 2 : 4, kGather = D == 128 ? 256 : 128;
-  static constexpr int oQ = 0, oO = 2 * kRow, oK = 4 * kRow, oV = oK + NSK * kCol, total = oV + NSV * kCol + 1024;   // Q, dO: two buffers each
+  static constexpr int NW = D == 128 ? 2 : 3, NSK = D == 128 ? 3 : 5, NSV = D == 128 ? 2 : 4, NQ = D == 128 ? 2 : 4, kGather = D == 128 ? 256 : 128;
+  static constexpr int oQ = 0, oO = NQ * kRow, oK = 2 * NQ * kRow, oV = oK + NSK * kCol, total = oV + NSV * kCol + 1024;   // Q, dO: NQ buffers each
   static constexpr int kThreads = NW * 128 + 128 + 64 + kGather;                     // + an epilogue warpgroup
   static constexpr uint32_t cAcc = NW * 2 * kN;            // two accumulators follow
 };
-struct Bars { uint64_t q_full[2], q_empty[2], k_full[5], k_empty[5], v_full[4], v_empty[4], s_full[3], ready[3], acc_done[2], acc_free[2]; };
+struct Bars { uint64_t q_full[4], q_empty[4], k_full[5], k_empty[5], v_full[4], v_empty[4], s_full[3], ready[3], acc_done[2], acc_free[2]; };
 }  // namespace rq
 
 template <int D>
@@ -343,13 +343,13 @@ k_ret_bwd_dq(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_con
              const __grid_constant__ RetIndex ri, bf16* __restrict__ dq_part, int* __restrict__ status) {
   using namespace rq;
   typedef Lay<D> LY;
-  constexpr int kRow = LY::kRow, kCol = LY::kCol, NW = LY::NW, NSK = LY::NSK, NSV = LY::NSV, G = D / 64, CPR = D / 8;
+  constexpr int kRow = LY::kRow, kCol = LY::kCol, NW = LY::NW, NSK = LY::NSK, NSV = LY::NSV, NQ = LY::NQ, G = D / 64, CPR = D / 8;
   constexpr int EW = NW * 4, MW = EW + 4, kReaders = 128 * (NW + 1);         // epilogue warps, MMA warp; threads that read a tile's scalars
   extern __shared__ __align__(1024) unsigned char sm_raw[];
   __shared__ Bars bars;
   __shared__ uint32_t tbase_s;
-  __shared__ int32_t ok_s[kOkCache], tok_s[2][kM], pid_s[2][kM], vs[2][kM], T_s[2];
-  __shared__ float Ls[2][kM], ds[2][kM];
+  __shared__ int32_t ok_s[kOkCache], tok_s[NQ][kM], pid_s[NQ][kM], vs[NQ][kM], T_s[NQ];
+  __shared__ float Ls[NQ][kM], ds[NQ][kM];
   if ((int)blockIdx.x >= ri.nitems[blockIdx.y]) return;
   const Group gr(dm, ri, off_k);
   if (gr.ntiles == 0) return;
@@ -360,8 +360,8 @@ k_ret_bwd_dq(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_con
     for (int b = tid; b <= dm.S; b += LY::kThreads) ok_s[b] = gr.okg[b];
   if (warp == MW) tc::tmem_alloc(&tbase_s, 512);
   if (tid == 0) {
+    for (int b = 0; b < NQ; ++b) { tc::mbar_init(&bars.q_full[b], LY::kGather); tc::mbar_init(&bars.q_empty[b], 1 + kReaders); }
     for (int b = 0; b < 2; ++b) {
-      tc::mbar_init(&bars.q_full[b], LY::kGather); tc::mbar_init(&bars.q_empty[b], 1 + kReaders);
       tc::mbar_init(&bars.acc_done[b], 1); tc::mbar_init(&bars.acc_free[b], 128);
     }
     for (int s = 0; s < NSK; ++s) { tc::mbar_init(&bars.k_full[s], 1); tc::mbar_init(&bars.k_empty[s], 1); }
@@ -391,12 +391,17 @@ k_ret_bwd_dq(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_con
     const float* Lp = LSE + (size_t)gr.pq * dm.N;
     const float* dp = delta + (size_t)gr.pq * dm.N;
     int pid = g < kM ? ld_pid(gr.g0 + gr.sub * kM + g) : -1;
+    int pending = 0;                                       // tiles whose copies have been issued but not announced
+    auto publish = [&](int k) { tc::fence_async_smem(); tc::mbar_arrive(&bars.q_full[k % NQ]); };
     for (int i = 0; i < cnt; ++i) {
-      const int b = i & 1, at = gr.g0 + (gr.sub + i * gr.nsub) * kM;
+      const int b = i % NQ, at = gr.g0 + (gr.sub + i * gr.nsub) * kM;
       const int pid_n = g < kM && i + 1 < cnt ? ld_pid(at + gr.nsub * kM + g) : -1;
       const int tok = pid >= 0 ? pid / gr.mk : -1;
       const float L = tok >= 0 ? Lp[tok] * kLog2e : 0.f, d_ = tok >= 0 ? dp[tok] : 0.f;
-      wait(&bars.q_empty[b], ((i >> 1) & 1) ^ 1);
+      if (!tc::mbar_test(&bars.q_empty[b], ((i / NQ) & 1) ^ 1)) {          // no free buffer: announce what is there before waiting
+        if (pending > 0) { asm volatile("cp.async.wait_group 0;" ::: "memory"); publish(i - 1); pending = 0; }
+        wait(&bars.q_empty[b], ((i / NQ) & 1) ^ 1);
+      }
       if (g < kM) {
         const int v = visible(tok);
         tok_s[b][g] = tok; pid_s[b][g] = pid; vs[b][g] = v;
@@ -414,11 +419,11 @@ k_ret_bwd_dq(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_con
       }
       asm volatile("cp.async.commit_group;" ::: "memory");
       if (g < kM) { Ls[b][g] = L; ds[b][g] = d_; }
-      asm volatile("cp.async.wait_group 0;" ::: "memory");
-      tc::fence_async_smem();
-      tc::mbar_arrive(&bars.q_full[b]);
+      if (pending > 0) { asm volatile("cp.async.wait_group 1;" ::: "memory"); publish(i - 1); }
+      pending = 1;
       pid = pid_n;
     }
+    if (pending > 0) { asm volatile("cp.async.wait_group 0;" ::: "memory"); publish(cnt - 1); }
   } else if (warp == MW + 1) {                             // ---- key and value tiles
     int sk = 0, phk = 0, sv = 0, phv = 0;
     auto last_pid = [&](int i) { return i < cnt ? ld_pid(min(gr.g1, gr.g0 + (gr.sub + i * gr.nsub + 1) * kM) - 1) : -1; };
@@ -455,9 +460,9 @@ k_ret_bwd_dq(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_con
     auto first = [&](bool must) {                          // false: nothing left, or (unless `must`) the next rows are still on their way
       while (ia < cnt) {
         if (Ta < 0) {
-          if (!must && !tc::mbar_try_wait(&bars.q_full[ia & 1], (ia >> 1) & 1)) return false;
-          wait(&bars.q_full[ia & 1], (ia >> 1) & 1);
-          Ta = T_s[ia & 1];
+          if (!must && !tc::mbar_test(&bars.q_full[ia % NQ], (ia / NQ) & 1)) return false;
+          wait(&bars.q_full[ia % NQ], (ia / NQ) & 1);
+          Ta = T_s[ia % NQ];
           ka = 0;
         }
         if (ka < Ta) break;
@@ -469,7 +474,7 @@ k_ret_bwd_dq(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_con
       wait(&bars.v_full[sv1], phv1);
       tc::fence_after_sync();
       const uint32_t c = tbase + (uint32_t)(n1 % NW) * 2 * kN;
-      const uint64_t a = tc::desc_step(dq0, (uint32_t)(ia & 1) * kRow), o = tc::desc_step(do0, (uint32_t)(ia & 1) * kRow);
+      const uint64_t a = tc::desc_step(dq0, (uint32_t)(ia % NQ) * kRow), o = tc::desc_step(do0, (uint32_t)(ia % NQ) * kRow);
       const uint64_t x = tc::desc_step(dk0, (uint32_t)sk1 * kCol), y = tc::desc_step(dv0, (uint32_t)sv1 * kCol);
 #pragma unroll
       for (int ks = 0; ks < D / 16; ++ks)
@@ -486,9 +491,9 @@ k_ret_bwd_dq(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_con
     };
     uint32_t used = 3u;                                    // bit b: parity to wait for before accumulator b is overwritten
     for (int i = 0, sk = 0; i < cnt && ok_; ++i) {
-      const int b = i & 1;
-      wait(&bars.q_full[b], (i >> 1) & 1);
-      const int T = T_s[b];
+      const int b = i & 1, qb = i % NQ;
+      wait(&bars.q_full[qb], (i / NQ) & 1);
+      const int T = T_s[qb];
       if (T > 0) { wait(&bars.acc_free[b], (used >> b) & 1u); used ^= 1u << b; }
       for (int t = 0; t < T && ok_; ++t, ++n2) {
         while (n1 - n2 < NW && first(n1 == n2)) {}
@@ -503,15 +508,15 @@ k_ret_bwd_dq(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_con
         if (++sk == NSK) sk = 0;
       }
       tc::mma_commit_warp(&bars.acc_done[b]);
-      tc::mma_commit_warp(&bars.q_empty[b]);
+      tc::mma_commit_warp(&bars.q_empty[qb]);
     }
   } else if (warp >= EW) {                                 // ---- the finished rows: thread = pair
     const int row = tid & 127;
     const uint32_t tl = tbase + ((uint32_t)((warp & 3) * 32) << 16);
     for (int i = 0; i < cnt; ++i) {
-      const int b = i & 1;
-      wait(&bars.q_full[b], (i >> 1) & 1);
-      const int pid = pid_s[b][row], T = T_s[b];
+      const int b = i & 1, qb = i % NQ;
+      wait(&bars.q_full[qb], (i / NQ) & 1);
+      const int pid = pid_s[qb][row], T = T_s[qb];
       wait(&bars.acc_done[b], (i >> 1) & 1);
       tc::fence_after_sync();
       const bool live = ok_ && pid >= 0;
@@ -527,7 +532,7 @@ k_ret_bwd_dq(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_con
         if (d0 + 32 == D) {
           tc::fence_before_sync();
           if (T > 0) tc::mbar_arrive(&bars.acc_free[b]);
-          tc::mbar_arrive(&bars.q_empty[b]);
+          tc::mbar_arrive(&bars.q_empty[qb]);
         }
         if (live) {
 #pragma unroll
@@ -546,8 +551,8 @@ k_ret_bwd_dq(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_con
     const float scale2 = dm.sigma * kLog2e;
     int n = 0;
     for (int i = 0; i < cnt; ++i) {
-      const int b = i & 1;
-      wait(&bars.q_full[b], (i >> 1) & 1);
+      const int b = i % NQ;
+      wait(&bars.q_full[b], (i / NQ) & 1);
       const int T = T_s[b], vis = vs[b][row], vmin = vs[b][0];                 // (the first pair sees the fewest keys)
       const bool whole = pid_s[b][kM - 1] >= 0;
       const float L2 = Ls[b][row], dl = ds[b][row];
@@ -623,15 +628,16 @@ int ret_bwd_short_tc(const Dims& d, const void* Q, const void* dO, const void* K
                      const float* delta, const int32_t* off_k, const RetIndex& ri, void* dq_part,
                      float* dK_perm, float* dV_perm, int* status, cudaStream_t st);
 
-// Two kernels, or one with five products per tile?  By the mean number of keys of a cluster: the fused kernel gathers a pair's
-// rows once per 64 keys and reads back the stored dQ row from the second time on, the two kernels gather it once more than
-// they have to when one sweep would have done.  Measured, fused | dK, dV + dQ, us:
-//   D = 64:   64 keys 566 | 311 + 569,  128 keys 469 | 233 + 293,  256 keys 1331 | 543 + 501,  512 keys 16860 | 5549 + 3808
-//   D = 128:  64 keys 850 | 484 + 438,  128 keys 684 | 353 + 261,  256 keys 1875 | 802 + 514
+// Two kernels, or one with five products per tile?  The fused kernel gathers a pair's rows once per 64 keys and reads back the stored
+// dQ row from the second time on; the two kernels gather it once more than they have to, and start twice as many CTAs.  So by the
+// mean keys and the mean pairs of a cluster.  Measured, fused | dK, dV + dQ, us:
+//   D = 64, 512 keys, 4096 pairs 16860 | 5410 + 3610;  256 keys, 2048 pairs 1331 | 543 + 501;  64 keys, 1024 pairs 2082 | 998 + 881;
+//           64 keys, 512 pairs 374 | 211 + 198;  32 keys, 256 pairs 364 | 217 + 209
+//   D = 128, 256 keys, 2048 pairs 1875 | 802 + 514;  128 keys, 1024 pairs 684 | 353 + 261;  64 keys, 2048 pairs 2754 | 1350 + 1340
 int ret_bwd_pairs_tc(const Dims& d, const void* Q, const void* dO, const void* Kp, const void* Vp, const float* LSE,
                      const float* delta, const int32_t* off_k, const RetIndex& ri, void* dq_part,
                      float* dK_perm, float* dV_perm, int* status, cudaStream_t st) {
-  if (d.N / d.Ck < (d.D == 128 ? 128 : 256))
+  if (d.N / d.Ck < (d.D == 128 ? 128 : 256) && (long long)d.N * d.m < 1024LL * d.Ck)
     return ret_bwd_short_tc(d, Q, dO, Kp, Vp, LSE, delta, off_k, ri, dq_part, dK_perm, dV_perm, status, st);
   return d.D == 128 ? ret_bwd_d<128>(d, Q, dO, Kp, Vp, LSE, delta, off_k, ri, dq_part, dK_perm, dV_perm, status, st)
                     : ret_bwd_d<64>(d, Q, dO, Kp, Vp, LSE, delta, off_k, ri, dq_part, dK_perm, dV_perm, status, st);

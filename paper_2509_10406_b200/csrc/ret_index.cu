@@ -152,7 +152,7 @@ size_t ret_index_elems(const Dims& d) {
 
 int build_ret_index(const Dims& d, const int32_t* sel, const int32_t* bsel, int32_t* scratch, RetIndex* out, cudaStream_t st) {
   const int pq = d.B * d.Hq, nkeys = d.SB * d.Ck, mk = d.m * (bsel ? d.k2 : 1);        // nkeys <= 32768
-  // Shares of 16 tiles; fewer where that would leave SMs without work (selections crowd on few clusters: one may have all of a head's
+  // Shares of 32 tiles; fewer where that would leave SMs without work (selections crowd on few clusters: one may have all of a head's
   // queries), not below 4 (a share loads its keys and adds its gradients once).
   const long long tiles = (long long)d.N * mk * pq / kRetTile, want = tiles / (8 * sm_count());
   out->share = (int)(want < kMinShare ? kMinShare : want > kMaxShare ? kMaxShare : want);
