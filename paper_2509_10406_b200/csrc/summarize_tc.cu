@@ -11,10 +11,12 @@
 // of a step before the sums of the one before it), four warps make weights, sixteen write snapshots; a snapshot's writers
 // give the accumulators back as soon as they hold them in registers.
 //
-// Bound by the snapshot writes, 6 D bytes per (query cluster, key cluster, plane), at D = 128 (3.5 TB/s; a memset reaches 4),
-// and at D = 64 by the weights of one step after the other.  Against one CTA per item with every phase behind a CTA barrier,
-// accumulators in registers and snapshots staged for TMA: 64k tokens, 128 x 128 clusters, D = 64, 32 heads 1499 -> 639 us;
-// 8k tokens, 64 x 128, 16 heads 304 -> 159; 64k, 256 x 1024, D = 128, 4 heads 1696 -> 1592; 128k, 512 x 2048 6.52 -> 6.28 ms.
+// Bound by the snapshot writes, 6 D bytes per (query cluster, key cluster, plane): 4.9 TB/s at 128k tokens, 512 x 2048 clusters,
+// D = 128; by the weights of one step after the other where the summaries are few.  Snapshots leave through shared memory
+// by TMA: written from registers, 32 bytes a thread, they kept the load/store unit busy for 3000 cycles a plane (6.28 ms
+// against 4.65).  Against one CTA per item with every phase behind a CTA barrier and accumulators in registers: 64k tokens,
+// 128 x 128 clusters, D = 64, 32 heads 1499 -> 605 us; 8k tokens, 64 x 128, 16 heads 304 -> 143; 16k, 128 x 256, 32 heads
+// 1202 -> 634; 64k, 256 x 1024, D = 128, 4 heads 1696 -> 1163; 128k, 512 x 2048 6.52 -> 4.65 ms.
 #include <cuda.h>
 #include "common.cuh"
 #include "tc05.cuh"
@@ -23,20 +25,24 @@ namespace muse {
 
 typedef __nv_bfloat16 bf16;
 int make_tmap_bf16_rows(void* out_map, const void* base, uint64_t rows, uint32_t cols, uint32_t box_rows);
+int make_tmap_bf16_nd(void* out_map, const void* base, int rank, const uint64_t* dims, const uint64_t* strides_bytes,
+                      const uint32_t* box);
 
 namespace st {
-constexpr int TI = 128, NU = 64, NS = 4;                   // query clusters of an item; keys of a step; steps in the ring
+constexpr int TI = 128;                                    // query clusters of an item
 constexpr int kSnapWarps = 16, kWeightWarp0 = 16, kMmaWarp = 20, kLoadWarp = 21, kDealWarp = 22, kThreads = 23 * 32;
 constexpr int kRing = 2, kTakers = kSnapWarps + 6;           // item ranges handed out ahead; warps that take each of them
 constexpr float kLazy = 8.f, kNever = -1e30f, kLog2e = 1.4426950408889634f;
 template <int D> struct Lay {                              // shared-memory offsets and TMEM columns for head dimension D
   static constexpr int G = D / 64;                         // 64-element (128-byte) column groups of a row
   static constexpr int NG = 128 / D;                       // groups of snapshot warps that take planes in turn (2 or 4 threads per row)
+  static constexpr int NU = D == 128 ? 32 : 64, NS = D == 128 ? 3 : 4;                 // keys of a step; steps in the ring
   static constexpr int kTile = TI * D * 2, kKeys = NU * D * 2;
-  static constexpr int oQhi = 0, oQlo = kTile, oKV = 2 * kTile, total = oKV + NS * 2 * kKeys + 1024;
+  static constexpr int oQhi = 0, oQlo = kTile, oKV = 2 * kTile, oStage = oKV + NS * 2 * kKeys;   // stage: kappa hi, kappa lo, nu of a snapshot, per group
+  static constexpr int total = oStage + NG * 3 * kTile + 1024;
   static constexpr uint32_t cUk = 0, cUv = D, cL = 2 * D, cLo = 2 * D + 2 * NU, cols = 512;
 };
-struct Bars { uint64_t q_full, q_free, kv_full[NS], kv_empty[NS], l_full[2], w_ready, u_step, u_done[2], acc_free[2], item_full[kRing], item_free[kRing]; };
+struct Bars { uint64_t q_full, q_free, kv_full[4], kv_empty[4], l_full[2], w_ready, u_step, u_done[2], acc_free[2], item_full[kRing], item_free[kRing]; };
 }  // namespace st
 
 __global__ void k_split_qbar(const float* __restrict__ qbar, long long n, float sigma, bf16* __restrict__ hi, bf16* __restrict__ lo, int* dealt) {
@@ -60,11 +66,11 @@ int split_qbar(const Dims& d, const float* qbar, void* qhi, void* qlo, int* deal
 template <int D>
 __global__ void __launch_bounds__(st::kThreads, 1)
 k_summarize_tc(Dims dm, const __grid_constant__ CUtensorMap tm_K, const __grid_constant__ CUtensorMap tm_V,
-               const __grid_constant__ CUtensorMap tm_qhi, const __grid_constant__ CUtensorMap tm_qlo, const int32_t* __restrict__ off_k,
-               SummPtrs sp, int per_block, int per, int* __restrict__ dealt, int* __restrict__ status) {
+               const __grid_constant__ CUtensorMap tm_qhi, const __grid_constant__ CUtensorMap tm_qlo, const __grid_constant__ CUtensorMap tm_okhi,
+               const __grid_constant__ CUtensorMap tm_oklo, const __grid_constant__ CUtensorMap tm_onu, const int32_t* __restrict__ off_k, SummPtrs sp, int per_block, int per, int* __restrict__ dealt, int* __restrict__ status) {
   using namespace st;   // per: items of a CTA, or 1: they are dealt out one by one; dealt: those dealt so far
   typedef Lay<D> LY;
-  constexpr int G = LY::G, NG = LY::NG, kKeys = LY::kKeys;
+  constexpr int G = LY::G, NG = LY::NG, NU = LY::NU, NS = LY::NS, kTile = LY::kTile, kKeys = LY::kKeys;
   extern __shared__ __align__(1024) unsigned char sm_raw[];
   __shared__ Bars bars;
   __shared__ uint32_t tbase_s;
@@ -329,6 +335,8 @@ k_summarize_tc(Dims dm, const __grid_constant__ CUtensorMap tm_K, const __grid_c
   } else {                                                 // ---- snapshots: thread = (query cluster, 32 dims of kappa and of nu)
     const int row = (warp & 3) * 32 + lane, part = (warp >> 2) & (D / 32 - 1), grp = NG == 2 ? warp >> 3 : 0;
     const uint32_t tl = tbase + ((uint32_t)((warp & 3) * 32) << 16) + 32 * part;
+    constexpr int kGroup = kSnapWarps * 32 / NG;
+    const bool lead = warp == grp * (kSnapWarps / NG);
     int k = 0;
     Plane P{-1, 0, 0, 0, 0, 0, 0, 0, 0, 0};
     for (take(P); P.it < items; take(P)) {
@@ -362,22 +370,48 @@ k_summarize_tc(Dims dm, const __grid_constant__ CUtensorMap tm_K, const __grid_c
           const __nv_bfloat162 nb = __floats2bfloat162_rn(inv > 0.f ? v[u] * inv : 0.f, inv > 0.f ? v[u + 1] * inv : 0.f);
           nw[u / 2] = *reinterpret_cast<const uint32_t*>(&nb);
         }
-        if (i < dm.Cq && ok) {                             // 32-byte stores: whole sectors
-          const size_t ent = (((size_t)pq * dm.SB + pl) * dm.Cq + i) * dm.Ck + j, at = ent * D + 32 * part;
-          if (part == 0) {
-            const float m_ = mass > 0.f ? (base + log2f(mass)) * 0.6931471805599453f : -INFINITY;
-            sp.mu[ent] = m_;
-            sp.beta[ent] = mass > 0.f ? m_ - T * inv : -INFINITY;
+        if (part == 0 && i < dm.Cq && ok) {
+          const size_t ent = (((size_t)pq * dm.SB + pl) * dm.Cq + i) * dm.Ck + j;
+          const float m_ = mass > 0.f ? (base + log2f(mass)) * 0.6931471805599453f : -INFINITY;
+          sp.mu[ent] = m_;
+          sp.beta[ent] = mass > 0.f ? m_ - T * inv : -INFINITY;
+        }
+        // three swizzled [128 rows][128 B] tiles per 64 dims, which leave by TMA (rows of consecutive query clusters are Ck entries apart)
+        unsigned char* stage = sm + LY::oStage + grp * 3 * kTile;
+        // Where DRAM is the bound (D = 128, dozens of items per CTA) each tile leaves on its own and the next snapshot's waits for that one
+        // alone (128k tokens, 512 x 2048 clusters: 4.95 -> 4.65 ms); else one pair of barriers for the three (50 x 200 clusters, 8 items
+        // per CTA: 121 -> 108 us).
+        const bool apart = D == 128 && items >= 32 * (int)gridDim.x;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          if (apart || a == 0) {
+            if (lead) { if (apart) tc::tma_store_wait_read_but_warp<2>(); else tc::tma_store_wait_read_warp(); }
+            tc::named_bar_sync(1 + grp, kGroup);
           }
 #pragma unroll
-          for (int c = 0; c < 2; ++c) {
-            tc::st_global_32B((bf16*)sp.khi + at + 16 * c, reinterpret_cast<uint32_t(&)[8]>(hw[8 * c]));
-            tc::st_global_32B((bf16*)sp.klo + at + 16 * c, reinterpret_cast<uint32_t(&)[8]>(lw[8 * c]));
-            tc::st_global_32B((bf16*)sp.nu + at + 16 * c, reinterpret_cast<uint32_t(&)[8]>(nw[8 * c]));
+          for (int c = 0; c < 4; ++c) {
+            const int ch = 4 * part + c;                   // 16-byte chunk of the row
+            const uint32_t* x = a == 0 ? hw : a == 1 ? lw : nw;
+            *reinterpret_cast<uint4*>(stage + a * kTile + (ch >> 3) * TI * 128 + tc::sw128_off(row, ch & 7)) = make_uint4(x[4 * c], x[4 * c + 1], x[4 * c + 2], x[4 * c + 3]);
+          }
+          if (apart || a == 2) {
+            tc::fence_async_smem();
+            tc::named_bar_sync(1 + grp, kGroup);
+            if (lead && ok) {
+#pragma unroll
+              for (int b = 0; b < 3; ++b) {
+                if (b > a || (apart && b < a)) continue;
+                const void* map = b == 0 ? (const void*)&tm_okhi : b == 1 ? (const void*)&tm_oklo : (const void*)&tm_onu;
+#pragma unroll
+                for (int g = 0; g < G; ++g) tc::tma_store_4d_warp(map, stage + b * kTile + g * TI * 128, 64 * g, j, P.i0, pq * dm.SB + pl);
+              }
+              tc::tma_store_commit_warp();
+            }
           }
         }
       }
     }
+    if (lead) tc::tma_store_wait_all_warp();
   }
   if (!ok && lane == 0) report_status(status, 7);
   tc::fence_before_sync();
@@ -403,15 +437,23 @@ int summarize_tc(const Dims& d, const void* Kp, const void* Vp, const int32_t* o
   if (rc == MUSE_OK) rc = make_tmap_bf16_rows(&tV, Vp, (uint64_t)d.B * d.Hkv * d.N, d.D, 16);
   if (rc != MUSE_OK) return rc;
   prof_mark("k_summarize_tc", stream);
+  // outputs as 4-D tensors (d, j, i, head * planes + plane); a box is 128 query clusters of one key cluster
+  CUtensorMap okhi, oklo, onu;
+  const uint64_t dims[4] = {(uint64_t)d.D, (uint64_t)d.Ck, (uint64_t)d.Cq, (uint64_t)d.B * d.Hq * d.SB};
+  const uint64_t strides[3] = {(uint64_t)d.D * 2, (uint64_t)d.Ck * d.D * 2, (uint64_t)d.Cq * d.Ck * d.D * 2};
+  const uint32_t box[4] = {64, 1, (uint32_t)st::TI, 1};
+  MUSE_RC(make_tmap_bf16_nd(&okhi, sp.khi, 4, dims, strides, box));
+  MUSE_RC(make_tmap_bf16_nd(&oklo, sp.klo, 4, dims, strides, box));
+  MUSE_RC(make_tmap_bf16_nd(&onu, sp.nu, 4, dims, strides, box));
   const long long items = (long long)d.Ck * cdiv(d.Cq, st::TI) * d.B * d.Hq;
   const int grid = (int)(items < sm_count() ? items : sm_count());
   // With many key clusters per tile the items are dealt out one by one, in order: all CTAs then write neighbouring rows at a time,
-  // which is what DRAM wants (128k tokens, 512 x 2048 clusters, 22 GB of summaries: 9.1 ms in one range per CTA, 6.3 ms dealt).
+  // which is what DRAM wants (128k tokens, 512 x 2048 clusters, 22 GB of summaries: 9.1 ms in one range per CTA, 6.3 dealt).
   // With few, every item would change the tile.
   const int per = d.Ck >= grid ? 1 : (int)((items + grid - 1) / grid);
   int* dealt = status + kItemWord;
-  if (d.D == 128) return launch_pdl(k_summarize_tc<128>, dim3(grid), st::kThreads, st::Lay<128>::total, stream, d, tK, tV, tqh, tql, off_k, sp, per_block, per, dealt, status);
-  return launch_pdl(k_summarize_tc<64>, dim3(grid), st::kThreads, st::Lay<64>::total, stream, d, tK, tV, tqh, tql, off_k, sp, per_block, per, dealt, status);
+  if (d.D == 128) return launch_pdl(k_summarize_tc<128>, dim3(grid), st::kThreads, st::Lay<128>::total, stream, d, tK, tV, tqh, tql, okhi, oklo, onu, off_k, sp, per_block, per, dealt, status);
+  return launch_pdl(k_summarize_tc<64>, dim3(grid), st::kThreads, st::Lay<64>::total, stream, d, tK, tV, tqh, tql, okhi, oklo, onu, off_k, sp, per_block, per, dealt, status);
 }
 
 }  // namespace muse

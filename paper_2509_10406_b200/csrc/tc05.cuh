@@ -187,6 +187,10 @@ __device__ __forceinline__ void tma_store_4d_warp(const void* tmap, const void* 
 }
 __device__ __forceinline__ void tma_store_commit_warp() { if (elect_one()) tma_store_commit(); }
 __device__ __forceinline__ void tma_store_wait_read_warp() { if (elect_one()) tma_store_wait_read(); __syncwarp(); }
+template <int N> __device__ __forceinline__ void tma_store_wait_read_but_warp() {         // all but the last N groups have been read
+  if (elect_one()) asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory");
+  __syncwarp();
+}
 __device__ __forceinline__ void tma_store_wait_all_warp() { if (elect_one()) tma_store_wait_all(); __syncwarp(); }
 // warp index that the compiler knows to be the same for the whole warp
 __device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
@@ -297,6 +301,11 @@ __device__ __forceinline__ void tmem_ld_use8(float (&v)[8]) {
 __device__ __forceinline__ void tmem_ld_use16(float (&v)[16]) {
   asm volatile("" : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]), "+f"(v[7]),
                     "+f"(v[8]), "+f"(v[9]), "+f"(v[10]), "+f"(v[11]), "+f"(v[12]), "+f"(v[13]), "+f"(v[14]), "+f"(v[15]) :: "memory");
+}
+
+// brings `bytes` (a multiple of 16) at `src` (16-byte aligned) into L2; one thread, no completion to wait for
+__device__ __forceinline__ void l2_prefetch(const void* src, uint32_t bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
 }
 
 // 32-byte global accesses (one full sector per thread)
