@@ -609,37 +609,40 @@ k_summ_bwd(Dims dm, const T* __restrict__ Kp, const T* __restrict__ Vp, const in
 template <class T, int D, class PT>      // PT: element type of the per-(query, slot) dq partials
 __global__ void k_final_dq(Dims dm, const float* __restrict__ dQacc, const PT* __restrict__ dq_part,
                            const int32_t* __restrict__ sel, const int32_t* __restrict__ bsel, int use_ret, T* __restrict__ dQ) {
-  const int pq = blockIdx.y;
-  const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (t >= dm.N) return;
+  constexpr int LPQ = D / 8, QPW = 32 / LPQ, NA = 64 / LPQ;  // lanes of a query (8 dims each), queries of a warp: as in the forward merge
+  const int pq = blockIdx.y, lane = threadIdx.x & 31, g = lane / LPQ, l = lane % LPQ, dd = l * 8;
+  const int t_ = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * QPW + g;
+  const bool live = t_ < dm.N;
+  const int t = live ? t_ : dm.N - 1;
   const size_t row = (size_t)pq * dm.N + t;
-  float acc[D / 32];
+  // which partial rows exist: one per slot, or with the two-level retrieval one per (slot, chosen block); at most 64
+  const int kk = bsel != nullptr ? dm.k2 : 1, n = dm.m * kk, pl = query_plane_b(dm, t);
+  float acc[8];
+  ld8(dQacc + row * D + dd, acc);
+  if (use_ret) {
 #pragma unroll
-  for (int k = 0; k < D / 32; ++k) acc[k] = dQacc[row * D + lane + 32 * k];
-  if (use_ret && query_plane_b(dm, t) >= 0) {
-    if (bsel == nullptr) {                                 // one partial row per slot
-      for (int s = 0; s < dm.m; ++s) {
-        const int c = sel[row * dm.m + s];
-        if (c < 0 || c >= dm.Ck) continue;                 // "none", or an entry outside [0, Ck), which counts as none
-#pragma unroll
-        for (int k = 0; k < D / 32; ++k) acc[k] += to_f(dq_part[(row * dm.m + s) * D + lane + 32 * k]);
+    for (int a = 0; a < NA; ++a) {
+      if (a * LPQ >= n) break;
+      const int s = a * LPQ + l;
+      bool ok = false;
+      if (pl >= 0 && s < n) {
+        const int c = sel[row * dm.m + s / kk];
+        ok = c >= 0 && c < dm.Ck;                          // "none", or an entry outside [0, Ck), counts as none
+        if (ok && bsel != nullptr) { const int bb = bsel[row * n + s]; ok = bb >= 0 && bb <= pl; }
       }
-    } else {                                               // two-level retrieval: one per (slot, chosen block)
-      const int kk = dm.k2, pl = query_plane_b(dm, t);
-      for (int s = 0; s < dm.m; ++s) {
-        const int c = sel[row * dm.m + s];
-        if (c < 0 || c >= dm.Ck) continue;
-        for (int e = 0; e < kk; ++e) {
-          const int bb = bsel[(row * dm.m + s) * kk + e];
-          if (bb < 0 || bb > pl) continue;
+      const unsigned have = __ballot_sync(0xffffffffu, ok) >> (g * LPQ);
+      const PT* src = dq_part + (row * n + a * LPQ) * D + dd;
+#pragma unroll 8
+      for (int u = 0; u < LPQ; ++u)
+        if ((have >> u) & 1u) {
+          float y[8];
+          ld8(src + u * D, y);
 #pragma unroll
-          for (int k = 0; k < D / 32; ++k) acc[k] += to_f(dq_part[((row * dm.m + s) * kk + e) * D + lane + 32 * k]);
+          for (int k = 0; k < 8; ++k) acc[k] += y[k];
         }
-      }
     }
   }
-#pragma unroll
-  for (int k = 0; k < D / 32; ++k) dQ[row * D + lane + 32 * k] = from_f<T>(acc[k]);
+  if (live) st8(dQ + row * D + dd, acc);
 }
 
 // dK[u] = sum over the query heads of the group of (local part at u + bucketed part at p), u = perm_k[p].
@@ -874,9 +877,9 @@ static int attn_bwd_t(const Dims& d, int dtype, const T* Q, const T* K, const T*
   }
   prof_mark("k_final_dq", st);
   if (kTensor)
-    k_final_dq<T, D, __nv_bfloat16><<<dim3(cdiv(d.N, 8), pq), 256, 0, st>>>(d, w.dQacc, (const __nv_bfloat16*)w.dq_part, sel, bsel, use_ret, dQ);
+    k_final_dq<T, D, __nv_bfloat16><<<dim3(cdiv(d.N, 8 * (256 / D)), pq), 256, 0, st>>>(d, w.dQacc, (const __nv_bfloat16*)w.dq_part, sel, bsel, use_ret, dQ);
   else
-    k_final_dq<T, D, float><<<dim3(cdiv(d.N, 8), pq), 256, 0, st>>>(d, w.dQacc, w.dq_part, sel, bsel, use_ret, dQ);
+    k_final_dq<T, D, float><<<dim3(cdiv(d.N, 8 * (256 / D)), pq), 256, 0, st>>>(d, w.dQacc, w.dq_part, sel, bsel, use_ret, dQ);
   MUSE_LAUNCH_OK();
   prof_mark("k_final_dkv", st);
   k_final_dkv<T, D><<<dim3(cdiv(d.N * (D / 4), 256), pk), 256, 0, st>>>(d, perm_k, w.dK_orig, w.dV_orig, w.dK_perm, w.dV_perm,

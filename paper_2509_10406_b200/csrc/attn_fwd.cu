@@ -369,7 +369,8 @@ k_local_fwd(Dims dm, const T* __restrict__ Q, const T* __restrict__ K, const T* 
 }
 
 // ---------------------------------------------------------------------------------------------
-// Merge: L = LSE over components, O = sum_c exp(lse_c - L) o_c.  One warp per query.
+// Merge: L = LSE over components, O = sum_c exp(lse_c - L) o_c.  Eight dims per lane, so two or four queries per warp: the
+// kernel waits for its scattered rows, and each lane has up to eight 16-byte loads of them in flight.
 // ---------------------------------------------------------------------------------------------
 template <class T, int D, class PT>      // PT: element type of the retrieval partial outputs
 __global__ void k_merge(Dims dm, const float* __restrict__ o_far, const float* __restrict__ lse_far,
@@ -377,9 +378,11 @@ __global__ void k_merge(Dims dm, const float* __restrict__ o_far, const float* _
                         const PT* __restrict__ o_part, const float* __restrict__ l_part,
                         const float* __restrict__ o_near, const float* __restrict__ lse_near,
                         const int32_t* __restrict__ sel, const int32_t* __restrict__ bsel, T* __restrict__ O, float* __restrict__ LSE) {
-  const int pq = blockIdx.y;
-  const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (t >= dm.N) return;
+  constexpr int LPQ = D / 8, QPW = 32 / LPQ, NA = 64 / LPQ;                    // lanes of a query (8 dims each), queries of a warp
+  const int pq = blockIdx.y, lane = threadIdx.x & 31, g = lane / LPQ, l = lane % LPQ, dd = l * 8;
+  const int t_ = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * QPW + g;
+  const bool live = t_ < dm.N;
+  const int t = live ? t_ : dm.N - 1;
   const size_t row = (size_t)pq * dm.N + t;
   const int pl = query_plane(dm, t);
   const bool far_ok = pl >= 0 && dm.SB > 0;
@@ -390,71 +393,68 @@ __global__ void k_merge(Dims dm, const float* __restrict__ o_far, const float* _
   float mx = fmaxf(fmaxf(lf, ll), ln);
   // retrieved partial results of this query: one per slot, or one per (slot, chosen block) with spatial block selection
   const int kk = bsel != nullptr ? dm.k2 : 1, m = dm.m * kk;
-  float lp_mine[2] = {-INFINITY, -INFINITY};        // partials lane, lane + 32
-  if (far_ok) {
+  float w[NA];                                      // log-sum-exp, then weight, of partials l, l + LPQ, ...
 #pragma unroll
-    for (int a = 0; a < 2; ++a) {
-      const int s = lane + 32 * a;
-      if (s < m && sel[row * dm.m + s / kk] >= 0 && (bsel == nullptr || bsel[row * m + s] >= 0)) lp_mine[a] = l_part[row * m + s];
-      mx = fmaxf(mx, lp_mine[a]);
-    }
+  for (int a = 0; a < NA; ++a) {
+    const int s = a * LPQ + l;
+    w[a] = -INFINITY;
+    if (a * LPQ < m && far_ok && s < m && sel[row * dm.m + s / kk] >= 0 && (bsel == nullptr || bsel[row * m + s] >= 0)) w[a] = l_part[row * m + s];
+    mx = fmaxf(mx, w[a]);
   }
-  mx = warp_max(mx);
+#pragma unroll
+  for (int o = LPQ / 2; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
   float tot = 0.f;
 #pragma unroll
-  for (int a = 0; a < 2; ++a) tot += lp_mine[a] == -INFINITY ? 0.f : expf(lp_mine[a] - mx);
-  tot = warp_sum(tot);
+  for (int a = 0; a < NA; ++a) {
+    if (a * LPQ >= m) break;
+    w[a] = w[a] == -INFINITY ? 0.f : expf(w[a] - mx);
+    tot += w[a];
+  }
+#pragma unroll
+  for (int o = LPQ / 2; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
   const float wf = lf == -INFINITY ? 0.f : expf(lf - mx), wl = ll == -INFINITY ? 0.f : expf(ll - mx);
   const float wn = ln == -INFINITY ? 0.f : expf(ln - mx);
   tot += wf + wl + wn;
   const float inv = 1.f / tot;
-  // lane owns EPL consecutive output dims: one vector load per input row and lane
-  constexpr int EPL = D / 32;
-  const int dd = lane * EPL;
-  float acc[EPL];
+  float acc[8], x[8];
 #pragma unroll
-  for (int k = 0; k < EPL; ++k) acc[k] = 0.f;
+  for (int k = 0; k < 8; ++k) acc[k] = 0.f;
   if (wf > 0.f) {
-    float x[EPL];
-    ldv<EPL>(o_far + row * D + dd, x);
+    ld8(o_far + row * D + dd, x);
 #pragma unroll
-    for (int k = 0; k < EPL; ++k) acc[k] = fmaf(wf, x[k], acc[k]);
+    for (int k = 0; k < 8; ++k) acc[k] = wf * x[k];
   }
   if (wl > 0.f) {
-    float x[EPL];
-    ldv<EPL>(o_loc + row * D + dd, x);
+    ld8(o_loc + row * D + dd, x);
 #pragma unroll
-    for (int k = 0; k < EPL; ++k) acc[k] = fmaf(wl, x[k], acc[k]);
+    for (int k = 0; k < 8; ++k) acc[k] = fmaf(wl, x[k], acc[k]);
   }
   if (wn > 0.f) {
-    float x[EPL];
-    ldv<EPL>(o_near + row * D + dd, x);
+    ld8(o_near + row * D + dd, x);
 #pragma unroll
-    for (int k = 0; k < EPL; ++k) acc[k] = fmaf(wn, x[k], acc[k]);
+    for (int k = 0; k < 8; ++k) acc[k] = fmaf(wn, x[k], acc[k]);
   }
-  // retrieved slots four at a time, so that four independent row loads are in flight
-  for (int s0 = 0; s0 < m; s0 += 4) {
-    float w[4], x[4][EPL];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int s = s0 + u;
-      const float lp = s < m ? __shfl_sync(0xffffffffu, lp_mine[s >> 5], s & 31) : -INFINITY;
-      w[u] = lp == -INFINITY ? 0.f : expf(lp - mx);
-      if (w[u] > 0.f) ldv<EPL>(o_part + (row * m + s) * D + dd, x[u]);
-      else {
+  for (int a = 0; a < NA; ++a) {
+    if (a * LPQ >= m) break;
+    const PT* src = o_part + (row * m + a * LPQ) * D + dd;
+#pragma unroll 8
+    for (int u = 0; u < LPQ; ++u) {
+      const float wu = __shfl_sync(0xffffffffu, w[a], g * LPQ + u);            // (0 past m)
+      if (wu > 0.f) {
+        float y[8];
+        ld8(src + u * D, y);
 #pragma unroll
-        for (int k = 0; k < EPL; ++k) x[u][k] = 0.f;
+        for (int k = 0; k < 8; ++k) acc[k] = fmaf(wu, y[k], acc[k]);
       }
     }
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-#pragma unroll
-      for (int k = 0; k < EPL; ++k) acc[k] = fmaf(w[u], x[u][k], acc[k]);
   }
 #pragma unroll
-  for (int k = 0; k < EPL; ++k) acc[k] *= inv;
-  stv<EPL>(O + row * D + dd, acc);
-  if (lane == 0) LSE[row] = mx + logf(tot);
+  for (int k = 0; k < 8; ++k) acc[k] *= inv;
+  if (live) {
+    st8(O + row * D + dd, acc);
+    if (l == 0) LSE[row] = mx + logf(tot);
+  }
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -567,11 +567,11 @@ static int attn_fwd_t(const Dims& d, const T* Q, const T* K, const T* V, const i
   }
   prof_mark("k_merge", st);
   if (kTensor)
-    k_merge<T, D, __nv_bfloat16><<<dim3(cdiv(d.N, 8), pq), 256, 0, st>>>(d, w.o_far, w.lse_far, w.o_loc, w.lse_loc,
+    k_merge<T, D, __nv_bfloat16><<<dim3(cdiv(d.N, 8 * (256 / D)), pq), 256, 0, st>>>(d, w.o_far, w.lse_far, w.o_loc, w.lse_loc,
                                                                        (const __nv_bfloat16*)w.o_part, w.l_part, two_level ? w.o_near : nullptr,
                                                                        two_level ? w.lse_near : nullptr, sel, bsel, O, LSE);
   else
-    k_merge<T, D, float><<<dim3(cdiv(d.N, 8), pq), 256, 0, st>>>(d, w.o_far, w.lse_far, w.o_loc, w.lse_loc, w.o_part, w.l_part, nullptr, nullptr,
+    k_merge<T, D, float><<<dim3(cdiv(d.N, 8 * (256 / D)), pq), 256, 0, st>>>(d, w.o_far, w.lse_far, w.o_loc, w.lse_loc, w.o_part, w.l_part, nullptr, nullptr,
                                                                sel, nullptr, O, LSE);
   MUSE_LAUNCH_OK();
   return MUSE_OK;

@@ -89,6 +89,28 @@ template <int EPL> __device__ __forceinline__ void stv(__nv_bfloat16* p, const f
   else { __nv_bfloat162 b = __floats2bfloat162_rn(x[0], x[1]); *reinterpret_cast<uint32_t*>(p) = *reinterpret_cast<uint32_t*>(&b); }
 }
 
+// 8 consecutive elements as floats / back, in 16-byte accesses
+__device__ __forceinline__ void ld8(const float* p, float (&x)[8]) {
+  const float4 a = ld4(p), b = ld4(p + 4);
+  x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w; x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
+}
+__device__ __forceinline__ void ld8(const __nv_bfloat16* p, float (&x)[8]) {
+  const uint4 u = *reinterpret_cast<const uint4*>(p);
+  const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+  for (int k = 0; k < 4; ++k) { x[2 * k] = __uint_as_float(w[k] << 16); x[2 * k + 1] = __uint_as_float(w[k] & 0xffff0000u); }
+}
+__device__ __forceinline__ void st8(float* p, const float (&x)[8]) {
+  st4(p, make_float4(x[0], x[1], x[2], x[3]));
+  st4(p + 4, make_float4(x[4], x[5], x[6], x[7]));
+}
+__device__ __forceinline__ void st8(__nv_bfloat16* p, const float (&x)[8]) {
+  uint32_t w[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) { const __nv_bfloat162 b = __floats2bfloat162_rn(x[2 * k], x[2 * k + 1]); w[k] = *reinterpret_cast<const uint32_t*>(&b); }
+  *reinterpret_cast<uint4*>(p) = make_uint4(w[0], w[1], w[2], w[3]);
+}
+
 // One step of a running arg-min as two selects (left to itself the compiler makes a branch of the comparison).  A NaN
 // never compares below the minimum.  The second form is for candidates in any order: the lower index on a tie.
 __device__ __forceinline__ void argmin_step(float v, int i, float& best, int& bidx) {
