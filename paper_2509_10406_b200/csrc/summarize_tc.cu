@@ -267,10 +267,10 @@ k_summarize_tc(Dims dm, const __grid_constant__ CUtensorMap tm_K, const __grid_c
               for (int u = 0; u < 16; ++u) v[u] = 16 * g + u < nk ? v[u] : kNever;
             }
           };
-          float cm = kNever;
+          float cm = kNever, v0[16];                       // (the first 16 stay in registers: a bucket often has no more)
 #pragma unroll 1
-          for (int g = 0; g < ng; ++g) {
-            float v[16];
+          for (int g = ng - 1; g >= 0; --g) {
+            float (&v)[16] = v0;
             tc::tmem_ld16(tL + 16 * g, v);
             mask(v, g);
             float m4[4] = {v[0], v[1], v[2], v[3]};
@@ -301,9 +301,8 @@ k_summarize_tc(Dims dm, const __grid_constant__ CUtensorMap tm_K, const __grid_c
           float ws[2] = {0.f, 0.f}, wl[2] = {0.f, 0.f};
 #pragma unroll 1
           for (int g = 0; g < ng; ++g) {
-            float v[16];
-            tc::tmem_ld16(tL + 16 * g, v);
-            mask(v, g);
+            float (&v)[16] = v0;
+            if (g > 0) { tc::tmem_ld16(tL + 16 * g, v); mask(v, g); }
             uint32_t hw[8], lw[8];
 #pragma unroll
             for (int u = 0; u < 16; u += 2) {
