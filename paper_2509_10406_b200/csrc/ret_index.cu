@@ -162,9 +162,10 @@ int build_ret_index(const Dims& d, const int32_t* sel, const int32_t* bsel, int3
   out->items = (int2*)(out->pairs + (size_t)pq * up64((size_t)d.N * mk));
   out->nitems = (int32_t*)(out->items + (size_t)pq * up64(2 * (size_t)item_cap(d, kMinShare)) / 2);
   if (d.m == 0 || nkeys == 0) return MUSE_OK;
-  // CTAs of a head: enough to fill the chip, of 2048 pairs or more
+  // CTAs of a head, of 2048 pairs or more: until half the SMs have one (a large cluster pays in its exchange of counts and in scheduling:
+  // 32 heads of 16k tokens, 16 slots 131 us with 8 CTAs, 87 with 4; 4 heads of 64k, 32 slots 181 us with 16, 326 with 8)
   int cl = 1;
-  while (cl < kRiMaxCluster && cl * pq < 2 * sm_count() && (long long)d.N * d.m >= 2LL * cl * kRiMinPairs) cl *= 2;
+  while (cl < kRiMaxCluster && cl * pq < sm_count() / 2 && (long long)d.N * d.m >= 2LL * cl * kRiMinPairs) cl *= 2;
   const size_t smem = (size_t)nkeys * sizeof(int32_t);
   const RiArgs g = {sel, bsel, *out, nkeys};
   if (cl > 8) MUSE_CUDA_OK(cudaFuncSetAttribute(k_ret_index, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
