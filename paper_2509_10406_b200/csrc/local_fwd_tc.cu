@@ -86,8 +86,8 @@ k_local_fwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_q, const __grid_c
   tc::fence_after_sync();
   const uint32_t tbase = tbase_s;
   bool ok = true;
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
 
   if (warp == MW + 1) {                                         // ---- loads
     auto load = [&](unsigned char* dst, const void* map, int row, uint64_t* bar) {
@@ -231,13 +231,14 @@ k_local_fwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_q, const __grid_c
         }
         tc::tmem_st8_issue(ts + W / 2 * half + 8 * g, pk);
       }
+      l += (rs[0] + rs[1]) + (rs[2] + rs[3]);
+      // every phase of pv_done is waited for before the next one can complete (a wait for a phase two behind never returns)
+      if (t > 0 && ok && !tc::mbar_wait(&bars.pv_done[q], (t - 1) & 1)) ok = false;
       tc::tmem_st_wait();
       tc::fence_before_sync();
       tc::mbar_arrive(&bars.p_ready[q]);
-      l += (rs[0] + rs[1]) + (rs[2] + rs[3]);
     }
     if (Tq > 0) {
-      if (ok && Tq > 1 && !tc::mbar_wait(&bars.pv_done[q], (Tq - 2) & 1)) ok = false;    // (a wait never skips a phase of its barrier)
       if (ok && !tc::mbar_wait(&bars.pv_done[q], (Tq - 1) & 1)) ok = false;
       tc::fence_after_sync();
       if (H == 2) {
