@@ -12,7 +12,8 @@ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) ==
 
 unsigned g_forced_paths = 0;
 
-// The status words are cleared once per public call (every kernel of the call reports into them).
+// The status words are cleared once per public call (every kernel of the call reports into them): by its first kernel where that
+// reports nothing itself, else by this.
 int clear_status(void* ws, cudaStream_t st) {
   return cudaMemsetAsync(ws, 0, kStatusWords * sizeof(int32_t), st) == cudaSuccess ? MUSE_OK : MUSE_ERR_CUDA;
 }
@@ -227,7 +228,6 @@ int muse_cluster(const muse_params_t* p, const void* Q, const void* K, const int
   Arena ar(ws);
   int* status = ar.take<int32_t>(kStatusWords);
   for (int k = 0; k < n; ++k) lloyd_side_ws(d, ar, sides[k]);
-  if (clear_status(ws, stream) != MUSE_OK) return MUSE_ERR_CUDA;
   rc = lloyd(d, p->dtype, sides, n, p->init_mode, p->seed, p->kmeans_iters, status, stream);
   prof_mark(nullptr, stream);
   return rc;
@@ -359,7 +359,7 @@ int muse_summarize(const muse_params_t* p, const void* K, const void* V, const i
   size_t need[6];
   muse_workspace_bytes(p, need);
   if (ws_bytes < need[1]) return MUSE_ERR_WORKSPACE;
-  if (clear_status(ws, stream) != MUSE_OK) return MUSE_ERR_CUDA;
+  if (assign_k == nullptr && clear_status(ws, stream) != MUSE_OK) return MUSE_ERR_CUDA;     // (else by the sort, the first kernel)
   rc = summarize(d, p->dtype, K, V, assign_k, qbar, off_k, perm_k, counts, ksum, vsum, summaries, ws, nullptr, stream);
   prof_mark(nullptr, stream);
   return rc;
@@ -377,7 +377,6 @@ int muse_attn_fwd(const muse_params_t* p, const void* Q, const void* K, const vo
   size_t need[6];
   muse_workspace_bytes(p, need);
   if (ws_bytes < need[2]) return MUSE_ERR_WORKSPACE;
-  if (clear_status(ws, stream) != MUSE_OK) return MUSE_ERR_CUDA;
   rc = attn_fwd(d, p->dtype, Q, K, V, assign_q, qbar, off_k, perm_k, summaries, sel_in, bsel_in, O, LSE, sel_out, bsel_out, ws, stream);
   prof_mark(nullptr, stream);
   return rc;
@@ -399,8 +398,9 @@ int muse_attn_bwd(const muse_params_t* p, const void* Q, const void* K, const vo
   size_t need[6];
   muse_workspace_bytes(p, need);
   if (ws_bytes < (summaries ? need[3] : need[5])) return MUSE_ERR_WORKSPACE;
-  if (clear_status(ws, stream) != MUSE_OK) return MUSE_ERR_CUDA;
-  if (summaries == nullptr) {
+  const bool rebuild = summaries == nullptr;
+  if (rebuild) {
+    if (clear_status(ws, stream) != MUSE_OK) return MUSE_ERR_CUDA;
     // Rebuild the summaries from the bucketed keys in the tail of the workspace (the keys keep the
     // bucketing that off_k / perm_k describe, so no sort is needed).
     char* tail = (char*)ws + need[3];
@@ -413,7 +413,7 @@ int muse_attn_bwd(const muse_params_t* p, const void* Q, const void* K, const vo
     if (rc != MUSE_OK) return rc;
     summaries = tail;
   }
-  rc = attn_bwd(d, p->dtype, Q, K, V, O, LSE, dO, assign_q, qbar, off_k, perm_k, summaries, sel, bsel, dQ, dK, dV, ws, stream);
+  rc = attn_bwd(d, p->dtype, Q, K, V, O, LSE, dO, assign_q, qbar, off_k, perm_k, summaries, sel, bsel, dQ, dK, dV, ws, !rebuild, stream);
   prof_mark(nullptr, stream);
   return rc;
 }

@@ -102,8 +102,8 @@ k_assign_tc(const __grid_constant__ CUtensorMap tx0, const __grid_constant__ CUt
   tc::fence_after_sync();
   const uint32_t tbase = tbase_s;
   bool ok = true;
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   Walk w(g);
 
   if (warp >= 8 && warp < 8 + kXProd) {

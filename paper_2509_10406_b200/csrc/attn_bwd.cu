@@ -37,12 +37,22 @@ __device__ __forceinline__ void load_tile_f32(float* __restrict__ dst, const T* 
   }
 }
 
-// delta_t = sum_d dO[t][d] * O[t][d]; one warp per row.
+// delta_t = sum_d dO[t][d] * O[t][d]; one warp per row.  The first kernel of the pass: it also zeroes the bucketed gradients, which later
+// kernels add to, and the status words.
 template <class T, int D>
-__global__ void k_delta(const T* __restrict__ O, const T* __restrict__ dO, long long rows, float* __restrict__ delta) {
+__global__ void k_delta(const T* __restrict__ O, const T* __restrict__ dO, long long rows, float* __restrict__ delta, float* __restrict__ dK_perm,
+                        float* __restrict__ dV_perm, int32_t* __restrict__ clear) {
   const long long r = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
+  pdl_wait();
+  pdl_trigger();
+  if (clear != nullptr && blockIdx.x == 0 && threadIdx.x < kStatusWords) clear[threadIdx.x] = 0;
   if (r >= rows) return;
+  constexpr int Z = D / 4;                                 // 16-byte pieces of an fp32 row
+  if (lane < Z) {
+    st4(dK_perm + r * D + 4 * lane, make_float4(0.f, 0.f, 0.f, 0.f));
+    st4(dV_perm + r * D + 4 * lane, make_float4(0.f, 0.f, 0.f, 0.f));
+  }
   float s = 0.f;
 #pragma unroll
   for (int k = 0; k < D / 32; ++k) s = fmaf(to_f(O[r * D + lane + 32 * k]), to_f(dO[r * D + lane + 32 * k]), s);
@@ -58,6 +68,8 @@ __global__ void __launch_bounds__(kFlashThreads)
 k_local_bwd_dkdv(Dims dm, const T* __restrict__ Q, const T* __restrict__ K, const T* __restrict__ V,
                  const T* __restrict__ dO, const float* __restrict__ LSE, const float* __restrict__ delta,
                  float* __restrict__ dK_orig, float* __restrict__ dV_orig) {
+  pdl_wait();
+  pdl_trigger();
   constexpr int LD = D + Pad<T>::v;
   extern __shared__ __align__(16) unsigned char smraw[];
   T* Ks = (T*)smraw; T* Vs = Ks + kTile * LD; T* Qs = Vs + kTile * LD; T* dOs = Qs + kTile * LD;
@@ -127,6 +139,8 @@ __global__ void __launch_bounds__(kFlashThreads)
 k_local_bwd_dq(Dims dm, const T* __restrict__ Q, const T* __restrict__ K, const T* __restrict__ V,
                const T* __restrict__ dO, const float* __restrict__ LSE, const float* __restrict__ delta,
                float* __restrict__ dQacc) {
+  pdl_wait();
+  pdl_trigger();
   constexpr int LD = D + Pad<T>::v;
   extern __shared__ __align__(16) unsigned char smraw[];
   T* Ks = (T*)smraw; T* Vs = Ks + kTile * LD; T* Qs = Vs + kTile * LD; T* dOs = Qs + kTile * LD;
@@ -200,6 +214,8 @@ k_ret_bwd(Dims dm, const T* __restrict__ Q, const T* __restrict__ dO, const T* _
           const T* __restrict__ Vp, const float* __restrict__ LSE, const float* __restrict__ delta,
           const int32_t* __restrict__ off_k, const int32_t* __restrict__ goff, const int32_t* __restrict__ pairs,
           float* __restrict__ dq_part, float* __restrict__ dK_perm, float* __restrict__ dV_perm, int planes, int shares) {
+  pdl_wait();
+  pdl_trigger();
   constexpr int LD = D + Pad<T>::v;
   extern __shared__ __align__(16) unsigned char smraw[];
   T* Ks = (T*)smraw; T* Vs = Ks + kTile * LD; T* Qs = Vs + kTile * LD; T* dOs = Qs + kTile * LD;
@@ -317,6 +333,8 @@ k_far_bwd(Dims dm, const T* __restrict__ Q, const T* __restrict__ dO, const floa
           const float* __restrict__ LSE, const float* __restrict__ delta, const int32_t* __restrict__ off_q,
           const int32_t* __restrict__ perm_q, const int32_t* __restrict__ sel, SummPtrs sp, float* __restrict__ dQacc,
           float* __restrict__ dkappa, float* __restrict__ dnu, float* __restrict__ dS) {
+  pdl_wait();
+  pdl_trigger();
   constexpr int LD = D + 4;
   extern __shared__ __align__(16) unsigned char smraw[];
   float* kap = (float*)smraw; float* nus = kap + kTile * LD; float* qr = nus + kTile * LD; float* dOs = qr + kTile * LD;
@@ -483,6 +501,8 @@ k_summ_bwd(Dims dm, const T* __restrict__ Kp, const T* __restrict__ Vp, const in
            const int32_t* __restrict__ off_q, const float* __restrict__ qbar, const float* __restrict__ mu,
            const GT* __restrict__ dkappa, const GT* __restrict__ dnu, const float* __restrict__ dS,
            float* __restrict__ dK_perm, float* __restrict__ dV_perm, int per_block) {
+  pdl_wait();
+  pdl_trigger();
   // per_block = 1: mu and the gradients belong to the PER-BLOCK summaries (two-level retrieval): bucket b' feeds only
   // its own summary, so there is no suffix over the planes (the factor below is zero)
   constexpr int LD = D + 4;
@@ -609,6 +629,8 @@ k_summ_bwd(Dims dm, const T* __restrict__ Kp, const T* __restrict__ Vp, const in
 template <class T, int D, class PT>      // PT: element type of the per-(query, slot) dq partials
 __global__ void k_final_dq(Dims dm, const float* __restrict__ dQacc, const PT* __restrict__ dq_part,
                            const int32_t* __restrict__ sel, const int32_t* __restrict__ bsel, int use_ret, T* __restrict__ dQ) {
+  pdl_wait();
+  pdl_trigger();
   constexpr int LPQ = D / 8, QPW = 32 / LPQ, NA = 64 / LPQ;  // lanes of a query (8 dims each), queries of a warp: as in the forward merge
   const int pq = blockIdx.y, lane = threadIdx.x & 31, g = lane / LPQ, l = lane % LPQ, dd = l * 8;
   const int t_ = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * QPW + g;
@@ -650,6 +672,8 @@ template <class T, int D>
 __global__ void k_final_dkv(Dims dm, const int32_t* __restrict__ perm_k, const float* __restrict__ dK_orig,
                             const float* __restrict__ dV_orig, const float* __restrict__ dK_perm,
                             const float* __restrict__ dV_perm, int use_orig, T* __restrict__ dK, T* __restrict__ dV) {
+  pdl_wait();
+  pdl_trigger();
   const int pk = blockIdx.y, b_ = pk / dm.Hkv, g = pk % dm.Hkv;
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= (long long)dm.N * (D / 4)) return;
@@ -730,7 +754,7 @@ template <class T, int D>
 static int attn_bwd_t(const Dims& d, int dtype, const T* Q, const T* K, const T* V, const T* O, const float* LSE,
                       const T* dO, const int32_t* assign_q, const float* qbar, const int32_t* off_k,
                       const int32_t* perm_k, const void* summaries, const int32_t* sel, const int32_t* bsel, T* dQ, T* dK, T* dV,
-                      void* ws, cudaStream_t st) {
+                      void* ws, bool fresh_status, cudaStream_t st) {
   Arena ar(ws);
   BwdWs w = bwd_ws(d, ar);
   if (d.k2 == 0) bsel = nullptr;
@@ -743,11 +767,8 @@ static int attn_bwd_t(const Dims& d, int dtype, const T* Q, const T* K, const T*
   const size_t nd = (size_t)pq * d.N * d.D * sizeof(float);
   const long long rows = (long long)pq * d.N;
   prof_mark("k_delta", st);
-  k_delta<T, D><<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(O, dO, rows, w.delta);
-  MUSE_LAUNCH_OK();
-  prof_mark("memset", st);
-  MUSE_CUDA_OK(cudaMemsetAsync(w.dK_perm, 0, nd, st));
-  MUSE_CUDA_OK(cudaMemsetAsync(w.dV_perm, 0, nd, st));
+  MUSE_RC(launch_pdl(k_delta<T, D>, dim3((unsigned)((rows + 7) / 8)), 256, 0, st, O, dO, rows, w.delta, w.dK_perm, w.dV_perm,
+                     fresh_status ? w.status : (int32_t*)nullptr));
   const size_t sm4 = 4 * tile_bytes<T, D>() + ptile_bytes();
   constexpr bool kTensor = sizeof(T) == 2;      // bf16 mode runs the exact-attention parts on tcgen05
   if (d.causal && kTensor) {
@@ -758,10 +779,10 @@ static int attn_bwd_t(const Dims& d, int dtype, const T* Q, const T* K, const T*
     MUSE_CUDA_OK(cudaFuncSetAttribute(k_local_bwd_dq<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm4));
     dim3 grid(d.S * cdiv(d.Bs, kTile), pq);
     prof_mark("k_local_bwd_dkdv", st);
-    k_local_bwd_dkdv<T, D><<<grid, kFlashThreads, sm4, st>>>(d, Q, K, V, dO, LSE, w.delta, w.dK_orig, w.dV_orig);
+    MUSE_RC(launch_pdl(k_local_bwd_dkdv<T, D>, grid, kFlashThreads, sm4, st, d, Q, K, V, dO, LSE, w.delta, w.dK_orig, w.dV_orig));
     MUSE_LAUNCH_OK();
     prof_mark("k_local_bwd_dq", st);
-    k_local_bwd_dq<T, D><<<grid, kFlashThreads, sm4, st>>>(d, Q, K, V, dO, LSE, w.delta, w.dQacc);
+    MUSE_RC(launch_pdl(k_local_bwd_dq<T, D>, grid, kFlashThreads, sm4, st, d, Q, K, V, dO, LSE, w.delta, w.dQacc));
     MUSE_LAUNCH_OK();
   } else {
     prof_mark("memset", st);
@@ -785,8 +806,7 @@ static int attn_bwd_t(const Dims& d, int dtype, const T* Q, const T* K, const T*
         // fewer (cluster, head) CTAs than two rounds of the chip: split by plane, and the planes' pair tiles in two
         const bool split = d.Ck * pq < 2 * sm_count();
         const int planes = split && d.SB > 1 ? d.SB : 1, shares = planes > 1 ? 2 : 1;
-        k_ret_bwd<T, D><<<dim3(d.Ck, pq, planes * shares), kFlashThreads, sm4, st>>>(d, Q, dO, Kp, Vp, LSE, w.delta, off_k, ri.goff, ri.pairs,
-                                                                                   w.dq_part, w.dK_perm, w.dV_perm, planes, shares);
+        MUSE_RC(launch_pdl(k_ret_bwd<T, D>, dim3(d.Ck, pq, planes * shares), kFlashThreads, sm4, st, d, Q, dO, Kp, Vp, LSE, w.delta, off_k, ri.goff, ri.pairs, w.dq_part, w.dK_perm, w.dV_perm, planes, shares));
         MUSE_LAUNCH_OK();
       }
       use_ret = 1;
@@ -815,8 +835,7 @@ static int attn_bwd_t(const Dims& d, int dtype, const T* Q, const T* K, const T*
     } else {
     MUSE_CUDA_OK(cudaFuncSetAttribute(k_far_bwd<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsm));
     prof_mark("k_far_bwd", st);
-    k_far_bwd<T, D><<<dim3(d.Cq, d.SB, pq), kFlashThreads, fsm, st>>>(d, Q, dO, qbar, LSE, delta_far, w.off_q, w.perm_q, sel, sp,
-                                                                    w.dQacc, w.dkappa, w.dnu, w.dS);
+    MUSE_RC(launch_pdl(k_far_bwd<T, D>, dim3(d.Cq, d.SB, pq), kFlashThreads, fsm, st, d, Q, dO, qbar, LSE, delta_far, w.off_q, w.perm_q, sel, sp, w.dQacc, w.dkappa, w.dnu, w.dS));
     MUSE_LAUNCH_OK();
     }
     if (d.dipole) {
@@ -831,13 +850,11 @@ static int attn_bwd_t(const Dims& d, int dtype, const T* Q, const T* K, const T*
       typedef __nv_bfloat16 GB;
       MUSE_CUDA_OK(cudaFuncSetAttribute(k_summ_bwd<T, D, GB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssm));
       prof_mark("k_summ_bwd", st);
-      k_summ_bwd<T, D, GB><<<dim3(d.Ck, pq, d.Ck * pq < 2 * sm_count() ? d.SB : 1), kFlashThreads, ssm, st>>>(d, Kp, Vp, off_k, w.off_q, qbar, mu, (const GB*)w.dkappa,
-                                                                     (const GB*)w.dnu, w.dS, w.dK_perm, w.dV_perm, 0);
+      MUSE_RC(launch_pdl(k_summ_bwd<T, D, GB>, dim3(d.Ck, pq, d.Ck * pq < 2 * sm_count() ? d.SB : 1), kFlashThreads, ssm, st, d, Kp, Vp, off_k, w.off_q, qbar, mu, (const GB*)w.dkappa, (const GB*)w.dnu, w.dS, w.dK_perm, w.dV_perm, 0));
     } else {
       MUSE_CUDA_OK(cudaFuncSetAttribute(k_summ_bwd<T, D, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssm));
       prof_mark("k_summ_bwd", st);
-      k_summ_bwd<T, D, float><<<dim3(d.Ck, pq, d.Ck * pq < 2 * sm_count() ? d.SB : 1), kFlashThreads, ssm, st>>>(d, Kp, Vp, off_k, w.off_q, qbar, mu, w.dkappa, w.dnu, w.dS,
-                                                                        w.dK_perm, w.dV_perm, 0);
+      MUSE_RC(launch_pdl(k_summ_bwd<T, D, float>, dim3(d.Ck, pq, d.Ck * pq < 2 * sm_count() ? d.SB : 1), kFlashThreads, ssm, st, d, Kp, Vp, off_k, w.off_q, qbar, mu, w.dkappa, w.dnu, w.dS, w.dK_perm, w.dV_perm, 0));
     }
     MUSE_LAUNCH_OK();
     if (d.dipole) {
@@ -870,20 +887,18 @@ static int attn_bwd_t(const Dims& d, int dtype, const T* Q, const T* K, const T*
       const size_t ssm = (size_t)(5 * kTile * (D + 4) + kTile * kLDP) * sizeof(float);
       MUSE_CUDA_OK(cudaFuncSetAttribute(k_summ_bwd<T, D, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssm));
       prof_mark("k_summ_bwd", st);
-      k_summ_bwd<T, D, float><<<dim3(d.Ck, pq, d.Ck * pq < 2 * sm_count() ? d.SB : 1), kFlashThreads, ssm, st>>>(d, Kp, Vp, off_k, w.off_q, qbar, spb.mu, w.dkappa_b, w.dnu_b, w.dS_b,
-                                                                        w.dK_perm, w.dV_perm, 1);
+      MUSE_RC(launch_pdl(k_summ_bwd<T, D, float>, dim3(d.Ck, pq, d.Ck * pq < 2 * sm_count() ? d.SB : 1), kFlashThreads, ssm, st, d, Kp, Vp, off_k, w.off_q, qbar, spb.mu, w.dkappa_b, w.dnu_b, w.dS_b, w.dK_perm, w.dV_perm, 1));
       MUSE_LAUNCH_OK();
     }
   }
   prof_mark("k_final_dq", st);
   if (kTensor)
-    k_final_dq<T, D, __nv_bfloat16><<<dim3(cdiv(d.N, 8 * (256 / D)), pq), 256, 0, st>>>(d, w.dQacc, (const __nv_bfloat16*)w.dq_part, sel, bsel, use_ret, dQ);
+    MUSE_RC(launch_pdl(k_final_dq<T, D, __nv_bfloat16>, dim3(cdiv(d.N, 8 * (256 / D)), pq), 256, 0, st, d, w.dQacc, (const __nv_bfloat16*)w.dq_part, sel, bsel, use_ret, dQ));
   else
-    k_final_dq<T, D, float><<<dim3(cdiv(d.N, 8 * (256 / D)), pq), 256, 0, st>>>(d, w.dQacc, w.dq_part, sel, bsel, use_ret, dQ);
+    MUSE_RC(launch_pdl(k_final_dq<T, D, float>, dim3(cdiv(d.N, 8 * (256 / D)), pq), 256, 0, st, d, w.dQacc, w.dq_part, sel, bsel, use_ret, dQ));
   MUSE_LAUNCH_OK();
   prof_mark("k_final_dkv", st);
-  k_final_dkv<T, D><<<dim3(cdiv(d.N * (D / 4), 256), pk), 256, 0, st>>>(d, perm_k, w.dK_orig, w.dV_orig, w.dK_perm, w.dV_perm,
-                                                                       d.causal, dK, dV);
+  MUSE_RC(launch_pdl(k_final_dkv<T, D>, dim3(cdiv(d.N * (D / 4), 256), pk), 256, 0, st, d, perm_k, w.dK_orig, w.dV_orig, w.dK_perm, w.dV_perm, d.causal, dK, dV));
   MUSE_LAUNCH_OK();
   return MUSE_OK;
 }
@@ -891,10 +906,10 @@ static int attn_bwd_t(const Dims& d, int dtype, const T* Q, const T* K, const T*
 int attn_bwd(const Dims& d, int dtype, const void* Q, const void* K, const void* V, const void* O, const float* LSE,
              const void* dO, const int32_t* assign_q, const float* qbar, const int32_t* off_k, const int32_t* perm_k,
              const void* summaries, const int32_t* sel, const int32_t* bsel, void* dQ, void* dK, void* dV, void* ws,
-             cudaStream_t st) {
+             bool fresh_status, cudaStream_t st) {
   typedef __nv_bfloat16 bf;
 #define MUSE_BWD(TT, DD) attn_bwd_t<TT, DD>(d, dtype, (const TT*)Q, (const TT*)K, (const TT*)V, (const TT*)O, LSE, (const TT*)dO, \
-                                            assign_q, qbar, off_k, perm_k, summaries, sel, bsel, (TT*)dQ, (TT*)dK, (TT*)dV, ws, st)
+                                            assign_q, qbar, off_k, perm_k, summaries, sel, bsel, (TT*)dQ, (TT*)dK, (TT*)dV, ws, fresh_status, st)
   if (dtype == MUSE_F32) return d.D == 64 ? MUSE_BWD(float, 64) : MUSE_BWD(float, 128);
   return d.D == 64 ? MUSE_BWD(bf, 64) : MUSE_BWD(bf, 128);
 #undef MUSE_BWD

@@ -36,6 +36,8 @@ __global__ void __launch_bounds__(kFarThreads)
 k_far_fwd(Dims dm, const T* __restrict__ Q, const float* __restrict__ qbar, const int32_t* __restrict__ off_q,
           const int32_t* __restrict__ perm_q, SummPtrs sp, const int32_t* __restrict__ sel_in, int32_t* __restrict__ sel_out,
           float* __restrict__ o_far, float* __restrict__ lse_far) {
+  pdl_wait();
+  pdl_trigger();
   constexpr int LD = D + 4;
   const int RT = far_rows(dm.Ck), Ck = dm.Ck, LDS_ = Ck + 4;
   extern __shared__ float smf[];
@@ -221,9 +223,12 @@ static size_t far_smem(int Ck, int D) {
 }
 
 // Queries that see no far field (block 0 when causal, or m > 0 rows never visited): defaults.
-__global__ void k_far_defaults(Dims d, float* __restrict__ lse_far, int32_t* __restrict__ sel_out) {
+__global__ void k_far_defaults(Dims d, float* __restrict__ lse_far, int32_t* __restrict__ sel_out, int32_t* __restrict__ clear) {
+  pdl_wait();
+  pdl_trigger();
   const int pq = blockIdx.y;
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (clear != nullptr && blockIdx.x == 0 && pq == 0 && threadIdx.x < kStatusWords) clear[threadIdx.x] = 0;
   if (t >= d.N) return;
   if (query_plane(d, t) >= 0) return;
   lse_far[(size_t)pq * d.N + t] = -INFINITY;
@@ -240,6 +245,8 @@ __global__ void __launch_bounds__(kFlashThreads)
 k_ret_fwd(Dims dm, const T* __restrict__ Q, const T* __restrict__ Kp, const T* __restrict__ Vp,
           const int32_t* __restrict__ off_k, const int32_t* __restrict__ goff, const int32_t* __restrict__ pairs,
           float* __restrict__ o_part, float* __restrict__ l_part) {
+  pdl_wait();
+  pdl_trigger();
   constexpr int LD = D + Pad<T>::v;
   extern __shared__ __align__(16) unsigned char smraw[];
   T* Qs = (T*)smraw; T* Ks = Qs + kTile * LD; T* Vs = Ks + kTile * LD;
@@ -311,6 +318,8 @@ template <class T, int D>
 __global__ void __launch_bounds__(kFlashThreads)
 k_local_fwd(Dims dm, const T* __restrict__ Q, const T* __restrict__ K, const T* __restrict__ V,
             float* __restrict__ o_loc, float* __restrict__ lse_loc) {
+  pdl_wait();
+  pdl_trigger();
   constexpr int LD = D + Pad<T>::v;
   extern __shared__ __align__(16) unsigned char smraw[];
   T* Qs = (T*)smraw; T* Ks = Qs + kTile * LD; T* Vs = Ks + kTile * LD;
@@ -378,6 +387,8 @@ __global__ void k_merge(Dims dm, const float* __restrict__ o_far, const float* _
                         const PT* __restrict__ o_part, const float* __restrict__ l_part,
                         const float* __restrict__ o_near, const float* __restrict__ lse_near,
                         const int32_t* __restrict__ sel, const int32_t* __restrict__ bsel, T* __restrict__ O, float* __restrict__ LSE) {
+  pdl_wait();
+  pdl_trigger();
   constexpr int LPQ = D / 8, QPW = 32 / LPQ, NA = 64 / LPQ;                    // lanes of a query (8 dims each), queries of a warp
   const int pq = blockIdx.y, lane = threadIdx.x & 31, g = lane / LPQ, l = lane % LPQ, dd = l * 8;
   const int t_ = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * QPW + g;
@@ -504,6 +515,9 @@ static int attn_fwd_t(const Dims& d, const T* Q, const T* K, const T* V, const i
   if (two_level && !kTensorT<T>()) return MUSE_ERR_UNSUPPORTED;   // spatial block selection is built on the bf16 retrieval kernel
   const size_t fl_smem = 3 * tile_bytes<T, D>() + ptile_bytes();
   constexpr bool kTensor = sizeof(T) == 2;      // bf16 mode runs the exact-attention parts on tcgen05
+  // (the first kernel: also clears the status words)
+  prof_mark("k_far_defaults", st);
+  MUSE_RC(launch_pdl(k_far_defaults, dim3(cdiv(d.N, 256), pq), 256, 0, st, d, w.lse_far, sel, w.status));
   // local attention
   if (d.causal && kTensor) {
     int rc = local_fwd_tc(d, Q, K, V, w.o_loc, w.lse_loc, w.status, st);
@@ -511,12 +525,8 @@ static int attn_fwd_t(const Dims& d, const T* Q, const T* K, const T* V, const i
   } else if (d.causal) {
     MUSE_CUDA_OK(cudaFuncSetAttribute(k_local_fwd<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fl_smem));
     prof_mark("k_local_fwd", st);
-    k_local_fwd<T, D><<<dim3(d.S * cdiv(d.Bs, kTile), pq), kFlashThreads, fl_smem, st>>>(d, Q, K, V, w.o_loc, w.lse_loc);
-    MUSE_LAUNCH_OK();
+    MUSE_RC(launch_pdl(k_local_fwd<T, D>, dim3(d.S * cdiv(d.Bs, kTile), pq), kFlashThreads, fl_smem, st, d, Q, K, V, w.o_loc, w.lse_loc));
   }
-  prof_mark("k_far_defaults", st);
-  k_far_defaults<<<dim3(cdiv(d.N, 256), pq), 256, 0, st>>>(d, w.lse_far, sel);
-  MUSE_LAUNCH_OK();
   if (d.SB > 0) {
     const SortSide side = {assign_q, w.off_q, w.perm_q, pq, d.Cq, 0};
     int rc = bucket_sort(&side, 1, d.N, d.S, d.Bs, st);
@@ -528,8 +538,7 @@ static int attn_fwd_t(const Dims& d, const T* Q, const T* K, const T* V, const i
       const size_t fs = far_smem(d.Ck, D);
       MUSE_CUDA_OK(cudaFuncSetAttribute(k_far_fwd<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fs));
       prof_mark("k_far_fwd", st);
-      k_far_fwd<T, D><<<dim3(d.Cq, d.SB, pq), kFarThreads, fs, st>>>(
-          d, Q, qbar, w.off_q, w.perm_q, summ_ptrs(L, base), sel_in, sel, w.o_far, w.lse_far);
+      MUSE_RC(launch_pdl(k_far_fwd<T, D>, dim3(d.Cq, d.SB, pq), kFarThreads, fs, st, d, Q, qbar, w.off_q, w.perm_q, summ_ptrs(L, base), sel_in, sel, w.o_far, w.lse_far));
       MUSE_LAUNCH_OK();
     }
     if (two_level) {
@@ -560,19 +569,16 @@ static int attn_fwd_t(const Dims& d, const T* Q, const T* K, const T* V, const i
       } else {
         MUSE_CUDA_OK(cudaFuncSetAttribute(k_ret_fwd<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fl_smem));
         prof_mark("k_ret_fwd", st);
-        k_ret_fwd<T, D><<<dim3(d.Ck, d.SB, pq), kFlashThreads, fl_smem, st>>>(d, Q, Kp, Vp, off_k, ri.goff, ri.pairs, w.o_part, w.l_part);
+        MUSE_RC(launch_pdl(k_ret_fwd<T, D>, dim3(d.Ck, d.SB, pq), kFlashThreads, fl_smem, st, d, Q, Kp, Vp, off_k, ri.goff, ri.pairs, w.o_part, w.l_part));
         MUSE_LAUNCH_OK();
       }
     }
   }
   prof_mark("k_merge", st);
   if (kTensor)
-    k_merge<T, D, __nv_bfloat16><<<dim3(cdiv(d.N, 8 * (256 / D)), pq), 256, 0, st>>>(d, w.o_far, w.lse_far, w.o_loc, w.lse_loc,
-                                                                       (const __nv_bfloat16*)w.o_part, w.l_part, two_level ? w.o_near : nullptr,
-                                                                       two_level ? w.lse_near : nullptr, sel, bsel, O, LSE);
+    MUSE_RC(launch_pdl(k_merge<T, D, __nv_bfloat16>, dim3(cdiv(d.N, 8 * (256 / D)), pq), 256, 0, st, d, w.o_far, w.lse_far, w.o_loc, w.lse_loc, (const __nv_bfloat16*)w.o_part, w.l_part, two_level ? w.o_near : nullptr, two_level ? w.lse_near : nullptr, sel, bsel, O, LSE));
   else
-    k_merge<T, D, float><<<dim3(cdiv(d.N, 8 * (256 / D)), pq), 256, 0, st>>>(d, w.o_far, w.lse_far, w.o_loc, w.lse_loc, w.o_part, w.l_part, nullptr, nullptr,
-                                                               sel, nullptr, O, LSE);
+    MUSE_RC(launch_pdl(k_merge<T, D, float>, dim3(cdiv(d.N, 8 * (256 / D)), pq), 256, 0, st, d, w.o_far, w.lse_far, w.o_loc, w.lse_loc, w.o_part, w.l_part, nullptr, nullptr, sel, nullptr, O, LSE));
   MUSE_LAUNCH_OK();
   return MUSE_OK;
 }
@@ -586,15 +592,14 @@ static int far_fwd_again_t(const Dims& d, int dtype, const T* Q, const float* qb
                            cudaStream_t st) {
   const int pq = d.B * d.Hq;
   prof_mark("k_far_defaults", st);
-  k_far_defaults<<<dim3(cdiv(d.N, 256), pq), 256, 0, st>>>(d, lse_far, sel_tmp);
-  MUSE_LAUNCH_OK();
+  MUSE_RC(launch_pdl(k_far_defaults, dim3(cdiv(d.N, 256), pq), 256, 0, st, d, lse_far, sel_tmp, (int32_t*)nullptr));
   if (d.SB == 0) return MUSE_OK;
   if (far_fwd_tc_supported(d, dtype) && !path_forced(kForceFarSimt))
     return far_fwd_tc(d, sp, Q, off_q, perm_q, sel_in, sel_tmp, o_far, lse_far, status, st);
   const size_t fs = far_smem(d.Ck, D);
   MUSE_CUDA_OK(cudaFuncSetAttribute(k_far_fwd<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fs));
   prof_mark("k_far_fwd", st);
-  k_far_fwd<T, D><<<dim3(d.Cq, d.SB, pq), kFarThreads, fs, st>>>(d, Q, qbar, off_q, perm_q, sp, sel_in, sel_tmp, o_far, lse_far);
+  MUSE_RC(launch_pdl(k_far_fwd<T, D>, dim3(d.Cq, d.SB, pq), kFarThreads, fs, st, d, Q, qbar, off_q, perm_q, sp, sel_in, sel_tmp, o_far, lse_far));
   MUSE_LAUNCH_OK();
   return MUSE_OK;
 }

@@ -38,6 +38,8 @@ __global__ void __launch_bounds__(BqLay<D>::kThreads, 2)
 k_block_select_q(Dims dm, const bf16* __restrict__ Q, const int32_t* __restrict__ off_q, const int32_t* __restrict__ perm_q,
                  const int32_t* __restrict__ sel, SummPtrs sp, const int32_t* __restrict__ bsel_in, int32_t* __restrict__ bsel_out,
                  float* __restrict__ o_near, float* __restrict__ lse_near) {
+  pdl_wait();
+  pdl_trigger();
   typedef BqLay<D> L;
   constexpr int kThreads = L::kThreads, kWarps = kThreads / 32, LD = L::LD, EPL = D / 32, KS = D / 16, G = kNbGroup;
   extern __shared__ __align__(16) unsigned char bq_smem[];
@@ -251,8 +253,7 @@ static int block_select_q_d(const Dims& d, const void* Q, const int32_t* off_q, 
   const int per = d.Cq * d.B * d.Hq, chunk = std::min(L::kQ, kNbPairs / d.m);
   const int share = std::max(1, std::min((4 * sm_count() + per - 1) / per, (d.N / d.Cq + chunk - 1) / chunk));
   prof_mark("k_block_select_q", st);
-  k_block_select_q<D><<<dim3(d.Cq, d.B * d.Hq, share), L::kThreads, smem, st>>>(d, (const bf16*)Q, off_q, perm_q, sel, sp, bsel_in, bsel_out, o_near,
-                                                                             lse_near);
+  MUSE_RC(launch_pdl(k_block_select_q<D>, dim3(d.Cq, d.B * d.Hq, share), L::kThreads, smem, st, d, (const bf16*)Q, off_q, perm_q, sel, sp, bsel_in, bsel_out, o_near, lse_near));
   MUSE_LAUNCH_OK();
   return MUSE_OK;
 }

@@ -28,11 +28,12 @@ __device__ __forceinline__ void split_centre(const LloydSide& sd, size_t e, floa
 // per centre.  The padding of cnorm is set to infinity here, once per call.
 template <class T>
 __global__ void __launch_bounds__(256)
-k_init_centres(const __grid_constant__ LloydSides g, int D, int init_mode, uint64_t seed) {
+k_init_centres(const __grid_constant__ LloydSides g, int D, int init_mode, uint64_t seed, int32_t* __restrict__ clear) {
   const int lane = threadIdx.x & 31;
   long long e = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
+  if (clear != nullptr && blockIdx.x == 0 && threadIdx.x < kStatusWords) clear[threadIdx.x] = 0;
   const LloydSide& sd = side_of_centre(g, e);
   if (e >= (long long)sd.problems * sd.C) return;
   const int prob = (int)(e / sd.C), c = (int)(e % sd.C);
@@ -83,8 +84,8 @@ k_assign(const __grid_constant__ LloydSides g, int distances) {
   if (second) prob -= g.s[0].problems;
   const int C = sd.C, row0 = blockIdx.x * ROWS;
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const float* Xp = (const float*)sd.X + (size_t)prob * N * D;
   const float* Cp = sd.centres + (size_t)prob * C * D;
   const float* cnp = sd.cnorm + cnorm_index(prob, 0, C);
@@ -206,8 +207,8 @@ k_update(const __grid_constant__ LloydSides g) {
   const T* Xp = (const T*)sd.X + (size_t)prob * N * D + q * VEC;
   const int32_t* o = sd.off + (size_t)prob * (C * S + 1);
   const int32_t* pm = sd.perm + (size_t)prob * N;
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   float s[VEC];
 #pragma unroll
   for (int k = 0; k < VEC; ++k) s[k] = 0.f;
@@ -267,7 +268,11 @@ k_update(const __grid_constant__ LloydSides g) {
 
 template <class T, int D>
 static int lloyd_t(LloydSides& g, const Dims& d, int nsides, int init_mode, uint64_t seed, int T_iters, int* status, cudaStream_t st) {
+  // the status words are cleared by the first kernel of the call (k-means++ reports into them, so before it by a memset)
+  int32_t* clear = status;
   if (init_mode == MUSE_INIT_KMEANSPP) {
+    MUSE_CUDA_OK(cudaMemsetAsync(status, 0, kStatusWords * sizeof(int32_t), st));
+    clear = nullptr;
     // the draws borrow two arrays that the iterations only fill later: perm as the running minimum distance
     // [problems, N] fp32, off (at least C + 1 words per problem) as the drawn indices [problems, C]
     KmeansppSide pp[2];
@@ -287,7 +292,7 @@ static int lloyd_t(LloydSides& g, const Dims& d, int nsides, int init_mode, uint
     sort[k] = SortSide{s.assign, s.off, s.perm, s.problems, s.C, s.kind};
   }
   prof_mark("k_init_centres", st);
-  MUSE_RC(launch_pdl(k_init_centres<T>, dim3((unsigned)((centres + 7) / 8)), 256, 0, st, g, D, init_mode, seed));
+  MUSE_RC(launch_pdl(k_init_centres<T>, dim3((unsigned)((centres + 7) / 8)), 256, 0, st, g, D, init_mode, seed, clear));
   for (int it = 0; it <= T_iters; ++it) {
     const bool last = it == T_iters;
     if (sizeof(T) == 2) {                      // bf16 inputs: distances on the tensor cores

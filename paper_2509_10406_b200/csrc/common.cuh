@@ -134,9 +134,11 @@ __device__ __forceinline__ float warp_max(float v) {
 
 // ---- launches -------------------------------------------------------------------------------
 // Programmatic dependent launch: a kernel started with launch_pdl may begin while its predecessor on the stream still
-// runs; it must call pdl_wait() before its first access to global memory (that wait covers the whole predecessor,
-// which in turn waited for its own).  pdl_trigger() lets the successor begin.  A stage here is a chain of short
-// kernels, and this takes the launch latency and the block set-up (barriers, tensor memory) out of the chain.
+// runs; every CTA must call pdl_wait() before its first access to global memory and before it returns (that wait covers the
+// whole predecessor, which in turn waited for its own).  pdl_trigger() lets the successor begin once every CTA of the kernel
+// has called it or has ended.  It comes after pdl_wait(), so that never more than two kernels overlap, and after the
+// allocation of tensor memory, which a successor that allocates before its own wait could otherwise hold for good.  A stage
+// here is a chain of short kernels, and this takes the launch latency (and for some the block set-up) out of the chain.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -216,7 +218,7 @@ bool path_forced(unsigned bit);
 // kind 0 (queries): segments (block, cluster) contiguous, off [C*S+1] by block * C + cluster;
 // kind 1 (keys): a cluster's blocks are one contiguous run, off [C*S+1] by cluster * S + block.
 struct SortSide { const int32_t* assign; int32_t* off; int32_t* perm; int problems, C, kind; };
-int bucket_sort(const SortSide* sides, int nsides, int N, int S, int Bs, cudaStream_t st);
+int bucket_sort(const SortSide* sides, int nsides, int N, int S, int Bs, cudaStream_t st, int32_t* clear = nullptr);   // clear: status words to zero
 
 // Lloyd iterations of one or both sides at once (kind 0 queries, 1 keys); the scratch pointers are carved from a
 // workspace by lloyd_side_ws.  cnorm is padded per problem to whole tiles of kAsgTile centres (infinity in the padding).
@@ -348,7 +350,7 @@ size_t attn_fwd_ws_bytes(const Dims& d, int dtype);
 int attn_bwd(const Dims& d, int dtype, const void* Q, const void* K, const void* V, const void* O,
              const float* LSE, const void* dO, const int32_t* assign_q, const float* qbar,
              const int32_t* off_k, const int32_t* perm_k, const void* summaries, const int32_t* sel, const int32_t* bsel,
-             void* dQ, void* dK, void* dV, void* ws, cudaStream_t st);
+             void* dQ, void* dK, void* dV, void* ws, bool fresh_status, cudaStream_t st);       // fresh_status: clear the status words
 size_t attn_bwd_ws_bytes(const Dims& d, int dtype);
 
 // retrieval inverse index, shared by forward and backward: groups the (query, slot) pairs by

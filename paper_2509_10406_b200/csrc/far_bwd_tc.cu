@@ -61,6 +61,7 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
              const int32_t* __restrict__ off_q, const int32_t* __restrict__ perm_q, const int32_t* __restrict__ sel,
              const float* __restrict__ beta, const float* __restrict__ mu, float* __restrict__ dQacc, bf16* __restrict__ dkappa,
              bf16* __restrict__ dnu, float* __restrict__ dS, int grad_by_key_cluster, int* __restrict__ status) {
+  pdl_wait();
   using namespace fb;
   typedef Lay<D> LY;
   constexpr int kTile = LY::kTile, kRows = LY::kRows, oHi = LY::oHi, oLo = LY::oLo, oNu = LY::oNu, oQ = LY::oQ, oDO = LY::oDO,
@@ -111,6 +112,7 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
+  pdl_trigger();                                           // (tensor memory has been allocated)
   const uint32_t tbase = tbase_s, tlane = tbase + ((uint32_t)((warp & 3) * 32) << 16);
   uint32_t ph_full = 0, ph1 = 0, ph2 = 0, ph3 = 0, ph_st = 0;
   const bool cw = warp < 8;                               // compute warp
@@ -468,15 +470,11 @@ int far_bwd_tc(const Dims& d, const SummPtrs& sp, const void* Q, const void* dO,
   if (d.D == 128) {
     const size_t smem = (size_t)fb::Lay<128>::oMask + mask_bytes + 1024;
     MUSE_CUDA_OK(cudaFuncSetAttribute(k_far_bwd_tc<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k_far_bwd_tc<128><<<dim3(d.Cq, d.SB, d.B * d.Hq), fb::THREADS, smem, st>>>(
-        d, khi, klo, nu, gka, gnu, (const bf16*)Q, (const bf16*)dO, qbar, LSE, delta, off_q, perm_q, sel, sp.beta, sp.mu, dQacc, (bf16*)dkappa,
-        (bf16*)dnu, dS, grad_by_key_cluster, status);
+    MUSE_RC(launch_pdl(k_far_bwd_tc<128>, dim3(d.Cq, d.SB, d.B * d.Hq), fb::THREADS, smem, st, d, khi, klo, nu, gka, gnu, (const bf16*)Q, (const bf16*)dO, qbar, LSE, delta, off_q, perm_q, sel, sp.beta, sp.mu, dQacc, (bf16*)dkappa, (bf16*)dnu, dS, grad_by_key_cluster, status));
   } else {
     const size_t smem = (size_t)fb::Lay<64>::oMask + mask_bytes + 1024;
     MUSE_CUDA_OK(cudaFuncSetAttribute(k_far_bwd_tc<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k_far_bwd_tc<64><<<dim3(d.Cq, d.SB, d.B * d.Hq), fb::THREADS, smem, st>>>(
-        d, khi, klo, nu, gka, gnu, (const bf16*)Q, (const bf16*)dO, qbar, LSE, delta, off_q, perm_q, sel, sp.beta, sp.mu, dQacc, (bf16*)dkappa,
-        (bf16*)dnu, dS, grad_by_key_cluster, status);
+    MUSE_RC(launch_pdl(k_far_bwd_tc<64>, dim3(d.Cq, d.SB, d.B * d.Hq), fb::THREADS, smem, st, d, khi, klo, nu, gka, gnu, (const bf16*)Q, (const bf16*)dO, qbar, LSE, delta, off_q, perm_q, sel, sp.beta, sp.mu, dQacc, (bf16*)dkappa, (bf16*)dnu, dS, grad_by_key_cluster, status));
   }
   MUSE_LAUNCH_OK();
   return MUSE_OK;

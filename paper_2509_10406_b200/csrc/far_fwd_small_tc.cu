@@ -83,7 +83,6 @@ k_far_fwd_small(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __gri
     for (int t = 0; t < NS; ++t) { tc::mbar_init(&bars.full[t], 1); tc::mbar_init(&bars.empty[t], 1); }
     tc::mbar_init(&bars.nu, 1); tc::mbar_init(&bars.done, 1); tc::mbar_init_fence();
   }
-  pdl_trigger();
   pdl_wait();
   const int32_t* oq = off_q + (size_t)pq * (dm.S * dm.Cq + 1) + (size_t)blk * dm.Cq + i;
   const int p0 = oq[0], p1 = oq[1];
@@ -115,6 +114,7 @@ k_far_fwd_small(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __gri
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
+  pdl_trigger();
   const uint32_t tbase = tbase_s;
   bool ok = true;
   uint32_t done_ph = 0, nu_ph = 0, cnt = 0;                // cnt: kappa tiles of earlier passes

@@ -232,6 +232,7 @@ k_far_fwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
              const int32_t* __restrict__ perm_q, const float* __restrict__ mu, const float* __restrict__ beta,
              const int32_t* __restrict__ sel_in, int32_t* __restrict__ sel_out, float* __restrict__ o_far,
              float* __restrict__ lse_far, int p_bytes, int sc_bytes, int nsA, int nsD, int tcols, int* __restrict__ status) {
+  pdl_wait();
   constexpr int NT = FQ * 32, NTG = FQ / 4, KT = 16 / NTG;   // threads; tile groups in the TMEM read-out; cluster tiles per group
   constexpr int kTileBytes = kFJ * D * 2, G = D / 64;        // one [128 clusters][D] bf16 operand tile; 128-byte column groups of a row
   extern __shared__ __align__(1024) unsigned char sm_raw[];
@@ -287,6 +288,7 @@ k_far_fwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
+  pdl_trigger();                                           // (tensor memory has been allocated)
   const uint32_t tbase = tbase_s;
   uint32_t cntA = 0, cntD = 0, done_ph = 0;   // tiles of the earlier passes (same in every thread); phase of `done`
   bool ok = true;
@@ -579,9 +581,8 @@ int far_fwd_tc(const Dims& d, const SummPtrs& sp, const void* Q, const int32_t* 
   while (tcols < FR * (CkP / kFJ)) tcols *= 2;
 #define MUSE_FAR_FWD_LAUNCH(FR_, FQ_, D_, NK_, MB_)                                                                              \
   do {                                                                                                                         \
-    MUSE_CUDA_OK(cudaFuncSetAttribute(k_far_fwd_tc<FR_, FQ_, D_, NK_, MB_>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
-    k_far_fwd_tc<FR_, FQ_, D_, NK_, MB_><<<dim3(d.Cq, d.SB, d.B * d.Hq), FQ_ * 32, smem, st>>>(                                   \
-        d, khi, klo, nu, (const bf16*)Q, off_q, perm_q, sp.mu, sp.beta, sel_in, sel_out, o_far, lse_far, p_bytes, sc_bytes, nsA, nsD, tcols, status); \
+    MUSE_RC(launch_pdl(k_far_fwd_tc<FR_, FQ_, D_, NK_, MB_>, dim3(d.Cq, d.SB, d.B * d.Hq), FQ_ * 32, smem, st,                     \
+        d, khi, klo, nu, (const bf16*)Q, off_q, perm_q, sp.mu, sp.beta, sel_in, sel_out, o_far, lse_far, p_bytes, sc_bytes, nsA, nsD, tcols, status));   \
   } while (0)
   if (wide) { if (d.D == 128) MUSE_FAR_FWD_LAUNCH(32, 8, 128, 64, 1); else MUSE_FAR_FWD_LAUNCH(32, 8, 64, 64, 1); }
   else if (d.Ck <= 256) { if (d.D == 128) MUSE_FAR_FWD_LAUNCH(64, 16, 128, 8, 2); else MUSE_FAR_FWD_LAUNCH(64, 16, 64, 8, 2); }

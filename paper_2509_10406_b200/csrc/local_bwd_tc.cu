@@ -84,8 +84,8 @@ k_local_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_a, const __grid_c
   tc::fence_after_sync();
   const uint32_t tbase = tbase_s;
   bool ok = true;
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
 
   if (warp == MW + 1) {                                    // ---- loads
     const int rrow = (KIND == 0 ? pk : pq) * dm.N + r0, crow = (KIND == 0 ? pq : pk) * dm.N + c_lo;

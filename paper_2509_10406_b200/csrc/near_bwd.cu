@@ -59,6 +59,8 @@ k_near_bwd(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ dO, con
            const float* __restrict__ delta, const int32_t* __restrict__ off_q, const int32_t* __restrict__ perm_q,
            const int32_t* __restrict__ sel, const int32_t* __restrict__ bsel, SummPtrs sp, float* __restrict__ dQacc,
            float* __restrict__ dkappa_b, float* __restrict__ dnu_b, float* __restrict__ dS_b, int grad_ji) {
+  pdl_wait();
+  pdl_trigger();
   // grad_ji: the gradient entries are laid out [plane][j][i] (what the tensor-core key-side kernel reads) instead of [plane][i][j]
   typedef NbLay<D> L;
   constexpr int kThreads = L::kThreads, kWarps = kThreads / 32, LD = L::LD, EPL = D / 32, KS = D / 16, G = kNbGroup;
@@ -297,6 +299,8 @@ k_near_bwd(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ dO, con
 
 // fp32 gradient rows -> bf16 (the operand type of the tensor-core key-side kernel), same layout
 __global__ void k_grad_to_bf16(const float* __restrict__ in, long long n4, __nv_bfloat16* __restrict__ out) {
+  pdl_wait();
+  pdl_trigger();
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= n4) return;
   st4(out + 4 * e, ld4(in + 4 * e));
@@ -305,7 +309,7 @@ __global__ void k_grad_to_bf16(const float* __restrict__ in, long long n4, __nv_
 int grad_to_bf16(const float* in, size_t n, void* out, cudaStream_t st) {
   const long long n4 = (long long)(n / 4);
   prof_mark("k_grad_to_bf16", st);
-  k_grad_to_bf16<<<(unsigned)((n4 + 255) / 256), 256, 0, st>>>(in, n4, (__nv_bfloat16*)out);
+  MUSE_RC(launch_pdl(k_grad_to_bf16, dim3((unsigned)((n4 + 255) / 256)), 256, 0, st, in, n4, (__nv_bfloat16*)out));
   MUSE_LAUNCH_OK();
   return MUSE_OK;
 }
@@ -321,8 +325,7 @@ static int near_bwd_d(const Dims& d, const void* Q, const void* dO, const float*
   const int per = d.Cq * d.B * d.Hq, chunk = std::min(L::kQ, kNbPairs / d.m);
   const int share = std::max(1, std::min((2 * sm_count() + per - 1) / per, (d.N / d.Cq + chunk - 1) / chunk));
   prof_mark("k_near_bwd", st);
-  k_near_bwd<D><<<dim3(d.Cq, d.B * d.Hq, share), L::kThreads, smem, st>>>(d, (const bf16*)Q, (const bf16*)dO, qbar, LSE, delta, off_q, perm_q, sel, bsel,
-                                                                       sp, dQacc, dkappa_b, dnu_b, dS_b, grad_ji);
+  MUSE_RC(launch_pdl(k_near_bwd<D>, dim3(d.Cq, d.B * d.Hq, share), L::kThreads, smem, st, d, (const bf16*)Q, (const bf16*)dO, qbar, LSE, delta, off_q, perm_q, sel, bsel, sp, dQacc, dkappa_b, dnu_b, dS_b, grad_ji));
   MUSE_LAUNCH_OK();
   return MUSE_OK;
 }

@@ -58,6 +58,7 @@ k_ret_bwd_sweeps(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ d
                    const bf16* __restrict__ Vp, const float* __restrict__ LSE, const float* __restrict__ delta,
                    const int32_t* __restrict__ off_k, const __grid_constant__ RetIndex ri,
                    bf16* __restrict__ dq_part, float* __restrict__ dK_perm, float* __restrict__ dV_perm, int* __restrict__ status) {
+  pdl_wait();
   using namespace rs;
   typedef Lay<D> LY;
   constexpr int kTile = LY::kTile, kPG = LY::kPG, oK = LY::oK, oV = LY::oV, oHalf = LY::oHalf, kHalf = LY::kHalf;
@@ -100,6 +101,7 @@ k_ret_bwd_sweeps(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ d
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
+  pdl_trigger();                                           // (tensor memory has been allocated)
   const bf16* Qb = Q + (size_t)pq * dm.N * D;
   const bf16* dOb = dO + (size_t)pq * dm.N * D;
   const bf16* Kb = Kp + ((size_t)pk * dm.N + k0) * D;
@@ -400,12 +402,10 @@ int ret_bwd_short_tc(const Dims& d, const void* Q, const void* dO, const void* K
   const dim3 grid(ri.cap, d.B * d.Hq);
   if (d.D == 128) {
     MUSE_CUDA_OK(cudaFuncSetAttribute(k_ret_bwd_sweeps<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, rs::Lay<128>::kSmem));
-    k_ret_bwd_sweeps<128><<<grid, rs::kThreads, rs::Lay<128>::kSmem, st>>>(
-        d, (const bf16*)Q, (const bf16*)dO, (const bf16*)Kp, (const bf16*)Vp, LSE, delta, off_k, ri, (bf16*)dq_part, dK_perm, dV_perm, status);
+    MUSE_RC(launch_pdl(k_ret_bwd_sweeps<128>, grid, rs::kThreads, rs::Lay<128>::kSmem, st, d, (const bf16*)Q, (const bf16*)dO, (const bf16*)Kp, (const bf16*)Vp, LSE, delta, off_k, ri, (bf16*)dq_part, dK_perm, dV_perm, status));
   } else {
     MUSE_CUDA_OK(cudaFuncSetAttribute(k_ret_bwd_sweeps<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, rs::Lay<64>::kSmem));
-    k_ret_bwd_sweeps<64><<<grid, rs::kThreads, rs::Lay<64>::kSmem, st>>>(
-        d, (const bf16*)Q, (const bf16*)dO, (const bf16*)Kp, (const bf16*)Vp, LSE, delta, off_k, ri, (bf16*)dq_part, dK_perm, dV_perm, status);
+    MUSE_RC(launch_pdl(k_ret_bwd_sweeps<64>, grid, rs::kThreads, rs::Lay<64>::kSmem, st, d, (const bf16*)Q, (const bf16*)dO, (const bf16*)Kp, (const bf16*)Vp, LSE, delta, off_k, ri, (bf16*)dq_part, dK_perm, dV_perm, status));
   }
   MUSE_LAUNCH_OK();
   return MUSE_OK;

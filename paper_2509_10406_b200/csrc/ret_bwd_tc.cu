@@ -84,6 +84,7 @@ k_ret_bwd_dkdv(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_c
                const bf16* __restrict__ dO, const float* __restrict__ LSE, const float* __restrict__ delta, const int32_t* __restrict__ off_k,
                const __grid_constant__ RetIndex ri, float* __restrict__ dK_perm, float* __restrict__ dV_perm,
                int* __restrict__ status) {
+  pdl_wait();
   using namespace rk;
   typedef Lay<D> LY;
   constexpr int kRow = LY::kRow, kCol = LY::kCol, NW = LY::NW, NS = LY::NS, G = D / 64, MW = NW * 4, CPR = D / 8;
@@ -112,6 +113,7 @@ k_ret_bwd_dkdv(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_c
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
+  pdl_trigger();                                           // (tensor memory has been allocated)
   const uint32_t tbase = tbase_s;
   bool ok_ = true;
   auto wait = [&](uint64_t* bar, uint32_t parity) { if (ok_ && !tc::mbar_wait(bar, parity)) ok_ = false; };
@@ -341,6 +343,7 @@ __global__ void __launch_bounds__(rq::Lay<D>::kThreads, 1)
 k_ret_bwd_dq(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v, const bf16* __restrict__ Q,
              const bf16* __restrict__ dO, const float* __restrict__ LSE, const float* __restrict__ delta, const int32_t* __restrict__ off_k,
              const __grid_constant__ RetIndex ri, bf16* __restrict__ dq_part, int* __restrict__ status) {
+  pdl_wait();
   using namespace rq;
   typedef Lay<D> LY;
   constexpr int kRow = LY::kRow, kCol = LY::kCol, NW = LY::NW, NSK = LY::NSK, NSV = LY::NSV, NQ = LY::NQ, G = D / 64, CPR = D / 8;
@@ -372,6 +375,7 @@ k_ret_bwd_dq(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_con
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
+  pdl_trigger();                                           // (tensor memory has been allocated)
   const uint32_t tbase = tbase_s;
   bool ok_ = true;
   auto wait = [&](uint64_t* bar, uint32_t parity) { if (ok_ && !tc::mbar_wait(bar, parity)) ok_ = false; };
@@ -613,13 +617,11 @@ static int ret_bwd_d(const Dims& d, const void* Q, const void* dO, const void* K
   const dim3 grid(ri.cap, d.B * d.Hq);
   prof_mark("k_ret_bwd_pairs_tc", st);
   MUSE_CUDA_OK(cudaFuncSetAttribute(k_ret_bwd_dkdv<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, rk::Lay<D>::total));
-  k_ret_bwd_dkdv<D><<<grid, rk::Lay<D>::kThreads, rk::Lay<D>::total, st>>>(d, k[0], v[0], (const bf16*)Q, (const bf16*)dO, LSE, delta, off_k, ri,
-                                                                       dK_perm, dV_perm, status);
+  MUSE_RC(launch_pdl(k_ret_bwd_dkdv<D>, grid, rk::Lay<D>::kThreads, rk::Lay<D>::total, st, d, k[0], v[0], (const bf16*)Q, (const bf16*)dO, LSE, delta, off_k, ri, dK_perm, dV_perm, status));
   MUSE_LAUNCH_OK();
   prof_mark("k_ret_bwd_dq", st);
   MUSE_CUDA_OK(cudaFuncSetAttribute(k_ret_bwd_dq<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, rq::Lay<D>::total));
-  k_ret_bwd_dq<D><<<grid, rq::Lay<D>::kThreads, rq::Lay<D>::total, st>>>(d, k[1], v[1], (const bf16*)Q, (const bf16*)dO, LSE, delta, off_k, ri,
-                                                                     (bf16*)dq_part, status);
+  MUSE_RC(launch_pdl(k_ret_bwd_dq<D>, grid, rq::Lay<D>::kThreads, rq::Lay<D>::total, st, d, k[1], v[1], (const bf16*)Q, (const bf16*)dO, LSE, delta, off_k, ri, (bf16*)dq_part, status));
   MUSE_LAUNCH_OK();
   return MUSE_OK;
 }

@@ -48,6 +48,7 @@ __global__ void __launch_bounds__(rl::Lay<D>::kThreads, 1)
 k_ret_fwd_long(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v, const bf16* __restrict__ Q,
                const int32_t* __restrict__ off_k, const __grid_constant__ RetIndex ri, bf16* __restrict__ o_part, float* __restrict__ l_part,
                int* __restrict__ status) {
+  pdl_wait();
   using namespace rl;
   typedef Lay<D> LY;
   constexpr int kTile = LY::kTile, NS = LY::NS, NB = LY::NB, NQ = LY::NQ, H = LY::H, kSoft = LY::kSoft, MW = kSoft / 32, G = D / 64, CPR = D / 8;
@@ -85,6 +86,7 @@ k_ret_fwd_long(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_c
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
+  pdl_trigger();                                           // (tensor memory has been allocated)
   const uint32_t tbase = tbase_s;
   bool ok_ = true;                                         // false once a bounded wait ran out (every role still walks all its units)
   auto wait = [&](uint64_t* bar, uint32_t parity) { if (ok_ && !tc::mbar_wait(bar, parity)) ok_ = false; };
@@ -362,7 +364,7 @@ static int ret_fwd_long_d(const Dims& d, const void* Q, const void* Kp, const vo
   MUSE_RC(make_tmap_bf16_rows(&v, Vp, (uint64_t)d.B * d.Hkv * d.N, D, rl::kKeys));
   MUSE_CUDA_OK(cudaFuncSetAttribute(k_ret_fwd_long<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, rl::Lay<D>::total));
   prof_mark("k_ret_fwd_pairs_tc", st);
-  k_ret_fwd_long<D><<<dim3(ri.cap, d.B * d.Hq), rl::Lay<D>::kThreads, rl::Lay<D>::total, st>>>(d, k, v, (const bf16*)Q, off_k, ri, (bf16*)o_part, l_part, status);
+  MUSE_RC(launch_pdl(k_ret_fwd_long<D>, dim3(ri.cap, d.B * d.Hq), rl::Lay<D>::kThreads, rl::Lay<D>::total, st, d, k, v, (const bf16*)Q, off_k, ri, (bf16*)o_part, l_part, status));
   MUSE_LAUNCH_OK();
   return MUSE_OK;
 }

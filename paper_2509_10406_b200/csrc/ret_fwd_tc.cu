@@ -50,6 +50,7 @@ __global__ void __launch_bounds__(rf::kThreads, 2)
 k_ret_fwd_pairs_tc(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ Kp, const bf16* __restrict__ Vp,
                    const int32_t* __restrict__ off_k, const __grid_constant__ RetIndex ri, bf16* __restrict__ o_part,
                    float* __restrict__ l_part, int* __restrict__ status) {
+  pdl_wait();
   using namespace rf;
   typedef Smem<D> SM;
   constexpr int CPR = D / 8;                               // 16-byte chunks per row
@@ -89,6 +90,7 @@ k_ret_fwd_pairs_tc(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
+  pdl_trigger();                                           // (tensor memory has been allocated)
   const uint32_t tbase = tbase_s;
   const bf16* Qb = Q + (size_t)pq * dm.N * D;
   const bf16* Kb = Kp + ((size_t)pk * dm.N + k0) * D;
@@ -384,10 +386,10 @@ int ret_fwd_pairs_tc(const Dims& d, const void* Q, const void* Kp, const void* V
   prof_mark("k_ret_fwd_pairs_tc", st);
   if (d.D == 128) {
     MUSE_CUDA_OK(cudaFuncSetAttribute(k_ret_fwd_pairs_tc<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, rf::Smem<128>::total));
-    k_ret_fwd_pairs_tc<128><<<grid, rf::kThreads, rf::Smem<128>::total, st>>>(d, (const bf16*)Q, (const bf16*)Kp, (const bf16*)Vp, off_k, ri, (bf16*)o_part, l_part, status);
+    MUSE_RC(launch_pdl(k_ret_fwd_pairs_tc<128>, grid, rf::kThreads, rf::Smem<128>::total, st, d, (const bf16*)Q, (const bf16*)Kp, (const bf16*)Vp, off_k, ri, (bf16*)o_part, l_part, status));
   } else {
     MUSE_CUDA_OK(cudaFuncSetAttribute(k_ret_fwd_pairs_tc<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, rf::Smem<64>::total));
-    k_ret_fwd_pairs_tc<64><<<grid, rf::kThreads, rf::Smem<64>::total, st>>>(d, (const bf16*)Q, (const bf16*)Kp, (const bf16*)Vp, off_k, ri, (bf16*)o_part, l_part, status);
+    MUSE_RC(launch_pdl(k_ret_fwd_pairs_tc<64>, grid, rf::kThreads, rf::Smem<64>::total, st, d, (const bf16*)Q, (const bf16*)Kp, (const bf16*)Vp, off_k, ri, (bf16*)o_part, l_part, status));
   }
   MUSE_LAUNCH_OK();
   return MUSE_OK;

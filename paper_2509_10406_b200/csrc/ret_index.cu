@@ -31,8 +31,8 @@ k_ret_index(Dims d, const __grid_constant__ RiArgs g) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nkeys = g.nkeys, ke = g.bsel ? d.k2 : 1;
   const int per = (d.N + CL - 1) / CL, t0 = min(d.N, rank * per), t1 = min(d.N, t0 + per);
   for (int k = tid; k < nkeys; k += kRiThreads) hist[k] = 0;
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   __syncthreads();
   // the key of pair `e` (counted over the CTA's tokens and slots), or -1: entries outside [0, Ck) count as "none"
   const int n = (t1 - t0) * d.m;

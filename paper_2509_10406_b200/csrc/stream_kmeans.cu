@@ -314,8 +314,8 @@ k_stream_kmeans_tc(const __grid_constant__ StArgs g, int* __restrict__ status) {
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tbase = tbase_s;
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
 
   // a centroid row from its totals: bf16 hi / lo into the resident tiles, |c|^2 and count
   auto put_centroid = [&](int jl, float (&t)[EPL], float c) {
@@ -622,8 +622,8 @@ k_bucket_rank(const __grid_constant__ RankArgs g) {
   const bool second = prob >= g.s[0].problems;
   const RankSide& sd = g.s[second ? 1 : 0];
   if (second) prob -= g.s[0].problems;
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   if (pos >= N) return;
   const int t = sd.perm[(size_t)prob * N + pos];
   if (!MUSE_IN_RANGE(t, N)) return;
@@ -650,8 +650,8 @@ k_cap_overflow(int N, int C, int S, int Bs, int cap, const float* dist, const in
   const int32_t* o = off + (size_t)prob * (C * S + 1) + (size_t)b * C;
   const int32_t* rk = rank + (size_t)prob * N;
   int32_t* as = assign + (size_t)prob * N;
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   for (int j = tid; j < C; j += kCapThreads) size[j] = min(o[j + 1] - o[j], cap);     // step 1: the first cap of a bucket keep it
   __syncthreads();
   for (int base = b * Bs; base < (b + 1) * Bs; base += kCapThreads) {

@@ -46,6 +46,7 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
               const int32_t* __restrict__ off_k, const int32_t* __restrict__ off_q,
               const float* __restrict__ mu, const float* __restrict__ dS, float* __restrict__ dK_perm,
               float* __restrict__ dV_perm, int per_block, int* __restrict__ status) {
+  pdl_wait();
   // per_block = 1 (two-level retrieval): mu and the gradients belong to the PER-BLOCK summaries, plane pl holds the summary
   // of bucket pl alone; a key chunk then meets only the planes whose bucket it overlaps, and the weights of a plane are
   // masked to that bucket's keys.
@@ -78,6 +79,7 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
+  pdl_trigger();                                           // (tensor memory has been allocated)
   const uint32_t tbase = tbase_s, tlane = tbase + ((uint32_t)((warp & 3) * 32) << 16);
   uint32_t ph_g[2] = {0, 0}, ph_kv = 0, ph_q = 0, ph_l = 0, ph1 = 0, ph2 = 0;
   bool ok = true;
@@ -364,12 +366,10 @@ int summ_bwd_tc(const Dims& d, const void* Kp, const void* Vp, const int32_t* of
   prof_mark("k_summ_bwd_tc", st);
   if (d.D == 128) {
     MUSE_CUDA_OK(cudaFuncSetAttribute(k_summ_bwd_tc<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, sb::Lay<128>::total));
-    k_summ_bwd_tc<128><<<dim3(d.Ck, d.B * d.Hq), sb::THREADS, sb::Lay<128>::total, st>>>(d, tdka, tdnu, tK, tV, tqh, tql, off_k, off_q, mu, dS,
-                                                                                    dK_perm, dV_perm, per_block, status);
+    MUSE_RC(launch_pdl(k_summ_bwd_tc<128>, dim3(d.Ck, d.B * d.Hq), sb::THREADS, sb::Lay<128>::total, st, d, tdka, tdnu, tK, tV, tqh, tql, off_k, off_q, mu, dS, dK_perm, dV_perm, per_block, status));
   } else {
     MUSE_CUDA_OK(cudaFuncSetAttribute(k_summ_bwd_tc<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, sb::Lay<64>::total));
-    k_summ_bwd_tc<64><<<dim3(d.Ck, d.B * d.Hq), sb::THREADS, sb::Lay<64>::total, st>>>(d, tdka, tdnu, tK, tV, tqh, tql, off_k, off_q, mu, dS,
-                                                                                  dK_perm, dV_perm, per_block, status);
+    MUSE_RC(launch_pdl(k_summ_bwd_tc<64>, dim3(d.Ck, d.B * d.Hq), sb::THREADS, sb::Lay<64>::total, st, d, tdka, tdnu, tK, tV, tqh, tql, off_k, off_q, mu, dS, dK_perm, dV_perm, per_block, status));
   }
   MUSE_LAUNCH_OK();
   return MUSE_OK;

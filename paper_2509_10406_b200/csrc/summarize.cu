@@ -43,10 +43,14 @@ SummLayout summ_layout(const Dims& d, int dtype) {
   return L;
 }
 
-// out[p] = in[perm[p]] for whole rows of D elements (16 bytes per thread).
+// out[p] = in[perm[p]] for whole rows of D elements (16 bytes per thread), keys and values (blockIdx.z) in one launch.
 template <class T>
-__global__ void k_gather_rows(const T* __restrict__ in, const int32_t* __restrict__ perm, int N, int D,
-                              T* __restrict__ out) {
+__global__ void k_gather_rows(const T* __restrict__ K, const T* __restrict__ V, const int32_t* __restrict__ perm, int N, int D,
+                              T* __restrict__ Kp, T* __restrict__ Vp) {
+  pdl_wait();
+  pdl_trigger();
+  const T* in = blockIdx.z == 0 ? K : V;
+  T* out = blockIdx.z == 0 ? Kp : Vp;
   const int vpr = D * (int)sizeof(T) / 16;           // 16-byte vectors per row
   const int prob = blockIdx.y;
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -97,6 +101,8 @@ template <class T, int D>
 __global__ void __launch_bounds__(kSumThreads)
 k_summarize(Dims dm, const T* __restrict__ Kp, const T* __restrict__ Vp, const int32_t* __restrict__ off_k,
             const float* __restrict__ qbar, SummPtrs sp, int per_block) {
+  pdl_wait();
+  pdl_trigger();
   constexpr int LDQ = D + 4, LDKV = 2 * D + 4, LDL = kSumKC + 1, NV = 2 * D / 32;
   extern __shared__ float smf[];
   float* qb = smf;                         // [64][LDQ]  sigma * qbar tile
@@ -239,19 +245,14 @@ static int summarize_t(const Dims& d, int dtype, const T* K, const T* V, const i
   if (status_in != nullptr) status = status_in;
   int rc = MUSE_OK;
   const SortSide side = {assign_k, off_k, perm_k, pk, d.Ck, 1};
-  if (assign_k != nullptr) rc = bucket_sort(&side, 1, d.N, d.S, d.Bs, st);
+  if (assign_k != nullptr) rc = bucket_sort(&side, 1, d.N, d.S, d.Bs, st, status_in == nullptr ? status : nullptr);
   if (rc != MUSE_OK) return rc;
   SummLayout L = summ_layout(d, dtype);
   char* base = (char*)summaries;
   T* Kp = (T*)(base + L.Kp); T* Vp = (T*)(base + L.Vp);
   const int vpr = D * (int)sizeof(T) / 16;
-  dim3 gg(cdiv(d.N * vpr, 256), pk);
   prof_mark("k_gather_rows", st);
-  k_gather_rows<T><<<gg, 256, 0, st>>>(K, perm_k, d.N, D, Kp);
-  MUSE_LAUNCH_OK();
-  prof_mark("k_gather_rows", st);
-  k_gather_rows<T><<<gg, 256, 0, st>>>(V, perm_k, d.N, D, Vp);
-  MUSE_LAUNCH_OK();
+  MUSE_RC(launch_pdl(k_gather_rows<T>, dim3(cdiv(d.N * vpr, 256), pk, 2), 256, 0, st, K, V, perm_k, d.N, D, Kp, Vp));
   if (counts != nullptr) {
     prof_mark("k_bucket_sums", st);
     k_bucket_sums<T, D><<<dim3(cdiv(d.Ck * d.S, 8), pk), 256, 0, st>>>(Kp, Vp, off_k, d.N, d.Ck * d.S, counts, ksum, vsum);
@@ -274,8 +275,7 @@ static int summarize_planes(const Dims& d, int dtype, const T* Kp, const T* Vp, 
   MUSE_CUDA_OK(cudaFuncSetAttribute(k_summarize<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   dim3 grid(d.Ck, cdiv(d.Cq, kSumI), d.B * d.Hq);
   prof_mark("k_summarize", st);
-  k_summarize<T, D><<<grid, kSumThreads, smem, st>>>(d, Kp, Vp, off_k, qbar, sp, per_block);
-  MUSE_LAUNCH_OK();
+  MUSE_RC(launch_pdl(k_summarize<T, D>, grid, kSumThreads, smem, st, d, Kp, Vp, off_k, qbar, sp, per_block));
   return MUSE_OK;
 }
 

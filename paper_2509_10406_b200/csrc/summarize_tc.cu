@@ -46,6 +46,8 @@ struct Bars { uint64_t q_full, q_free, kv_full[4], kv_empty[4], l_full[2], w_rea
 }  // namespace st
 
 __global__ void k_split_qbar(const float* __restrict__ qbar, long long n, float sigma, bf16* __restrict__ hi, bf16* __restrict__ lo, int* dealt) {
+  pdl_wait();
+  pdl_trigger();
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (e == 0 && dealt != nullptr) *dealt = 0;              // the item counter of the kernel that follows
   if (e >= n) return;
@@ -58,9 +60,7 @@ __global__ void k_split_qbar(const float* __restrict__ qbar, long long n, float 
 int split_qbar(const Dims& d, const float* qbar, void* qhi, void* qlo, int* dealt, cudaStream_t st) {
   const long long n = (long long)d.B * d.Hq * d.Cq * d.D;
   prof_mark("k_split_qbar", st);
-  k_split_qbar<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(qbar, n, d.sigma, (bf16*)qhi, (bf16*)qlo, dealt);
-  MUSE_LAUNCH_OK();
-  return MUSE_OK;
+  return launch_pdl(k_split_qbar, dim3((unsigned)((n + 255) / 256)), 256, 0, st, qbar, n, d.sigma, (bf16*)qhi, (bf16*)qlo, dealt);
 }
 
 template <int D>
@@ -128,8 +128,8 @@ k_summarize_tc(Dims dm, const __grid_constant__ CUtensorMap tm_K, const __grid_c
     if (w.nxt.it < items) advance(w.nxt);
   };
   auto next = [&](Walk& w) { w.cur = w.nxt; if (w.nxt.it < items) advance(w.nxt); };
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
 
   if (warp == kDealWarp) {                                 // ---- hands out ranges of items
     for (int n = 0, it = 0; it < items && ok; ++n) {       // (a short ring: what a CTA has taken no other can)
