@@ -556,7 +556,7 @@ static int attn_fwd_t(const Dims& d, const T* Q, const T* K, const T* V, const i
     }
     if (d.m > 0) {
       RetIndex ri;
-      rc = build_ret_index(d, sel, bsel, w.ret_scratch, &ri, st);
+      rc = build_ret_index(d, sel, bsel, off_k, w.ret_scratch, &ri, st);
       if (rc != MUSE_OK) return rc;
       if (d.dipole) {
         rc = dipole_apply(d, dtype, Q, qbar, assign_q, w.off_q, w.perm_q, dipole_ptrs(L, base), w.lse_far, sel, ri.goff, ri.pairs,

@@ -355,12 +355,21 @@ size_t attn_bwd_ws_bytes(const Dims& d, int dtype);
 
 // retrieval inverse index, shared by forward and backward: groups the (query, slot) pairs by
 // (query block - 1, key cluster).  pair id = t * m + slot.
-// The tensor-core kernels take the pairs of a group (a key cluster, or a bucket) in shares of `share` tiles of 128: items, for each head,
-// lists (group, share | shares << 16).
+// The tensor-core kernels take the pairs of a group (a key cluster, or a bucket) in shares of `share` tiles of 128, one CTA per share:
+// `items` lists them for each head, with what a CTA would otherwise look up through two more dependent loads.
 constexpr int kRetTile = 128, kMinShare = 4, kMaxShare = 32;
-struct RetIndex { int32_t* goff; int32_t* pairs; int2* items; int32_t* nitems; int cap, share; };
+struct __align__(16) RetItem { int group, share, g0, g1, k0, nk, pad[2]; };   // share | shares << 16; its pairs [g0, g1), its first key, keys that some pair sees
+struct RetIndex { int32_t* goff; int32_t* pairs; RetItem* items; int32_t* nitems; int cap, share; };
 size_t ret_index_elems(const Dims& d);     // int32 elements per query head
 // bsel != nullptr (k2 > 0): groups are the (cluster, chosen block) buckets, pair id = (t * m + slot) * k2 + e
-int build_ret_index(const Dims& d, const int32_t* sel, const int32_t* bsel, int32_t* scratch, RetIndex* out, cudaStream_t st);
+int build_ret_index(const Dims& d, const int32_t* sel, const int32_t* bsel, const int32_t* off_k, int32_t* scratch, RetIndex* out, cudaStream_t st);
+// this CTA's item, or false if there is none (the item is loaded beside the number of items: the list's memory reaches to ri.cap)
+__device__ __forceinline__ bool ret_item(const RetIndex& ri, int pq, RetItem& it) {
+  const int4* p = reinterpret_cast<const int4*>(ri.items + (size_t)pq * ri.cap + blockIdx.x);
+  const int4 a = p[0], b = p[1];
+  const int n = ri.nitems[pq];
+  it.group = a.x; it.share = a.y; it.g0 = a.z; it.g1 = a.w; it.k0 = b.x; it.nk = b.y;
+  return (int)blockIdx.x < n;
+}
 
 }  // namespace muse

@@ -72,17 +72,17 @@ k_ret_bwd_sweeps(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ d
   // chosen block) triples that chose the block, and every one of them sees the whole bucket (as in the forward kernel).
   const bool bucket = dm.k2 > 0;
   const int pq = blockIdx.y;
-  if ((int)blockIdx.x >= ri.nitems[pq]) return;
-  const int2 item = ri.items[(size_t)pq * ri.cap + blockIdx.x];               // group, share of its tiles (dealt round-robin)
-  const int j = bucket ? item.x / dm.SB : item.x, bb = bucket ? item.x % dm.SB : 0, sub = item.y & 0xffff, nsub = item.y >> 16;
+  RetItem item;                                             // group, share of its tiles (dealt round-robin)
+  if (!ret_item(ri, pq, item)) return;
+  const int j = bucket ? item.group / dm.SB : item.group, bb = bucket ? item.group % dm.SB : 0, sub = item.share & 0xffff, nsub = item.share >> 16;
   const int mk = dm.m * (bucket ? dm.k2 : 1);               // partial dQ rows per query
   const int b_ = pq / dm.Hq, h = pq % dm.Hq, pk = b_ * dm.Hkv + dm.hm.g[h];
   const int ngroups = dm.SB * dm.Ck;
   const int32_t* go = ri.goff + (size_t)pq * (ngroups + 1) + (size_t)j * dm.SB + bb;   // the group's pairs: plane pl is [go[pl], go[pl + 1])
-  const int g0 = go[0], g1 = go[bucket ? 1 : dm.SB];
+  const int g0 = item.g0, g1 = item.g1;
   const int ntiles = (g1 - g0 + kPairs - 1) / kPairs;
   const int32_t* okg = off_k + (size_t)pk * (dm.Ck * dm.S + 1) + (size_t)j * dm.S;   // okg[b]: first key of bucket (j, b)
-  const int k0 = okg[bb], kall = (bucket ? okg[bb + 1] : okg[dm.SB]) - k0;   // keys that some pair of the group sees
+  const int k0 = item.k0, kall = item.nk;                  // keys that some pair of the group sees
   if (tc::smem_u32(sm) & 1023u) {                           // the tiles fill the whole dynamic allocation: no room to realign
     if (tid == 0) report_status(status, MUSE_STATUS_BWD_TIMEOUT);
     return;

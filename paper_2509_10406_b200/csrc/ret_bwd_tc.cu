@@ -45,18 +45,18 @@ struct Group {
   bool bucket;
   int j, bb, sub, pq, pk, mk, g0, g1, k0, kall, ntiles, nsub;
   const int32_t *go, *okg;
-  __device__ __forceinline__ Group(const Dims& dm, const RetIndex& ri, const int32_t* off_k) {
+  __device__ __forceinline__ Group(const Dims& dm, const RetIndex& ri, const RetItem& item, const int32_t* off_k) {
     bucket = dm.k2 > 0;
     pq = blockIdx.y;
-    const int2 item = ri.items[(size_t)pq * ri.cap + blockIdx.x];             // group, share of its tiles (dealt round-robin)
-    j = bucket ? item.x / dm.SB : item.x; bb = bucket ? item.x % dm.SB : 0; sub = item.y & 0xffff; nsub = item.y >> 16;
+    j = bucket ? item.group / dm.SB : item.group; bb = bucket ? item.group % dm.SB : 0;
+    sub = item.share & 0xffff; nsub = item.share >> 16;    // share of its tiles (dealt round-robin)
     mk = dm.m * (bucket ? dm.k2 : 1);
     const int b_ = pq / dm.Hq, h = pq % dm.Hq;
     pk = b_ * dm.Hkv + dm.hm.g[h];
     go = ri.goff + (size_t)pq * (dm.SB * dm.Ck + 1) + (size_t)j * dm.SB + bb;      // plane pl's pairs: [go[pl], go[pl + 1])
-    g0 = go[0]; g1 = go[bucket ? 1 : dm.SB];
+    g0 = item.g0; g1 = item.g1;
     okg = off_k + (size_t)pk * (dm.Ck * dm.S + 1) + (size_t)j * dm.S;           // okg[b]: first key of bucket (j, b)
-    k0 = okg[bb]; kall = (bucket ? okg[bb + 1] : okg[dm.SB]) - k0;              // keys that some pair of the group sees
+    k0 = item.k0; kall = item.nk;                          // keys that some pair of the group sees
     ntiles = (g1 - g0 + kM - 1) / kM;
   }
 };
@@ -95,8 +95,9 @@ k_ret_bwd_dkdv(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_c
   __shared__ int32_t ok_s[kOkCache], tok_s[4][kN];
   __shared__ __align__(16) float Ls[NS][kN], ds[NS][kN];
   __shared__ __align__(16) int vs[NS][kN];                  // keys each pair of the tile sees, counted from the cluster's first
-  if ((int)blockIdx.x >= ri.nitems[blockIdx.y]) return;
-  const Group gr(dm, ri, off_k);
+  RetItem item;
+  if (!ret_item(ri, blockIdx.y, item)) return;
+  const Group gr(dm, ri, item, off_k);
   if (gr.kall <= 0) return;
   const int tid = threadIdx.x, warp = tc::warp_index(), lane = tid & 31;
   unsigned char* sm = sm_raw + ((1024u - (tc::smem_u32(sm_raw) & 1023u)) & 1023u);
@@ -353,8 +354,9 @@ k_ret_bwd_dq(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_con
   __shared__ uint32_t tbase_s;
   __shared__ int32_t ok_s[kOkCache], tok_s[NQ][kM], pid_s[NQ][kM], vs[NQ][kM], T_s[NQ];
   __shared__ float Ls[NQ][kM], ds[NQ][kM];
-  if ((int)blockIdx.x >= ri.nitems[blockIdx.y]) return;
-  const Group gr(dm, ri, off_k);
+  RetItem item;
+  if (!ret_item(ri, blockIdx.y, item)) return;
+  const Group gr(dm, ri, item, off_k);
   if (gr.ntiles == 0) return;
   const int tid = threadIdx.x, warp = tc::warp_index(), lane = tid & 31;
   unsigned char* sm = sm_raw + ((1024u - (tc::smem_u32(sm_raw) & 1023u)) & 1023u);

@@ -60,13 +60,13 @@ k_ret_fwd_long(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_c
   __shared__ float mx_s[2][2][kPairs];
   const int tid = threadIdx.x, warp = tc::warp_index(), lane = tid & 31;
   const int pq = blockIdx.y;
-  if ((int)blockIdx.x >= ri.nitems[pq]) return;
-  const int2 item = ri.items[(size_t)pq * ri.cap + blockIdx.x];              // key cluster, share of its units (dealt round-robin)
-  const int j = item.x, sub = item.y & 0xffff, nsub = item.y >> 16, b_ = pq / dm.Hq, h = pq % dm.Hq, pk = b_ * dm.Hkv + dm.hm.g[h];
+  RetItem item;                                             // key cluster, share of its units (dealt round-robin)
+  if (!ret_item(ri, pq, item)) return;
+  const int j = item.group, sub = item.share & 0xffff, nsub = item.share >> 16, b_ = pq / dm.Hq, h = pq % dm.Hq, pk = b_ * dm.Hkv + dm.hm.g[h];
   const int32_t* go = ri.goff + (size_t)pq * (dm.SB * dm.Ck + 1) + (size_t)j * dm.SB;      // plane pl's pairs: [go[pl], go[pl + 1])
-  const int g0 = go[0], g1 = go[dm.SB], ntiles = (g1 - g0 + kPairs - 1) / kPairs, nunits = (ntiles + 1) / 2;
+  const int g0 = item.g0, g1 = item.g1, ntiles = (g1 - g0 + kPairs - 1) / kPairs, nunits = (ntiles + 1) / 2;
   const int32_t* okg = off_k + (size_t)pk * (dm.Ck * dm.S + 1) + (size_t)j * dm.S;      // okg[b]: first key of bucket (j, b)
-  const int k0 = okg[0];
+  const int k0 = item.k0;
   const int32_t* ok = dm.S + 1 <= kOkCache ? ok_s : okg;
   if (dm.S + 1 <= kOkCache)
     for (int b = tid; b <= dm.S; b += LY::kThreads) ok_s[b] = okg[b];

@@ -65,17 +65,17 @@ k_ret_fwd_pairs_tc(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__
   // (query, slot, chosen block) triples that chose this block, and every one of them sees the whole bucket.
   const bool bucket = dm.k2 > 0;
   const int pq = blockIdx.y;
-  if ((int)blockIdx.x >= ri.nitems[pq]) return;
-  const int2 item = ri.items[(size_t)pq * ri.cap + blockIdx.x];              // group, share of its tiles (dealt round-robin)
-  const int j = bucket ? item.x / dm.SB : item.x, bb = bucket ? item.x % dm.SB : 0, sub = item.y & 0xffff, nsub = item.y >> 16;
+  RetItem item;                                             // group, share of its tiles (dealt round-robin)
+  if (!ret_item(ri, pq, item)) return;
+  const int j = bucket ? item.group / dm.SB : item.group, bb = bucket ? item.group % dm.SB : 0, sub = item.share & 0xffff, nsub = item.share >> 16;
   const int mk = dm.m * (bucket ? dm.k2 : 1);              // partial results per query
   const int b_ = pq / dm.Hq, h = pq % dm.Hq, pk = b_ * dm.Hkv + dm.hm.g[h];
   const int ngroups = dm.SB * dm.Ck;
   const int32_t* go = ri.goff + (size_t)pq * (ngroups + 1) + (size_t)j * dm.SB + bb;   // the group's pairs: plane pl is [go[pl], go[pl + 1])
-  const int g0 = go[0], g1 = go[bucket ? 1 : dm.SB];
+  const int g0 = item.g0, g1 = item.g1;
   const int ntiles = (g1 - g0 + kPairs - 1) / kPairs;
   const int32_t* okg = off_k + (size_t)pk * (dm.Ck * dm.S + 1) + (size_t)j * dm.S;   // okg[b]: first key of bucket (j, b)
-  const int k0 = okg[bb], kall = (bucket ? okg[bb + 1] : okg[dm.SB]) - k0;   // keys that some pair of the group sees
+  const int k0 = item.k0, kall = item.nk;                  // keys that some pair of the group sees
   const int32_t* ok = dm.S + 1 <= kOkCache ? ok_s : okg;
   if (dm.S + 1 <= kOkCache)
     for (int b = tid; b <= dm.S; b += kThreads) ok_s[b] = okg[b];

@@ -20,7 +20,7 @@ namespace muse {
 
 constexpr int kRiThreads = 1024, kRiMaxCluster = 16, kRiMinPairs = 2048;
 
-struct RiArgs { const int32_t *sel, *bsel; RetIndex ri; int nkeys; };
+struct RiArgs { const int32_t *sel, *bsel, *off_k; RetIndex ri; int nkeys; };
 
 __global__ void __launch_bounds__(kRiThreads)
 k_ret_index(Dims d, const __grid_constant__ RiArgs g) {
@@ -104,10 +104,13 @@ k_ret_index(Dims d, const __grid_constant__ RiArgs g) {
   cluster.sync();
   if (rank == 0) {                                         // the shares of every group's pairs (this CTA has the tokens of block 0, which have no pairs)
     const int stride = g.bsel ? 1 : d.SB, G = nkeys / stride;
-    int2* items = g.ri.items + (size_t)pq * g.ri.cap;
+    RetItem* items = g.ri.items + (size_t)pq * g.ri.cap;
+    const int32_t* ok = g.off_k + (size_t)(pq / d.Hq * d.Hkv + d.hm.g[pq % d.Hq]) * (d.Ck * d.S + 1);
     int carry2 = 0;
     for (int k0 = 0; k0 < G; k0 += kRiThreads) {
-      const int k = k0 + tid, np = k < G ? __ldcg(goff + (k + 1) * stride) - __ldcg(goff + k * stride) : 0;
+      const int k = k0 + tid, p0 = k < G ? __ldcg(goff + k * stride) : 0, p1 = k < G ? __ldcg(goff + (k + 1) * stride) : 0, np = p1 - p0;
+      const int b0 = g.bsel ? k / d.SB * d.S + k % d.SB : k * d.S;             // the group's first bucket; it ends with that one, or with the block SB
+      const int kf = k < G ? ok[b0] : 0, nk = k < G ? ok[b0 + (g.bsel ? 1 : d.SB)] - kf : 0;
       const int tiles = (np + kRetTile - 1) / kRetTile, ns = min(32767, (tiles + g.ri.share - 1) / g.ri.share);
       int inc = ns;
 #pragma unroll
@@ -118,7 +121,7 @@ k_ret_index(Dims d, const __grid_constant__ RiArgs g) {
       int at = carry2 + inc - ns;
       for (int w = 0; w < 32; ++w) { const int v = wsum[w]; if (w < warp) at += v; carry2 += v; }
       for (int s = 0; s < ns; ++s)
-        if (MUSE_IN_RANGE(at + s, g.ri.cap)) items[at + s] = make_int2(k, s | ns << 16);
+        if (MUSE_IN_RANGE(at + s, g.ri.cap)) items[at + s] = RetItem{k, s | ns << 16, p0, p1, kf, nk, {0, 0}};
     }
     if (tid == 0) g.ri.nitems[pq] = carry2;
   }
@@ -146,11 +149,11 @@ static int item_cap(const Dims& d, int share) {
 }
 
 size_t ret_index_elems(const Dims& d) {
-  // goff [SB*Ck+1] + pairs [N*m*max(k2,1)] + items (2 each) + their number, each rounded up to 64 ints
-  return up64((size_t)d.SB * d.Ck + 1) + up64((size_t)d.N * d.m * (d.k2 > 0 ? d.k2 : 1)) + up64(2 * (size_t)item_cap(d, kMinShare)) + 64;
+  // goff [SB*Ck+1] + pairs [N*m*max(k2,1)] + items (8 each) + their number, each rounded up to 64 ints
+  return up64((size_t)d.SB * d.Ck + 1) + up64((size_t)d.N * d.m * (d.k2 > 0 ? d.k2 : 1)) + up64(8 * (size_t)item_cap(d, kMinShare)) + 64;
 }
 
-int build_ret_index(const Dims& d, const int32_t* sel, const int32_t* bsel, int32_t* scratch, RetIndex* out, cudaStream_t st) {
+int build_ret_index(const Dims& d, const int32_t* sel, const int32_t* bsel, const int32_t* off_k, int32_t* scratch, RetIndex* out, cudaStream_t st) {
   const int pq = d.B * d.Hq, nkeys = d.SB * d.Ck, mk = d.m * (bsel ? d.k2 : 1);        // nkeys <= 32768
   // Shares of 32 tiles; fewer where that would leave SMs without work (selections crowd on few clusters: one may have all of a head's
   // queries), not below 4 (a share loads its keys and adds its gradients once).
@@ -159,15 +162,15 @@ int build_ret_index(const Dims& d, const int32_t* sel, const int32_t* bsel, int3
   out->cap = item_cap(d, out->share);
   out->goff = scratch;                                     // (indexed with its natural stride, nkeys + 1)
   out->pairs = out->goff + (size_t)pq * up64((size_t)nkeys + 1);
-  out->items = (int2*)(out->pairs + (size_t)pq * up64((size_t)d.N * mk));
-  out->nitems = (int32_t*)(out->items + (size_t)pq * up64(2 * (size_t)item_cap(d, kMinShare)) / 2);
+  out->items = (RetItem*)(out->pairs + (size_t)pq * up64((size_t)d.N * mk));
+  out->nitems = (int32_t*)(out->items + (size_t)pq * up64(8 * (size_t)item_cap(d, kMinShare)) / 8);
   if (d.m == 0 || nkeys == 0) return MUSE_OK;
   // CTAs of a head, of 2048 pairs or more: until half the SMs have one (a large cluster pays in its exchange of counts and in scheduling:
   // 32 heads of 16k tokens, 16 slots 131 us with 8 CTAs, 87 with 4; 4 heads of 64k, 32 slots 181 us with 16, 326 with 8)
   int cl = 1;
   while (cl < kRiMaxCluster && cl * pq < sm_count() / 2 && (long long)d.N * d.m >= 2LL * cl * kRiMinPairs) cl *= 2;
   const size_t smem = (size_t)nkeys * sizeof(int32_t);
-  const RiArgs g = {sel, bsel, *out, nkeys};
+  const RiArgs g = {sel, bsel, off_k, *out, nkeys};
   if (cl > 8) MUSE_CUDA_OK(cudaFuncSetAttribute(k_ret_index, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
   prof_mark("k_ret_index", st);
   return launch_pdl_cluster(k_ret_index, dim3(pq * cl), kRiThreads, smem, cl, st, d, g);
