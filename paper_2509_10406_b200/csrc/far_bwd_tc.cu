@@ -10,9 +10,13 @@
 // dkappa and dnu are stored as bf16 rows for the key-side pass, dS as fp32.
 // A segment of few queries pays for its own rows only (multiples of 16), not for 64.  At D = 64 dnu and dkappa take the
 // tensor-memory columns of the consumed scores and are staged in the consumed P and G tiles, so that two CTAs fill each
-// other's waits on an SM.  Bound by DRAM at D = 128 (4.1 TB/s of reads and writes at 4 heads of 64k tokens, 256 x 1024
-// clusters), by the phases' latency at D = 64.  Measured, before | after: 32 heads of 64k tokens, 128 x 128 clusters, D = 64
-// 3243 | 1778 us; 32 heads of 16k, 128 x 256 2490 | 1330; 16 heads of 8k, 64 x 128 488 | 267; 4 heads, D = 128 2425 | 2274.
+// other's waits on an SM.
+// Bound by DRAM at D = 128 (4.6 TB/s of reads and writes at 4 heads of 64k tokens, 256 x 1024 clusters), by the phases' latency
+// at D = 64: of a CTA's life 45 % went into loads that waited for one another before the first product (row numbers, rows,
+// log-sum-exps, selections: 10000 cycles); in flight together they take 7400.  32 heads of 64k tokens, 128 x 128 clusters,
+// D = 64, segments of 64 queries: 3243 us with one CTA per SM, 1778 with two, 1646 with the sums of all sweeps kept on chip,
+// 1419 with the loads together; 32 heads of 16k, 128 x 256 2490 -> 1160; 16 heads of 8k, 64 x 128 488 -> 224; 4 heads, D = 128
+// 2425 -> 2053.
 #include <cuda.h>
 #include "common.cuh"
 #include "tc05.cuh"
@@ -28,7 +32,7 @@ int make_tmap_bf16_nd(void* out_map, const void* base, int rank, const uint64_t*
 namespace fb {
 constexpr int TJ = 128, NR = 64, NP = 1;
 constexpr int THREADS = 288, CW = 256, ISSUER = 256;   // warps 0-7 do the arithmetic; lane 0 of a ninth warp issues every TMA transfer and MMA
-template <int D> struct Lay {
+template <int D, bool ONE> struct Lay {
   static constexpr int kTile = TJ * D * 2;        // operand tile [128 clusters][D] bf16
   static constexpr int kRows = NR * D * 2;        // tile of 64 query rows
   static constexpr int oHi = 0, oLo = oHi + kTile, oNu = oLo + kTile;
@@ -39,8 +43,9 @@ template <int D> struct Lay {
   // (at D = 64: dkappa in the P tile, dnu in the G tile once the dq products have read it; two CTAs then fit an SM)
   static constexpr int oStK = oPt, oStN = D == 64 ? oGt : oGt + TJ * NR * 2;
   static constexpr int oMask = oStN + kTile;      // [NP*NR rows][Ck/32] words follow
-  // TMEM columns; at D = 64 dnu and dkappa take the place of the consumed S and dPnu
-  static constexpr uint32_t cS = 0, cDP = 64, cDNU = D == 64 ? 0 : 128, cDKA = D == 64 ? 64 : 256, cDQ = D == 64 ? 128 : 384, cols = D == 64 ? 256 : 512;
+  // TMEM columns; at D = 64 dnu and dkappa take the place of the consumed S and dPnu, or (one tile of clusters) dq that of S
+  static constexpr uint32_t cS = 0, cDP = 64, cDNU = D == 64 && !ONE ? 0 : 128, cDKA = D == 64 ? (ONE ? 192 : 64) : 256,
+                            cDQ = D == 64 ? (ONE ? 0 : 128) : 384, cols = D == 64 ? 256 : 512;
   static constexpr int kMin = D == 64 ? 2 : 1;    // CTAs per SM
 };
 constexpr float kLog2e = 1.4426950408889634f;
@@ -52,8 +57,10 @@ __device__ __forceinline__ float fast_exp2(float x) {
   return y;
 }
 
-template <int D>
-__global__ void __launch_bounds__(fb::THREADS, fb::Lay<D>::kMin)
+// ONE: Ck <= 128.  The tiles of the only cluster tile stay for all sweeps of the segment, and dnu, dkappa and the sums behind dS
+// are accumulated over them on chip and stored once.  (With more tiles each sweep reloads the tiles and adds to the stored rows.)
+template <int D, bool ONE>
+__global__ void __launch_bounds__(fb::THREADS, fb::Lay<D, ONE>::kMin)
 k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_constant__ CUtensorMap tm_klo,
              const __grid_constant__ CUtensorMap tm_nu, const __grid_constant__ CUtensorMap tm_gka,
              const __grid_constant__ CUtensorMap tm_gnu, const bf16* __restrict__ Q, const bf16* __restrict__ dO,
@@ -63,7 +70,7 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
              bf16* __restrict__ dnu, float* __restrict__ dS, int grad_by_key_cluster, int* __restrict__ status) {
   pdl_wait();
   using namespace fb;
-  typedef Lay<D> LY;
+  typedef Lay<D, ONE> LY;
   constexpr int kTile = LY::kTile, kRows = LY::kRows, oHi = LY::oHi, oLo = LY::oLo, oNu = LY::oNu, oQ = LY::oQ, oDO = LY::oDO,
                 oPt = LY::oPt, oGt = LY::oGt, oStK = LY::oStK, oStN = LY::oStN, oMask = LY::oMask, G = D / 64, CPR = D / 8;
   constexpr uint32_t cS = LY::cS, cDP = LY::cDP, cDNU = LY::cDNU, cDKA = LY::cDKA, cDQ = LY::cDQ;
@@ -131,37 +138,61 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
     tc::mbar_expect_tx_warp(&bar_nu, kTile);
     for (int g = 0; g < G; ++g) tc::tma_load_3d_warp(sm + oNu + g * TJ * 128, &tm_nu, 64 * g, jt_ * TJ, seg, &bar_nu);
   };
+  float gsum = 0.f, gt2 = 0.f, pdp = 0.f;
   for (int s0 = p0; s0 < p1 && ok; s0 += NP * NR) {        // sweep: up to 64 rows
+    const bool load = !ONE || s0 == p0, store = !ONE || s0 + NP * NR >= p1;
     const int ns = min(NP * NR, p1 - s0), np = (ns + NR - 1) / NR;
     // the products take only as many rows as there are: nc of them (a multiple of 8) per warpgroup, nr in all
     const int nc = ((ns + 1) / 2 + 7) & ~7, nr = 2 * nc;
     __syncthreads();
     // the operand tiles are free (every product of the previous sweep has completed): the first cluster
     // tile travels while the rows are gathered
-    if (warp == ISSUER / 32) { issue_kappa(0); issue_nu(0); }
-    if (tid < NP * NR) {
-      int t = tid < ns && MUSE_IN_RANGE(s0 + tid, dm.N) ? pm[s0 + tid] : -1;
+    if (load && warp == ISSUER / 32) { issue_kappa(0); issue_nu(0); }
+    // a chain of loads whose latency nothing hides but the SM's other CTA: every thread finds its rows itself, and all that
+    // hangs on a row (Q, dO, log-sum-exp, delta, the selection) is on its way at once
+    auto row_of = [&](int r) {
+      int t = r < ns && MUSE_IN_RANGE(s0 + r, dm.N) ? pm[s0 + r] : -1;
       if (t >= 0 && !MUSE_IN_RANGE(t, dm.N)) t = -1;
-      rows[tid] = t;
-      Ls[tid] = t >= 0 ? LSE[(size_t)pq * dm.N + t] * kLog2e : 0.f;
-      ds[tid] = t >= 0 ? delta[(size_t)pq * dm.N + t] : 0.f;
+      return t;
+    };
+    constexpr int IT = (NR * CPR + THREADS - 1) / THREADS, IS = 4;      // 16-byte pieces of a row, selected clusters per thread and turn
+    int ta[IT], tsel[IS];
+    const int tr = tid < NP * NR ? row_of(tid) : -1;
+#pragma unroll
+    for (int it = 0; it < IT; ++it) { const int r = (tid + it * THREADS) / CPR; ta[it] = r < nr ? row_of(r) : -1; }
+#pragma unroll
+    for (int it = 0; it < IS; ++it) { const int e = tid + it * THREADS; tsel[it] = e < ns * m ? row_of(e / m) : -1; }
+    const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+    uint4 va[IT], vb[IT];
+#pragma unroll
+    for (int it = 0; it < IT; ++it) {
+      const int ck = (tid + it * THREADS) % CPR;
+      va[it] = ta[it] >= 0 ? reinterpret_cast<const uint4*>(Qp + (size_t)ta[it] * D)[ck] : zero;
+      vb[it] = ta[it] >= 0 ? reinterpret_cast<const uint4*>(dOp + (size_t)ta[it] * D)[ck] : zero;
     }
+#pragma unroll
+    for (int it = 0; it < IS; ++it) tsel[it] = tsel[it] >= 0 ? sel[((size_t)pq * dm.N + tsel[it]) * m + (tid + it * THREADS) % m] : -1;
+    const float lse_r = tr >= 0 ? LSE[(size_t)pq * dm.N + tr] : 0.f, del_r = tr >= 0 ? delta[(size_t)pq * dm.N + tr] : 0.f;
+    float bnext = L < Ck ? beta[ent0 + L] : -INFINITY;
     for (int e = tid; e < 2 * NJ * TJ; e += THREADS) smask[e] = 0u;
     __syncthreads();
-    for (int e = tid; e < nr * CPR; e += THREADS) {
-      const int r = e / CPR, ck = e % CPR, kb = ck >> 3, c = ck & 7, p = r / NR, rr = r % NR;
-      uint4 a = make_uint4(0u, 0u, 0u, 0u), b = a;
-      if (r < ns && rows[r] >= 0) {
-        a = reinterpret_cast<const uint4*>(Qp + (size_t)rows[r] * D)[ck];
-        b = reinterpret_cast<const uint4*>(dOp + (size_t)rows[r] * D)[ck];
-      }
-      *reinterpret_cast<uint4*>(sm + oQ + p * kRows + kb * NR * 128 + tc::sw128_off(rr, c)) = a;
-      *reinterpret_cast<uint4*>(sm + oDO + p * kRows + kb * NR * 128 + tc::sw128_off(rr, c)) = b;
+    if (tid < NP * NR) { rows[tid] = tr; Ls[tid] = lse_r * kLog2e; ds[tid] = del_r; }
+#pragma unroll
+    for (int it = 0; it < IT; ++it) {
+      const int e = tid + it * THREADS, r = e / CPR, ck = e % CPR;
+      if (r >= nr) continue;
+      const int at = (ck >> 3) * NR * 128 + tc::sw128_off(r, ck & 7);
+      *reinterpret_cast<uint4*>(sm + oQ + at) = va[it];
+      *reinterpret_cast<uint4*>(sm + oDO + at) = vb[it];
     }
-    for (int e = tid; e < ns * m; e += THREADS) {
-      const int r = e / m, k = e % m;
-      const int c = rows[r] >= 0 ? sel[((size_t)pq * dm.N + rows[r]) * m + k] : -1;
+#pragma unroll
+    for (int it = 0; it < IS; ++it) {
+      const int c = tsel[it], r = (tid + it * THREADS) / max(m, 1);
       if (c >= 0 && c < Ck) atomicOr(&smask[2 * c + (r >> 5)], 1u << (r & 31));     // [cluster][row bits]
+    }
+    for (int e = tid + IS * THREADS; e < ns * m; e += THREADS) {                    // (long selections)
+      const int r = e / m, t = row_of(r), c = t >= 0 ? sel[((size_t)pq * dm.N + t) * m + e % m] : -1;
+      if (c >= 0 && c < Ck) atomicOr(&smask[2 * c + (r >> 5)], 1u << (r & 31));
     }
     tc::fence_async_smem();
     __syncthreads();
@@ -170,8 +201,7 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
     long long pc[6] = {0, 0, 0, 0, 0, 0};
 #endif
     static_assert(NP == 1, "one pass per sweep");
-    float bnext = L < Ck ? beta[ent0 + L] : -INFINITY;
-    const bool later_sweep = s0 > p0;                       // gradients of earlier sweeps are already stored: add to them
+    const bool later_sweep = !ONE && s0 > p0;               // gradients of earlier sweeps are already stored: add to them
     if (later_sweep) {
       if (warp == ISSUER / 32) tc::tma_store_wait_all_warp();
       __syncthreads();
@@ -188,12 +218,12 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
       const bool alive = bj != -INFINITY;                   // an empty cluster has beta = mu = -inf
       const float sig2 = dm.sigma * kLog2e, bj2 = alive ? bj * kLog2e : 0.f;
       if (jt + 1 < NJ) bnext = j + TJ < Ck ? beta[ent0 + j + TJ] : -INFINITY;
-      float gsum = 0.f, gt2 = 0.f, pdp = 0.f;
+      if constexpr (!ONE) gsum = gt2 = pdp = 0.f;
       const float mu1 = j < Ck ? 1.f + mu[ent0 + j] : 0.f;                              // 1 + accumulated log-mass of cluster j
       for (int p = 0; p < np && ok; ++p) {
         const uint32_t aQ = tc::smem_u32(sm + oQ + p * kRows), aDO = tc::smem_u32(sm + oDO + p * kRows);
         if (warp == ISSUER / 32) {
-          if (p == 0) {
+          if (p == 0 && load) {
             if (!tc::mbar_wait(&bar_full, ph_full)) ok = false;
             if (!tc::mbar_wait(&bar_nu, ph_full)) ok = false;
           }
@@ -212,7 +242,7 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
             tc::mma_bf16_ss_warp(tbase + cDP, tc::smem_desc_sw128(aNu + (ks / 4) * TJ * 128 + (ks % 4) * 32, 16, 1024),
                             tc::smem_desc_sw128(aDO + (ks / 4) * NR * 128 + (ks % 4) * 32, 16, 1024), idesc, ks > 0);
           tc::mma_commit_warp(&bar1);
-          if (p == 0) {
+          if (!ONE && p == 0) {
             tc::tma_store_wait_read_warp();        // the previous tile's stores have read the staging tiles, which the
             if (tc::elect_one()) tc::mbar_arrive(&bar_st);         // compute warps write again (P / G tiles first)
           }
@@ -231,7 +261,7 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
           const int nv = ns - wg * nc;
           const unsigned long long m64 = smask[2 * j] | (unsigned long long)smask[2 * j + 1] << 32;
           const uint32_t near = alive ? ((uint32_t)(m64 >> (wg * nc)) | (nv >= 32 ? 0u : nv <= 0 ? 0xffffffffu : 0xffffffffu << nv)) : 0xffffffffu;
-          if (p == 0) {                                    // (the previous tile's stores have read the staging tiles)
+          if (!ONE && p == 0) {                            // (the previous tile's stores have read the staging tiles)
             if (!tc::mbar_wait(&bar_st, ph_st)) ok = false;
             ph_st ^= 1;
           }
@@ -296,11 +326,11 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
 #pragma unroll
           for (int ks = 0; ks < NR / 16; ++ks) if (16 * ks < nr)
             tc::mma_bf16_ss_warp(tbase + cDNU, tc::smem_desc_sw128(aPt + ks * 32, 16, 1024),
-                            tc::smem_desc_sw128(aDO + ks * 16 * 128, NR * 128, 1024), id_row, !(p == 0 && ks == 0));
+                            tc::smem_desc_sw128(aDO + ks * 16 * 128, NR * 128, 1024), id_row, !(p == 0 && ks == 0 && load));
 #pragma unroll
           for (int ks = 0; ks < NR / 16; ++ks) if (16 * ks < nr)
             tc::mma_bf16_ss_warp(tbase + cDKA, tc::smem_desc_sw128(aGt + ks * 32, 16, 1024),
-                            tc::smem_desc_sw128(aQ + ks * 16 * 128, NR * 128, 1024), id_row, !(p == 0 && ks == 0));
+                            tc::smem_desc_sw128(aQ + ks * 16 * 128, NR * 128, 1024), id_row, !(p == 0 && ks == 0 && load));
           tc::mma_commit_warp(&bar2);              // the read-out of dnu / dkappa can start while the dq products still run
 #pragma unroll
           for (int ks = 0; ks < TJ / 16; ++ks)
@@ -326,6 +356,7 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
 #ifdef MUSE_PHASE_CLOCKS
       k3_ = clock64();
 #endif
+      if (!store) continue;
       // ---- tile read-out: warpgroup 0 -> dnu, warpgroup 1 -> dkappa; both need sum_r g
       float gtot = 0.f;
       if (cw) {
@@ -467,15 +498,16 @@ int far_bwd_tc(const Dims& d, const SummPtrs& sp, const void* Q, const void* dO,
   MUSE_RC(make_tmap_bf16_nd(&gnu, dnu, 4, grad_by_key_cluster ? dims_a : dims_b, grad_by_key_cluster ? str_a : str_b, box4));
   const size_t mask_bytes = (size_t)cdiv(d.Ck, fb::TJ) * fb::TJ * 8;
   prof_mark("k_far_bwd_tc", st);
-  if (d.D == 128) {
-    const size_t smem = (size_t)fb::Lay<128>::oMask + mask_bytes + 1024;
-    MUSE_CUDA_OK(cudaFuncSetAttribute(k_far_bwd_tc<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    MUSE_RC(launch_pdl(k_far_bwd_tc<128>, dim3(d.Cq, d.SB, d.B * d.Hq), fb::THREADS, smem, st, d, khi, klo, nu, gka, gnu, (const bf16*)Q, (const bf16*)dO, qbar, LSE, delta, off_q, perm_q, sel, sp.beta, sp.mu, dQacc, (bf16*)dkappa, (bf16*)dnu, dS, grad_by_key_cluster, status));
-  } else {
-    const size_t smem = (size_t)fb::Lay<64>::oMask + mask_bytes + 1024;
-    MUSE_CUDA_OK(cudaFuncSetAttribute(k_far_bwd_tc<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    MUSE_RC(launch_pdl(k_far_bwd_tc<64>, dim3(d.Cq, d.SB, d.B * d.Hq), fb::THREADS, smem, st, d, khi, klo, nu, gka, gnu, (const bf16*)Q, (const bf16*)dO, qbar, LSE, delta, off_q, perm_q, sel, sp.beta, sp.mu, dQacc, (bf16*)dkappa, (bf16*)dnu, dS, grad_by_key_cluster, status));
-  }
+#define MUSE_FAR_BWD(D_, ONE_)                                                                                                  \
+  do {                                                                                                                         \
+    const size_t smem = (size_t)fb::Lay<D_, ONE_>::oMask + mask_bytes + 1024;                                                   \
+    MUSE_CUDA_OK(cudaFuncSetAttribute(k_far_bwd_tc<D_, ONE_>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));         \
+    MUSE_RC(launch_pdl(k_far_bwd_tc<D_, ONE_>, dim3(d.Cq, d.SB, d.B * d.Hq), fb::THREADS, smem, st, d, khi, klo, nu, gka, gnu, (const bf16*)Q, (const bf16*)dO, qbar, LSE, delta, off_q, perm_q, sel, sp.beta, sp.mu, dQacc, (bf16*)dkappa, (bf16*)dnu, dS, grad_by_key_cluster, status)); \
+  } while (0)
+  const bool one = d.Ck <= fb::TJ;
+  if (d.D == 128) { if (one) MUSE_FAR_BWD(128, true); else MUSE_FAR_BWD(128, false); }
+  else { if (one) MUSE_FAR_BWD(64, true); else MUSE_FAR_BWD(64, false); }
+#undef MUSE_FAR_BWD
   MUSE_LAUNCH_OK();
   return MUSE_OK;
 }

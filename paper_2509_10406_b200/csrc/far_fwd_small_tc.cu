@@ -11,8 +11,8 @@
 // largest score and its votes; here 500 to 700 serve eight or four queries at once.
 //
 // Bound by instruction issue and the latency of the phases; two or three CTAs share an SM.  Against the other kernel: 32 heads
-// of 64k tokens, D = 64, 128 x 128 clusters, 8 slots 3130 -> 934 us; 32 heads of 16k, 128 x 256, 16 slots 1562 -> 686; 16 heads
-// of 8k, 64 x 128 367 -> 131; 6 heads of 9k, D = 128, 50 x 200, 10 slots 230 -> 94.
+// of 64k tokens, D = 64, 128 x 128 clusters, 8 slots 3130 -> 880 us; 32 heads of 16k, 128 x 256, 16 slots 1562 -> 621; 16 heads
+// of 8k, 64 x 128 367 -> 125; 6 heads of 9k, D = 128, 50 x 200, 10 slots 230 -> 94.
 #include <cuda.h>
 #include "common.cuh"
 #include "tc05.cuh"
@@ -138,14 +138,26 @@ k_far_fwd_small(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __gri
       rows[tid] = t;
     }
     // query rows -> K-major swizzled tile [64][D] bf16 (G blocks of [64][128 B])
-    for (int e = tid; e < n16 * (D / 8); e += kThreads) {
-      const int r = e / (D / 8), ck = e % (D / 8);
-      uint4 v = make_uint4(0u, 0u, 0u, 0u);
-      if (r < n && MUSE_IN_RANGE(pm[r0 + r], dm.N)) v = reinterpret_cast<const uint4*>(Qp + (size_t)pm[r0 + r] * D)[ck];
-      *reinterpret_cast<uint4*>(Qs + (ck >> 3) * kR * 128 + tc::sw128_off(r, ck & 7)) = v;
+    // (all of a thread's row numbers, then all of its rows are on their way at once: nothing else hides their latency)
+    constexpr int IT = kR * (D / 8) / kThreads;
+    int tq[IT];
+    uint4 vq[IT];
+#pragma unroll
+    for (int it = 0; it < IT; ++it) {
+      const int r = (tid + it * kThreads) / (D / 8);
+      tq[it] = r < n ? pm[r0 + r] : -1;
+      if (tq[it] >= 0 && !MUSE_IN_RANGE(tq[it], dm.N)) tq[it] = -1;
     }
     const int jb = (CT == 2 ? (warp >> 2) * kJ : 0) + (tid & 127);
     const float bq = jb < Ck ? beta[ent0 + jb] : -INFINITY;  // beta of this thread's cluster in phase B
+#pragma unroll
+    for (int it = 0; it < IT; ++it)
+      vq[it] = tq[it] >= 0 ? reinterpret_cast<const uint4*>(Qp + (size_t)tq[it] * D)[(tid + it * kThreads) % (D / 8)] : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+    for (int it = 0; it < IT; ++it) {
+      const int r = (tid + it * kThreads) / (D / 8), ck = (tid + it * kThreads) % (D / 8);
+      if (r < n16) *reinterpret_cast<uint4*>(Qs + (ck >> 3) * kR * 128 + tc::sw128_off(r, ck & 7)) = vq[it];
+    }
     tc::fence_async_smem();
     __syncthreads();
     if (warp == 0) {

@@ -330,11 +330,23 @@ k_far_fwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
         if (wa == prod) produce_a(t);
     if (tid < FR) rows[tid] = tid < n ? pm[r0 + tid] : -1;
     // query rows -> K-major swizzled tile [FR][D] bf16 (G blocks of [FR][128 B])
-    for (int e = tid; e < FR * (D / 8); e += NT) {
-      const int r = e / (D / 8), ck = e % (D / 8), kb = ck >> 3, c = ck & 7;
-      uint4 v = make_uint4(0u, 0u, 0u, 0u);
-      if (r < n && MUSE_IN_RANGE(r0 + r, dm.N) && MUSE_IN_RANGE(pm[r0 + r], dm.N)) v = reinterpret_cast<const uint4*>(Qp + (size_t)pm[r0 + r] * D)[ck];
-      *reinterpret_cast<uint4*>(Qs + kb * FR * 128 + tc::sw128_off(r, c)) = v;
+    // (all of a thread's row numbers, then all of its rows are on their way at once: nothing else hides their latency)
+    constexpr int IT = (FR * (D / 8) + NT - 1) / NT;
+    int tq[IT];
+    uint4 vq[IT];
+#pragma unroll
+    for (int it = 0; it < IT; ++it) {
+      const int r = (tid + it * NT) / (D / 8);
+      tq[it] = r < n && MUSE_IN_RANGE(r0 + r, dm.N) ? pm[r0 + r] : -1;
+      if (tq[it] >= 0 && !MUSE_IN_RANGE(tq[it], dm.N)) tq[it] = -1;
+    }
+#pragma unroll
+    for (int it = 0; it < IT; ++it)
+      vq[it] = tq[it] >= 0 ? reinterpret_cast<const uint4*>(Qp + (size_t)tq[it] * D)[(tid + it * NT) % (D / 8)] : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+    for (int it = 0; it < IT; ++it) {
+      const int r = (tid + it * NT) / (D / 8), ck = (tid + it * NT) % (D / 8);
+      if (r < FR) *reinterpret_cast<uint4*>(Qs + (ck >> 3) * FR * 128 + tc::sw128_off(r, ck & 7)) = vq[it];
     }
     tc::fence_async_smem();
     tc::fence_before_sync();

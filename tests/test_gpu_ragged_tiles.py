@@ -74,3 +74,11 @@ def test_selection_and_far_field_of_few_clusters(base, Cq, Ck, m):
     """Lists of 8 and 16 (and one more, which another kernel takes), one and two tiles of clusters, several passes over a segment."""
     w = CASES[base].with_(Hq=2, Hkv=1, N=1020, S=4, Cq=Cq, Ck=Ck, m=m, components=64)
     _forward_parity(w, 128.0, expect_kernels=TC_FWD_KERNELS)
+
+
+@pytest.mark.parametrize("base,Cq,Ck,m", [("d64", 1, 128, 20), ("d64", 2, 129, 33), ("d128", 1, 128, 33), ("d128", 3, 90, 4)])
+def test_far_field_and_key_side_backward_over_long_segments(base, Cq, Ck, m):
+    """Segments of several sweeps over one tile of clusters (accumulated on chip) and over two (added in memory), and selections
+    longer than the far-field backward keeps in flight."""
+    w = CASES[base].with_(Hq=2, Hkv=1, N=1020, S=4, Cq=Cq, Ck=Ck, m=m, components=64)
+    _backward_parity(w, 128.0, expect_kernels=TC_BWD_KERNELS)
