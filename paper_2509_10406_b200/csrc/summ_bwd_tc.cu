@@ -12,6 +12,13 @@
 // the planes in registers and contracted with them once.  Planes are handled independently and
 // accumulate, together with the query-cluster tiles, in tensor memory; the far-field backward
 // stores its gradients [plane][j][i] so that each (plane, j, 128 i) tile is one contiguous TMA box.
+//
+// Bound by the latency of a plane's steps at D = 64 (two CTAs per SM), by DRAM and that latency at D = 128.  c needs only the
+// sum of its two contractions, so they share an accumulator; the tilt logits stay in tensor memory; with the freed registers
+// nothing spills, which matters because the tiles leave next to no L1 cache (spilled words, and the bucket offsets that are now
+// in shared memory, came from L2 on every plane: 2000 cycles).  32 heads of 64k tokens, 128 x 128 clusters, D = 64 2485 ->
+// 1682 us; 32 heads of 16k, 128 x 256 1222 -> 771; 16 heads of 8k, 64 x 128 322 -> 209; 4 heads of 64k, D = 128, 256 x 1024
+// 1280 -> 1201.
 #include <cuda.h>
 #include "common.cuh"
 #include "tc05.cuh"
@@ -32,7 +39,9 @@ template <int D> struct Lay {
   static constexpr int oK = oDnu1 + kTile, oV = oK + kKeys, oW = oV + kKeys;
   static constexpr int total = oW + TI * NU * 2;           // 112 KB at D = 64, two CTAs per SM: no slack, the kernel checks the alignment of its base
 };
-constexpr uint32_t cL = 0, cX1 = 0, cX2 = 64, cDK = 128, cDV = 192, cols = 256;        // (X1 over the tilt logits, which go to registers)
+// tilt logits, X = dkappa.k + dnu.v of a plane, the accumulators
+constexpr uint32_t cL = 0, cX = 64, cDK = 128, cDV = 192, cols = 256;
+constexpr int kOkCache = 72;                   // bucket offsets of the cluster kept in shared memory (S + 1 <= 72)
 }  // namespace sb
 
 // 2-D tensor map over a bf16 matrix with an arbitrary row pitch (bytes), 128B swizzle, box [box_rows][64]
@@ -57,20 +66,25 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
   extern __shared__ __align__(1024) unsigned char sm_raw[];
   __shared__ uint64_t bar_g[2], bar_kv, bar_q, bar_l, bar1, bar2;
   __shared__ uint32_t tbase_s;
+  __shared__ int32_t oks[kOkCache];
   const int j = blockIdx.x, pq = blockIdx.y;
   const int b_ = pq / dm.Hq, h = pq % dm.Hq, pk = b_ * dm.Hkv + dm.hm.g[h];
   const int tid = threadIdx.x, warp = tc::warp_index(), wg = tid >> 7, L = tid & 127;
   const bool cw = warp < 8;                               // compute warp (the ninth warp only issues)
-  const int32_t* ok_ = off_k + (size_t)pk * (dm.Ck * dm.S + 1) + (size_t)j * dm.S;
+  const int32_t* okg = off_k + (size_t)pk * (dm.Ck * dm.S + 1) + (size_t)j * dm.S;
   const int32_t* oq = off_q + (size_t)pq * (dm.S * dm.Cq + 1);
-  const int kbeg = ok_[0];
-  (void)MUSE_IN_RANGE(ok_[dm.SB], dm.N + 1); (void)MUSE_IN_RANGE(kbeg, ok_[dm.SB] + 1);   // (the tiles come through tensor maps, which clip)
-  if (kbeg >= ok_[dm.SB]) return;                       // no key of this cluster is ever summarised
+  const int kbeg = okg[0], kvis = okg[dm.SB];
+  (void)MUSE_IN_RANGE(kvis, dm.N + 1); (void)MUSE_IN_RANGE(kbeg, kvis + 1);   // (the tiles come through tensor maps, which clip)
+  if (kbeg >= kvis) return;                       // no key of this cluster is ever summarised
   unsigned char* sm = sm_raw;
   if ((tc::smem_u32(sm_raw) & 1023u) != 0u) {              // (the toolchain honours the declared alignment)
     if (tid == 0) report_status(status, 5);
     return;
   }
+  // (the tiles leave little of the L1 cache: what every plane asks for is kept in shared memory)
+  const bool cached = dm.SB < kOkCache;
+  if (cached && tid <= dm.SB) oks[tid] = okg[tid];
+  const int32_t* ok_ = cached ? oks : okg;
   if (warp == 0) tc::tmem_alloc(&tbase_s, cols);
   if (tid == 0) {
     tc::mbar_init(&bar_g[0], 1); tc::mbar_init(&bar_g[1], 1); tc::mbar_init(&bar_kv, 1); tc::mbar_init(&bar_q, 1); tc::mbar_init(&bar_l, 1);
@@ -80,13 +94,13 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
   __syncthreads();
   tc::fence_after_sync();
   pdl_trigger();                                           // (tensor memory has been allocated)
+  uint32_t livemask = 0u;
   const uint32_t tbase = tbase_s, tlane = tbase + ((uint32_t)((warp & 3) * 32) << 16);
-  uint32_t ph_g[2] = {0, 0}, ph_kv = 0, ph_q = 0, ph_l = 0, ph1 = 0, ph2 = 0;
+  uint32_t ph_g = 0, ph_kv = 0, ph_q = 0, ph_l = 0, ph1 = 0, ph2 = 0;
   bool ok = true;
   const uint32_t aQhi = tc::smem_u32(sm + oQhi), aQlo = tc::smem_u32(sm + oQlo), aK = tc::smem_u32(sm + oK),
                  aV = tc::smem_u32(sm + oV), aW = tc::smem_u32(sm + oW);
 
-  const int kvis = ok_[dm.SB];
 #ifdef MUSE_PHASE_CLOCKS
   long long pc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
   long long t_ = clock64();
@@ -108,8 +122,8 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
     while (pl0 < dm.SB && ok_[pl0 + 1] <= c0) ++pl0;
     int pl_end = dm.SB;
     if (per_block) { pl_end = pl0; while (pl_end < dm.SB && ok_[pl_end] < c0 + NU) ++pl_end; }
-    if (!tc::mbar_wait(&bar_kv, ph_kv)) ok = false;
-    ph_kv ^= 1;
+    // (D = 128: the gradient tiles of the chunk queue up behind its keys in DRAM: 1240 -> 1201 us)
+    if (D == 128 && !tc::mbar_wait(&bar_kv, ph_kv)) ok = false;
     bool started = false;                                 // dK^T / dV^T accumulate in TMEM over all (i tile, plane)
     for (int i0 = 0; i0 < dm.Cq && ok; i0 += TI) {
       const int i = i0 + L;
@@ -136,15 +150,25 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
         }
         if (pl0 < pl_end) issue_grad(pl0, 0);
       }
-      // which planes hold a non-empty segment of query cluster i (others were never written by the far-field pass)
-      uint32_t livemask = 0u;
-      for (int pl = pl0; pl < pl_end; ++pl) {
-        const int blk = dm.causal ? pl + 1 : 0;
-        // (per-block gradients are zero-filled before they are accumulated: every plane's rows are valid)
-        if (in_range && (per_block || oq[(size_t)blk * dm.Cq + i + 1] > oq[(size_t)blk * dm.Cq + i])) livemask |= 1u << pl;
+      // which planes hold a non-empty segment of query cluster i (others were never written by the far-field pass); the same for
+      // every chunk of keys
+      if (cw && (c0 == kbeg || dm.Cq > TI)) {
+        livemask = 0u;
+#pragma unroll 4
+        for (int pl = 0; pl < dm.SB; ++pl) {
+          const int32_t* o = oq + (size_t)(dm.causal ? pl + 1 : 0) * dm.Cq + ic;
+          // (per-block gradients are zero-filled before they are accumulated: every plane's rows are valid)
+          livemask |= in_range && (per_block || o[1] > o[0]) ? 1u << pl : 0u;
+        }
       }
+      // per-plane scalars, loaded one plane ahead
+      auto ent_of = [&](int pl) { return (((size_t)pq * dm.SB + pl) * dm.Cq + ic) * dm.Ck + j; };        // summaries: [plane][i][j]
+      auto gent_of = [&](int pl) { return (((size_t)pq * dm.SB + pl) * dm.Ck + j) * dm.Cq + ic; };      // gradients: [plane][j][i]
+      float mu_n = 0.f, dS_n = 0.f;
+      if (pl0 < pl_end && ((livemask >> pl0) & 1u)) { mu_n = mu[ent_of(pl0)]; dS_n = dS[gent_of(pl0)]; }
       // tilt logits l_iu = sigma qbar_i . k_u, the same for every plane: once per centroid tile
       if (warp == ISSUER / 32) {
+        if (D == 64 && i0 == 0 && !tc::mbar_wait(&bar_kv, ph_kv)) ok = false;
         if (!tc::mbar_wait(&bar_q, ph_q)) ok = false;
         tc::fence_after_sync();
         const uint32_t idesc = tc::idesc_bf16(TI, NU, 0, 0);
@@ -158,29 +182,17 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
                           tc::smem_desc_sw128(aK + (ks / 4) * NU * 128 + (ks % 4) * 32, 16, 1024), idesc, 1);
         tc::mma_commit_warp(&bar_l);
       }
+      if (i0 == 0) ph_kv ^= 1;
       ph_q ^= 1;
       __syncwarp();
       if (!tc::mbar_wait(&bar_l, ph_l)) ok = false;       // from here on the low tile's space is free
       ph_l ^= 1;
       tc::fence_after_sync();
       PCLK(0)
-      float lg[32];
-      if (cw) {                                                   // this thread's logits: row i, keys 32 wg .. 32 wg + 31 (log2 units)
-        tc::tmem_ld32(tlane + cL + 32 * wg, lg);
-#pragma unroll
-        for (int c = 0; c < 32; ++c) lg[c] *= 1.4426950408889634f;
-      }
       float wc[32];                                               // sum over the planes of w c: contracted with the centroids once, below
 #pragma unroll
       for (int c = 0; c < 32; ++c) wc[c] = 0.f;
-      tc::fence_before_sync();
-      __syncthreads();                                            // the products of the first plane overwrite the logits
-      tc::fence_after_sync();
-      // per-plane scalars, loaded one plane ahead
-      auto ent_of = [&](int pl) { return (((size_t)pq * dm.SB + pl) * dm.Cq + ic) * dm.Ck + j; };        // summaries: [plane][i][j]
-      auto gent_of = [&](int pl) { return (((size_t)pq * dm.SB + pl) * dm.Ck + j) * dm.Cq + ic; };      // gradients: [plane][j][i]
-      float mu_n = 0.f, dS_n = 0.f;
-      if (pl0 < pl_end && ((livemask >> pl0) & 1u)) { mu_n = mu[ent_of(pl0)]; dS_n = dS[gent_of(pl0)]; }
+      bool early = false;                                         // (issuer) the D-contractions of the plane are under way
       for (int pl = pl0, k = 0; pl < pl_end && ok; ++pl, ++k) {
         const int buf = k & 1;
         const int nk = min(NU, ok_[pl + 1] - c0);
@@ -191,26 +203,32 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
         const uint32_t aDka = tc::smem_u32(sm + oDka), aDnu = tc::smem_u32(sm + oDnu);
         if (pl + 1 < pl_end && ((livemask >> (pl + 1)) & 1u)) { mu_n = mu[ent_of(pl + 1)]; dS_n = dS[gent_of(pl + 1)]; }
         // The far-field pass wrote every row of the gradient tensors (zeros for an empty segment), so the
-        // tiles go to the tensor cores as they land.  The D-contractions of this plane do not depend on the
-        // previous plane's i-contractions: they are issued first, and only the W tile and the other
-        // gradient buffer wait for those.
-        if (warp == ISSUER / 32) {
-          if (!tc::mbar_wait(&bar_g[buf], ph_g[buf])) ok = false;
-          tc::fence_after_sync();
-          const uint32_t idesc = tc::idesc_bf16(TI, NU, 0, 0);
+        // tiles go to the tensor cores as they land.  The D-contractions of a plane do not depend on the
+        // previous plane's i-contractions: they are issued before them if the tiles are there by then, and only the W
+        // tile and the other gradient buffer wait for those.
+        auto issue_x = [&](int kk) {
+          const uint32_t aA = tc::smem_u32(sm + ((kk & 1) ? oQlo : oDka0)), aB = tc::smem_u32(sm + ((kk & 1) ? oDnu1 : oDnu0));
+          const uint32_t idesc = tc::idesc_bf16(TI, NU, 0, 0), col = tbase + cX;
 #pragma unroll
           for (int ks = 0; ks < D / 16; ++ks)
-            tc::mma_bf16_ss_warp(tbase + cX1, tc::smem_desc_sw128(aDka + (ks / 4) * TI * 128 + (ks % 4) * 32, 16, 1024),
+            tc::mma_bf16_ss_warp(col, tc::smem_desc_sw128(aA + (ks / 4) * TI * 128 + (ks % 4) * 32, 16, 1024),
                             tc::smem_desc_sw128(aK + (ks / 4) * NU * 128 + (ks % 4) * 32, 16, 1024), idesc, ks > 0);
 #pragma unroll
           for (int ks = 0; ks < D / 16; ++ks)
-            tc::mma_bf16_ss_warp(tbase + cX2, tc::smem_desc_sw128(aDnu + (ks / 4) * TI * 128 + (ks % 4) * 32, 16, 1024),
-                            tc::smem_desc_sw128(aV + (ks / 4) * NU * 128 + (ks % 4) * 32, 16, 1024), idesc, ks > 0);
+            tc::mma_bf16_ss_warp(col, tc::smem_desc_sw128(aB + (ks / 4) * TI * 128 + (ks % 4) * 32, 16, 1024),
+                            tc::smem_desc_sw128(aV + (ks / 4) * NU * 128 + (ks % 4) * 32, 16, 1024), idesc, 1);
           tc::mma_commit_warp(&bar1);
+        };
+        if (warp == ISSUER / 32) {
+          if (!early) {
+            if (!tc::mbar_wait(&bar_g[buf], (ph_g >> buf) & 1u)) ok = false;
+            tc::fence_after_sync();
+            issue_x(k);
+          }
           if (k > 0 && !tc::mbar_wait(&bar2, ph2)) ok = false;      // the previous plane's MMAs are done with the other buffer
           if (pl + 1 < pl_end && ok) issue_grad(pl + 1, buf ^ 1);
         }
-        ph_g[buf] ^= 1;
+        ph_g ^= 1u << buf;
         PCLK(1)
         if (cw && !tc::mbar_wait(&bar1, ph1)) ok = false;
         ph1 ^= 1;
@@ -219,30 +237,46 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
         if (cw) {
           const int lo = live ? klo - 32 * wg : 32, hi = live ? nk - 32 * wg : 0;      // this thread's keys of the plane: [lo, hi)
           const bool whole = lo <= 0 && hi >= 32;
-          if (k > 0 && !tc::mbar_wait(&bar2, ph2)) ok = false;      // the previous plane's MMAs have read W
-#pragma unroll
-          for (int g = 0; g < 4; ++g) {
-            float x1[8], x2[8];
-            tc::tmem_ld8_issue(tlane + cX1 + 32 * wg + 8 * g, x1);
-            tc::tmem_ld8_issue(tlane + cX2 + 32 * wg + 8 * g, x2);
-            tc::tmem_ld_wait();
-            tc::tmem_ld_use8(x1);
-            tc::tmem_ld_use8(x2);
-            uint32_t ww[4];
+          const uint32_t tx = tlane + cX + 32 * wg, tl = tlane + cL + 32 * wg;
+          auto weigh = [&](int g, const float* l, const float* x, uint32_t* ww) {
 #pragma unroll
             for (int c = 0; c < 8; c += 2) {
               float w[2];
 #pragma unroll
               for (int e = 0; e < 2; ++e) {
                 const int u = 8 * g + c + e;
-                w[e] = tc::fast_exp2(lg[u] - mu_i);
+                w[e] = tc::fast_exp2(fmaf(l[c + e], 1.4426950408889634f, -mu_i));
                 if (!whole) w[e] = u >= lo && u < hi ? w[e] : 0.f;
-                wc[u] = fmaf(w[e], dS_i + x1[c + e] + x2[c + e], wc[u]);
+                wc[u] = fmaf(w[e], dS_i + x[c + e], wc[u]);
               }
               const __nv_bfloat162 a = __floats2bfloat162_rn(w[0], w[1]);
               ww[c / 2] = *reinterpret_cast<const uint32_t*>(&a);
             }
-            *reinterpret_cast<uint4*>(sm + oW + tc::sw128_off(L, 4 * wg + g)) = make_uint4(ww[0], ww[1], ww[2], ww[3]);
+          };
+          float l[2][8], x[2][8];
+          uint32_t ww[2][4];
+          tc::tmem_ld8_issue(tl, l[0]);
+          tc::tmem_ld8_issue(tx, x[0]);
+          tc::tmem_ld_wait();
+          tc::tmem_ld_use8(l[0]);
+          tc::tmem_ld_use8(x[0]);
+#pragma unroll
+          for (int g = 0; g < 4; ++g) {
+            if (g < 3) {
+              tc::tmem_ld8_issue(tl + 8 * (g + 1), l[(g + 1) & 1]);
+              tc::tmem_ld8_issue(tx + 8 * (g + 1), x[(g + 1) & 1]);
+            }
+            weigh(g, l[g & 1], x[g & 1], ww[g & 1]);
+            if (g == 1) {
+              if (k > 0 && !tc::mbar_wait(&bar2, ph2)) ok = false;  // the previous plane's MMAs have read W
+              *reinterpret_cast<uint4*>(sm + oW + tc::sw128_off(L, 4 * wg)) = make_uint4(ww[0][0], ww[0][1], ww[0][2], ww[0][3]);
+            }
+            if (g > 0) *reinterpret_cast<uint4*>(sm + oW + tc::sw128_off(L, 4 * wg + g)) = make_uint4(ww[g & 1][0], ww[g & 1][1], ww[g & 1][2], ww[g & 1][3]);
+            if (g < 3) {
+              tc::tmem_ld_wait();
+              tc::tmem_ld_use8(l[(g + 1) & 1]);
+              tc::tmem_ld_use8(x[(g + 1) & 1]);
+            }
           }
         }
         if (k > 0) ph2 ^= 1;
@@ -251,6 +285,8 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
         __syncthreads();
         if (warp == ISSUER / 32) {
           tc::fence_after_sync();
+          early = D == 64 && pl + 1 < pl_end && ok && __all_sync(0xffffffffu, tc::mbar_test(&bar_g[buf ^ 1], (ph_g >> (buf ^ 1)) & 1u));
+          if (early) issue_x(k + 1);
           // A [i][d] and B [i][u]: both contract over rows.  M = 128 output dims even when D = 64: the second 64-dim group
           // of the A operand is then the tile that follows in shared memory, and output lanes 64..127 hold numbers that nobody reads
           const uint32_t idesc = tc::idesc_bf16(128, NU, 1, 1);
