@@ -37,27 +37,32 @@ __device__ __forceinline__ void load_tile_f32(float* __restrict__ dst, const T* 
   }
 }
 
-// delta_t = sum_d dO[t][d] * O[t][d]; one warp per row.  The first kernel of the pass: it also zeroes the bucketed gradients, which later
-// kernels add to, and the status words.
+// delta_t = sum_d dO[t][d] * O[t][d]; 8 dims per lane, D / 8 lanes per row.  The first kernel of the pass: it also zeroes the bucketed
+// gradients, which later kernels add to, and the status words.
 template <class T, int D>
 __global__ void k_delta(const T* __restrict__ O, const T* __restrict__ dO, long long rows, float* __restrict__ delta, float* __restrict__ dK_perm,
                         float* __restrict__ dV_perm, int32_t* __restrict__ clear) {
-  const long long r = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
+  constexpr int L = D / 8;
+  const long long r = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / L;
+  const int d0 = threadIdx.x % L * 8;
   pdl_wait();
   pdl_trigger();
   if (clear != nullptr && blockIdx.x == 0 && threadIdx.x < kStatusWords) clear[threadIdx.x] = 0;
-  if (r >= rows) return;
-  constexpr int Z = D / 4;                                 // 16-byte pieces of an fp32 row
-  if (lane < Z) {
-    st4(dK_perm + r * D + 4 * lane, make_float4(0.f, 0.f, 0.f, 0.f));
-    st4(dV_perm + r * D + 4 * lane, make_float4(0.f, 0.f, 0.f, 0.f));
+  const bool in = r < rows;
+  const long long at = (in ? r : 0) * D + d0;
+  float a[8], b[8], s = 0.f;
+  ld8(O + at, a);
+  ld8(dO + at, b);
+  if (in) {
+    const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+    st4(dK_perm + at, z); st4(dK_perm + at + 4, z);
+    st4(dV_perm + at, z); st4(dV_perm + at + 4, z);
   }
-  float s = 0.f;
 #pragma unroll
-  for (int k = 0; k < D / 32; ++k) s = fmaf(to_f(O[r * D + lane + 32 * k]), to_f(dO[r * D + lane + 32 * k]), s);
-  s = warp_sum(s);
-  if (lane == 0) delta[r] = s;
+  for (int k = 0; k < 8; ++k) s = fmaf(a[k], b[k], s);
+#pragma unroll
+  for (int o = L / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (in && d0 == 0) delta[r] = s;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -767,7 +772,7 @@ static int attn_bwd_t(const Dims& d, int dtype, const T* Q, const T* K, const T*
   const size_t nd = (size_t)pq * d.N * d.D * sizeof(float);
   const long long rows = (long long)pq * d.N;
   prof_mark("k_delta", st);
-  MUSE_RC(launch_pdl(k_delta<T, D>, dim3((unsigned)((rows + 7) / 8)), 256, 0, st, O, dO, rows, w.delta, w.dK_perm, w.dV_perm,
+  MUSE_RC(launch_pdl(k_delta<T, D>, dim3((unsigned)((rows * (D / 8) + 255) / 256)), 256, 0, st, O, dO, rows, w.delta, w.dK_perm, w.dV_perm,
                      fresh_status ? w.status : (int32_t*)nullptr));
   const size_t sm4 = 4 * tile_bytes<T, D>() + ptile_bytes();
   constexpr bool kTensor = sizeof(T) == 2;      // bf16 mode runs the exact-attention parts on tcgen05
