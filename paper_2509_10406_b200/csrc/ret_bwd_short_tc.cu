@@ -9,14 +9,19 @@
 //   P, G                               one thread per pair row, written as bf16 tiles to shared memory
 //   dQ = G K                           over the tensor-memory columns that S and dP have vacated
 //   dV^T += dO^T P,  dK^T += Q^T G     [D][keys], accumulated in tensor memory over all of the CTA's tiles
-// The tiles of Q, dO, P and G fill shared memory, so only one CTA fits an SM; to keep the tensor cores, the
-// load/store unit and the arithmetic warps busy at the same time, the CTA runs TWO independent pipelines
-// ("halves") that share the key / value tiles and take alternate pair tiles.  Each half has four row warps,
+// To keep the tensor cores, the load/store unit and the arithmetic warps busy at the same time, an SM runs TWO independent
+// pipelines.  At D = 64 they are two CTAs, so that the start of one cluster (its index entries, keys and first rows) and the end of
+// another run beside products.  At D = 128 the tiles of Q, dO, P and G of two pipelines ("halves") fill shared memory and one CTA
+// has both, which share the key / value tiles and take alternate pair tiles.  Each pipeline has four row warps,
 // an MMA-issuing warp and four gather warps (the Q and dO rows arrive by 16-byte asynchronous copies, whose rate
 // grows with the number of threads that issue them; no arithmetic warp spends its time on them), its own 256 tensor-memory columns, its own
 // barriers and its own dV^T / dK^T accumulators, added to global memory with float atomics at the end of a sweep.
 // A cluster with more than 64 visible keys takes further sweeps over the tiles that see them; later sweeps
 // add to the stored dQ rows.
+//
+// Bound by the latency of a tile's chain (gather, S, P and G, dQ) where a cluster has only a few tiles.  D = 64: 16 heads of 8k
+// tokens, 128 clusters, 8 slots 361 -> 254 us; 24 heads of 4k, 128 clusters, 8 slots, non-causal 353 -> 238; D = 128: 6 heads of 9k,
+// 200 clusters, 10 slots 265 -> 235.
 #include <cuda.h>
 #include "common.cuh"
 #include "tc05.cuh"
@@ -27,13 +32,15 @@ typedef __nv_bfloat16 bf16;
 
 namespace rs {
 constexpr int kPairs = 128, kKeys = 64;
-constexpr int kRowWarps = 4, kIssuerWarp0 = 8, kGatherWarp0 = 10, kGather = 128, kThreads = (kGatherWarp0 + 2 * kGather / 32) * 32;
+constexpr int kRowWarps = 4, kGather = 128;
 constexpr int kOkCache = 72;
 constexpr float kLog2e = 1.4426950408889634f;
 template <int D> struct Lay {
+  static constexpr int NH = D == 64 ? 1 : 2;               // pipelines of a CTA; at D = 64 there are two CTAs on an SM instead
+  static constexpr int kIssuerWarp0 = NH * kRowWarps, kGatherWarp0 = kIssuerWarp0 + NH, kThreads = (kGatherWarp0 + NH * kGather / 32) * 32;
   static constexpr int kTile = kPairs * D * 2, kKV = kKeys * D * 2, kPG = kPairs * kKeys * 2;
   static constexpr int oK = 0, oV = kKV, oHalf = 2 * kKV, kHalf = 2 * kTile + 2 * kPG;   // per half: Q | dO | P | G
-  static constexpr int kSmem = oHalf + 2 * kHalf;           // 224 KB at D = 128: no slack, the kernel checks the alignment of its base
+  static constexpr int kSmem = oHalf + NH * kHalf;          // 224 KB at D = 128: no slack, the kernel checks the alignment of its base
 };
 constexpr uint32_t cS = 0, cDP = 64, cDQ = 0, cDV = 128, cDK = 192, kCols = 256;   // per half; dQ reuses the columns of S and dP
 
@@ -53,7 +60,7 @@ template <int ROWS> __device__ __forceinline__ uint64_t desc_mn(uint32_t base, i
 }  // namespace rs
 
 template <int D>
-__global__ void __launch_bounds__(rs::kThreads, 1)
+__global__ void __launch_bounds__(rs::Lay<D>::kThreads, D == 64 ? 2 : 1)
 k_ret_bwd_sweeps(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ dO, const bf16* __restrict__ Kp,
                    const bf16* __restrict__ Vp, const float* __restrict__ LSE, const float* __restrict__ delta,
                    const int32_t* __restrict__ off_k, const __grid_constant__ RetIndex ri,
@@ -62,11 +69,12 @@ k_ret_bwd_sweeps(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ d
   using namespace rs;
   typedef Lay<D> LY;
   constexpr int kTile = LY::kTile, kPG = LY::kPG, oK = LY::oK, oV = LY::oV, oHalf = LY::oHalf, kHalf = LY::kHalf;
+  constexpr int NH = LY::NH, kIssuerWarp0 = LY::kIssuerWarp0, kGatherWarp0 = LY::kGatherWarp0, kThreads = LY::kThreads;
   extern __shared__ __align__(1024) unsigned char sm[];
-  __shared__ Bars bars[2];
+  __shared__ Bars bars[NH];
   __shared__ uint32_t tbase_s;
   __shared__ int32_t ok_s[kOkCache];
-  __shared__ int32_t tok_s[2][kPairs];                      // tokens of the tile each half is gathering
+  __shared__ int32_t tok_s[NH][kPairs];                     // tokens of the tile each half is gathering
   const int tid = threadIdx.x, warp = tc::warp_index(), lane = tid & 31;
   // With spatial block selection (k2 > 0) the CTA owns one BUCKET (cluster j, block bb): its pairs are the (query, slot,
   // chosen block) triples that chose the block, and every one of them sees the whole bucket (as in the forward kernel).
@@ -90,9 +98,9 @@ k_ret_bwd_sweeps(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ d
   const int32_t* ok = dm.S + 1 <= kOkCache ? ok_s : okg;
   if (dm.S + 1 <= kOkCache)
     for (int b = tid; b <= dm.S; b += kThreads) ok_s[b] = okg[b];
-  if (warp == 0) tc::tmem_alloc(&tbase_s, 2 * kCols);
+  if (warp == 0) tc::tmem_alloc(&tbase_s, NH * kCols);
   if (tid == 0) {
-    for (int v = 0; v < 2; ++v) {
+    for (int v = 0; v < NH; ++v) {
       tc::mbar_init(&bars[v].q_full, kGather); tc::mbar_init(&bars[v].q_empty, 1); tc::mbar_init(&bars[v].s_done, 1);
       tc::mbar_init(&bars[v].pg_ready, kRowWarps * 32); tc::mbar_init(&bars[v].m2_done, 1); tc::mbar_init(&bars[v].dq_free, kRowWarps * 32);
     }
@@ -109,7 +117,7 @@ k_ret_bwd_sweeps(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ d
   const int32_t* pr = ri.pairs + (size_t)pq * dm.N * mk;
   const size_t pbase = (size_t)pq * dm.N * mk;
   // role of this warp: half v, and row / issuing / gather warp
-  const bool roww = warp < 2 * kRowWarps, issw = warp >= kIssuerWarp0 && warp < kIssuerWarp0 + 2, gatw = warp >= kGatherWarp0;
+  const bool roww = warp < NH * kRowWarps, issw = warp >= kIssuerWarp0 && warp < kIssuerWarp0 + NH, gatw = warp >= kGatherWarp0;
   const int v = roww ? warp / kRowWarps : issw ? warp - kIssuerWarp0 : (warp - kGatherWarp0) / (kGather / 32);
   Bars& B = bars[v];
   unsigned char* hb = sm + oHalf + v * kHalf;               // this half's Q | dO | P | G tiles
@@ -143,24 +151,30 @@ k_ret_bwd_sweeps(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ d
       while (pl + 1 < dm.SB && ok[pl + 1] - k0 <= kc) ++pl;
       tile_lo = (go[pl] - g0) / kPairs;
     }
-    const int tile0 = tile_lo + ((sub - tile_lo % nsub) + nsub) % nsub + v * nsub;   // this half's first tile; it takes every second of the CTA's
-    const int tstep = 2 * nsub;
+    const int tile0 = tile_lo + ((sub - tile_lo % nsub) + nsub) % nsub + v * nsub;   // this half's first tile; it takes every NH-th of the CTA's
+    const int tstep = NH * nsub;
     __syncthreads();                                        // the previous sweep's products are complete, its accumulators read
     // the sweep's keys and values as [2][64 rows][128 B] swizzled tiles (K-major and MN-major operands); rows past the cluster are zeros
-    for (int e = tid; e < kKeys * (D / 8); e += kThreads) {
-      const int r = e / (D / 8), ck = e % (D / 8);
-      uint4 a = make_uint4(0u, 0u, 0u, 0u), b = a;
-      if (r < nkc && MUSE_IN_RANGE(k0 + kc + r, dm.N)) {
-        a = reinterpret_cast<const uint4*>(Kb + (size_t)(kc + r) * D)[ck];
-        b = reinterpret_cast<const uint4*>(Vb + (size_t)(kc + r) * D)[ck];
+    // (the gather warps have begun with the first tile meanwhile)
+    const int at0 = g0 + tile0 * kPairs + (tid & 127);
+    const int id0 = roww && tile0 < ntiles && at0 < g1 ? __ldg(pr + at0) : -1;
+    if (!gatw) {
+      constexpr int NT = kGatherWarp0 * 32;
+      for (int e = tid; e < kKeys * (D / 8); e += NT) {
+        const int r = e / (D / 8), ck = e % (D / 8);
+        uint4 a = make_uint4(0u, 0u, 0u, 0u), b = a;
+        if (r < nkc && MUSE_IN_RANGE(k0 + kc + r, dm.N)) {
+          a = reinterpret_cast<const uint4*>(Kb + (size_t)(kc + r) * D)[ck];
+          b = reinterpret_cast<const uint4*>(Vb + (size_t)(kc + r) * D)[ck];
+        }
+        const uint32_t off = (ck >> 3) * kKeys * 128 + tc::sw128_off(r, ck & 7);
+        if (!MUSE_IN_RANGE(off, kKeys * D * 2 - 15)) continue;
+        *reinterpret_cast<uint4*>(sm + oK + off) = a;
+        *reinterpret_cast<uint4*>(sm + oV + off) = b;
       }
-      const uint32_t off = (ck >> 3) * kKeys * 128 + tc::sw128_off(r, ck & 7);
-      if (!MUSE_IN_RANGE(off, kKeys * D * 2 - 15)) continue;
-      *reinterpret_cast<uint4*>(sm + oK + off) = a;
-      *reinterpret_cast<uint4*>(sm + oV + off) = b;
+      tc::fence_async_smem();                               // the tensor cores read the tiles through the async proxy
+      tc::named_bar_sync(1 + NH, NT);
     }
-    tc::fence_async_smem();                                 // the tensor cores read the tiles through the async proxy
-    __syncthreads();
 
     if (roww) {
       // ================= P, G and the dQ rows: thread = pair row =================
@@ -170,7 +184,7 @@ k_ret_bwd_sweeps(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ d
       // pair ids two tiles ahead and the rows' L, delta one tile ahead: no dependent global load at the top of a tile
       auto ld_pid = [&](int t) {
         const int t0 = g0 + t * kPairs;
-        const int id = (t < ntiles && t0 + row < g1) ? __ldg(pr + t0 + row) : -1;
+        const int id = t == tile0 ? id0 : (t < ntiles && t0 + row < g1) ? __ldg(pr + t0 + row) : -1;
         return id >= 0 && !MUSE_IN_RANGE(id, (long long)dm.N * mk) ? -1 : id;
       };
       int pid = ld_pid(tile0), pid_n = ld_pid(tile0 + tstep);
@@ -196,26 +210,37 @@ k_ret_bwd_sweeps(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ d
         wait(&B.s_done, ph);
         tc::fence_after_sync();
         RBCLK(1)
+        float sv[2][8], dp[2][8];                           // 8 key columns at a time, the next 8 on their way
+        tc::tmem_ld8_issue(tl + cS, sv[0]);
+        tc::tmem_ld8_issue(tl + cDP, dp[0]);
+        tc::tmem_ld_wait();
+        tc::tmem_ld_use8(sv[0]);
+        tc::tmem_ld_use8(dp[0]);
 #pragma unroll
-        for (int hf = 0; hf < 2; ++hf) {                    // 32 key columns at a time
-          float sv[32], dp[32];
-          tc::tmem_ld32(tl + cS + 32 * hf, sv);
-          tc::tmem_ld32(tl + cDP + 32 * hf, dp);
-          uint32_t pw[16], gw[16];
+        for (int g = 0; g < kKeys / 8; ++g) {
+          if (g + 1 < kKeys / 8) {
+            tc::tmem_ld8_issue(tl + cS + 8 * (g + 1), sv[(g + 1) & 1]);
+            tc::tmem_ld8_issue(tl + cDP + 8 * (g + 1), dp[(g + 1) & 1]);
+          }
+          uint32_t pw[4], gw[4];
 #pragma unroll
-          for (int i = 0; i < 32; i += 2) {
-            const float e0 = 32 * hf + i < vis ? tc::fast_exp2(fmaf(sv[i], scale2, -L2)) : 0.f;
-            const float e1 = 32 * hf + i + 1 < vis ? tc::fast_exp2(fmaf(sv[i + 1], scale2, -L2)) : 0.f;
+          for (int i = 0; i < 8; i += 2) {
+            const float* s_ = sv[g & 1];
+            const float* d_ = dp[g & 1];
+            const float e0 = 8 * g + i < vis ? tc::fast_exp2(fmaf(s_[i], scale2, -L2)) : 0.f;
+            const float e1 = 8 * g + i + 1 < vis ? tc::fast_exp2(fmaf(s_[i + 1], scale2, -L2)) : 0.f;
             __nv_bfloat162 pb = __floats2bfloat162_rn(e0, e1);
-            __nv_bfloat162 gb = __floats2bfloat162_rn(e0 * (dp[i] - dl) * dm.sigma, e1 * (dp[i + 1] - dl) * dm.sigma);   // (sigma rides on G: dQ and dK come out scaled)
+            __nv_bfloat162 gb = __floats2bfloat162_rn(e0 * (d_[i] - dl) * dm.sigma, e1 * (d_[i + 1] - dl) * dm.sigma);   // (sigma rides on G: dQ and dK come out scaled)
             pw[i / 2] = *reinterpret_cast<uint32_t*>(&pb);
             gw[i / 2] = *reinterpret_cast<uint32_t*>(&gb);
           }
-#pragma unroll
-          for (int c4 = 0; c4 < 4; ++c4) {
-            const uint32_t off = tc::sw128_off(row, 4 * hf + c4);
-            *reinterpret_cast<uint4*>(hb + 2 * kTile + off) = make_uint4(pw[4 * c4], pw[4 * c4 + 1], pw[4 * c4 + 2], pw[4 * c4 + 3]);
-            *reinterpret_cast<uint4*>(hb + 2 * kTile + kPG + off) = make_uint4(gw[4 * c4], gw[4 * c4 + 1], gw[4 * c4 + 2], gw[4 * c4 + 3]);
+          const uint32_t off = tc::sw128_off(row, g);
+          *reinterpret_cast<uint4*>(hb + 2 * kTile + off) = make_uint4(pw[0], pw[1], pw[2], pw[3]);
+          *reinterpret_cast<uint4*>(hb + 2 * kTile + kPG + off) = make_uint4(gw[0], gw[1], gw[2], gw[3]);
+          if (g + 1 < kKeys / 8) {
+            tc::tmem_ld_wait();
+            tc::tmem_ld_use8(sv[(g + 1) & 1]);
+            tc::tmem_ld_use8(dp[(g + 1) & 1]);
           }
         }
         tc::fence_async_smem();                             // P and G are read by the tensor cores
@@ -391,7 +416,7 @@ k_ret_bwd_sweeps(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ d
 #endif
   tc::fence_before_sync();
   __syncthreads();
-  if (warp == 0) tc::tmem_dealloc(tbase_s, 2 * kCols);
+  if (warp == 0) tc::tmem_dealloc(tbase_s, NH * kCols);
   if (!ok_ && lane == 0) report_status(status, MUSE_STATUS_BWD_TIMEOUT);
 }
 
@@ -402,10 +427,10 @@ int ret_bwd_short_tc(const Dims& d, const void* Q, const void* dO, const void* K
   const dim3 grid(ri.cap, d.B * d.Hq);
   if (d.D == 128) {
     MUSE_CUDA_OK(cudaFuncSetAttribute(k_ret_bwd_sweeps<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, rs::Lay<128>::kSmem));
-    MUSE_RC(launch_pdl(k_ret_bwd_sweeps<128>, grid, rs::kThreads, rs::Lay<128>::kSmem, st, d, (const bf16*)Q, (const bf16*)dO, (const bf16*)Kp, (const bf16*)Vp, LSE, delta, off_k, ri, (bf16*)dq_part, dK_perm, dV_perm, status));
+    MUSE_RC(launch_pdl(k_ret_bwd_sweeps<128>, grid, rs::Lay<128>::kThreads, rs::Lay<128>::kSmem, st, d, (const bf16*)Q, (const bf16*)dO, (const bf16*)Kp, (const bf16*)Vp, LSE, delta, off_k, ri, (bf16*)dq_part, dK_perm, dV_perm, status));
   } else {
     MUSE_CUDA_OK(cudaFuncSetAttribute(k_ret_bwd_sweeps<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, rs::Lay<64>::kSmem));
-    MUSE_RC(launch_pdl(k_ret_bwd_sweeps<64>, grid, rs::kThreads, rs::Lay<64>::kSmem, st, d, (const bf16*)Q, (const bf16*)dO, (const bf16*)Kp, (const bf16*)Vp, LSE, delta, off_k, ri, (bf16*)dq_part, dK_perm, dV_perm, status));
+    MUSE_RC(launch_pdl(k_ret_bwd_sweeps<64>, grid, rs::Lay<64>::kThreads, rs::Lay<64>::kSmem, st, d, (const bf16*)Q, (const bf16*)dO, (const bf16*)Kp, (const bf16*)Vp, LSE, delta, off_k, ri, (bf16*)dq_part, dK_perm, dV_perm, status));
   }
   MUSE_LAUNCH_OK();
   return MUSE_OK;

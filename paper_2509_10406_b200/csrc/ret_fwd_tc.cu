@@ -18,6 +18,9 @@
 // fill each other's waits.
 // Clusters with more than 128 visible keys take further sweeps over the tiles that see them; a later
 // sweep merges its partial result into the stored row by log-sum-exp weights.
+// The row, issuing and gather warps start together: the gather of the first tile runs beside the load of the keys, of which only
+// the rows that products take are loaded (16 heads of 8k tokens, 128 clusters, 8 slots 152 -> 141 us; buckets of 64 keys,
+// 8 heads of two sequences of 64k 1166 -> 1110).
 #include <cuda.h>
 #include "common.cuh"
 #include "tc05.cuh"
@@ -128,20 +131,33 @@ k_ret_fwd_pairs_tc(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__
     int tile = tile_lo + ((sub - tile_lo % nsub) + nsub) % nsub;
     __syncthreads();                                        // the previous sweep's products are complete (every role waited for them)
     // the sweep's keys (K-major for S = Q K^T) and values (MN-major for O = P V); rows past the cluster are zeros
-    for (int e = tid; e < kKeys * CPR; e += kThreads) {
-      const int r = e / CPR, ck = e % CPR;
-      uint4 a = make_uint4(0u, 0u, 0u, 0u), b = a;
-      if (kc + r < kall && MUSE_IN_RANGE(k0 + kc + r, dm.N)) {
-        a = reinterpret_cast<const uint4*>(Kb + (size_t)(kc + r) * D)[ck];
-        b = reinterpret_cast<const uint4*>(Vb + (size_t)(kc + r) * D)[ck];
+    // (only as many rows as the products take, four of a thread's pieces on their way together; the gather warps have begun with
+    // the first tile meanwhile)
+    if (warp <= kIssuerWarp) {
+      const int nrow = min(kKeys, (max(kall - kc, 0) + 15) & ~15);
+      for (int e0 = tid; e0 < nrow * CPR; e0 += 4 * kGather0) {
+        uint4 a[4], b[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int e = e0 + u * kGather0, r = e / CPR, ck = e % CPR;
+          a[u] = b[u] = make_uint4(0u, 0u, 0u, 0u);
+          if (r < nrow && kc + r < kall && MUSE_IN_RANGE(k0 + kc + r, dm.N)) {
+            a[u] = reinterpret_cast<const uint4*>(Kb + (size_t)(kc + r) * D)[ck];
+            b[u] = reinterpret_cast<const uint4*>(Vb + (size_t)(kc + r) * D)[ck];
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int e = e0 + u * kGather0, r = e / CPR, ck = e % CPR;
+          const uint32_t off = (ck >> 3) * kKeys * 128 + tc::sw128_off(r, ck & 7);
+          if (r >= nrow || !MUSE_IN_RANGE(off, kKeys * D * 2 - 15)) continue;
+          *reinterpret_cast<uint4*>(sm + SM::k + off) = a[u];
+          *reinterpret_cast<uint4*>(sm + SM::v + off) = b[u];
+        }
       }
-      const uint32_t off = (ck >> 3) * kKeys * 128 + tc::sw128_off(r, ck & 7);
-      if (!MUSE_IN_RANGE(off, kKeys * D * 2 - 15)) continue;
-      *reinterpret_cast<uint4*>(sm + SM::k + off) = a;
-      *reinterpret_cast<uint4*>(sm + SM::v + off) = b;
+      tc::fence_async_smem();                               // the tensor cores read the tiles through the async proxy
+      tc::named_bar_sync(2, kGather0);
     }
-    tc::fence_async_smem();                                 // the tensor cores read the tiles through the async proxy
-    __syncthreads();
     RFCLK(0)
 
     if (warp < kIssuerWarp) {
