@@ -634,14 +634,20 @@ int ret_bwd_short_tc(const Dims& d, const void* Q, const void* dO, const void* K
 
 // Two kernels, or one with five products per tile?  The fused kernel gathers a pair's rows once per 64 keys and reads back the stored
 // dQ row from the second time on; the two kernels gather it once more than they have to, and start twice as many CTAs.  So by the
-// mean keys and the mean pairs of a cluster.  Measured, fused | dK, dV + dQ, us:
-//   D = 64, 512 keys, 4096 pairs 16860 | 5410 + 3610;  256 keys, 2048 pairs 1331 | 543 + 501;  64 keys, 1024 pairs 2082 | 998 + 881;
-//           64 keys, 512 pairs 374 | 211 + 198;  32 keys, 256 pairs 364 | 217 + 209
-//   D = 128, 256 keys, 2048 pairs 1875 | 802 + 514;  128 keys, 1024 pairs 684 | 353 + 261;  64 keys, 2048 pairs 2754 | 1350 + 1340
+// mean keys of a cluster, and where that leaves it open by its mean pairs.  Measured, fused | dK, dV + dQ, us (16 heads of 16k tokens):
+//   D = 64:  256 keys, 1024 pairs 963 | 836;  164 keys, 655 pairs 674 | 645;  128 keys, 512 pairs 519 | 571, 1024 pairs 822 | 809,
+//            2048 pairs 1424 | 1289;  109 keys, 437 pairs 464 | 537, 1747 pairs 1219 | 1184;  96 keys, 1542 pairs 1053 | 1113;
+//            64 keys, 1024 pairs 834 | 1095, 2048 pairs 1382 | 1851
+//   D = 128: 128 keys, 512 pairs 1176 | 893;  96 keys, 386 pairs 926 | 787;  82 keys, 328 pairs 773 | 710, 1311 pairs 1754 | 1702;
+//            64 keys, 1024 pairs 1433 | 1598, 2048 pairs 2448 | 2836
+static bool ret_bwd_fused(const Dims& d) {
+  const int keys = d.N / d.Ck;
+  return d.D == 128 ? keys < 80 : keys < 100 || (keys < 160 && (long long)d.N * d.m < 1024LL * d.Ck);
+}
 int ret_bwd_pairs_tc(const Dims& d, const void* Q, const void* dO, const void* Kp, const void* Vp, const float* LSE,
                      const float* delta, const int32_t* off_k, const RetIndex& ri, void* dq_part,
                      float* dK_perm, float* dV_perm, int* status, cudaStream_t st) {
-  if (d.N / d.Ck < (d.D == 128 ? 128 : 256) && (long long)d.N * d.m < 1024LL * d.Ck)
+  if (ret_bwd_fused(d))
     return ret_bwd_short_tc(d, Q, dO, Kp, Vp, LSE, delta, off_k, ri, dq_part, dK_perm, dV_perm, status, st);
   return d.D == 128 ? ret_bwd_d<128>(d, Q, dO, Kp, Vp, LSE, delta, off_k, ri, dq_part, dK_perm, dV_perm, status, st)
                     : ret_bwd_d<64>(d, Q, dO, Kp, Vp, LSE, delta, off_k, ri, dq_part, dK_perm, dV_perm, status, st);

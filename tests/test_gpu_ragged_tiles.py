@@ -50,12 +50,13 @@ def test_streaming_both_sides_at_once_equals_each_side_alone(Hq, Hkv, D, Cq, Ck,
         assert size.sum() == N // S and size.max() <= max(1, int(np.ceil(cap * (N // S) / C)))
 
 
-@pytest.mark.parametrize("base,Ck,two_kernels", [("d64", 7, True), ("d64", 8, False), ("d64", 2, True), ("d128", 15, True), ("d128", 16, False),
-                                                 ("d128", 3, True)])
-def test_retrieval_on_both_sides_of_the_cluster_length_rule(base, Ck, two_kernels):
-    """2040 keys: clusters of 255 (D = 64) or 127 keys (D = 128) and shorter take the fused kernel (and, before it, the forward
-    kernel with resident keys)."""
-    w = CASES[base].with_(Hq=2, Hkv=1, N=2040, S=4, Cq=9, Ck=Ck, m=min(Ck, 3), components=64)
+@pytest.mark.parametrize("base,Ck,m,two_kernels", [("d64", 7, 3, True), ("d64", 8, 3, True), ("d64", 2, 2, True), ("d64", 12, 3, True),
+                                                   ("d64", 13, 3, False), ("d64", 20, 11, True), ("d64", 21, 11, False), ("d128", 15, 3, True),
+                                                   ("d128", 16, 3, True), ("d128", 25, 3, True), ("d128", 26, 3, False)])
+def test_retrieval_on_both_sides_of_the_cluster_length_rule(base, Ck, m, two_kernels):
+    """2040 keys: below 80 (D = 128) or 100 keys a cluster, or 160 with few pairs, the fused backward kernel; below 128 or 256 the forward
+    kernel with resident keys."""
+    w = CASES[base].with_(Hq=2, Hkv=1, N=2040, S=4, Cq=9, Ck=Ck, m=m, components=64)
     with kernels_launched() as rec:
         _backward_parity_run(w, 128.0)
     assert "k_ret_bwd_pairs_tc" in rec.names and ("k_ret_bwd_dq" in rec.names) == two_kernels
