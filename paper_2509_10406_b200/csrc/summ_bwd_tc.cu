@@ -47,7 +47,9 @@ constexpr int kOkCache = 72;                   // bucket offsets of the cluster 
 // 2-D tensor map over a bf16 matrix with an arbitrary row pitch (bytes), 128B swizzle, box [box_rows][64]
 int make_tmap_bf16_pitched(void* out_map, const void* base, uint64_t rows, uint64_t cols, uint64_t pitch_bytes, uint32_t box_rows);
 
-template <int D>
+// WIDE: more than 32 planes, so that which of them are live is looked up 32 at a time (one instance for both, deciding at run
+// time, spilled 28 bytes at D = 64).
+template <int D, bool WIDE>
 __global__ void __launch_bounds__(sb::THREADS, D == 64 ? 2 : 1)
 k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_constant__ CUtensorMap tm_dnu,
               const __grid_constant__ CUtensorMap tm_K, const __grid_constant__ CUtensorMap tm_V,
@@ -94,7 +96,7 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
   __syncthreads();
   tc::fence_after_sync();
   pdl_trigger();                                           // (tensor memory has been allocated)
-  uint32_t livemask = 0u;
+  uint32_t livemask = 0u;                                  // of the 32 planes around the current one: bit pl & 31
   const uint32_t tbase = tbase_s, tlane = tbase + ((uint32_t)((warp & 3) * 32) << 16);
   uint32_t ph_g = 0, ph_kv = 0, ph_q = 0, ph_l = 0, ph1 = 0, ph2 = 0;
   bool ok = true;
@@ -150,22 +152,24 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
         }
         if (pl0 < pl_end) issue_grad(pl0, 0);
       }
-      // which planes hold a non-empty segment of query cluster i (others were never written by the far-field pass); the same for
-      // every chunk of keys
-      if (cw && (c0 == kbeg || dm.Cq > TI)) {
+      // which planes hold a non-empty segment of query cluster i (others were never written by the far-field pass), 32 planes at
+      // a time; up to 32 planes it is the same for every chunk of keys
+      auto look_up = [&](int first) {                     // the planes from `first`, a multiple of 32
         livemask = 0u;
+        const int n = WIDE ? min(32, dm.SB - first) : dm.SB;
 #pragma unroll 4
-        for (int pl = 0; pl < dm.SB; ++pl) {
-          const int32_t* o = oq + (size_t)(dm.causal ? pl + 1 : 0) * dm.Cq + ic;
+        for (int e = 0; e < n; ++e) {
+          const int32_t* o = oq + (size_t)(dm.causal ? first + e + 1 : 0) * dm.Cq + ic;
           // (per-block gradients are zero-filled before they are accumulated: every plane's rows are valid)
-          livemask |= in_range && (per_block || o[1] > o[0]) ? 1u << pl : 0u;
+          livemask |= in_range && (per_block || o[1] > o[0]) ? 1u << e : 0u;
         }
-      }
+      };
+      if (cw && (c0 == kbeg || dm.Cq > TI || WIDE)) look_up(WIDE ? pl0 & ~31 : 0);
       // per-plane scalars, loaded one plane ahead
       auto ent_of = [&](int pl) { return (((size_t)pq * dm.SB + pl) * dm.Cq + ic) * dm.Ck + j; };        // summaries: [plane][i][j]
       auto gent_of = [&](int pl) { return (((size_t)pq * dm.SB + pl) * dm.Ck + j) * dm.Cq + ic; };      // gradients: [plane][j][i]
       float mu_n = 0.f, dS_n = 0.f;
-      if (pl0 < pl_end && ((livemask >> pl0) & 1u)) { mu_n = mu[ent_of(pl0)]; dS_n = dS[gent_of(pl0)]; }
+      if (pl0 < pl_end && ((livemask >> (pl0 & 31)) & 1u)) { mu_n = mu[ent_of(pl0)]; dS_n = dS[gent_of(pl0)]; }
       // tilt logits l_iu = sigma qbar_i . k_u, the same for every plane: once per centroid tile
       if (warp == ISSUER / 32) {
         if (D == 64 && i0 == 0 && !tc::mbar_wait(&bar_kv, ph_kv)) ok = false;
@@ -197,11 +201,12 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
         const int buf = k & 1;
         const int nk = min(NU, ok_[pl + 1] - c0);
         const int klo = per_block ? max(0, ok_[pl] - c0) : 0;      // first key of the chunk that this plane weighs
-        const bool live = (livemask >> pl) & 1u;
+        const bool live = (livemask >> (pl & 31)) & 1u;
         const float mu_i = mu_n * 1.4426950408889634f, dS_i = dS_n;
         const int oDka = buf ? oQlo : oDka0, oDnu = buf ? oDnu1 : oDnu0;
         const uint32_t aDka = tc::smem_u32(sm + oDka), aDnu = tc::smem_u32(sm + oDnu);
-        if (pl + 1 < pl_end && ((livemask >> (pl + 1)) & 1u)) { mu_n = mu[ent_of(pl + 1)]; dS_n = dS[gent_of(pl + 1)]; }
+        if (WIDE && cw && pl + 1 < pl_end && ((pl + 1) & 31) == 0) look_up(pl + 1);
+        if (pl + 1 < pl_end && ((livemask >> ((pl + 1) & 31)) & 1u)) { mu_n = mu[ent_of(pl + 1)]; dS_n = dS[gent_of(pl + 1)]; }
         // The far-field pass wrote every row of the gradient tensors (zeros for an empty segment), so the
         // tiles go to the tensor cores as they land.  The D-contractions of a plane do not depend on the
         // previous plane's i-contractions: they are issued before them if the tiles are there by then, and only the W
@@ -400,15 +405,12 @@ int summ_bwd_tc(const Dims& d, const void* Kp, const void* Vp, const int32_t* of
   if (rc == MUSE_OK) rc = make_tmap_bf16_rows(&tV, Vp, (uint64_t)d.B * d.Hkv * d.N, d.D, sb::NU);
   if (rc != MUSE_OK) return rc;
   prof_mark("k_summ_bwd_tc", st);
-  if (d.D == 128) {
-    MUSE_CUDA_OK(cudaFuncSetAttribute(k_summ_bwd_tc<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, sb::Lay<128>::total));
-    MUSE_RC(launch_pdl(k_summ_bwd_tc<128>, dim3(d.Ck, d.B * d.Hq), sb::THREADS, sb::Lay<128>::total, st, d, tdka, tdnu, tK, tV, tqh, tql, off_k, off_q, mu, dS, dK_perm, dV_perm, per_block, status));
-  } else {
-    MUSE_CUDA_OK(cudaFuncSetAttribute(k_summ_bwd_tc<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, sb::Lay<64>::total));
-    MUSE_RC(launch_pdl(k_summ_bwd_tc<64>, dim3(d.Ck, d.B * d.Hq), sb::THREADS, sb::Lay<64>::total, st, d, tdka, tdnu, tK, tV, tqh, tql, off_k, off_q, mu, dS, dK_perm, dV_perm, per_block, status));
-  }
-  MUSE_LAUNCH_OK();
-  return MUSE_OK;
+  auto launch = [&](auto kernel, int smem) {
+    return launch_pdl(kernel, dim3(d.Ck, d.B * d.Hq), sb::THREADS, smem, st, d, tdka, tdnu, tK, tV, tqh, tql, off_k, off_q, mu, dS, dK_perm, dV_perm, per_block, status);
+  };
+  const bool wide = d.SB > 32;
+  if (d.D == 128) return wide ? launch(k_summ_bwd_tc<128, true>, sb::Lay<128>::total) : launch(k_summ_bwd_tc<128, false>, sb::Lay<128>::total);
+  return wide ? launch(k_summ_bwd_tc<64, true>, sb::Lay<64>::total) : launch(k_summ_bwd_tc<64, false>, sb::Lay<64>::total);
 }
 
 }  // namespace muse
