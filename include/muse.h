@@ -35,6 +35,12 @@
  *     assignment outside [0, C) is treated as the nearest valid cluster index and a selection entry
  *     outside [0, Ck) as -1 (none); a row of Q or K that holds NaN or infinities is assigned to
  *     cluster 0.
+ *   - Q, K, V and dO are expected to be finite, padding included.  A masked entry has weight 0 and
+ *     0 * NaN is NaN, so a NaN or an infinity in K or V may also reach queries that do not attend to
+ *     its row: in the block-diagonal part those whose tile of 128 rows it shares (in the last tile of a
+ *     block that 128 does not divide, rows of the next block or head), in the summaries those of the
+ *     bucket up to 15 rows before it, in retrieval those of the same cluster.  Rows of other clusters
+ *     and other heads never enter retrieval.
  *   - Spatial blocks: block(t) = t / (N / n_blocks).  Keys are bucketed cluster-major,
  *     block-minor: bucket (j,b) occupies positions [off_k[j*S+b], off_k[j*S+b+1]) of the
  *     permutation perm_k (position -> original key index, stable, i.e. ascending inside a

@@ -9,6 +9,8 @@
 // gather warps bring the scattered Q and dO rows by 16-byte asynchronous copies.
 //   k_ret_bwd_dkdv   128 keys resident, tiles of 64 pairs gathered:  S^T = K Q^T, dP^T = V dO^T;  dV += P^T dO, dK += G^T Q
 //   k_ret_bwd_dq     128 pairs gathered (four buffers at D = 64, two at D = 128), tiles of 64 keys by TMA:  S = Q K^T, dP = dO V^T;  dQ += G K
+// A tile of streamed keys may reach past the cluster, into the keys of the next one or of the next head: those rows are zeroed before
+// they meet G, and G is 0 (not 0 times what the row gave) wherever a pair does not see the key.
 // A pair's rows are gathered once for dQ and once per 128 keys it sees for dK and dV, and its dQ row is written once.
 // (One kernel for all five products has to keep dK and dV of the keys at hand in tensor memory, so it takes 64 keys per
 // sweep: the rows were then gathered, and the stored dQ row read and rewritten, once per 64 keys.)
@@ -439,7 +441,7 @@ k_ret_bwd_dq(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_con
       const int T = (visible(pid >= 0 ? pid / gr.mk : -1) + kN - 1) / kN;
       pid = pid_n;
       for (int t = 0; t < T && ok_; ++t) {
-        const int row = gr.pk * dm.N + gr.k0 + t * kN;     // (rows past the cluster are other keys; they are masked)
+        const int row = gr.pk * dm.N + gr.k0 + t * kN;     // (rows past the cluster are other keys: see the products)
         wait(&bars.k_empty[sk], phk ^ 1);
         if (tc::elect_one()) {
           tc::mbar_expect_tx(&bars.k_full[sk], kCol);
@@ -479,6 +481,8 @@ k_ret_bwd_dq(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_con
       wait(&bars.k_full[sk1], phk1);
       wait(&bars.v_full[sv1], phv1);
       tc::fence_after_sync();
+      const int own = gr.kall - ka * kN;                   // the cluster's keys among the tile's
+      if (own < kN) tc::zero_rows<G, kN>(sm + LY::oK + sk1 * kCol, own, kN);
       const uint32_t c = tbase + (uint32_t)(n1 % NW) * 2 * kN;
       const uint64_t a = tc::desc_step(dq0, (uint32_t)(ia % NQ) * kRow), o = tc::desc_step(do0, (uint32_t)(ia % NQ) * kRow);
       const uint64_t x = tc::desc_step(dk0, (uint32_t)sk1 * kCol), y = tc::desc_step(dv0, (uint32_t)sv1 * kCol);
@@ -581,9 +585,8 @@ k_ret_bwd_dq(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_con
           if (q < 3) { tc::tmem_ld16_issue(ts + 16 * (q + 1), sn); tc::tmem_ld16_issue(ts + kN + 16 * (q + 1), dn_); }
 #pragma unroll
           for (int c = 0; c < 16; ++c) {
-            float p = tc::fast_exp2(fmaf(sv[c], scale2, -L2));
-            if (!full) p = 16 * q + c < v ? p : 0.f;
-            dp[c] = p * (dp[c] - dl);
+            dp[c] = tc::fast_exp2(fmaf(sv[c], scale2, -L2)) * (dp[c] - dl);
+            if (!full) dp[c] = 16 * q + c < v ? dp[c] : 0.f;
           }
           uint32_t gw[8];
 #pragma unroll

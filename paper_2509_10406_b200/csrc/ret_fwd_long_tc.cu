@@ -5,6 +5,8 @@
 //   S_q = Q_q K^T        Q rows gathered once per tile by 16-byte asynchronous copies, keys and values streamed by TMA
 //   P_q                  two threads per pair row at D = 64, one at D = 128; bf16 over the consumed logits in tensor memory
 //   O_q += P_q V         accumulated in tensor memory over the tile's keys, rescaled lazily
+// A key tile reaches past the keys that its pair tile sees, into those of later blocks, of the next cluster and of the next head: O += P V
+// takes only the 16-key groups that hold a visible key, and the rows past the cluster in the last of them are zeroed first.
 // The (pair tile, key tile) products, numbered n over all units, go through NB logit buffers; products are issued in the
 // order ... O += P(n) V, S(n + NB) = Q K ..., which the tensor core keeps, so S(n + NB) may overwrite P(n) and the tensor
 // cores need not wait at a unit's end.  A pair's partial row is written once.
@@ -145,7 +147,7 @@ k_ret_fwd_long(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_c
     for (int u = sub; u < nunits; u += nsub) {
       const int T = max(key_tiles(l0), key_tiles(l1));
       l0 = ld_last(2 * (u + nsub)); l1 = ld_last(2 * (u + nsub) + 1);
-      for (int t = 0; t < T; ++t) {                        // (rows past the keys that the tile sees are loaded too; they are masked)
+      for (int t = 0; t < T; ++t) {                        // (rows past the keys that the tile sees are loaded too)
         const int row = pk * dm.N + k0 + t * kKeys;
         wait(&bars.k_empty[s], ph ^ 1);
         if (ok_) load(sm + LY::oK + s * kTile, &tm_k, row, &bars.k_full[s]);
@@ -158,10 +160,11 @@ k_ret_fwd_long(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_c
     const uint32_t id_s = tc::idesc_bf16(kPairs, kKeys, 0, 0), id_o = tc::idesc_bf16(kPairs, D, 0, 1);
     const uint64_t dq = tc::smem_desc_sw128(tc::smem_u32(sm + LY::oQ), 16, 1024), dk = tc::smem_desc_sw128(tc::smem_u32(sm + LY::oK), 16, 1024),
                    dv = tc::smem_desc_sw128(tc::smem_u32(sm + LY::oV), kKeys * 128, 1024);
-    // a cursor over the sequence of products (unit, key tile t, pair tile q); T: key tiles of the unit's two pair tiles
-    struct Cur { int u, t, q, T0, T1, T, l0, l1, n, e0, e1, o; };
+    // a cursor over the sequence of products (unit, key tile t, pair tile q); V, T: keys and key tiles that the unit's two pair tiles see
+    struct Cur { int u, t, q, V0, V1, T0, T1, T, l0, l1, n, e0, e1, o; };
     auto enter = [&](Cur& c) {                             // the unit's numbers of key tiles; its successor's last pairs are on their way
-      c.T0 = key_tiles(c.l0); c.T1 = key_tiles(c.l1); c.T = max(c.T0, c.T1);
+      c.V0 = visible(c.l0); c.V1 = visible(c.l1);
+      c.T0 = (c.V0 + kKeys - 1) / kKeys; c.T1 = (c.V1 + kKeys - 1) / kKeys; c.T = max(c.T0, c.T1);
       c.l0 = ld_last(2 * (c.u + nsub)); c.l1 = ld_last(2 * (c.u + nsub) + 1);
       c.t = c.q = 0;
     };
@@ -203,16 +206,22 @@ k_ret_fwd_long(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_c
       while (cp.u < nunits && cp.t >= cp.T) { cp.u += nsub; if (cp.u < nunits) enter(cp); }
       if (cp.u >= nunits) break;
       const int q = cp.q;
-      if (q == 0) { wait(&bars.v_full[sv], phv); tc::fence_after_sync(); }
+      if (q == 0) {
+        wait(&bars.v_full[sv], phv);
+        tc::fence_after_sync();
+        const int own = item.nk - cp.t * kKeys;            // the cluster's keys among the tile's
+        if (own < kKeys && (own & 15) != 0) tc::zero_rows<G, kKeys>(sm + LY::oV + sv * kTile, own, (own + 15) & ~15);
+      }
       if (cp.t < (q == 0 ? cp.T0 : cp.T1)) {
         const int e = q == 0 ? cp.e0++ : cp.e1++;
         wait(&bars.p_ready[q][e & 1], (e >> 1) & 1);
         tc::fence_after_sync();
         const uint64_t b = tc::desc_step(dv, (uint32_t)sv * kTile);
         const uint32_t c = tbase + (uint32_t)(cp.n % NB) * kKeys;
+        const int groups = ((q == 0 ? cp.V0 : cp.V1) - cp.t * kKeys + 15) >> 4;          // of 16 keys, that hold one the tile sees
 #pragma unroll
         for (int ks = 0; ks < kKeys / 16; ++ks)
-          tc::mma_bf16_ts_warp(tbase + cO + q * D, c + 8 * ks, tc::desc_step(b, ks * 16 * 128), id_o, cp.t > 0 || ks > 0);
+          if (ks < groups) tc::mma_bf16_ts_warp(tbase + cO + q * D, c + 8 * ks, tc::desc_step(b, ks * 16 * 128), id_o, cp.t > 0 || ks > 0);
         tc::mma_commit_warp(&bars.pv_done[q]);
       }
       issue_s();

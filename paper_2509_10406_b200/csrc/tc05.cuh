@@ -326,6 +326,17 @@ __device__ __forceinline__ float fast_exp2(float x) {
 }
 
 // ---- swizzled shared-memory tiles ------------------------------------------------------------------------
+// Zeros the rows [r, end) of a swizzled tile of G column groups [ROWS][128 B] that TMA has filled; the whole warp, which then
+// issues the products that read them.  (What a box brought beside the rows that count must not meet a weight of 0: 0 * NaN is NaN.)
+template <int G, int ROWS> __device__ __forceinline__ void zero_rows(unsigned char* tile, int r, int end) {
+#pragma unroll
+  for (int g = 0; g < G; ++g)
+#pragma unroll 1
+    for (int o = r * 128 + (int)(threadIdx.x & 31) * 16; o < end * 128; o += 512) *reinterpret_cast<uint4*>(tile + g * ROWS * 128 + o) = make_uint4(0u, 0u, 0u, 0u);
+  fence_async_smem();                                      // the tensor cores read the tile through the async proxy
+  __syncwarp();
+}
+
 // Byte offset of the 16-byte chunk `c` (0..7) of row `r` inside a [rows][128 B] tile with the
 // 128-byte swizzle (tile base 1024-byte aligned).
 __device__ __forceinline__ uint32_t sw128_off(int r, int c) { return (uint32_t)(r * 128 + ((c ^ (r & 7)) << 4)); }
