@@ -168,8 +168,10 @@ MUSE_API int muse_cluster(const muse_params_t* p, const void* Q, const void* K,
  * allocation would stall every stream, plugins living under a framework whose pool already
  * owns the whole GPU, or hosts that must not fail with out-of-memory in mid-request.
  *   - Every GPU that loads the library carries the 32 MiB until the process exits.
- *   - Problems whose clustering scratch (muse_workspace_bytes out[0]) exceeds
- *     muse_cluster_noalloc_max_bytes() are rejected with MUSE_ERR_WORKSPACE; nothing is launched.
+ *   - Queries and keys are clustered side by side where the scratch of both (muse_workspace_bytes
+ *     out[0]) fits in muse_cluster_noalloc_max_bytes(), else one after the other.  A problem whose
+ *     queries or keys alone need more is rejected with MUSE_ERR_WORKSPACE.  All arguments are checked
+ *     first: a call that is refused launches nothing.
  *   - Every call looks up the array's device address for the current device.  The first lookup on
  *     a device loads the library's device image there, and that is when the driver reserves the
  *     32 MiB: this first call can therefore return MUSE_ERR_CUDA (no memory left for the image) and

@@ -87,6 +87,44 @@ int sm_count() {
   }
   return n;
 }
+
+int cluster_check(const muse_params_t* p, const void* Q, const void* K, const int32_t* init_q, const int32_t* init_k, int32_t* assign_q,
+                  int32_t* assign_k, float* qbar, float* kcent, size_t ws_bytes, bool may_split, ClusterCall* c) {
+  *c = ClusterCall{};
+  Dims& d = c->d;
+  const int rc = resolve(p, &d);
+  if (rc != MUSE_OK) return rc;
+  if (Q == nullptr && K == nullptr) return MUSE_ERR_INVALID_ARG;
+  if (ws_bytes < cluster_ws_bytes(d, Q != nullptr, K != nullptr)) {
+    c->split = may_split && Q != nullptr && K != nullptr && ws_bytes >= cluster_ws_bytes(d, true, false) && ws_bytes >= cluster_ws_bytes(d, false, true);
+    if (!c->split) return MUSE_ERR_WORKSPACE;
+  }
+  c->dtype = p->dtype; c->init_mode = p->init_mode; c->iters = p->kmeans_iters; c->seed = p->seed;
+  for (int kind = 0; kind < 2; ++kind) {
+    const void* X = kind == 0 ? Q : K;
+    if (X == nullptr) continue;
+    LloydSide& s = c->sides[c->n++];
+    s.X = X; s.kind = kind;
+    s.problems = d.B * (kind == 0 ? d.Hq : d.Hkv); s.C = kind == 0 ? d.Cq : d.Ck;
+    s.init_idx = kind == 0 ? init_q : init_k; s.assign = kind == 0 ? assign_q : assign_k; s.centres = kind == 0 ? qbar : kcent;
+    if (s.assign == nullptr || s.centres == nullptr || !aligned16(X) || !aligned16(s.centres)) return MUSE_ERR_INVALID_ARG;
+    if (p->init_mode == MUSE_INIT_INDICES && s.init_idx == nullptr) return MUSE_ERR_INVALID_ARG;
+  }
+  return MUSE_OK;
+}
+
+int cluster_launch(ClusterCall& c, void* ws, cudaStream_t st) {
+  const int per = c.split ? 1 : c.n;                       // sides of a launch
+  int rc = MUSE_OK;
+  for (int k = 0; k < c.n && rc == MUSE_OK; k += per) {
+    Arena ar(ws);
+    int* status = ar.take<int32_t>(kStatusWords);
+    for (int s = k; s < k + per; ++s) lloyd_side_ws(c.d, ar, c.sides[s]);
+    rc = lloyd(c.d, c.dtype, c.sides + k, per, c.init_mode, c.seed, c.iters, k == 0, status, st);       // (one clear for the call)
+  }
+  prof_mark(nullptr, st);
+  return rc;
+}
 }  // namespace muse
 
 #ifdef MUSE_DEBUG
@@ -207,30 +245,9 @@ int muse_cluster(const muse_params_t* p, const void* Q, const void* K, const int
   int rc = resolve(p, &d);
   if (rc != MUSE_OK) return rc;
   if (ws == nullptr || !aligned16(ws)) return MUSE_ERR_INVALID_ARG;
-  if (Q == nullptr && K == nullptr) return MUSE_ERR_INVALID_ARG;
-  if (ws_bytes < cluster_ws_bytes(d, Q != nullptr, K != nullptr)) return MUSE_ERR_WORKSPACE;
-  LloydSide sides[2] = {};
-  int n = 0;
-  if (Q != nullptr) {
-    if (assign_q == nullptr || qbar == nullptr || !aligned16(Q) || !aligned16(qbar)) return MUSE_ERR_INVALID_ARG;
-    if (p->init_mode == MUSE_INIT_INDICES && init_q == nullptr) return MUSE_ERR_INVALID_ARG;
-    sides[n].X = Q; sides[n].problems = d.B * d.Hq; sides[n].C = d.Cq; sides[n].kind = 0;
-    sides[n].init_idx = init_q; sides[n].assign = assign_q; sides[n].centres = qbar;
-    ++n;
-  }
-  if (K != nullptr) {
-    if (assign_k == nullptr || kcent == nullptr || !aligned16(K) || !aligned16(kcent)) return MUSE_ERR_INVALID_ARG;
-    if (p->init_mode == MUSE_INIT_INDICES && init_k == nullptr) return MUSE_ERR_INVALID_ARG;
-    sides[n].X = K; sides[n].problems = d.B * d.Hkv; sides[n].C = d.Ck; sides[n].kind = 1;
-    sides[n].init_idx = init_k; sides[n].assign = assign_k; sides[n].centres = kcent;
-    ++n;
-  }
-  Arena ar(ws);
-  int* status = ar.take<int32_t>(kStatusWords);
-  for (int k = 0; k < n; ++k) lloyd_side_ws(d, ar, sides[k]);
-  rc = lloyd(d, p->dtype, sides, n, p->init_mode, p->seed, p->kmeans_iters, status, stream);
-  prof_mark(nullptr, stream);
-  return rc;
+  ClusterCall c;
+  rc = cluster_check(p, Q, K, init_q, init_k, assign_q, assign_k, qbar, kcent, ws_bytes, false, &c);
+  return rc == MUSE_OK ? cluster_launch(c, ws, stream) : rc;
 }
 
 static size_t up256(size_t x) { return (x + 255) & ~size_t(255); }

@@ -267,11 +267,11 @@ k_update(const __grid_constant__ LloydSides g) {
 }
 
 template <class T, int D>
-static int lloyd_t(LloydSides& g, const Dims& d, int nsides, int init_mode, uint64_t seed, int T_iters, int* status, cudaStream_t st) {
+static int lloyd_t(LloydSides& g, const Dims& d, int nsides, int init_mode, uint64_t seed, int T_iters, bool fresh, int* status, cudaStream_t st) {
   // the status words are cleared by the first kernel of the call (k-means++ reports into them, so before it by a memset)
-  int32_t* clear = status;
+  int32_t* clear = fresh ? status : nullptr;
   if (init_mode == MUSE_INIT_KMEANSPP) {
-    MUSE_CUDA_OK(cudaMemsetAsync(status, 0, kStatusWords * sizeof(int32_t), st));
+    if (fresh) MUSE_CUDA_OK(cudaMemsetAsync(status, 0, kStatusWords * sizeof(int32_t), st));
     clear = nullptr;
     // the draws borrow two arrays that the iterations only fill later: perm as the running minimum distance
     // [problems, N] fp32, off (at least C + 1 words per problem) as the drawn indices [problems, C]
@@ -333,14 +333,15 @@ size_t lloyd_ws_bytes(const Dims& d, int problems, int C) {
   return ar.used;
 }
 
-int lloyd(const Dims& d, int dtype, LloydSide* sides, int nsides, int init_mode, uint64_t seed, int T, int* status, cudaStream_t st) {
+int lloyd(const Dims& d, int dtype, LloydSide* sides, int nsides, int init_mode, uint64_t seed, int T, bool clear, int* status, cudaStream_t st) {
   LloydSides g = {};
   for (int k = 0; k < nsides; ++k) g.s[k] = sides[k];
   g.N = d.N; g.S = d.S;
   if (dtype == MUSE_F32)
-    return d.D == 64 ? lloyd_t<float, 64>(g, d, nsides, init_mode, seed, T, status, st) : lloyd_t<float, 128>(g, d, nsides, init_mode, seed, T, status, st);
-  return d.D == 64 ? lloyd_t<__nv_bfloat16, 64>(g, d, nsides, init_mode, seed, T, status, st)
-                   : lloyd_t<__nv_bfloat16, 128>(g, d, nsides, init_mode, seed, T, status, st);
+    return d.D == 64 ? lloyd_t<float, 64>(g, d, nsides, init_mode, seed, T, clear, status, st)
+                     : lloyd_t<float, 128>(g, d, nsides, init_mode, seed, T, clear, status, st);
+  return d.D == 64 ? lloyd_t<__nv_bfloat16, 64>(g, d, nsides, init_mode, seed, T, clear, status, st)
+                   : lloyd_t<__nv_bfloat16, 128>(g, d, nsides, init_mode, seed, T, clear, status, st);
 }
 
 }  // namespace muse

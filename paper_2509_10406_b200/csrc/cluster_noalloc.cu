@@ -26,14 +26,6 @@ int scratch_address(void** out) {
   return MUSE_OK;
 }
 
-// scratch of one side alone (an upper bound: the dimensions are checked by muse_workspace_bytes before)
-size_t side_bytes(const muse_params_t* p, bool queries) {
-  muse::Dims d = {};
-  d.N = p->N; d.D = p->D; d.S = p->causal ? (p->n_blocks == 0 ? 8 : p->n_blocks) : 1;
-  return muse::kStatusWords * sizeof(int32_t) +
-         (queries ? muse::lloyd_ws_bytes(d, p->B * p->Hq, p->Cq) : muse::lloyd_ws_bytes(d, p->B * p->Hkv, p->Ck));
-}
-
 }  // namespace
 
 extern "C" {
@@ -43,27 +35,16 @@ size_t muse_cluster_noalloc_max_bytes(void) { return kStaticScratchBytes; }
 int muse_cluster_noalloc(const muse_params_t* p, const void* Q, const void* K, const int32_t* init_q,
                          const int32_t* init_k, int32_t* assign_q, int32_t* assign_k, float* qbar, float* kcent,
                          cudaStream_t stream) {
-  size_t need[6];
-  int rc = muse_workspace_bytes(p, need);
+  // Every check first: a call that is refused launches nothing.  Both sides at once when their scratch fits together, else one after
+  // the other.
+  muse::ClusterCall c;
+  int rc = muse::cluster_check(p, Q, K, init_q, init_k, assign_q, assign_k, qbar, kcent, kStaticScratchBytes, true, &c);
   if (rc != MUSE_OK) return rc;
-  // Both sides at once when their scratch fits together, else one after the other; a side whose own scratch is larger
-  // than the built-in array is what makes a problem too large.
-  const bool together = need[0] <= kStaticScratchBytes;
-  if (!together) {
-    if (Q == nullptr || K == nullptr) {
-      if (side_bytes(p, Q != nullptr) > kStaticScratchBytes) return MUSE_ERR_WORKSPACE;
-    } else if (side_bytes(p, true) > kStaticScratchBytes || side_bytes(p, false) > kStaticScratchBytes) return MUSE_ERR_WORKSPACE;
-  }
   void* ws = nullptr;
   rc = scratch_address(&ws);
-  if (rc != MUSE_OK) return rc;
   // Same launches as muse_cluster, on the built-in scratch.  Nothing needs pre-clearing beyond what the stage already
   // clears itself (its status words; every other array is fully written before it is read).
-  if (together || Q == nullptr || K == nullptr)
-    return muse_cluster(p, Q, K, init_q, init_k, assign_q, assign_k, qbar, kcent, ws, kStaticScratchBytes, stream);
-  rc = muse_cluster(p, Q, nullptr, init_q, nullptr, assign_q, nullptr, qbar, nullptr, ws, kStaticScratchBytes, stream);
-  if (rc != MUSE_OK) return rc;
-  return muse_cluster(p, nullptr, K, nullptr, init_k, nullptr, assign_k, nullptr, kcent, ws, kStaticScratchBytes, stream);
+  return rc == MUSE_OK ? muse::cluster_launch(c, ws, stream) : rc;
 }
 
 // The status word of the last muse_cluster_noalloc call lives inside the built-in array, where the

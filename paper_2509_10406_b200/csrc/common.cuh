@@ -232,7 +232,14 @@ struct LloydSide {
   float* cnorm; int32_t* off; int32_t* perm; void* chi; void* clo;
 };
 void lloyd_side_ws(const Dims& d, Arena& ar, LloydSide& s);
-int lloyd(const Dims& d, int dtype, LloydSide* sides, int nsides, int init_mode, uint64_t seed, int T, int* status, cudaStream_t st);
+// clear: the first kernel of the call is among these, which clear the status words
+int lloyd(const Dims& d, int dtype, LloydSide* sides, int nsides, int init_mode, uint64_t seed, int T, bool clear, int* status, cudaStream_t st);
+// muse_cluster in two steps (api.cu): every check of its arguments, then its launches.  may_split: where the scratch does not hold both
+// sides, take them one after the other if it holds each.
+struct ClusterCall { Dims d; LloydSide sides[2]; int n, dtype, init_mode, iters; bool split; uint64_t seed; };
+int cluster_check(const muse_params_t* p, const void* Q, const void* K, const int32_t* init_q, const int32_t* init_k, int32_t* assign_q,
+                  int32_t* assign_k, float* qbar, float* kcent, size_t ws_bytes, bool may_split, ClusterCall* c);
+int cluster_launch(ClusterCall& c, void* ws, cudaStream_t st);
 size_t lloyd_ws_bytes(const Dims& d, int problems, int C);      // scratch of one side (without the status words)
 int assign_tc(const LloydSide* sides, int nsides, int N, int D, int distances, int* status, cudaStream_t st);
 int assign_distances(const Dims& d, int dtype, const LloydSide& side, int* status, cudaStream_t st);   // after lloyd on the same centres
