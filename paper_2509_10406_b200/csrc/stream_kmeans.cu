@@ -732,7 +732,8 @@ int balanced_assign(const Dims& d, int dtype, const BalancedSide* sides, int n, 
   }
   const BalancedWs w = balanced_ws(d, ar, s, n);
   // step 1: nearest centroid of every vector (the Lloyd path's final assignment against given centres)
-  MUSE_RC(lloyd(d, dtype, s, n, MUSE_INIT_CENTRES, 0, 0, true, w.status, st));
+  // (the entry points have cleared the status words; what the streaming pass reported there stays)
+  MUSE_RC(lloyd(d, dtype, s, n, MUSE_INIT_CENTRES, 0, 0, false, w.status, st));
   // the sides whose cap can bind; for the others the nearest centroid is the answer
   SortSide sort[2];
   RankArgs r = {};

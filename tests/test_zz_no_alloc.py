@@ -137,3 +137,21 @@ def test_noalloc_clears_the_status_words_once_per_call():
         call()
         torch.cuda.synchronize()
         assert _status_clears(call) == (2, 1)
+
+
+@pytest.mark.gpu
+def test_streaming_and_lloyd_clear_the_status_words_once_per_call():
+    from paper_2509_10406_b200 import binding as mb
+    p = mb.make_params(B=1, Hq=2, Hkv=2, N=2048, D=64, Cq=24, Ck=40, m=0, seed=1)
+    Q, K = (torch.randn(1, 2, 2048, 64, device="cuda", dtype=torch.bfloat16) for _ in range(2))
+    buf = mb.MuseBuffers(p, backward=False)
+    ws = torch.empty(mb.muse_stream_workspace_bytes(p), dtype=torch.uint8, device="cuda")
+    call = lambda: mb.muse_cluster_streaming(p, Q, K, buf.assign_q, buf.assign_k, buf.qbar, buf.kcent, ws)  # noqa: E731
+    call()
+    torch.cuda.synchronize()
+    assert _status_clears(call) == (1, 1)
+    call = lambda: mb.muse_cluster(p, Q, K, buf.sel, buf.sel, buf.assign_q, buf.assign_k, buf.qbar, buf.kcent, buf.ws)  # noqa: E731
+    p.init_mode = 1
+    call()
+    torch.cuda.synchronize()
+    assert _status_clears(call) == (1, 1)
