@@ -163,6 +163,25 @@ inline int launch_pdl_cluster(void (*kernel)(KA...), dim3 grid, int threads, siz
   if (cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...) != cudaSuccess) { cudaGetLastError(); return MUSE_ERR_CUDA; }
   return MUSE_OK;
 }
+// Can the current device hold one thread-block cluster of this size (which a size above 8 has to be allowed for first)?
+template <class... KA>
+inline bool cluster_fits(void (*kernel)(KA...), int threads, size_t smem, int cluster) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = cluster; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  cfg.gridDim = dim3(cluster);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  int n = 0;
+  const bool ok = (cluster <= 8 || cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) &&
+                  (smem <= 48 * 1024 || cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess) &&
+                  cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess;
+  if (!ok) cudaGetLastError();                             // (a size that the device does not know is an answer, not an error)
+  return ok && n > 0;
+}
 template <class... KA, class... A>
 inline int launch_pdl(void (*kernel)(KA...), dim3 grid, int threads, size_t smem, cudaStream_t st, A&&... args) {
   return launch_pdl_cluster(kernel, grid, threads, smem, 1, st, std::forward<A>(args)...);

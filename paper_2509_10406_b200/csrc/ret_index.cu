@@ -174,7 +174,8 @@ int build_ret_index(const Dims& d, const int32_t* sel, const int32_t* bsel, cons
   while (cl < kRiMaxCluster && cl * pq < sm_count() / 2 && (long long)d.N * d.m >= 2LL * cl * kRiMinPairs) cl *= 2;
   const size_t smem = (size_t)nkeys * sizeof(int32_t);
   const RiArgs g = {sel, bsel, off_k, *out, nkeys};
-  if (cl > 8) MUSE_CUDA_OK(cudaFuncSetAttribute(k_ret_index, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  // More than 8 CTAs are not promised by every device: they have to share a processor group, each with up to 128 KB of shared memory.
+  if (cl > 8 && !cluster_fits(k_ret_index, kRiThreads, smem, cl)) cl = 8;
   prof_mark("k_ret_index", st);
   return launch_pdl_cluster(k_ret_index, dim3(pq * cl), kRiThreads, smem, cl, st, d, g);
 }

@@ -42,3 +42,10 @@ def test_forward_and_backward_of_many_blocks(base, Cq, Ck, m, S):
                 dV=rel_err(to_np(buf.dV)[:, :, :late], e[2][:, :, :late]))
     print(base, S, errs)
     assert all(v <= tol(w.dtype) for v in errs.values()), errs
+
+
+@pytest.mark.parametrize("base,N,Ck,m,S", [("d64", 8192, 1024, 4, 32), ("d64", 8192, 4096, 8, 8)])
+def test_retrieval_index_with_the_most_buckets(base, N, Ck, m, S):
+    """One head whose index takes the largest thread-block cluster (16 CTAs where the device holds them) at 124 and 112 KB a CTA."""
+    w = CASES[base].with_(Hq=1, Hkv=1, N=N, S=S, Cq=4, Ck=Ck, m=m, components=64)
+    _forward_parity(w, 128.0, expect_kernels={"k_ret_index"})
