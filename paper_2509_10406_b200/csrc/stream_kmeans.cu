@@ -570,7 +570,7 @@ static int stream_kmeans_ffma(const Dims& d, const StreamSide& s, uint64_t seed,
   const size_t smem = stream_smem_bytes<D>(s.C);
   // CTAs per problem: enough that a CTA owns at most two chunks of 64 centroids, as long as the GPU has room for them
   int cs = 1;
-  while (cs < kSkMaxCluster && s.C > 2 * kSkChunk * cs && (long long)s.problems * cs * 2 <= 2 * 148) cs *= 2;
+  while (cs < kSkMaxCluster && s.C > 2 * kSkChunk * cs && (long long)s.problems * cs * 2 <= 2 * sm_count()) cs *= 2;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
