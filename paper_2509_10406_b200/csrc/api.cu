@@ -376,7 +376,7 @@ int muse_summarize(const muse_params_t* p, const void* K, const void* V, const i
   size_t need[6];
   muse_workspace_bytes(p, need);
   if (ws_bytes < need[1]) return MUSE_ERR_WORKSPACE;
-  if (assign_k == nullptr && clear_status(ws, stream) != MUSE_OK) return MUSE_ERR_CUDA;     // (else by the sort, the first kernel)
+  // (the sort, the first kernel, clears the status words)
   rc = summarize(d, p->dtype, K, V, assign_k, qbar, off_k, perm_k, counts, ksum, vsum, summaries, ws, nullptr, stream);
   prof_mark(nullptr, stream);
   return rc;

@@ -1,5 +1,6 @@
-// Exact-attention backward on the Blackwell tensor cores (bf16 inputs, fp32 accumulation in
-// tensor memory), for the local block-diagonal component and the retrieved-cluster component.
+// A second implementation of the retrieval backward (bf16 inputs, fp32 accumulation in tensor memory), which shares no kernel code
+// with ret_bwd_tc.cu and ret_bwd_short_tc.cu: the tests hold both to the same oracle.  It runs only where the test hook asks for it
+// (muse_test_force_paths, bit 16); the dispatch of the retrieval backward is at the end.
 // With L the merged log-sum-exp and delta = dO.O (Appendix "Centroid Gradient Flow" fixes what
 // is constant):  P = exp(sigma q.k - L),  G = P (dO.v - delta),
 //                dV = P^T dO,  dK = sigma G^T Q,  dQ = sigma G K.
@@ -62,9 +63,6 @@ template <int ROWS> __device__ __forceinline__ uint64_t desc_mn(uint32_t base, i
 }
 
 struct BwdCtx {
-#ifdef MUSE_PHASE_CLOCKS
-  long long pc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-#endif
   unsigned char* sm;
   uint64_t* bar;
   uint32_t tbase, ph0, ph1;
@@ -86,19 +84,6 @@ __device__ __forceinline__ void bwd_teardown(BwdCtx& c, uint32_t cols, int tid, 
   __syncthreads();
   if ((tid >> 5) == 0) tc::tmem_dealloc(c.tbase, cols);
   if (!c.ok && tid == 0) report_status(status, 2);
-}
-
-__device__ __forceinline__ void store_row64(unsigned char* tile, int row, const float (&x)[kBN]) {
-#pragma unroll
-  for (int ch = 0; ch < kBN / 8; ++ch) {
-    uint32_t w[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      __nv_bfloat162 b = __floats2bfloat162_rn(x[ch * 8 + 2 * k], x[ch * 8 + 2 * k + 1]);
-      w[k] = *reinterpret_cast<uint32_t*>(&b);
-    }
-    *reinterpret_cast<uint4*>(tile + tc::sw128_off(row, ch)) = make_uint4(w[0], w[1], w[2], w[3]);
-  }
 }
 
 // half a row (32 columns, chunks 4*half .. 4*half+3) of a [128][64] bf16 tile
@@ -302,15 +287,9 @@ __device__ __forceinline__ void dkdv_step_tc(BwdCtx& c, const float* __restrict_
   const uint32_t t_s = c.tbase + ((uint32_t)((warp & 3) * 32) << 16), t_dp = t_s + kBN;
   const uint32_t ka = tc::smem_u32(c.sm + SM::k), va = tc::smem_u32(c.sm + SM::v), qa = tc::smem_u32(c.sm + SM::q),
                  da = tc::smem_u32(c.sm + SM::dO), pa = tc::smem_u32(c.sm + SM::pt), ga = tc::smem_u32(c.sm + SM::gt);
-#ifdef MUSE_PHASE_CLOCKS
-  const long long z0 = clock64();
-#endif
   tc::fence_async_smem();
   tc::fence_before_sync();
   __syncthreads();
-#ifdef MUSE_PHASE_CLOCKS
-  const long long z1 = clock64();
-#endif
   if (tid == 0) {
     tc::fence_after_sync();
     const uint32_t idesc = tc::idesc_bf16(kBM, kBN, 0, 0);
@@ -321,15 +300,9 @@ __device__ __forceinline__ void dkdv_step_tc(BwdCtx& c, const float* __restrict_
     tc::mma_commit(&c.bar[0]);
   }
   prefetch();                                  // global loads of the next query tile, overlapped with the MMAs
-#ifdef MUSE_PHASE_CLOCKS
-  const long long z2 = clock64();
-#endif
   if (!tc::mbar_wait(&c.bar[0], c.ph0)) { c.ok = false; return; }
   c.ph0 ^= 1;
   tc::fence_after_sync();
-#ifdef MUSE_PHASE_CLOCKS
-  const long long z3 = clock64();
-#endif
   {
     const int h = wg;
     float s[32], dp[32], Lc[32], dc[32], p[32], g[32];
@@ -353,9 +326,6 @@ __device__ __forceinline__ void dkdv_step_tc(BwdCtx& c, const float* __restrict_
     store_row32(c.sm + SM::pt, row, h, p);
     store_row32(c.sm + SM::gt, row, h, g);
   }
-#ifdef MUSE_PHASE_CLOCKS
-  const long long z4 = clock64();
-#endif
   tc::fence_async_smem();
   tc::fence_before_sync();
   __syncthreads();
@@ -374,10 +344,6 @@ __device__ __forceinline__ void dkdv_step_tc(BwdCtx& c, const float* __restrict_
   if (!tc::mbar_wait(&c.bar[1], c.ph1)) { c.ok = false; return; }
   c.ph1 ^= 1;
   tc::fence_after_sync();
-#ifdef MUSE_PHASE_CLOCKS
-  const long long z5 = clock64();
-  c.pc[0] += z1 - z0; c.pc[1] += z2 - z1; c.pc[2] += z3 - z2; c.pc[3] += z4 - z3; c.pc[4] += z5 - z4; c.pc[5] += 1;
-#endif
 }
 
 constexpr int kKeysThreads = 256;       // keys-on-M kernels: two warpgroups share the 64 query columns
@@ -478,10 +444,6 @@ k_ret_bwd_dkdv_tc(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ 
     }
     tc::fence_before_sync();
   }
-#ifdef MUSE_PHASE_CLOCKS
-  if (tid == 0 && c.pc[5] >= 8 && atomicCAS(status + 40, 0, 1) == 0)
-    for (int k = 0; k < 7; ++k) status[41 + k] = (int)c.pc[k];
-#endif
   bwd_teardown(c, SM::cols, tid, status);
 }
 

@@ -1,6 +1,7 @@
-// Exact-attention forward on the Blackwell tensor cores (bf16 inputs, fp32 accumulation in
-// tensor memory): the local block-diagonal component and the retrieved-cluster component of
-// Algorithm 1.  One CTA = 128 query rows (one thread per row); keys stream in tiles of 64.
+// A second implementation of the retrieval forward (bf16 inputs, fp32 accumulation in tensor memory), which shares no kernel code
+// with ret_fwd_tc.cu and ret_fwd_long_tc.cu: the tests hold both to the same oracle.  It runs only where the test hook asks
+// for it (muse_test_force_paths, bit 8); the dispatch of the retrieval forward is at the end.  One CTA = 128 query rows (one
+// thread per row); keys stream in tiles of 64.
 //   S  = Q K^T      tcgen05.mma, A = Q tile, B = K tile, both K-major in 128B-swizzled smem
 //   P  = softmax piece, one thread per row straight out of TMEM, written back as bf16 to smem
 //   PV              tcgen05.mma, A = P tile (K-major), B = V tile (MN-major), read from TMEM

@@ -238,8 +238,6 @@ k_block_select(Dims dm, const T* __restrict__ Q, const int32_t* __restrict__ off
   }
 }
 
-bool block_select_supported(const Dims& d) { return d.causal && d.S - 1 <= kBsMaxBlocks && d.k2 <= 8; }
-
 template <class T, int D>
 static int block_select_t(const Dims& d, const T* Q, const int32_t* off_q, const int32_t* perm_q, const int32_t* sel, const SummPtrs& sp,
                           const int32_t* bsel_in, int32_t* bsel_out, float* o_near, float* lse_near, cudaStream_t st) {

@@ -194,7 +194,6 @@ void prof_mark(const char* name, cudaStream_t st);
 
 // Status words: the first kStatusWords int32 of every stage's workspace.  Word 0 holds the first
 // MUSE_STATUS_* code a kernel reported (0 = none); the entry points clear the words once per call.
-// Words from 8 up carry diagnostics of instrumented builds only.
 constexpr int kStatusWords = 64;
 constexpr int kItemWord = 4;               // work counter of the persistent summary kernel (zeroed by the kernel before it)
 __device__ __forceinline__ void report_status(int* status, int code) { atomicCAS(status, 0, code); }
@@ -314,7 +313,6 @@ inline SummPtrs summ_ptrs_blk(const SummLayout& L, const void* base_) {      // 
   return SummPtrs{(float*)(b + L.blk), (float*)(b + L.blk_beta), b + L.blk_khi, b + L.blk_klo, b + L.blk_nu};
 }
 // dipole correction (dipole.cu): construction at summary time, consumption after the far field
-size_t dipole_fwd_ws_bytes(const Dims& d);
 // its backward (dipole_bwd.cu); scratch carved from the backward workspace
 struct DipoleBwdWs { int32_t* sel_tmp; float *lse_far, *zq, *dz, *delta_far, *xq, *corr, *csub, *dcbar, *dcov, *dpw, *dzs; void* dcbar_bf; };
 DipoleBwdWs dipole_bwd_ws(const Dims& d, Arena& ar);       // sized for either kind of contraction kernel

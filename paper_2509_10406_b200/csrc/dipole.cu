@@ -406,14 +406,6 @@ int dipole_tilt_point(const Dims& d, const int32_t* assign_q, const float* qbar,
 }
 
 // ---- host side ------------------------------------------------------------------------------------
-// Scratch of the forward pass (and of the backward's recomputation): the retrieved clusters' rows.
-size_t dipole_fwd_ws_bytes(const Dims& d) {
-  if (!d.dipole || d.m == 0 || d.SB == 0) return 0;
-  Arena ar(nullptr);
-  ar.take<float>((size_t)d.B * d.Hq * d.N * d.D);
-  return ar.used;
-}
-
 template <class T, class ST, int D>
 static int dipole_build_t(const Dims& d, int dtype, const T* Kp, const T* Vp, const int32_t* off_k, const float* mu,
                           const DipolePtrs& dp, int* status, cudaStream_t st) {

@@ -84,10 +84,6 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
   const int i = blockIdx.x, pl = blockIdx.y, pq = blockIdx.z;
   const int blk = dm.causal ? pl + 1 : 0, Ck = dm.Ck, NJ = (Ck + TJ - 1) / TJ, m = dm.m;
   const int tid = threadIdx.x, warp = tc::warp_index(), wg = tid >> 7, L = tid & 127;
-#ifdef MUSE_PHASE_CLOCKS
-  const long long t_in_ = clock64();
-  long long t_loop_ = 0, t_end_ = 0;
-#endif
   const int32_t* oq = off_q + (size_t)pq * (dm.S * dm.Cq + 1) + (size_t)blk * dm.Cq + i;
   const int p0 = oq[0], p1 = oq[1];
   if (p0 >= p1) {
@@ -197,23 +193,14 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
     tc::fence_async_smem();
     __syncthreads();
 
-#ifdef MUSE_PHASE_CLOCKS
-    long long pc[6] = {0, 0, 0, 0, 0, 0};
-#endif
     static_assert(NP == 1, "one pass per sweep");
     const bool later_sweep = !ONE && s0 > p0;               // gradients of earlier sweeps are already stored: add to them
     if (later_sweep) {
       if (warp == ISSUER / 32) tc::tma_store_wait_all_warp();
       __syncthreads();
     }
-#ifdef MUSE_PHASE_CLOCKS
-    t_loop_ = clock64();
-#endif
     for (int jt = 0; jt < NJ && ok; ++jt) {
       const int j = jt * TJ + L;
-#ifdef MUSE_PHASE_CLOCKS
-      long long k0_ = clock64(), k1_ = 0, k2_ = 0, k3_ = 0, k4_ = 0;
-#endif
       const float bj = bnext;                               // loaded one tile ahead
       const bool alive = bj != -INFINITY;                   // an empty cluster has beta = mu = -inf
       const float sig2 = dm.sigma * kLog2e, bj2 = alive ? bj * kLog2e : 0.f;
@@ -252,9 +239,6 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
         if (cw && !tc::mbar_wait(&bar1, ph1)) ok = false;
         ph1 ^= 1;
         tc::fence_after_sync();
-#ifdef MUSE_PHASE_CLOCKS
-        if (p == 0) k1_ = clock64();
-#endif
         if (cw) {
           // bit r of `near`: row r of this warpgroup's nc is not in the far set of cluster j (retrieved, past the end of the
           // segment, or the cluster is empty)
@@ -311,9 +295,6 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
           }
           gsum += gs2[0] + gs2[1]; gt2 += gt[0] + gt[1]; pdp += pd[0] + pd[1];
         }
-#ifdef MUSE_PHASE_CLOCKS
-        if (p == 0) k2_ = clock64();
-#endif
         tc::fence_async_smem();
         tc::fence_before_sync();
         __syncthreads();
@@ -353,9 +334,6 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
         tc::fence_after_sync();
       }
       ph_full ^= 1;
-#ifdef MUSE_PHASE_CLOCKS
-      k3_ = clock64();
-#endif
       if (!store) continue;
       // ---- tile read-out: warpgroup 0 -> dnu, warpgroup 1 -> dkappa; both need sum_r g
       float gtot = 0.f;
@@ -366,10 +344,6 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
         tc::named_bar_sync(1, CW);                          // the issuer is still waiting for the dq products
         gtot = part[0][L] + part[1][L];
       }
-#ifdef MUSE_PHASE_CLOCKS
-      const bool rec_ = (tid == 0 || tid == 128) && blockIdx.x == 5 && blockIdx.y == 3 && blockIdx.z == 0 && jt == 3;
-      if (rec_) status[34 + 3 * wg] = (int)(clock64() - k3_);
-#endif
       // gradient entry: [plane][i][j] like the summaries, or [plane][j][i] so that the key-side
       // pass finds the 128 query clusters of one key cluster in one contiguous tile
       const size_t gent = grad_by_key_cluster ? (((size_t)pq * dm.SB + pl) * Ck + j) * dm.Cq + i : ent0 + j;
@@ -407,16 +381,10 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
           }
         }
       }
-#ifdef MUSE_PHASE_CLOCKS
-      if (rec_) status[35 + 3 * wg] = (int)(clock64() - k3_);
-#endif
       // the two gradient tiles leave by TMA: 128 rows of 256 bytes each, Cq entries apart in the
       // [plane][j][i] layout (adjacent in the [plane][i][j] one)
       tc::fence_async_smem();
       __syncthreads();
-#ifdef MUSE_PHASE_CLOCKS
-      if (rec_) status[36 + 3 * wg] = (int)(clock64() - k3_);
-#endif
       if (warp == ISSUER / 32 && ok) {
         const int c1 = grad_by_key_cluster ? i : 0, c2 = jt * TJ, c3 = grad_by_key_cluster ? pq * dm.SB + pl : seg;
         if (!later_sweep) {
@@ -434,16 +402,7 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
       }
       tc::fence_before_sync();
       if (wg == 0 && ok && j < Ck) dS[gent] = (later_sweep ? dS[gent] : 0.f) + dsid[0][L] + dsid[1][L];
-#ifdef MUSE_PHASE_CLOCKS
-      k4_ = clock64();
-      pc[0] += k1_ - k0_; pc[1] += k2_ - k1_; pc[2] += k3_ - k2_; pc[3] += k4_ - k3_; pc[4] += 1; pc[5] = np;
-#endif
     }
-#ifdef MUSE_PHASE_CLOCKS
-    if (tid == 0 && blockIdx.x == 5 && blockIdx.y == 3 && blockIdx.z == 0 && s0 == p0)
-      for (int k = 0; k < 6; ++k) status[24 + k] = (int)pc[k];
-    t_end_ = clock64();
-#endif
     // ---- dq: warpgroup p reads pass p (thread = output dim), adds into the fp32 accumulator
     if (cw && !tc::mbar_wait(&bar3, ph3 ^ 1)) ok = false;     // the last tile's dq products
     tc::fence_after_sync();
@@ -467,11 +426,6 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
   if (warp == ISSUER / 32) tc::tma_store_wait_read_warp();             // the staging tiles must outlive the stores' reads only
   if (warp == 0) tc::tmem_dealloc(tbase, LY::cols);
   if (!ok && tid == 0) report_status(status, 4);
-#ifdef MUSE_PHASE_CLOCKS
-  if (tid == 0 && blockIdx.x == 5 && blockIdx.y == 3 && blockIdx.z == 0) {
-    status[56] = (int)(t_loop_ - t_in_); status[57] = (int)(t_end_ - t_loop_); status[58] = (int)(clock64() - t_end_);
-  }
-#endif
 }
 
 bool far_bwd_tc_supported(const Dims& d, int dtype) {

@@ -48,12 +48,7 @@ struct FarBars { uint64_t fullA[kMaxStA], emptyA[kMaxStA], fullD[kMaxStD], empty
 template <int NKMAX>
 __device__ __forceinline__ void select_top_m(float* s, int Ck, int m, int32_t* so, int lane, unsigned char* cand, int seg,
                                              bool may_compact, int* dbg = nullptr) {
-#ifdef MUSE_PHASE_CLOCKS
-  long long c0_ = clock64(), c1_ = 0, c2_ = 0, c3_ = 0, c4_ = 0;
-#define MUSE_SEL_CLOCK(x) x = clock64()
-#else
 #define MUSE_SEL_CLOCK(x)
-#endif
   const int NK = Ck >> 5;                       // scores per lane (<= NKMAX)
   auto to_key = [](float x) {
     const uint32_t b = __float_as_uint(x);
@@ -141,9 +136,6 @@ __device__ __forceinline__ void select_top_m(float* s, int Ck, int m, int32_t* s
         if (c >= m) { T = c2; if (c == m) break; }
       }
       MUSE_SEL_CLOCK(c4_);
-#ifdef MUSE_PHASE_CLOCKS
-      if (dbg && lane == 0) { dbg[0] = (int)(c1_ - c0_); dbg[1] = (int)(c2_ - c1_); dbg[2] = (int)(c3_ - c2_); dbg[3] = (int)(c4_ - c3_); dbg[4] = ncand; dbg[5] = 1; }
-#endif
       int need = m - count4(T + 1u);                            // ties at T still to take (>= 0)
       const int ntie = (int)__reduce_add_sync(0xffffffffu, (unsigned)((ck[0] == T) + (ck[1] == T) + (ck[2] == T) + (ck[3] == T)));
       bool take[4];
@@ -304,9 +296,6 @@ k_far_fwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
 
   for (int r0 = p0; r0 < p1 && ok; r0 += FR) {
     const int n = min(FR, p1 - r0);
-#ifdef MUSE_PHASE_CLOCKS
-    long long ck0 = clock64(), ck1 = 0, ck3 = 0, ck4 = 0;
-#endif
     // ---- A: scores^T for all clusters, kappa_hi / kappa_lo tiles through an nsA-stage TMA ring;
     //         the producers load (TMA), thread 32 consumes (MMA), so neither waits for the other's latency.
     //         The first ring-full of tiles is requested before the query rows are gathered.
@@ -360,17 +349,8 @@ k_far_fwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
       const uint32_t idesc = tc::idesc_bf16(kFJ, FR, 0, 0);
       const uint64_t dq0 = tc::smem_desc_sw128(tc::smem_u32(Qs), 16, 1024), da0 = tc::smem_desc_sw128(tc::smem_u32(sm), 16, 1024);
       const int T = 2 * NJ;
-#ifdef MUSE_PHASE_CLOCKS
-      long long ta0_ = clock64();
-#endif
       for (int u = 0, s = sA0, ph = phA0; u < T; ++u) {
         if (!tc::mbar_wait(&bars.fullA[s], ph)) { ok = false; break; }
-#ifdef MUSE_PHASE_CLOCKS
-        if (blockIdx.x == 200 && blockIdx.y == 5 && blockIdx.z == 1 && r0 == p0) {
-          if (u == 0) status[62] = (int)(clock64() - ta0_);
-          if (u == T - 1) status[63] = (int)(clock64() - ta0_);
-        }
-#endif
         const uint64_t da = tc::desc_step(da0, (uint32_t)s * kTileBytes);
         const uint32_t dcol = tbase + (u >> 1) * FR;
 
@@ -395,14 +375,8 @@ k_far_fwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
     done_ph ^= 1;
     cntA += TA;
     tc::fence_after_sync();
-#ifdef MUSE_PHASE_CLOCKS
-    ck1 = clock64();
-#endif
     for (int qs = 0; qs * FQ < n; ++qs) {
       // ---- B: TMEM -> sc[r][j] for the 16 queries of this step
-#ifdef MUSE_PHASE_CLOCKS
-      long long cb0 = clock64(), cb1 = 0, cb2 = 0, cb3 = 0;
-#endif
 #pragma unroll
       for (int k = 0; k < KT; ++k) {
         const int jt = tg + NTG * k;
@@ -416,9 +390,6 @@ k_far_fwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
         for (int r = 0; r < FQ; ++r) sc[r * CkP + j] = b == -INFINITY ? -INFINITY : fmaf(v[r], dm.sigma, b);
       }
       __syncthreads();
-#ifdef MUSE_PHASE_CLOCKS
-      cb1 = clock64();
-#endif
       // ---- C: selection + softmax of the far set; P (bf16) as a K-major operand [64][Ck]
       const int r = qs * FQ + warp;                    // one query per warp
       float* s = sc + warp * CkP;
@@ -434,15 +405,9 @@ k_far_fwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
         } else if (m > 0) {
           // this query's own (not yet written) P row doubles as the candidate scratch
           int* dbg = nullptr;
-#ifdef MUSE_PHASE_CLOCKS
-          if (warp == 0 && blockIdx.x == 200 && blockIdx.y == 5 && blockIdx.z == 1 && r0 == p0 && qs == 0) dbg = status + 56;
-#endif
           select_top_m<NKMAX>(s, CkP, m, so, lane, Pm + r * 128, FR * 128, CkP >= 512, dbg);
         }
         __syncwarp();
-#ifdef MUSE_PHASE_CLOCKS
-        cb2 = clock64();
-#endif
         for (int j = lane; j < CkP; j += 32) mx = fmaxf(mx, s[j]);
         mx = warp_max(mx);
       }
@@ -466,20 +431,11 @@ k_far_fwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
         rinv[r] = sum > 0.f ? 1.f / sum : 0.f;
         if (r < n) lse_far[(size_t)pq * dm.N + rows[r]] = sum > 0.f ? mx + logf(sum) : -INFINITY;
       }
-#ifdef MUSE_PHASE_CLOCKS
-      cb3 = clock64();
-      if (tid == 0 && blockIdx.x == 200 && blockIdx.y == 5 && blockIdx.z == 1 && r0 == p0 && qs == 0) {
-        status[9] = (int)(cb1 - cb0); status[13] = (int)(cb2 - cb1); status[14] = (int)(cb3 - cb2);
-      }
-#endif
       __syncthreads();
     }
     tc::fence_async_smem();
     tc::fence_before_sync();
     __syncthreads();
-#ifdef MUSE_PHASE_CLOCKS
-    ck3 = clock64();
-#endif
     // ---- D: out^T = nu^T P^T, nu tiles through an nsD-stage TMA ring in the score region
     if (prod >= 0 && prod < WD && ok) {
       unsigned char* ring = sm + p_bytes;
@@ -499,17 +455,8 @@ k_far_fwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
       const uint32_t idesc = tc::idesc_bf16(128, FR, 1, 0);
       const uint64_t dp0 = tc::smem_desc_sw128(tc::smem_u32(Pm), 16, 1024);
       const uint64_t dn0 = tc::smem_desc_sw128(tc::smem_u32(sm + p_bytes), kFJ * 128, 1024);
-#ifdef MUSE_PHASE_CLOCKS
-      long long td0_ = clock64();
-#endif
       for (int u = 0, s = sD0, ph = phD0; u < NJ; ++u) {
         if (!tc::mbar_wait(&bars.fullD[s], ph)) { ok = false; break; }
-#ifdef MUSE_PHASE_CLOCKS
-        if (blockIdx.x == 200 && blockIdx.y == 5 && blockIdx.z == 1 && r0 == p0) {
-          if (u == 0) status[15] = (int)(clock64() - td0_);
-          if (u == NJ - 1) status[16] = (int)(clock64() - td0_);
-        }
-#endif
         const uint64_t da = tc::desc_step(dn0, (uint32_t)s * kTileBytes), dp = tc::desc_step(dp0, (uint32_t)(2 * u) * (FR * 128));
 #pragma unroll
         for (int ks = 0; ks < kFJ / 16; ++ks)
@@ -528,13 +475,6 @@ k_far_fwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
     done_ph ^= 1;
     cntD += NJ;
     tc::fence_after_sync();
-#ifdef MUSE_PHASE_CLOCKS
-    ck4 = clock64();
-    if (tid == 0 && blockIdx.x == 200 && blockIdx.y == 5 && blockIdx.z == 1 && r0 == p0) {
-      status[8] = (int)(ck1 - ck0); status[9] = 0; status[10] = (int)(ck3 - ck1); status[11] = (int)(ck4 - ck3);
-      status[12] = n;
-    }
-#endif
     // ---- E: thread = output dim d; warps 0-3 read queries 0..31, warps 4-7 queries 32..63
     if (warp < FR / 8) {
       const int half = warp >> 2;

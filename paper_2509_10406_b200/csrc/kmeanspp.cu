@@ -233,8 +233,6 @@ k_kmeanspp(const __grid_constant__ PpArgs g, int N, uint64_t seed, int md_shared
   cluster.sync();                               // no CTA leaves while another may still write into its shared memory
 }
 
-size_t kmeanspp_ws_floats(int problems, int N) { return (size_t)problems * N; }
-
 template <class T, int D>
 struct PpPlan { int stages; int md_shared; size_t smem; };
 
@@ -301,8 +299,8 @@ static int kmeanspp_t(const KmeansppSide* sides, int nsides, int N, uint64_t see
   return kmeanspp_v<T, D, 2>(g, problems, N, seed, cs, pl.md_shared, pl.smem, false, nullptr, status, st);
 }
 
-// Start indices [problems, C] of every problem of one or both sides; mind2 is scratch of kmeanspp_ws_floats(problems, N)
-// floats per side.
+// Start indices [problems, C] of every problem of one or both sides; mind2 is scratch of problems * N floats
+// per side.
 int kmeanspp(int dtype, const KmeansppSide* sides, int nsides, int N, int D, uint64_t seed, int* status, cudaStream_t st) {
   typedef __nv_bfloat16 bf;
   if (dtype == MUSE_F32) return D == 64 ? kmeanspp_t<float, 64>(sides, nsides, N, seed, status, st) : kmeanspp_t<float, 128>(sides, nsides, N, seed, status, st);

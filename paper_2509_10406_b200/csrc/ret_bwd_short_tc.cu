@@ -132,14 +132,6 @@ k_ret_bwd_sweeps(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ d
   };
 
   uint32_t np = 0;                                          // tiles this half has processed: the phase count of its barriers
-#ifdef MUSE_PHASE_CLOCKS
-  long long pc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  const long long t_in_ = clock64();
-  long long z_ = t_in_;
-#define RBCLK(k) { long long n_ = clock64(); pc[k] += n_ - z_; z_ = n_; }
-#else
-#define RBCLK(k)
-#endif
   // (a cluster none of whose keys is visible, possible with forced selections, still takes one sweep: its dQ rows are zeros)
   for (int kc = 0; kc == 0 || kc < kall; kc += kKeys) {
     const bool first = kc == 0;
@@ -206,10 +198,8 @@ k_ret_bwd_sweeps(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ d
         }
         const int vis = pid >= 0 ? visible(pid, kc) : 0;
         const uint32_t ph = np & 1;
-        RBCLK(0)
         wait(&B.s_done, ph);
         tc::fence_after_sync();
-        RBCLK(1)
         float sv[2][8], dp[2][8];                           // 8 key columns at a time, the next 8 on their way
         tc::tmem_ld8_issue(tl + cS, sv[0]);
         tc::tmem_ld8_issue(tl + cDP, dp[0]);
@@ -246,10 +236,8 @@ k_ret_bwd_sweeps(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ d
         tc::fence_async_smem();                             // P and G are read by the tensor cores
         tc::fence_before_sync();
         tc::mbar_arrive(&B.pg_ready);
-        RBCLK(2)
         wait(&B.m2_done, ph);
         tc::fence_after_sync();
-        RBCLK(3)
         started = true;
         const bool live = pid >= 0 && ok_;
         bf16* drow = dq_part + (pbase + max(pid, 0)) * D;
@@ -285,10 +273,6 @@ k_ret_bwd_sweeps(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ d
           }
         }
         pid = pid_n; pid_n = pid_nn; L2 = L2_n; dl = dl_n;
-        RBCLK(4)
-#ifdef MUSE_PHASE_CLOCKS
-        pc[7] += 1;
-#endif
       }
       // dV^T and dK^T of this sweep's keys: thread = output dim, one key per column; the other half of the CTA
       // (and other CTAs that share the cluster) add theirs to the same rows
@@ -317,22 +301,17 @@ k_ret_bwd_sweeps(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ d
       for (int tile = tile0; tile < ntiles; tile += tstep, ++np) {
         {
           const uint32_t ph = np & 1;
-          RBCLK(0)
           wait(&B.q_full, ph);                               // the tile's Q and dO rows are in shared memory
-          RBCLK(1)
           if (np > 0) wait(&B.dq_free, ph ^ 1);              // the previous dQ rows have been read out of the columns S and dP go to
           tc::fence_after_sync();
-          RBCLK(2)
           const uint32_t id1 = tc::idesc_bf16(kPairs, kKeys, 0, 0);
 #pragma unroll
           for (int ks = 0; ks < D / 16; ++ks) tc::mma_bf16_ss_warp(tbase + cS, desc_k<kPairs>(qa, ks), desc_k<kKeys>(ka, ks), id1, ks > 0);
 #pragma unroll
           for (int ks = 0; ks < D / 16; ++ks) tc::mma_bf16_ss_warp(tbase + cDP, desc_k<kPairs>(da, ks), desc_k<kKeys>(va, ks), id1, ks > 0);
           tc::mma_commit_warp(&B.s_done);
-          RBCLK(3)
           wait(&B.pg_ready, ph);                             // P and G are in shared memory, S and dP consumed
           tc::fence_after_sync();
-          RBCLK(4)
           const uint32_t id_dq = tc::idesc_bf16(kPairs, D, 0, 1);        // A = G (contraction over keys), B = key rows MN-major
           // A = dO / Q tile and B = P / G tile, both contracted over pairs.  M = 128 output dims even when D = 64: the second
           // 64-dim group of the A operand is then the tile that follows in shared memory, and lanes 64..127 hold numbers nobody reads
@@ -349,10 +328,6 @@ k_ret_bwd_sweeps(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ d
             tc::mma_bf16_ss_warp(tbase + cDK, desc_mn<kPairs>(qa, ks), tc::smem_desc_sw128(ga + ks * 16 * 128, kPairs * 128, 1024), id_t, acc || ks > 0);
           tc::mma_commit_warp(&B.m2_done);
           tc::mma_commit_warp(&B.q_empty);                        // ... and the Q / dO tiles refilled
-          RBCLK(5)
-#ifdef MUSE_PHASE_CLOCKS
-          pc[7] += 1;
-#endif
         }
         __syncwarp();
       }
@@ -374,9 +349,7 @@ k_ret_bwd_sweeps(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ d
       int pa_ = ld1(tile0);
       for (int tile = tile0; tile < ntiles; tile += tstep, ++np) {
         const int pa_n = ld1(tile + tstep);
-        RBCLK(0)
         if (np > 0) wait(&B.q_empty, (np - 1) & 1);          // the previous tile's products have read the buffers
-        RBCLK(1)
         tok_s[v][g] = pa_ >= 0 ? pa_ / mk : -1;
         tc::named_bar_sync(1 + v, kGather);
 #pragma unroll 4
@@ -388,32 +361,15 @@ k_ret_bwd_sweeps(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ d
           cp_async16(od + tc::sw128_off(r, ck & 7), dOb + at, tok >= 0);
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
-        RBCLK(2)
         asm volatile("cp.async.wait_group 0;" ::: "memory");
         tc::fence_async_smem();                              // the tensor cores read the rows through the async proxy
         tc::mbar_arrive(&B.q_full);
-        RBCLK(3)
         tc::named_bar_sync(1 + v, kGather);                  // tok_s may be rewritten
         pa_ = pa_n;
-#ifdef MUSE_PHASE_CLOCKS
-        pc[7] += 1;
-#endif
       }
     }
     tc::fence_before_sync();
   }
-#ifdef MUSE_PHASE_CLOCKS
-  // (instrumented builds only: words 8..22 of the status block, five per role, in units of 16 clocks)
-  if (pc[7] >= 20 && lane == 0 && v == 0 && (warp == 0 || warp == kIssuerWarp0 || warp == kGatherWarp0)) {
-    const int slot = warp == 0 ? 0 : warp == kIssuerWarp0 ? 1 : 2;
-    if (atomicCAS(status + 5 + slot, 0, 1) == 0) {
-      int* o = status + 8 + 5 * slot;
-      if (slot == 0) { o[0] = (int)(pc[1] / 16); o[1] = (int)(pc[2] / 16); o[2] = (int)(pc[3] / 16); o[3] = (int)(pc[4] / 16); o[4] = (int)pc[7]; }
-      if (slot == 1) { o[0] = (int)(pc[1] / 16); o[1] = (int)(pc[2] / 16); o[2] = (int)(pc[4] / 16); o[3] = (int)(pc[5] / 16); o[4] = (int)((clock64() - t_in_) / 16); }
-      if (slot == 2) { o[0] = (int)(pc[1] / 16); o[1] = (int)(pc[2] / 16); o[2] = (int)(pc[3] / 16); o[3] = (int)pc[7]; o[4] = kall; }
-    }
-  }
-#endif
   tc::fence_before_sync();
   __syncthreads();
   if (warp == 0) tc::tmem_dealloc(tbase_s, NH * kCols);

@@ -65,7 +65,6 @@ k_ret_fwd_long(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_c
   RetItem item;                                             // key cluster, share of its units (dealt round-robin)
   if (!ret_item(ri, pq, item)) return;
   const int j = item.group, sub = item.share & 0xffff, nsub = item.share >> 16, b_ = pq / dm.Hq, h = pq % dm.Hq, pk = b_ * dm.Hkv + dm.hm.g[h];
-  const int32_t* go = ri.goff + (size_t)pq * (dm.SB * dm.Ck + 1) + (size_t)j * dm.SB;      // plane pl's pairs: [go[pl], go[pl + 1])
   const int g0 = item.g0, g1 = item.g1, ntiles = (g1 - g0 + kPairs - 1) / kPairs, nunits = (ntiles + 1) / 2;
   const int32_t* okg = off_k + (size_t)pk * (dm.Ck * dm.S + 1) + (size_t)j * dm.S;      // okg[b]: first key of bucket (j, b)
   const int k0 = item.k0;

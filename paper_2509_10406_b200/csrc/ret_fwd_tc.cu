@@ -108,14 +108,6 @@ k_ret_fwd_pairs_tc(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__
     const int tok = pid / dm.m;
     return min(kKeys, max(0, ok[dm.causal ? tok / dm.Bs : 1] - k0 - kc));
   };
-#ifdef MUSE_PHASE_CLOCKS
-  long long pc[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
-  const long long t_in_ = clock64();
-  long long z_ = t_in_;
-#define RFCLK(k) { long long n_ = clock64(); pc[k] += n_ - z_; z_ = n_; }
-#else
-#define RFCLK(k)
-#endif
 
   // Number of completed phases of each barrier, the same on every role: a tile with visible keys completes each once.
   uint32_t nproc = 0;
@@ -158,7 +150,6 @@ k_ret_fwd_pairs_tc(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__
       tc::fence_async_smem();                               // the tensor cores read the tiles through the async proxy
       tc::named_bar_sync(2, kGather0);
     }
-    RFCLK(0)
 
     if (warp < kIssuerWarp) {
       // ================= softmax and read-out: thread = pair row =================
@@ -197,12 +188,10 @@ k_ret_fwd_pairs_tc(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__
         if (pid >= 0) set_range(0, visible(pid, kc));
         const float lse_old = (!first && pid >= 0) ? l_part[pbase + pid] : -INFINITY;
         float M = -INFINITY, l = 0.f;
-        RFCLK(1)
         if (nk16 > 0) {
           const uint32_t ph = nproc & 1;
           wait(&bars.s_done, ph);
           tc::fence_after_sync();
-          RFCLK(2)
           // the logits are read twice (row maximum, then probabilities) rather than kept in registers
           float mx = -INFINITY;
           for (int g = 0; 32 * g < nk16; ++g) {
@@ -214,7 +203,6 @@ k_ret_fwd_pairs_tc(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__
           }
           M = mx * scale2;                                 // (scale2 > 0)
           const float base = M == -INFINITY ? 0.f : M;
-          RFCLK(3)
           for (int g = 0; 32 * g < nk16; ++g) {
             float sv[32];
             tc::tmem_ld32(tl + SM::cS + 32 * g, sv);
@@ -234,10 +222,8 @@ k_ret_fwd_pairs_tc(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__
           }
           tc::fence_before_sync();
           tc::mbar_arrive(&bars.p_ready);
-          RFCLK(4)
           wait(&bars.o_done, ph);
           tc::fence_after_sync();
-          RFCLK(5)
         }
         const bool live = pid >= 0 && ok_;
         const float inv = l > 0.f ? 1.f / l : 0.f;
@@ -292,10 +278,6 @@ k_ret_fwd_pairs_tc(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__
         if (live) l_part[pbase + pid] = lse_new;
         if (nk16 > 0) ++nproc;
         pid = pid_n; last = last_n;
-        RFCLK(6)
-#ifdef MUSE_PHASE_CLOCKS
-        pc[9] += 1;
-#endif
       }
     } else if (warp == kIssuerWarp) {
       // ================= MMA issue =================
@@ -376,12 +358,6 @@ k_ret_fwd_pairs_tc(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__
       }
     }
   }
-#ifdef MUSE_PHASE_CLOCKS
-  if (tid == 0 && pc[9] >= 6 && atomicCAS(status + 40, 0, 1) == 0) {
-    for (int k = 0; k < 10; ++k) status[41 + k] = (int)pc[k];
-    status[51] = (int)(clock64() - t_in_); status[52] = ntiles; status[53] = nsub; status[54] = kall; status[55] = g1 - g0;
-  }
-#endif
   tc::fence_before_sync();
   __syncthreads();
   if (warp == 0) tc::tmem_dealloc(tbase, SM::cols);

@@ -44,9 +44,6 @@ constexpr uint32_t cL = 0, cX = 64, cDK = 128, cDV = 192, cols = 256;
 constexpr int kOkCache = 72;                   // bucket offsets of the cluster kept in shared memory (S + 1 <= 72)
 }  // namespace sb
 
-// 2-D tensor map over a bf16 matrix with an arbitrary row pitch (bytes), 128B swizzle, box [box_rows][64]
-int make_tmap_bf16_pitched(void* out_map, const void* base, uint64_t rows, uint64_t cols, uint64_t pitch_bytes, uint32_t box_rows);
-
 // WIDE: more than 32 planes, so that which of them are live is looked up 32 at a time (one instance for both, deciding at run
 // time, spilled 28 bytes at D = 64).
 template <int D, bool WIDE>
@@ -103,13 +100,6 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
   const uint32_t aQhi = tc::smem_u32(sm + oQhi), aQlo = tc::smem_u32(sm + oQlo), aK = tc::smem_u32(sm + oK),
                  aV = tc::smem_u32(sm + oV), aW = tc::smem_u32(sm + oW);
 
-#ifdef MUSE_PHASE_CLOCKS
-  long long pc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  long long t_ = clock64();
-#define PCLK(k) { long long n_ = clock64(); pc[k] += n_ - t_; t_ = n_; }
-#else
-#define PCLK(k)
-#endif
   for (int c0 = kbeg; c0 < kvis && ok; c0 += NU) {        // 64 keys of the cluster at a time (usually one chunk)
     __syncthreads();
     if (warp == ISSUER / 32) {
@@ -141,7 +131,6 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
           tc::tma_load_3d_warp(dnu + g * TI * 128, &tm_dnu, 64 * g, i0, row, &bar_g[buf]);
         }
       };
-      PCLK(7)
       __syncthreads();                                    // every MMA that read the centroid tiles has completed (bar2 waited)
       if (warp == ISSUER / 32) {
         // sigma * qbar tile as bf16 hi + lo operands (split once per layer), and the first gradient tiles
@@ -192,7 +181,6 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
       if (!tc::mbar_wait(&bar_l, ph_l)) ok = false;       // from here on the low tile's space is free
       ph_l ^= 1;
       tc::fence_after_sync();
-      PCLK(0)
       float wc[32];                                               // sum over the planes of w c: contracted with the centroids once, below
 #pragma unroll
       for (int c = 0; c < 32; ++c) wc[c] = 0.f;
@@ -234,11 +222,9 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
           if (pl + 1 < pl_end && ok) issue_grad(pl + 1, buf ^ 1);
         }
         ph_g ^= 1u << buf;
-        PCLK(1)
         if (cw && !tc::mbar_wait(&bar1, ph1)) ok = false;
         ph1 ^= 1;
         tc::fence_after_sync();
-        PCLK(3)
         if (cw) {
           const int lo = live ? klo - 32 * wg : 32, hi = live ? nk - 32 * wg : 0;      // this thread's keys of the plane: [lo, hi)
           const bool whole = lo <= 0 && hi >= 32;
@@ -307,10 +293,6 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
         }
         started = true;
         __syncwarp();
-        PCLK(4)
-#ifdef MUSE_PHASE_CLOCKS
-        pc[6] += 1;
-#endif
       }
       if (pl0 < pl_end) {                                 // last plane's MMAs
         if (!tc::mbar_wait(&bar2, ph2)) ok = false;
@@ -348,7 +330,6 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
         }
       }
     }
-    PCLK(5)
     // read-out once per key chunk: thread = d, warpgroup = half of the keys; add into the fp32 accumulators
     const int nkc = min(NU, kvis - c0);
     if (cw) {
@@ -371,9 +352,6 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
   tc::fence_before_sync();
   __syncthreads();
   if (warp == 0) tc::tmem_dealloc(tbase, cols);
-#ifdef MUSE_PHASE_CLOCKS
-  if (tid == 0 && blockIdx.x == 5 && blockIdx.y == 0) for (int k = 0; k < 8; ++k) status[56 + k] = (int)pc[k];
-#endif
   if (!ok && tid == 0) report_status(status, 5);
 }
 
