@@ -449,7 +449,9 @@ def main():
         stages[n1] = stages.get(n1, 0.0) + dt / args.steps
         t_step += dt
     per_step.append(t_step)
-    prof = mb.muse_profile_report()
+    prof = mb.muse_profile_report(kernels=True)
+    variants = [k for k in prof if "/" in k]
+    prof = {k: v for k, v in prof.items() if "/" not in k}
     mb.muse_profile(False)
     clocks = sampler.stop() if rank == 0 else None
     if world > 1:
@@ -569,7 +571,9 @@ def main():
     launches = sum(v[0] for v in prof.values() if True)
     kernels = {k: {"launches": v[0] // args.steps, "ms_per_step": v[1] / args.steps, "share": v[1] / total_ms}
                for k, v in sorted(prof.items(), key=lambda kv: -kv[1][1])}
-    if "k_ret_bwd_dq" in kernels:                            # two kernels: S, dP, dV, dK in the other one
+    for k in variants:                                       # which of its kernels a step that has several has run
+        kernels[k.split("/")[0]]["kernel"] = k.split("/")[1]
+    if "k_ret_bwd_pairs_tc/k_ret_bwd_dkdv" in variants:      # S, dP, dV, dK; k_ret_bwd_dq has S, dP, dQ
         model["k_ret_bwd_pairs_tc"] = ("tensor", model["k_ret_bwd_pairs_tc"][1] * 0.8)
     top = next(iter(kernels))
     roof = {"kernel": top, "bound": None, "achieved": None, "peak": None, "unit": None, "frac": None, "traffic": None}

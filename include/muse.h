@@ -317,7 +317,9 @@ MUSE_API int muse_cluster_streaming(const muse_params_t* p, const void* Q, const
  * kernel launch (events are created on demand and reused); muse_profile(0) stops recording.
  * muse_profile_report waits for the last recorded event, then writes one text line per kernel
  * name, "name launches total_ms", into buf (HOST, cap bytes) and returns the byte count, or a
- * negative MUSE_ERR_* code.  Not thread-safe with respect to concurrent library calls. */
+ * negative MUSE_ERR_* code.  Where one name stands for a step that has several kernels (the far field
+ * and retrieval choose by size), a further line "name/kernel launches total_ms" says which ran; its
+ * launches and time are part of the step's line.  Not thread-safe with respect to concurrent library calls. */
 MUSE_API int muse_profile(int enable);
 MUSE_API long muse_profile_report(char* buf, size_t cap);
 

@@ -145,8 +145,9 @@ def muse_profile(enable: bool) -> None:
     _check(lib().muse_profile(int(enable)), "muse_profile")
 
 
-def muse_profile_report() -> dict:
-    """{kernel name: (launches, total ms)} since muse_profile(True)."""
+def muse_profile_report(kernels: bool = False) -> dict:
+    """{kernel name: (launches, total ms)} since muse_profile(True).  kernels: also "name/kernel" entries, which say which of its
+    kernels a step that has several has run (a part of the step's own entry)."""
     buf = ctypes.create_string_buffer(1 << 16)
     n = lib().muse_profile_report(buf, len(buf))
     if n < 0:
@@ -154,7 +155,8 @@ def muse_profile_report() -> dict:
     out = {}
     for line in buf.value.decode().splitlines():
         name, launches, ms = line.split()
-        out[name] = (int(launches), float(ms))
+        if kernels or "/" not in name:
+            out[name] = (int(launches), float(ms))
     return out
 
 

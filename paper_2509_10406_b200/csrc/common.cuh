@@ -189,8 +189,9 @@ inline int launch_pdl(void (*kernel)(KA...), dim3 grid, int threads, size_t smem
 #define MUSE_RC(expr) do { int rc_ = (expr); if (rc_ != MUSE_OK) return rc_; } while (0)
 int sm_count();                            // multiprocessors of the current device (api.cu)
 
-// per-kernel timing hook (no-op unless muse_profile(1) was called); name = nullptr ends a call
-void prof_mark(const char* name, cudaStream_t st);
+// per-kernel timing hook (no-op unless muse_profile(1) was called); name = nullptr ends a call.  kernel: which of the kernels of a
+// step that has several with one name
+void prof_mark(const char* name, cudaStream_t st, const char* kernel = nullptr);
 
 // Status words: the first kStatusWords int32 of every stage's workspace.  Word 0 holds the first
 // MUSE_STATUS_* code a kernel reported (0 = none); the entry points clear the words once per call.

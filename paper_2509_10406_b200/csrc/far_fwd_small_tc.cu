@@ -400,7 +400,7 @@ int far_fwd_small(const Dims& d, const SummPtrs& sp, const void* Q, const int32_
   MUSE_RC(make_tmap_bf16_nd(&khi, sp.khi, 3, dims, strides, box));
   MUSE_RC(make_tmap_bf16_nd(&klo, sp.klo, 3, dims, strides, box));
   MUSE_RC(make_tmap_bf16_nd(&nu, sp.nu, 3, dims, strides, box));
-  prof_mark("k_far_fwd_tc", st);
+  prof_mark("k_far_fwd_tc", st, "k_far_fwd_small");
   const bool two = d.Ck > fs::kJ, long_list = d.m > 8;
 #define MUSE_FS(D_, CT_, ML_) far_fwd_small_t<D_, CT_, ML_>(d, khi, klo, nu, sp, Q, off_q, perm_q, sel_in, sel_out, o_far, lse_far, status, st)
   if (d.D == 128) return two ? (long_list ? MUSE_FS(128, 2, 16) : MUSE_FS(128, 2, 8)) : (long_list ? MUSE_FS(128, 1, 16) : MUSE_FS(128, 1, 8));

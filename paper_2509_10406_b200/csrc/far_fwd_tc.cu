@@ -527,7 +527,7 @@ int far_fwd_tc(const Dims& d, const SummPtrs& sp, const void* Q, const int32_t* 
   nsD = nsD > kMaxStD ? kMaxStD : nsD;
   // (D = 64: one more tile of room behind the ring, which the padded 128-row products of phase D read past)
   const size_t smem = (size_t)p_bytes + sc_bytes + FR * d.D * 2 + 1024 + (d.D == 64 ? tile_bytes : 0);
-  prof_mark("k_far_fwd_tc", st);
+  prof_mark("k_far_fwd_tc", st, "k_far_fwd_tc");
   // TMEM columns: all FR x Ck scores of a pass (the output of phase D reuses them), a power of two >= 32
   int tcols = 32;
   while (tcols < FR * (CkP / kFJ)) tcols *= 2;

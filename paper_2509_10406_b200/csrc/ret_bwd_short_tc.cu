@@ -379,7 +379,7 @@ k_ret_bwd_sweeps(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ d
 int ret_bwd_short_tc(const Dims& d, const void* Q, const void* dO, const void* Kp, const void* Vp, const float* LSE,
                      const float* delta, const int32_t* off_k, const RetIndex& ri, void* dq_part,
                      float* dK_perm, float* dV_perm, int* status, cudaStream_t st) {
-  prof_mark("k_ret_bwd_pairs_tc", st);
+  prof_mark("k_ret_bwd_pairs_tc", st, "k_ret_bwd_sweeps");
   const dim3 grid(ri.cap, d.B * d.Hq);
   if (d.D == 128) {
     MUSE_CUDA_OK(cudaFuncSetAttribute(k_ret_bwd_sweeps<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, rs::Lay<128>::kSmem));

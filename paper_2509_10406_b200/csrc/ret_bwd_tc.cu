@@ -620,7 +620,7 @@ static int ret_bwd_d(const Dims& d, const void* Q, const void* dO, const void* K
     MUSE_RC(make_tmap_bf16_rows(&v[i], Vp, rk, D, i == 0 ? rb::kM : rb::kN));
   }
   const dim3 grid(ri.cap, d.B * d.Hq);
-  prof_mark("k_ret_bwd_pairs_tc", st);
+  prof_mark("k_ret_bwd_pairs_tc", st, "k_ret_bwd_dkdv");
   MUSE_CUDA_OK(cudaFuncSetAttribute(k_ret_bwd_dkdv<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, rk::Lay<D>::total));
   MUSE_RC(launch_pdl(k_ret_bwd_dkdv<D>, grid, rk::Lay<D>::kThreads, rk::Lay<D>::total, st, d, k[0], v[0], (const bf16*)Q, (const bf16*)dO, LSE, delta, off_k, ri, dK_perm, dV_perm, status));
   MUSE_LAUNCH_OK();

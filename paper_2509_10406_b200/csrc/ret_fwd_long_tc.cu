@@ -371,7 +371,7 @@ static int ret_fwd_long_d(const Dims& d, const void* Q, const void* Kp, const vo
   MUSE_RC(make_tmap_bf16_rows(&k, Kp, (uint64_t)d.B * d.Hkv * d.N, D, rl::kKeys));
   MUSE_RC(make_tmap_bf16_rows(&v, Vp, (uint64_t)d.B * d.Hkv * d.N, D, rl::kKeys));
   MUSE_CUDA_OK(cudaFuncSetAttribute(k_ret_fwd_long<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, rl::Lay<D>::total));
-  prof_mark("k_ret_fwd_pairs_tc", st);
+  prof_mark("k_ret_fwd_pairs_tc", st, "k_ret_fwd_long");
   MUSE_RC(launch_pdl(k_ret_fwd_long<D>, dim3(ri.cap, d.B * d.Hq), rl::Lay<D>::kThreads, rl::Lay<D>::total, st, d, k, v, (const bf16*)Q, off_k, ri, (bf16*)o_part, l_part, status));
   MUSE_LAUNCH_OK();
   return MUSE_OK;

@@ -375,7 +375,7 @@ int ret_fwd_pairs_tc(const Dims& d, const void* Q, const void* Kp, const void* V
   if (d.k2 == 0 && d.N / d.Ck >= (d.D == 128 ? 128 : 256))             // mean keys of a cluster
     return ret_fwd_long_tc(d, Q, Kp, Vp, off_k, ri, o_part, l_part, status, st);
   const dim3 grid(ri.cap, d.B * d.Hq);
-  prof_mark("k_ret_fwd_pairs_tc", st);
+  prof_mark("k_ret_fwd_pairs_tc", st, "k_ret_fwd_pairs_tc");
   if (d.D == 128) {
     MUSE_CUDA_OK(cudaFuncSetAttribute(k_ret_fwd_pairs_tc<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, rf::Smem<128>::total));
     MUSE_RC(launch_pdl(k_ret_fwd_pairs_tc<128>, grid, rf::kThreads, rf::Smem<128>::total, st, d, (const bf16*)Q, (const bf16*)Kp, (const bf16*)Vp, off_k, ri, (bf16*)o_part, l_part, status));

@@ -77,7 +77,7 @@ class Case:
 
 class kernels_launched:
     """Context manager: records the library's kernel names launched inside the block (through the
-    library's own per-kernel timing hook), so that a test can assert which path ran."""
+    library's own per-kernel timing hook; "step/kernel" where a step has several), so that a test can assert which path ran."""
 
     def __enter__(self):
         from paper_2509_10406_b200 import binding as mb
@@ -88,6 +88,6 @@ class kernels_launched:
 
     def __exit__(self, *exc):
         torch.cuda.synchronize()
-        self.names = set(self.mb.muse_profile_report())
+        self.names = set(self.mb.muse_profile_report(kernels=True))
         self.mb.muse_profile(False)
         return False

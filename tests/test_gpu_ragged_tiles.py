@@ -8,7 +8,7 @@ from tests import test_gpu_k2
 from tests.gpu_util import kernels_launched, to_np
 from tests.test_gpu_backward import _backward_parity, _backward_parity_run
 from tests.test_gpu_cluster import CASES
-from tests.test_gpu_forward import TC_BWD_KERNELS, TC_FWD_KERNELS, _forward_parity
+from tests.test_gpu_forward import TC_BWD_KERNELS, TC_FWD_KERNELS, _forward_parity, _forward_parity_run
 
 pytestmark = pytest.mark.gpu
 
@@ -60,6 +60,10 @@ def test_retrieval_on_both_sides_of_the_cluster_length_rule(base, Ck, m, two_ker
     with kernels_launched() as rec:
         _backward_parity_run(w, 128.0)
     assert "k_ret_bwd_pairs_tc" in rec.names and ("k_ret_bwd_dq" in rec.names) == two_kernels
+    streamed = 2040 // Ck >= (128 if w.D == 128 else 256)
+    assert {n for n in rec.names if n.startswith(("k_ret_fwd_pairs_tc/", "k_ret_bwd_pairs_tc/"))} == {
+        "k_ret_fwd_pairs_tc/" + ("k_ret_fwd_long" if streamed else "k_ret_fwd_pairs_tc"),
+        "k_ret_bwd_pairs_tc/" + ("k_ret_bwd_dkdv" if two_kernels else "k_ret_bwd_sweeps")}, sorted(rec.names)
 
 
 @pytest.mark.parametrize("base,Cq,Ck,m,S,k2", [("d64", 5, 9, 4, 10, 1), ("d64", 3, 40, 33, 3, 1), ("d128", 7, 10, 5, 12, 2), ("d128", 1, 6, 6, 2, 1)])
@@ -74,7 +78,12 @@ def test_near_field_backward_over_groups_of_blocks(monkeypatch, base, Cq, Ck, m,
 def test_selection_and_far_field_of_few_clusters(base, Cq, Ck, m):
     """Lists of 8 and 16 (and one more, which another kernel takes), one and two tiles of clusters, several passes over a segment."""
     w = CASES[base].with_(Hq=2, Hkv=1, N=1020, S=4, Cq=Cq, Ck=Ck, m=m, components=64)
-    _forward_parity(w, 128.0, expect_kernels=TC_FWD_KERNELS)
+    with kernels_launched() as rec:
+        _forward_parity_run(w, 128.0)
+    assert TC_FWD_KERNELS <= rec.names, sorted(rec.names)
+    # (once with the GPU's selection, once with the oracle's: a given selection may be of any length)
+    assert {n for n in rec.names if n.startswith("k_far_fwd_tc/")} == (
+        {"k_far_fwd_tc/k_far_fwd_small"} | ({"k_far_fwd_tc/k_far_fwd_tc"} if m > 16 else set())), sorted(rec.names)
 
 
 @pytest.mark.parametrize("base,Cq,Ck,m", [("d64", 1, 128, 20), ("d64", 2, 129, 33), ("d128", 1, 128, 33), ("d128", 3, 90, 4)])
