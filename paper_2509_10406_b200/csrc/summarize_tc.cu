@@ -11,12 +11,12 @@
 // of a step before the sums of the one before it), four warps make weights, sixteen write snapshots; a snapshot's writers
 // give the accumulators back as soon as they hold them in registers.
 //
-// Bound by the snapshot writes, 6 D bytes per (query cluster, key cluster, plane): 4.9 TB/s at 128k tokens, 512 x 2048 clusters,
+// Bound by the snapshot writes, 6 D bytes per (query cluster, key cluster, plane): 5.0 TB/s at 128k tokens, 512 x 2048 clusters,
 // D = 128; by the weights of one step after the other where the summaries are few.  Snapshots leave through shared memory
 // by TMA: written from registers, 32 bytes a thread, they kept the load/store unit busy for 3000 cycles a plane (6.28 ms
-// against 4.65).  Against one CTA per item with every phase behind a CTA barrier and accumulators in registers: 64k tokens,
+// against 4.57).  Against one CTA per item with every phase behind a CTA barrier and accumulators in registers: 64k tokens,
 // 128 x 128 clusters, D = 64, 32 heads 1499 -> 605 us; 8k tokens, 64 x 128, 16 heads 304 -> 143; 16k, 128 x 256, 32 heads
-// 1202 -> 634; 64k, 256 x 1024, D = 128, 4 heads 1696 -> 1163; 128k, 512 x 2048 6.52 -> 4.65 ms.
+// 1202 -> 634; 64k, 256 x 1024, D = 128, 4 heads 1696 -> 1144; 128k, 512 x 2048 6.52 -> 4.57 ms.
 #include <cuda.h>
 #include "common.cuh"
 #include "tc05.cuh"
@@ -377,36 +377,31 @@ k_summarize_tc(Dims dm, const __grid_constant__ CUtensorMap tm_K, const __grid_c
         }
         // three swizzled [128 rows][128 B] tiles per 64 dims, which leave by TMA (rows of consecutive query clusters are Ck entries apart)
         unsigned char* stage = sm + LY::oStage + grp * 3 * kTile;
-        // Where DRAM is the bound (D = 128, dozens of items per CTA) each tile leaves on its own and the next snapshot's waits for that one
-        // alone (128k tokens, 512 x 2048 clusters: 4.95 -> 4.65 ms); else one pair of barriers for the three (50 x 200 clusters, 8 items
-        // per CTA: 121 -> 108 us).
-        const bool apart = D == 128 && items >= 32 * (int)gridDim.x;
+        // One pair of barriers for the three tiles: to let each leave on its own while the next snapshot waits for that one alone was slower
+        // at 34 sizes of 3 to 221 items per CTA (D = 128, us, together | apart: 50 x 200 clusters, 8 items 111 | 119, 130 items 1448 |
+        // 1565; 128 x 512, 7 items 150 | 159, 110 items 2177 | 2250; 256 x 1024, 28 items 582 | 597; 512 x 2048, 55 items 1144 | 1159,
+        // 221 items 4568 | 4612).
+        if (lead) tc::tma_store_wait_read_warp();
+        tc::named_bar_sync(1 + grp, kGroup);
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-          if (apart || a == 0) {
-            if (lead) { if (apart) tc::tma_store_wait_read_but_warp<2>(); else tc::tma_store_wait_read_warp(); }
-            tc::named_bar_sync(1 + grp, kGroup);
-          }
 #pragma unroll
           for (int c = 0; c < 4; ++c) {
             const int ch = 4 * part + c;                   // 16-byte chunk of the row
             const uint32_t* x = a == 0 ? hw : a == 1 ? lw : nw;
             *reinterpret_cast<uint4*>(stage + a * kTile + (ch >> 3) * TI * 128 + tc::sw128_off(row, ch & 7)) = make_uint4(x[4 * c], x[4 * c + 1], x[4 * c + 2], x[4 * c + 3]);
           }
-          if (apart || a == 2) {
-            tc::fence_async_smem();
-            tc::named_bar_sync(1 + grp, kGroup);
-            if (lead && ok) {
+        }
+        tc::fence_async_smem();
+        tc::named_bar_sync(1 + grp, kGroup);
+        if (lead && ok) {
 #pragma unroll
-              for (int b = 0; b < 3; ++b) {
-                if (b > a || (apart && b < a)) continue;
-                const void* map = b == 0 ? (const void*)&tm_okhi : b == 1 ? (const void*)&tm_oklo : (const void*)&tm_onu;
+          for (int a = 0; a < 3; ++a) {
+            const void* map = a == 0 ? (const void*)&tm_okhi : a == 1 ? (const void*)&tm_oklo : (const void*)&tm_onu;
 #pragma unroll
-                for (int g = 0; g < G; ++g) tc::tma_store_4d_warp(map, stage + b * kTile + g * TI * 128, 64 * g, j, P.i0, pq * dm.SB + pl);
-              }
-              tc::tma_store_commit_warp();
-            }
+            for (int g = 0; g < G; ++g) tc::tma_store_4d_warp(map, stage + a * kTile + g * TI * 128, 64 * g, j, P.i0, pq * dm.SB + pl);
           }
+          tc::tma_store_commit_warp();
         }
       }
     }

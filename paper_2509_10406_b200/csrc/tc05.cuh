@@ -182,10 +182,6 @@ __device__ __forceinline__ void tma_store_4d_warp(const void* tmap, const void* 
 }
 __device__ __forceinline__ void tma_store_commit_warp() { if (elect_one()) tma_store_commit(); }
 __device__ __forceinline__ void tma_store_wait_read_warp() { if (elect_one()) tma_store_wait_read(); __syncwarp(); }
-template <int N> __device__ __forceinline__ void tma_store_wait_read_but_warp() {         // all but the last N groups have been read
-  if (elect_one()) asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory");
-  __syncwarp();
-}
 __device__ __forceinline__ void tma_store_wait_all_warp() { if (elect_one()) tma_store_wait_all(); __syncwarp(); }
 // warp index that the compiler knows to be the same for the whole warp
 __device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
