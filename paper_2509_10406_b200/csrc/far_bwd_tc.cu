@@ -31,7 +31,7 @@ int make_tmap_bf16_nd(void* out_map, const void* base, int rank, const uint64_t*
 
 namespace fb {
 constexpr int TJ = 128, NR = 64, NP = 1;
-constexpr int THREADS = 288, CW = 256, ISSUER = 256;   // warps 0-7 do the arithmetic; lane 0 of a ninth warp issues every TMA transfer and MMA
+constexpr int THREADS = 288, CW = 256, ISSUER = 256;   // warps 0-7 do the arithmetic; a ninth warp issues every TMA transfer and MMA
 template <int D, bool ONE> struct Lay {
   static constexpr int kTile = TJ * D * 2;        // operand tile [128 clusters][D] bf16
   static constexpr int kRows = NR * D * 2;        // tile of 64 query rows

@@ -16,8 +16,8 @@
 // sweep: the rows were then gathered, and the stored dQ row read and rewritten, once per 64 keys.)
 //
 // Bound: the tensor cores where clusters are long (7 products, 784 + 588 cycles per 128 x 64 tile at D = 64), else the
-// gather of rows (23-26 B/clk per SM).  64 heads of two sequences of 64k tokens, D = 64, 512 keys per cluster, 8 slots:
-// 16.86 ms in one kernel with five products per tile (ret_bwd_short_tc.cu, which short clusters keep), 5.41 + 3.61 ms here.
+// gather of rows (23-26 B/clk per SM).  16 heads of two sequences of 64k tokens, D = 64, 512 keys per cluster, 8 slots:
+// 16.86 ms in one kernel with five products per tile (ret_bwd_short_tc.cu, which short clusters keep), 5.26 + 3.46 ms here.
 #include <cuda.h>
 #include "common.cuh"
 #include "tc05.cuh"

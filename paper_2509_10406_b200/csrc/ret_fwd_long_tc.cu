@@ -11,8 +11,8 @@
 // order ... O += P(n) V, S(n + NB) = Q K ..., which the tensor core keeps, so S(n + NB) may overwrite P(n) and the tensor
 // cores need not wait at a unit's end.  A pair's partial row is written once.
 //
-// Bound by the exponentials (16 per clock and SM) and the latency of a warp's pass over its logits.  64 heads of two
-// sequences of 64k tokens, D = 64, 512 keys per cluster, 8 slots: 7.32 ms with 128 resident keys per sweep, 4.47 ms here.
+// Bound by the exponentials (16 per clock and SM) and the latency of a warp's pass over its logits.  16 heads of two
+// sequences of 64k tokens, D = 64, 512 keys per cluster, 8 slots: 7.32 ms with 128 resident keys per sweep, 4.29 ms here.
 #include <cuda.h>
 #include "common.cuh"
 #include "tc05.cuh"

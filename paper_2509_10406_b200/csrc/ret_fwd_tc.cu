@@ -9,7 +9,7 @@
 //   O = P V                 tcgen05.mma with P as the tensor-memory operand; the result is read out,
 //                           normalised and stored as a bf16 partial row with its log-sum-exp (the
 //                           merge kernel combines a query's slots)
-// Warp roles: warps 0-3 softmax and read-out (thread = pair row), lane 0 of warp 4 issues the MMAs,
+// Warp roles: warps 0-3 softmax and read-out (thread = pair row), warp 4 issues the MMAs,
 // warps 5-6 gather the Q rows of the next tile as soon as the first product has released the single Q
 // buffer (16-byte asynchronous copies; an SM's load/store unit moves such scattered 256-byte rows at
 // about 25 bytes per clock at best, so no arithmetic warp should spend its time issuing them; more
@@ -367,10 +367,12 @@ k_ret_fwd_pairs_tc(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__
 int ret_fwd_long_tc(const Dims& d, const void* Q, const void* Kp, const void* Vp, const int32_t* off_k, const RetIndex& ri, void* o_part, float* l_part, int* status, cudaStream_t st);
 
 // The kernel here keeps 128 keys resident and two CTAs on an SM, but a cluster of more keys takes sweeps that gather the rows again and
-// read back the stored ones; the other streams the keys, and a tile of few keys pays for its longer pipeline.  Measured,
-// resident | streamed, us:
-//   D = 64:   64 keys 258 | 403,  128 keys 249 | 260 (sharp selections 219 | 275),  256 keys 727 | 544,  512 keys 7320 | 4470
-//   D = 128:  64 keys 408 | 506,  128 keys 366 | 319,  256 keys 993 | 665
+// read back the stored ones; the other streams the keys, and a tile of few keys pays for its longer pipeline.  From 256 keys
+// (D = 64) and 128 (D = 128) on the streamed one is faster at every size measured, sharp selections or flat; the crossings themselves are
+// near 170 and 80 keys, and between them and the lines the resident kernel gives away up to a fifth.  Resident | streamed, us, 16 heads
+// of 16k tokens in 8 blocks, 8 slots, flat selections (sharp ones: 3 to 40% more on both sides, the same order):
+//   D = 64:   64 keys 278 | 379,  128 keys 379 | 411,  160 keys 418 | 427,  192 keys 483 | 446,  256 keys 597 | 478,  512 keys 942 | 589
+//   D = 128:  32 keys 388 | 480,  64 keys 506 | 519,  96 keys 604 | 548,  128 keys 733 | 579,  256 keys 1072 | 669,  512 keys 1722 | 807
 int ret_fwd_pairs_tc(const Dims& d, const void* Q, const void* Kp, const void* Vp, const int32_t* off_k, const RetIndex& ri, void* o_part, float* l_part, int* status, cudaStream_t st) {
   if (d.k2 == 0 && d.N / d.Ck >= (d.D == 128 ? 128 : 256))             // mean keys of a cluster
     return ret_fwd_long_tc(d, Q, Kp, Vp, off_k, ri, o_part, l_part, status, st);

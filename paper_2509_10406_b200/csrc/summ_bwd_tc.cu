@@ -29,7 +29,7 @@ typedef __nv_bfloat16 bf16;
 
 namespace sb {
 constexpr int TI = 128, NU = 64;
-constexpr int THREADS = 288, ISSUER = 256;     // warps 0-7 do the arithmetic; lane 0 of a ninth warp issues every TMA load and MMA
+constexpr int THREADS = 288, ISSUER = 256;     // warps 0-7 do the arithmetic; a ninth warp issues every TMA load and MMA
 template <int D> struct Lay {
   static constexpr int kTile = TI * D * 2;     // [128 query clusters][D] bf16
   static constexpr int kKeys = NU * D * 2;     // [64 keys][D] bf16
@@ -121,7 +121,7 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
       const int i = i0 + L;
       const bool in_range = cw && i < dm.Cq;
       const int ic = in_range ? i : 0;
-      auto issue_grad = [&](int pl, int buf) {            // thread 0: both gradient tiles of (plane, j, i0..i0+127)
+      auto issue_grad = [&](int pl, int buf) {            // the ninth warp: both gradient tiles of (plane, j, i0..i0+127)
         tc::mbar_expect_tx_warp(&bar_g[buf], 2 * kTile);
         const int row = (pq * dm.SB + pl) * dm.Ck + j;    // (rows i >= Cq are zeros)
         unsigned char* dka = sm + (buf ? oQlo : oDka0);
