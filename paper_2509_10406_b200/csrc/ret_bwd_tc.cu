@@ -10,7 +10,9 @@
 //   k_ret_bwd_dkdv   128 keys resident, tiles of 64 pairs gathered:  S^T = K Q^T, dP^T = V dO^T;  dV += P^T dO, dK += G^T Q
 //   k_ret_bwd_dq     128 pairs gathered (four buffers at D = 64, two at D = 128), tiles of 64 keys by TMA:  S = Q K^T, dP = dO V^T;  dQ += G K
 // A tile of streamed keys may reach past the cluster, into the keys of the next one or of the next head: those rows are zeroed before
-// they meet G, and G is 0 (not 0 times what the row gave) wherever a pair does not see the key.
+// they meet G, and G is 0 (not 0 times what the row gave) wherever a pair does not see the key.  (The rows while G is being made, G by
+// masks on packed pairs: buckets of 64 keys, 8 heads of two sequences of 64k, 1207 us without any of it, 1293 zeroed before the
+// first products with G selected in fp32, 1251 so.)
 // A pair's rows are gathered once for dQ and once per 128 keys it sees for dK and dV, and its dQ row is written once.
 // (One kernel for all five products has to keep dK and dV of the keys at hand in tensor memory, so it takes 64 keys per
 // sweep: the rows were then gathered, and the stored dQ row read and rewritten, once per 64 keys.)
@@ -481,8 +483,6 @@ k_ret_bwd_dq(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_con
       wait(&bars.k_full[sk1], phk1);
       wait(&bars.v_full[sv1], phv1);
       tc::fence_after_sync();
-      const int own = gr.kall - ka * kN;                   // the cluster's keys among the tile's
-      if (own < kN) tc::zero_rows<G, kN>(sm + LY::oK + sk1 * kCol, own, kN);
       const uint32_t c = tbase + (uint32_t)(n1 % NW) * 2 * kN;
       const uint64_t a = tc::desc_step(dq0, (uint32_t)(ia % NQ) * kRow), o = tc::desc_step(do0, (uint32_t)(ia % NQ) * kRow);
       const uint64_t x = tc::desc_step(dk0, (uint32_t)sk1 * kCol), y = tc::desc_step(dv0, (uint32_t)sv1 * kCol);
@@ -507,7 +507,11 @@ k_ret_bwd_dq(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_con
       if (T > 0) { wait(&bars.acc_free[b], (used >> b) & 1u); used ^= 1u << b; }
       for (int t = 0; t < T && ok_; ++t, ++n2) {
         while (n1 - n2 < NW && first(n1 == n2)) {}
-        const int w = n2 % NW;
+        const int w = n2 % NW, own = gr.kall - t * kN;     // the cluster's keys among the tile's
+        if (own < kN) {                                    // while G is being made, once the first products have read the tile
+          wait(&bars.s_full[w], (n2 / NW) & 1);
+          tc::zero_rows<G, kN>(sm + LY::oK + sk * kCol, own, kN);
+        }
         wait(&bars.ready[w], (n2 / NW) & 1);
         tc::fence_after_sync();
         const uint32_t c = tbase + (uint32_t)w * 2 * kN, acc = tbase + LY::cAcc + (uint32_t)b * D;
@@ -586,11 +590,13 @@ k_ret_bwd_dq(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_con
 #pragma unroll
           for (int c = 0; c < 16; ++c) {
             dp[c] = tc::fast_exp2(fmaf(sv[c], scale2, -L2)) * (dp[c] - dl);
-            if (!full) dp[c] = 16 * q + c < v ? dp[c] : 0.f;
           }
           uint32_t gw[8];
 #pragma unroll
-          for (int k = 0; k < 8; ++k) gw[k] = pack2(dp[2 * k], dp[2 * k + 1]);
+          for (int k = 0; k < 8; ++k) {
+            gw[k] = pack2(dp[2 * k], dp[2 * k + 1]);
+            if (!full) gw[k] = 16 * q + 2 * k + 1 < v ? gw[k] : 16 * q + 2 * k < v ? gw[k] & 0xffffu : 0u;
+          }
           tc::tmem_st8_issue(ts + 8 * q, gw);              // over logits already consumed
           if (q < 3) {
 #pragma unroll

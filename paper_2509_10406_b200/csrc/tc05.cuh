@@ -301,7 +301,7 @@ __device__ __forceinline__ float fast_exp2(float x) {
 template <int G, int ROWS> __device__ __forceinline__ void zero_rows(unsigned char* tile, int r, int end) {
 #pragma unroll
   for (int g = 0; g < G; ++g)
-#pragma unroll 1
+#pragma unroll 4
     for (int o = r * 128 + (int)(threadIdx.x & 31) * 16; o < end * 128; o += 512) *reinterpret_cast<uint4*>(tile + g * ROWS * 128 + o) = make_uint4(0u, 0u, 0u, 0u);
   fence_async_smem();                                      // the tensor cores read the tile through the async proxy
   __syncwarp();
