@@ -14,8 +14,10 @@
 // buffer (16-byte asynchronous copies; an SM's load/store unit moves such scattered 256-byte rows at
 // about 25 bytes per clock at best, so no arithmetic warp should spend its time issuing them; more
 // gather warps were slower: their copies crowd out the row warps' stores).  The CTA is deliberately
-// small (96 KB of shared memory, 256 TMEM columns, 224 threads) so that two of them share an SM and
-// fill each other's waits.
+// small (D = 128: 96 KB of shared memory, 256 TMEM columns, 224 threads) so that two of them share an SM and
+// fill each other's waits; at D = 64 three do (48 KB, 128 columns: the output takes the columns of logits that P has left, and
+// 80 registers): 16 heads of 8k tokens, 64 keys a cluster 137 -> 123 us, 32 heads of 16k 919 -> 801, 32 keys 141 -> 128; four CTAs
+// (72 registers, spills) 129, 872 and 132.
 // Clusters with more than 128 visible keys take further sweeps over the tiles that see them; a later
 // sweep merges its partial result into the stored row by log-sum-exp weights.
 // The row, issuing and gather warps start together: the gather of the first tile runs beside the load of the keys, of which only
@@ -37,7 +39,9 @@ constexpr int kOkCache = 72;                               // bucket offsets of 
 template <int D> struct Smem {
   static constexpr int kv = kKeys * D * 2;                 // the K tile, and the V tile
   static constexpr int k = 0, v = kv, q = 2 * kv, total = q + kPairs * D * 2 + 1024;
-  static constexpr uint32_t cS = 0, cO = kKeys, cols = 256;      // TMEM: logits, then P (packed bf16) over them | output
+  // TMEM: logits, then P (packed bf16) over the first half of them | output (D = 64: over the second half)
+  static constexpr uint32_t cS = 0, cO = D == 64 ? kKeys / 2 : kKeys, cols = D == 64 ? 128 : 256;
+  static constexpr int ctas = D == 64 ? 3 : 2;             // on an SM
 };
 
 struct Bars { uint64_t q_full, q_empty, s_done, p_ready, o_done, o_free; };
@@ -49,7 +53,7 @@ __device__ __forceinline__ void cp_async16(void* smem_dst, const void* src, bool
 }  // namespace rf
 
 template <int D>
-__global__ void __launch_bounds__(rf::kThreads, 2)
+__global__ void __launch_bounds__(rf::kThreads, rf::Smem<D>::ctas)
 k_ret_fwd_pairs_tc(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ Kp, const bf16* __restrict__ Vp,
                    const int32_t* __restrict__ off_k, const __grid_constant__ RetIndex ri, bf16* __restrict__ o_part,
                    float* __restrict__ l_part, int* __restrict__ status) {
@@ -292,7 +296,7 @@ k_ret_fwd_pairs_tc(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__
         const uint32_t ph = nproc & 1;
         {
           wait(&bars.q_full, ph);                            // the tile's Q rows are in shared memory
-          if (nproc > 0) wait(&bars.o_done, ph ^ 1);         // the previous product has read P: the logits may be overwritten
+          if (nproc > 0) wait(D == 64 ? &bars.o_free : &bars.o_done, ph ^ 1);      // the previous product has read P (D = 64: ... and its output has been read)
           tc::fence_after_sync();
           const uint32_t idesc = tc::idesc_bf16(kPairs, nk16, 0, 0);
 #pragma unroll
@@ -302,7 +306,7 @@ k_ret_fwd_pairs_tc(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__
           tc::mma_commit_warp(&bars.s_done);
           tc::mma_commit_warp(&bars.q_empty);                     // ... and the Q buffer refilled, once these products are done
           wait(&bars.p_ready, ph);                           // P is in tensor memory
-          if (nproc > 0) wait(&bars.o_free, ph ^ 1);         // the previous output has been read out
+          if (D != 64 && nproc > 0) wait(&bars.o_free, ph ^ 1);          // the previous output has been read out
           tc::fence_after_sync();
           const uint32_t idesc2 = tc::idesc_bf16(kPairs, D, 0, 1);
           for (int ks = 0; ks < nk16 / 16; ++ks)
