@@ -23,6 +23,9 @@ namespace cg = cooperative_groups;
 namespace muse {
 
 constexpr int kPpThreads = 256, kPpCluster = 8, kPpWarps = kPpThreads / 32;
+// Vectors of a CTA at least.  A draw costs the larger of its pass over a slice and the exchange of candidates: 1024 fp32 vectors, 8 and 16
+// start points, 101 us in one CTA, 49 in four, 44 in eight.
+constexpr int kPpSlice = 128;
 struct PpArgs { KmeansppSide s[2]; };
 
 __device__ __forceinline__ bool pp_better(float k, int i, float bk, int bi) { return k > bk || (k == bk && i < bi); }
@@ -275,11 +278,11 @@ static int kmeanspp_t(const KmeansppSide* sides, int nsides, int N, uint64_t see
   PpArgs g = {};
   int problems = 0;
   for (int k = 0; k < nsides; ++k) { g.s[k] = sides[k]; problems += sides[k].problems; }
-  // CTAs per problem: the most (up to 8, slices of at least 1024 vectors) for which all problems' clusters can be resident
+  // CTAs per problem: the most (up to 8, slices of at least kPpSlice vectors) for which all problems' clusters can be resident
   // at once.  The draws are sequential, so a cluster that has to wait for a free slot doubles the stage's time; a GPU
   // whose processor groups leave no room for every cluster of 8 does better with clusters of 7 or 6.
   int cs_max = 1;
-  while (cs_max < kPpCluster && N >= 1024 * (cs_max + 1)) ++cs_max;
+  while (cs_max < kPpCluster && N >= kPpSlice * (cs_max + 1)) ++cs_max;
   int cs = cs_max;
   for (int c = cs_max; c >= 1; --c) {
     const PpPlan<T, D> pl = pp_plan<T, D>((N + c - 1) / c);
