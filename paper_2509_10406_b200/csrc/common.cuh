@@ -163,9 +163,9 @@ inline int launch_pdl_cluster(void (*kernel)(KA...), dim3 grid, int threads, siz
   if (cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...) != cudaSuccess) { cudaGetLastError(); return MUSE_ERR_CUDA; }
   return MUSE_OK;
 }
-// Can the current device hold one thread-block cluster of this size (which a size above 8 has to be allowed for first)?
+// Thread-block clusters of this size that the current device holds at once (a size above 8 has to be allowed for first); 0: none.
 template <class... KA>
-inline bool cluster_fits(void (*kernel)(KA...), int threads, size_t smem, int cluster) {
+inline int max_clusters(void (*kernel)(KA...), int threads, size_t smem, int cluster) {
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -180,8 +180,10 @@ inline bool cluster_fits(void (*kernel)(KA...), int threads, size_t smem, int cl
                   (smem <= 48 * 1024 || cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess) &&
                   cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess;
   if (!ok) cudaGetLastError();                             // (a size that the device does not know is an answer, not an error)
-  return ok && n > 0;
+  return ok ? n : 0;
 }
+template <class... KA>
+inline bool cluster_fits(void (*kernel)(KA...), int threads, size_t smem, int cluster) { return max_clusters(kernel, threads, smem, cluster) > 0; }
 template <class... KA, class... A>
 inline int launch_pdl(void (*kernel)(KA...), dim3 grid, int threads, size_t smem, cudaStream_t st, A&&... args) {
   return launch_pdl_cluster(kernel, grid, threads, smem, 1, st, std::forward<A>(args)...);
@@ -228,7 +230,7 @@ __device__ __forceinline__ bool dbg_in_range(long long v, long long n, int line)
 // the tensor-core kernel (muse_test_force_paths; never set in production).
 enum ForcePath : unsigned {
   kForceSummFwdSimt = 1u, kForceFarSimt = 2u, kForceSummBwdSimt = 4u, kForceRetFwdStream = 8u,
-  kForceRetBwdSplit = 16u, kForceDipoleSimt = 32u, kForceBlockSelectWarp = 64u
+  kForceRetBwdSplit = 16u, kForceDipoleSimt = 32u, kForceBlockSelectWarp = 64u, kForceLloydChain = 128u
 };
 bool path_forced(unsigned bit);
 
@@ -260,6 +262,8 @@ int cluster_check(const muse_params_t* p, const void* Q, const void* K, const in
                   int32_t* assign_k, float* qbar, float* kcent, size_t ws_bytes, bool may_split, ClusterCall* c);
 int cluster_launch(ClusterCall& c, void* ws, cudaStream_t st);
 size_t lloyd_ws_bytes(const Dims& d, int problems, int C);      // scratch of one side (without the status words)
+// all iterations of small bf16 problems in one launch after the start (lloyd_small.cu); *taken: they qualified and the launch was made
+int lloyd_small(const Dims& d, const LloydSide* sides, int nsides, int T, bool* taken, int* status, cudaStream_t st);
 int assign_tc(const LloydSide* sides, int nsides, int N, int D, int distances, int* status, cudaStream_t st);
 int assign_distances(const Dims& d, int dtype, const LloydSide& side, int* status, cudaStream_t st);   // after lloyd on the same centres
 

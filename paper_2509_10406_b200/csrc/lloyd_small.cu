@@ -1,0 +1,407 @@
+// Lloyd iterations of small problems in one launch (bf16 inputs; cluster.cu has the start and, for the others, a chain of launches).  A problem (one
+// head's queries or keys) is owned by one thread-block cluster: its CTAs split the points for the assignment and the centres for the
+// update, and two cluster barriers an iteration take the place of three launches:
+//   centres     every CTA reads all centres (fp32) and lays them out as bf16 hi + lo tiles, as the assignment kernel's operands
+//   assignment  |c|^2 - 2 x.c over tiles of 128 points: points by TMA through a ring, products by tcgen05 into up to four
+//               accumulators, four warps an accumulator take the arg-min                        (same products, same order: assign_tc.cu)
+//   sort        every CTA collects the points of ITS centres in order, as 16-bit numbers in shared memory (a stable counting sort)
+//   update      two warps a centre; the fixed reduction tree of k_update, so that every bit of a centre is the chain's
+// The arrays of the assignment (centre and point tiles) and of the update (counts, lists, partial sums) share the CTA's memory.
+//
+// Bound by latency: a 128-point tile's chain (products, arg-min) 2000 cycles with four in flight, a pass over the assignments (L2),
+// a centre's rows (L2 again; from some hundred rows on the SM's rate of scattered rows, 18 to 26 bytes a clock), barriers 1000 each.
+// Three iterations, chain | here, us: 4 heads of 2k points, D = 128, 32 and 128 centres 66 | 44; 16 heads of 8k, D = 64, 64 and 128
+// 154 | 106; 12 heads of 5005, 37 and 90 96 | 63; 24 heads of 4k, 64 and 128 140 | 121 (48 problems: two CTAs each, not three);
+// 64 heads of 1k, 16 and 32 156 | 54.
+#include <cooperative_groups.h>
+#include <cuda.h>
+#include "common.cuh"
+#include "tc05.cuh"
+
+namespace cg = cooperative_groups;
+
+namespace muse {
+
+typedef __nv_bfloat16 bf16;
+int make_tmap_bf16_rows(void* out_map, const void* base, uint64_t rows, uint32_t cols, uint32_t box_rows);
+
+namespace ls {
+constexpr int kThreads = 512, kGroups = 4;                 // a group: four warps and an accumulator of 128 columns
+constexpr int kRows = 128, kMaxCentres = 256, kMaxStages = 8, kTeam = 64, kTeams = kThreads / kTeam, kMaxSegs = 1024;
+constexpr int kMaxCluster = 16, kMaxSmem = 220 * 1024;
+struct Bars { uint64_t xfull[kMaxStages], done[kGroups], read[kGroups]; };
+struct Side { const bf16* X; int32_t* assign; float *centres, *cnorm; int problems, C, kind; };
+struct Args { Side s[2]; int N, S, Bs, T, nx; };
+
+__host__ __device__ inline int segs(int C, int CL, int kind, int S) { return (C + CL - 1) / CL * (kind == 0 ? S : 1); }
+__host__ __device__ inline int centre_bytes(int C, int D) { return 2 * ((C + 127) / 128) * 128 * D * 2; }
+__host__ __device__ inline int stretch(int N) { return ((N + 15) / 16 + 31) & ~31; }   // points that a warp sorts
+// update: partial sums | counts [16][segs] | first places [segs + 1] | list | the warps' points
+__host__ __device__ inline int update_bytes(int C, int CL, int kind, int N, int S) {
+  return kTeams * 256 * 8 * 4 + 16 * segs(C, CL, kind, S) * 4 + (segs(C, CL, kind, S) + 4) / 4 * 16 + (N + 7) / 8 * 16 + 16 * stretch(N) * 4;
+}
+}  // namespace ls
+
+template <int D>
+__global__ void __launch_bounds__(ls::kThreads, 1)
+k_lloyd_small(const __grid_constant__ CUtensorMap tx0, const __grid_constant__ CUtensorMap tx1, const __grid_constant__ ls::Args g, int* __restrict__ status) {
+  using namespace ls;
+  constexpr int kTile = kRows * D * 2, G = D / 64;
+  constexpr int LPR = D / 8, SLOTS = 256 / LPR, RPT = kTeam / LPR, SG = SLOTS / RPT;   // k_update's slots; rows of a team's pass; passes
+  extern __shared__ __align__(1024) unsigned char sm_raw[];
+  __shared__ Bars bars;
+  __shared__ uint32_t tbase_s;
+  __shared__ __align__(16) float cn_s[kMaxCentres];
+  __shared__ int wsum[16];
+  __shared__ float n2_s[kTeams][4];
+  cg::cluster_group cluster = cg::this_cluster();
+  const int CL = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+  const int tid = threadIdx.x, warp = tc::warp_index(), lane = tid & 31;
+  unsigned char* sm = sm_raw + ((1024u - (tc::smem_u32(sm_raw) & 1023u)) & 1023u);
+  int prob = blockIdx.x / CL;
+  const bool second = prob >= g.s[0].problems;
+  const Side& sd = g.s[second ? 1 : 0];
+  if (second) prob -= g.s[0].problems;
+  const int N = g.N, C = sd.C, kind = sd.kind, NT = (C + 127) / 128;
+  const int tiles = (N + kRows - 1) / kRows, tper = (tiles + CL - 1) / CL, tile0 = min(tiles, rank * tper), nt = min(tiles, tile0 + tper) - tile0;
+  const int nx = nt <= g.nx ? max(nt, 1) : g.nx > 4 ? g.nx & ~3 : g.nx, ng = min(nx, kGroups);     // ring stages, working groups (a stage is always the same group's)
+  const int cper = (C + CL - 1) / CL, c0 = min(C, rank * cper), c1 = min(C, c0 + cper);
+  const bf16* Xp = sd.X + (size_t)prob * N * D;
+  int32_t* as = sd.assign + (size_t)prob * N;
+  float* cen = sd.centres + (size_t)prob * C * D;
+  float* cnp = sd.cnorm + (size_t)prob * NT * 128;
+  if (warp == 0) tc::tmem_alloc(&tbase_s, 512);
+  if (tid == 0) {
+    for (int s = 0; s < kMaxStages; ++s) tc::mbar_init(&bars.xfull[s], 1);
+    for (int b = 0; b < kGroups; ++b) { tc::mbar_init(&bars.done[b], 1); tc::mbar_init(&bars.read[b], kRows); }
+    tc::mbar_init_fence();
+  }
+  tc::fence_before_sync();
+  __syncthreads();
+  tc::fence_after_sync();
+  const uint32_t tbase = tbase_s;
+  pdl_wait();
+  pdl_trigger();
+  bool ok = true;                                          // false once a bounded wait ran out (every role still walks all its tiles)
+  auto wait = [&](uint64_t* bar, uint32_t parity) { if (ok && !tc::mbar_wait(bar, parity)) ok = false; };
+
+  int turn = 0;                                            // products of this group so far
+  for (int it = 0;; ++it) {
+    unsigned char* Xs = sm + 2 * NT * kTile;
+    auto load = [&](int i) {                               // point tile i into its stage of the ring
+      const int st_ = i % nx;
+      tc::mbar_expect_tx_warp(&bars.xfull[st_], kTile);
+#pragma unroll
+      for (int q = 0; q < G; ++q) tc::tma_load_2d_warp(Xs + st_ * kTile + q * kRows * 128, second ? &tx1 : &tx0, 64 * q, prob * N + (tile0 + i) * kRows, &bars.xfull[st_]);
+    };
+    if (warp < min(nx, nt)) load(warp);                    // (a box costs its issuer some 270 cycles: as many warps as boxes)
+    // ---- centres: bf16 hi | lo tiles of 128 rows, swizzled; rows past C (up to a multiple of 16) are zeros
+    const int rows16 = (C + 15) & ~15;
+    for (int e = tid; e < rows16 * (D / 8); e += kThreads) {
+      const int r = e / (D / 8), ck = e % (D / 8);
+      float x[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+      if (r < C) {
+        const float4 a = __ldcg(reinterpret_cast<const float4*>(cen + (size_t)r * D + 8 * ck)), b = __ldcg(reinterpret_cast<const float4*>(cen + (size_t)r * D + 8 * ck + 4));
+        x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w; x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
+      }
+      uint32_t hw[4], lw[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const __nv_bfloat162 h = __floats2bfloat162_rn(x[2 * k], x[2 * k + 1]);
+        const __nv_bfloat162 l = __floats2bfloat162_rn(x[2 * k] - __low2float(h), x[2 * k + 1] - __high2float(h));
+        hw[k] = *reinterpret_cast<const uint32_t*>(&h);
+        lw[k] = *reinterpret_cast<const uint32_t*>(&l);
+      }
+      unsigned char* dst = sm + (r >> 7) * kTile + (ck >> 3) * kRows * 128 + tc::sw128_off(r & 127, ck & 7);
+      *reinterpret_cast<uint4*>(dst) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
+      *reinterpret_cast<uint4*>(dst + NT * kTile) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
+    }
+    for (int r = tid; r < NT * 128; r += kThreads) cn_s[r] = r < C ? __ldcg(cnp + r) : INFINITY;
+    tc::fence_async_smem();                                // read by the tensor cores; what the update wrote there makes room for the points
+    __syncthreads();
+
+    // ---- assignment
+    const int grp = warp >> 2;
+    if (grp < ng) {
+      const uint64_t dx = tc::smem_desc_sw128(tc::smem_u32(Xs), 16, 1024), dc = tc::smem_desc_sw128(tc::smem_u32(sm), 16, 1024);
+      const uint32_t acc = tbase + grp * 128, tl = acc + ((uint32_t)((warp & 3) * 32) << 16);
+      const bool lead = (warp & 3) == 0;                   // issues its group's products and loads
+      for (int i = grp; i < nt; i += ng) {
+        const int st_ = i % nx, at = (tile0 + i) * kRows + (tid & 127);
+        float best[4];
+        int bidx[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) { best[e] = INFINITY; bidx[e] = 0x7fffffff; }
+        for (int t = 0; t < NT; ++t, ++turn) {
+          const int cols = min(128, rows16 - 128 * t);
+          if (lead) {
+            if (t == 0) wait(&bars.xfull[st_], (it * ((nt - st_ + nx - 1) / nx) + i / nx) & 1);
+            if (turn > 0) wait(&bars.read[grp], (turn - 1) & 1);
+            tc::fence_after_sync();
+            const uint32_t idesc = tc::idesc_bf16(kRows, cols, 0, 0);
+            const uint64_t a = tc::desc_step(dx, (uint32_t)st_ * kTile);
+#pragma unroll
+            for (int p = 0; p < 2; ++p) {                  // high parts, low parts
+              const uint64_t c = tc::desc_step(dc, (uint32_t)(p * NT + t) * kTile);
+#pragma unroll
+              for (int ks = 0; ks < D / 16; ++ks)
+                tc::mma_bf16_ss_warp(acc, tc::desc_step(a, (ks / 4) * kRows * 128 + (ks % 4) * 32), tc::desc_step(c, (ks / 4) * kRows * 128 + (ks % 4) * 32), idesc, (p | ks) != 0);
+            }
+            tc::mma_commit_warp(&bars.done[grp]);
+          }
+          wait(&bars.done[grp], turn & 1);
+          tc::fence_after_sync();
+          if (lead && t == NT - 1 && i + nx < nt && ok) load(i + nx);          // the products have read the stage
+#pragma unroll 2
+          for (int q = 0; q < cols; q += 16) {             // (rows past C: their norm is infinite)
+            float v[16];
+            tc::tmem_ld16(tl + q, v);
+#pragma unroll
+            for (int k = 0; k < 16; k += 4) {
+              const int j = 128 * t + q + k;
+              const float4 n4 = *reinterpret_cast<const float4*>(cn_s + j);
+              argmin_step(fmaf(-2.f, v[k], n4.x), j, best[0], bidx[0]);
+              argmin_step(fmaf(-2.f, v[k + 1], n4.y), j + 1, best[1], bidx[1]);
+              argmin_step(fmaf(-2.f, v[k + 2], n4.z), j + 2, best[2], bidx[2]);
+              argmin_step(fmaf(-2.f, v[k + 3], n4.w), j + 3, best[3], bidx[3]);
+            }
+          }
+          tc::fence_before_sync();
+          tc::mbar_arrive(&bars.read[grp]);
+        }
+#pragma unroll
+        for (int e = 1; e < 4; ++e) argmin_tie_step(best[e], bidx[e], best[0], bidx[0]);
+        // a row of NaN or infinities never compares below the running minimum: it goes to cluster 0
+        if (ok && at < N) as[at] = (unsigned)bidx[0] < (unsigned)C ? bidx[0] : 0;
+      }
+    }
+    if (it == g.T) break;
+    cluster.sync();                                        // every assignment of the problem has been written; the tiles have been read
+
+    {
+      // ---- sort: the points of centres [c0, c1) in order, by (centre, block) on the query side (whose update restarts at every block)
+      const int Sx = kind == 0 ? g.S : 1, nseg = cper * Sx;
+      float* part = reinterpret_cast<float*>(sm);          // [teams][SLOTS][D]
+      int* hist = reinterpret_cast<int*>(part + kTeams * SLOTS * D);                   // [16][nseg] counts of a warp's stretch, then its first place in the segment
+      int* first = hist + 16 * nseg;                       // [nseg + 1]
+      uint16_t* list = reinterpret_cast<uint16_t*>(first + (nseg + 4) / 4 * 4);        // [N] points by segment
+            for (int k = tid; k < 16 * nseg; k += kThreads) hist[k] = 0;
+      __syncthreads();
+      const int wl = stretch(N), w0 = min(N, warp * wl), w1 = min(N, w0 + wl);
+      uint32_t* own = reinterpret_cast<uint32_t*>(list + (N + 7) / 8 * 8) + warp * wl; // segment | point of this warp's stretch, this CTA's centres only
+      int* h = hist + warp * nseg;
+      const uint32_t inv_bs = 0xffffffffu / (uint32_t)g.Bs + 1u;                       // t / Bs = t * this >> 32 (exact: t * Bs < 2^32; 0: Bs = 1)
+      int no = 0;
+      for (int tb = w0; tb < w1; tb += 256) {
+        int v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = tb + 32 * u + lane < w1 ? __ldcg(as + tb + 32 * u + lane) - c0 : -1;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const bool in = (unsigned)v[u] < (unsigned)(c1 - c0);
+          const unsigned who = __ballot_sync(0xffffffffu, in);
+          if (in) {
+            const int t = tb + 32 * u + lane, k = kind == 0 ? v[u] * Sx + (inv_bs != 0u ? (int)__umulhi((uint32_t)t, inv_bs) : t) : v[u];
+            own[no + __popc(who & ((1u << lane) - 1u))] = (uint32_t)k << 16 | (uint32_t)t;
+            atomicAdd(&h[k], 1);
+          }
+          no += __popc(who);
+        }
+      }
+      __syncthreads();
+      const int per = (nseg + kThreads - 1) / kThreads, k0 = min(nseg, tid * per), k1 = min(nseg, k0 + per);
+      int mine = 0;
+      for (int k = k0; k < k1; ++k) {
+        int run = 0;
+#pragma unroll
+        for (int w = 0; w < 16; ++w) { const int x = hist[w * nseg + k]; hist[w * nseg + k] = run; run += x; }
+        first[k] = mine;
+        mine += run;
+      }
+      int inc = mine;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) { const int x = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += x; }
+      if (lane == 31) wsum[warp] = inc;
+      __syncthreads();
+      int base = inc - mine;
+#pragma unroll
+      for (int w = 0; w < 16; ++w) base += w < warp ? wsum[w] : 0;
+      for (int k = k0; k < k1; ++k) first[k] += base;
+      if (tid == kThreads - 1) first[nseg] = base + mine;
+      __syncthreads();
+      for (int e = lane; e - lane < no; e += 32) {
+        const uint32_t x = e < no ? own[e] : 0xffffffffu;
+        const int k = (int)(x >> 16);
+        const unsigned peers = __match_any_sync(0xffffffffu, k);
+        const int rk = __popc(peers & ((1u << lane) - 1u)), at = e < no ? h[k] : 0;
+        __syncwarp();
+        if (e < no) {
+          if (rk == 0) h[k] = at + __popc(peers);
+          const int p = first[k] + at + rk;
+          if (MUSE_IN_RANGE(p, N)) list[p] = (uint16_t)x;
+        }
+        __syncwarp();
+      }
+      __syncthreads();
+      // ---- update: thread = (row of a pass, 8 dims); slot s of a centre adds the members s, s + SLOTS, ... of a segment in order
+      const int team = warp >> 1, tt = tid & (kTeam - 1), sub = tt / LPR, q = tt % LPR;
+      const bf16* Xq = Xp + q * 8;
+      float* pt = part + team * SLOTS * D;
+      for (int c = c0 + team; c < c1; c += kTeams) {
+        float s[SG][8];
+#pragma unroll
+        for (int x = 0; x < SG; ++x)
+#pragma unroll
+          for (int k = 0; k < 8; ++k) s[x][k] = 0.f;
+        const int* f = first + (c - c0) * Sx;
+        const int count = f[Sx] - f[0];
+        auto load = [&](int at, int end) {                 // 8 dims of a member's row; past the segment's end zeros
+          uint4 v = make_uint4(0u, 0u, 0u, 0u);
+          if (at < end && MUSE_IN_RANGE(at, N)) v = *reinterpret_cast<const uint4*>(Xq + (size_t)list[at] * D);
+          return v;
+        };
+        auto add = [&](const uint4& v, float (&t)[8]) {
+          const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+          for (int k = 0; k < 4; ++k) { t[2 * k] += __uint_as_float(w[k] << 16); t[2 * k + 1] += __uint_as_float(w[k] & 0xffff0000u); }
+        };
+        // a step is SLOTS members of a segment or its rest; four steps at a time, whose rows are in flight together: all of them where the
+        // segments are short (half the slots at most), in two halves otherwise
+        int b = 0, p = f[0], p1 = f[1];
+        while (b < Sx) {
+          int from[4], end[4];
+          bool small = true;
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            while (b < Sx && p >= p1) { ++b; if (b < Sx) { p = f[b]; p1 = f[b + 1]; } }
+            from[i] = p; end[i] = b < Sx ? p1 : 0;
+            small = small && end[i] - p <= SLOTS / 2;
+            if (b < Sx) p += SLOTS;
+          }
+          if (small) {
+            uint4 v[4][SG / 2];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+              for (int x = 0; x < SG / 2; ++x) v[i][x] = load(from[i] + x * RPT + sub, end[i]);
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+              for (int x = 0; x < SG / 2; ++x) add(v[i][x], s[x]);
+          } else {
+#pragma unroll
+            for (int i = 0; i < 4; i += 2) {
+              uint4 v[2][SG];
+#pragma unroll
+              for (int x = 0; x < 2 * SG; ++x) v[x / SG][x % SG] = load(from[i + x / SG] + x % SG * RPT + sub, end[i + x / SG]);
+#pragma unroll
+              for (int x = 0; x < 2 * SG; ++x) add(v[x / SG][x % SG], s[x % SG]);
+            }
+          }
+        }
+#pragma unroll
+        for (int x = 0; x < SG; ++x) st8(pt + (x * RPT + sub) * D + q * 8, s[x]);
+        tc::named_bar_sync(1 + team, kTeam);
+#pragma unroll
+        for (int e = 0; e < D / kTeam; ++e) {
+          const int d = tt + e * kTeam;
+          float tot = 0.f;
+          float* dst = cen + (size_t)c * D + d;
+#pragma unroll
+          for (int k = 0; k < SLOTS; ++k) tot += pt[k * D + d];
+          if (count > 0) { tot *= 1.f / (float)count; *dst = tot; }
+          else tot = __ldcg(dst);                          // an empty cluster keeps its centre
+          const float n2 = warp_sum(tot * tot);
+          if (lane == 0) n2_s[team][2 * e + (warp & 1)] = n2;
+        }
+        tc::named_bar_sync(1 + team, kTeam);
+        if (tt == 0) {
+          float t = 0.f;
+#pragma unroll
+          for (int k = 0; k < D / 32; ++k) t += n2_s[team][k];
+          cnp[c] = t;
+        }
+      }
+    }
+    tc::fence_async_smem();
+    cluster.sync();                                        // the new centres have been written
+  }
+  if (!ok) {                                               // (copies still in flight land before the memory is released)
+    if (lane == 0) report_status(status, MUSE_STATUS_ASSIGN_TIMEOUT);
+    const long long t0 = clock64();
+    while (clock64() - t0 < (1ll << 24)) { }
+  }
+  tc::fence_before_sync();
+  __syncthreads();
+  if (warp == 0) tc::tmem_dealloc(tbase, 512);
+}
+
+// CTAs per problem: the most (up to 16, of at least one tile of points each) for which every problem's cluster is resident at once; 0
+// where the problems do not qualify.
+template <int D>
+static int lloyd_small_plan(const ls::Args& g, int nsides, size_t* smem, int* nx) {
+  using namespace ls;
+  int problems = 0, C = 0;
+  for (int k = 0; k < nsides; ++k) { problems += g.s[k].problems; C = C > g.s[k].C ? C : g.s[k].C; }
+  if (C > kMaxCentres || g.N > 16384 || problems > sm_count()) return 0;
+  const int tile = kRows * D * 2, cb = centre_bytes(C, D), tiles = cdiv(g.N, kRows);
+  int cl = sm_count() / problems;
+  if (cl >= 16 && tiles >= 16) cl = 16;
+  else if (cl > 8) cl = 8;
+  if (cl > tiles && cl > cdiv(C, 16)) cl = tiles > cdiv(C, 16) ? tiles : cdiv(C, 16);
+  for (; cl >= 1; cl = cl > 8 ? 8 : cl - 1) {
+    const int per = cdiv(tiles, cl);
+    int up = 0, seg = 0;
+    for (int k = 0; k < nsides; ++k) {
+      const int u = update_bytes(g.s[k].C, cl, g.s[k].kind, g.N, g.S), s = segs(g.s[k].C, cl, g.s[k].kind, g.S);
+      up = u > up ? u : up;
+      seg = s > seg ? s : seg;
+    }
+    *nx = (kMaxSmem - cb) / tile;
+    if (*nx > kMaxStages) *nx = kMaxStages;
+    if (*nx > per) *nx = per;
+    const size_t need = cb + (size_t)*nx * tile > (size_t)up ? cb + (size_t)*nx * tile : (size_t)up;
+    if (seg > kMaxSegs || need > (size_t)kMaxSmem || *nx < 1) return 0;      // (fewer CTAs need more)
+    *smem = need + 1024;
+    if (max_clusters(k_lloyd_small<D>, kThreads, *smem, cl) < problems) continue;
+    // The chain spreads the products over all SMs and pays for its launches, and for a problem's share of them; this kernel uses the SMs of
+    // its clusters.  Work: products of a CTA in tiles of 128 x 128 x 64; idle: the SMs without a CTA.  The line lies where most of 230
+    // sizes (1 to 64 heads of 1k to 16k points, 32 to 256 centres) cross: within it 1.1 to 2.9 times the chain's speed (a few at 0.95 to
+    // 1.05), beyond it 0.6 to 1.2: one head of 8k points, D = 128, 256 centres 77 us | 83 here; 4 heads of 16k, D = 128, 128
+    // centres 120 | 133; 24 heads of 16k, D = 64, 256 centres 454 | 495.
+    const float work = (float)per * C * D / (128 * 64), idle = 1.15f - (float)(problems * cl) / sm_count();
+    return work * idle <= 9.f + 0.6f * (problems > 16 ? problems - 16 : 0) ? cl : 0;
+  }
+  return 0;
+}
+
+template <int D>
+static int lloyd_small_d(ls::Args& g, int nsides, bool* taken, int* status, cudaStream_t st) {
+  size_t smem;
+  const int cl = lloyd_small_plan<D>(g, nsides, &smem, &g.nx);
+  if (cl == 0) return MUSE_OK;
+  *taken = true;
+  CUtensorMap m[2];
+  int problems = 0;
+  for (int k = 0; k < 2; ++k) {
+    const ls::Side& s = g.s[k < nsides ? k : 0];           // (a missing side's map is never used)
+    MUSE_RC(make_tmap_bf16_rows(&m[k], s.X, (uint64_t)s.problems * g.N, (uint32_t)D, ls::kRows));
+    if (k < nsides) problems += s.problems;
+  }
+  prof_mark("k_lloyd_small", st);
+  return launch_pdl_cluster(k_lloyd_small<D>, dim3(problems * cl), ls::kThreads, smem, cl, st, m[0], m[1], g, status);
+}
+
+int lloyd_small(const Dims& d, const LloydSide* sides, int nsides, int T, bool* taken, int* status, cudaStream_t st) {
+  *taken = false;
+  if (T < 1 || path_forced(kForceLloydChain)) return MUSE_OK;  // (the balanced assignment, T = 0, goes on to use the planes that the chain writes)
+  ls::Args g = {};
+  for (int k = 0; k < nsides; ++k) {
+    const LloydSide& s = sides[k];
+    g.s[k] = ls::Side{(const bf16*)s.X, s.assign, s.centres, s.cnorm, s.problems, s.C, s.kind};
+  }
+  g.N = d.N; g.S = d.S; g.Bs = d.Bs; g.T = T;
+  return d.D == 64 ? lloyd_small_d<64>(g, nsides, taken, status, st) : lloyd_small_d<128>(g, nsides, taken, status, st);
+}
+
+}  // namespace muse
