@@ -1,7 +1,9 @@
 // Accumulated tilted summaries on the tensor cores (bf16 mode, D = 64 or 128): Eq. 3-5 and the exclusive causal
 // accumulation of Algorithm 1 in one online-softmax walk over the buckets of a key cluster.  An item is (key cluster j, 128
 // query clusters, head); a CTA walks the planes of a contiguous range of items, so that the rows it writes and its logits'
-// query operand stay close.  A bucket comes in steps of at most 64 keys:
+// query operand stay close.  With at most 64 (32) query clusters an item is P = 2 (4) key clusters: the tile's 128 rows hold the
+// query clusters once for each of them, a step brings keys of all, and the sums of a key cluster are products of which the tensor core
+// writes only that cluster's rows.  A bucket comes in steps of at most 64 / P (D = 128: 32 / P) keys:
 //   L   = sigma qbar K^T        query clusters as bf16 hi + lo; keys and values of a step by TMA through a ring
 //   w_u = exp(l_u - base)       thread = query cluster; bf16 hi + lo over the consumed logits in tensor memory, A operands of
 //   U  += W [K | V]             accumulated in tensor memory over the whole cluster; rescaled only when a logit exceeds the
@@ -17,6 +19,8 @@
 // against 4.57).  Against one CTA per item with every phase behind a CTA barrier and accumulators in registers: 64k tokens,
 // 128 x 128 clusters, D = 64, 32 heads 1499 -> 605 us; 8k tokens, 64 x 128, 16 heads 304 -> 143; 16k, 128 x 256, 32 heads
 // 1202 -> 634; 64k, 256 x 1024, D = 128, 4 heads 1696 -> 1144; 128k, 512 x 2048 6.52 -> 4.57 ms.
+// Several key clusters per item: 16 heads of 8k, 64 x 128 140 -> 98 us; 4 heads of 2k, D = 128, 32 x 128 70 -> 45; 12 heads of 5005,
+// 37 x 90 75 -> 51; 6 heads of 9k, D = 128, 50 x 200 108 -> 76.
 #include <cuda.h>
 #include "common.cuh"
 #include "tc05.cuh"
@@ -33,10 +37,11 @@ constexpr int TI = 128;                                    // query clusters of 
 constexpr int kSnapWarps = 16, kWeightWarp0 = 16, kMmaWarp = 20, kLoadWarp = 21, kDealWarp = 22, kThreads = 23 * 32;
 constexpr int kRing = 2, kTakers = kSnapWarps + 6;           // item ranges handed out ahead; warps that take each of them
 constexpr float kLazy = 8.f, kNever = -1e30f, kLog2e = 1.4426950408889634f;
-template <int D> struct Lay {                              // shared-memory offsets and TMEM columns for head dimension D
+template <int D, int P> struct Lay {                       // shared-memory offsets and TMEM columns for head dimension D, P key clusters of an item
   static constexpr int G = D / 64;                         // 64-element (128-byte) column groups of a row
   static constexpr int NG = 128 / D;                       // groups of snapshot warps that take planes in turn (2 or 4 threads per row)
   static constexpr int NU = D == 128 ? 32 : 64, NS = D == 128 ? 3 : 4;                 // keys of a step; steps in the ring
+  static constexpr int RP = TI / P, NK = NU / P;           // rows and keys of a step of one of the item's key clusters
   static constexpr int kTile = TI * D * 2, kKeys = NU * D * 2;
   static constexpr int oQhi = 0, oQlo = kTile, oKV = 2 * kTile, oStage = oKV + NS * 2 * kKeys;   // stage: kappa hi, kappa lo, nu of a snapshot, per group
   static constexpr int total = oStage + NG * 3 * kTile + 1024;
@@ -63,14 +68,14 @@ int split_qbar(const Dims& d, const float* qbar, void* qhi, void* qlo, int* deal
   return launch_pdl(k_split_qbar, dim3((unsigned)((n + 255) / 256)), 256, 0, st, qbar, n, d.sigma, (bf16*)qhi, (bf16*)qlo, dealt);
 }
 
-template <int D>
+template <int D, int P>
 __global__ void __launch_bounds__(st::kThreads, 1)
 k_summarize_tc(Dims dm, const __grid_constant__ CUtensorMap tm_K, const __grid_constant__ CUtensorMap tm_V,
                const __grid_constant__ CUtensorMap tm_qhi, const __grid_constant__ CUtensorMap tm_qlo, const __grid_constant__ CUtensorMap tm_okhi,
                const __grid_constant__ CUtensorMap tm_oklo, const __grid_constant__ CUtensorMap tm_onu, const int32_t* __restrict__ off_k, SummPtrs sp, int per_block, int per, int* __restrict__ dealt, int* __restrict__ status) {
   using namespace st;   // per: items of a CTA, or 1: they are dealt out one by one; dealt: those dealt so far
-  typedef Lay<D> LY;
-  constexpr int G = LY::G, NG = LY::NG, NU = LY::NU, NS = LY::NS, kTile = LY::kTile, kKeys = LY::kKeys;
+  typedef Lay<D, P> LY;
+  constexpr int G = LY::G, NG = LY::NG, NU = LY::NU, NS = LY::NS, RP = LY::RP, NK = LY::NK, kTile = LY::kTile, kKeys = LY::kKeys;
   extern __shared__ __align__(1024) unsigned char sm_raw[];
   __shared__ Bars bars;
   __shared__ uint32_t tbase_s;
@@ -90,39 +95,46 @@ k_summarize_tc(Dims dm, const __grid_constant__ CUtensorMap tm_K, const __grid_c
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tbase = tbase_s;
-  const int NI = (dm.Cq + TI - 1) / TI, items = NI * dm.Ck * dm.B * dm.Hq;             // (head, tile of query clusters, key cluster), in this order
+  const int NI = (dm.Cq + TI - 1) / TI, CkP = (dm.Ck + P - 1) / P, items = NI * CkP * dm.B * dm.Hq;    // (head, tile of query clusters, P key clusters), in this order
   bool ok = true;                                          // false once a bounded wait ran out (every role then runs off the end of its items)
   auto wait = [&](uint64_t* bar, uint32_t parity) { if (ok && !tc::mbar_wait(bar, parity)) ok = false; };
-  // one plane of one item: its key cluster, tile, head, and its bucket's keys [p0, p1); taken: ranges of items so far
-  struct Plane { int it, end, taken, pl, j, i0, pq, pk, p0, p1; };
-  auto take = [&](Plane& P) {                              // the next item
-    if (++P.it < P.end) return;
-    const int r = P.taken % kRing;
-    wait(&bars.item_full[r], (P.taken / kRing) & 1);
-    P.it = ok ? item_s[r] : items;
-    P.end = min(P.it + per, items);
-    ++P.taken;
+  // one plane of one item: its first key cluster, tile, head, the first key and the number of keys of its buckets and the most keys of
+  // one; taken: ranges of items so far
+  struct Plane { int it, end, taken, pl, j, i0, pq, pk, p0[P], nk[P], n; };
+  auto take = [&](Plane& x) {                              // the next item
+    if (++x.it < x.end) return;
+    const int r = x.taken % kRing;
+    wait(&bars.item_full[r], (x.taken / kRing) & 1);
+    x.it = ok ? item_s[r] : items;
+    x.end = min(x.it + per, items);
+    ++x.taken;
     __syncwarp();
     if (lane == 0) tc::mbar_arrive(&bars.item_free[r]);
   };
-  auto place = [&](Plane& P) {
-    P.pl = 0;
-    P.j = P.it % dm.Ck;
-    P.i0 = P.it / dm.Ck % NI * TI;
-    P.pq = P.it / dm.Ck / NI;
-    P.pk = P.pq / dm.Hq * dm.Hkv + dm.hm.g[P.pq % dm.Hq];
+  auto place = [&](Plane& x) {
+    x.pl = 0;
+    x.j = x.it % CkP * P;
+    x.i0 = x.it / CkP % NI * TI;
+    x.pq = x.it / CkP / NI;
+    x.pk = x.pq / dm.Hq * dm.Hkv + dm.hm.g[x.pq % dm.Hq];
   };
-  auto advance = [&](Plane& P) {                           // the next plane (fetched one ahead of its use)
-    if (++P.pl == dm.SB) { take(P); if (P.it < items) place(P); }
-    if (P.it >= items) return;
-    const int32_t* off = off_k + (size_t)P.pk * (dm.Ck * dm.S + 1) + (size_t)P.j * dm.S + P.pl;
-    P.p0 = __ldg(off);
-    P.p1 = __ldg(off + 1);
-    (void)MUSE_IN_RANGE(P.p1, dm.N + 1); (void)MUSE_IN_RANGE(P.p0, P.p1 + 1);          // (the tiles come through tensor maps, which clip)
+  auto advance = [&](Plane& x) {                           // the next plane (fetched one ahead of its use)
+    if (++x.pl == dm.SB) { take(x); if (x.it < items) place(x); }
+    if (x.it >= items) return;
+    const int32_t* off = off_k + (size_t)x.pk * (dm.Ck * dm.S + 1) + (size_t)x.j * dm.S + x.pl;
+    x.n = 0;
+#pragma unroll
+    for (int c = 0; c < P; ++c) {
+      const bool in = P == 1 || x.j + c < dm.Ck;           // (the last item of a tile may hold fewer key clusters)
+      x.p0[c] = in ? __ldg(off + c * dm.S) : 0;
+      x.nk[c] = in ? __ldg(off + c * dm.S + 1) - x.p0[c] : 0;
+      x.n = max(x.n, x.nk[c]);
+      (void)MUSE_IN_RANGE(x.nk[c], dm.N + 1); (void)MUSE_IN_RANGE(x.p0[c], dm.N + 1);    // (the tiles come through tensor maps, which clip)
+    }
   };
   struct Walk { Plane cur, nxt; };
   auto start = [&](Walk& w) {
-    w.cur = Plane{-1, 0, 0, dm.SB - 1, 0, 0, 0, 0, 0, 0};
+    w.cur = Plane{-1, 0, 0, dm.SB - 1};
     advance(w.cur);
     w.nxt = w.cur;
     if (w.nxt.it < items) advance(w.nxt);
@@ -144,46 +156,54 @@ k_summarize_tc(Dims dm, const __grid_constant__ CUtensorMap tm_K, const __grid_c
     start(w);
     int n = 0, nq = 0, tile = -1;
     for (; w.cur.it < items; next(w)) {
-      if (w.cur.pl == 0 && w.cur.it / dm.Ck != tile) {        // another tile of query clusters
-        tile = w.cur.it / dm.Ck;
+      if (w.cur.pl == 0 && w.cur.it / CkP != tile) {          // another tile of query clusters
+        tile = w.cur.it / CkP;
         if (nq > 0) wait(&bars.q_free, (nq - 1) & 1);
         ++nq;
         if (ok) {
           tc::mbar_expect_tx_warp(&bars.q_full, 2 * LY::kTile);
           const int r = w.cur.pq * dm.Cq + w.cur.i0;
-          for (int g = 0; g < G; ++g) {
-            tc::tma_load_2d_warp(sm + LY::oQhi + g * TI * 128, &tm_qhi, 64 * g, r, &bars.q_full);
-            tc::tma_load_2d_warp(sm + LY::oQlo + g * TI * 128, &tm_qlo, 64 * g, r, &bars.q_full);
-          }
+          for (int g = 0; g < G; ++g)
+            for (int c = 0; c < P; ++c) {                  // (the same query clusters for each of the item's key clusters)
+              tc::tma_load_2d_warp(sm + LY::oQhi + (g * TI + c * RP) * 128, &tm_qhi, 64 * g, r, &bars.q_full);
+              tc::tma_load_2d_warp(sm + LY::oQlo + (g * TI + c * RP) * 128, &tm_qlo, 64 * g, r, &bars.q_full);
+            }
         }
       }
-      for (int c0 = w.cur.p0; c0 < w.cur.p1; c0 += NU, ++n) {
-        const int s = n % NS, ng = (min(NU, w.cur.p1 - c0) + 15) >> 4;   // a bucket often holds far fewer than 64 keys: only the 16-key groups in use
+      for (int c0 = 0; c0 < w.cur.n; c0 += NK, ++n) {
+        const int s = n % NS;                              // a bucket often holds far fewer keys than a step: only the 16-key groups in use
+        int all = 0;
+#pragma unroll
+        for (int c = 0; c < P; ++c) all += (max(0, min(NK, w.cur.nk[c] - c0)) + 15) >> 4;
         wait(&bars.kv_empty[s], ((n / NS) & 1) ^ 1);
         if (!ok) continue;
-        tc::mbar_expect_tx_warp(&bars.kv_full[s], ng * 2 * G * (16 * 128));
-        const int r = w.cur.pk * dm.N + c0;
-        unsigned char* kv = sm + LY::oKV + s * 2 * kKeys;
-        for (int g = 0; g < ng; ++g)
-          for (int cg = 0; cg < G; ++cg) {
-            tc::tma_load_2d_warp(kv + cg * NU * 128 + g * 16 * 128, &tm_K, 64 * cg, r + 16 * g, &bars.kv_full[s]);
-            tc::tma_load_2d_warp(kv + kKeys + cg * NU * 128 + g * 16 * 128, &tm_V, 64 * cg, r + 16 * g, &bars.kv_full[s]);
-          }
+        tc::mbar_expect_tx_warp(&bars.kv_full[s], all * 2 * G * (16 * 128));
+#pragma unroll
+        for (int c = 0; c < P; ++c) {
+          const int r = w.cur.pk * dm.N + w.cur.p0[c] + c0, ng = (max(0, min(NK, w.cur.nk[c] - c0)) + 15) >> 4;
+          unsigned char* kv = sm + LY::oKV + s * 2 * kKeys + c * NK * 128;
+          for (int g = 0; g < ng; ++g)
+            for (int cg = 0; cg < G; ++cg) {
+              tc::tma_load_2d_warp(kv + cg * NU * 128 + g * 16 * 128, &tm_K, 64 * cg, r + 16 * g, &bars.kv_full[s]);
+              tc::tma_load_2d_warp(kv + kKeys + cg * NU * 128 + g * 16 * 128, &tm_V, 64 * cg, r + 16 * g, &bars.kv_full[s]);
+            }
+        }
       }
     }
   } else if (warp == kMmaWarp) {                           // ---- products
     const uint64_t dqh = tc::smem_desc_sw128(tc::smem_u32(sm + LY::oQhi), 16, 1024), dql = tc::smem_desc_sw128(tc::smem_u32(sm + LY::oQlo), 16, 1024),
                    dk = tc::smem_desc_sw128(tc::smem_u32(sm + LY::oKV), 16, 1024), dn = tc::smem_desc_sw128(tc::smem_u32(sm + LY::oKV), NU * 128, 1024);
     int el = 0, nq = 0, tile = -1;                         // non-empty steps whose logits have been issued, tiles so far
-    auto issue_l = [&](int it, int pl, int c, int p1) {    // the logits of the step that starts at key c of a bucket that ends at p1
-      if (pl == 0 && it / dm.Ck != tile) {
-        tile = it / dm.Ck;
+    auto issue_l = [&](int it, int pl, int c, int n) {     // the logits of the step that starts at key c of buckets of at most n keys
+      if (pl == 0 && it / CkP != tile) {
+        tile = it / CkP;
         if (nq > 0) tc::mma_commit_warp(&bars.q_free);
         wait(&bars.q_full, nq & 1);
         ++nq;
       }
-      if (c >= p1) return;
-      const int s = el % NS, ng = (min(NU, p1 - c) + 15) >> 4;
+      if (c >= n) return;
+      // (P > 1: all columns; what rows or columns of other key clusters or without keys make of it nobody reads)
+      const int s = el % NS, ng = P > 1 ? NU / 16 : (min(NU, n - c) + 15) >> 4;
       wait(&bars.kv_full[s], (el / NS) & 1);
       tc::fence_after_sync();
       const uint32_t idesc = tc::idesc_bf16(TI, 16 * ng, 0, 0), tl = tbase + LY::cL + (el & 1) * NU;
@@ -201,36 +221,56 @@ k_summarize_tc(Dims dm, const __grid_constant__ CUtensorMap tm_K, const __grid_c
     Walk w;
     start(w);
     int n = -1, e = 0, k = 0;                              // steps (-1: only the first step's logits), non-empty steps, snapshots
-    bool acc_in = false, held = false;                     // held: snapshot k - 1 has not been waited for
-    int c0 = w.cur.p0;
+    uint32_t acc_in = 0;                                   // key clusters whose accumulators hold something
+    bool held = false;                                     // snapshot k - 1 has not been waited for
+    int c0 = 0;
     while (w.cur.it < items) {
       // the next step's logits, before this step's sums (an empty bucket is one step without keys)
-      const bool same = n < 0 || c0 + NU < w.cur.p1;
-      const int cn = n < 0 ? c0 : same ? c0 + NU : w.nxt.p0;
-      if (same || w.nxt.it < items) issue_l(same ? w.cur.it : w.nxt.it, same ? w.cur.pl : w.nxt.pl, cn, same ? w.cur.p1 : w.nxt.p1);
+      const bool same = n < 0 || c0 + NK < w.cur.n;
+      const int cn = n >= 0 && same ? c0 + NK : 0;
+      if (same || w.nxt.it < items) issue_l(same ? w.cur.it : w.nxt.it, same ? w.cur.pl : w.nxt.pl, cn, same ? w.cur.n : w.nxt.n);
       if (n < 0) { n = 0; continue; }
-      const int nk = min(NU, w.cur.p1 - c0);
-      if (c0 == w.cur.p0 && (w.cur.pl == 0 || per_block)) acc_in = false;
+      if (c0 == 0 && (w.cur.pl == 0 || per_block)) acc_in = 0;
       wait(&bars.w_ready, n & 1);
       ++n;
-      if (nk > 0) {
+      if (w.cur.n > c0) {
         if (held) { wait(&bars.acc_free[(k - 1) % NG], ((k - 1) / NG) & 1); held = false; }
         tc::fence_after_sync();
-        const int s = e % NS, ng = (nk + 15) >> 4;
-        const uint32_t hi = tbase + LY::cL + (e & 1) * NU, lo = tbase + LY::cLo + (e & 1) * (NU / 2);
-        const uint64_t x = tc::desc_step(dn, (uint32_t)s * 2 * kKeys), y = tc::desc_step(x, kKeys);
+        const int s = e % NS;
+#pragma unroll
+        for (int c = 0; c < P; ++c) {
+          const int ng = (max(0, min(NK, w.cur.nk[c] - c0)) + 15) >> 4;
+          const uint32_t hi = tbase + LY::cL + (e & 1) * NU + c * NK, lo = tbase + LY::cLo + (e & 1) * (NU / 2) + c * (NK / 2);
+          const uint64_t x = tc::desc_step(dn, (uint32_t)s * 2 * kKeys + c * NK * 128), y = tc::desc_step(x, kKeys);
+          const uint32_t in = (acc_in >> c) & 1u;
+          if constexpr (P == 1) {
 #pragma unroll 1
-        for (int ks = 0; ks < ng; ++ks) {
-          tc::mma_bf16_ts_warp(tbase + LY::cUk, hi + 8 * ks, tc::desc_step(x, ks * 16 * 128), idesc, acc_in || ks > 0);
-          tc::mma_bf16_ts_warp(tbase + LY::cUv, hi + 8 * ks, tc::desc_step(y, ks * 16 * 128), idesc, acc_in || ks > 0);
-          tc::mma_bf16_ts_warp(tbase + LY::cUk, lo + 8 * ks, tc::desc_step(x, ks * 16 * 128), idesc, 1);
-          tc::mma_bf16_ts_warp(tbase + LY::cUv, lo + 8 * ks, tc::desc_step(y, ks * 16 * 128), idesc, 1);
+            for (int ks = 0; ks < ng; ++ks) {
+              tc::mma_bf16_ts_warp(tbase + LY::cUk, hi + 8 * ks, tc::desc_step(x, ks * 16 * 128), idesc, in || ks > 0);
+              tc::mma_bf16_ts_warp(tbase + LY::cUv, hi + 8 * ks, tc::desc_step(y, ks * 16 * 128), idesc, in || ks > 0);
+              tc::mma_bf16_ts_warp(tbase + LY::cUk, lo + 8 * ks, tc::desc_step(x, ks * 16 * 128), idesc, 1);
+              tc::mma_bf16_ts_warp(tbase + LY::cUv, lo + 8 * ks, tc::desc_step(y, ks * 16 * 128), idesc, 1);
+            }
+          } else {
+            // only the rows of key cluster c are written: the weights of the others' columns need not be there, and nothing of one
+            // cluster's keys reaches another's sums
+            uint32_t off[4];
+#pragma unroll
+            for (int w4 = 0; w4 < 4; ++w4) off[w4] = w4 / (4 / P) == c ? 0u : 0xffffffffu;
+#pragma unroll 1
+            for (int ks = 0; ks < ng; ++ks) {
+              tc::mma_bf16_ts_rows_warp(tbase + LY::cUk, hi + 8 * ks, tc::desc_step(x, ks * 16 * 128), idesc, off, in || ks > 0);
+              tc::mma_bf16_ts_rows_warp(tbase + LY::cUv, hi + 8 * ks, tc::desc_step(y, ks * 16 * 128), idesc, off, in || ks > 0);
+              tc::mma_bf16_ts_rows_warp(tbase + LY::cUk, lo + 8 * ks, tc::desc_step(x, ks * 16 * 128), idesc, off, 1);
+              tc::mma_bf16_ts_rows_warp(tbase + LY::cUv, lo + 8 * ks, tc::desc_step(y, ks * 16 * 128), idesc, off, 1);
+            }
+          }
+          if (ng > 0) acc_in |= 1u << c;
         }
-        acc_in = true;
         tc::mma_commit_warp(&bars.kv_empty[s]);
         ++e;
       }
-      const bool last = !(c0 + NU < w.cur.p1);
+      const bool last = !(c0 + NK < w.cur.n);
       if (last) {
         if (held) wait(&bars.acc_free[(k - 1) % NG], ((k - 1) / NG) & 1);              // (a wait never skips a phase)
         tc::mma_commit_warp(&bars.u_done[k % NG]);
@@ -238,13 +278,13 @@ k_summarize_tc(Dims dm, const __grid_constant__ CUtensorMap tm_K, const __grid_c
         held = true;
       }
       tc::mma_commit_warp(&bars.u_step);
-      c0 += NU;
-      if (last) { next(w); c0 = w.cur.p0; }
+      c0 += NK;
+      if (last) { next(w); c0 = 0; }
     }
     if (held) wait(&bars.acc_free[(k - 1) % NG], ((k - 1) / NG) & 1);
     if (n > 0) wait(&bars.u_step, (n - 1) & 1);
   } else if (warp >= kWeightWarp0) {                       // ---- weights: thread = query cluster
-    const int row = tid - kWeightWarp0 * 32;
+    const int row = tid - kWeightWarp0 * 32, sub = P == 1 ? 0 : (warp & 3) / (4 / P);  // sub: the row's key cluster (the same for a warp)
     const uint32_t tl = tbase + ((uint32_t)((warp & 3) * 32) << 16);
     Walk w;
     start(w);
@@ -252,14 +292,17 @@ k_summarize_tc(Dims dm, const __grid_constant__ CUtensorMap tm_K, const __grid_c
     float base = -INFINITY, s = 0.f, T = 0.f;              // (log2 units) mass and sum of w * logit, relative to the base
     for (; w.cur.it < items; next(w)) {
       if (w.cur.pl == 0 || per_block) { base = -INFINITY; s = 0.f; T = 0.f; }
-      int c0 = w.cur.p0;
+      int mine = w.cur.nk[0];                              // keys of the row's bucket
+#pragma unroll
+      for (int c = 1; c < P; ++c) mine = sub == c ? w.cur.nk[c] : mine;
+      int c0 = 0;
       do {
-        const int nk = min(NU, w.cur.p1 - c0), ng = nk > 0 ? (nk + 15) >> 4 : 0;
+        const int nk = min(NK, mine - c0), ng = nk > 0 ? (nk + 15) >> 4 : 0;
         bool stepped = n == 0;                             // the previous step's products have been waited for
+        if (w.cur.n > c0) wait(&bars.l_full[e & 1], (e >> 1) & 1);
         if (nk > 0) {
-          wait(&bars.l_full[e & 1], (e >> 1) & 1);
           tc::fence_after_sync();
-          const uint32_t tL = tl + LY::cL + (e & 1) * NU, tLo = tl + LY::cLo + (e & 1) * (NU / 2);
+          const uint32_t tL = tl + LY::cL + (e & 1) * NU + sub * NK, tLo = tl + LY::cLo + (e & 1) * (NU / 2) + sub * (NK / 2);
           // two sweeps over the logits in tensor memory (maximum, then weights); columns past the bucket's keys count as kNever
           auto mask = [&](float (&v)[16], int g) {
             if (16 * g + 16 > nk) {
@@ -320,16 +363,16 @@ k_summarize_tc(Dims dm, const __grid_constant__ CUtensorMap tm_K, const __grid_c
             tc::tmem_st8_issue(tLo + 8 * g, lw);
           }
           s += ws[0] + ws[1]; T += wl[0] + wl[1];
-          ++e;
         }
-        c0 += NU;
-        if (c0 >= w.cur.p1) { base_s[k & 3][row] = base; s_s[k & 3][row] = s; T_s[k & 3][row] = T; ++k; }
+        if (w.cur.n > c0) ++e;
+        c0 += NK;
+        if (c0 >= w.cur.n) { base_s[k & 3][row] = base; s_s[k & 3][row] = s; T_s[k & 3][row] = T; ++k; }
         if (!stepped) wait(&bars.u_step, (n - 1) & 1);     // (no more than one step ahead of the products)
         tc::tmem_st_wait();
         tc::fence_before_sync();
         tc::mbar_arrive(&bars.w_ready);
         ++n;
-      } while (c0 < w.cur.p1);
+      } while (c0 < w.cur.n);
     }
   } else {                                                 // ---- snapshots: thread = (query cluster, 32 dims of kappa and of nu)
     const int row = (warp & 3) * 32 + lane, part = (warp >> 2) & (D / 32 - 1), grp = NG == 2 ? warp >> 3 : 0;
@@ -337,10 +380,10 @@ k_summarize_tc(Dims dm, const __grid_constant__ CUtensorMap tm_K, const __grid_c
     constexpr int kGroup = kSnapWarps * 32 / NG;
     const bool lead = warp == grp * (kSnapWarps / NG);
     int k = 0;
-    Plane P{-1, 0, 0, 0, 0, 0, 0, 0, 0, 0};
-    for (take(P); P.it < items; take(P)) {
-      place(P);
-      const int j = P.j, i = P.i0 + row, pq = P.pq;
+    Plane x{-1};
+    for (take(x); x.it < items; take(x)) {
+      place(x);
+      const int j = x.j + row / RP, i = x.i0 + row % RP, pq = x.pq;
       for (int pl = 0; pl < dm.SB; ++pl, ++k) {
         if (k % NG != grp) continue;
         wait(&bars.u_done[grp], (k / NG) & 1);
@@ -369,7 +412,7 @@ k_summarize_tc(Dims dm, const __grid_constant__ CUtensorMap tm_K, const __grid_c
           const __nv_bfloat162 nb = __floats2bfloat162_rn(inv > 0.f ? v[u] * inv : 0.f, inv > 0.f ? v[u + 1] * inv : 0.f);
           nw[u / 2] = *reinterpret_cast<const uint32_t*>(&nb);
         }
-        if (part == 0 && i < dm.Cq && ok) {
+        if (part == 0 && i < dm.Cq && (P == 1 || j < dm.Ck) && ok) {
           const size_t ent = (((size_t)pq * dm.SB + pl) * dm.Cq + i) * dm.Ck + j;
           const float m_ = mass > 0.f ? (base + log2f(mass)) * 0.6931471805599453f : -INFINITY;
           sp.mu[ent] = m_;
@@ -388,8 +431,8 @@ k_summarize_tc(Dims dm, const __grid_constant__ CUtensorMap tm_K, const __grid_c
 #pragma unroll
           for (int c = 0; c < 4; ++c) {
             const int ch = 4 * part + c;                   // 16-byte chunk of the row
-            const uint32_t* x = a == 0 ? hw : a == 1 ? lw : nw;
-            *reinterpret_cast<uint4*>(stage + a * kTile + (ch >> 3) * TI * 128 + tc::sw128_off(row, ch & 7)) = make_uint4(x[4 * c], x[4 * c + 1], x[4 * c + 2], x[4 * c + 3]);
+            const uint32_t* o = a == 0 ? hw : a == 1 ? lw : nw;
+            *reinterpret_cast<uint4*>(stage + a * kTile + (ch >> 3) * TI * 128 + tc::sw128_off(row, ch & 7)) = make_uint4(o[4 * c], o[4 * c + 1], o[4 * c + 2], o[4 * c + 3]);
           }
         }
         tc::fence_async_smem();
@@ -399,7 +442,10 @@ k_summarize_tc(Dims dm, const __grid_constant__ CUtensorMap tm_K, const __grid_c
           for (int a = 0; a < 3; ++a) {
             const void* map = a == 0 ? (const void*)&tm_okhi : a == 1 ? (const void*)&tm_oklo : (const void*)&tm_onu;
 #pragma unroll
-            for (int g = 0; g < G; ++g) tc::tma_store_4d_warp(map, stage + a * kTile + g * TI * 128, 64 * g, j, P.i0, pq * dm.SB + pl);
+            for (int g = 0; g < G; ++g)
+#pragma unroll
+              for (int c = 0; c < P; ++c)
+                if (P == 1 || x.j + c < dm.Ck) tc::tma_store_4d_warp(map, stage + a * kTile + (g * TI + c * RP) * 128, 64 * g, x.j + c, x.i0, pq * dm.SB + pl);
           }
           tc::tma_store_commit_warp();
         }
@@ -415,39 +461,49 @@ k_summarize_tc(Dims dm, const __grid_constant__ CUtensorMap tm_K, const __grid_c
 
 bool summarize_tc_supported(const Dims& d, int dtype) { return dtype == MUSE_BF16 && (d.D == 64 || d.D == 128); }
 
+template <int D, int P>
+static int summarize_tc_p(const Dims& d, const void* Kp, const void* Vp, const int32_t* off_k, const bf16* qhi, const bf16* qlo, const SummPtrs& sp,
+                          int per_block, int* status, cudaStream_t stream) {
+  constexpr int RP = st::Lay<D, P>::RP;
+  CUtensorMap tqh, tql, tK, tV, okhi, oklo, onu;
+  MUSE_RC(make_tmap_bf16_rows(&tqh, qhi, (uint64_t)d.B * d.Hq * d.Cq, D, RP));
+  MUSE_RC(make_tmap_bf16_rows(&tql, qlo, (uint64_t)d.B * d.Hq * d.Cq, D, RP));
+  MUSE_RC(make_tmap_bf16_rows(&tK, Kp, (uint64_t)d.B * d.Hkv * d.N, D, 16));           // boxes of 16 keys
+  MUSE_RC(make_tmap_bf16_rows(&tV, Vp, (uint64_t)d.B * d.Hkv * d.N, D, 16));
+  prof_mark("k_summarize_tc", stream);
+  // outputs as 4-D tensors (d, j, i, head * planes + plane); a box is the query clusters that an item holds of one key cluster
+  const uint64_t dims[4] = {(uint64_t)D, (uint64_t)d.Ck, (uint64_t)d.Cq, (uint64_t)d.B * d.Hq * d.SB};
+  const uint64_t strides[3] = {(uint64_t)D * 2, (uint64_t)d.Ck * D * 2, (uint64_t)d.Cq * d.Ck * D * 2};
+  const uint32_t box[4] = {64, 1, (uint32_t)RP, 1};
+  MUSE_RC(make_tmap_bf16_nd(&okhi, sp.khi, 4, dims, strides, box));
+  MUSE_RC(make_tmap_bf16_nd(&oklo, sp.klo, 4, dims, strides, box));
+  MUSE_RC(make_tmap_bf16_nd(&onu, sp.nu, 4, dims, strides, box));
+  const int groups = cdiv(d.Ck, P);                        // of key clusters, items of a tile
+  const long long items = (long long)groups * cdiv(d.Cq, st::TI) * d.B * d.Hq;
+  const int grid = (int)(items < sm_count() ? items : sm_count());
+  // With many key clusters per tile the items are dealt out one by one, in order: all CTAs then write neighbouring rows at a time,
+  // which is what DRAM wants (128k tokens, 512 x 2048 clusters, 22 GB of summaries: 9.1 ms in one range per CTA, 6.3 dealt).
+  // With few, every item would change the tile.
+  const int per = groups >= grid ? 1 : (int)((items + grid - 1) / grid);
+  return launch_pdl(k_summarize_tc<D, P>, dim3(grid), st::kThreads, st::Lay<D, P>::total, stream, d, tK, tV, tqh, tql, okhi, oklo, onu, off_k, sp, per_block, per,
+                    status + kItemWord, status);
+}
+
 int summarize_tc(const Dims& d, const void* Kp, const void* Vp, const int32_t* off_k, const float* qbar, const SummPtrs& sp,
                  int per_block, void* qsplit, int* status, cudaStream_t stream) {
   // qsplit: 2 * B*Hq*Cq*D bf16 of scratch for the split centroids
   bf16* qhi = (bf16*)qsplit;
   bf16* qlo = qhi + (size_t)d.B * d.Hq * d.Cq * d.D;
-  int rcq = split_qbar(d, qbar, qhi, qlo, status + kItemWord, stream);
-  if (rcq != MUSE_OK) return rcq;
-  CUtensorMap tqh, tql;
-  rcq = make_tmap_bf16_rows(&tqh, qhi, (uint64_t)d.B * d.Hq * d.Cq, d.D, st::TI);
-  if (rcq == MUSE_OK) rcq = make_tmap_bf16_rows(&tql, qlo, (uint64_t)d.B * d.Hq * d.Cq, d.D, st::TI);
-  if (rcq != MUSE_OK) return rcq;
-  CUtensorMap tK, tV;
-  int rc = make_tmap_bf16_rows(&tK, Kp, (uint64_t)d.B * d.Hkv * d.N, d.D, 16);       // boxes of 16 keys
-  if (rc == MUSE_OK) rc = make_tmap_bf16_rows(&tV, Vp, (uint64_t)d.B * d.Hkv * d.N, d.D, 16);
-  if (rc != MUSE_OK) return rc;
-  prof_mark("k_summarize_tc", stream);
-  // outputs as 4-D tensors (d, j, i, head * planes + plane); a box is 128 query clusters of one key cluster
-  CUtensorMap okhi, oklo, onu;
-  const uint64_t dims[4] = {(uint64_t)d.D, (uint64_t)d.Ck, (uint64_t)d.Cq, (uint64_t)d.B * d.Hq * d.SB};
-  const uint64_t strides[3] = {(uint64_t)d.D * 2, (uint64_t)d.Ck * d.D * 2, (uint64_t)d.Cq * d.Ck * d.D * 2};
-  const uint32_t box[4] = {64, 1, (uint32_t)st::TI, 1};
-  MUSE_RC(make_tmap_bf16_nd(&okhi, sp.khi, 4, dims, strides, box));
-  MUSE_RC(make_tmap_bf16_nd(&oklo, sp.klo, 4, dims, strides, box));
-  MUSE_RC(make_tmap_bf16_nd(&onu, sp.nu, 4, dims, strides, box));
-  const long long items = (long long)d.Ck * cdiv(d.Cq, st::TI) * d.B * d.Hq;
-  const int grid = (int)(items < sm_count() ? items : sm_count());
-  // With many key clusters per tile the items are dealt out one by one, in order: all CTAs then write neighbouring rows at a time,
-  // which is what DRAM wants (128k tokens, 512 x 2048 clusters, 22 GB of summaries: 9.1 ms in one range per CTA, 6.3 dealt).
-  // With few, every item would change the tile.
-  const int per = d.Ck >= grid ? 1 : (int)((items + grid - 1) / grid);
-  int* dealt = status + kItemWord;
-  if (d.D == 128) return launch_pdl(k_summarize_tc<128>, dim3(grid), st::kThreads, st::Lay<128>::total, stream, d, tK, tV, tqh, tql, okhi, oklo, onu, off_k, sp, per_block, per, dealt, status);
-  return launch_pdl(k_summarize_tc<64>, dim3(grid), st::kThreads, st::Lay<64>::total, stream, d, tK, tV, tqh, tql, okhi, oklo, onu, off_k, sp, per_block, per, dealt, status);
+  MUSE_RC(split_qbar(d, qbar, qhi, qlo, status + kItemWord, stream));
+  // Few query clusters: a tile's 128 rows take them two or four times over, for as many key clusters (one with fewer key clusters would
+  // have rows without work).
+  const int P = d.D == 64 && d.Cq <= 32 && d.Ck >= 4 ? 4 : d.Cq <= 64 && d.Ck >= 2 ? 2 : 1;      // (D = 128: no room for four clusters' keys)
+#define MUSE_ST(DD, PP) return summarize_tc_p<DD, PP>(d, Kp, Vp, off_k, qhi, qlo, sp, per_block, status, stream)
+  if (d.D == 128) { if (P > 1) MUSE_ST(128, 2); MUSE_ST(128, 1); }
+  if (P == 4) MUSE_ST(64, 4);
+  if (P == 2) MUSE_ST(64, 2);
+  MUSE_ST(64, 1);
+#undef MUSE_ST
 }
 
 }  // namespace muse

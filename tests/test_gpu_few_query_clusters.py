@@ -1,0 +1,52 @@
+"""GPU: summaries and key-side pass where a tile's 128 rows hold few query clusters two or four times over (for as many key clusters,
+or planes): query clusters around 32 and 64, key clusters and planes that two and four do not divide, buckets of none to several steps of
+keys, against the library's FFMA kernels.  Summaries: kappa is kept as bf16 hi + lo (2^-17 of its size) and mu to fp32, so 1e-4 as in
+the oracle's test; nu, dK and dV are bf16 numbers whose weights are rounded to bf16 on one side: two roundings, 2^-7 of the scale."""
+import numpy as np
+import pytest
+import torch
+
+from tests.gpu_util import rel_err, to_np
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("D,Cq,Ck,S,N,causal", [
+    (64, 1, 2, 2, 600, True), (64, 31, 5, 4, 1000, True), (64, 32, 4, 8, 2048, True), (64, 33, 3, 3, 999, True), (64, 64, 7, 6, 1500, True), (64, 32, 9, 33, 1056, True),
+    (64, 64, 40, 1, 900, False), (128, 8, 3, 3, 900, True), (128, 32, 6, 5, 1000, True), (128, 50, 2, 8, 1600, True), (128, 64, 5, 2, 800, True), (128, 20, 10, 34, 1020, True)])
+def test_packed_tiles_match_the_ffma_kernels(D, Cq, Ck, S, N, causal):
+    from paper_2509_10406_b200 import binding as mb
+    from tests.gpu_util import kernels_launched
+    B, Hq, Hkv = 1, 4, 2
+    g = torch.Generator(device="cuda").manual_seed(N + Cq)
+    e = lambda h, n: torch.randn(B, h, n, D, generator=g, device="cuda")  # noqa: E731
+    Q, K, V, dO = (e(h, N).to(torch.bfloat16) for h in (Hq, Hkv, Hkv, Hq))
+    p = mb.make_params(B=B, Hq=Hq, Hkv=Hkv, N=N, D=D, Cq=Cq, Ck=Ck, m=1, n_blocks=S, causal=causal)
+    rng = np.random.default_rng(N)
+    a = np.minimum(rng.integers(0, Ck, (B, Hkv, N)), rng.integers(0, Ck, (B, Hkv, N))).astype(np.int32)    # uneven, some buckets empty
+    a_k = torch.from_numpy(a).cuda()
+    a_q = torch.randint(0, Cq, (B, Hq, N), generator=g, device="cuda", dtype=torch.int32)
+    qbar = 0.7 * e(Hq, Cq)
+    got = []
+    for mask in (1 | 4, 0):
+        buf = mb.MuseBuffers(p, backward=True)
+        mb.muse_test_force_paths(mask)
+        try:
+            with kernels_launched() as k:
+                mb.muse_summarize(p, K, V, a_k, qbar, buf.off_k, buf.perm_k, buf.summaries, buf.ws)
+                mb.muse_attn_fwd(p, Q, K, V, a_q, qbar, buf.off_k, buf.perm_k, buf.summaries, got[0][1] if got else None, buf.O, buf.LSE, buf.sel, buf.ws)
+                mb.muse_attn_bwd(p, Q, K, V, buf.O, buf.LSE, dO, a_q, qbar, buf.off_k, buf.perm_k, buf.summaries, buf.sel, buf.dQ, buf.dK, buf.dV, buf.ws)
+        finally:
+            mb.muse_test_force_paths(0)
+        assert {"k_summarize_tc", "k_summ_bwd_tc"} <= set(k.names) if mask == 0 else not {"k_summarize_tc", "k_summ_bwd_tc"} & set(k.names)
+        got.append(([to_np(x) for x in buf.summary_planes()], buf.sel.clone(), to_np(buf.dK), to_np(buf.dV)))
+    (mu0, be0, ka0, nu0), sel0, dk0, dv0 = got[0]
+    (mu1, be1, ka1, nu1), sel1, dk1, dv1 = got[1]
+    assert np.array_equal(np.isfinite(mu0), np.isfinite(mu1)) and np.array_equal(np.isfinite(be0), np.isfinite(be1))
+    fin = np.isfinite(mu0)
+    for x, y in ((mu0, mu1), (be0, be1)):
+        assert np.abs(x[fin] - y[fin]).max() <= 1e-4 * max(1.0, np.abs(x[fin]).max())
+    assert rel_err(ka1, ka0) <= 1e-4
+    assert rel_err(nu1, nu0) <= 2.0 ** -7
+    assert torch.equal(sel0, sel1)
+    assert rel_err(dk1, dk0) <= 2.0 ** -7 and rel_err(dv1, dv0) <= 2.0 ** -7
