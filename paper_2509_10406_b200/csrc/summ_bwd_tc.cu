@@ -18,7 +18,8 @@
 // nothing spills, which matters because the tiles leave next to no L1 cache (spilled words, and the bucket offsets that are now
 // in shared memory, came from L2 on every plane: 2000 cycles).  32 heads of 64k tokens, 128 x 128 clusters, D = 64 2485 ->
 // 1682 us; 32 heads of 16k, 128 x 256 1222 -> 771; 16 heads of 8k, 64 x 128 322 -> 209; 4 heads of 64k, D = 128, 256 x 1024
-// 1280 -> 1201.
+// 1280 -> 1201.  Two planes a step with at most 64 query clusters: 16 heads of 8k, 64 x 128, 7 planes 209 -> 168 us; 6 heads of 9k,
+// D = 128, 50 x 200, 5 planes 153 -> 121; four with at most 32: 10 heads of 1k, D = 128, 8 x 128, 3 planes 92 -> 71.
 #include <cuda.h>
 #include "common.cuh"
 #include "tc05.cuh"
@@ -46,7 +47,9 @@ constexpr int kOkCache = 72;                   // bucket offsets of the cluster 
 
 // WIDE: more than 32 planes, so that which of them are live is looked up 32 at a time (one instance for both, deciding at run
 // time, spilled 28 bytes at D = 64).
-template <int D, bool WIDE>
+// P: planes of a step.  With at most 64 (32) query clusters a tile's rows hold those of two (four) consecutive planes: row L is query
+// cluster L % RP of plane pl + L / RP, and the contractions over the rows add up the planes as they do the query clusters.
+template <int D, bool WIDE, int P>
 __global__ void __launch_bounds__(sb::THREADS, D == 64 ? 2 : 1)
 k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_constant__ CUtensorMap tm_dnu,
               const __grid_constant__ CUtensorMap tm_K, const __grid_constant__ CUtensorMap tm_V,
@@ -60,6 +63,8 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
   // masked to that bucket's keys.
   using namespace sb;
   typedef Lay<D> LY;
+  static_assert(P == 1 || !WIDE, "planes are looked up 32 at a time only one by one");
+  constexpr int RP = TI / P;
   constexpr int kTile = LY::kTile, kKeys = LY::kKeys, oQhi = LY::oQhi, oQlo = LY::oQlo, oDka0 = LY::oDka0, oDnu0 = LY::oDnu0,
                 oDnu1 = LY::oDnu1, oK = LY::oK, oV = LY::oV, oW = LY::oW, G = D / 64;
   extern __shared__ __align__(1024) unsigned char sm_raw[];
@@ -118,27 +123,30 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
     if (D == 128 && !tc::mbar_wait(&bar_kv, ph_kv)) ok = false;
     bool started = false;                                 // dK^T / dV^T accumulate in TMEM over all (i tile, plane)
     for (int i0 = 0; i0 < dm.Cq && ok; i0 += TI) {
-      const int i = i0 + L;
+      const int i = i0 + L % RP, lp = P > 1 ? L / RP : 0;   // the row's query cluster, its plane within a step
       const bool in_range = cw && i < dm.Cq;
       const int ic = in_range ? i : 0;
       auto issue_grad = [&](int pl, int buf) {            // the ninth warp: both gradient tiles of (plane, j, i0..i0+127)
         tc::mbar_expect_tx_warp(&bar_g[buf], 2 * kTile);
-        const int row = (pq * dm.SB + pl) * dm.Ck + j;    // (rows i >= Cq are zeros)
         unsigned char* dka = sm + (buf ? oQlo : oDka0);
         unsigned char* dnu = sm + (buf ? oDnu1 : oDnu0);
-        for (int g = 0; g < G; ++g) {
-          tc::tma_load_3d_warp(dka + g * TI * 128, &tm_dka, 64 * g, i0, row, &bar_g[buf]);
-          tc::tma_load_3d_warp(dnu + g * TI * 128, &tm_dnu, 64 * g, i0, row, &bar_g[buf]);
+        for (int c = 0; c < P; ++c) {                     // (rows i >= Cq are zeros, and so are those of a plane past the last, from past the tensor's end)
+          const int row = P == 1 || pl + c < pl_end ? (pq * dm.SB + pl + c) * dm.Ck + j : dm.B * dm.Hq * dm.SB * dm.Ck;
+          for (int g = 0; g < G; ++g) {
+            tc::tma_load_3d_warp(dka + (g * TI + c * RP) * 128, &tm_dka, 64 * g, i0, row, &bar_g[buf]);
+            tc::tma_load_3d_warp(dnu + (g * TI + c * RP) * 128, &tm_dnu, 64 * g, i0, row, &bar_g[buf]);
+          }
         }
       };
       __syncthreads();                                    // every MMA that read the centroid tiles has completed (bar2 waited)
       if (warp == ISSUER / 32) {
         // sigma * qbar tile as bf16 hi + lo operands (split once per layer), and the first gradient tiles
         tc::mbar_expect_tx_warp(&bar_q, 2 * kTile);
-        for (int g = 0; g < G; ++g) {
-          tc::tma_load_3d_warp(sm + oQhi + g * TI * 128, &tm_qhi, 64 * g, i0, pq, &bar_q);
-          tc::tma_load_3d_warp(sm + oQlo + g * TI * 128, &tm_qlo, 64 * g, i0, pq, &bar_q);
-        }
+        for (int g = 0; g < G; ++g)
+          for (int c = 0; c < P; ++c) {
+            tc::tma_load_3d_warp(sm + oQhi + (g * TI + c * RP) * 128, &tm_qhi, 64 * g, i0, pq, &bar_q);
+            tc::tma_load_3d_warp(sm + oQlo + (g * TI + c * RP) * 128, &tm_qlo, 64 * g, i0, pq, &bar_q);
+          }
         if (pl0 < pl_end) issue_grad(pl0, 0);
       }
       // which planes hold a non-empty segment of query cluster i (others were never written by the far-field pass), 32 planes at
@@ -158,7 +166,7 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
       auto ent_of = [&](int pl) { return (((size_t)pq * dm.SB + pl) * dm.Cq + ic) * dm.Ck + j; };        // summaries: [plane][i][j]
       auto gent_of = [&](int pl) { return (((size_t)pq * dm.SB + pl) * dm.Ck + j) * dm.Cq + ic; };      // gradients: [plane][j][i]
       float mu_n = 0.f, dS_n = 0.f;
-      if (pl0 < pl_end && ((livemask >> (pl0 & 31)) & 1u)) { mu_n = mu[ent_of(pl0)]; dS_n = dS[gent_of(pl0)]; }
+      if (pl0 + lp < pl_end && ((livemask >> ((pl0 + lp) & 31)) & 1u)) { mu_n = mu[ent_of(pl0 + lp)]; dS_n = dS[gent_of(pl0 + lp)]; }
       // tilt logits l_iu = sigma qbar_i . k_u, the same for every plane: once per centroid tile
       if (warp == ISSUER / 32) {
         if (D == 64 && i0 == 0 && !tc::mbar_wait(&bar_kv, ph_kv)) ok = false;
@@ -185,16 +193,16 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
 #pragma unroll
       for (int c = 0; c < 32; ++c) wc[c] = 0.f;
       bool early = false;                                         // (issuer) the D-contractions of the plane are under way
-      for (int pl = pl0, k = 0; pl < pl_end && ok; ++pl, ++k) {
-        const int buf = k & 1;
-        const int nk = min(NU, ok_[pl + 1] - c0);
-        const int klo = per_block ? max(0, ok_[pl] - c0) : 0;      // first key of the chunk that this plane weighs
-        const bool live = (livemask >> (pl & 31)) & 1u;
+      for (int pl = pl0, k = 0; pl < pl_end && ok; pl += P, ++k) {
+        const int buf = k & 1, rp = P == 1 ? pl : min(pl + lp, dm.SB - 1);
+        const int nk = min(NU, ok_[rp + 1] - c0);
+        const int klo = per_block ? max(0, ok_[rp] - c0) : 0;      // first key of the chunk that the row's plane weighs
+        const bool live = (P == 1 || pl + lp < pl_end) && ((livemask >> (rp & 31)) & 1u);
         const float mu_i = mu_n * 1.4426950408889634f, dS_i = dS_n;
         const int oDka = buf ? oQlo : oDka0, oDnu = buf ? oDnu1 : oDnu0;
         const uint32_t aDka = tc::smem_u32(sm + oDka), aDnu = tc::smem_u32(sm + oDnu);
         if (WIDE && cw && pl + 1 < pl_end && ((pl + 1) & 31) == 0) look_up(pl + 1);
-        if (pl + 1 < pl_end && ((livemask >> ((pl + 1) & 31)) & 1u)) { mu_n = mu[ent_of(pl + 1)]; dS_n = dS[gent_of(pl + 1)]; }
+        if (pl + P + lp < pl_end && ((livemask >> ((pl + P + lp) & 31)) & 1u)) { mu_n = mu[ent_of(pl + P + lp)]; dS_n = dS[gent_of(pl + P + lp)]; }
         // The far-field pass wrote every row of the gradient tensors (zeros for an empty segment), so the
         // tiles go to the tensor cores as they land.  The D-contractions of a plane do not depend on the
         // previous plane's i-contractions: they are issued before them if the tiles are there by then, and only the W
@@ -219,7 +227,7 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
             issue_x(k);
           }
           if (k > 0 && !tc::mbar_wait(&bar2, ph2)) ok = false;      // the previous plane's MMAs are done with the other buffer
-          if (pl + 1 < pl_end && ok) issue_grad(pl + 1, buf ^ 1);
+          if (pl + P < pl_end && ok) issue_grad(pl + P, buf ^ 1);
         }
         ph_g ^= 1u << buf;
         if (cw && !tc::mbar_wait(&bar1, ph1)) ok = false;
@@ -276,7 +284,7 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
         __syncthreads();
         if (warp == ISSUER / 32) {
           tc::fence_after_sync();
-          early = D == 64 && pl + 1 < pl_end && ok && __all_sync(0xffffffffu, tc::mbar_test(&bar_g[buf ^ 1], (ph_g >> (buf ^ 1)) & 1u));
+          early = D == 64 && pl + P < pl_end && ok && __all_sync(0xffffffffu, tc::mbar_test(&bar_g[buf ^ 1], (ph_g >> (buf ^ 1)) & 1u));
           if (early) issue_x(k + 1);
           // A [i][d] and B [i][u]: both contract over rows.  M = 128 output dims even when D = 64: the second 64-dim group
           // of the A operand is then the tile that follows in shared memory, and output lanes 64..127 hold numbers that nobody reads
@@ -373,7 +381,8 @@ int summ_bwd_tc(const Dims& d, const void* Kp, const void* Vp, const int32_t* of
   const uint64_t Dd = (uint64_t)d.D, Cq = (uint64_t)d.Cq;
   const uint64_t str[2] = {Dd * 2, Cq * Dd * 2};
   const uint64_t dims_q[3] = {Dd, Cq, (uint64_t)d.B * d.Hq}, dims_g[3] = {Dd, Cq, (uint64_t)d.B * d.Hq * d.SB * d.Ck};   // gradients [plane][j][i]
-  const uint32_t box[3] = {64, (uint32_t)sb::TI, 1};
+  const int P = d.Cq <= 32 && d.SB >= 3 && d.SB <= 32 ? 4 : d.Cq <= 64 && d.SB >= 2 && d.SB <= 32 ? 2 : 1;           // planes of a step
+  const uint32_t box[3] = {64, (uint32_t)(sb::TI / P), 1};
   CUtensorMap tqh, tql, tdka, tdnu, tK, tV;
   int rc = make_tmap_bf16_nd(&tqh, qhi, 3, dims_q, str, box);
   if (rc == MUSE_OK) rc = make_tmap_bf16_nd(&tql, qlo, 3, dims_q, str, box);
@@ -387,8 +396,14 @@ int summ_bwd_tc(const Dims& d, const void* Kp, const void* Vp, const int32_t* of
     return launch_pdl(kernel, dim3(d.Ck, d.B * d.Hq), sb::THREADS, smem, st, d, tdka, tdnu, tK, tV, tqh, tql, off_k, off_q, mu, dS, dK_perm, dV_perm, per_block, status);
   };
   const bool wide = d.SB > 32;
-  if (d.D == 128) return wide ? launch(k_summ_bwd_tc<128, true>, sb::Lay<128>::total) : launch(k_summ_bwd_tc<128, false>, sb::Lay<128>::total);
-  return wide ? launch(k_summ_bwd_tc<64, true>, sb::Lay<64>::total) : launch(k_summ_bwd_tc<64, false>, sb::Lay<64>::total);
+  if (d.D == 128) {
+    constexpr int smem = sb::Lay<128>::total;
+    return P == 4 ? launch(k_summ_bwd_tc<128, false, 4>, smem) : P == 2 ? launch(k_summ_bwd_tc<128, false, 2>, smem)
+           : wide ? launch(k_summ_bwd_tc<128, true, 1>, smem) : launch(k_summ_bwd_tc<128, false, 1>, smem);
+  }
+  constexpr int smem = sb::Lay<64>::total;
+  return P == 4 ? launch(k_summ_bwd_tc<64, false, 4>, smem) : P == 2 ? launch(k_summ_bwd_tc<64, false, 2>, smem)
+         : wide ? launch(k_summ_bwd_tc<64, true, 1>, smem) : launch(k_summ_bwd_tc<64, false, 1>, smem);
 }
 
 }  // namespace muse
