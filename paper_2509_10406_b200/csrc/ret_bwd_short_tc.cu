@@ -19,9 +19,12 @@
 // A cluster with more than 64 visible keys takes further sweeps over the tiles that see them; later sweeps
 // add to the stored dQ rows.
 //
-// Bound by the latency of a tile's chain (gather, S, P and G, dQ) where a cluster has only a few tiles.  D = 64: 16 heads of 8k
-// tokens, 128 clusters, 8 slots 361 -> 254 us; 24 heads of 4k, 128 clusters, 8 slots, non-causal 353 -> 238; D = 128: 6 heads of 9k,
-// 200 clusters, 10 slots 265 -> 235.
+// Bound by the latency of a tile's chain (gather, S, P and G, dQ) where a cluster has only a few tiles.  At D = 64 the rows of the next
+// tile arrive beside it in a second pair of buffers; in a later sweep the stored dQ rows are on their way while the products run.
+// D = 64: 16 heads of 8k tokens, 128 clusters, 8 slots 361 -> 216 us; 24 heads of 4k, 128 clusters, 8 slots, non-causal 353 -> 213;
+// 32 heads of 16k, 256 clusters, 16 slots 1851 -> 1614; D = 128: 6 heads of 9k, 200 clusters, 10 slots 265 -> 220; 4 heads of 64k, 1024
+// clusters, 32 slots 2515 -> 2430.  dQ rows staged in shared memory and stored 16 bytes a lane: 2157 and 2941 us at the last
+// and third of these sizes.
 #include <cuda.h>
 #include "common.cuh"
 #include "tc05.cuh"
@@ -39,12 +42,13 @@ template <int D> struct Lay {
   static constexpr int NH = D == 64 ? 1 : 2;               // pipelines of a CTA; at D = 64 there are two CTAs on an SM instead
   static constexpr int kIssuerWarp0 = NH * kRowWarps, kGatherWarp0 = kIssuerWarp0 + NH, kThreads = (kGatherWarp0 + NH * kGather / 32) * 32;
   static constexpr int kTile = kPairs * D * 2, kKV = kKeys * D * 2, kPG = kPairs * kKeys * 2;
-  static constexpr int oK = 0, oV = kKV, oHalf = 2 * kKV, kHalf = 2 * kTile + 2 * kPG;   // per half: Q | dO | P | G
-  static constexpr int kSmem = oHalf + NH * kHalf;          // 224 KB at D = 128: no slack, the kernel checks the alignment of its base
+  static constexpr int NQ = D == 64 ? 2 : 1;               // tiles of gathered rows in the ring of a half
+  static constexpr int oK = 0, oV = kKV, oHalf = 2 * kKV, oPG = 2 * NQ * kTile, kHalf = oPG + 2 * kPG;   // per half: NQ x (Q | dO) | P | G
+  static constexpr int kSmem = oHalf + NH * kHalf;          // 224 KB on an SM (one CTA, or two): no slack, the kernel checks the alignment of its base
 };
 constexpr uint32_t cS = 0, cDP = 64, cDQ = 0, cDV = 128, cDK = 192, kCols = 256;   // per half; dQ reuses the columns of S and dP
 
-struct Bars { uint64_t q_full, q_empty, s_done, pg_ready, m2_done, dq_free; };
+struct Bars { uint64_t q_full[2], q_empty[2], s_done, pg_ready, m2_done, dq_free; };
 
 __device__ __forceinline__ void cp_async16(void* smem_dst, const void* src, bool valid) {
   const int n = valid ? 16 : 0;                             // 0 source bytes: the 16 bytes are zero-filled
@@ -68,7 +72,7 @@ k_ret_bwd_sweeps(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ d
   pdl_wait();
   using namespace rs;
   typedef Lay<D> LY;
-  constexpr int kTile = LY::kTile, kPG = LY::kPG, oK = LY::oK, oV = LY::oV, oHalf = LY::oHalf, kHalf = LY::kHalf;
+  constexpr int kTile = LY::kTile, kPG = LY::kPG, oK = LY::oK, oV = LY::oV, oHalf = LY::oHalf, oPG = LY::oPG, kHalf = LY::kHalf, NQ = LY::NQ;
   constexpr int NH = LY::NH, kIssuerWarp0 = LY::kIssuerWarp0, kGatherWarp0 = LY::kGatherWarp0, kThreads = LY::kThreads;
   extern __shared__ __align__(1024) unsigned char sm[];
   __shared__ Bars bars[NH];
@@ -95,13 +99,35 @@ k_ret_bwd_sweeps(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ d
     if (tid == 0) report_status(status, MUSE_STATUS_BWD_TIMEOUT);
     return;
   }
+  // role of this warp: half v, and row / issuing / gather warp
+  const bool roww = warp < NH * kRowWarps, issw = warp >= kIssuerWarp0 && warp < kIssuerWarp0 + NH, gatw = warp >= kGatherWarp0;
+  const int v = roww ? warp / kRowWarps : issw ? warp - kIssuerWarp0 : (warp - kGatherWarp0) / (kGather / 32);
+  // The keys and values of a sweep come through the row and issuing warps, all pieces of a thread in flight together (one by one they
+  // took 3800 cycles, as long as a tile).  Rows past the cluster are zeros.  (Fetched during the set-up, or while the sums of the
+  // sweep before leave, they make the compiler lay the whole sweep out twice: 72 KB of code instead of 49, and slower for it.)
+  const bf16* Kb = Kp + ((size_t)pk * dm.N + k0) * D;
+  const bf16* Vb = Vp + ((size_t)pk * dm.N + k0) * D;
+  constexpr int NT = kGatherWarp0 * 32, KP = (kKeys * (D / 8) + NT - 1) / NT;            // threads, pieces of a thread
+  uint4 kr[KP], vr[KP];
+  auto fetch_keys = [&](int kc) {
+#pragma unroll
+    for (int u = 0; u < KP; ++u) {
+      const int e = tid + u * NT, r = e / (D / 8), ck = e % (D / 8);
+      kr[u] = vr[u] = make_uint4(0u, 0u, 0u, 0u);
+      if (r < min(kKeys, kall - kc) && MUSE_IN_RANGE(k0 + kc + r, dm.N)) {
+        kr[u] = reinterpret_cast<const uint4*>(Kb + (size_t)(kc + r) * D)[ck];
+        vr[u] = reinterpret_cast<const uint4*>(Vb + (size_t)(kc + r) * D)[ck];
+      }
+    }
+  };
   const int32_t* ok = dm.S + 1 <= kOkCache ? ok_s : okg;
   if (dm.S + 1 <= kOkCache)
     for (int b = tid; b <= dm.S; b += kThreads) ok_s[b] = okg[b];
   if (warp == 0) tc::tmem_alloc(&tbase_s, NH * kCols);
   if (tid == 0) {
     for (int v = 0; v < NH; ++v) {
-      tc::mbar_init(&bars[v].q_full, kGather); tc::mbar_init(&bars[v].q_empty, 1); tc::mbar_init(&bars[v].s_done, 1);
+      for (int q = 0; q < NQ; ++q) { tc::mbar_init(&bars[v].q_full[q], kGather); tc::mbar_init(&bars[v].q_empty[q], 1); }
+      tc::mbar_init(&bars[v].s_done, 1);
       tc::mbar_init(&bars[v].pg_ready, kRowWarps * 32); tc::mbar_init(&bars[v].m2_done, 1); tc::mbar_init(&bars[v].dq_free, kRowWarps * 32);
     }
     tc::mbar_init_fence();
@@ -112,15 +138,10 @@ k_ret_bwd_sweeps(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ d
   pdl_trigger();                                           // (tensor memory has been allocated)
   const bf16* Qb = Q + (size_t)pq * dm.N * D;
   const bf16* dOb = dO + (size_t)pq * dm.N * D;
-  const bf16* Kb = Kp + ((size_t)pk * dm.N + k0) * D;
-  const bf16* Vb = Vp + ((size_t)pk * dm.N + k0) * D;
   const int32_t* pr = ri.pairs + (size_t)pq * dm.N * mk;
   const size_t pbase = (size_t)pq * dm.N * mk;
-  // role of this warp: half v, and row / issuing / gather warp
-  const bool roww = warp < NH * kRowWarps, issw = warp >= kIssuerWarp0 && warp < kIssuerWarp0 + NH, gatw = warp >= kGatherWarp0;
-  const int v = roww ? warp / kRowWarps : issw ? warp - kIssuerWarp0 : (warp - kGatherWarp0) / (kGather / 32);
   Bars& B = bars[v];
-  unsigned char* hb = sm + oHalf + v * kHalf;               // this half's Q | dO | P | G tiles
+  unsigned char* hb = sm + oHalf + v * kHalf;               // this half's rings of Q and dO, P and G tiles
   const uint32_t tbase = tbase_s + v * kCols;
   bool ok_ = true;                                          // false once a bounded wait ran out (every role still walks all its tiles)
   auto wait = [&](uint64_t* bar, uint32_t parity) { if (ok_ && !tc::mbar_wait(bar, parity)) ok_ = false; };
@@ -146,23 +167,19 @@ k_ret_bwd_sweeps(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ d
     const int tile0 = tile_lo + ((sub - tile_lo % nsub) + nsub) % nsub + v * nsub;   // this half's first tile; it takes every NH-th of the CTA's
     const int tstep = NH * nsub;
     __syncthreads();                                        // the previous sweep's products are complete, its accumulators read
-    // the sweep's keys and values as [2][64 rows][128 B] swizzled tiles (K-major and MN-major operands); rows past the cluster are zeros
+    // the sweep's keys and values as [2][64 rows][128 B] swizzled tiles (K-major and MN-major operands)
     // (the gather warps have begun with the first tile meanwhile)
     const int at0 = g0 + tile0 * kPairs + (tid & 127);
     const int id0 = roww && tile0 < ntiles && at0 < g1 ? __ldg(pr + at0) : -1;
     if (!gatw) {
-      constexpr int NT = kGatherWarp0 * 32;
-      for (int e = tid; e < kKeys * (D / 8); e += NT) {
-        const int r = e / (D / 8), ck = e % (D / 8);
-        uint4 a = make_uint4(0u, 0u, 0u, 0u), b = a;
-        if (r < nkc && MUSE_IN_RANGE(k0 + kc + r, dm.N)) {
-          a = reinterpret_cast<const uint4*>(Kb + (size_t)(kc + r) * D)[ck];
-          b = reinterpret_cast<const uint4*>(Vb + (size_t)(kc + r) * D)[ck];
-        }
+      fetch_keys(kc);
+#pragma unroll
+      for (int u = 0; u < KP; ++u) {
+        const int e = tid + u * NT, r = e / (D / 8), ck = e % (D / 8);
         const uint32_t off = (ck >> 3) * kKeys * 128 + tc::sw128_off(r, ck & 7);
-        if (!MUSE_IN_RANGE(off, kKeys * D * 2 - 15)) continue;
-        *reinterpret_cast<uint4*>(sm + oK + off) = a;
-        *reinterpret_cast<uint4*>(sm + oV + off) = b;
+        if (e >= kKeys * (D / 8) || !MUSE_IN_RANGE(off, kKeys * D * 2 - 15)) continue;
+        *reinterpret_cast<uint4*>(sm + oK + off) = kr[u];
+        *reinterpret_cast<uint4*>(sm + oV + off) = vr[u];
       }
       tc::fence_async_smem();                               // the tensor cores read the tiles through the async proxy
       tc::named_bar_sync(1 + NH, NT);
@@ -225,8 +242,8 @@ k_ret_bwd_sweeps(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ d
             gw[i / 2] = *reinterpret_cast<uint32_t*>(&gb);
           }
           const uint32_t off = tc::sw128_off(row, g);
-          *reinterpret_cast<uint4*>(hb + 2 * kTile + off) = make_uint4(pw[0], pw[1], pw[2], pw[3]);
-          *reinterpret_cast<uint4*>(hb + 2 * kTile + kPG + off) = make_uint4(gw[0], gw[1], gw[2], gw[3]);
+          *reinterpret_cast<uint4*>(hb + oPG + off) = make_uint4(pw[0], pw[1], pw[2], pw[3]);
+          *reinterpret_cast<uint4*>(hb + oPG + kPG + off) = make_uint4(gw[0], gw[1], gw[2], gw[3]);
           if (g + 1 < kKeys / 8) {
             tc::tmem_ld_wait();
             tc::tmem_ld_use8(sv[(g + 1) & 1]);
@@ -236,11 +253,22 @@ k_ret_bwd_sweeps(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ d
         tc::fence_async_smem();                             // P and G are read by the tensor cores
         tc::fence_before_sync();
         tc::mbar_arrive(&B.pg_ready);
+        const bool live = pid >= 0 && ok_;
+        bf16* drow = dq_part + (pbase + max(pid, 0)) * D;
+        uint32_t old[2][16];                                // a later sweep adds to the stored row, 64 dims of which are on their way
+        auto ld_old = [&](int d0, uint32_t (&o)[16]) {
+          uint32_t w[8];
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            if (live) tc::ld_global_32B(drow + d0 + 16 * c, w);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) o[8 * c + e] = live ? w[e] : 0u;
+          }
+        };
+        if (!first) { ld_old(0, old[0]); ld_old(32, old[1]); }
         wait(&B.m2_done, ph);
         tc::fence_after_sync();
         started = true;
-        const bool live = pid >= 0 && ok_;
-        bf16* drow = dq_part + (pbase + max(pid, 0)) * D;
 #pragma unroll
         for (int d0 = 0; d0 < D; d0 += 32) {
           float x[32];
@@ -249,24 +277,20 @@ k_ret_bwd_sweeps(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ d
             tc::fence_before_sync();
             tc::mbar_arrive(&B.dq_free);
           }
+          if (!first) {
+            uint32_t (&o)[16] = old[(d0 >> 5) & 1];
+#pragma unroll
+            for (int e = 0; e < 16; ++e) { x[2 * e] += __uint_as_float(o[e] << 16); x[2 * e + 1] += __uint_as_float(o[e] & 0xffff0000u); }
+            if (d0 + 64 < D) ld_old(d0 + 64, o);
+          }
           if (live) {
 #pragma unroll
             for (int c = 0; c < 2; ++c) {                   // 16 columns = 32 bytes per store
               uint32_t w[8];
-              if (!first) {
-                tc::ld_global_32B(drow + d0 + 16 * c, w);
 #pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                  const __nv_bfloat162 o2 = *reinterpret_cast<const __nv_bfloat162*>(&w[e]);
-                  __nv_bfloat162 b2 = __floats2bfloat162_rn(x[16 * c + 2 * e] + __low2float(o2), x[16 * c + 2 * e + 1] + __high2float(o2));
-                  w[e] = *reinterpret_cast<uint32_t*>(&b2);
-                }
-              } else {
-#pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                  __nv_bfloat162 b2 = __floats2bfloat162_rn(x[16 * c + 2 * e], x[16 * c + 2 * e + 1]);
-                  w[e] = *reinterpret_cast<uint32_t*>(&b2);
-                }
+              for (int e = 0; e < 8; ++e) {
+                __nv_bfloat162 b2 = __floats2bfloat162_rn(x[16 * c + 2 * e], x[16 * c + 2 * e + 1]);
+                w[e] = *reinterpret_cast<uint32_t*>(&b2);
               }
               tc::st_global_32B(drow + d0 + 16 * c, w);
             }
@@ -283,6 +307,7 @@ k_ret_bwd_sweeps(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ d
           float* dst = (w2 == 0 ? dV_perm : dK_perm) + ((size_t)pq * dm.N + k0 + kc) * D + dd;
 #pragma unroll
           for (int u0 = 0; u0 < kKeys; u0 += 32) {
+            if (u0 >= nkc) break;
             float x[32];
             tc::tmem_ld32(tl + (w2 == 0 ? cDV : cDK) + u0, x);
             if (ok_) {
@@ -295,13 +320,13 @@ k_ret_bwd_sweeps(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ d
       }
     } else if (issw) {
       // ================= MMA issue =================
-      const uint32_t qa = tc::smem_u32(hb), da = qa + kTile, pa = da + kTile, ga = pa + kPG;
+      const uint32_t q0 = tc::smem_u32(hb), pa = q0 + oPG, ga = pa + kPG;
       const uint32_t ka = tc::smem_u32(sm + oK), va = tc::smem_u32(sm + oV);
       const uint32_t np0 = np;
       for (int tile = tile0; tile < ntiles; tile += tstep, ++np) {
         {
-          const uint32_t ph = np & 1;
-          wait(&B.q_full, ph);                               // the tile's Q and dO rows are in shared memory
+          const uint32_t ph = np & 1, st_ = np % NQ, qa = q0 + st_ * 2 * kTile, da = qa + kTile;
+          wait(&B.q_full[st_], (np / NQ) & 1);               // the tile's Q and dO rows are in shared memory
           if (np > 0) wait(&B.dq_free, ph ^ 1);              // the previous dQ rows have been read out of the columns S and dP go to
           tc::fence_after_sync();
           const uint32_t id1 = tc::idesc_bf16(kPairs, kKeys, 0, 0);
@@ -327,7 +352,7 @@ k_ret_bwd_sweeps(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ d
           for (int ks = 0; ks < kPairs / 16; ++ks)
             tc::mma_bf16_ss_warp(tbase + cDK, desc_mn<kPairs>(qa, ks), tc::smem_desc_sw128(ga + ks * 16 * 128, kPairs * 128, 1024), id_t, acc || ks > 0);
           tc::mma_commit_warp(&B.m2_done);
-          tc::mma_commit_warp(&B.q_empty);                        // ... and the Q / dO tiles refilled
+          tc::mma_commit_warp(&B.q_empty[st_]);                   // ... and the Q / dO tiles refilled
         }
         __syncwarp();
       }
@@ -349,7 +374,9 @@ k_ret_bwd_sweeps(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ d
       int pa_ = ld1(tile0);
       for (int tile = tile0; tile < ntiles; tile += tstep, ++np) {
         const int pa_n = ld1(tile + tstep);
-        if (np > 0) wait(&B.q_empty, (np - 1) & 1);          // the previous tile's products have read the buffers
+        const uint32_t st_ = np % NQ;
+        unsigned char *qs = qd + st_ * 2 * kTile, *os = od + st_ * 2 * kTile;
+        wait(&B.q_empty[st_], ((np / NQ) & 1) ^ 1);          // the products of the tile before in the buffers have read them
         tok_s[v][g] = pa_ >= 0 ? pa_ / mk : -1;
         tc::named_bar_sync(1 + v, kGather);
 #pragma unroll 4
@@ -357,13 +384,13 @@ k_ret_bwd_sweeps(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ d
           const int tok = tok_s[v][r];
           const size_t at = (size_t)max(tok, 0) * D + ck * 8;
           if (!MUSE_IN_RANGE(tok + 1, dm.N + 1) || !MUSE_IN_RANGE((ck >> 3) * kPairs * 128 + tc::sw128_off(r, ck & 7), kPairs * D * 2 - 15)) continue;
-          cp_async16(qd + tc::sw128_off(r, ck & 7), Qb + at, tok >= 0);
-          cp_async16(od + tc::sw128_off(r, ck & 7), dOb + at, tok >= 0);
+          cp_async16(qs + tc::sw128_off(r, ck & 7), Qb + at, tok >= 0);
+          cp_async16(os + tc::sw128_off(r, ck & 7), dOb + at, tok >= 0);
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
         asm volatile("cp.async.wait_group 0;" ::: "memory");
         tc::fence_async_smem();                              // the tensor cores read the rows through the async proxy
-        tc::mbar_arrive(&B.q_full);
+        tc::mbar_arrive(&B.q_full[st_]);
         tc::named_bar_sync(1 + v, kGather);                  // tok_s may be rewritten
         pa_ = pa_n;
       }
