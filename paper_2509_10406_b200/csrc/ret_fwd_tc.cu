@@ -16,8 +16,10 @@
 // gather warps were slower: their copies crowd out the row warps' stores).  The CTA is deliberately
 // small (D = 128: 96 KB of shared memory, 256 TMEM columns, 224 threads) so that two of them share an SM and
 // fill each other's waits; at D = 64 three do (48 KB, 128 columns: the output takes the columns of logits that P has left, and
-// 80 registers): 16 heads of 8k tokens, 64 keys a cluster 137 -> 123 us, 32 heads of 16k 919 -> 801, 32 keys 141 -> 128; four CTAs
-// (72 registers, spills) 129, 872 and 132.
+// 80 registers): 16 heads of 8k tokens, 64 keys a cluster 137 -> 123 us, 32 heads of 16k 919 -> 801, 32 keys 141 -> 128 (four CTAs of 72
+// registers 129, 872 and 132).  A row's logits are masked where they are read and its first 32 stay in registers for the second
+// sweep over them, with 10 KB less code (short CTAs in different phases share an instruction cache): 109, 740 and 106 us; D = 128,
+// 64 keys, 4 heads of 64k 1169 -> 1100.
 // Clusters with more than 128 visible keys take further sweeps over the tiles that see them; a later
 // sweep merges its partial result into the stored row by log-sum-exp weights.
 // The row, issuing and gather warps start together: the gather of the first tile runs beside the load of the keys, of which only
@@ -179,43 +181,39 @@ k_ret_fwd_pairs_tc(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__
           asm volatile("prefetch.global.L2 [%0];" ::"l"(l_part + pbase + pid_n));
         }
         const int nk = visible(last, kc), nk16 = (nk + 15) & ~15;      // the tile's last pair has the latest plane: it sees the most keys
-        // which of the sweep's 128 key columns this row sees (a prefix: the cluster's keys of the earlier blocks, or the bucket)
-        uint32_t vm[4] = {0u, 0u, 0u, 0u};
-        auto set_range = [&](int lo, int hi) {               // columns [lo, hi) of the sweep
-          lo = max(lo, 0); hi = min(hi, kKeys);
-#pragma unroll
-          for (int g = 0; g < 4; ++g) {
-            const int a = max(lo - 32 * g, 0), z = min(hi - 32 * g, 32);
-            if (z > a) vm[g] |= (z - a >= 32 ? 0xffffffffu : ((1u << (z - a)) - 1u) << a);
-          }
-        };
-        if (pid >= 0) set_range(0, visible(pid, kc));
+        const int lim = pid >= 0 ? visible(pid, kc) : 0;     // columns [0, lim) of the sweep are keys that this row sees
         const float lse_old = (!first && pid >= 0) ? l_part[pbase + pid] : -INFINITY;
         float M = -INFINITY, l = 0.f;
         if (nk16 > 0) {
           const uint32_t ph = nproc & 1;
           wait(&bars.s_done, ph);
           tc::fence_after_sync();
-          // the logits are read twice (row maximum, then probabilities) rather than kept in registers
-          float mx = -INFINITY;
-          for (int g = 0; 32 * g < nk16; ++g) {
-            float sv[32];
+          // two sweeps over the logits (row maximum, then probabilities), of which the first 32 stay in registers: many tiles have no more
+          float sv[32], mx = -INFINITY;
+          auto logits = [&](int g) {
             tc::tmem_ld32(tl + SM::cS + 32 * g, sv);
-            const uint32_t w = vm[g];
+            if (__any_sync(0xffffffffu, lim < 32 * g + 32)) {
 #pragma unroll
-            for (int i = 0; i < 32; ++i) mx = fmaxf(mx, (w >> i) & 1u ? sv[i] : -INFINITY);
+              for (int i = 0; i < 32; ++i) sv[i] = 32 * g + i < lim ? sv[i] : -INFINITY;
+            }
+          };
+#pragma unroll 1
+          for (int g = (nk16 - 1) >> 5; g >= 0; --g) {
+            logits(g);
+            float m4[4] = {sv[0], sv[1], sv[2], sv[3]};
+#pragma unroll
+            for (int i = 4; i < 32; ++i) m4[i & 3] = fmaxf(m4[i & 3], sv[i]);
+            mx = fmaxf(mx, fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])));
           }
           M = mx * scale2;                                 // (scale2 > 0)
           const float base = M == -INFINITY ? 0.f : M;
+#pragma unroll 1
           for (int g = 0; 32 * g < nk16; ++g) {
-            float sv[32];
-            tc::tmem_ld32(tl + SM::cS + 32 * g, sv);
-            const uint32_t w = vm[g];
+            if (g > 0) logits(g);
             uint32_t pk2[16];
 #pragma unroll
             for (int i = 0; i < 32; i += 2) {
-              const float e0 = (w >> i) & 1u ? tc::fast_exp2(fmaf(sv[i], scale2, -base)) : 0.f;
-              const float e1 = (w >> (i + 1)) & 1u ? tc::fast_exp2(fmaf(sv[i + 1], scale2, -base)) : 0.f;
+              const float e0 = tc::fast_exp2(fmaf(sv[i], scale2, -base)), e1 = tc::fast_exp2(fmaf(sv[i + 1], scale2, -base));
               l += e0 + e1;
               __nv_bfloat162 b2 = __floats2bfloat162_rn(e0, e1);
               pk2[i / 2] = *reinterpret_cast<uint32_t*>(&b2);
