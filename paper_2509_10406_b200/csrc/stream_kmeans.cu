@@ -225,13 +225,14 @@ k_stream_kmeans(const T* __restrict__ X, int N, int C, uint64_t seed, int kind, 
 // Bound by the latency of one step, N / 64 of them in a chain, so everything that a step does not need from the one
 // before it is done elsewhere: four gather warps compute the shuffled positions and bring in the next minibatch by
 // asynchronous copies; sixteen compute warps read the distances (every second pair of warps a half's 64 rows, a quarter
-// of a tile's columns each), post one candidate per quarter, and after a single barrier every warp derives all 64
-// assignments in registers and updates the centroids whose first vector falls to it (a group of D / 8 lanes per vector).
-// Two barriers per step, the second a cluster barrier when a problem's centroids are spread over several CTAs.  Totals
-// stay in shared memory and centre rows leave for global memory once, at the end.  Measured at 32 + 32 problems of 65536
-// vectors, D = 64, 128 centroids: 5.4 us per step and one side after the other (11.15 ms) before, 3.6 us per step for
-// both now.  A step is some 1000 dependent-ish instructions per warp at 7 cycles each, spread evenly over products
-// (1200 cycles), arg-min (1400), candidates (1100) and update (2300): no single part is left to take out.
+// of a tile's columns each) and post one candidate per quarter; two of them take the best of a vector's candidates, and all update the
+// centroids whose first vector falls to them (a group of D / 8 lanes per vector).  Three barriers per step, the second a cluster
+// barrier when a problem's centroids are spread over several CTAs.  Totals stay in shared memory and centre rows leave for global
+// memory once, at the end.  Measured at 32 + 32 problems of 65536 vectors, D = 64, 128 centroids: 5.4 us per step and one side
+// after the other (11.15 ms) at first, 3.6 us per step for both with two CTAs a problem and every warp taking the best candidates of all
+// 64 vectors (16 warps of 130 instructions, on the step's path), 3.1 us now.  A step: products 1100 cycles, arg-min 1300, barriers
+// 500, candidates 400, update 2500 (four groups' ballots, members in order, eight divisions, |c|^2 by shuffles).  Slower: divisions by a
+// reciprocal and two corrections (3.4 us), columns as immediates in the arg-min with all norms loaded first (3.3 us).
 // ---------------------------------------------------------------------------------------------
 constexpr int kStCompute = 512, kStGather = 128, kStThreads = kStCompute + kStGather;
 
@@ -276,7 +277,7 @@ k_stream_kmeans_tc(const __grid_constant__ StArgs g, int* __restrict__ status) {
   __shared__ uint64_t sdone;
   __shared__ uint32_t tbase_s;
   __shared__ int2 cand[2][4 * kSkMaxCluster][kSkBatch];      // (distance bits, centroid) by step parity, CTA and column quarter
-  __shared__ int pos_s[kSkBatch];
+  __shared__ int pos_s[kSkBatch], as_s[kSkBatch];            // positions of the next minibatch, assignments of this one
   unsigned char* sm = st_raw + ((1024u - (tc::smem_u32(st_raw) & 1023u)) & 1023u);
   int prob = blockIdx.x / CS;
   const bool second = prob >= g.s[0].problems;
@@ -439,15 +440,16 @@ k_stream_kmeans_tc(const __grid_constant__ StArgs g, int* __restrict__ status) {
         for (int r = 0; r < CS; ++r) *cluster.map_shared_rank(&cand[par][rank * 4 + quarter][p], r) = mine;
     }
     if (CS == 1) tc::named_bar_sync(1, kStCompute); else cluster.sync();     // B: every candidate has arrived
-    // every warp: the minibatch's assignments, two per lane (lower distance wins, the lower centroid on a tie)
-    auto assigned = [&](int p) {
+    // two warps: the minibatch's assignments (lower distance wins, the lower centroid on a tie); every warp then holds all, two per lane
+    if (tid < kSkBatch) {
       float dv = INFINITY;
       int iv = 0x7fffffff;
 #pragma unroll 4
-      for (int r = 0; r < 4 * CS; ++r) argmin_tie_step(__int_as_float(cand[par][r][p].x), cand[par][r][p].y, dv, iv);
-      return p < nb ? ((unsigned)iv < (unsigned)C ? iv : 0) : -1;            // (a NaN row goes to centroid 0)
-    };
-    const int a_lo = assigned(lane), a_hi = assigned(lane + 32);
+      for (int r = 0; r < 4 * CS; ++r) argmin_tie_step(__int_as_float(cand[par][r][tid].x), cand[par][r][tid].y, dv, iv);
+      as_s[tid] = tid < nb ? ((unsigned)iv < (unsigned)C ? iv : 0) : -1;     // (a NaN row goes to centroid 0)
+    }
+    tc::named_bar_sync(1, kStCompute);
+    const int a_lo = as_s[lane], a_hi = as_s[lane + 32];
     // update: the first vector of the minibatch on a centroid replays all of that centroid's vectors in stream order.
     // A group of D / 8 lanes takes a vector (8 dims per lane), so a warp works on several centroids at once.
 #pragma unroll
@@ -547,11 +549,12 @@ static int stream_kmeans_tc(const Dims& d, const StreamSide* sides, int n, uint6
   g.N = d.N; g.first_batch = first_batch; g.n_batches = n_batches; g.beta = beta; g.seed = seed;
   int problems = 0, C = 0;
   for (int k = 0; k < n; ++k) { problems += sides[k].problems; C = sides[k].C > C ? sides[k].C : C; }
-  // CTAs per problem: at most 256 centroids (two tiles) per CTA; more CTAs, down to 32 centroids each, as long as every
-  // CTA still has an SM of its own (a step's arg-min and update then touch that many fewer centroids, which outweighs
-  // the cluster barrier)
+  // CTAs per problem: at most 256 centroids (two tiles) per CTA; from 256 per CTA on twice the CTAs, as long as every CTA still has an SM
+  // of its own.  (A cluster barrier and the exchange of candidates cost more than half as many columns of an arg-min: us a step, lines at
+  // 64 | 128 | 256 | 512 centroids: 64 problems of 128 centroids, D = 64 3.70 | 3.69 | 3.31 | 3.32, D = 128 6.53 | 6.53 | 5.46 | 5.46; 2 of 64
+  // and 128 5.28 | 5.00 | 3.65 | 3.65; 20 of 152 and 256 3.96 | 3.96 | 3.79 | 3.90; 8 of 64 and 256, D = 128 6.14 | 5.35 | 5.24 | 5.47.)
   int cs = 1;
-  while (cs < kSkMaxCluster && (C > 256 * cs || (C >= 64 * cs && (long long)problems * cs * 2 <= sm_count()))) cs *= 2;
+  while (cs < kSkMaxCluster && (C > 256 * cs || (C >= 256 * cs && (long long)problems * cs * 2 <= sm_count()))) cs *= 2;
   size_t smem = 0;
   for (int k = 0; k < n; ++k) {
     const StreamSide& s = sides[k];
