@@ -16,7 +16,9 @@
 // N = 64 product takes 49 cycles per 16-deep step instead of 32: its A operand has to come out of memory).  NW is the
 // most that tensor memory holds beside the accumulators.  Against products issued by one thread around CTA-wide barriers,
 // with P and G through shared memory: 64k tokens in 8 blocks, D = 64, 32 heads, dK/dV 9490 -> 5650 us (780 TFLOP/s) and dQ
-// 5810 -> 3400 us (970); D = 128, 4 heads, 1540 -> 980 (1130) and 1070 -> 670 us (1230).
+// 5810 -> 3400 us (970); D = 128, 4 heads, 1540 -> 980 (1130) and 1070 -> 670 us (1230).  With masks as a branch of a group of 16 and two
+// numbers per instruction where one rounds like the other (11.5 instructions an entry before): D = 64 5620 -> 4770 and 3440 -> 3240
+// us, D = 128 969 -> 895 and 678 -> 670.
 #include <cuda.h>
 #include "common.cuh"
 #include "tc05.cuh"
@@ -97,13 +99,13 @@ k_local_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_a, const __grid_c
         tc::tma_load_2d(sm + LY::oB + g * kM * 128, &tm_b, 64 * g, rrow, &bars.res);
       }
     }
-    float l0 = 0.f, l1 = 0.f, d0 = 0.f, d1 = 0.f;          // L (log2 units) and delta of the next tile's columns lane, lane + 32
+    float l0 = 0.f, l1 = 0.f, d0 = 0.f, d1 = 0.f;          // -L (log2 units) and -delta of the next tile's columns lane, lane + 32
     auto scalars = [&](int t) {
       if (KIND != 0 || t >= T) return;
       const int q = c_lo + t * kN + lane;
       const size_t at = (size_t)pq * dm.N;
-      l0 = q < bend ? LSE[at + q] * kLog2e : 0.f; d0 = q < bend ? delta[at + q] : 0.f;
-      l1 = q + 32 < bend ? LSE[at + q + 32] * kLog2e : 0.f; d1 = q + 32 < bend ? delta[at + q + 32] : 0.f;
+      l0 = q < bend ? -(LSE[at + q] * kLog2e) : 0.f; d0 = q < bend ? -delta[at + q] : 0.f;
+      l1 = q + 32 < bend ? -(LSE[at + q + 32] * kLog2e) : 0.f; d1 = q + 32 < bend ? -delta[at + q + 32] : 0.f;
     };
     scalars(0);
     for (int t = 0, s = 0, ph = 0; t < T && ok; ++t) {
@@ -172,8 +174,12 @@ k_local_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_a, const __grid_c
     const int w = warp >> 2, row = tid & 127, u = r0 + row;
     const uint32_t tl = tbase + ((uint32_t)((warp & 3) * 32) << 16), ts = tl + (uint32_t)w * 2 * kN;
     const float scale2 = dm.sigma * kLog2e;
-    float L2 = 0.f, dl = 0.f;
-    if (KIND == 1 && row < nr) { L2 = LSE[(size_t)pq * dm.N + u] * kLog2e; dl = delta[(size_t)pq * dm.N + u]; }
+    const uint64_t sc2 = tc::pair(scale2, scale2);
+    uint64_t L2 = 0u, dl = 0u;                             // -L (log2 units) and -delta of the row, twice
+    if (KIND == 1 && row < nr) {
+      const float a = -(LSE[(size_t)pq * dm.N + u] * kLog2e), b = -delta[(size_t)pq * dm.N + u];
+      L2 = tc::pair(a, a); dl = tc::pair(b, b);
+    }
     int s = w % NS;
     for (int t = w, ph = 0; t < T; t += NW, ph ^= 1) {
       if (ok && !tc::mbar_wait(&bars.s_full[w], ph)) ok = false;
@@ -196,25 +202,22 @@ k_local_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_a, const __grid_c
         tc::tmem_ld_use16(dp);
         float sn[16], dn_[16];
         if (g < 3) { tc::tmem_ld16_issue(ts + 16 * (g + 1), sn); tc::tmem_ld16_issue(ts + kN + 16 * (g + 1), dn_); }
-        uint32_t pw[8], gw[8];
-        float p[16];
+        if (!full) {                                       // (a branch for the whole group: masks of single entries cost three instructions each in every tile)
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          float Lc[4], dc[4];
-          if (KIND == 0) {
-            const float4 a = *reinterpret_cast<const float4*>(&Ls[s][16 * g + 4 * k]), b = *reinterpret_cast<const float4*>(&ds[s][16 * g + 4 * k]);
-            Lc[0] = a.x; Lc[1] = a.y; Lc[2] = a.z; Lc[3] = a.w; dc[0] = b.x; dc[1] = b.y; dc[2] = b.z; dc[3] = b.w;
-          }
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const int c = 4 * k + e;
-            p[c] = tc::fast_exp2(fmaf(sv[c], scale2, KIND == 0 ? -Lc[e] : -L2));
-            if (!full) p[c] = 16 * g + c >= lo && 16 * g + c < hi ? p[c] : 0.f;
-            dp[c] = p[c] * (dp[c] - (KIND == 0 ? dc[e] : dl));
-          }
+          for (int c = 0; c < 16; ++c) sv[c] = 16 * g + c >= lo && 16 * g + c < hi ? sv[c] : -INFINITY;
         }
+        uint32_t pw[8], gw[8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) { pw[k] = pack2(p[2 * k], p[2 * k + 1]); gw[k] = pack2(dp[2 * k], dp[2 * k + 1]); }
+        for (int k = 0; k < 8; ++k) {
+          const uint64_t nl = KIND == 0 ? *reinterpret_cast<const uint64_t*>(&Ls[s][16 * g + 2 * k]) : L2,
+                         nd = KIND == 0 ? *reinterpret_cast<const uint64_t*>(&ds[s][16 * g + 2 * k]) : dl;
+          float x0, x1, g0, g1;
+          tc::unpair(tc::fma2(tc::pair(sv[2 * k], sv[2 * k + 1]), sc2, nl), x0, x1);
+          const float p0 = tc::fast_exp2(x0), p1 = tc::fast_exp2(x1);
+          tc::unpair(tc::mul2(tc::pair(p0, p1), tc::add2(tc::pair(dp[2 * k], dp[2 * k + 1]), nd)), g0, g1);
+          pw[k] = pack2(p0, p1);
+          gw[k] = pack2(g0, g1);
+        }
         // over logits already consumed: columns [16 g, 16 g + 16) -> words [8 g, 8 g + 8)
         if (KIND == 0) { tc::tmem_st8_issue(ts + 8 * g, pw); tc::tmem_st8_issue(ts + kN + 8 * g, gw); }
         else tc::tmem_st8_issue(ts + 8 * g, gw);

@@ -19,7 +19,8 @@
 // tokens, at D = 128 two threads per row were slower (638 -> 1060 us) and there is no room for a third buffer.
 // Against one 128-query tile per CTA with P through shared memory and a CTA barrier per tile: 64k tokens in 8 blocks,
 // D = 64, 32 heads 5926 -> 3300 us (667 TFLOP/s); D = 128, 4 heads 908 -> 638 us (862); 128k tokens, 4 heads 3400 ->
-// 2290 us (960).
+// 2290 us (960).  Since then two logits per instruction where one rounds like the other, three per maximum and no spills around the
+// rescaling: 32 heads, D = 64 3600 -> 3000 us; 4 heads, D = 128 637 -> 505.
 #include <cuda.h>
 #include "common.cuh"
 #include "tc05.cuh"
@@ -159,6 +160,7 @@ k_local_fwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_q, const __grid_c
     const int qrow = q0 + q * kRows + row;
     const uint32_t tl = tbase + ((uint32_t)((warp & 3) * 32) << 16), to = tl + cO + q * D + half * OD;
     const float scale2 = dm.sigma * 1.4426950408889634f;
+    const uint64_t sc2 = tc::pair(scale2, scale2);
     // m2 is the exponent base in use for this row (log2 units): it follows the running maximum lazily, only when that has
     // grown by more than kLazy (probabilities then stay below 2^kLazy), and only then is the accumulator rescaled.
     constexpr float kLazy = 8.f;
@@ -182,16 +184,16 @@ k_local_fwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_q, const __grid_c
 #pragma unroll
           for (int i = 0; i < 16; ++i) s[g][i] = 16 * g + i <= lim ? s[g][i] : -INFINITY;
       }
-      float mx[4];
+      float mx[W / 16];                                    // (three at a time)
 #pragma unroll
-      for (int g = 0; g < 4; ++g) {
-        mx[g] = s[g][0];
+      for (int g = 0; g < W / 16; ++g) {
+        mx[g] = fmaxf(s[g][0], s[g][1]);
 #pragma unroll
-        for (int k = g; k < W / 16; k += 4)
-#pragma unroll
-          for (int i = 0; i < 16; ++i) mx[g] = fmaxf(mx[g], s[k][i]);
+        for (int i = 2; i < 16; i += 2) mx[g] = tc::max3(mx[g], s[g][i], s[g][i + 1]);
       }
-      const float mt = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * scale2;
+#pragma unroll
+      for (int g = W / 16 - 1; g > 0; --g) mx[g - 1] = fmaxf(mx[g - 1], mx[g]);
+      const float mt = mx[0] * scale2;
       // (also: both halves have read their logits before either writes P over them)
       const bool grow = t == 0 || mt > m2 + kLazy;
       if (H == 2 ? bar_or(1 + q, kSoft / 2, grow) : __any_sync(0xffffffffu, grow)) {
@@ -206,32 +208,39 @@ k_local_fwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_q, const __grid_c
           if (ok && !tc::mbar_wait(&bars.pv_done[q], (t - 1) & 1)) ok = false;
           tc::fence_after_sync();
           const float resc = tc::fast_exp2(m2 - mn);
+#pragma unroll 1
+          for (int d0 = 0; d0 < OD; d0 += 16) {            // (16 at a time: the logits stay in registers meanwhile)
+            float v[16];
+            uint32_t x[16];
+            tc::tmem_ld16(to + d0, v);
 #pragma unroll
-          for (int d0 = 0; d0 < OD; d0 += 32) {
-            float v[32];
-            tc::tmem_ld32(to + d0, v);
-#pragma unroll
-            for (int i = 0; i < 32; ++i) v[i] *= resc;
-            tc::tmem_st32(to + d0, v);
+            for (int i = 0; i < 16; ++i) x[i] = __float_as_uint(v[i] * resc);
+            tc::tmem_st16_issue(to + d0, x);
           }
+          tc::tmem_st_wait();
           l *= resc;
         }
         m2 = mn;
       }
       const float base = m2 == -INFINITY ? 0.f : m2;
-      float rs[4] = {0.f, 0.f, 0.f, 0.f};
+      const uint64_t nb = tc::pair(-base, -base);
+      uint64_t rs[4] = {0u, 0u, 0u, 0u};                   // (pairs of zeros)
 #pragma unroll
       for (int g = 0; g < W / 16; ++g) {
         uint32_t pk[8];
 #pragma unroll
         for (int i = 0; i < 16; i += 2) {
-          __nv_bfloat162 e2 = __floats2bfloat162_rn(tc::fast_exp2(fmaf(s[g][i], scale2, -base)), tc::fast_exp2(fmaf(s[g][i + 1], scale2, -base)));
-          rs[(i / 2) & 3] += __low2float(e2) + __high2float(e2);              // the rounded values, as the P V product sees them
-          pk[i / 2] = *reinterpret_cast<uint32_t*>(&e2);
+          float x0, x1;
+          tc::unpair(tc::fma2(tc::pair(s[g][i], s[g][i + 1]), sc2, nb), x0, x1);
+          const __nv_bfloat162 e2 = __floats2bfloat162_rn(tc::fast_exp2(x0), tc::fast_exp2(x1));
+          pk[i / 2] = *reinterpret_cast<const uint32_t*>(&e2);
+          rs[(i / 2) & 3] = tc::add2(rs[(i / 2) & 3], tc::pair_of_bf16(pk[i / 2]));      // the rounded values, as the P V product sees them
         }
         tc::tmem_st8_issue(ts + W / 2 * half + 8 * g, pk);
       }
-      l += (rs[0] + rs[1]) + (rs[2] + rs[3]);
+      float l0, l1;
+      tc::unpair(tc::add2(tc::add2(rs[0], rs[1]), tc::add2(rs[2], rs[3])), l0, l1);
+      l += l0 + l1;
       // every phase of pv_done is waited for before the next one can complete (a wait for a phase two behind never returns)
       if (t > 0 && ok && !tc::mbar_wait(&bars.pv_done[q], (t - 1) & 1)) ok = false;
       tc::tmem_st_wait();

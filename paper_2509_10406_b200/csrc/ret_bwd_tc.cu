@@ -19,7 +19,8 @@
 //
 // Bound: the tensor cores where clusters are long (7 products, 784 + 588 cycles per 128 x 64 tile at D = 64), else the
 // gather of rows (23-26 B/clk per SM).  16 heads of two sequences of 64k tokens, D = 64, 512 keys per cluster, 8 slots:
-// 16.86 ms in one kernel with five products per tile (ret_bwd_short_tc.cu, which short clusters keep), 5.26 + 3.46 ms here.
+// 16.86 ms in one kernel with five products per tile (ret_bwd_short_tc.cu, which short clusters keep), 5.30 + 3.40 ms here, 5.05 +
+// 3.34 with two numbers per instruction (local_bwd_tc.cu; in ret_bwd_short_tc.cu the same made 1614 us 1673).
 #include <cuda.h>
 #include "common.cuh"
 #include "tc05.cuh"
@@ -97,7 +98,7 @@ k_ret_bwd_dkdv(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_c
   __shared__ Bars bars;
   __shared__ uint32_t tbase_s;
   __shared__ int32_t ok_s[kOkCache], tok_s[4][kN];
-  __shared__ __align__(16) float Ls[NS][kN], ds[NS][kN];
+  __shared__ __align__(16) float Ls[NS][kN], ds[NS][kN];   // -L (log2 units) and -delta of each pair
   __shared__ __align__(16) int vs[NS][kN];                  // keys each pair of the tile sees, counted from the cluster's first
   RetItem item;
   if (!ret_item(ri, blockIdx.y, item)) return;
@@ -162,7 +163,7 @@ k_ret_bwd_dkdv(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_c
         wait(&bars.empty[s], ((n / NS) & 1) ^ 1);
         if (g < kN) {
           tok_s[n & 3][g] = tok;
-          Ls[s][g] = L * kLog2e; ds[s][g] = d_;
+          Ls[s][g] = -(L * kLog2e); ds[s][g] = -d_;
           vs[s][g] = tok < 0 ? 0 : gr.bucket ? gr.kall : ok[dm.causal ? tok / dm.Bs : 1] - gr.k0;
         }
         tc::named_bar_sync(1, LY::kGather);
@@ -247,6 +248,7 @@ k_ret_bwd_dkdv(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_c
     const int w = warp >> 2, row = tid & 127;
     const uint32_t tl = tbase + ((uint32_t)((warp & 3) * 32) << 16), ts = tl + (uint32_t)w * 2 * kN;
     const float scale2 = dm.sigma * kLog2e;
+    const uint64_t sc2 = tc::pair(scale2, scale2);
     int n = 0, sweep = 0;
     for (int kc = 0; kc < gr.kall; kc += kM) {
       const int t0 = first_tile(kc);
@@ -270,25 +272,26 @@ k_ret_bwd_dkdv(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_c
           tc::tmem_ld_use16(dp);
           float sn[16], dn_[16];
           if (q < 3) { tc::tmem_ld16_issue(ts + 16 * (q + 1), sn); tc::tmem_ld16_issue(ts + kN + 16 * (q + 1), dn_); }
-          float p[16];
+          if (!full) {                                     // (a branch for the whole group: masks of single entries cost three instructions each in every tile)
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const float4 a = *reinterpret_cast<const float4*>(&Ls[s][16 * q + 4 * k]), b = *reinterpret_cast<const float4*>(&ds[s][16 * q + 4 * k]);
-            const float Lc[4] = {a.x, a.y, a.z, a.w}, dc[4] = {b.x, b.y, b.z, b.w};
-            int4 vv = make_int4(0x7fffffff, 0x7fffffff, 0x7fffffff, 0x7fffffff);
-            if (!full) vv = *reinterpret_cast<const int4*>(&vs[s][16 * q + 4 * k]);
-            const int vc[4] = {vv.x, vv.y, vv.z, vv.w};
+            for (int k = 0; k < 4; ++k) {
+              const int4 vv = *reinterpret_cast<const int4*>(&vs[s][16 * q + 4 * k]);
+              const int vc[4] = {vv.x, vv.y, vv.z, vv.w};
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              const int c = 4 * k + e;
-              p[c] = tc::fast_exp2(fmaf(sv[c], scale2, -Lc[e]));
-              if (!full) p[c] = kc + row < vc[e] ? p[c] : 0.f;
-              dp[c] = p[c] * (dp[c] - dc[e]);
+              for (int e = 0; e < 4; ++e) sv[4 * k + e] = kc + row < vc[e] ? sv[4 * k + e] : -INFINITY;
             }
           }
           uint32_t pw[8], gw[8];
 #pragma unroll
-          for (int k = 0; k < 8; ++k) { pw[k] = pack2(p[2 * k], p[2 * k + 1]); gw[k] = pack2(dp[2 * k], dp[2 * k + 1]); }
+          for (int k = 0; k < 8; ++k) {
+            const uint64_t nl = *reinterpret_cast<const uint64_t*>(&Ls[s][16 * q + 2 * k]), nd = *reinterpret_cast<const uint64_t*>(&ds[s][16 * q + 2 * k]);
+            float x0, x1, g0, g1;
+            tc::unpair(tc::fma2(tc::pair(sv[2 * k], sv[2 * k + 1]), sc2, nl), x0, x1);
+            const float p0 = tc::fast_exp2(x0), p1 = tc::fast_exp2(x1);
+            tc::unpair(tc::mul2(tc::pair(p0, p1), tc::add2(tc::pair(dp[2 * k], dp[2 * k + 1]), nd)), g0, g1);
+            pw[k] = pack2(p0, p1);
+            gw[k] = pack2(g0, g1);
+          }
           tc::tmem_st8_issue(ts + 8 * q, pw);              // over logits already consumed
           tc::tmem_st8_issue(ts + kN + 8 * q, gw);
           if (q < 3) {
@@ -563,13 +566,14 @@ k_ret_bwd_dq(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_con
     const int w = warp >> 2, row = tid & 127;
     const uint32_t ts = tbase + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)w * 2 * kN;
     const float scale2 = dm.sigma * kLog2e;
+    const uint64_t sc2 = tc::pair(scale2, scale2);
     int n = 0;
     for (int i = 0; i < cnt; ++i) {
       const int b = i % NQ;
       wait(&bars.q_full[b], (i / NQ) & 1);
       const int T = T_s[b], vis = vs[b][row], vmin = vs[b][0];                 // (the first pair sees the fewest keys)
       const bool whole = pid_s[b][kM - 1] >= 0;
-      const float L2 = Ls[b][row], dl = ds[b][row];
+      const uint64_t nl = tc::pair(-Ls[b][row], -Ls[b][row]), nd = tc::pair(-ds[b][row], -ds[b][row]);
       tc::mbar_arrive(&bars.q_empty[b]);                   // (the scalars are in registers; the rows are the products' concern)
       for (int t = 0; t < T; ++t, ++n) {
         if (n % NW != w) continue;
@@ -587,15 +591,17 @@ k_ret_bwd_dq(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_con
           tc::tmem_ld_use16(dp);
           float sn[16], dn_[16];
           if (q < 3) { tc::tmem_ld16_issue(ts + 16 * (q + 1), sn); tc::tmem_ld16_issue(ts + kN + 16 * (q + 1), dn_); }
-#pragma unroll
-          for (int c = 0; c < 16; ++c) {
-            dp[c] = tc::fast_exp2(fmaf(sv[c], scale2, -L2)) * (dp[c] - dl);
-          }
           uint32_t gw[8];
 #pragma unroll
           for (int k = 0; k < 8; ++k) {
-            gw[k] = pack2(dp[2 * k], dp[2 * k + 1]);
-            if (!full) gw[k] = 16 * q + 2 * k + 1 < v ? gw[k] : 16 * q + 2 * k < v ? gw[k] & 0xffffu : 0u;
+            float x0, x1, g0, g1;
+            tc::unpair(tc::fma2(tc::pair(sv[2 * k], sv[2 * k + 1]), sc2, nl), x0, x1);
+            tc::unpair(tc::mul2(tc::pair(tc::fast_exp2(x0), tc::fast_exp2(x1)), tc::add2(tc::pair(dp[2 * k], dp[2 * k + 1]), nd)), g0, g1);
+            gw[k] = pack2(g0, g1);
+          }
+          if (!full) {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) gw[k] = 16 * q + 2 * k + 1 < v ? gw[k] : 16 * q + 2 * k < v ? gw[k] & 0xffffu : 0u;
           }
           tc::tmem_st8_issue(ts + 8 * q, gw);              // over logits already consumed
           if (q < 3) {

@@ -12,7 +12,8 @@
 // cores need not wait at a unit's end.  A pair's partial row is written once.
 //
 // Bound by the exponentials (16 per clock and SM) and the latency of a warp's pass over its logits.  16 heads of two
-// sequences of 64k tokens, D = 64, 512 keys per cluster, 8 slots: 7.32 ms with 128 resident keys per sweep, 4.29 ms here.
+// sequences of 64k tokens, D = 64, 512 keys per cluster, 8 slots: 7.32 ms with 128 resident keys per sweep, 4.40 ms here, 3.84
+// with two logits per instruction (local_fwd_tc.cu).
 #include <cuda.h>
 #include "common.cuh"
 #include "tc05.cuh"
@@ -233,6 +234,7 @@ k_ret_fwd_long(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_c
     const int q = warp / (4 * H), half = H == 2 ? (warp >> 2) & 1 : 0, row = tid & 127;
     const uint32_t tl = tbase + ((uint32_t)((warp & 3) * 32) << 16), to = tl + cO + q * D + half * OD;
     const float scale2 = dm.sigma * 1.4426950408889634f;
+    const uint64_t sc2 = tc::pair(scale2, scale2);
     constexpr float kLazy = 8.f;                           // see the local forward kernel
     int e = 0, n0 = q;                                     // products of this pair tile so far; number of the unit's first
     struct Ids { int pid, first, l0, l1; };
@@ -265,16 +267,16 @@ k_ret_fwd_long(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_c
 #pragma unroll
             for (int i = 0; i < 16; ++i) s[g][i] = 16 * g + i < lim ? s[g][i] : -INFINITY;
         }
-        float mx[4];
+        float mx[W / 16];                                    // (three at a time)
 #pragma unroll
-        for (int g = 0; g < 4; ++g) {
-          mx[g] = s[g][0];
+        for (int g = 0; g < W / 16; ++g) {
+          mx[g] = fmaxf(s[g][0], s[g][1]);
 #pragma unroll
-          for (int k = g; k < W / 16; k += 4)
-#pragma unroll
-            for (int i = 0; i < 16; ++i) mx[g] = fmaxf(mx[g], s[k][i]);
+          for (int i = 2; i < 16; i += 2) mx[g] = tc::max3(mx[g], s[g][i], s[g][i + 1]);
         }
-        const float mt = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * scale2;
+#pragma unroll
+        for (int g = W / 16 - 1; g > 0; --g) mx[g - 1] = fmaxf(mx[g - 1], mx[g]);
+        const float mt = mx[0] * scale2;
         // (also: both halves have read their logits before either writes P over them)
         const bool grow = t == 0 || mt > m2 + kLazy;
         if (H == 2 ? bar_or(1 + q, kSoft / 2, grow) : __any_sync(0xffffffffu, grow)) {
@@ -289,32 +291,39 @@ k_ret_fwd_long(Dims dm, const __grid_constant__ CUtensorMap tm_k, const __grid_c
             wait(&bars.pv_done[q], (e - 1) & 1);           // (complete ever since: the wait below returns at once)
             tc::fence_after_sync();
             const float resc = mn == -INFINITY ? 1.f : tc::fast_exp2(m2 - mn);
+#pragma unroll 1
+            for (int d0 = 0; d0 < OD; d0 += 16) {            // (16 at a time: the logits stay in registers meanwhile)
+              float v[16];
+              uint32_t x[16];
+              tc::tmem_ld16(to + d0, v);
 #pragma unroll
-            for (int d0 = 0; d0 < OD; d0 += 32) {
-              float v[32];
-              tc::tmem_ld32(to + d0, v);
-#pragma unroll
-              for (int i = 0; i < 32; ++i) v[i] *= resc;
-              tc::tmem_st32(to + d0, v);
+              for (int i = 0; i < 16; ++i) x[i] = __float_as_uint(v[i] * resc);
+              tc::tmem_st16_issue(to + d0, x);
             }
+            tc::tmem_st_wait();
             l *= resc;
           }
           m2 = mn;
         }
         const float base = m2 == -INFINITY ? 0.f : m2;
-        float rs[4] = {0.f, 0.f, 0.f, 0.f};
+        const uint64_t nb = tc::pair(-base, -base);
+        uint64_t rs[4] = {0u, 0u, 0u, 0u};                   // (pairs of zeros)
 #pragma unroll
         for (int g = 0; g < W / 16; ++g) {
           uint32_t pk2[8];
 #pragma unroll
           for (int i = 0; i < 16; i += 2) {
-            __nv_bfloat162 e2 = __floats2bfloat162_rn(tc::fast_exp2(fmaf(s[g][i], scale2, -base)), tc::fast_exp2(fmaf(s[g][i + 1], scale2, -base)));
-            rs[(i / 2) & 3] += __low2float(e2) + __high2float(e2);            // the rounded values, as the P V product sees them
-            pk2[i / 2] = *reinterpret_cast<uint32_t*>(&e2);
+            float x0, x1;
+            tc::unpair(tc::fma2(tc::pair(s[g][i], s[g][i + 1]), sc2, nb), x0, x1);
+            const __nv_bfloat162 e2 = __floats2bfloat162_rn(tc::fast_exp2(x0), tc::fast_exp2(x1));
+            pk2[i / 2] = *reinterpret_cast<const uint32_t*>(&e2);
+            rs[(i / 2) & 3] = tc::add2(rs[(i / 2) & 3], tc::pair_of_bf16(pk2[i / 2]));      // the rounded values, as the P V product sees them
           }
           tc::tmem_st8_issue(ts + W / 2 * half + 8 * g, pk2);
         }
-        l += (rs[0] + rs[1]) + (rs[2] + rs[3]);
+        float l0, l1;
+        tc::unpair(tc::add2(tc::add2(rs[0], rs[1]), tc::add2(rs[2], rs[3])), l0, l1);
+        l += l0 + l1;
         if (e > 0) wait(&bars.pv_done[q], (e - 1) & 1);    // every phase is waited for, before the next one can complete
         tc::tmem_st_wait();
         tc::fence_before_sync();

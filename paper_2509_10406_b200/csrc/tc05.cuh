@@ -302,6 +302,36 @@ __device__ __forceinline__ float fast_exp2(float x) {
   return y;
 }
 
+// ---- two fp32 numbers per instruction (the same roundings as one by one) and a maximum of three ----------------
+__device__ __forceinline__ uint64_t pair(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void unpair(uint64_t v, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ float max3(float a, float b, float c) {
+  float r;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+// the two numbers of a packed bf16 pair
+__device__ __forceinline__ uint64_t pair_of_bf16(uint32_t v) { return pair(__uint_as_float(v << 16), __uint_as_float(v & 0xffff0000u)); }
+
 // ---- swizzled shared-memory tiles ------------------------------------------------------------------------
 // Zeros the rows [r, end) of a swizzled tile of G column groups [ROWS][128 B] that TMA has filled; the whole warp, which then
 // issues the products that read them.  (What a box brought beside the rows that count must not meet a weight of 0: 0 * NaN is NaN.)
