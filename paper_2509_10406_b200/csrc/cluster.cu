@@ -1,6 +1,6 @@
 // Clustering stage: Lloyd k-means (Appendix "Clustering Details").  The query side and the key side are independent
 // problems of the same shape of work, so every kernel takes both in one launch: an iteration is three launches
-// (assignment, bucket_sort, k_update); small bf16 problems take all iterations in one (lloyd_small.cu).
+// (assignment, bucket_sort, k_update); small problems take all iterations in one (lloyd_small.cu).
 #include "common.cuh"
 #include "feistel.cuh"
 
@@ -293,11 +293,9 @@ static int lloyd_t(LloydSides& g, const Dims& d, int nsides, int init_mode, uint
   }
   prof_mark("k_init_centres", st);
   MUSE_RC(launch_pdl(k_init_centres<T>, dim3((unsigned)((centres + 7) / 8)), 256, 0, st, g, D, init_mode, seed, clear));
-  if (sizeof(T) == 2) {
-    bool taken = false;
-    MUSE_RC(lloyd_small(d, g.s, nsides, T_iters, &taken, status, st));
-    if (taken) return MUSE_OK;
-  }
+  bool taken = false;
+  MUSE_RC(lloyd_small(d, sizeof(T) == 2 ? MUSE_BF16 : MUSE_F32, g.s, nsides, T_iters, &taken, status, st));
+  if (taken) return MUSE_OK;
   for (int it = 0; it <= T_iters; ++it) {
     const bool last = it == T_iters;
     if (sizeof(T) == 2) {                      // bf16 inputs: distances on the tensor cores

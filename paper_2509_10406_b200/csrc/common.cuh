@@ -262,8 +262,8 @@ int cluster_check(const muse_params_t* p, const void* Q, const void* K, const in
                   int32_t* assign_k, float* qbar, float* kcent, size_t ws_bytes, bool may_split, ClusterCall* c);
 int cluster_launch(ClusterCall& c, void* ws, cudaStream_t st);
 size_t lloyd_ws_bytes(const Dims& d, int problems, int C);      // scratch of one side (without the status words)
-// all iterations of small bf16 problems in one launch after the start (lloyd_small.cu); *taken: they qualified and the launch was made
-int lloyd_small(const Dims& d, const LloydSide* sides, int nsides, int T, bool* taken, int* status, cudaStream_t st);
+// all iterations of small problems in one launch after the start (lloyd_small.cu); *taken: they qualified and the launch was made
+int lloyd_small(const Dims& d, int dtype, const LloydSide* sides, int nsides, int T, bool* taken, int* status, cudaStream_t st);
 int assign_tc(const LloydSide* sides, int nsides, int N, int D, int distances, int* status, cudaStream_t st);
 int assign_distances(const Dims& d, int dtype, const LloydSide& side, int* status, cudaStream_t st);   // after lloyd on the same centres
 

@@ -1,9 +1,11 @@
-// Lloyd iterations of small problems in one launch (bf16 inputs; cluster.cu has the start and, for the others, a chain of launches).  A problem (one
+// Lloyd iterations of small problems in one launch (cluster.cu has the start and, for the others, a chain of launches).  A problem (one
 // head's queries or keys) is owned by one thread-block cluster: its CTAs split the points for the assignment and the centres for the
 // update, and two cluster barriers an iteration take the place of three launches:
 //   centres     every CTA reads all centres (fp32) and lays them out as bf16 hi + lo tiles, as the assignment kernel's operands
 //   assignment  |c|^2 - 2 x.c over tiles of 128 points: points by TMA through a ring, products by tcgen05 into up to four
 //               accumulators, four warps an accumulator take the arg-min                        (same products, same order: assign_tc.cu)
+//               (fp32 inputs: FFMA, 32 points at least a CTA, two or four points by one to four centres a thread, all centres in shared
+//               memory; a thread's centres are 16 apart, so that its lanes read all banks)
 //   sort        every CTA collects the points of ITS centres in order, as 16-bit numbers in shared memory (a stable counting sort)
 //   update      two warps a centre; the fixed reduction tree of k_update, so that every bit of a centre is the chain's
 // The arrays of the assignment (centre and point tiles) and of the update (counts, lists, partial sums) share the CTA's memory.
@@ -12,9 +14,10 @@
 // a centre's rows (L2 again; from some hundred rows on the SM's rate of scattered rows, 18 to 26 bytes a clock), barriers 1000 each.
 // Three iterations, chain | here, us: 4 heads of 2k points, D = 128, 32 and 128 centres 66 | 44; 16 heads of 8k, D = 64, 64 and 128
 // 154 | 106; 12 heads of 5005, 37 and 90 96 | 63; 24 heads of 4k, 64 and 128 140 | 121 (48 problems: two CTAs each, not three);
-// 64 heads of 1k, 16 and 32 156 | 54.
+// 64 heads of 1k, 16 and 32 156 | 54.  fp32: the rule at the end of the plan.
 #include <cooperative_groups.h>
 #include <cuda.h>
+#include <type_traits>
 #include "common.cuh"
 #include "tc05.cuh"
 
@@ -30,11 +33,15 @@ constexpr int kThreads = 512, kGroups = 4;                 // a group: four warp
 constexpr int kRows = 128, kMaxCentres = 256, kMaxStages = 8, kTeam = 64, kTeams = kThreads / kTeam, kMaxSegs = 1024;
 constexpr int kMaxCluster = 16, kMaxSmem = 220 * 1024;
 struct Bars { uint64_t xfull[kMaxStages], done[kGroups], read[kGroups]; };
-struct Side { const bf16* X; int32_t* assign; float *centres, *cnorm; int problems, C, kind; };
+struct Side { const void* X; int32_t* assign; float *centres, *cnorm; int problems, C, kind; };
 struct Args { Side s[2]; int N, S, Bs, T, nx; };
 
 __host__ __device__ inline int segs(int C, int CL, int kind, int S) { return (C + CL - 1) / CL * (kind == 0 ? S : 1); }
 __host__ __device__ inline int centre_bytes(int C, int D) { return 2 * ((C + 127) / 128) * 128 * D * 2; }
+// fp32: points of a CTA; rows of centres and points in shared memory, 16 bytes longer than their contents
+__host__ __device__ inline int share_f32(int N, int CL) { return ((N + CL - 1) / CL + 31) & ~31; }
+__host__ __device__ inline int tile_f32(int share) { return share > 64 ? 128 : 64; }
+__host__ __device__ inline int assign_bytes_f32(int N, int C, int CL, int D) { return (((C + 15) & ~15) + tile_f32(share_f32(N, CL))) * (D + 4) * 4; }
 __host__ __device__ inline int stretch(int N) { return ((N + 15) / 16 + 31) & ~31; }   // points that a warp sorts
 // update: partial sums | counts [16][segs] | first places [segs + 1] | list | the warps' points
 __host__ __device__ inline int update_bytes(int C, int CL, int kind, int N, int S) {
@@ -42,12 +49,66 @@ __host__ __device__ inline int update_bytes(int C, int CL, int kind, int N, int 
 }
 }  // namespace ls
 
-template <int D>
+// fp32: arg-min over all centres (Cs: rows of D + 4) for RPT points of a thread (Xs: rows row, row + 1, ...); distances as k_assign has them
+template <int D, int RPT>
+__device__ __forceinline__ void assign_rows_f32(const float* Xs, const float* Cs, const float* cn, int C16, int tx, int row, float (&best)[RPT], int (&bidx)[RPT]) {
+  constexpr int LD = D + 4;
+#pragma unroll
+  for (int r = 0; r < RPT; ++r) { best[r] = INFINITY; bidx[r] = 0x7fffffff; }
+  auto chunk = [&](int c0, auto groups) {                  // 16 centres per group
+    constexpr int CG = decltype(groups)::value;
+    float acc[RPT][CG];
+#pragma unroll
+    for (int r = 0; r < RPT; ++r)
+#pragma unroll
+      for (int k = 0; k < CG; ++k) acc[r][k] = 0.f;
+#pragma unroll 4
+    for (int d = 0; d < D; d += 4) {
+      float4 cv[CG];
+#pragma unroll
+      for (int k = 0; k < CG; ++k) cv[k] = ld4(Cs + (c0 + 16 * k + tx) * LD + d);
+#pragma unroll
+      for (int r = 0; r < RPT; ++r) {
+        const float4 xv = ld4(Xs + (row + r) * LD + d);
+#pragma unroll
+        for (int k = 0; k < CG; ++k) {
+          acc[r][k] = fmaf(xv.x, cv[k].x, acc[r][k]);
+          acc[r][k] = fmaf(xv.y, cv[k].y, acc[r][k]);
+          acc[r][k] = fmaf(xv.z, cv[k].z, acc[r][k]);
+          acc[r][k] = fmaf(xv.w, cv[k].w, acc[r][k]);
+        }
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < CG; ++k)
+#pragma unroll
+      for (int r = 0; r < RPT; ++r) {
+        const int c = c0 + 16 * k + tx;
+        const float dist = fmaf(-2.f, acc[r][k], cn[c]);
+        if (dist < best[r]) { best[r] = dist; bidx[r] = c; }          // ascending c: ties keep the lower
+      }
+  };
+  int c0 = 0;
+  for (; c0 + 64 <= C16; c0 += 64) chunk(c0, std::integral_constant<int, 4>());
+  if (C16 - c0 >= 32) { chunk(c0, std::integral_constant<int, 2>()); c0 += 32; }
+  if (C16 - c0 >= 16) chunk(c0, std::integral_constant<int, 1>());
+#pragma unroll
+  for (int r = 0; r < RPT; ++r)
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) {
+      const float ob = __shfl_xor_sync(0xffffffffu, best[r], o);
+      const int oi = __shfl_xor_sync(0xffffffffu, bidx[r], o);
+      argmin_tie_step(ob, oi, best[r], bidx[r]);
+    }
+}
+
+template <class T, int D>
 __global__ void __launch_bounds__(ls::kThreads, 1)
 k_lloyd_small(const __grid_constant__ CUtensorMap tx0, const __grid_constant__ CUtensorMap tx1, const __grid_constant__ ls::Args g, int* __restrict__ status) {
   using namespace ls;
   constexpr int kTile = kRows * D * 2, G = D / 64;
-  constexpr int LPR = D / 8, SLOTS = 256 / LPR, RPT = kTeam / LPR, SG = SLOTS / RPT;   // k_update's slots; rows of a team's pass; passes
+  constexpr bool F32 = sizeof(T) == 4;
+  constexpr int VEC = 16 / (int)sizeof(T), LPR = D / VEC, SLOTS = 256 / LPR, RPT = kTeam / LPR, SG = SLOTS / RPT;   // k_update's slots; rows of a team's pass; passes
   extern __shared__ __align__(1024) unsigned char sm_raw[];
   __shared__ Bars bars;
   __shared__ uint32_t tbase_s;
@@ -66,12 +127,12 @@ k_lloyd_small(const __grid_constant__ CUtensorMap tx0, const __grid_constant__ C
   const int tiles = (N + kRows - 1) / kRows, tper = (tiles + CL - 1) / CL, tile0 = min(tiles, rank * tper), nt = min(tiles, tile0 + tper) - tile0;
   const int nx = nt <= g.nx ? max(nt, 1) : g.nx > 4 ? g.nx & ~3 : g.nx, ng = min(nx, kGroups);     // ring stages, working groups (a stage is always the same group's)
   const int cper = (C + CL - 1) / CL, c0 = min(C, rank * cper), c1 = min(C, c0 + cper);
-  const bf16* Xp = sd.X + (size_t)prob * N * D;
+  const T* Xp = (const T*)sd.X + (size_t)prob * N * D;
   int32_t* as = sd.assign + (size_t)prob * N;
   float* cen = sd.centres + (size_t)prob * C * D;
   float* cnp = sd.cnorm + (size_t)prob * NT * 128;
-  if (warp == 0) tc::tmem_alloc(&tbase_s, 512);
-  if (tid == 0) {
+  if (!F32 && warp == 0) tc::tmem_alloc(&tbase_s, 512);
+  if (!F32 && tid == 0) {
     for (int s = 0; s < kMaxStages; ++s) tc::mbar_init(&bars.xfull[s], 1);
     for (int b = 0; b < kGroups; ++b) { tc::mbar_init(&bars.done[b], 1); tc::mbar_init(&bars.read[b], kRows); }
     tc::mbar_init_fence();
@@ -79,7 +140,7 @@ k_lloyd_small(const __grid_constant__ CUtensorMap tx0, const __grid_constant__ C
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
-  const uint32_t tbase = tbase_s;
+  const uint32_t tbase = F32 ? 0u : tbase_s;
   pdl_wait();
   pdl_trigger();
   bool ok = true;                                          // false once a bounded wait ran out (every role still walks all its tiles)
@@ -87,6 +148,37 @@ k_lloyd_small(const __grid_constant__ CUtensorMap tx0, const __grid_constant__ C
 
   int turn = 0;                                            // products of this group so far
   for (int it = 0;; ++it) {
+    if constexpr (F32) {
+      constexpr int LD = D + 4;
+      const int share = share_f32(N, CL), r0 = min(N, rank * share), r1 = min(N, r0 + share), rows = tile_f32(share), C16 = (C + 15) & ~15;
+      float* Cs = reinterpret_cast<float*>(sm);
+      float* Xs = Cs + C16 * LD;
+      for (int e = tid; e < C16 * (D / 4); e += kThreads) {
+        const int r = e / (D / 4), q = 4 * (e % (D / 4));
+        st4(Cs + r * LD + q, r < C ? __ldcg(reinterpret_cast<const float4*>(cen + (size_t)r * D + q)) : make_float4(0.f, 0.f, 0.f, 0.f));
+      }
+      for (int r = tid; r < C16; r += kThreads) cn_s[r] = r < C ? __ldcg(cnp + r) : INFINITY;
+      for (int row0 = r0; row0 < r1; row0 += rows) {
+        if (row0 > r0) __syncthreads();
+        for (int e = tid; e < rows * (D / 4); e += kThreads) {
+          const int r = e / (D / 4), q = 4 * (e % (D / 4));
+          st4(Xs + r * LD + q, row0 + r < r1 ? ld4((const float*)Xp + (size_t)(row0 + r) * D + q) : make_float4(0.f, 0.f, 0.f, 0.f));
+        }
+        __syncthreads();
+        auto points = [&](auto per) {
+          constexpr int RPT_ = decltype(per)::value;
+          const int row = (tid >> 4) * RPT_;
+          float best[RPT_];
+          int bidx[RPT_];
+          assign_rows_f32<D, RPT_>(Xs, Cs, cn_s, C16, tid & 15, row, best, bidx);
+#pragma unroll
+          for (int r = 0; r < RPT_; ++r)                   // a row of NaN or infinities never compares below the running minimum: it goes to cluster 0
+            if ((tid & 15) == 0 && row0 + row + r < r1) as[row0 + row + r] = (unsigned)bidx[r] < (unsigned)C ? bidx[r] : 0;
+        };
+        if (rows == 64) points(std::integral_constant<int, 2>());
+        else points(std::integral_constant<int, 4>());
+      }
+    } else {
     unsigned char* Xs = sm + 2 * NT * kTile;
     auto load = [&](int i) {                               // point tile i into its stage of the ring
       const int st_ = i % nx;
@@ -175,6 +267,7 @@ k_lloyd_small(const __grid_constant__ CUtensorMap tx0, const __grid_constant__ C
         if (ok && at < N) as[at] = (unsigned)bidx[0] < (unsigned)C ? bidx[0] : 0;
       }
     }
+    }
     if (it == g.T) break;
     cluster.sync();                                        // every assignment of the problem has been written; the tiles have been read
 
@@ -185,7 +278,7 @@ k_lloyd_small(const __grid_constant__ CUtensorMap tx0, const __grid_constant__ C
       int* hist = reinterpret_cast<int*>(part + kTeams * SLOTS * D);                   // [16][nseg] counts of a warp's stretch, then its first place in the segment
       int* first = hist + 16 * nseg;                       // [nseg + 1]
       uint16_t* list = reinterpret_cast<uint16_t*>(first + (nseg + 4) / 4 * 4);        // [N] points by segment
-            for (int k = tid; k < 16 * nseg; k += kThreads) hist[k] = 0;
+      for (int k = tid; k < 16 * nseg; k += kThreads) hist[k] = 0;
       __syncthreads();
       const int wl = stretch(N), w0 = min(N, warp * wl), w1 = min(N, w0 + wl);
       uint32_t* own = reinterpret_cast<uint32_t*>(list + (N + 7) / 8 * 8) + warp * wl; // segment | point of this warp's stretch, this CTA's centres only
@@ -243,27 +336,29 @@ k_lloyd_small(const __grid_constant__ CUtensorMap tx0, const __grid_constant__ C
         __syncwarp();
       }
       __syncthreads();
-      // ---- update: thread = (row of a pass, 8 dims); slot s of a centre adds the members s, s + SLOTS, ... of a segment in order
+      // ---- update: thread = (row of a pass, 16 bytes of it); slot s of a centre adds the members s, s + SLOTS, ... of a segment in order
       const int team = warp >> 1, tt = tid & (kTeam - 1), sub = tt / LPR, q = tt % LPR;
-      const bf16* Xq = Xp + q * 8;
+      const T* Xq = Xp + q * VEC;
       float* pt = part + team * SLOTS * D;
       for (int c = c0 + team; c < c1; c += kTeams) {
-        float s[SG][8];
+        float s[SG][VEC];
 #pragma unroll
         for (int x = 0; x < SG; ++x)
 #pragma unroll
-          for (int k = 0; k < 8; ++k) s[x][k] = 0.f;
+          for (int k = 0; k < VEC; ++k) s[x][k] = 0.f;
         const int* f = first + (c - c0) * Sx;
         const int count = f[Sx] - f[0];
-        auto load = [&](int at, int end) {                 // 8 dims of a member's row; past the segment's end zeros
+        auto load = [&](int at, int end) {                 // 16 bytes of a member's row; past the segment's end zeros
           uint4 v = make_uint4(0u, 0u, 0u, 0u);
           if (at < end && MUSE_IN_RANGE(at, N)) v = *reinterpret_cast<const uint4*>(Xq + (size_t)list[at] * D);
           return v;
         };
-        auto add = [&](const uint4& v, float (&t)[8]) {
+        auto add = [&](const uint4& v, float (&t)[VEC]) {
           const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-          for (int k = 0; k < 4; ++k) { t[2 * k] += __uint_as_float(w[k] << 16); t[2 * k + 1] += __uint_as_float(w[k] & 0xffff0000u); }
+          for (int k = 0; k < 4; ++k)
+            if constexpr (F32) t[k] += __uint_as_float(w[k]);
+            else { t[2 * k] += __uint_as_float(w[k] << 16); t[2 * k + 1] += __uint_as_float(w[k] & 0xffff0000u); }
         };
         // a step is SLOTS members of a segment or its rest; four steps at a time, whose rows are in flight together: all of them where the
         // segments are short (half the slots at most), in two halves otherwise
@@ -300,7 +395,10 @@ k_lloyd_small(const __grid_constant__ CUtensorMap tx0, const __grid_constant__ C
           }
         }
 #pragma unroll
-        for (int x = 0; x < SG; ++x) st8(pt + (x * RPT + sub) * D + q * 8, s[x]);
+        for (int x = 0; x < SG; ++x) {
+#pragma unroll
+          for (int k = 0; k < VEC; k += 4) st4(pt + (x * RPT + sub) * D + q * VEC + k, make_float4(s[x][k], s[x][k + 1], s[x][k + 2], s[x][k + 3]));
+        }
         tc::named_bar_sync(1 + team, kTeam);
 #pragma unroll
         for (int e = 0; e < D / kTeam; ++e) {
@@ -333,18 +431,19 @@ k_lloyd_small(const __grid_constant__ CUtensorMap tx0, const __grid_constant__ C
   }
   tc::fence_before_sync();
   __syncthreads();
-  if (warp == 0) tc::tmem_dealloc(tbase, 512);
+  if (!F32 && warp == 0) tc::tmem_dealloc(tbase, 512);
 }
 
 // CTAs per problem: the most (up to 16, of at least one tile of points each) for which every problem's cluster is resident at once; 0
 // where the problems do not qualify.
-template <int D>
+template <class T, int D>
 static int lloyd_small_plan(const ls::Args& g, int nsides, size_t* smem, int* nx) {
   using namespace ls;
+  constexpr bool F32 = sizeof(T) == 4;
   int problems = 0, C = 0;
   for (int k = 0; k < nsides; ++k) { problems += g.s[k].problems; C = C > g.s[k].C ? C : g.s[k].C; }
   if (C > kMaxCentres || g.N > 16384 || problems > sm_count()) return 0;
-  const int tile = kRows * D * 2, cb = centre_bytes(C, D), tiles = cdiv(g.N, kRows);
+  const int tile = kRows * D * 2, cb = centre_bytes(C, D), tiles = cdiv(g.N, F32 ? 32 : kRows);
   int cl = sm_count() / problems;
   if (cl >= 16 && tiles >= 16) cl = 16;
   else if (cl > 8) cl = 8;
@@ -357,13 +456,30 @@ static int lloyd_small_plan(const ls::Args& g, int nsides, size_t* smem, int* nx
       up = u > up ? u : up;
       seg = s > seg ? s : seg;
     }
-    *nx = (kMaxSmem - cb) / tile;
-    if (*nx > kMaxStages) *nx = kMaxStages;
-    if (*nx > per) *nx = per;
-    const size_t need = cb + (size_t)*nx * tile > (size_t)up ? cb + (size_t)*nx * tile : (size_t)up;
-    if (seg > kMaxSegs || need > (size_t)kMaxSmem || *nx < 1) return 0;      // (fewer CTAs need more)
+    size_t need;
+    if (F32) {
+      need = (size_t)assign_bytes_f32(g.N, C, cl, D);
+    } else {
+      *nx = (kMaxSmem - cb) / tile;
+      if (*nx > kMaxStages) *nx = kMaxStages;
+      if (*nx > per) *nx = per;
+      if (*nx < 1) return 0;
+      need = cb + (size_t)*nx * tile;
+    }
+    if (need < (size_t)up) need = up;
+    if (seg > kMaxSegs || need > (size_t)kMaxSmem) return 0;                 // (fewer CTAs need more)
     *smem = need + 1024;
-    if (max_clusters(k_lloyd_small<D>, kThreads, *smem, cl) < problems) continue;
+    if (max_clusters(k_lloyd_small<T, D>, kThreads, *smem, cl) < problems) continue;
+    if (F32) {
+      // Against the chain, whose assignment has tiles of its own for problems that fill the chip, at 168 sizes (1 to 32 heads of 1k to 9k
+      // points, 8 to 256 centres; three iterations, chain | here, us, D = 64): 2 problems of 1k, 16 centres 49 | 37, 256 centres 208 | 71;
+      // 16 of 2k, 128 centres 277 | 137; 32 of 2k, 16 centres 185 | 87.  Few centres over a long problem are a pass over the points that
+      // every CTA repeats (2 of 4k, 16 centres 60 | 67), and where the chip is full many centres are FFMA work that the chain spreads
+      // better (16 of 4k, 128 centres 232 | 249).
+      const bool full = (long long)problems * cdiv(g.N, kRows) >= 2 * sm_count();
+      const bool take = C <= 16 ? full || g.N <= 2048 : full ? g.N <= 2048 && g.N * C <= 2048 * 128 : g.N <= 4096;
+      return take ? cl : 0;
+    }
     // The chain spreads the products over all SMs and pays for its launches, and for a problem's share of them; this kernel uses the SMs of
     // its clusters.  Work: products of a CTA in tiles of 128 x 128 x 64; idle: the SMs without a CTA.  The line lies where most of 230
     // sizes (1 to 64 heads of 1k to 16k points, 32 to 256 centres) cross: within it 1.1 to 2.9 times the chain's speed (a few at 0.95 to
@@ -375,33 +491,36 @@ static int lloyd_small_plan(const ls::Args& g, int nsides, size_t* smem, int* nx
   return 0;
 }
 
-template <int D>
+template <class T, int D>
 static int lloyd_small_d(ls::Args& g, int nsides, bool* taken, int* status, cudaStream_t st) {
   size_t smem;
-  const int cl = lloyd_small_plan<D>(g, nsides, &smem, &g.nx);
+  g.nx = 0;
+  const int cl = lloyd_small_plan<T, D>(g, nsides, &smem, &g.nx);
   if (cl == 0) return MUSE_OK;
   *taken = true;
-  CUtensorMap m[2];
+  CUtensorMap m[2] = {};                                   // (fp32: not used)
   int problems = 0;
   for (int k = 0; k < 2; ++k) {
     const ls::Side& s = g.s[k < nsides ? k : 0];           // (a missing side's map is never used)
-    MUSE_RC(make_tmap_bf16_rows(&m[k], s.X, (uint64_t)s.problems * g.N, (uint32_t)D, ls::kRows));
+    if (sizeof(T) == 2) MUSE_RC(make_tmap_bf16_rows(&m[k], s.X, (uint64_t)s.problems * g.N, (uint32_t)D, ls::kRows));
     if (k < nsides) problems += s.problems;
   }
   prof_mark("k_lloyd_small", st);
-  return launch_pdl_cluster(k_lloyd_small<D>, dim3(problems * cl), ls::kThreads, smem, cl, st, m[0], m[1], g, status);
+  return launch_pdl_cluster(k_lloyd_small<T, D>, dim3(problems * cl), ls::kThreads, smem, cl, st, m[0], m[1], g, status);
 }
 
-int lloyd_small(const Dims& d, const LloydSide* sides, int nsides, int T, bool* taken, int* status, cudaStream_t st) {
+int lloyd_small(const Dims& d, int dtype, const LloydSide* sides, int nsides, int T, bool* taken, int* status, cudaStream_t st) {
   *taken = false;
   if (T < 1 || path_forced(kForceLloydChain)) return MUSE_OK;  // (the balanced assignment, T = 0, goes on to use the planes that the chain writes)
   ls::Args g = {};
   for (int k = 0; k < nsides; ++k) {
     const LloydSide& s = sides[k];
-    g.s[k] = ls::Side{(const bf16*)s.X, s.assign, s.centres, s.cnorm, s.problems, s.C, s.kind};
+    g.s[k] = ls::Side{s.X, s.assign, s.centres, s.cnorm, s.problems, s.C, s.kind};
   }
   g.N = d.N; g.S = d.S; g.Bs = d.Bs; g.T = T;
-  return d.D == 64 ? lloyd_small_d<64>(g, nsides, taken, status, st) : lloyd_small_d<128>(g, nsides, taken, status, st);
+  if (dtype == MUSE_F32)
+    return d.D == 64 ? lloyd_small_d<float, 64>(g, nsides, taken, status, st) : lloyd_small_d<float, 128>(g, nsides, taken, status, st);
+  return d.D == 64 ? lloyd_small_d<bf16, 64>(g, nsides, taken, status, st) : lloyd_small_d<bf16, 128>(g, nsides, taken, status, st);
 }
 
 }  // namespace muse
