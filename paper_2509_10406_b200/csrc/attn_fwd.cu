@@ -515,9 +515,15 @@ static int attn_fwd_t(const Dims& d, const T* Q, const T* K, const T* V, const i
   if (two_level && !kTensorT<T>()) return MUSE_ERR_UNSUPPORTED;   // spatial block selection is built on the bf16 retrieval kernel
   const size_t fl_smem = 3 * tile_bytes<T, D>() + ptile_bytes();
   constexpr bool kTensor = sizeof(T) == 2;      // bf16 mode runs the exact-attention parts on tcgen05
-  // (the first kernel: also clears the status words)
-  prof_mark("k_far_defaults", st);
-  MUSE_RC(launch_pdl(k_far_defaults, dim3(cdiv(d.N, 256), pq), 256, 0, st, d, w.lse_far, sel, w.status));
+  // the first kernel clears the status words and writes what queries without a far field get
+  if (d.SB > 0) {
+    const SortSide side = {assign_q, w.off_q, w.perm_q, pq, d.Cq, 0};
+    const FarDefaults none = {w.lse_far, sel, d.m};
+    MUSE_RC(bucket_sort(&side, 1, d.N, d.S, d.Bs, st, w.status, d.causal ? &none : nullptr));
+  } else {
+    prof_mark("k_far_defaults", st);
+    MUSE_RC(launch_pdl(k_far_defaults, dim3(cdiv(d.N, 256), pq), 256, 0, st, d, w.lse_far, sel, w.status));
+  }
   // local attention
   if (d.causal && kTensor) {
     int rc = local_fwd_tc(d, Q, K, V, w.o_loc, w.lse_loc, w.status, st);
@@ -528,9 +534,7 @@ static int attn_fwd_t(const Dims& d, const T* Q, const T* K, const T* V, const i
     MUSE_RC(launch_pdl(k_local_fwd<T, D>, dim3(d.S * cdiv(d.Bs, kTile), pq), kFlashThreads, fl_smem, st, d, Q, K, V, w.o_loc, w.lse_loc));
   }
   if (d.SB > 0) {
-    const SortSide side = {assign_q, w.off_q, w.perm_q, pq, d.Cq, 0};
-    int rc = bucket_sort(&side, 1, d.N, d.S, d.Bs, st);
-    if (rc != MUSE_OK) return rc;
+    int rc = MUSE_OK;
     if (far_fwd_tc_supported(d, dtype) && !path_forced(kForceFarSimt)) {
       rc = far_fwd_tc(d, summ_ptrs(L, base), Q, w.off_q, w.perm_q, sel_in, sel, w.o_far, w.lse_far, w.status, st);
       if (rc != MUSE_OK) return rc;

@@ -19,7 +19,7 @@ namespace muse {
 // took turns), both sides of a clustering iteration: 8192 tokens x 16 heads 90 -> 13 us, 65536 tokens x 4 heads 145 -> 25 us.
 constexpr int kSortMaxCluster = 8;
 
-struct SortArgs { SortSide s[2]; int N, S, Bs, q; int32_t* clear; };
+struct SortArgs { SortSide s[2]; int N, S, Bs, q; int32_t* clear; FarDefaults none; };
 
 __global__ void __launch_bounds__(512)
 k_bucket_sort(const __grid_constant__ SortArgs g) {
@@ -39,6 +39,11 @@ k_bucket_sort(const __grid_constant__ SortArgs g) {
   pdl_wait();
   pdl_trigger();
   if (g.clear != nullptr && blockIdx.x == 0 && tid < kStatusWords) g.clear[tid] = 0;
+  if (g.none.lse != nullptr && !second) {                  // (stores that nothing here waits for)
+    const int step = CL * nt, nm = g.Bs * g.none.m;
+    for (int e = rank * nt + tid; e < g.Bs; e += step) g.none.lse[(size_t)prob * N + e] = -INFINITY;
+    for (int e = rank * nt + tid; e < nm; e += step) g.none.sel[(size_t)prob * N * g.none.m + e] = -1;
+  }
   const int32_t* a = sd.assign + (size_t)prob * N;
   int32_t* pm = sd.perm + (size_t)prob * N;
   int32_t* off = sd.off + (size_t)prob * ((size_t)C * S + 1);
@@ -149,11 +154,12 @@ k_bucket_sort(const __grid_constant__ SortArgs g) {
   }
 }
 
-int bucket_sort(const SortSide* sides, int nsides, int N, int S, int Bs, cudaStream_t st, int32_t* clear) {
+int bucket_sort(const SortSide* sides, int nsides, int N, int S, int Bs, cudaStream_t st, int32_t* clear, const FarDefaults* none) {
   SortArgs g = {};
   int total = 0, C = 0;
   for (int k = 0; k < nsides; ++k) { g.s[k] = sides[k]; total += sides[k].problems; C = C > sides[k].C ? C : sides[k].C; }
   g.N = N; g.S = S; g.Bs = Bs; g.clear = clear;
+  if (none != nullptr) g.none = *none;
   g.q = S <= kSortMaxCluster ? kSortMaxCluster / S : 0;
   const int cl = g.q > 0 ? S * g.q : kSortMaxCluster;
   const int warps = C <= 2048 ? 16 : 8;                                    // private histograms of at most 128 KB

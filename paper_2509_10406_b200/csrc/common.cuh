@@ -198,7 +198,7 @@ void prof_mark(const char* name, cudaStream_t st, const char* kernel = nullptr);
 // Status words: the first kStatusWords int32 of every stage's workspace.  Word 0 holds the first
 // MUSE_STATUS_* code a kernel reported (0 = none); the entry points clear the words once per call.
 constexpr int kStatusWords = 64;
-constexpr int kItemWord = 4;               // work counter of the persistent summary kernel (zeroed by the kernel before it)
+constexpr int kItemWord = 4;               // two work counters of the persistent summary kernel: accumulated and per-block summaries (zeroed by the kernel before it)
 __device__ __forceinline__ void report_status(int* status, int code) { atomicCAS(status, 0, code); }
 
 // Bounds-checked build (compiled with -DMUSE_DEBUG into a second library): every index that a kernel derives from data
@@ -239,7 +239,10 @@ bool path_forced(unsigned bit);
 // kind 0 (queries): segments (block, cluster) contiguous, off [C*S+1] by block * C + cluster;
 // kind 1 (keys): a cluster's blocks are one contiguous run, off [C*S+1] by cluster * S + block.
 struct SortSide { const int32_t* assign; int32_t* off; int32_t* perm; int problems, C, kind; };
-int bucket_sort(const SortSide* sides, int nsides, int N, int S, int Bs, cudaStream_t st, int32_t* clear = nullptr);   // clear: status words to zero
+// what a forward pass says of the queries that see no far field (the first block, when causal): log-sum-exp -infinity, no cluster selected
+struct FarDefaults { float* lse; int32_t* sel; int m; };
+// clear: status words to zero; none: defaults of the first block of side 0 to write beside the sort
+int bucket_sort(const SortSide* sides, int nsides, int N, int S, int Bs, cudaStream_t st, int32_t* clear = nullptr, const FarDefaults* none = nullptr);
 
 // Lloyd iterations of one or both sides at once (kind 0 queries, 1 keys); the scratch pointers are carved from a
 // workspace by lloyd_side_ws.  cnorm is padded per problem to whole tiles of kAsgTile centres (infinity in the padding).
@@ -287,7 +290,17 @@ size_t summarize_ws_bytes(const Dims& d, int dtype);
 
 // sigma * qbar as two bf16 planes (hi + lo keeps ~16 mantissa bits), [B*Hq*Cq][D] each: the tensor-core
 // summary kernels load their centroid tiles from these by TMA instead of converting them per CTA
-int split_qbar(const Dims& d, const float* qbar, void* qhi, void* qlo, int* dealt, cudaStream_t st);   // dealt: zeroed, if given
+// sigma q-bar as bf16 hi + lo planes (n elements); dealt: the two item counters of the summaries kernel, zeroed beside them
+struct SplitQbar {
+  const float* qbar; long long n; float sigma; __nv_bfloat16 *hi, *lo; int* dealt;
+  __device__ __forceinline__ void element(long long e) const {
+    const float x = qbar[e] * sigma;
+    const __nv_bfloat16 h = __float2bfloat16_rn(x);
+    hi[e] = h;
+    lo[e] = __float2bfloat16_rn(x - __bfloat162float(h));
+  }
+};
+int split_qbar(const Dims& d, const float* qbar, void* qhi, void* qlo, cudaStream_t st);
 
 
 // Byte offsets inside the caller's summaries buffer.  Per entry (b, h, plane, i, j):

@@ -376,7 +376,7 @@ int summ_bwd_tc(const Dims& d, const void* Kp, const void* Vp, const int32_t* of
   // qsplit: 2 * B*Hq*Cq*D bf16 of scratch for the split centroids
   bf16* qhi = (bf16*)qsplit;
   bf16* qlo = qhi + (size_t)d.B * d.Hq * d.Cq * d.D;
-  int rcq = split_qbar(d, qbar, qhi, qlo, nullptr, st);
+  int rcq = split_qbar(d, qbar, qhi, qlo, st);
   if (rcq != MUSE_OK) return rcq;
   const uint64_t Dd = (uint64_t)d.D, Cq = (uint64_t)d.Cq;
   const uint64_t str[2] = {Dd * 2, Cq * Dd * 2};

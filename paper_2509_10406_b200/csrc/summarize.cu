@@ -7,7 +7,7 @@
 namespace muse {
 
 bool summarize_tc_supported(const Dims& d, int dtype);
-int summarize_tc(const Dims& d, const void* Kp, const void* Vp, const int32_t* off_k, const float* qbar, const SummPtrs& sp,
+int summarize_tc(const Dims& d, const void* Kp, const void* Vp, const int32_t* off_k, const SummPtrs& sp,
                  int per_block, void* qsplit, int* status, cudaStream_t stream);
 
 SummLayout summ_layout(const Dims& d, int dtype) {
@@ -43,12 +43,18 @@ SummLayout summ_layout(const Dims& d, int dtype) {
   return L;
 }
 
-// out[p] = in[perm[p]] for whole rows of D elements (16 bytes per thread), keys and values (blockIdx.z) in one launch.
+// out[p] = in[perm[p]] for whole rows of D elements (16 bytes per thread), keys and values (blockIdx.z) in one launch.  On the side, for the
+// summaries kernel that follows (split.hi != nullptr): the centroids' bf16 planes and its item counters.
 template <class T>
 __global__ void k_gather_rows(const T* __restrict__ K, const T* __restrict__ V, const int32_t* __restrict__ perm, int N, int D,
-                              T* __restrict__ Kp, T* __restrict__ Vp) {
+                              T* __restrict__ Kp, T* __restrict__ Vp, const SplitQbar split) {
   pdl_wait();
   pdl_trigger();
+  if (split.hi != nullptr && blockIdx.z == 0) {
+    const long long f = ((long long)blockIdx.y * gridDim.x + blockIdx.x) * blockDim.x + threadIdx.x, all = (long long)gridDim.y * gridDim.x * blockDim.x;
+    if (f < 2) split.dealt[f] = 0;
+    for (long long q = f; q < split.n; q += all) split.element(q);
+  }
   const T* in = blockIdx.z == 0 ? K : V;
   T* out = blockIdx.z == 0 ? Kp : Vp;
   const int vpr = D * (int)sizeof(T) / 16;           // 16-byte vectors per row
@@ -251,15 +257,18 @@ static int summarize_t(const Dims& d, int dtype, const T* K, const T* V, const i
   char* base = (char*)summaries;
   T* Kp = (T*)(base + L.Kp); T* Vp = (T*)(base + L.Vp);
   const int vpr = D * (int)sizeof(T) / 16;
+  const size_t nq = (size_t)d.B * d.Hq * d.Cq * d.D;
+  __nv_bfloat16* qsplit = ar.take<__nv_bfloat16>(2 * nq);                       // split centroids for the tensor kernel
+  SplitQbar split = {};
+  if (d.SB > 0 && summarize_tc_supported(d, dtype) && !path_forced(kForceSummFwdSimt)) split = SplitQbar{qbar, (long long)nq, d.sigma, qsplit, qsplit + nq, status + kItemWord};
   prof_mark("k_gather_rows", st);
-  MUSE_RC(launch_pdl(k_gather_rows<T>, dim3(cdiv(d.N * vpr, 256), pk, 2), 256, 0, st, K, V, perm_k, d.N, D, Kp, Vp));
+  MUSE_RC(launch_pdl(k_gather_rows<T>, dim3(cdiv(d.N * vpr, 256), pk, 2), 256, 0, st, K, V, perm_k, d.N, D, Kp, Vp, split));
   if (counts != nullptr) {
     prof_mark("k_bucket_sums", st);
     k_bucket_sums<T, D><<<dim3(cdiv(d.Ck * d.S, 8), pk), 256, 0, st>>>(Kp, Vp, off_k, d.N, d.Ck * d.S, counts, ksum, vsum);
     MUSE_LAUNCH_OK();
   }
   if (d.SB == 0) return MUSE_OK;
-  void* qsplit = ar.take<__nv_bfloat16>(2 * (size_t)d.B * d.Hq * d.Cq * d.D);   // split centroids for the tensor kernel
   rc = summarize_planes<T, D>(d, dtype, Kp, Vp, off_k, qbar, summ_ptrs(L, base), 0, qsplit, status, st);
   if (rc == MUSE_OK && d.k2 > 0) rc = summarize_planes<T, D>(d, dtype, Kp, Vp, off_k, qbar, summ_ptrs_blk(L, base), 1, qsplit, status, st);
   if (rc != MUSE_OK || !d.dipole || d.SB == 0) return rc;     // one causal block: no far field, nothing to correct
@@ -270,7 +279,7 @@ template <class T, int D>
 static int summarize_planes(const Dims& d, int dtype, const T* Kp, const T* Vp, const int32_t* off_k, const float* qbar,
                             const SummPtrs& sp, int per_block, void* qsplit, int32_t* status, cudaStream_t st) {
   if (summarize_tc_supported(d, dtype) && !path_forced(kForceSummFwdSimt))
-    return summarize_tc(d, Kp, Vp, off_k, qbar, sp, per_block, qsplit, status, st);
+    return summarize_tc(d, Kp, Vp, off_k, sp, per_block, qsplit, status, st);
   const size_t smem = (size_t)(kSumI * (D + 4) + kSumKC * (2 * D + 4) + kSumI * (kSumKC + 1)) * sizeof(float);
   MUSE_CUDA_OK(cudaFuncSetAttribute(k_summarize<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   dim3 grid(d.Ck, cdiv(d.Cq, kSumI), d.B * d.Hq);

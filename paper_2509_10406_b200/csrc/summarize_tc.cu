@@ -50,22 +50,17 @@ template <int D, int P> struct Lay {                       // shared-memory offs
 struct Bars { uint64_t q_full, q_free, kv_full[4], kv_empty[4], l_full[2], w_ready, u_step, u_done[2], acc_free[2], item_full[kRing], item_free[kRing]; };
 }  // namespace st
 
-__global__ void k_split_qbar(const float* __restrict__ qbar, long long n, float sigma, bf16* __restrict__ hi, bf16* __restrict__ lo, int* dealt) {
+__global__ void k_split_qbar(const SplitQbar split) {
   pdl_wait();
   pdl_trigger();
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e == 0 && dealt != nullptr) *dealt = 0;              // the item counter of the kernel that follows
-  if (e >= n) return;
-  const float x = qbar[e] * sigma;
-  const bf16 h = __float2bfloat16_rn(x);
-  hi[e] = h;
-  lo[e] = __float2bfloat16_rn(x - __bfloat162float(h));
+  if (e < split.n) split.element(e);
 }
 
-int split_qbar(const Dims& d, const float* qbar, void* qhi, void* qlo, int* dealt, cudaStream_t st) {
+int split_qbar(const Dims& d, const float* qbar, void* qhi, void* qlo, cudaStream_t st) {
   const long long n = (long long)d.B * d.Hq * d.Cq * d.D;
   prof_mark("k_split_qbar", st);
-  return launch_pdl(k_split_qbar, dim3((unsigned)((n + 255) / 256)), 256, 0, st, qbar, n, d.sigma, (bf16*)qhi, (bf16*)qlo, dealt);
+  return launch_pdl(k_split_qbar, dim3((unsigned)((n + 255) / 256)), 256, 0, st, SplitQbar{qbar, n, d.sigma, (bf16*)qhi, (bf16*)qlo, nullptr});
 }
 
 template <int D, int P>
@@ -486,15 +481,14 @@ static int summarize_tc_p(const Dims& d, const void* Kp, const void* Vp, const i
   // With few, every item would change the tile.
   const int per = groups >= grid ? 1 : (int)((items + grid - 1) / grid);
   return launch_pdl(k_summarize_tc<D, P>, dim3(grid), st::kThreads, st::Lay<D, P>::total, stream, d, tK, tV, tqh, tql, okhi, oklo, onu, off_k, sp, per_block, per,
-                    status + kItemWord, status);
+                    status + kItemWord + per_block, status);
 }
 
-int summarize_tc(const Dims& d, const void* Kp, const void* Vp, const int32_t* off_k, const float* qbar, const SummPtrs& sp,
+int summarize_tc(const Dims& d, const void* Kp, const void* Vp, const int32_t* off_k, const SummPtrs& sp,
                  int per_block, void* qsplit, int* status, cudaStream_t stream) {
-  // qsplit: 2 * B*Hq*Cq*D bf16 of scratch for the split centroids
+  // qsplit: the split centroids, 2 * B*Hq*Cq*D bf16; they and the item counters come from k_gather_rows
   bf16* qhi = (bf16*)qsplit;
   bf16* qlo = qhi + (size_t)d.B * d.Hq * d.Cq * d.D;
-  MUSE_RC(split_qbar(d, qbar, qhi, qlo, status + kItemWord, stream));
   // Few query clusters: a tile's 128 rows take them two or four times over, for as many key clusters (one with fewer key clusters would
   // have rows without work).
   const int P = d.D == 64 && d.Cq <= 32 && d.Ck >= 4 ? 4 : d.Cq <= 64 && d.Ck >= 2 ? 2 : 1;      // (D = 128: no room for four clusters' keys)
