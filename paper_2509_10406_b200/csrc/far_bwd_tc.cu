@@ -16,7 +16,8 @@
 // log-sum-exps, selections: 10000 cycles); in flight together they take 7400.  32 heads of 64k tokens, 128 x 128 clusters,
 // D = 64, segments of 64 queries: 3243 us with one CTA per SM, 1778 with two, 1646 with the sums of all sweeps kept on chip,
 // 1419 with the loads together; 32 heads of 16k, 128 x 256 2490 -> 1160; 16 heads of 8k, 64 x 128 488 -> 224; 4 heads, D = 128
-// 2425 -> 2053.
+// 2425 -> 2053.  With the first tile on its way before the CTA's threads meet, and the dq rows added by both warpgroups with their row
+// numbers in registers (a read of shared memory between two adds waited for the first): 1160 -> 1098, 224 -> 211, 2066 -> 2014.
 #include <cuda.h>
 #include "common.cuh"
 #include "tc05.cuh"
@@ -85,6 +86,7 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
   const int blk = dm.causal ? pl + 1 : 0, Ck = dm.Ck, NJ = (Ck + TJ - 1) / TJ, m = dm.m;
   const int tid = threadIdx.x, warp = tc::warp_index(), wg = tid >> 7, L = tid & 127;
   const int32_t* oq = off_q + (size_t)pq * (dm.S * dm.Cq + 1) + (size_t)blk * dm.Cq + i;
+  const float qv = tid < D ? qbar[((size_t)pq * dm.Cq + i) * D + tid] : 0.f;              // (on its way beside the offsets)
   const int p0 = oq[0], p1 = oq[1];
   if (p0 >= p1) {
     // An empty segment: its gradient rows are zeros.  The key-side tensor-core pass (the reader of the
@@ -109,20 +111,7 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
   const int32_t* pm = perm_q + (size_t)pq * dm.N;
 
   if (warp == 0) tc::tmem_alloc(&tbase_s, LY::cols);
-  if (tid == 0) { tc::mbar_init(&bar_full, 1); tc::mbar_init(&bar1, 1); tc::mbar_init(&bar2, 1); tc::mbar_init(&bar3, 1);
-                  tc::mbar_init(&bar_nu, 1); tc::mbar_init(&bar_st, 1); tc::mbar_init_fence(); }
-  if (tid < D) qb[tid] = qbar[((size_t)pq * dm.Cq + i) * D + tid];
-  tc::fence_before_sync();
-  __syncthreads();
-  tc::fence_after_sync();
-  pdl_trigger();                                           // (tensor memory has been allocated)
-  const uint32_t tbase = tbase_s, tlane = tbase + ((uint32_t)((warp & 3) * 32) << 16);
-  uint32_t ph_full = 0, ph1 = 0, ph2 = 0, ph3 = 0, ph_st = 0;
-  const bool cw = warp < 8;                               // compute warp
-  bool ok = true;
-  const uint32_t aHi = tc::smem_u32(sm + oHi), aLo = tc::smem_u32(sm + oLo), aNu = tc::smem_u32(sm + oNu),
-                 aPt = tc::smem_u32(sm + oPt), aGt = tc::smem_u32(sm + oGt);
-
+  // the issuer makes the barriers, and has the first cluster tile on its way before the others meet it
   auto issue_kappa = [&](int jt_) {                       // issuer: the two kappa tiles of cluster tile jt_
     tc::mbar_expect_tx_warp(&bar_full, 2 * kTile);
     for (int g = 0; g < G; ++g) {                         // (rows past Ck are zeros)
@@ -134,16 +123,44 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
     tc::mbar_expect_tx_warp(&bar_nu, kTile);
     for (int g = 0; g < G; ++g) tc::tma_load_3d_warp(sm + oNu + g * TJ * 128, &tm_nu, 64 * g, jt_ * TJ, seg, &bar_nu);
   };
+  if (warp == ISSUER / 32) {
+    if (tc::elect_one()) {
+      tc::mbar_init(&bar_full, 1); tc::mbar_init(&bar1, 1); tc::mbar_init(&bar2, 1); tc::mbar_init(&bar3, 1);
+      tc::mbar_init(&bar_nu, 1); tc::mbar_init(&bar_st, 1); tc::mbar_init_fence();
+    }
+    __syncwarp();
+    issue_kappa(0);
+    issue_nu(0);
+  }
+  if (tid < D) qb[tid] = qv;
+  tc::fence_before_sync();
+  __syncthreads();
+  tc::fence_after_sync();
+  pdl_trigger();                                           // (tensor memory has been allocated)
+  const uint32_t tbase = tbase_s, tlane = tbase + ((uint32_t)((warp & 3) * 32) << 16);
+  uint32_t ph_full = 0, ph1 = 0, ph2 = 0, ph3 = 0, ph_st = 0;
+  const bool cw = warp < 8;                               // compute warp
+  bool ok = true;
+  // operand descriptors, each made once and stepped from product to product: K-major (clusters or rows in 8-row groups), and MN-major
+  // (dims of the cluster tiles and of the query rows, rows of G)
+  const uint64_t kHi = tc::smem_desc_sw128(tc::smem_u32(sm + oHi), 16, 1024), kLo = tc::smem_desc_sw128(tc::smem_u32(sm + oLo), 16, 1024),
+                 kNu = tc::smem_desc_sw128(tc::smem_u32(sm + oNu), 16, 1024), kPt = tc::smem_desc_sw128(tc::smem_u32(sm + oPt), 16, 1024),
+                 kGt = tc::smem_desc_sw128(tc::smem_u32(sm + oGt), 16, 1024), kQ = tc::smem_desc_sw128(tc::smem_u32(sm + oQ), 16, 1024),
+                 kDO = tc::smem_desc_sw128(tc::smem_u32(sm + oDO), 16, 1024);
+  const uint64_t nHi = tc::smem_desc_sw128(tc::smem_u32(sm + oHi), TJ * 128, 1024), nLo = tc::smem_desc_sw128(tc::smem_u32(sm + oLo), TJ * 128, 1024),
+                 nGt = tc::smem_desc_sw128(tc::smem_u32(sm + oGt), TJ * 128, 1024), nQ = tc::smem_desc_sw128(tc::smem_u32(sm + oQ), NR * 128, 1024),
+                 nDO = tc::smem_desc_sw128(tc::smem_u32(sm + oDO), NR * 128, 1024);
+
   float gsum = 0.f, gt2 = 0.f, pdp = 0.f;
   for (int s0 = p0; s0 < p1 && ok; s0 += NP * NR) {        // sweep: up to 64 rows
-    const bool load = !ONE || s0 == p0, store = !ONE || s0 + NP * NR >= p1;
+    const bool first = s0 == p0, load = !ONE || first, store = !ONE || s0 + NP * NR >= p1;
     const int ns = min(NP * NR, p1 - s0), np = (ns + NR - 1) / NR;
     // the products take only as many rows as there are: nc of them (a multiple of 8) per warpgroup, nr in all
     const int nc = ((ns + 1) / 2 + 7) & ~7, nr = 2 * nc;
     __syncthreads();
     // the operand tiles are free (every product of the previous sweep has completed): the first cluster
     // tile travels while the rows are gathered
-    if (load && warp == ISSUER / 32) { issue_kappa(0); issue_nu(0); }
+    if (load && !first && warp == ISSUER / 32) { issue_kappa(0); issue_nu(0); }
     // a chain of loads whose latency nothing hides but the SM's other CTA: every thread finds its rows itself, and all that
     // hangs on a row (Q, dO, log-sum-exp, delta, the selection) is on its way at once
     auto row_of = [&](int r) {
@@ -208,7 +225,6 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
       if constexpr (!ONE) gsum = gt2 = pdp = 0.f;
       const float mu1 = j < Ck ? 1.f + mu[ent0 + j] : 0.f;                              // 1 + accumulated log-mass of cluster j
       for (int p = 0; p < np && ok; ++p) {
-        const uint32_t aQ = tc::smem_u32(sm + oQ + p * kRows), aDO = tc::smem_u32(sm + oDO + p * kRows);
         if (warp == ISSUER / 32) {
           if (p == 0 && load) {
             if (!tc::mbar_wait(&bar_full, ph_full)) ok = false;
@@ -218,16 +234,16 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
           const uint32_t idesc = tc::idesc_bf16(TJ, nr, 0, 0);
 #pragma unroll
           for (int ks = 0; ks < D / 16; ++ks)
-            tc::mma_bf16_ss_warp(tbase + cS, tc::smem_desc_sw128(aHi + (ks / 4) * TJ * 128 + (ks % 4) * 32, 16, 1024),
-                            tc::smem_desc_sw128(aQ + (ks / 4) * NR * 128 + (ks % 4) * 32, 16, 1024), idesc, ks > 0);
+            tc::mma_bf16_ss_warp(tbase + cS, tc::desc_step(kHi, (ks / 4) * TJ * 128 + (ks % 4) * 32),
+                            tc::desc_step(kQ, (ks / 4) * NR * 128 + (ks % 4) * 32), idesc, ks > 0);
 #pragma unroll
           for (int ks = 0; ks < D / 16; ++ks)
-            tc::mma_bf16_ss_warp(tbase + cS, tc::smem_desc_sw128(aLo + (ks / 4) * TJ * 128 + (ks % 4) * 32, 16, 1024),
-                            tc::smem_desc_sw128(aQ + (ks / 4) * NR * 128 + (ks % 4) * 32, 16, 1024), idesc, 1);
+            tc::mma_bf16_ss_warp(tbase + cS, tc::desc_step(kLo, (ks / 4) * TJ * 128 + (ks % 4) * 32),
+                            tc::desc_step(kQ, (ks / 4) * NR * 128 + (ks % 4) * 32), idesc, 1);
 #pragma unroll
           for (int ks = 0; ks < D / 16; ++ks)
-            tc::mma_bf16_ss_warp(tbase + cDP, tc::smem_desc_sw128(aNu + (ks / 4) * TJ * 128 + (ks % 4) * 32, 16, 1024),
-                            tc::smem_desc_sw128(aDO + (ks / 4) * NR * 128 + (ks % 4) * 32, 16, 1024), idesc, ks > 0);
+            tc::mma_bf16_ss_warp(tbase + cDP, tc::desc_step(kNu, (ks / 4) * TJ * 128 + (ks % 4) * 32),
+                            tc::desc_step(kDO, (ks / 4) * NR * 128 + (ks % 4) * 32), idesc, ks > 0);
           tc::mma_commit_warp(&bar1);
           if (!ONE && p == 0) {
             tc::tma_store_wait_read_warp();        // the previous tile's stores have read the staging tiles, which the
@@ -306,21 +322,21 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
           const uint32_t id_dq = tc::idesc_bf16(128, nr, 1, 1);
 #pragma unroll
           for (int ks = 0; ks < NR / 16; ++ks) if (16 * ks < nr)
-            tc::mma_bf16_ss_warp(tbase + cDNU, tc::smem_desc_sw128(aPt + ks * 32, 16, 1024),
-                            tc::smem_desc_sw128(aDO + ks * 16 * 128, NR * 128, 1024), id_row, !(p == 0 && ks == 0 && load));
+            tc::mma_bf16_ss_warp(tbase + cDNU, tc::desc_step(kPt, ks * 32),
+                            tc::desc_step(nDO, ks * 16 * 128), id_row, !(p == 0 && ks == 0 && load));
 #pragma unroll
           for (int ks = 0; ks < NR / 16; ++ks) if (16 * ks < nr)
-            tc::mma_bf16_ss_warp(tbase + cDKA, tc::smem_desc_sw128(aGt + ks * 32, 16, 1024),
-                            tc::smem_desc_sw128(aQ + ks * 16 * 128, NR * 128, 1024), id_row, !(p == 0 && ks == 0 && load));
+            tc::mma_bf16_ss_warp(tbase + cDKA, tc::desc_step(kGt, ks * 32),
+                            tc::desc_step(nQ, ks * 16 * 128), id_row, !(p == 0 && ks == 0 && load));
           tc::mma_commit_warp(&bar2);              // the read-out of dnu / dkappa can start while the dq products still run
 #pragma unroll
           for (int ks = 0; ks < TJ / 16; ++ks)
-            tc::mma_bf16_ss_warp(tbase + cDQ + p * NR, tc::smem_desc_sw128(aHi + ks * 16 * 128, TJ * 128, 1024),
-                            tc::smem_desc_sw128(aGt + ks * 16 * 128, TJ * 128, 1024), id_dq, !(jt == 0 && ks == 0));
+            tc::mma_bf16_ss_warp(tbase + cDQ + p * NR, tc::desc_step(nHi, ks * 16 * 128),
+                            tc::desc_step(nGt, ks * 16 * 128), id_dq, !(jt == 0 && ks == 0));
 #pragma unroll
           for (int ks = 0; ks < TJ / 16; ++ks)
-            tc::mma_bf16_ss_warp(tbase + cDQ + p * NR, tc::smem_desc_sw128(aLo + ks * 16 * 128, TJ * 128, 1024),
-                            tc::smem_desc_sw128(aGt + ks * 16 * 128, TJ * 128, 1024), id_dq, 1);
+            tc::mma_bf16_ss_warp(tbase + cDQ + p * NR, tc::desc_step(nLo, ks * 16 * 128),
+                            tc::desc_step(nGt, ks * 16 * 128), id_dq, 1);
           tc::mma_commit_warp(&bar3);
           // every MMA on the operand tiles has completed: the next cluster tile may overwrite them
           if (!tc::mbar_wait(&bar3, ph3)) ok = false;
@@ -403,19 +419,21 @@ k_far_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
       tc::fence_before_sync();
       if (wg == 0 && ok && j < Ck) dS[gent] = (later_sweep ? dS[gent] : 0.f) + dsid[0][L] + dsid[1][L];
     }
-    // ---- dq: warpgroup p reads pass p (thread = output dim), adds into the fp32 accumulator
+    // ---- dq: thread = output dim, a warpgroup its rows of the sweep; adds into the fp32 accumulator
     if (cw && !tc::mbar_wait(&bar3, ph3 ^ 1)) ok = false;     // the last tile's dq products
     tc::fence_after_sync();
-    for (int p = 0; cw && p < np; ++p) {
-      for (int c0 = 32 * wg; c0 < NR; c0 += 64) {
-        float v[32];
-        tc::tmem_ld32(tlane + cDQ + p * NR + c0, v);
-        if (ok && L < D) {
+    if (cw && ok && (L & ~31) < D) {                         // (whole warps)
+      const int lane = tid & 31, nv = min(nc, ns - wg * nc);
+      const int row = lane < nv ? rows[wg * nc + lane] : -1;  // (by shuffles below: a read of shared memory would wait for the add before it)
+      float* out = dQacc + (size_t)pq * dm.N * D + L;
+#pragma unroll 1
+      for (int c0 = 0; c0 < nv; c0 += 8) {
+        float v[8];
+        tc::tmem_ld8(tlane + cDQ + wg * nc + c0, v);
 #pragma unroll
-          for (int r = 0; r < 32; ++r) {
-            const int rr = p * NR + c0 + r;
-            if (rr < ns && rows[rr] >= 0) atomicAdd(dQacc + ((size_t)pq * dm.N + rows[rr]) * D + L, v[r]);   // (result unused: no round trip)
-          }
+        for (int r = 0; r < 8; ++r) {
+          const int t = __shfl_sync(0xffffffffu, row, c0 + r);
+          if (t >= 0) atomicAdd(out + (size_t)t * D, v[r]);  // (result unused: no round trip)
         }
       }
     }
