@@ -8,7 +8,7 @@
 //   S = Q K^T, dP = dO V^T            tcgen05.mma into tensor memory
 //   P, G                               one thread per pair row, written as bf16 tiles to shared memory
 //   dQ = G K                           over the tensor-memory columns that S and dP have vacated
-//   dV^T += dO^T P,  dK^T += Q^T G     [D][keys], accumulated in tensor memory over all of the CTA's tiles
+//   dV^T += dO^T P,  dK^T += Q^T G     [D][keys], accumulated in tensor memory over all of the CTA's tiles (D = 64: two quarters of one product)
 // To keep the tensor cores, the load/store unit and the arithmetic warps busy at the same time, an SM runs TWO independent
 // pipelines.  At D = 64 they are two CTAs, so that the start of one cluster (its index entries, keys and first rows) and the end of
 // another run beside products.  At D = 128 the tiles of Q, dO, P and G of two pipelines ("halves") fill shared memory and one CTA
@@ -19,10 +19,11 @@
 // A cluster with more than 64 visible keys takes further sweeps over the tiles that see them; later sweeps
 // add to the stored dQ rows.
 //
-// Bound by the latency of a tile's chain (gather, S, P and G, dQ) where a cluster has only a few tiles.  At D = 64 the rows of the next
+// Bound by what the products read from shared memory (168 KB a tile at D = 64 with five of them, 136 KB with dV and dK as one; twice the
+// row warps, half of a row each, gave nothing) and by the chain of a tile (gather, S, P and G, dQ) where a cluster has only a few.  At D = 64 the rows of the next
 // tile arrive beside it in a second pair of buffers; in a later sweep the stored dQ rows are on their way while the products run.
-// D = 64: 16 heads of 8k tokens, 128 clusters, 8 slots 361 -> 216 us; 24 heads of 4k, 128 clusters, 8 slots, non-causal 353 -> 213;
-// 32 heads of 16k, 256 clusters, 16 slots 1851 -> 1614; D = 128: 6 heads of 9k, 200 clusters, 10 slots 265 -> 220; 4 heads of 64k, 1024
+// D = 64: 16 heads of 8k tokens, 128 clusters, 8 slots 361 -> 203 us (217 before the one product); 24 heads of 4k, 128 clusters, 8
+// slots, non-causal 353 -> 198 (211); 32 heads of 16k, 256 clusters, 16 slots 1851 -> 1571 (1624); D = 128: 6 heads of 9k, 200 clusters, 10 slots 265 -> 220; 4 heads of 64k, 1024
 // clusters, 32 slots 2515 -> 2430.  dQ rows staged in shared memory and stored 16 bytes a lane: 2157 and 2941 us at the last
 // and third of these sizes.
 #include <cuda.h>
@@ -300,16 +301,18 @@ k_ret_bwd_sweeps(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ d
       }
       // dV^T and dK^T of this sweep's keys: thread = output dim, one key per column; the other half of the CTA
       // (and other CTAs that share the cluster) add theirs to the same rows
-      if (started && (warp & 3) * 32 < D) {                  // (warp-uniform: the lanes of a warp hold 32 consecutive dims)
-        const int dd = (warp & 3) * 32 + lane;
+      if (started) {
+        // (D = 128: a warp has 32 dims of both; D = 64: lanes 0 to 63 the dims of dK^T, lanes 64 to 127 those of dV^T)
+        const int dd = (warp & 3) * 32 % D + lane;
 #pragma unroll
-        for (int w2 = 0; w2 < 2; ++w2) {
-          float* dst = (w2 == 0 ? dV_perm : dK_perm) + ((size_t)pq * dm.N + k0 + kc) * D + dd;
+        for (int w2 = 0; w2 < D / 64; ++w2) {
+          const bool dv = D == 64 ? (warp & 2) != 0 : w2 == 0;
+          float* dst = (dv ? dV_perm : dK_perm) + ((size_t)pq * dm.N + k0 + kc) * D + dd;
 #pragma unroll
           for (int u0 = 0; u0 < kKeys; u0 += 32) {
             if (u0 >= nkc) break;
             float x[32];
-            tc::tmem_ld32(tl + (w2 == 0 ? cDV : cDK) + u0, x);
+            tc::tmem_ld32(tl + (dv ? cDV : cDK) + u0, x);
             if (ok_) {
 #pragma unroll
               for (int u = 0; u < 32; ++u)
@@ -338,19 +341,27 @@ k_ret_bwd_sweeps(Dims dm, const bf16* __restrict__ Q, const bf16* __restrict__ d
           wait(&B.pg_ready, ph);                             // P and G are in shared memory, S and dP consumed
           tc::fence_after_sync();
           const uint32_t id_dq = tc::idesc_bf16(kPairs, D, 0, 1);        // A = G (contraction over keys), B = key rows MN-major
-          // A = dO / Q tile and B = P / G tile, both contracted over pairs.  M = 128 output dims even when D = 64: the second
-          // 64-dim group of the A operand is then the tile that follows in shared memory, and lanes 64..127 hold numbers nobody reads
-          const uint32_t id_t = tc::idesc_bf16(128, kKeys, 1, 1);
           const bool acc = np > np0;                                     // the accumulators start at zero in every sweep
 #pragma unroll
           for (int ks = 0; ks < kKeys / 16; ++ks)
             tc::mma_bf16_ss_warp(tbase + cDQ, tc::smem_desc_sw128(ga + ks * 32, 16, 1024), desc_mn<kKeys>(ka, ks), id_dq, ks > 0);
+          // A = Q / dO tile and B = G / P tile, both contracted over pairs
+          if constexpr (D == 64) {
+            // One product [Q | dO]^T [P | G] of 128 dims by 128 keys, of which dK^T and dV^T are a quarter each and nobody reads the
+            // rest: the two tiles are read once, instead of twice with 64 of the 128 rows of the instruction idle
+            const uint32_t id_t = tc::idesc_bf16(128, 2 * kKeys, 1, 1);
 #pragma unroll
-          for (int ks = 0; ks < kPairs / 16; ++ks)
-            tc::mma_bf16_ss_warp(tbase + cDV, desc_mn<kPairs>(da, ks), tc::smem_desc_sw128(pa + ks * 16 * 128, kPairs * 128, 1024), id_t, acc || ks > 0);
+            for (int ks = 0; ks < kPairs / 16; ++ks)
+              tc::mma_bf16_ss_warp(tbase + cDV, desc_mn<kPairs>(qa, ks), tc::smem_desc_sw128(pa + ks * 16 * 128, kPG, 1024), id_t, acc || ks > 0);
+          } else {
+            const uint32_t id_t = tc::idesc_bf16(128, kKeys, 1, 1);
 #pragma unroll
-          for (int ks = 0; ks < kPairs / 16; ++ks)
-            tc::mma_bf16_ss_warp(tbase + cDK, desc_mn<kPairs>(qa, ks), tc::smem_desc_sw128(ga + ks * 16 * 128, kPairs * 128, 1024), id_t, acc || ks > 0);
+            for (int ks = 0; ks < kPairs / 16; ++ks)
+              tc::mma_bf16_ss_warp(tbase + cDV, desc_mn<kPairs>(da, ks), tc::smem_desc_sw128(pa + ks * 16 * 128, kPairs * 128, 1024), id_t, acc || ks > 0);
+#pragma unroll
+            for (int ks = 0; ks < kPairs / 16; ++ks)
+              tc::mma_bf16_ss_warp(tbase + cDK, desc_mn<kPairs>(qa, ks), tc::smem_desc_sw128(ga + ks * 16 * 128, kPairs * 128, 1024), id_t, acc || ks > 0);
+          }
           tc::mma_commit_warp(&B.m2_done);
           tc::mma_commit_warp(&B.q_empty[st_]);                   // ... and the Q / dO tiles refilled
         }
