@@ -15,11 +15,13 @@
 //
 // Bound by the latency of a plane's steps at D = 64 (two CTAs per SM), by DRAM and that latency at D = 128.  c needs only the
 // sum of its two contractions, so they share an accumulator; the tilt logits stay in tensor memory; with the freed registers
-// nothing spills, which matters because the tiles leave next to no L1 cache (spilled words, and the bucket offsets that are now
+// next to nothing spills, which matters because the tiles leave next to no L1 cache (spilled words, and the bucket offsets that are now
 // in shared memory, came from L2 on every plane: 2000 cycles).  32 heads of 64k tokens, 128 x 128 clusters, D = 64 2485 ->
 // 1682 us; 32 heads of 16k, 128 x 256 1222 -> 771; 16 heads of 8k, 64 x 128 322 -> 209; 4 heads of 64k, D = 128, 256 x 1024
 // 1280 -> 1201.  Two planes a step with at most 64 query clusters: 16 heads of 8k, 64 x 128, 7 planes 209 -> 168 us; 6 heads of 9k,
 // D = 128, 50 x 200, 5 planes 153 -> 121; four with at most 32: 10 heads of 1k, D = 128, 8 x 128, 3 planes 92 -> 71.
+// At D = 64 dK^T and dV^T as the two halves of one product, and read out by all warps: 168 -> 140 us, 32 heads of 16k 779 -> 681, 32
+// heads of 64k 1671 -> 1451.
 #include <cuda.h>
 #include "common.cuh"
 #include "tc05.cuh"
@@ -40,8 +42,8 @@ template <int D> struct Lay {
   static constexpr int oK = oDnu1 + kTile, oV = oK + kKeys, oW = oV + kKeys;
   static constexpr int total = oW + TI * NU * 2;           // 112 KB at D = 64, two CTAs per SM: no slack, the kernel checks the alignment of its base
 };
-// tilt logits, X = dkappa.k + dnu.v of a plane, the accumulators
-constexpr uint32_t cL = 0, cX = 64, cDK = 128, cDV = 192, cols = 256;
+// tilt logits, X = dkappa.k + dnu.v of a plane, the accumulators (D = 64: dK^T and dV^T in the lanes of one, the centroids' part of dK^T)
+constexpr uint32_t cL = 0, cX = 64, cDK = 128, cDV = 192, cQC = cDV, cols = 256;
 constexpr int kOkCache = 72;                   // bucket offsets of the cluster kept in shared memory (S + 1 <= 72)
 }  // namespace sb
 
@@ -286,17 +288,19 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
           tc::fence_after_sync();
           early = D == 64 && pl + P < pl_end && ok && __all_sync(0xffffffffu, tc::mbar_test(&bar_g[buf ^ 1], (ph_g >> (buf ^ 1)) & 1u));
           if (early) issue_x(k + 1);
-          // A [i][d] and B [i][u]: both contract over rows.  M = 128 output dims even when D = 64: the second 64-dim group
-          // of the A operand is then the tile that follows in shared memory, and output lanes 64..127 hold numbers that nobody reads
-          const uint32_t idesc = tc::idesc_bf16(128, NU, 1, 1);
+          // A [i][d] and B [i][u]: both contract over rows.  At D = 64 the two 64-dim groups of one A operand are the dkappa and the dnu
+          // tile: one product gives dK^T (lanes 0..63) and dV^T (lanes 64..127)
+          const uint32_t idesc = tc::idesc_bf16(128, NU, 1, 1), group = D == 64 ? (uint32_t)(oDnu - oDka) : TI * 128;
 #pragma unroll
           for (int ks = 0; ks < TI / 16; ++ks)
-            tc::mma_bf16_ss_warp(tbase + cDK, tc::smem_desc_sw128(aDka + ks * 16 * 128, TI * 128, 1024),
+            tc::mma_bf16_ss_warp(tbase + cDK, tc::smem_desc_sw128(aDka + ks * 16 * 128, group, 1024),
                             tc::smem_desc_sw128(aW + ks * 16 * 128, TI * 128, 1024), idesc, started || ks > 0);
+          if constexpr (D == 128) {
 #pragma unroll
-          for (int ks = 0; ks < TI / 16; ++ks)
-            tc::mma_bf16_ss_warp(tbase + cDV, tc::smem_desc_sw128(aDnu + ks * 16 * 128, TI * 128, 1024),
-                            tc::smem_desc_sw128(aW + ks * 16 * 128, TI * 128, 1024), idesc, started || ks > 0);
+            for (int ks = 0; ks < TI / 16; ++ks)
+              tc::mma_bf16_ss_warp(tbase + cDV, tc::smem_desc_sw128(aDnu + ks * 16 * 128, TI * 128, 1024),
+                              tc::smem_desc_sw128(aW + ks * 16 * 128, TI * 128, 1024), idesc, started || ks > 0);
+          }
           tc::mma_commit_warp(&bar2);
         }
         started = true;
@@ -324,11 +328,12 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
           __syncthreads();
           if (warp == ISSUER / 32) {
             tc::fence_after_sync();
+            // (at D = 64 in an accumulator of its own, whose lanes 64..127 hold numbers that nobody reads)
             const uint32_t idesc = tc::idesc_bf16(128, NU, 1, 1);
 #pragma unroll
             for (int ks = 0; ks < TI / 16; ++ks)
-              tc::mma_bf16_ss_warp(tbase + cDK, tc::smem_desc_sw128(aQhi + ks * 16 * 128, TI * 128, 1024),
-                                   tc::smem_desc_sw128(aW + ks * 16 * 128, TI * 128, 1024), idesc, 1);
+              tc::mma_bf16_ss_warp(tbase + (D == 64 ? cQC : cDK), tc::smem_desc_sw128(aQhi + ks * 16 * 128, TI * 128, 1024),
+                                   tc::smem_desc_sw128(aW + ks * 16 * 128, TI * 128, 1024), idesc, D == 128 || i0 > 0 || ks > 0);
             tc::mma_commit_warp(&bar2);
           }
           __syncwarp();
@@ -338,19 +343,24 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
         }
       }
     }
-    // read-out once per key chunk: thread = d, warpgroup = half of the keys; add into the fp32 accumulators
+    // read-out once per key chunk: thread = d (D = 64: of dK or dV), warpgroup = half of the keys; add into the fp32 accumulators
     const int nkc = min(NU, kvis - c0);
     if (cw) {
-      float a[32], b[32];
-      tc::tmem_ld32(tlane + cDK + 32 * wg, a);
-      tc::tmem_ld32(tlane + cDV + 32 * wg, b);
-      if (ok && started && L < D) {
+      const bool to_dv = D == 64 && (warp & 2) != 0;
+      const size_t at0 = ((size_t)pq * dm.N + c0 + 32 * wg) * D + L % D;
+      float* dst = (to_dv ? dV_perm : dK_perm) + at0;
+#pragma unroll 1
+      for (int h = 0; h < 32; h += 16) {
+        float a[16], b[16];
+        tc::tmem_ld16(tlane + cDK + 32 * wg + h, a);
+        tc::tmem_ld16(tlane + (D == 128 ? cDV : cQC) + 32 * wg + h, b);      // (D = 64: used where the centroids' part has been made, lanes 0..63)
+        if (!ok || !started) continue;
+        const bool sum = D == 64 && dm.agg_grad && !to_dv;
 #pragma unroll
-        for (int u = 0; u < 32; ++u) {
-          if (32 * wg + u < nkc) {
-            const size_t at = ((size_t)pq * dm.N + c0 + 32 * wg + u) * D + L;
-            atomicAdd(dK_perm + at, a[u]);                 // (result unused: no round trip; one CTA owns the element)
-            atomicAdd(dV_perm + at, b[u]);
+        for (int u = 0; u < 16; ++u) {
+          if (32 * wg + h + u < nkc) {
+            atomicAdd(dst + (size_t)(h + u) * D, sum ? a[u] + b[u] : a[u]);   // (result unused: no round trip; one CTA owns the element)
+            if constexpr (D == 128) atomicAdd(dV_perm + at0 + (size_t)(h + u) * D, b[u]);
           }
         }
       }
