@@ -9,8 +9,10 @@
 // the shares in which the tensor-core kernels take the groups.
 //
 // Bound by the scattered 4-byte stores of the last pass (a store per lane) and shared-memory atomics.  32 heads of 64k tokens,
-// 8 slots, 128 clusters, 8 blocks: 160 us; a memset, a counting kernel, a scan and a placing kernel that combined equal keys
-// of a warp into one global atomic took 1480 us.
+// 8 slots, 128 clusters, 8 blocks: 126 us (161 with two divisions a pair for its plane); a memset, a counting kernel, a scan and a
+// placing kernel that combined equal keys of a warp into one global atomic took 1480 us.  4 heads of 128k, 32 slots, 2048 clusters
+// 348 -> 275; 4 heads of 64k, 32 slots, 1024 clusters 184 -> 148; 16 heads of 8k, whose few pairs a CTA keeps between the passes,
+// 37 -> 31.
 #include <cooperative_groups.h>
 #include "common.cuh"
 
@@ -18,7 +20,7 @@ namespace cg = cooperative_groups;
 
 namespace muse {
 
-constexpr int kRiThreads = 1024, kRiMaxCluster = 16, kRiMinPairs = 2048;
+constexpr int kRiThreads = 1024, kRiMaxCluster = 16, kRiMinPairs = 2048, kRiKept = 8;   // kept: pairs of a thread that stay in registers between the passes
 
 struct RiArgs { const int32_t *sel, *bsel, *off_k; RetIndex ri; int nkeys; };
 
@@ -38,22 +40,41 @@ k_ret_index(Dims d, const __grid_constant__ RiArgs g) {
   const int n = (t1 - t0) * d.m;
   const int32_t* sel = g.sel + ((size_t)pq * d.N + t0) * d.m;
   const int32_t* bsel = g.bsel ? g.bsel + ((size_t)pq * d.N + t0) * d.m * ke : nullptr;
-  auto key_of = [&](int e, int c, int x) {
-    const int pl = d.causal ? (t0 + e / d.m) / d.Bs - 1 : 0;                   // block 0 sees no other block
+  // (a thread's pairs ascend, so their plane is followed from block to block: two divisions a pair were a third of the instructions)
+  struct Plane { int pl; unsigned end; };                  // of the next pair, and the first pair of a later block
+  const unsigned bm = (unsigned)d.Bs * d.m;
+  const Plane pl0 = d.causal ? Plane{t0 / d.Bs - 1, (unsigned)(t0 / d.Bs + 1) * bm - (unsigned)t0 * d.m} : Plane{0, 0xffffffffu};
+  auto key_of = [&](Plane& p, int e, int c, int x) {
+    while ((unsigned)e >= p.end) { ++p.pl; p.end = p.pl + 1 < d.S - 1 ? p.end + bm : 0xffffffffu; }
+    const int pl = p.pl;                                   // block 0 sees no other block
     if (c < 0 || c >= d.Ck || pl < 0) return -1;
     if (bsel == nullptr) return c * d.SB + pl;
     const int bb = bsel[(size_t)e * ke + x];
     return bb < 0 || bb > pl ? -1 : c * d.SB + bb;                             // (an earlier block than the query's block pl + 1)
   };
   constexpr int U = 4;                                     // pairs in flight per thread
-  for (int e0 = tid; e0 < n; e0 += U * kRiThreads) {
+  // a CTA of few pairs counts and remembers what the count said: key | place among the CTA's pairs of the key << 15
+  const bool keep = ke == 1 && g.bsel == nullptr && n <= kRiKept * kRiThreads;
+  uint32_t kept[kRiKept];
+  Plane p = pl0;
+  if (keep) {
+    int c[kRiKept];
+#pragma unroll
+    for (int u = 0; u < kRiKept; ++u) c[u] = tid + u * kRiThreads < n ? sel[tid + u * kRiThreads] : -1;
+#pragma unroll
+    for (int u = 0; u < kRiKept; ++u) {
+      const int key = c[u] >= 0 ? key_of(p, tid + u * kRiThreads, c[u], 0) : -1;
+      kept[u] = key >= 0 ? (uint32_t)key | (uint32_t)atomicAdd(&hist[key], 1) << 15 : 0xffffffffu;
+    }
+  }
+  for (int e0 = tid; !keep && e0 < n; e0 += U * kRiThreads) {
     int c[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) c[u] = e0 + u * kRiThreads < n ? sel[e0 + u * kRiThreads] : -1;
 #pragma unroll
     for (int u = 0; u < U; ++u)
       for (int x = 0; x < ke; ++x) {
-        const int key = key_of(e0 + u * kRiThreads, c[u], x);
+        const int key = key_of(p, e0 + u * kRiThreads, c[u], x);
         if (key >= 0) atomicAdd(&hist[key], 1);
       }
   }
@@ -61,9 +82,16 @@ k_ret_index(Dims d, const __grid_constant__ RiArgs g) {
   // this CTA's share of the keys: totals over the CTAs, their exclusive prefix within the share
   const int kper = (nkeys + CL - 1) / CL, ka = min(nkeys, rank * kper), kb = min(nkeys, ka + kper);
   int32_t* goff = g.ri.goff + (size_t)pq * (nkeys + 1);
-  int share = 0;
-  for (int k = ka + tid; k < kb; k += kRiThreads)
-    for (int c = 0; c < CL; ++c) share += cluster.map_shared_rank(hist, c)[k];
+  int share = 0, v[kRiMaxCluster], all = 0;                // counts of a key in every CTA
+  auto counts = [&](int k) {
+    all = 0;
+#pragma unroll
+    for (int c = 0; c < kRiMaxCluster; ++c) {
+      v[c] = c < CL && k < kb ? cluster.map_shared_rank(hist, min(c, CL - 1))[k] : 0;
+      all += v[c];
+    }
+  };
+  for (int k0 = ka; k0 < kb; k0 += kRiThreads) { counts(k0 + tid); share += all; }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) share += __shfl_xor_sync(0xffffffffu, share, o);
   if (lane == 0) wsum[warp] = share;
@@ -79,12 +107,7 @@ k_ret_index(Dims d, const __grid_constant__ RiArgs g) {
   for (int c = 0; c < rank; ++c) carry += share_s[c];
   for (int k0 = ka; k0 < kb; k0 += kRiThreads) {
     const int k = k0 + tid;
-    int v[kRiMaxCluster], all = 0;
-#pragma unroll
-    for (int c = 0; c < kRiMaxCluster; ++c) {
-      v[c] = c < CL && k < kb ? cluster.map_shared_rank(hist, min(c, CL - 1))[k] : 0;
-      all += v[c];
-    }
+    if (kper > kRiThreads) counts(k);                      // (else this thread's one key is still here)
     int inc = all;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) { const int x = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += x; }
@@ -127,15 +150,27 @@ k_ret_index(Dims d, const __grid_constant__ RiArgs g) {
   }
   const size_t npairs = (size_t)d.N * d.m * ke;
   int32_t* pairs = g.ri.pairs + (size_t)pq * npairs;
+  if (keep) {
+#pragma unroll
+    for (int u = 0; u < kRiKept; ++u) {
+      if (kept[u] == 0xffffffffu) continue;
+      const int at = hist[kept[u] & 0x7fffu] + (int)(kept[u] >> 15);
+      if (MUSE_IN_RANGE(at, npairs)) pairs[at] = t0 * d.m + tid + u * kRiThreads;
+    }
+    return;
+  }
+  p = pl0;
   for (int e0 = tid; e0 < n; e0 += U * kRiThreads) {
     int c[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) c[u] = e0 + u * kRiThreads < n ? sel[e0 + u * kRiThreads] : -1;
+    const Plane p0 = p;
     for (int x = 0; x < ke; ++x) {
+      p = p0;
       int at[U];                                           // (the places of all before the first store: the atomics overlap)
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        const int key = key_of(e0 + u * kRiThreads, c[u], x);
+        const int key = key_of(p, e0 + u * kRiThreads, c[u], x);
         at[u] = key >= 0 ? atomicAdd(&hist[key], 1) : -1;
       }
 #pragma unroll
