@@ -8,7 +8,9 @@
 //      kappa tiles streamed by TMA through a ring that spans the whole operand area;
 //      score = sigma * that + beta[j] (Eq. 6).  All 64 x Ck scores stay in TMEM (512 columns).
 //   B  16 queries at a time: TMEM -> shared memory transposed to [r][j] fp32
-//   C  per query (one warp each): top-m selection, far-set softmax, P written as a bf16 operand
+//   C  per query (one warp each): top-m selection, far-set softmax, P written as a bf16 operand; the scores stay in registers from
+//      one end to the other (read again for the maximum and the weights: 4800 cycles a step of eight queries, now 2900; the whole
+//      kernel 6.25 -> 5.99 ms at 128k tokens, 512 x 2048 clusters, D = 128; 1461 -> 1450 us at 64k, 256 x 1024)
 //   D  out^T[d][r] = sum_j nu[j][d] P[r][j]      nu tiles (MN-major A operand) streamed by TMA
 //      (bringing them, or the next segment's kappa, into L2 while phase C runs evicts what others are about to read:
 //      6.25 ms without, 6.56 with nu, 6.9 to 8.4 with kappa at 128k tokens, 512 x 2048 clusters, D = 128)
@@ -32,31 +34,40 @@ constexpr int kCandMax = 128;                       // candidates kept by the co
 struct FarBars { uint64_t fullA[kMaxStA], emptyA[kMaxStA], fullD[kMaxStD], emptyD[kMaxStD], done; };
 
 
-// Top-m of one query's scores s[0..Ck) (one warp; Ck <= 32 NKMAX).  Writes the chosen clusters to
+// Scores of a lane: fours of consecutive clusters, 128 apart; v[k] is cluster 4 lane + 128 (k / 4) + k % 4.  (16-byte reads of a
+// score row without bank conflicts, and eight bytes of P at a time.)
+__device__ __forceinline__ int cluster_of(int lane, int k) { return 4 * lane + 128 * (k >> 2) + (k & 3); }
+template <int NKMAX>
+__device__ __forceinline__ void load_scores(const float* s, int NK, int lane, float (&v)[NKMAX]) {
+#pragma unroll
+  for (int k = 0; k < NKMAX; k += 4) {
+    float4 x = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+    if (k < NK) x = *reinterpret_cast<const float4*>(s + 4 * lane + 32 * k);
+    v[k] = x.x; v[k + 1] = x.y; v[k + 2] = x.z; v[k + 3] = x.w;
+  }
+}
+
+// Top-m of one query's scores s[0..Ck) (one warp; Ck <= 32 NKMAX), which the lanes hold in v.  Writes the chosen clusters to
 // so[0..m) (-1 padded, in no particular order), and removes them from the far set by setting
-// their score to -inf.  Scores become order-preserving integer keys; everything above the key T
+// their score to -inf, in v at least.  Scores become order-preserving integer keys; everything above the key T
 // of the m-th largest is taken and, among ties at T, the lowest cluster indices.
 //
 // Fast path (m <= 64, `may_compact`): the m-th largest of the 64 per-lane top-two keys, found by a
 // bitonic sort across the warp (two keys per lane, shuffles only), bounds the m-th largest score
 // from below, and on random data only about m + 4 scores reach it.  Those candidates are
 // compacted into `cand` (kCandMax keys then kCandMax indices, 128-byte segments `seg` bytes apart;
-// a lane-prefix sum gives every lane its slots, so the scatter needs no votes) and T is found by
-// bisection over 4 keys per lane.  The code is laid out for instruction-level parallelism: a
-// warp's chain of dependent votes and reductions, not the issue rate, bounds the selection.
+// a lane-prefix sum gives every lane its slots, so the scatter needs no votes) and T is the largest key that m candidates reach: a
+// lane counts for its two (bisection over 4 keys per lane, 20 dependent reductions, where there are more than 64).  The code is laid
+// out for instruction-level parallelism: a warp's chain of dependent votes and reductions, not the issue rate, bounds the selection.
 // General path (any m, many equal scores, fewer than m finite scores): bisection over all keys.
 template <int NKMAX>
 __device__ __forceinline__ void select_top_m(float* s, int Ck, int m, int32_t* so, int lane, unsigned char* cand, int seg,
-                                             bool may_compact, int* dbg = nullptr) {
-#define MUSE_SEL_CLOCK(x)
+                                             bool may_compact, float (&v)[NKMAX]) {
   const int NK = Ck >> 5;                       // scores per lane (<= NKMAX)
   auto to_key = [](float x) {
     const uint32_t b = __float_as_uint(x);
     return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
   };
-  float v[NKMAX];
-#pragma unroll
-  for (int k = 0; k < NKMAX; ++k) v[k] = k < NK ? s[lane + 32 * k] : -INFINITY;
   const uint32_t kFinite = 0x00800000u;         // smallest key above key(-inf) = 0x007fffff
   const uint32_t lt = (1u << lane) - 1u;
   float f1 = -INFINITY, f2 = -INFINITY;         // the lane's largest and second largest score
@@ -66,7 +77,6 @@ __device__ __forceinline__ void select_top_m(float* s, int Ck, int m, int32_t* s
     f1 = fmaxf(f1, v[k]);
   }
   const uint32_t m1 = to_key(f1), m2 = to_key(f2);
-  MUSE_SEL_CLOCK(c1_);
   if (may_compact && m >= 1 && m <= 64) {
     // bitonic sort, descending, of the 64 keys e = 2 lane + r held as (v0, v1)
     uint32_t v0 = m1, v1 = m2;
@@ -87,7 +97,6 @@ __device__ __forceinline__ void select_top_m(float* s, int Ck, int m, int32_t* s
     }
     const uint32_t lb = __shfl_sync(0xffffffffu, ((m - 1) & 1) ? v1 : v0, (m - 1) >> 1);
     const uint32_t kmx = __shfl_sync(0xffffffffu, v0, 0);
-    MUSE_SEL_CLOCK(c2_);
     uint32_t msk[(NKMAX + 31) / 32] = {};                     // this lane's candidates, one bit per score
     // (float comparison: the same set as by key, plus -0 beside +0, which does no harm)
     const uint32_t lbb = (lb & 0x80000000u) ? (lb & 0x7fffffffu) : ~lb;
@@ -110,13 +119,12 @@ __device__ __forceinline__ void select_top_m(float* s, int Ck, int m, int32_t* s
 #pragma unroll
       for (int w = 0; w < (NKMAX + 31) / 32; ++w) {
         for (uint32_t mm = msk[w]; mm != 0u; mm &= mm - 1u, ++pos) {
-          const int j = lane + 32 * (32 * w + __ffs((int)mm) - 1);
+          const int j = cluster_of(lane, 32 * w + __ffs((int)mm) - 1);
           *reinterpret_cast<uint32_t*>(cand + (pos >> 5) * seg + (pos & 31) * 4) = to_key(s[j]);
           *reinterpret_cast<int32_t*>(cand + (4 + (pos >> 5)) * seg + (pos & 31) * 4) = j;
         }
       }
       __syncwarp();
-      MUSE_SEL_CLOCK(c3_);
       uint32_t ck[4];
       int32_t ci[4];
 #pragma unroll
@@ -128,15 +136,26 @@ __device__ __forceinline__ void select_top_m(float* s, int Ck, int m, int32_t* s
       auto count4 = [&](uint32_t thr) {
         return (int)__reduce_add_sync(0xffffffffu, (unsigned)((ck[0] >= thr) + (ck[1] >= thr) + (ck[2] >= thr) + (ck[3] >= thr)));
       };
-      const int shared = __clz((int)(kmx ^ lb));              // 32 if the interval is a single key
-      uint32_t T = shared >= 32 ? kmx : (kmx & ~(0xffffffffu >> shared));
-      for (int bit = 31 - shared; bit >= 0; --bit) {
-        const uint32_t c2 = T | (1u << bit);
-        const int c = count4(c2);
-        if (c >= m) { T = c2; if (c == m) break; }
+      uint32_t T;
+      if (ncand <= 64) {
+        int c0 = 0, c1 = 0;                                     // candidates that reach this lane's two
+        for (int q = 0; q < ncand; q += 4) {
+          const uint4 x = *reinterpret_cast<const uint4*>(cand + (q >> 5) * seg + (q & 31) * 4);       // (past ncand: what was there before)
+          c0 += (x.x >= ck[0]) + (q + 1 < ncand && x.y >= ck[0]) + (q + 2 < ncand && x.z >= ck[0]) + (q + 3 < ncand && x.w >= ck[0]);
+          c1 += (x.x >= ck[1]) + (q + 1 < ncand && x.y >= ck[1]) + (q + 2 < ncand && x.z >= ck[1]) + (q + 3 < ncand && x.w >= ck[1]);
+        }
+        T = __reduce_max_sync(0xffffffffu, max(c0 >= m ? ck[0] : 0u, c1 >= m ? ck[1] : 0u));
+      } else {
+        const int shared = __clz((int)(kmx ^ lb));              // 32 if the interval is a single key
+        T = shared >= 32 ? kmx : (kmx & ~(0xffffffffu >> shared));
+        for (int bit = 31 - shared; bit >= 0; --bit) {
+          const uint32_t c2 = T | (1u << bit);
+          const int c = count4(c2);
+          if (c >= m) { T = c2; if (c == m) break; }
+        }
       }
-      MUSE_SEL_CLOCK(c4_);
-      int need = m - count4(T + 1u);                            // ties at T still to take (>= 0)
+      const int places = m - count4(T + 1u);                    // ties at T to take (>= 0)
+      int need = places;
       const int ntie = (int)__reduce_add_sync(0xffffffffu, (unsigned)((ck[0] == T) + (ck[1] == T) + (ck[2] == T) + (ck[3] == T)));
       bool take[4];
 #pragma unroll
@@ -152,23 +171,33 @@ __device__ __forceinline__ void select_top_m(float* s, int Ck, int m, int32_t* s
           for (int q = 0; q < 4; ++q) take[q] = take[q] || (ck[q] == T && ci[q] == jm);
         }
       }
+      // T as a number tells the taken ones, but where some of its ties are not, or where it is a zero (-0 has a key of its own)
+      const float Tf = __uint_as_float((T & 0x80000000u) ? (T & 0x7fffffffu) : ~T);
+      const bool mark = ntie > places || Tf == 0.f;
       int base = 0;
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         if (32 * q < ncand) {
           const uint32_t ms = __ballot_sync(0xffffffffu, take[q]);
-          if (take[q]) { so[base + __popc(ms & lt)] = ci[q]; s[ci[q]] = -INFINITY; }
+          if (take[q]) { so[base + __popc(ms & lt)] = ci[q]; if (mark) s[ci[q]] = -INFINITY; }
           base += __popc(ms);
         }
       }
       for (int k = base + lane; k < m; k += 32) so[k] = -1;
+      if (mark) {
+        __syncwarp();
+        load_scores<NKMAX>(s, NK, lane, v);
+      } else {
+#pragma unroll
+        for (int k = 0; k < NKMAX; ++k) v[k] = v[k] >= Tf ? -INFINITY : v[k];
+      }
       return;
     }
   }
 
-  uint32_t key[NKMAX];
+  uint32_t key[NKMAX];                          // here a lane's scores are 32 apart: the order of the votes is that of the clusters
 #pragma unroll
-  for (int k = 0; k < NKMAX; ++k) key[k] = to_key(v[k]);
+  for (int k = 0; k < NKMAX; ++k) key[k] = to_key(k < NK ? s[lane + 32 * k] : -INFINITY);
   auto count_ge = [&](uint32_t thr) {           // lane-local count, then one warp reduction
     int c = 0;
 #pragma unroll
@@ -212,6 +241,8 @@ __device__ __forceinline__ void select_top_m(float* s, int Ck, int m, int32_t* s
     }
   }
   for (int k = base + lane; k < m; k += 32) so[k] = -1;
+  __syncwarp();
+  load_scores<NKMAX>(s, NK, lane, v);
 }
 
 // NKMAX: scores per lane that the selection keeps in registers (Ck <= 32 NKMAX); MINB: CTAs per SM the register
@@ -394,37 +425,43 @@ k_far_fwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
       const int r = qs * FQ + warp;                    // one query per warp
       float* s = sc + warp * CkP;
       float sum = 0.f, mx = -INFINITY;
+      float v[NKMAX];                                  // (rows past the segment's end are masked below)
+      const int NK = CkP >> 5;
       if (r < n) {
         const int t = rows[r];
         int32_t* so = sel_out + ((size_t)pq * dm.N + t) * m;
-        if (sel_in != nullptr) {
-          const int32_t* si = sel_in + ((size_t)pq * dm.N + t) * m;
+        if (sel_in != nullptr || dm.sel_mode == MUSE_SEL_PER_QCLUSTER) {
+          const int32_t* si = sel_in != nullptr ? sel_in + ((size_t)pq * dm.N + t) * m : selq;
           for (int k = lane; k < m; k += 32) { int c = si[k]; c = (c >= 0 && c < Ck) ? c : -1; so[k] = c; if (c >= 0) s[c] = -INFINITY; }
-        } else if (dm.sel_mode == MUSE_SEL_PER_QCLUSTER) {
-          for (int k = lane; k < m; k += 32) { int c = selq[k]; so[k] = c; if (c >= 0) s[c] = -INFINITY; }
-        } else if (m > 0) {
+          __syncwarp();
+          load_scores<NKMAX>(s, NK, lane, v);
+        } else {
+          load_scores<NKMAX>(s, NK, lane, v);
           // this query's own (not yet written) P row doubles as the candidate scratch
-          int* dbg = nullptr;
-          select_top_m<NKMAX>(s, CkP, m, so, lane, Pm + r * 128, FR * 128, CkP >= 512, dbg);
+          if (m > 0) select_top_m<NKMAX>(s, CkP, m, so, lane, Pm + r * 128, FR * 128, CkP >= 512, v);
         }
-        __syncwarp();
-        for (int j = lane; j < CkP; j += 32) mx = fmaxf(mx, s[j]);
-        mx = warp_max(mx);
-      }
-      // probabilities, 8 consecutive clusters (one 16-byte chunk) per lane and step
-      for (int q = lane; q < CkP / 8; q += 32) {
-        const float4 s0 = *reinterpret_cast<const float4*>(s + q * 8), s1 = *reinterpret_cast<const float4*>(s + q * 8 + 4);
-        const float sv[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
-        uint32_t w[4];
+        float m4[4] = {v[0], v[1], v[2], v[3]};
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          float p0_ = 0.f, p1_ = 0.f;
-          if (mx != -INFINITY) { p0_ = __expf(sv[2 * k] - mx); p1_ = __expf(sv[2 * k + 1] - mx); }
-          __nv_bfloat162 b = __floats2bfloat162_rn(p0_, p1_);
-          sum += __low2float(b) + __high2float(b);
-          w[k] = *reinterpret_cast<uint32_t*>(&b);
+        for (int k = 4; k < NKMAX; ++k) m4[k & 3] = fmaxf(m4[k & 3], v[k]);
+        mx = warp_max(fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])));
+      }
+      __syncwarp();                                    // (the candidates have been read: P takes their place)
+      // probabilities, four consecutive clusters (eight bytes) at a time
+      const bool some = mx != -INFINITY;
+#pragma unroll
+      for (int k = 0; k < NKMAX; k += 4) {
+        if (k >= NK) break;
+        uint32_t w[2] = {0u, 0u};
+        if (some) {
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            const __nv_bfloat162 b = __floats2bfloat162_rn(__expf(v[k + 2 * e] - mx), __expf(v[k + 2 * e + 1] - mx));
+            sum += __low2float(b) + __high2float(b);
+            w[e] = *reinterpret_cast<const uint32_t*>(&b);
+          }
         }
-        *reinterpret_cast<uint4*>(Pm + (q >> 3) * (FR * 128) + tc::sw128_off(r, q & 7)) = make_uint4(w[0], w[1], w[2], w[3]);
+        const int q = (4 * lane + 32 * k) >> 3;
+        *reinterpret_cast<uint2*>(Pm + (q >> 3) * (FR * 128) + tc::sw128_off(r, q & 7) + 8 * (lane & 1)) = make_uint2(w[0], w[1]);
       }
       sum = warp_sum(sum);
       if (lane == 0) {
