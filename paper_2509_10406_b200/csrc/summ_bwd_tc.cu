@@ -20,8 +20,9 @@
 // 1682 us; 32 heads of 16k, 128 x 256 1222 -> 771; 16 heads of 8k, 64 x 128 322 -> 209; 4 heads of 64k, D = 128, 256 x 1024
 // 1280 -> 1201.  Two planes a step with at most 64 query clusters: 16 heads of 8k, 64 x 128, 7 planes 209 -> 168 us; 6 heads of 9k,
 // D = 128, 50 x 200, 5 planes 153 -> 121; four with at most 32: 10 heads of 1k, D = 128, 8 x 128, 3 planes 92 -> 71.
-// At D = 64 dK^T and dV^T as the two halves of one product, and read out by all warps: 168 -> 140 us, 32 heads of 16k 779 -> 681, 32
-// heads of 64k 1671 -> 1451.
+// At D = 64 dK^T and dV^T as the two halves of one product, and read out by all warps: 168 -> 142 us, 32 heads of 16k 779 -> 681, 32
+// heads of 64k 1671 -> 1451.  The first keys and centroids requested before the CTA's threads meet: 1451 -> 1417, D = 128 121 -> 114 and
+// 1195 -> 1169 (the first gradients too: the same).
 #include <cuda.h>
 #include "common.cuh"
 #include "tc05.cuh"
@@ -92,9 +93,43 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
   if (cached && tid <= dm.SB) oks[tid] = okg[tid];
   const int32_t* ok_ = cached ? oks : okg;
   if (warp == 0) tc::tmem_alloc(&tbase_s, cols);
-  if (tid == 0) {
-    tc::mbar_init(&bar_g[0], 1); tc::mbar_init(&bar_g[1], 1); tc::mbar_init(&bar_kv, 1); tc::mbar_init(&bar_q, 1); tc::mbar_init(&bar_l, 1);
-    tc::mbar_init(&bar1, 1); tc::mbar_init(&bar2, 1); tc::mbar_init_fence();
+  auto issue_kv = [&](int c0) {                           // the ninth warp: a chunk of keys and values
+    tc::mbar_expect_tx_warp(&bar_kv, 2 * kKeys);
+    const int row = (int)((size_t)pk * dm.N + c0);
+    for (int g = 0; g < G; ++g) {
+      tc::tma_load_2d_warp(sm + oK + g * NU * 128, &tm_K, 64 * g, row, &bar_kv);
+      tc::tma_load_2d_warp(sm + oV + g * NU * 128, &tm_V, 64 * g, row, &bar_kv);
+    }
+  };
+  auto issue_q = [&](int i0) {                            // ... sigma * qbar tile as bf16 hi + lo operands (split once per layer)
+    tc::mbar_expect_tx_warp(&bar_q, 2 * kTile);
+    for (int g = 0; g < G; ++g)
+      for (int c = 0; c < P; ++c) {
+        tc::tma_load_3d_warp(sm + oQhi + (g * TI + c * RP) * 128, &tm_qhi, 64 * g, i0, pq, &bar_q);
+        tc::tma_load_3d_warp(sm + oQlo + (g * TI + c * RP) * 128, &tm_qlo, 64 * g, i0, pq, &bar_q);
+      }
+  };
+  auto issue_grad = [&](int i0, int pl, int pl_end, int buf) {        // ... both gradient tiles of (plane, j, i0..i0+127)
+    tc::mbar_expect_tx_warp(&bar_g[buf], 2 * kTile);
+    unsigned char* dka = sm + (buf ? oQlo : oDka0);
+    unsigned char* dnu = sm + (buf ? oDnu1 : oDnu0);
+    for (int c = 0; c < P; ++c) {                         // (rows i >= Cq are zeros, and so are those of a plane past the last, from past the tensor's end)
+      const int row = P == 1 || pl + c < pl_end ? (pq * dm.SB + pl + c) * dm.Ck + j : dm.B * dm.Hq * dm.SB * dm.Ck;
+      for (int g = 0; g < G; ++g) {
+        tc::tma_load_3d_warp(dka + (g * TI + c * RP) * 128, &tm_dka, 64 * g, i0, row, &bar_g[buf]);
+        tc::tma_load_3d_warp(dnu + (g * TI + c * RP) * 128, &tm_dnu, 64 * g, i0, row, &bar_g[buf]);
+      }
+    }
+  };
+  // the issuer makes the barriers and has the first keys and centroids on their way before the others meet it
+  if (warp == ISSUER / 32) {
+    if (tc::elect_one()) {
+      tc::mbar_init(&bar_g[0], 1); tc::mbar_init(&bar_g[1], 1); tc::mbar_init(&bar_kv, 1); tc::mbar_init(&bar_q, 1); tc::mbar_init(&bar_l, 1);
+      tc::mbar_init(&bar1, 1); tc::mbar_init(&bar2, 1); tc::mbar_init_fence();
+    }
+    __syncwarp();
+    issue_kv(kbeg);
+    issue_q(0);
   }
   tc::fence_before_sync();
   __syncthreads();
@@ -109,14 +144,7 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
 
   for (int c0 = kbeg; c0 < kvis && ok; c0 += NU) {        // 64 keys of the cluster at a time (usually one chunk)
     __syncthreads();
-    if (warp == ISSUER / 32) {
-      tc::mbar_expect_tx_warp(&bar_kv, 2 * kKeys);
-      const int row = (int)((size_t)pk * dm.N + c0);
-      for (int g = 0; g < G; ++g) {
-        tc::tma_load_2d_warp(sm + oK + g * NU * 128, &tm_K, 64 * g, row, &bar_kv);
-        tc::tma_load_2d_warp(sm + oV + g * NU * 128, &tm_V, 64 * g, row, &bar_kv);
-      }
-    }
+    if (warp == ISSUER / 32 && c0 > kbeg) issue_kv(c0);
     int pl0 = 0;                                          // planes [pl0, pl_end) see this chunk (bucket ends grow with the plane)
     while (pl0 < dm.SB && ok_[pl0 + 1] <= c0) ++pl0;
     int pl_end = dm.SB;
@@ -128,28 +156,10 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
       const int i = i0 + L % RP, lp = P > 1 ? L / RP : 0;   // the row's query cluster, its plane within a step
       const bool in_range = cw && i < dm.Cq;
       const int ic = in_range ? i : 0;
-      auto issue_grad = [&](int pl, int buf) {            // the ninth warp: both gradient tiles of (plane, j, i0..i0+127)
-        tc::mbar_expect_tx_warp(&bar_g[buf], 2 * kTile);
-        unsigned char* dka = sm + (buf ? oQlo : oDka0);
-        unsigned char* dnu = sm + (buf ? oDnu1 : oDnu0);
-        for (int c = 0; c < P; ++c) {                     // (rows i >= Cq are zeros, and so are those of a plane past the last, from past the tensor's end)
-          const int row = P == 1 || pl + c < pl_end ? (pq * dm.SB + pl + c) * dm.Ck + j : dm.B * dm.Hq * dm.SB * dm.Ck;
-          for (int g = 0; g < G; ++g) {
-            tc::tma_load_3d_warp(dka + (g * TI + c * RP) * 128, &tm_dka, 64 * g, i0, row, &bar_g[buf]);
-            tc::tma_load_3d_warp(dnu + (g * TI + c * RP) * 128, &tm_dnu, 64 * g, i0, row, &bar_g[buf]);
-          }
-        }
-      };
       __syncthreads();                                    // every MMA that read the centroid tiles has completed (bar2 waited)
       if (warp == ISSUER / 32) {
-        // sigma * qbar tile as bf16 hi + lo operands (split once per layer), and the first gradient tiles
-        tc::mbar_expect_tx_warp(&bar_q, 2 * kTile);
-        for (int g = 0; g < G; ++g)
-          for (int c = 0; c < P; ++c) {
-            tc::tma_load_3d_warp(sm + oQhi + (g * TI + c * RP) * 128, &tm_qhi, 64 * g, i0, pq, &bar_q);
-            tc::tma_load_3d_warp(sm + oQlo + (g * TI + c * RP) * 128, &tm_qlo, 64 * g, i0, pq, &bar_q);
-          }
-        if (pl0 < pl_end) issue_grad(pl0, 0);
+        if (c0 > kbeg || i0 > 0) issue_q(i0);
+        if (pl0 < pl_end) issue_grad(i0, pl0, pl_end, 0);
       }
       // which planes hold a non-empty segment of query cluster i (others were never written by the far-field pass), 32 planes at
       // a time; up to 32 planes it is the same for every chunk of keys
@@ -229,7 +239,7 @@ k_summ_bwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_dka, const __grid_
             issue_x(k);
           }
           if (k > 0 && !tc::mbar_wait(&bar2, ph2)) ok = false;      // the previous plane's MMAs are done with the other buffer
-          if (pl + P < pl_end && ok) issue_grad(pl + P, buf ^ 1);
+          if (pl + P < pl_end && ok) issue_grad(i0, pl + P, pl_end, buf ^ 1);
         }
         ph_g ^= 1u << buf;
         if (cw && !tc::mbar_wait(&bar1, ph1)) ok = false;
