@@ -1,9 +1,10 @@
 // Far-field forward on the tensor cores for few key clusters (Ck <= 256) and short selections (m <= 16, or selections that
 // are given); far_fwd_tc.cu has the definitions and the kernel for the rest.  One CTA per (query cluster i, plane, head)
-// segment, 64 of its queries per pass (32 above 128 clusters):
+// segment, 64 of its queries per pass (32 above 128 clusters, or where segments are short):
 //   A  scores^T[j][r] = (kappa_hi[j] + kappa_lo[j]) . q[r]   clusters on the M side (tiles of 128), queries on the N side
 //   B  tensor memory -> shared memory, transposed to [r][j] fp32, beta added; the nu tiles are on their way meanwhile
-//   C  32 scores per thread, in registers (four threads per query up to 128 clusters, eight above): groups of 8 or 16 sorted by
+//   C  32 scores per thread, in registers (four threads per query up to 128 clusters, eight above; 16 scores and eight threads where
+//      segments are short): groups of 8 or 16 sorted by
 //      a branch-free network, merged to the thread's and then the query's largest m; all scores from the m-th largest up are
 //      selected (ties beyond m: lowest cluster first); softmax over the rest, P written as a bf16 operand
 //   D  out^T[d][r] = sum_j nu[j][d] P[r][j]
@@ -12,7 +13,7 @@
 //
 // Bound by instruction issue and the latency of the phases; two or three CTAs share an SM.  Against the other kernel: 32 heads
 // of 64k tokens, D = 64, 128 x 128 clusters, 8 slots 3130 -> 880 us; 32 heads of 16k, 128 x 256, 16 slots 1562 -> 621; 16 heads
-// of 8k, 64 x 128 367 -> 125; 6 heads of 9k, D = 128, 50 x 200, 10 slots 230 -> 94.
+// of 8k, 64 x 128 367 -> 101; 6 heads of 9k, D = 128, 50 x 200, 10 slots 230 -> 94.
 #include <cuda.h>
 #include "common.cuh"
 #include "tc05.cuh"
@@ -23,16 +24,16 @@ typedef __nv_bfloat16 bf16;
 int make_tmap_bf16_nd(void* out_map, const void* base, int rank, const uint64_t* dims, const uint64_t* strides_bytes, const uint32_t* box);
 
 namespace fs {
-constexpr int kJ = 128, kThreads = 256, NV = 32;           // clusters of a tile; scores per thread
-template <int D, int CT> struct Lay {                      // CT: tiles of clusters
-  static constexpr int kR = 64 / CT, TQ = 4 * CT;          // queries of a pass, threads per query
+constexpr int kJ = 128, kThreads = 256;                    // clusters of a tile
+template <int D, int CT, int NV> struct Lay {              // CT: tiles of clusters; NV: scores per thread
+  static constexpr int kR = 2 * NV / CT, TQ = kThreads / kR;                  // queries of a pass, threads per query
   static constexpr int kTile = kJ * D * 2, LD = CT * kJ + 4;                  // LD: floats per score row (16-byte reads of 8 rows do not conflict)
   // phase A: a ring of kappa tiles; then the nu tiles, and behind them the scores, later P.  (At D = 64 the 128-row products of
   // phase D read one tile past nu, and ignore the result.)
   static constexpr int kScore = (kR * LD * 4 + 1023) / 1024 * 1024, kArea0 = CT * kTile + (kScore > kTile ? kScore : kTile);
   static constexpr int NS = kArea0 / kTile < 2 * CT ? kArea0 / kTile : 2 * CT, kArea = kArea0;
   static constexpr int oNu = 0, oScore = CT * kTile, oQ = kArea, total = oQ + kR * D * 2 + 1024;
-  static constexpr int kMin = total <= 75 * 1024 ? 3 : 2;  // CTAs per SM
+  static constexpr int kMin = NV == 16 && total <= 55 * 1024 ? 4 : total <= 75 * 1024 ? 3 : 2;        // CTAs per SM
 };
 // descending sorting network (Batcher's odd-even merge) over N registers at a[o ..); P, K: the stage
 template <int N, int P = 1, int K = 1> __device__ __forceinline__ void sort_desc(float* a) {
@@ -58,14 +59,14 @@ template <int N> __device__ __forceinline__ void merge_desc(float* a, const floa
 struct Bars { uint64_t full[4], empty[4], nu, done; };
 }  // namespace fs
 
-template <int D, int CT, int ML>
-__global__ void __launch_bounds__(fs::kThreads, fs::Lay<D, CT>::kMin)
+template <int D, int CT, int ML, int NV>
+__global__ void __launch_bounds__(fs::kThreads, fs::Lay<D, CT, NV>::kMin)
 k_far_fwd_small(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_constant__ CUtensorMap tm_klo, const __grid_constant__ CUtensorMap tm_nu,
                 const bf16* __restrict__ Q, const int32_t* __restrict__ off_q, const int32_t* __restrict__ perm_q, const float* __restrict__ mu,
                 const float* __restrict__ beta, const int32_t* __restrict__ sel_in, int32_t* __restrict__ sel_out, float* __restrict__ o_far,
                 float* __restrict__ lse_far, int* __restrict__ status) {
   using namespace fs;
-  typedef Lay<D, CT> LY;
+  typedef Lay<D, CT, NV> LY;
   constexpr int G = D / 64, kTile = LY::kTile, LD = LY::LD, kR = LY::kR, TQ = LY::TQ, NS = LY::NS;
   constexpr uint32_t kCols = 64;
   extern __shared__ __align__(1024) unsigned char sm_raw[];
@@ -139,7 +140,7 @@ k_far_fwd_small(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __gri
     }
     // query rows -> K-major swizzled tile [64][D] bf16 (G blocks of [64][128 B])
     // (all of a thread's row numbers, then all of its rows are on their way at once: nothing else hides their latency)
-    constexpr int IT = kR * (D / 8) / kThreads;
+    constexpr int IT = (kR * (D / 8) + kThreads - 1) / kThreads;
     int tq[IT];
     uint4 vq[IT];
 #pragma unroll
@@ -199,7 +200,7 @@ k_far_fwd_small(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __gri
     }
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      const int t = CT == 2 ? warp >> 2 : 0, c0 = (CT == 2 ? 0 : 32 * (warp >> 2)) + 16 * h, j = t * kJ + (tid & 127);
+      const int t = CT == 2 ? warp >> 2 : 0, c0 = CT == 2 ? 16 * h : 16 * (warp >> 2) + 32 * h, j = t * kJ + (tid & 127);
       if (c0 < n16) {
         const float b = bq;
         float v[16];
@@ -356,8 +357,8 @@ k_far_fwd_small(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __gri
     // ---- E: thread = output dim; the two groups of four warps take half of the queries each
     if ((warp & 3) * 32 < D) {
 #pragma unroll
-      for (int c = 0; c < kR / 32; ++c) {
-        const int h = (warp >> 2) * (kR / 2) + 16 * c;
+      for (int c = 0; c < kR; c += 32) {
+        const int h = 16 * (warp >> 2) + c;
         if (h < n) {
           float x[16];
           tc::tmem_ld16(tbase + ((uint32_t)((warp & 3) * 32) << 16) + h, x);
@@ -382,11 +383,11 @@ bool far_fwd_small_supported(const Dims& d, bool sel_given) {
   return d.Ck <= 256 && (d.m <= 16 || sel_given || d.sel_mode == MUSE_SEL_PER_QCLUSTER);
 }
 
-template <int D, int CT, int ML>
+template <int D, int CT, int ML, int NV>
 static int far_fwd_small_t(const Dims& d, const CUtensorMap& khi, const CUtensorMap& klo, const CUtensorMap& nu, const SummPtrs& sp, const void* Q,
                            const int32_t* off_q, const int32_t* perm_q, const int32_t* sel_in, int32_t* sel_out, float* o_far, float* lse_far,
                            int* status, cudaStream_t st) {
-  return launch_pdl(k_far_fwd_small<D, CT, ML>, dim3(d.Cq, d.SB, d.B * d.Hq), fs::kThreads, fs::Lay<D, CT>::total, st, d, khi, klo, nu, (const bf16*)Q,
+  return launch_pdl(k_far_fwd_small<D, CT, ML, NV>, dim3(d.Cq, d.SB, d.B * d.Hq), fs::kThreads, fs::Lay<D, CT, NV>::total, st, d, khi, klo, nu, (const bf16*)Q,
                     off_q, perm_q, sp.mu, sp.beta, sel_in, sel_out, o_far, lse_far, status);
 }
 
@@ -402,9 +403,23 @@ int far_fwd_small(const Dims& d, const SummPtrs& sp, const void* Q, const int32_
   MUSE_RC(make_tmap_bf16_nd(&nu, sp.nu, 3, dims, strides, box));
   prof_mark("k_far_fwd_tc", st, "k_far_fwd_small");
   const bool two = d.Ck > fs::kJ, long_list = d.m > 8;
-#define MUSE_FS(D_, CT_, ML_) far_fwd_small_t<D_, CT_, ML_>(d, khi, klo, nu, sp, Q, off_q, perm_q, sel_in, sel_out, o_far, lse_far, status, st)
-  if (d.D == 128) return two ? (long_list ? MUSE_FS(128, 2, 16) : MUSE_FS(128, 2, 8)) : (long_list ? MUSE_FS(128, 1, 16) : MUSE_FS(128, 1, 8));
-  return two ? (long_list ? MUSE_FS(64, 2, 16) : MUSE_FS(64, 2, 8)) : (long_list ? MUSE_FS(64, 1, 16) : MUSE_FS(64, 1, 8));
+  // Short segments: half the queries a pass, twice the threads for each (a pass of 64 queries leaves three warps in four without one at 16
+  // a segment), and with less memory and fewer registers four CTAs on an SM at D = 64.  A segment of more queries than a pass takes a
+  // second one: 12 heads of 5005 tokens, 90 clusters, 64 | 32 queries a pass at a mean of 19 to a segment 51.7 | 48.1 us, 26 44.6 |
+  // 43.8, 32 40.0 | 42.4; 16 heads of 8k, 128 clusters at 16 122.8 | 100.7, 32 80.2 | 80.1; 4 heads of 2k, D = 128, at 8 28 | 23.  Above 128
+  // clusters it is slower from 11 queries on (D = 64; D = 128 at any number).
+  const bool few = !two && (long long)d.N <= 28ll * (d.causal ? d.S : 1) * d.Cq;
+#define MUSE_FS(D_, CT_, ML_, NV_) return far_fwd_small_t<D_, CT_, ML_, NV_>(d, khi, klo, nu, sp, Q, off_q, perm_q, sel_in, sel_out, o_far, lse_far, status, st)
+#define MUSE_FS_D(D_)                                                                                                                      \
+  do {                                                                                                                                     \
+    if (two) { if (long_list) MUSE_FS(D_, 2, 16, 32); MUSE_FS(D_, 2, 8, 32); }                                                             \
+    if (few) { if (long_list) MUSE_FS(D_, 1, 16, 16); MUSE_FS(D_, 1, 8, 16); }                                                             \
+    if (long_list) MUSE_FS(D_, 1, 16, 32);                                                                                                 \
+    MUSE_FS(D_, 1, 8, 32);                                                                                                                 \
+  } while (0)
+  if (d.D == 128) MUSE_FS_D(128);
+  MUSE_FS_D(64);
+#undef MUSE_FS_D
 #undef MUSE_FS
 }
 
