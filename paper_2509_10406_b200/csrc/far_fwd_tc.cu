@@ -11,7 +11,8 @@
 //   C  per query (one warp each): top-m selection, far-set softmax, P written as a bf16 operand; the scores stay in registers from
 //      one end to the other (read again for the maximum and the weights: 4800 cycles a step of eight queries, now 2900; the whole
 //      kernel 6.25 -> 5.99 ms at 128k tokens, 512 x 2048 clusters, D = 128; 1461 -> 1450 us at 64k, 256 x 1024)
-//   D  out^T[d][r] = sum_j nu[j][d] P[r][j]      nu tiles (MN-major A operand) streamed by TMA
+//   D  out^T[d][r] = sum_j nu[j][d] P[r][j]      nu in units of 16 KB (MN-major A operand) streamed by TMA through the score rows and,
+//      as it is used up, P (through the score rows alone, 64 KB, 27 bytes a clock: 5.99 -> 5.75 ms, 1450 -> 1429 us)
 //      (bringing them, or the next segment's kappa, into L2 while phase C runs evicts what others are about to read:
 //      6.25 ms without, 6.56 with nu, 6.9 to 8.4 with kappa at 128k tokens, 512 x 2048 clusters, D = 128)
 //   E  TMEM -> o_far (thread = d, coalesced over d for each query)
@@ -28,10 +29,11 @@ constexpr int kFJ = 128;                            // clusters per tile
 // Queries per pass FR and per selection step FQ (one warp each) are template parameters: 64 / 16 up to 1024
 // key clusters, 32 / 8 up to 2048 (all FR x Ck scores of a pass live in the 512 TMEM columns, P and the score
 // rows of a step in shared memory).
-constexpr int kMaxStA = 6, kMaxStD = 4;
+constexpr int kMaxStA = 6;
+constexpr int kSlot = 16 * 1024, kMaxUnits = 32;    // phase D: nu comes in units of 16 KB (64 clusters at D = 128, 128 at D = 64)
 constexpr int kCandMax = 128;                       // candidates kept by the compacting selection (4 per lane)
 
-struct FarBars { uint64_t fullA[kMaxStA], emptyA[kMaxStA], fullD[kMaxStD], emptyD[kMaxStD], done; };
+struct FarBars { uint64_t fullA[kMaxStA], emptyA[kMaxStA], fullD[kMaxUnits], emptyD[kMaxUnits], done; };
 
 
 // Scores of a lane: fours of consecutive clusters, 128 apart; v[k] is cluster 4 lane + 128 (k / 4) + k % 4.  (16-byte reads of a
@@ -254,7 +256,7 @@ k_far_fwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
              const __grid_constant__ CUtensorMap tm_nu, const bf16* __restrict__ Q, const int32_t* __restrict__ off_q,
              const int32_t* __restrict__ perm_q, const float* __restrict__ mu, const float* __restrict__ beta,
              const int32_t* __restrict__ sel_in, int32_t* __restrict__ sel_out, float* __restrict__ o_far,
-             float* __restrict__ lse_far, int p_bytes, int sc_bytes, int nsA, int nsD, int tcols, int* __restrict__ status) {
+             float* __restrict__ lse_far, int p_bytes, int sc_bytes, int nsA, int tcols, int* __restrict__ status) {
   pdl_wait();
   constexpr int NT = FQ * 32, NTG = FQ / 4, KT = 16 / NTG;   // threads; tile groups in the TMEM read-out; cluster tiles per group
   constexpr int kTileBytes = kFJ * D * 2, G = D / 64;        // one [128 clusters][D] bf16 operand tile; 128-byte column groups of a row
@@ -264,6 +266,10 @@ k_far_fwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
   __shared__ int32_t rows[FR];
   __shared__ float rinv[FR];
   __shared__ int32_t selq[kMaxM];
+  // phase D: where unit u of nu goes, and after which unit's products (-1: at once).  The first units go to the score region; a unit's place
+  // is free after its own products, and so is the part of P that they have read last: every kPer units' worth of P makes a further place
+  constexpr int KU = kSlot / (D * 2), kPer = kSlot / (KU * FR * 2);
+  __shared__ int16_t slot_s[kMaxUnits], after_s[kMaxUnits];
   const int i = blockIdx.x, pl = blockIdx.y, pq = blockIdx.z;
   const int blk = dm.causal ? pl + 1 : 0, Ck = dm.Ck, NJ = (Ck + kFJ - 1) / kFJ, CkP = NJ * kFJ, m = dm.m;   // CkP: clusters rounded up to whole tiles
   const int tid = threadIdx.x, warp = tc::warp_index(), lane = tid & 31;
@@ -271,7 +277,7 @@ k_far_fwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
   const int p0 = oq[0], p1 = oq[1];
   if (p0 >= p1) return;
   // operand area: phase A uses all of it as the kappa ring; afterwards P (bf16 [64][Ck]) sits at
-  // its start and the score rows of the current 16 queries, later the nu ring, behind it
+  // its start and the score rows of the current 16 queries, later nu, behind it
   unsigned char* sm = sm_raw + ((1024u - (tc::smem_u32(sm_raw) & 1023u)) & 1023u);
   unsigned char* Pm = sm;
   float* sc = reinterpret_cast<float*>(sm + p_bytes);
@@ -286,7 +292,7 @@ k_far_fwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
   if (warp == 0) tc::tmem_alloc(&tbase_s, tcols);
   if (tid == 0) {
     for (int s = 0; s < kMaxStA; ++s) { tc::mbar_init(&bars.fullA[s], 1); tc::mbar_init(&bars.emptyA[s], 1); }
-    for (int s = 0; s < kMaxStD; ++s) { tc::mbar_init(&bars.fullD[s], 1); tc::mbar_init(&bars.emptyD[s], 1); }
+    for (int s = 0; s < kMaxUnits; ++s) { tc::mbar_init(&bars.fullD[s], 1); tc::mbar_init(&bars.emptyD[s], 1); }
     tc::mbar_init(&bars.done, 1);
     tc::mbar_init_fence();
   }
@@ -308,12 +314,20 @@ k_far_fwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
       __syncwarp();
     }
   }
+  if (tid == 64) {
+    const int n0 = sc_bytes / kSlot, NU = CkP / KU;
+    for (int u = 0; u < NU; ++u) {
+      const int e = u - n0, g = e / (kPer + 1), r = e % (kPer + 1);            // (of kPer + 1 places in turn the last one is P's)
+      slot_s[u] = (int16_t)(e < 0 ? u : r < kPer ? slot_s[g * kPer + r] : n0 + g);
+      after_s[u] = (int16_t)(e < 0 ? -1 : g * kPer + min(r, kPer - 1));
+    }
+  }
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
   pdl_trigger();                                           // (tensor memory has been allocated)
   const uint32_t tbase = tbase_s;
-  uint32_t cntA = 0, cntD = 0, done_ph = 0;   // tiles of the earlier passes (same in every thread); phase of `done`
+  uint32_t cntA = 0, done_ph = 0, phD = 0;   // tiles of the earlier passes (same in every thread); phase of `done`
   bool ok = true;
   // TMA producers: warps 0, 2, 3, 4 (an elected lane each).  One thread sustains only about 30 bytes per clock
   // (every bulk-tensor instruction holds it for some 270 clocks per 16 KB box, every wait after one
@@ -322,7 +336,6 @@ k_far_fwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
   // belongs to one producer and its waits on the stage's barrier never fall a phase behind.
   const int prod = warp == 0 ? 0 : (warp >= 2 && warp <= 4) ? warp - 1 : -1;
   const int WA = nsA % 4 == 0 ? 4 : nsA % 3 == 0 ? 3 : nsA % 2 == 0 ? 2 : 1;
-  const int WD = nsD % 4 == 0 ? 4 : nsD % 2 == 0 ? 2 : 1;
   const int lq = warp & 3, tg = warp >> 2;            // TMEM lane quarter of this warp, tile group
 
   for (int r0 = p0; r0 < p1 && ok; r0 += FR) {
@@ -331,7 +344,7 @@ k_far_fwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
     //         the producers load (TMA), thread 32 consumes (MMA), so neither waits for the other's latency.
     //         The first ring-full of tiles is requested before the query rows are gathered.
     // (ring stage, phase and owning producer of a tile advance by increments: no division per tile)
-    const int sA0 = cntA % nsA, phA0 = (cntA / nsA) & 1, sD0 = cntD % nsD, phD0 = (cntD / nsD) & 1;
+    const int sA0 = cntA % nsA, phA0 = (cntA / nsA) & 1;
     int sa = sA0, pha = phA0, wa = sA0 % WA;             // of the next tile this producer looks at
     auto next_a = [&]() {
       if (++sa == nsA) { sa = 0; pha ^= 1; }
@@ -473,34 +486,32 @@ k_far_fwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
     tc::fence_async_smem();
     tc::fence_before_sync();
     __syncthreads();
-    // ---- D: out^T = nu^T P^T, nu tiles through an nsD-stage TMA ring in the score region
-    if (prod >= 0 && prod < WD && ok) {
-      unsigned char* ring = sm + p_bytes;
-      for (int t = 0, s = sD0, ph = phD0, w = sD0 % WD; t < NJ; ++t) {
-        const int s_ = s, ph_ = ph, w_ = w;
-        if (++s == nsD) { s = 0; ph ^= 1; }
-        if (++w == WD) w = 0;
-        if (w_ != prod) continue;
-        if (!tc::mbar_wait(&bars.emptyD[s_], ph_ ^ 1)) { ok = false; break; }
-        tc::mbar_expect_tx_warp(&bars.fullD[s_], kTileBytes);
-        for (int g = 0; g < G; ++g) tc::tma_load_3d_warp(ring + s_ * kTileBytes + g * kFJ * 128, &tm_nu, 64 * g, t * kFJ, seg, &bars.fullD[s_]);
+    // ---- D: out^T = nu^T P^T, nu by units through the score region and the part of P that has been used
+    const int NU = CkP / KU;
+    if (prod >= 0 && ok) {
+      for (int u = prod; u < NU; u += 4) {
+        if (after_s[u] >= 0 && !tc::mbar_wait(&bars.emptyD[after_s[u]], phD)) { ok = false; break; }
+        const int s = slot_s[u], n0 = sc_bytes / kSlot;
+        unsigned char* dst = s < n0 ? sm + p_bytes + s * kSlot : sm + (s - n0) * kSlot;
+        tc::mbar_expect_tx_warp(&bars.fullD[u], kSlot);
+        for (int g = 0; g < G; ++g) tc::tma_load_3d_warp(dst + g * KU * 128, &tm_nu, 64 * g, u * KU, seg, &bars.fullD[u]);
       }
     } else if (warp == 1 && ok) {
       tc::fence_after_sync();
       // M = 128 output dims even when D = 64: the second 64-dim group of the MN-major operand then reads whatever
-      // follows the tile in shared memory, and output lanes 64..127 hold numbers that nobody reads
+      // follows the unit in shared memory, and output lanes 64..127 hold numbers that nobody reads
       const uint32_t idesc = tc::idesc_bf16(128, FR, 1, 0);
       const uint64_t dp0 = tc::smem_desc_sw128(tc::smem_u32(Pm), 16, 1024);
-      const uint64_t dn0 = tc::smem_desc_sw128(tc::smem_u32(sm + p_bytes), kFJ * 128, 1024);
-      for (int u = 0, s = sD0, ph = phD0; u < NJ; ++u) {
-        if (!tc::mbar_wait(&bars.fullD[s], ph)) { ok = false; break; }
-        const uint64_t da = tc::desc_step(dn0, (uint32_t)s * kTileBytes), dp = tc::desc_step(dp0, (uint32_t)(2 * u) * (FR * 128));
+      const uint64_t dn0 = tc::smem_desc_sw128(tc::smem_u32(sm), KU * 128, 1024);
+      for (int u = 0; u < NU; ++u) {
+        const int s = slot_s[u], n0 = sc_bytes / kSlot;
+        const uint64_t da = tc::desc_step(dn0, (uint32_t)(s < n0 ? p_bytes + s * kSlot : (s - n0) * kSlot)), dp = tc::desc_step(dp0, (uint32_t)(u * (KU / 64)) * (FR * 128));
+        if (!tc::mbar_wait(&bars.fullD[u], phD)) { ok = false; break; }
 #pragma unroll
-        for (int ks = 0; ks < kFJ / 16; ++ks)
+        for (int ks = 0; ks < KU / 16; ++ks)
           tc::mma_bf16_ss_warp(tbase, tc::desc_step(da, ks * 16 * 128), tc::desc_step(dp, (ks / 4) * (FR * 128) + (ks % 4) * 32), idesc,
                           u > 0 || ks > 0);
-        tc::mma_commit_warp(&bars.emptyD[s]);
-        if (++s == nsD) { s = 0; ph ^= 1; }
+        tc::mma_commit_warp(&bars.emptyD[u]);
       }
       if (ok) tc::mma_commit_warp(&bars.done);
     }
@@ -510,7 +521,7 @@ k_far_fwd_tc(Dims dm, const __grid_constant__ CUtensorMap tm_khi, const __grid_c
     }
     ok = __syncthreads_and(ok);
     done_ph ^= 1;
-    cntD += NJ;
+    phD ^= 1;
     tc::fence_after_sync();
     // ---- E: thread = output dim d; warps 0-3 read queries 0..31, warps 4-7 queries 32..63
     if (warp < FR / 8) {
@@ -547,21 +558,20 @@ int far_fwd_tc(const Dims& d, const SummPtrs& sp, const void* Q, const int32_t* 
   // [segments][Ck][D]
   const uint64_t dims[3] = {(uint64_t)d.D, (uint64_t)d.Ck, (uint64_t)d.B * d.Hq * d.SB * d.Cq};
   const uint64_t strides[2] = {(uint64_t)d.D * 2, (uint64_t)d.Ck * d.D * 2};
-  const uint32_t box[3] = {64, kFJ, 1};
+  const uint32_t box[3] = {64, kFJ, 1}, box_nu[3] = {64, (uint32_t)(kSlot / (d.D * 2)), 1};
   CUtensorMap khi, klo, nu;
   MUSE_RC(make_tmap_bf16_nd(&khi, sp.khi, 3, dims, strides, box));
   MUSE_RC(make_tmap_bf16_nd(&klo, sp.klo, 3, dims, strides, box));
-  MUSE_RC(make_tmap_bf16_nd(&nu, sp.nu, 3, dims, strides, box));
+  MUSE_RC(make_tmap_bf16_nd(&nu, sp.nu, 3, dims, strides, box_nu));
   const int CkP = cdiv(d.Ck, kFJ) * kFJ;
   const bool wide = d.Ck > 1024;                                         // 32 queries per pass, 8 per selection step
   const int FR = wide ? 32 : 64, FQ = wide ? 8 : 16;
   const int tile_bytes = kFJ * d.D * 2;
   const int p_bytes = FR * CkP * 2;                                    // P: bf16 [FR][Ck]
-  int sc_bytes = FQ * CkP * 4;                                         // FQ score rows, later the nu ring
+  int sc_bytes = FQ * CkP * 4;                                         // FQ score rows, later nu
   if (sc_bytes < 2 * tile_bytes) sc_bytes = 2 * tile_bytes;
-  int nsA = (p_bytes + sc_bytes) / tile_bytes, nsD = sc_bytes / tile_bytes;
+  int nsA = (p_bytes + sc_bytes) / tile_bytes;
   nsA = nsA > kMaxStA ? kMaxStA : nsA;
-  nsD = nsD > kMaxStD ? kMaxStD : nsD;
   // (D = 64: one more tile of room behind the ring, which the padded 128-row products of phase D read past)
   const size_t smem = (size_t)p_bytes + sc_bytes + FR * d.D * 2 + 1024 + (d.D == 64 ? tile_bytes : 0);
   prof_mark("k_far_fwd_tc", st, "k_far_fwd_tc");
@@ -571,7 +581,7 @@ int far_fwd_tc(const Dims& d, const SummPtrs& sp, const void* Q, const int32_t* 
 #define MUSE_FAR_FWD_LAUNCH(FR_, FQ_, D_, NK_, MB_)                                                                              \
   do {                                                                                                                         \
     MUSE_RC(launch_pdl(k_far_fwd_tc<FR_, FQ_, D_, NK_, MB_>, dim3(d.Cq, d.SB, d.B * d.Hq), FQ_ * 32, smem, st,                     \
-        d, khi, klo, nu, (const bf16*)Q, off_q, perm_q, sp.mu, sp.beta, sel_in, sel_out, o_far, lse_far, p_bytes, sc_bytes, nsA, nsD, tcols, status));   \
+        d, khi, klo, nu, (const bf16*)Q, off_q, perm_q, sp.mu, sp.beta, sel_in, sel_out, o_far, lse_far, p_bytes, sc_bytes, nsA, tcols, status));   \
   } while (0)
   if (wide) { if (d.D == 128) MUSE_FAR_FWD_LAUNCH(32, 8, 128, 64, 1); else MUSE_FAR_FWD_LAUNCH(32, 8, 64, 64, 1); }
   else if (d.Ck <= 256) { if (d.D == 128) MUSE_FAR_FWD_LAUNCH(64, 16, 128, 8, 2); else MUSE_FAR_FWD_LAUNCH(64, 16, 64, 8, 2); }

@@ -15,10 +15,23 @@ FAR_SIMT = 2                                   # muse_test_force_paths: the FFMA
     (64, 40, 1, 4, 1, True), (64, 40, 9, 5, 8, True), (64, 33, 127, 3, 16, True), (64, 64, 128, 8, 0, True), (64, 90, 120, 6, 9, True),
     (64, 128, 64, 1, 5, False), (128, 40, 17, 4, 9, True), (128, 48, 128, 5, 8, True), (128, 70, 100, 4, 16, True)])
 def test_short_segments_match_the_ffma_kernel(D, Cq, Ck, S, m, causal):
+    _compare(D, Cq, Ck, S, m, causal, S * Cq * 20, "k_far_fwd_tc/k_far_fwd_small")
+
+
+@pytest.mark.parametrize("D,Cq,Ck,S,m", [
+    (64, 12, 257, 3, 20), (64, 8, 1024, 2, 32), (64, 10, 1100, 2, 17), (64, 6, 2048, 2, 40), (128, 12, 300, 3, 33), (128, 9, 640, 2, 20),
+    (128, 8, 1152, 2, 64), (128, 10, 1500, 2, 8), (128, 6, 2048, 2, 32)])
+def test_many_clusters_match_the_ffma_kernel(D, Cq, Ck, S, m):
+    """The kernel for more than 256 clusters, or longer selections: nu units that come through few and many places, passes of 32 and 64
+    queries, one to three of them."""
+    _compare(D, Cq, Ck, S, m, True, S * Cq * 60, "k_far_fwd_tc/k_far_fwd_tc")
+
+
+def _compare(D, Cq, Ck, S, m, causal, N, kernel):
     from paper_2509_10406_b200 import binding as mb
     from tests.gpu_util import kernels_launched
-    B, Hq, Hkv, per = 1, 4, 2, 20
-    N = S * Cq * per
+    N = max(N, -(-Ck // S) * S)
+    B, Hq, Hkv = 1, 4, 2
     g = torch.Generator(device="cuda").manual_seed(N + Ck)
     e = lambda h, n: torch.randn(B, h, n, D, generator=g, device="cuda")  # noqa: E731
     Q, K, V = (e(Hq, N) * 2).to(torch.bfloat16), e(Hkv, N).to(torch.bfloat16), e(Hkv, N).to(torch.bfloat16)
@@ -39,7 +52,7 @@ def test_short_segments_match_the_ffma_kernel(D, Cq, Ck, S, m, causal):
         finally:
             mb.muse_test_force_paths(0)
         assert mb.muse_status(buf.ws) == 0
-        assert ("k_far_fwd_tc/k_far_fwd_small" in k.names) == (mask == 0)
+        assert (kernel in k.names) == (mask == 0)
         got.append((buf.sel[..., :min(m, Ck)].sort(dim=-1).values.clone(), buf.O.float(), buf.LSE.clone()))
     (s0, o0, l0), (s1, o1, l1) = got
     same = (s0 == s1).all(dim=-1)
