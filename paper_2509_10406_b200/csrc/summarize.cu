@@ -113,7 +113,8 @@ k_summarize(Dims dm, const T* __restrict__ Kp, const T* __restrict__ Vp, const i
   extern __shared__ float smf[];
   float* qb = smf;                         // [64][LDQ]  sigma * qbar tile
   float* kv = qb + kSumI * LDQ;            // [KC][LDKV] rows [k | v]
-  float* Ls = kv + kSumKC * LDKV;          // [64][LDL]  tilt logits
+  float* Ls = kv + kSumKC * LDKV;          // [64][LDL]  weights exp(tilt logit - running maximum)
+  __shared__ float M_s[kSumI], sc_s[kSumI];  // the rows' running maxima, and what a chunk rescales the sums by
   const int j = blockIdx.x, i0 = blockIdx.y * kSumI, pq = blockIdx.z;
   const int b_ = pq / dm.Hq, h = pq % dm.Hq, pk = b_ * dm.Hkv + dm.hm.g[h];
   const int tid = threadIdx.x;
@@ -131,7 +132,7 @@ k_summarize(Dims dm, const T* __restrict__ Kp, const T* __restrict__ Vp, const i
   const int ip = tid >> 3, sl = tid & 7;           // phase 2: i pair, dim slice
   const int li = tid >> 2, ug = tid & 3;           // phase 1: i, group of 4 keys
   float acc[2][NV][4];
-  float M[2] = {-INFINITY, -INFINITY}, s[2] = {0.f, 0.f};
+  float M = -INFINITY, s[2] = {0.f, 0.f};      // M: of row li (the same in its four threads)
 #pragma unroll
   for (int a = 0; a < 2; ++a)
 #pragma unroll
@@ -142,9 +143,10 @@ k_summarize(Dims dm, const T* __restrict__ Kp, const T* __restrict__ Vp, const i
   for (int b = 0; b < dm.SB; ++b) {
     const int p0 = off[b], p1 = off[b + 1];
     if (per_block) {                                    // the summary of block b alone: the running state starts afresh
+      M = -INFINITY;
 #pragma unroll
       for (int a = 0; a < 2; ++a) {
-        M[a] = -INFINITY; s[a] = 0.f;
+        s[a] = 0.f;
 #pragma unroll
         for (int k = 0; k < NV; ++k)
 #pragma unroll
@@ -175,30 +177,39 @@ k_summarize(Dims dm, const T* __restrict__ Kp, const T* __restrict__ Vp, const i
             }
           }
         }
+        // the weights, once per row and key (each of the eight threads that share a row's dims used to make all of them)
+        float cm = -INFINITY;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) Ls[li * LDL + ug * 4 + u] = dot[u];
+        for (int u = 0; u < 4; ++u) cm = ug * 4 + u < n ? fmaxf(cm, dot[u]) : cm;
+        cm = fmaxf(cm, __shfl_xor_sync(0xffffffffu, cm, 1));
+        cm = fmaxf(cm, __shfl_xor_sync(0xffffffffu, cm, 2));
+        const float Mn = fmaxf(M, cm);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) if (ug * 4 + u < n) Ls[li * LDL + ug * 4 + u] = expf(dot[u] - Mn);
+        if (ug == 0) { sc_s[li] = expf(M - Mn); M_s[li] = Mn; }       // exp(-inf) = 0 on the first keys
+        M = Mn;
       }
       __syncthreads();
+      const float sc[2] = {sc_s[ip * 2], sc_s[ip * 2 + 1]};
 #pragma unroll
       for (int a = 0; a < 2; ++a) {
-        const float* Lr = Ls + (ip * 2 + a) * LDL;
-        float cm = -INFINITY;
-        for (int u = 0; u < n; ++u) cm = fmaxf(cm, Lr[u]);
-        const float Mn = fmaxf(M[a], cm);
-        const float sc = expf(M[a] - Mn);            // exp(-inf) = 0 on the first keys
-        M[a] = Mn; s[a] *= sc;
+        s[a] *= sc[a];
 #pragma unroll
         for (int k = 0; k < NV; ++k)
 #pragma unroll
-          for (int c = 0; c < 4; ++c) acc[a][k][c] *= sc;
-        for (int u = 0; u < n; ++u) {
-          const float w = expf(Lr[u] - Mn);
-          s[a] += w;
+          for (int c = 0; c < 4; ++c) acc[a][k][c] *= sc[a];
+      }
+#pragma unroll 2
+      for (int u = 0; u < n; ++u) {
+        const float w[2] = {Ls[ip * 2 * LDL + u], Ls[(ip * 2 + 1) * LDL + u]};
+        s[0] += w[0]; s[1] += w[1];
 #pragma unroll
-          for (int k = 0; k < NV; ++k) {
-            float4 x = ld4(kv + u * LDKV + sl * 4 + 32 * k);
-            acc[a][k][0] = fmaf(w, x.x, acc[a][k][0]); acc[a][k][1] = fmaf(w, x.y, acc[a][k][1]);
-            acc[a][k][2] = fmaf(w, x.z, acc[a][k][2]); acc[a][k][3] = fmaf(w, x.w, acc[a][k][3]);
+        for (int k = 0; k < NV; ++k) {
+          const float4 x = ld4(kv + u * LDKV + sl * 4 + 32 * k);
+#pragma unroll
+          for (int a = 0; a < 2; ++a) {
+            acc[a][k][0] = fmaf(w[a], x.x, acc[a][k][0]); acc[a][k][1] = fmaf(w[a], x.y, acc[a][k][1]);
+            acc[a][k][2] = fmaf(w[a], x.z, acc[a][k][2]); acc[a][k][3] = fmaf(w[a], x.w, acc[a][k][3]);
           }
         }
       }
@@ -227,7 +238,7 @@ k_summarize(Dims dm, const T* __restrict__ Kp, const T* __restrict__ Vp, const i
       }
       qk += __shfl_xor_sync(0xffffffffu, qk, 1); qk += __shfl_xor_sync(0xffffffffu, qk, 2); qk += __shfl_xor_sync(0xffffffffu, qk, 4);
       if (sl == 0 && live) {
-        const float m_ = some ? M[a] + logf(s[a]) : -INFINITY;
+        const float m_ = some ? M_s[ip * 2 + a] + logf(s[a]) : -INFINITY;
         sp.mu[ent] = m_;
         sp.beta[ent] = some ? m_ - qk : -INFINITY;
       }
