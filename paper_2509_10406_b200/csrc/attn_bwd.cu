@@ -268,8 +268,8 @@ k_ret_bwd(Dims dm, const T* __restrict__ Q, const T* __restrict__ dO, const T* _
         load_tile<T, D>(dOs, dOb, nq, [&](int r) { return pid_s[r] / dm.m; }, tid);
         __syncthreads();
         float s[4][4], dp[4][4];
-        mm_nt<T, D>(Qs, Ks, s, ty, tx);
-        mm_nt<T, D>(dOs, Vs, dp, ty, tx);
+        mm_nt<T, D>(Qs, Ks, s, ty, tx, nq);
+        mm_nt<T, D>(dOs, Vs, dp, ty, tx, nq);
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
           const int row = ty * 4 + r;
@@ -282,15 +282,15 @@ k_ret_bwd(Dims dm, const T* __restrict__ Q, const T* __restrict__ dO, const T* _
           st4(Ps + row * kLDP + tx * 4, make_float4(p[0], p[1], p[2], p[3]));
         }
         __syncthreads();
-        mm_tn<T, D>(Ps, dOs, dv, ty, tx);
+        mm_tn<T, D>(Ps, dOs, dv, ty, tx, nq, nk);
         __syncthreads();
 #pragma unroll
         for (int r = 0; r < 4; ++r) st4(Ps + (ty * 4 + r) * kLDP + tx * 4, make_float4(dp[r][0], dp[r][1], dp[r][2], dp[r][3]));
         __syncthreads();
-        mm_tn<T, D>(Ps, Qs, dk, ty, tx);
+        mm_tn<T, D>(Ps, Qs, dk, ty, tx, nq, nk);
         float dq[4][D / 64][4];
         zero_acc<D>(dq);
-        mm_pn<T, D>(Ps, Ks, dq, ty, tx);
+        mm_pn<T, D>(Ps, Ks, dq, ty, tx, nq, nk);
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
           const int row = ty * 4 + r;
@@ -408,8 +408,8 @@ k_far_bwd(Dims dm, const T* __restrict__ Q, const T* __restrict__ dO, const floa
       __syncthreads();
       if (!single) { load_rows(r0, n); zero_acc<D>(dq); }
       float s[4][4], dp[4][4];
-      mm_nt<float, D>(qr, kap, s, ty, tx);
-      mm_nt<float, D>(dOs, nus, dp, ty, tx);
+      mm_nt<float, D>(qr, kap, s, ty, tx, n);
+      mm_nt<float, D>(dOs, nus, dp, ty, tx, n);
 #pragma unroll
       for (int r = 0; r < 4; ++r) {
         const int row = ty * 4 + r;
@@ -425,14 +425,14 @@ k_far_bwd(Dims dm, const T* __restrict__ Q, const T* __restrict__ dO, const floa
         st4(Ps + row * kLDP + tx * 4, make_float4(p[0], p[1], p[2], p[3]));
       }
       __syncthreads();
-      mm_tn<float, D>(Ps, dOs, dnv, ty, tx);
+      mm_tn<float, D>(Ps, dOs, dnv, ty, tx, n, Ck - j0);
       __syncthreads();
 #pragma unroll
       for (int r = 0; r < 4; ++r) st4(Ps + (ty * 4 + r) * kLDP + tx * 4, make_float4(dp[r][0], dp[r][1], dp[r][2], dp[r][3]));
       __syncthreads();
-      mm_tn<float, D>(Ps, qr, dka, ty, tx);
-      mm_pn<float, D>(Ps, kap, dq, ty, tx);
-      if (tid < kTile) { float cs = 0.f; for (int r = 0; r < kTile; ++r) cs += Ps[r * kLDP + tid]; dmu_acc += cs; }
+      mm_tn<float, D>(Ps, qr, dka, ty, tx, n, Ck - j0);
+      mm_pn<float, D>(Ps, kap, dq, ty, tx, n, min(kTile, Ck - j0));
+      if (tid < kTile) { float cs = 0.f; for (int r = 0; r < n; ++r) cs += Ps[r * kLDP + tid]; dmu_acc += cs; }
       if (!single) {
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
@@ -526,6 +526,7 @@ k_summ_bwd(Dims dm, const T* __restrict__ Kp, const T* __restrict__ Vp, const in
   const int pl_last = gridDim.z > 1 ? (int)blockIdx.z : 0;
   if (gridDim.z > 1 && ok[pl_last] >= ok[pl_last + 1]) return;
   for (int i0 = 0; i0 < dm.Cq; i0 += kTile) {
+    const int ni = min(kTile, dm.Cq - i0);
     __syncthreads();
     for (int e = tid; e < kTile * (D / 4); e += kFlashThreads) {
       const int r = e / (D / 4), q = e % (D / 4);
@@ -554,7 +555,7 @@ k_summ_bwd(Dims dm, const T* __restrict__ Kp, const T* __restrict__ Vp, const in
         else if (per_block) muref[tid] = INFINITY;       // an empty bucket has no weights of its own
       }
       __syncthreads();
-      for (int e = tid; e < kTile * (D / 4); e += kFlashThreads) {
+      for (int e = tid; e < ni * (D / 4); e += kFlashThreads) {
         const int r = e / (D / 4), q = e % (D / 4);
         float4 u = ld4(GU + r * LD + q * 4), w = ld4(GW + r * LD + q * 4);
         const float f = fac[r];
@@ -580,9 +581,9 @@ k_summ_bwd(Dims dm, const T* __restrict__ Kp, const T* __restrict__ Vp, const in
         load_tile_f32<T, D>(Vs, Vb, nk, [&](int r) { return c0 + r; }, tid);
         __syncthreads();
         float l[4][4], x1[4][4], x2[4][4];
-        mm_nt<float, D>(qb, Ks, l, ty, tx);
-        mm_nt<float, D>(GU, Ks, x1, ty, tx);
-        mm_nt<float, D>(GW, Vs, x2, ty, tx);
+        mm_nt<float, D>(qb, Ks, l, ty, tx, ni);
+        mm_nt<float, D>(GU, Ks, x1, ty, tx, ni);
+        mm_nt<float, D>(GW, Vs, x2, ty, tx, ni);
         float wc[4][4];
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
@@ -600,14 +601,14 @@ k_summ_bwd(Dims dm, const T* __restrict__ Kp, const T* __restrict__ Vp, const in
         __syncthreads();
         float dk[4][D / 64][4], dv[4][D / 64][4];
         zero_acc<D>(dk); zero_acc<D>(dv);
-        mm_tn<float, D>(Ps, GU, dk, ty, tx);
-        mm_tn<float, D>(Ps, GW, dv, ty, tx);
+        mm_tn<float, D>(Ps, GU, dk, ty, tx, ni, nk);
+        mm_tn<float, D>(Ps, GW, dv, ty, tx, ni, nk);
         if (dm.agg_grad) {
           __syncthreads();
 #pragma unroll
           for (int r = 0; r < 4; ++r) st4(Ps + (ty * 4 + r) * kLDP + tx * 4, make_float4(wc[r][0], wc[r][1], wc[r][2], wc[r][3]));
           __syncthreads();
-          mm_tn<float, D>(Ps, qb, dk, ty, tx);
+          mm_tn<float, D>(Ps, qb, dk, ty, tx, ni, nk);
         }
 #pragma unroll
         for (int r = 0; r < 4; ++r) {

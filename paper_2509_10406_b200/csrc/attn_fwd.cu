@@ -287,14 +287,14 @@ k_ret_fwd(Dims dm, const T* __restrict__ Q, const T* __restrict__ Kp, const T* _
       load_tile<T, D>(Vs, Vb, nk, [&](int r) { return c0 + r; }, tid);
       __syncthreads();
       float s[4][4];
-      mm_nt<T, D>(Qs, Ks, s, ty, tx);
+      mm_nt<T, D>(Qs, Ks, s, ty, tx, nq);
 #pragma unroll
       for (int r = 0; r < 4; ++r)
 #pragma unroll
         for (int c = 0; c < 4; ++c) s[r][c] = (tx * 4 + c < nk) ? s[r][c] * dm.sigma : -INFINITY;
       online_softmax_step<D>(s, m_run, l_run, o, Ps, ty, tx);
       __syncthreads();
-      mm_pn<T, D>(Ps, Vs, o, ty, tx);
+      mm_pn<T, D>(Ps, Vs, o, ty, tx, nq, nk);
     }
 #pragma unroll
     for (int r = 0; r < 4; ++r) {

@@ -13,14 +13,18 @@ constexpr int kLDP = kTile + 4;    // leading dimension of the fp32 probability 
 
 template <class T> struct Pad { static constexpr int v = 16 / sizeof(T); };
 
-// acc[r][c] = sum_d A[ty*4+r][d] * B[tx*4+c][d]
+// Tiles are rarely full where clusters and segments are small (16 queries by 8 keys of the 64 by 64 in a retrieval of 2k tokens, 128
+// clusters), so the products take the rows, and the outputs, that there are; the rest are zeros.
+
+// acc[r][c] = sum_d A[ty*4+r][d] * B[tx*4+c][d], rows of A below `rows`
 template <class T, int D>
-__device__ __forceinline__ void mm_nt(const T* __restrict__ A, const T* __restrict__ B, float acc[4][4], int ty, int tx) {
+__device__ __forceinline__ void mm_nt(const T* __restrict__ A, const T* __restrict__ B, float acc[4][4], int ty, int tx, int rows = kTile) {
   constexpr int LD = D + Pad<T>::v;
 #pragma unroll
   for (int r = 0; r < 4; ++r)
 #pragma unroll
     for (int c = 0; c < 4; ++c) acc[r][c] = 0.f;
+  if (ty * 4 >= rows) return;
 #pragma unroll 4
   for (int d = 0; d < D; d += 4) {
     float4 a[4], b[4];
@@ -38,12 +42,13 @@ __device__ __forceinline__ void mm_nt(const T* __restrict__ A, const T* __restri
   }
 }
 
-// acc[r][k][c] += sum_j P[ty*4+r][j] * B[j][tx*4 + 64k + c]     (P fp32 [64][kLDP])
+// acc[r][k][c] += sum_j P[ty*4+r][j] * B[j][tx*4 + 64k + c]     (P fp32 [64][kLDP]), rows of P below `rows`, j below `inner`
 template <class T, int D>
-__device__ __forceinline__ void mm_pn(const float* __restrict__ P, const T* __restrict__ B, float acc[4][D / 64][4], int ty, int tx) {
+__device__ __forceinline__ void mm_pn(const float* __restrict__ P, const T* __restrict__ B, float acc[4][D / 64][4], int ty, int tx, int rows = kTile, int inner = kTile) {
   constexpr int LD = D + Pad<T>::v;
+  if (ty * 4 >= rows) return;
 #pragma unroll 2
-  for (int j = 0; j < kTile; j += 4) {
+  for (int j = 0; j < inner; j += 4) {
     float4 p[4];
 #pragma unroll
     for (int r = 0; r < 4; ++r) p[r] = ld4(P + (ty * 4 + r) * kLDP + j);
@@ -62,12 +67,13 @@ __device__ __forceinline__ void mm_pn(const float* __restrict__ P, const T* __re
   }
 }
 
-// acc[jj][k][c] += sum_r P[r][ty*4+jj] * B[r][tx*4 + 64k + c]   (P transposed on the fly)
+// acc[jj][k][c] += sum_r P[r][ty*4+jj] * B[r][tx*4 + 64k + c]   (P transposed on the fly), r below `inner`, columns of P below `outs`
 template <class T, int D>
-__device__ __forceinline__ void mm_tn(const float* __restrict__ P, const T* __restrict__ B, float acc[4][D / 64][4], int ty, int tx) {
+__device__ __forceinline__ void mm_tn(const float* __restrict__ P, const T* __restrict__ B, float acc[4][D / 64][4], int ty, int tx, int inner = kTile, int outs = kTile) {
   constexpr int LD = D + Pad<T>::v;
+  if (ty * 4 >= outs) return;
 #pragma unroll 4
-  for (int r = 0; r < kTile; ++r) {
+  for (int r = 0; r < inner; ++r) {
     float4 p = ld4(P + r * kLDP + ty * 4);
 #pragma unroll
     for (int k = 0; k < D / 64; ++k) {
