@@ -207,18 +207,20 @@ k_local_bwd_dq(Dims dm, const T* __restrict__ Q, const T* __restrict__ K, const 
 }
 
 // ---------------------------------------------------------------------------------------------
-// Retrieval backward: one CTA per (key cluster j, head), or per (j, head, plane, share of the plane's
-// pair tiles) when that leaves most of the chip idle (planes > 1; the fp32 check layer has 16 clusters: 585 -> 101 us).
-// Key chunks are the outer loop so that dK, dV of a chunk accumulate in registers over every plane
-// and query tile of the CTA that sees it; split CTAs add them to the zeroed accumulators.  The
-// per-pair dq partials are owned by one CTA (a pair retrieves exactly one cluster).
+// Retrieval backward: one CTA per (key cluster j, head, plane, half of the plane's pair tiles).  Key chunks are the outer loop so that
+// dK, dV of a chunk accumulate in registers over every query tile of the CTA; the CTAs of a cluster add them to the zeroed
+// accumulators.  The per-pair dq partials are owned by one CTA (a pair retrieves exactly one cluster).
+// Queries crowd on few clusters, so a CTA per cluster, which stored its sums, left the chip waiting for the largest one: 4 heads of 2k
+// tokens, 128 clusters, 8 slots 781 -> 168 us; 16 heads of 4k 2632 -> 1170; 32 heads of 4k 3121 -> 2145; D = 128, 8 heads of 4k 3111 ->
+// 1321; the fp32 check layer of 16 clusters 585 -> 75.  Four or eight parts a plane gain up to 17 % there and lose 16 % and more at 32 heads.
 // ---------------------------------------------------------------------------------------------
+constexpr int kRetShares = 2;
 template <class T, int D>
 __global__ void __launch_bounds__(kFlashThreads)
 k_ret_bwd(Dims dm, const T* __restrict__ Q, const T* __restrict__ dO, const T* __restrict__ Kp,
           const T* __restrict__ Vp, const float* __restrict__ LSE, const float* __restrict__ delta,
           const int32_t* __restrict__ off_k, const int32_t* __restrict__ goff, const int32_t* __restrict__ pairs,
-          float* __restrict__ dq_part, float* __restrict__ dK_perm, float* __restrict__ dV_perm, int planes, int shares) {
+          float* __restrict__ dq_part, float* __restrict__ dK_perm, float* __restrict__ dV_perm) {
   pdl_wait();
   pdl_trigger();
   constexpr int LD = D + Pad<T>::v;
@@ -237,10 +239,10 @@ k_ret_bwd(Dims dm, const T* __restrict__ Q, const T* __restrict__ dO, const T* _
   const T* Qb = Q + (size_t)pq * dm.N * D; const T* dOb = dO + (size_t)pq * dm.N * D;
   const T* Kb = Kp + (size_t)pk * dm.N * D; const T* Vb = Vp + (size_t)pk * dm.N * D;
   const int32_t* pr = pairs + (size_t)pq * dm.N * dm.m;
-  const int part = blockIdx.z / shares, share = blockIdx.z % shares;      // this CTA's planes: [pl0, pl1)
-  const int pl0 = planes > 1 ? part : 0, pl1 = planes > 1 ? part + 1 : dm.SB;
-  if (go[(size_t)j * dm.SB + pl0] + share * kTile >= go[(size_t)j * dm.SB + pl1]) return;
-  const int kend = ok[pl1];                                               // keys that these planes see
+  const int pl = blockIdx.z / kRetShares, share = blockIdx.z % kRetShares;
+  const int g0 = go[(size_t)j * dm.SB + pl], g1 = go[(size_t)j * dm.SB + pl + 1];
+  if (g0 + share * kTile >= g1) return;
+  const int kend = ok[pl + 1];                                            // keys that the plane sees
   for (int c0 = kbeg; c0 < kend; c0 += kTile) {
     __syncthreads();
     const int nkc = min(kTile, kend - c0);
@@ -248,60 +250,54 @@ k_ret_bwd(Dims dm, const T* __restrict__ Q, const T* __restrict__ dO, const T* _
     load_tile<T, D>(Vs, Vb, nkc, [&](int r) { return c0 + r; }, tid);
     float dk[4][D / 64][4], dv[4][D / 64][4];
     zero_acc<D>(dk); zero_acc<D>(dv);
-    for (int pl = pl0; pl < pl1; ++pl) {
-      const int vis_end = ok[pl + 1];
-      if (c0 >= vis_end) continue;
-      const int nk = min(kTile, vis_end - c0);
-      const int g0 = go[(size_t)j * dm.SB + pl], g1 = go[(size_t)j * dm.SB + pl + 1];
-      for (int t0 = g0 + share * kTile; t0 < g1; t0 += shares * kTile) {
-        const int nq = min(kTile, g1 - t0);
-        __syncthreads();
-        if (tid < kTile) {
-          const int pid = tid < nq ? pr[t0 + tid] : 0;
-          pid_s[tid] = pid;
-          const size_t t = (size_t)pq * dm.N + pid / dm.m;
-          Ls[tid] = tid < nq ? LSE[t] : 0.f;
-          ds[tid] = tid < nq ? delta[t] : 0.f;
+    for (int t0 = g0 + share * kTile; t0 < g1; t0 += kRetShares * kTile) {
+      const int nq = min(kTile, g1 - t0);
+      __syncthreads();
+      if (tid < kTile) {
+        const int pid = tid < nq ? pr[t0 + tid] : 0;
+        pid_s[tid] = pid;
+        const size_t t = (size_t)pq * dm.N + pid / dm.m;
+        Ls[tid] = tid < nq ? LSE[t] : 0.f;
+        ds[tid] = tid < nq ? delta[t] : 0.f;
+      }
+      __syncthreads();
+      load_tile<T, D>(Qs, Qb, nq, [&](int r) { return pid_s[r] / dm.m; }, tid);
+      load_tile<T, D>(dOs, dOb, nq, [&](int r) { return pid_s[r] / dm.m; }, tid);
+      __syncthreads();
+      float s[4][4], dp[4][4];
+      mm_nt<T, D>(Qs, Ks, s, ty, tx, nq);
+      mm_nt<T, D>(dOs, Vs, dp, ty, tx, nq);
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const int row = ty * 4 + r;
+        float p[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          p[c] = (row < nq && tx * 4 + c < nkc) ? expf(s[r][c] * dm.sigma - Ls[row]) : 0.f;
+          dp[r][c] = p[c] * (dp[r][c] - ds[row]);
         }
-        __syncthreads();
-        load_tile<T, D>(Qs, Qb, nq, [&](int r) { return pid_s[r] / dm.m; }, tid);
-        load_tile<T, D>(dOs, dOb, nq, [&](int r) { return pid_s[r] / dm.m; }, tid);
-        __syncthreads();
-        float s[4][4], dp[4][4];
-        mm_nt<T, D>(Qs, Ks, s, ty, tx, nq);
-        mm_nt<T, D>(dOs, Vs, dp, ty, tx, nq);
+        st4(Ps + row * kLDP + tx * 4, make_float4(p[0], p[1], p[2], p[3]));
+      }
+      __syncthreads();
+      mm_tn<T, D>(Ps, dOs, dv, ty, tx, nq, nkc);
+      __syncthreads();
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          const int row = ty * 4 + r;
-          float p[4];
+      for (int r = 0; r < 4; ++r) st4(Ps + (ty * 4 + r) * kLDP + tx * 4, make_float4(dp[r][0], dp[r][1], dp[r][2], dp[r][3]));
+      __syncthreads();
+      mm_tn<T, D>(Ps, Qs, dk, ty, tx, nq, nkc);
+      float dq[4][D / 64][4];
+      zero_acc<D>(dq);
+      mm_pn<T, D>(Ps, Ks, dq, ty, tx, nq, nkc);
 #pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            p[c] = (row < nq && tx * 4 + c < nk) ? expf(s[r][c] * dm.sigma - Ls[row]) : 0.f;
-            dp[r][c] = p[c] * (dp[r][c] - ds[row]);
-          }
-          st4(Ps + row * kLDP + tx * 4, make_float4(p[0], p[1], p[2], p[3]));
-        }
-        __syncthreads();
-        mm_tn<T, D>(Ps, dOs, dv, ty, tx, nq, nk);
-        __syncthreads();
+      for (int r = 0; r < 4; ++r) {
+        const int row = ty * 4 + r;
+        if (row < nq) {
+          float* dst = dq_part + ((size_t)pq * dm.N * dm.m + pid_s[row]) * D + tx * 4;
 #pragma unroll
-        for (int r = 0; r < 4; ++r) st4(Ps + (ty * 4 + r) * kLDP + tx * 4, make_float4(dp[r][0], dp[r][1], dp[r][2], dp[r][3]));
-        __syncthreads();
-        mm_tn<T, D>(Ps, Qs, dk, ty, tx, nq, nk);
-        float dq[4][D / 64][4];
-        zero_acc<D>(dq);
-        mm_pn<T, D>(Ps, Ks, dq, ty, tx, nq, nk);
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          const int row = ty * 4 + r;
-          if (row < nq) {
-            float* dst = dq_part + ((size_t)pq * dm.N * dm.m + pid_s[row]) * D + tx * 4;
-#pragma unroll
-            for (int k = 0; k < D / 64; ++k) {
-              float4 v = make_float4(dq[r][k][0] * dm.sigma, dq[r][k][1] * dm.sigma, dq[r][k][2] * dm.sigma, dq[r][k][3] * dm.sigma);
-              if (c0 != kbeg) { float4 o = ld4(dst + 64 * k); v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w; }
-              st4(dst + 64 * k, v);
-            }
+          for (int k = 0; k < D / 64; ++k) {
+            float4 v = make_float4(dq[r][k][0] * dm.sigma, dq[r][k][1] * dm.sigma, dq[r][k][2] * dm.sigma, dq[r][k][3] * dm.sigma);
+            if (c0 != kbeg) { float4 o = ld4(dst + 64 * k); v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w; }
+            st4(dst + 64 * k, v);
           }
         }
       }
@@ -317,8 +313,8 @@ k_ret_bwd(Dims dm, const T* __restrict__ Q, const T* __restrict__ dO, const T* _
           const float4 b = make_float4(dv[r][k][0], dv[r][k][1], dv[r][k][2], dv[r][k][3]);
           float* pa = dK_perm + u * D + tx * 4 + 64 * k;
           float* pb = dV_perm + u * D + tx * 4 + 64 * k;
-          if (planes > 1) { atomicAdd(reinterpret_cast<float4*>(pa), a); atomicAdd(reinterpret_cast<float4*>(pb), b); }
-          else { st4(pa, a); st4(pb, b); }
+          atomicAdd(reinterpret_cast<float4*>(pa), a);
+          atomicAdd(reinterpret_cast<float4*>(pb), b);
         }
       }
     }
@@ -809,10 +805,7 @@ static int attn_bwd_t(const Dims& d, int dtype, const T* Q, const T* K, const T*
       } else {
         MUSE_CUDA_OK(cudaFuncSetAttribute(k_ret_bwd<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm4));
         prof_mark("k_ret_bwd", st);
-        // fewer (cluster, head) CTAs than two rounds of the chip: split by plane, and the planes' pair tiles in two
-        const bool split = d.Ck * pq < 2 * sm_count();
-        const int planes = split && d.SB > 1 ? d.SB : 1, shares = planes > 1 ? 2 : 1;
-        MUSE_RC(launch_pdl(k_ret_bwd<T, D>, dim3(d.Ck, pq, planes * shares), kFlashThreads, sm4, st, d, Q, dO, Kp, Vp, LSE, w.delta, off_k, ri.goff, ri.pairs, w.dq_part, w.dK_perm, w.dV_perm, planes, shares));
+        MUSE_RC(launch_pdl(k_ret_bwd<T, D>, dim3(d.Ck, pq, d.SB * kRetShares), kFlashThreads, sm4, st, d, Q, dO, Kp, Vp, LSE, w.delta, off_k, ri.goff, ri.pairs, w.dq_part, w.dK_perm, w.dV_perm));
         MUSE_LAUNCH_OK();
       }
       use_ret = 1;
